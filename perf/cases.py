@@ -232,3 +232,116 @@ def tolerance(case):
     if case["feature"] or case["out_norm"]:
         return {"rel": 1.6e-2, "max": 0.14}
     return {"rel": 6.6e-3, "max": 1.6e-2}
+
+
+# ------------------------------------------------------------------ the same in 64 bits
+def _swish_slope(x):
+    g = torch.sigmoid(x)
+    return g * (1.0 + x * (1.0 - g))
+
+
+def _decay(c, gate):
+    """a (the share of its memory that a slot keeps) and d a / d gate."""
+    x = gate.double()
+    if c["gate"] == "a":
+        return x, torch.ones_like(x)
+    if c["gate"] == "log":
+        return x.exp(), x.exp()
+    a = torch.exp(torch.nn.functional.logsigmoid(x) / c["tau"])
+    return a, a * torch.sigmoid(-x) / c["tau"]
+
+
+def _step(K, V, a, q, k, v):
+    """One token of the recurrence; the memories K, V [N, m, d] are updated in place.  Returns o and the slot weights."""
+    w = (1.0 - a).unsqueeze(2)
+    K.mul_(a.unsqueeze(2)).baddbmm_(w, k.unsqueeze(1))
+    V.mul_(a.unsqueeze(2)).baddbmm_(w, v.unsqueeze(1))
+    p = torch.softmax(torch.bmm(K, q.unsqueeze(2)).squeeze(2), 1)
+    return torch.bmm(p.unsqueeze(1), V).squeeze(1), p
+
+
+def _exact_decode(s):
+    c, out = s["case"], []
+    for x in (s["layers"][0], s["layers"][-1]):
+        n = c["B"] * c["H"]
+        q, k, v = (x[t].double().view(n, c["d"]) for t in ("q", "k", "v"))
+        K, V = (x[t].double().view(n, c["m"], c["d"]).clone() for t in ("K", "V"))
+        o, _ = _step(K, V, _decay(c, x["gate"])[0].view(n, c["m"]), q, k, v)
+        out += [o.view(x["o"].shape), K.view(x["K"].shape), V.view(x["V"].shape)]
+    return out
+
+
+@torch.no_grad()
+def exact(case, seed):
+    s = prepare(case, seed)
+    c = s["case"]
+    if c["kind"] == "decode":
+        return _exact_decode(s)
+    B, T, H, d, m = (c[n] for n in ("B", "T", "H", "d", "m"))
+    N = B * H
+
+    def by_time(x):                                       # [B, T, H, n] -> [T, B H, n]
+        return x.double().permute(1, 0, 2, 3).reshape(T, N, -1)
+
+    def by_batch(x):
+        return x.view(T, B, H, -1).permute(1, 0, 2, 3).contiguous()
+
+    raw = {n: by_time(s["x"][n]) for n in ("q", "k", "v")}
+    q, k, v = (torch.nn.functional.silu(raw[n]) if c["feature"] else raw[n] for n in ("q", "k", "v"))
+    a, slope = _decay(c, by_time(s["x"]["gate"]))
+    starts = set(_offsets(c, seed).tolist()[1:-1]) if c["nseq"] else set()
+    K = s["K0"].double().view(N, m, d).clone() if c["carry"] else torch.zeros(N, m, d, dtype=torch.float64, device="cuda")
+    V = s["V0"].double().view(N, m, d).clone() if c["carry"] else torch.zeros_like(K)
+    o, p = torch.empty_like(v), torch.empty_like(a)
+    kept = {}                                             # the memories before every 64th token, for the way back
+
+    def forward(t):
+        if t in starts:
+            K.zero_(), V.zero_()
+        o[t], p[t] = _step(K, V, a[t], q[t], k[t], v[t])
+
+    for t in range(T):
+        if c["kind"] == "train" and t % 64 == 0:
+            kept[t] = K.clone(), V.clone()
+        forward(t)
+    if c["kind"] == "forward":
+        return {"o": by_batch(o), "KT": K.view(B, H, m, d).clone(), "VT": V.view(B, H, m, d).clone()}
+    out = {}
+    d_o = by_time(s["dy"])
+    ob = by_batch(o)
+    if c["out_norm"]:
+        with torch.enable_grad():
+            x, w = ob.clone().requires_grad_(), s["norm_weight"].double().requires_grad_()
+            y = torch.nn.functional.rms_norm(torch.nn.functional.silu(x).view(B, T, H * d), (H * d,), w, 1e-6)
+            gx, out["dweight"] = torch.autograd.grad(y, (x, w), s["dy"].double().view(B, T, H * d))
+        out["y"] = y.detach().view(B, T, H, d)
+        d_o = by_time(gx)
+    out["o"] = ob
+    dq, dk, dv, da = torch.empty_like(q), torch.empty_like(k), torch.empty_like(v), torch.empty_like(a)
+    gK, gV = torch.zeros_like(K), torch.zeros_like(V)     # gradients w.r.t. the memories after token t
+    for t0 in reversed(range(0, T, 64)):
+        K.copy_(kept[t0][0]), V.copy_(kept[t0][1])
+        before, after = [], []
+        for t in range(t0, min(t0 + 64, T)):
+            if t in starts:
+                K.zero_(), V.zero_()
+            before.append((K.clone(), V.clone()))
+            forward(t)
+            after.append((K.clone(), V.clone()))
+        for t in reversed(range(t0, min(t0 + 64, T))):
+            (K0, V0), (K1, V1) = before[t - t0], after[t - t0]
+            dp = torch.bmm(V1, d_o[t].unsqueeze(2)).squeeze(2)
+            dz = p[t] * (dp - (p[t] * dp).sum(1, keepdim=True))
+            dq[t] = torch.bmm(dz.unsqueeze(1), K1).squeeze(1)
+            gK.baddbmm_(dz.unsqueeze(2), q[t].unsqueeze(1))
+            gV.baddbmm_(p[t].unsqueeze(2), d_o[t].unsqueeze(1))
+            w = (1.0 - a[t]).unsqueeze(1)
+            dk[t], dv[t] = torch.bmm(w, gK).squeeze(1), torch.bmm(w, gV).squeeze(1)
+            da[t] = ((gK * K0).sum(2) + (gV * V0).sum(2) - torch.bmm(gK, k[t].unsqueeze(2)).squeeze(2)
+                     - torch.bmm(gV, v[t].unsqueeze(2)).squeeze(2))
+            keep = torch.zeros_like(a[t]) if t in starts else a[t]
+            gK.mul_(keep.unsqueeze(2)), gV.mul_(keep.unsqueeze(2))
+    for n, g in (("q", dq), ("k", dk), ("v", dv)):
+        out["d" + n] = by_batch(g * _swish_slope(raw[n]) if c["feature"] else g)
+    out["dgate"] = by_batch(da * slope)
+    return out
