@@ -19,6 +19,7 @@ bool dim_ok(int d) { return d == 64 || d == 128 || d == 256 || d == 512; }
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+constexpr int kSMs = 148;             // B200
 constexpr int kPaddedSlots = 64;      // slot width of the tensor-core tiles (see pads_slots)
 
 gsa_status_t check_params(const gsa_params_t* p, bool need_T) {
@@ -50,6 +51,13 @@ gsa_status_t check_params(const gsa_params_t* p, bool need_T) {
 }
 
 // Does this call run the tensor-core chunk kernels?
+bool use_tc(const gsa_params_t& p);
+// The parameters of a call as the host code passes them on: the caller's, and how many segments its scans may be
+// cut into (see segments_of; less than that rule would take only where the scratch memory is a fixed one).
+struct CallParams : gsa_params_t {
+    int max_segments;
+    CallParams(const gsa_params_t& p, int max_seg = 1 << 30) : gsa_params_t(p), max_segments(max_seg) {}
+};
 bool use_tc(const gsa_params_t& p) {
     if (p.impl == GSA_IMPL_SIMT) return false;
     return p.io == GSA_BF16 && tc_supported(p.d_k, p.d_v, p.m);
@@ -62,8 +70,8 @@ bool use_tc(const gsa_params_t& p) {
 bool pads_slots(const gsa_params_t& p) {
     return p.impl != GSA_IMPL_SIMT && p.io == GSA_BF16 && p.m == 32 && tc_supported(p.d_k, p.d_v, kPaddedSlots);
 }
-gsa_params_t internal_params(const gsa_params_t& p) {
-    gsa_params_t q = p;
+CallParams internal_params(const CallParams& p) {
+    CallParams q = p;
     if (pads_slots(p)) q.m = kPaddedSlots;
     return q;
 }
@@ -85,17 +93,44 @@ Slices slices(const gsa_params_t& p) {
     return {p.d_k / 64, p.d_v / 64};
 }
 
-// Segment-parallel scheduling of the forward: when (batch, head, slice) triples cannot fill the
-// GPU, long sequences are cut into nseg segments that run as independent sequences (the
-// memories are linear in (k, v), so every segment's start memories follow from a first pass
-// that runs the segments from empty memories).  1 = off.
-int segments_of(const gsa_params_t& p) {
-    if (!use_tc(p)) return 1;
-    const int chunk = tc_chunk();
-    const long long ctas = (long long)p.B * p.H * tc_value_side_slices(p.d_k < p.d_v ? p.d_k : p.d_v);
-    int nseg = 1;
-    while (ctas * nseg * 2 <= 160 && p.T % (nseg * 2 * chunk) == 0 && p.T / (nseg * 2) >= 8 * chunk) nseg *= 2;
-    return nseg;
+// Segment-parallel scheduling: when (batch, head, slice) triples cannot fill the GPU, a sequence is cut into n
+// segments of t tokens (whole chunks; the last segment takes what is left) that run as independent sequences:
+// the memories are linear in (k, v), so every segment's start memories follow from a first run of the segments
+// from empty memories, for their end memories only.  n = 1: off.
+//
+// The rule: the n with the smallest time by this model of a forward, one wave of CTAs at most,
+//     n = 1:  2 (chunks * scan + launch)        n > 1:  2 (chunks / n * (scan + state) + 2 launch) + combine
+// (two scans, two state-only runs, the scans over the segments), if it saves a sixth of the time.  The times per
+// chunk and launch, in tenths of a microsecond, are measured ones.  Forward, us: B = 1, T = 4096, 32 heads of 128 as
+// one segment 227, two 218, four (the rule's) 185; T = 1431, 4 heads of 512 as one (the rule's) 86, six 105 (the
+// launches); training steps: T = 5001, 4 heads of 512: one 500, four 321, nine (the rule's) 289; fp32, B = 2,
+// T = 1024, 4 heads of 256: one 2030, four 782, eight (the rule's) 618.
+struct Segments { int n, t; };
+Segments segments_of(const CallParams& p) {
+    const bool tc = use_tc(p);
+    const int chunk = chunk_of(p), chunks = (p.T + chunk - 1) / chunk;
+    const Slices sl = slices(p);
+    const long long ctas = (long long)p.B * p.H * (sl.k < sl.v ? sl.k : sl.v);
+    if (use_fused(p)) {       // (the fused kernel sees segments as batch elements: equal ones)
+        int n = 1;
+        while (ctas * n * 2 <= 160 && p.T % (n * 2 * chunk) == 0 && p.T / (n * 2) >= 8 * chunk && n * 2 <= p.max_segments) n *= 2;
+        return {n, p.T / n};
+    }
+    const int slots = tc || p.m > 64 ? kSMs : 2 * kSMs;       // CTAs of a scan that the GPU holds at a time
+    const int scan = tc ? 27 : (p.m > 64 ? 280 : 150), state = tc ? 10 : scan / 3, launch = tc ? 100 : 50,
+              combine = tc ? 200 : 110;
+    long long most = slots / ctas;
+    if (most > p.max_segments) most = p.max_segments;
+    if (most > chunks) most = chunks;
+    const long long alone = 2LL * ((long long)chunks * scan + launch);
+    int best = chunks;
+    long long best_cost = alone - alone / 6;
+    for (int n = 2; n <= most; ++n) {
+        const int per = (chunks + n - 1) / n;
+        const long long cost = 2LL * ((long long)per * (scan + state) + 2 * launch) + combine;
+        if (cost < best_cost) { best = per; best_cost = cost; }
+    }
+    return {(chunks + best - 1) / best, best * chunk};
 }
 
 struct Carver {
@@ -117,13 +152,13 @@ struct Workspace {
     size_t bytes;
 };
 
-Workspace carve(const gsa_params_t& p, int which, void* ws) {
+Workspace carve(const CallParams& p, int which, void* ws) {
     Workspace w;
     memset(&w, 0, sizeof(w));
     const size_t mt = (size_t)p.B * p.T * p.H * p.m;
     const Slices s = slices(p);
     Carver c{static_cast<char*>(ws), 0};
-    const int nseg = segments_of(p);
+    const int nseg = segments_of(p).n;
     w.strong = reinterpret_cast<int*>(c.take((size_t)p.B * p.H * nseg));
     if (nseg > 1) {
         const size_t pairs = (size_t)p.B * nseg * p.H;
@@ -171,11 +206,11 @@ struct GateSums {
     float *seg_decay, *Kstart, *Vstart, *KT, *VT;     // nseg > 1 only
     size_t bytes;
 };
-GateSums carve_gate(const gsa_params_t& p, void* base) {
+GateSums carve_gate(const CallParams& p, void* base) {
     GateSums g;
     memset(&g, 0, sizeof(g));
     const size_t mt = (size_t)p.B * p.T * p.H * p.m;
-    const int nseg = segments_of(p);
+    const int nseg = segments_of(p).n;
     Carver c{static_cast<char*>(base), 0};
     g.strong = reinterpret_cast<int*>(c.take((size_t)p.B * p.H * nseg));
     g.G = c.take(mt);
@@ -198,7 +233,7 @@ GateSums carve_gate(const gsa_params_t& p, void* base) {
     return g;
 }
 // points the workspace's gate products at the block; false if the block is missing or too small
-bool use_gate_block(const gsa_params_t& p, Workspace* w, void* block, size_t block_bytes) {
+bool use_gate_block(const CallParams& p, Workspace* w, void* block, size_t block_bytes) {
     if (block == nullptr || (reinterpret_cast<uintptr_t>(block) & 255u) != 0) return false;
     const GateSums g = carve_gate(p, block);
     if (block_bytes < g.bytes) return false;
@@ -370,11 +405,11 @@ FeatureBuffers carve_features(const gsa_params_t& p, void* base) {
     f.bytes = 2 * nk + nv;
     return f;
 }
-gsa_status_t apply_feature_map(const gsa_params_t& p, int which, const void** q, const void** k, const void** v, void* ws,
+gsa_status_t apply_feature_map(const CallParams& p, int which, const void** q, const void** k, const void** v, void* ws,
                                size_t ws_bytes, cudaStream_t st) {
     if (p.feature_map != GSA_FEAT_SWISH) return GSA_OK;
     if (ws == nullptr || (reinterpret_cast<uintptr_t>(ws) & 255u) != 0) return GSA_ERR_WORKSPACE;
-    const gsa_params_t pi = internal_params(p);
+    const CallParams pi = internal_params(p);
     const size_t before = carve(pi, which, nullptr).bytes + pad_bytes(p, which) + gate_conv_bytes(p, which);
     const FeatureBuffers f = carve_features(p, static_cast<char*>(ws) + before);
     if (ws_bytes < before + f.bytes) return GSA_ERR_WORKSPACE;
@@ -442,6 +477,14 @@ const char* gsa_status_string(gsa_status_t status) {
     return "unknown status";
 }
 
+namespace {
+size_t workspace_bytes(const CallParams& p, int32_t which) {
+    const CallParams pi = internal_params(p);
+    if (which == GSA_WS_GATE) return carve_gate(pi, nullptr).bytes;
+    return carve(pi, which, nullptr).bytes + pad_bytes(p, which) + gate_conv_bytes(p, which) + carve_features(p, nullptr).bytes;
+}
+}  // namespace
+
 size_t gsa_workspace_bytes(const gsa_params_t* params, int32_t which) {
     if (which == GSA_WS_DECODE) return 0;
     if (which != GSA_WS_FWD && which != GSA_WS_BWD && which != GSA_WS_GATE && which != GSA_WS_SHARD) return 0;
@@ -452,10 +495,7 @@ size_t gsa_workspace_bytes(const gsa_params_t* params, int32_t which) {
         return carve(*params, GSA_WS_FWD, nullptr).bytes +
                align_up((size_t)params->B * params->T * params->H * params->d_v * esz, 256);
     }
-    const gsa_params_t pi = internal_params(*params);
-    if (which == GSA_WS_GATE) return carve_gate(pi, nullptr).bytes;
-    return carve(pi, which, nullptr).bytes + pad_bytes(*params, which) + gate_conv_bytes(*params, which) +
-           carve_features(*params, nullptr).bytes;
+    return workspace_bytes(*params, which);
 }
 
 gsa_status_t gsa_gate_cumsum(const gsa_params_t* params, const float* gate, float* G, float* I,
@@ -468,17 +508,17 @@ gsa_status_t gsa_gate_cumsum(const gsa_params_t* params, const float* gate, floa
     const gsa_params_t& p = *params;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     GSA_LAUNCH("gate_cumsum", launch_gate_cumsum(gate, p.gate_kind, inv_tau(p), G, I, p.B, p.T,
-                                                 p.H, p.m, chunk_of(internal_params(p)), nullptr, 1, nullptr, 0, st,
+                                                 p.H, p.m, chunk_of(internal_params(p)), nullptr, 1, p.T, nullptr, 0, st,
                                                  p.cu_seqlens, p.nseq));
     return GSA_OK;
 }
 
 namespace {
-gsa_status_t fwd_core(const gsa_params_t* params, int m_active, const void* q, const void* k, const void* v,
+gsa_status_t fwd_core(const CallParams* params, int m_active, const void* q, const void* k, const void* v,
                       const float* gate, const float* K0, const float* V0, void* o,
                       float* ok_save, float* KT, float* VT, bool save_gate, void* gate_save, size_t gate_save_bytes,
                       void* ws, size_t ws_bytes, void* stream, int32_t* dev_status) {
-    const gsa_params_t& p = *params;
+    const CallParams& p = *params;
     if (ws == nullptr || (reinterpret_cast<uintptr_t>(ws) & 255u) != 0) return GSA_ERR_WORKSPACE;
     Workspace w = carve(p, GSA_WS_FWD, ws);
     if (ws_bytes < w.bytes) return GSA_ERR_WORKSPACE;
@@ -487,19 +527,18 @@ gsa_status_t fwd_core(const gsa_params_t* params, int m_active, const void* q, c
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const Slices s = slices(p);
 
-    const int nseg = segments_of(p);
+    const Segments segs = segments_of(p);
+    const int nseg = segs.n, tseg = segs.t;
     GSA_CUDA(cudaMemsetAsync(w.strong, 0, sizeof(int) * (size_t)p.B * p.H * nseg, st));
     if (p.gate_kind == GSA_GATE_ABC)      // no decay, write weights from the cumulative softmax of the scores
         GSA_LAUNCH("abc_write", launch_abc_write(gate, w.G, w.I, w.Id, p.B, p.T, p.H, p.m, st));
     else
         GSA_LAUNCH("gate_cumsum", launch_gate_cumsum(gate, p.gate_kind, inv_tau(p), w.G, w.I, p.B, p.T,
-                                                     p.H, p.m, chunk_of(p), w.strong, nseg, w.Id, p.io == GSA_BF16, st,
+                                                     p.H, p.m, chunk_of(p), w.strong, nseg, tseg, w.Id, p.io == GSA_BF16, st,
                                                      p.cu_seqlens, p.nseq));
     float* ok = ok_save;      // the scaled logits leave the softmax kernel only if the caller keeps them
     // the pipelined kernels leave the row factor of the pass-1 sums to the softmax kernel
-    const PendingDecay pend = use_tc(p) ? PendingDecay{w.G, w.strong, p.T, p.H, nseg} : PendingDecay{nullptr, nullptr, 1, 1, 1};
-    // [B,T,H,.] cut into nseg segments is the same memory as [B*nseg, T/nseg, H, .]
-    const int Bs = p.B * nseg, Ts = p.T / nseg;
+    const PendingDecay pend = use_tc(p) ? PendingDecay{w.G, w.strong, p.T, p.H, nseg, tseg, 0} : PendingDecay{nullptr, nullptr, 1, 1, 1, 1, 0};
     const float *Kin = K0, *Vin = V0;
     float *Kout = KT, *Vout = VT;
     if (nseg > 1) {
@@ -507,10 +546,12 @@ gsa_status_t fwd_core(const gsa_params_t* params, int m_active, const void* q, c
         // land in buffers that the second pass overwrites); then the start memories of all
         // segments, and the final memories, by a scan over the segments
         GSA_LAUNCH("segment_logdecay", launch_segment_logdecay(w.G, w.seg_decay, p.B, p.T, p.H, p.m, nseg,
-                                                               chunk_of(p), st));
-        ValueSideArgs s1{q, k, w.I, w.G, nullptr, w.Kloc, w.okpart, Bs, Ts, p.H, p.d_k, w.Id, 1};
+                                                               tseg, chunk_of(p), st));
+        ValueSideArgs s1{q, k, w.I, w.G, nullptr, w.Kloc, w.okpart, p.B, p.T, p.H, p.d_k, w.Id, 1};
+        s1.nseg = nseg; s1.tseg = tseg;
         GSA_LAUNCH("segment_pass1_states", value_side(p, s1, 0, w.strong, st, dev_status));
-        KeySideArgs s2{w.I, w.I, w.G, v, nullptr, w.Vloc, o, Bs, Ts, p.H, p.d_v, w.Id, w.Id, 1};
+        KeySideArgs s2{w.I, w.I, w.G, v, nullptr, w.Vloc, o, p.B, p.T, p.H, p.d_v, w.Id, w.Id, 1};
+        s2.nseg = nseg; s2.tseg = tseg;
         GSA_LAUNCH("segment_pass2_states", key_side(p, s2, 0, w.strong, st, dev_status));
         // (when the backward is to reuse them, the final memories land in the saved block first)
         float* KTc = save_gate ? w.KT : KT;
@@ -527,9 +568,11 @@ gsa_status_t fwd_core(const gsa_params_t* params, int m_active, const void* q, c
         Kout = nullptr; Vout = nullptr;
     }
     // pass 1: o' = GLA(q, k, 1-a) with the decay on the slot (value) side
-    ValueSideArgs a1{q, k, w.I, w.G, Kin, Kout, w.okpart, Bs, Ts, p.H, p.d_k, w.Id};
+    ValueSideArgs a1{q, k, w.I, w.G, Kin, Kout, w.okpart, p.B, p.T, p.H, p.d_k, w.Id};
+    a1.nseg = nseg; a1.tseg = tseg;
     // pass 2: o = GLA(softmax(o'), 1-a, v) with the decay on the slot (key) side
-    KeySideArgs a2{w.p, w.I, w.G, v, Vin, Vout, o, Bs, Ts, p.H, p.d_v, w.Pd, w.Id};
+    KeySideArgs a2{w.p, w.I, w.G, v, Vin, Vout, o, p.B, p.T, p.H, p.d_v, w.Pd, w.Id};
+    a2.nseg = nseg; a2.tseg = tseg;
     if (use_fused(p)) {
         // One kernel for pass 1 -> softmax -> pass 2; the logits are written only if the caller wants
         // them.  The (batch, head) pairs flagged for strong decay take the general kernels and the
@@ -543,7 +586,7 @@ gsa_status_t fwd_core(const gsa_params_t* params, int m_active, const void* q, c
             GSA_CUDA(cudaEventRecord(side->fork, st));
             GSA_CUDA(cudaStreamWaitEvent(ss, side->fork, 0));
         }
-        GSA_LAUNCH("fused_fwd", launch_fused_pair(0, q, k, w.Id, v, o, w.G, Kin, Vin, Kout, Vout, Bs, Ts, p.H, p.d_k,
+        GSA_LAUNCH("fused_fwd", launch_fused_pair(0, q, k, w.Id, v, o, w.G, Kin, Vin, Kout, Vout, p.B * nseg, tseg, p.H, p.d_k,
                                                   p.d_v, p.scale, p.slot_act, ok_save, nullptr, nullptr, nullptr, w.strong,
                                                   st, dev_status));
         GSA_CUDA(launch_value_side_general(a1, p.m, 0, w.strong, ss, dev_status));
@@ -563,7 +606,7 @@ gsa_status_t fwd_core(const gsa_params_t* params, int m_active, const void* q, c
 }
 
 // Validation, and the padded-slot mode around the core (see pads_slots).
-gsa_status_t fwd_impl(const gsa_params_t* params, const void* q, const void* k, const void* v,
+gsa_status_t fwd_impl(const CallParams* params, const void* q, const void* k, const void* v,
                       const float* gate, const float* K0, const float* V0, void* o,
                       float* ok_save, float* KT, float* VT, bool save_gate, void* gate_save, size_t gate_save_bytes,
                       void* ws, size_t ws_bytes, void* stream, int32_t* dev_status) {
@@ -574,7 +617,7 @@ gsa_status_t fwd_impl(const gsa_params_t* params, const void* q, const void* k, 
         return GSA_ERR_INVALID_ARG;
     {
         // a bfloat16 gate tensor is widened once; everything downstream reads fp32
-        const gsa_params_t pi0 = internal_params(*params);
+        const CallParams pi0 = internal_params(*params);
         const size_t before = carve(pi0, GSA_WS_FWD, nullptr).bytes + pad_bytes(*params, GSA_WS_FWD);
         rc = gate_as_f32(*params, GSA_WS_FWD, gate, ws, ws_bytes, before, static_cast<cudaStream_t>(stream), &gate);
         if (rc != GSA_OK) return rc;
@@ -584,8 +627,8 @@ gsa_status_t fwd_impl(const gsa_params_t* params, const void* q, const void* k, 
     if (!pads_slots(*params))
         return fwd_core(params, 0, q, k, v, gate, K0, V0, o, ok_save, KT, VT, save_gate, gate_save, gate_save_bytes, ws,
                         ws_bytes, stream, dev_status);
-    const gsa_params_t& p = *params;
-    const gsa_params_t pi = internal_params(p);
+    const CallParams& p = *params;
+    const CallParams pi = internal_params(p);
     if (ws == nullptr || (reinterpret_cast<uintptr_t>(ws) & 255u) != 0) return GSA_ERR_WORKSPACE;
     const size_t core = carve(pi, GSA_WS_FWD, nullptr).bytes;
     const PadBuffers pb = carve_pad(p, GSA_WS_FWD, static_cast<char*>(ws) + core);
@@ -613,7 +656,9 @@ gsa_status_t gsa_fwd(const gsa_params_t* params, const void* q, const void* k, c
                      const float* gate, const float* K0, const float* V0, void* o,
                      float* ok_save, float* KT, float* VT, void* ws, size_t ws_bytes,
                      void* stream, int32_t* dev_status) {
-    return fwd_impl(params, q, k, v, gate, K0, V0, o, ok_save, KT, VT, false, nullptr, 0, ws, ws_bytes, stream,
+    if (params == nullptr) return GSA_ERR_INVALID_ARG;
+    const CallParams cp(*params);
+    return fwd_impl(&cp, q, k, v, gate, K0, V0, o, ok_save, KT, VT, false, nullptr, 0, ws, ws_bytes, stream,
                     dev_status);
 }
 
@@ -621,17 +666,36 @@ gsa_status_t gsa_fwd_save_gate(const gsa_params_t* params, const void* q, const 
                                const float* gate, const float* K0, const float* V0, void* o,
                                float* ok_save, float* KT, float* VT, void* gate_save, size_t gate_save_bytes,
                                void* ws, size_t ws_bytes, void* stream, int32_t* dev_status) {
-    return fwd_impl(params, q, k, v, gate, K0, V0, o, ok_save, KT, VT, true, gate_save, gate_save_bytes, ws,
+    if (params == nullptr) return GSA_ERR_INVALID_ARG;
+    const CallParams cp(*params);
+    return fwd_impl(&cp, q, k, v, gate, K0, V0, o, ok_save, KT, VT, true, gate_save, gate_save_bytes, ws,
                     ws_bytes, stream, dev_status);
 }
 
+}  // extern "C"
+
+// The forward in a scratch memory of a given size: with as many segments as fit it.
+gsa_status_t gsa::fwd_within(const gsa_params_t* params, const void* q, const void* k, const void* v, const float* gate,
+                             const float* K0, const float* V0, void* o, float* ok_save, float* KT, float* VT, void* ws,
+                             size_t ws_bytes, void* stream, int32_t* dev_status) {
+    const gsa_status_t rc = check_params(params, true);
+    if (rc != GSA_OK) return rc;
+    CallParams cp(*params);
+    cp.max_segments = segments_of(internal_params(cp)).n;
+    while (cp.max_segments > 1 && workspace_bytes(cp, GSA_WS_FWD) > ws_bytes) --cp.max_segments;
+    if (workspace_bytes(cp, GSA_WS_FWD) > ws_bytes) return GSA_ERR_WORKSPACE;
+    return fwd_impl(&cp, q, k, v, gate, K0, V0, o, ok_save, KT, VT, false, nullptr, 0, ws, ws_bytes, stream, dev_status);
+}
+
+extern "C" {
+
 namespace {
-gsa_status_t bwd_core(const gsa_params_t* params, int m_active, const void* q, const void* k, const void* v,
+gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, const void* k, const void* v,
                       const float* gate, const float* K0, const float* V0, const float* ok_saved,
                       const void* dO, const float* dKT, const float* dVT, void* dq, void* dk,
                       void* dv, float* dgate, float* dK0, float* dV0, bool gate_is_saved, const void* gate_saved,
                       size_t gate_saved_bytes, void* ws, size_t ws_bytes, void* stream, int32_t* dev_status) {
-    const gsa_params_t& p = *params;
+    const CallParams& p = *params;
     if (ws == nullptr || (reinterpret_cast<uintptr_t>(ws) & 255u) != 0) return GSA_ERR_WORKSPACE;
     Workspace w = carve(p, GSA_WS_BWD, ws);
     if (ws_bytes < w.bytes) return GSA_ERR_WORKSPACE;
@@ -639,22 +703,22 @@ gsa_status_t bwd_core(const gsa_params_t* params, int m_active, const void* q, c
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const Slices s = slices(p);
 
-    // Long sequences with few (batch, head) pairs run as nseg independent segments (see gsa_fwd):
-    // [B,T,H,.] viewed as [B*nseg, T/nseg, H, .], every scan starting from the state that enters its
-    // segment -- from the left for the forward-direction scans, from the right for the reversed ones.
-    const int nseg = segments_of(p);
-    const int Bs = p.B * nseg, Ts = p.T / nseg;
+    // Sequences with few (batch, head) pairs run as nseg independent segments (see segments_of), every scan
+    // starting from the state that enters its segment -- from the left for the forward-direction scans, from
+    // the right for the reversed ones.
+    const Segments segs = segments_of(p);
+    const int nseg = segs.n, tseg = segs.t;
     if (!gate_is_saved) {      // (a forward of the same call left the gate kernel's products otherwise)
         GSA_CUDA(cudaMemsetAsync(w.strong, 0, sizeof(int) * (size_t)p.B * p.H * nseg, st));
         if (p.gate_kind == GSA_GATE_ABC)
             GSA_LAUNCH("abc_write", launch_abc_write(gate, w.G, w.I, w.Id, p.B, p.T, p.H, p.m, st));
         else
             GSA_LAUNCH("gate_cumsum", launch_gate_cumsum(gate, p.gate_kind, inv_tau(p), w.G, w.I, p.B, p.T,
-                                                         p.H, p.m, chunk_of(p), w.strong, nseg, w.Id, p.io == GSA_BF16, st,
+                                                         p.H, p.m, chunk_of(p), w.strong, nseg, tseg, w.Id, p.io == GSA_BF16, st,
                                                          p.cu_seqlens, p.nseq));
     }
     const float* ok = ok_saved;
-    const PendingDecay pend = use_tc(p) ? PendingDecay{w.G, w.strong, p.T, p.H, nseg} : PendingDecay{nullptr, nullptr, 1, 1, 1};
+    const PendingDecay pend = use_tc(p) ? PendingDecay{w.G, w.strong, p.T, p.H, nseg, tseg, 0} : PendingDecay{nullptr, nullptr, 1, 1, 1, 1, 0};
     const float *Kin = K0, *Vin = V0;        // states entering the forward-direction scans
     float* KTout = dKT ? w.KT : nullptr;     // final memories, for the gate gradient's final-memory term
     float* VTout = dVT ? w.VT : nullptr;
@@ -665,10 +729,12 @@ gsa_status_t bwd_core(const gsa_params_t* params, int m_active, const void* q, c
         KTout = nullptr; VTout = nullptr;
     } else if (nseg > 1) {
         GSA_LAUNCH("segment_logdecay", launch_segment_logdecay(w.G, w.seg_decay, p.B, p.T, p.H, p.m, nseg,
-                                                               chunk_of(p), st));
-        ValueSideArgs s1{q, k, w.I, w.G, nullptr, w.Kloc, w.okpart, Bs, Ts, p.H, p.d_k, w.Id, 1};
+                                                               tseg, chunk_of(p), st));
+        ValueSideArgs s1{q, k, w.I, w.G, nullptr, w.Kloc, w.okpart, p.B, p.T, p.H, p.d_k, w.Id, 1};
+        s1.nseg = nseg; s1.tseg = tseg;
         GSA_LAUNCH("segment_pass1_states", value_side(p, s1, 0, w.strong, st, dev_status));
-        KeySideArgs s2{w.I, w.I, w.G, v, nullptr, w.Vloc, dv, Bs, Ts, p.H, p.d_v, w.Id, w.Id, 1};
+        KeySideArgs s2{w.I, w.I, w.G, v, nullptr, w.Vloc, dv, p.B, p.T, p.H, p.d_v, w.Id, w.Id, 1};
+        s2.nseg = nseg; s2.tseg = tseg;
         GSA_LAUNCH("segment_pass2_states", key_side(p, s2, 0, w.strong, st, dev_status));
         GSA_LAUNCH("segment_combine", launch_segment_combine(w.seg_decay, w.Kloc, K0, w.Kstart, KTout, p.B, p.H, p.m,
                                                              p.d_k, nseg, 0, st));
@@ -678,16 +744,19 @@ gsa_status_t bwd_core(const gsa_params_t* params, int m_active, const void* q, c
         KTout = nullptr; VTout = nullptr;
     }
     if (ok == nullptr) {  // recompute pass 1 and its logits
-        ValueSideArgs a1{q, k, w.I, w.G, Kin, nullptr, w.okpart, Bs, Ts, p.H, p.d_k, w.Id};
+        ValueSideArgs a1{q, k, w.I, w.G, Kin, nullptr, w.okpart, p.B, p.T, p.H, p.d_k, w.Id};
+        a1.nseg = nseg; a1.tseg = tseg;
         GSA_LAUNCH("pass1_value_side", value_side(p, a1, 0, w.strong, st, dev_status));
         GSA_LAUNCH("slot_softmax", launch_slot_softmax_fwd(w.okpart, s.k, p.scale, p.slot_act, w.ok, w.p, p.B, p.T * p.H, p.m, pend.G,
                                                            nullptr, pend, st, m_active));
         ok = w.ok;
     }
     // gradient w.r.t. the pass-2 queries p: the pass-1 form on (dO, v, 1-a); carries V~
-    ValueSideArgs adp{dO, v, w.I, w.G, Vin, VTout, w.dppart, Bs, Ts, p.H, p.d_v, w.Id};
+    ValueSideArgs adp{dO, v, w.I, w.G, Vin, VTout, w.dppart, p.B, p.T, p.H, p.d_v, w.Id};
+    adp.nseg = nseg; adp.tseg = tseg;
     // dq: the pass-2 form on (dz, 1-a, k); carries K~
-    KeySideArgs adq{w.dz, w.I, w.G, k, Kin, KTout, dq, Bs, Ts, p.H, p.d_k, w.Zd, w.Id};
+    KeySideArgs adq{w.dz, w.I, w.G, k, Kin, KTout, dq, p.B, p.T, p.H, p.d_k, w.Zd, w.Id};
+    adq.nseg = nseg; adq.tseg = tseg;
     const bool fused = use_fused(p);
     // With the forward's slot weights in the saved block (and the logits saved, so that nothing here
     // rewrites them), the dv and dI^v scans depend on nothing this call computes: they start at once,
@@ -715,7 +784,7 @@ gsa_status_t bwd_core(const gsa_params_t* params, int m_active, const void* q, c
             GSA_CUDA(cudaEventRecord(side->fork, st));
             GSA_CUDA(cudaStreamWaitEvent(ss, side->fork, 0));
         }
-        GSA_LAUNCH("fused_bwd", launch_fused_pair(1, dO, v, w.Id, k, dq, w.G, Vin, Kin, VTout, KTout, Bs, Ts, p.H, p.d_v,
+        GSA_LAUNCH("fused_bwd", launch_fused_pair(1, dO, v, w.Id, k, dq, w.G, Vin, Kin, VTout, KTout, p.B * nseg, tseg, p.H, p.d_v,
                                                   p.d_k, p.scale, p.slot_act, const_cast<float*>(ok), w.u, w.Pd, w.Zd,
                                                   w.strong, st, dev_status));
         GSA_CUDA(launch_value_side_general(adp, p.m, 0, w.strong, ss, dev_status));
@@ -729,8 +798,10 @@ gsa_status_t bwd_core(const gsa_params_t* params, int m_active, const void* q, c
     } else {
         GSA_LAUNCH("bwd_dp_value_side", value_side(p, adp, 0, w.strong, sc, dev_status));
         if (early) {
-            KeySideArgs adv{w.I, w.p, w.G, dO, dVT, dV0, dv, Bs, Ts, p.H, p.d_v, w.Id, w.Pd};
-            ValueSideArgs adIv{v, dO, w.p, w.G, dVT, nullptr, w.dIv, Bs, Ts, p.H, p.d_v, w.Pd};
+            KeySideArgs adv{w.I, w.p, w.G, dO, dVT, dV0, dv, p.B, p.T, p.H, p.d_v, w.Id, w.Pd};
+            adv.nseg = nseg; adv.tseg = tseg;
+            ValueSideArgs adIv{v, dO, w.p, w.G, dVT, nullptr, w.dIv, p.B, p.T, p.H, p.d_v, w.Pd};
+            adIv.nseg = nseg; adIv.tseg = tseg;
             adv.single = adIv.single = p.tc_operands == GSA_TC_SINGLE;
             if (g_pair_scans.load(std::memory_order_relaxed) != 0 && rev_pair_supported(adIv, adv, p.m)) {
                 GSA_CUDA(launch_rev_pair_tc(adIv, adv, p.m, w.strong, lanes->stream[0], dev_status));
@@ -754,9 +825,11 @@ gsa_status_t bwd_core(const gsa_params_t* params, int m_active, const void* q, c
         // reversed scans of every segment from empty states, for their end states only (the outputs
         // land in dk / dv, which the real scans overwrite); then the states entering every segment,
         // and dK0 / dV0, by a scan over the segments from the last one down
-        KeySideArgs r1{w.I, w.dz, w.G, q, nullptr, w.Kloc, dk, Bs, Ts, p.H, p.d_k, w.Id, w.Zd, 1};
+        KeySideArgs r1{w.I, w.dz, w.G, q, nullptr, w.Kloc, dk, p.B, p.T, p.H, p.d_k, w.Id, w.Zd, 1};
+        r1.nseg = nseg; r1.tseg = tseg;
         GSA_LAUNCH("segment_dk_states", key_side(p, r1, 1, w.strong, st, dev_status));
-        KeySideArgs r2{w.I, w.p, w.G, dO, nullptr, w.Vloc, dv, Bs, Ts, p.H, p.d_v, w.Id, w.Pd, 1};
+        KeySideArgs r2{w.I, w.p, w.G, dO, nullptr, w.Vloc, dv, p.B, p.T, p.H, p.d_v, w.Id, w.Pd, 1};
+        r2.nseg = nseg; r2.tseg = tseg;
         GSA_LAUNCH("segment_dv_states", key_side(p, r2, 1, w.strong, st, dev_status));
         GSA_LAUNCH("segment_combine", launch_segment_combine(w.seg_decay, w.Kloc, dKT, w.dKend, dK0, p.B, p.H, p.m,
                                                              p.d_k, nseg, 1, st));
@@ -766,10 +839,14 @@ gsa_status_t bwd_core(const gsa_params_t* params, int m_active, const void* q, c
         dK0out = nullptr; dV0out = nullptr;
     }
     // time-reversed runs: dv and dI^v share the state dV~; dk and dI^k share dK~
-    KeySideArgs adv{w.I, w.p, w.G, dO, dVin, dV0out, dv, Bs, Ts, p.H, p.d_v, w.Id, w.Pd};
-    ValueSideArgs adIv{v, dO, w.p, w.G, dVin, nullptr, w.dIv, Bs, Ts, p.H, p.d_v, w.Pd};
-    KeySideArgs adk{w.I, w.dz, w.G, q, dKin, dK0out, dk, Bs, Ts, p.H, p.d_k, w.Id, w.Zd};
-    ValueSideArgs adIk{k, q, w.dz, w.G, dKin, nullptr, w.dIk, Bs, Ts, p.H, p.d_k, w.Zd};
+    KeySideArgs adv{w.I, w.p, w.G, dO, dVin, dV0out, dv, p.B, p.T, p.H, p.d_v, w.Id, w.Pd};
+    adv.nseg = nseg; adv.tseg = tseg;
+    ValueSideArgs adIv{v, dO, w.p, w.G, dVin, nullptr, w.dIv, p.B, p.T, p.H, p.d_v, w.Pd};
+    adIv.nseg = nseg; adIv.tseg = tseg;
+    KeySideArgs adk{w.I, w.dz, w.G, q, dKin, dK0out, dk, p.B, p.T, p.H, p.d_k, w.Id, w.Zd};
+    adk.nseg = nseg; adk.tseg = tseg;
+    ValueSideArgs adIk{k, q, w.dz, w.G, dKin, nullptr, w.dIk, p.B, p.T, p.H, p.d_k, w.Zd};
+    adIk.nseg = nseg; adIk.tseg = tseg;
     // the reversed scans that share a state run as one kernel each (dv with dI^v, dk with dI^k)
     ValueSideArgs pIv = adIv, pIk = adIk;
     KeySideArgs pv = adv, pk = adk;
@@ -824,7 +901,7 @@ gsa_status_t bwd_core(const gsa_params_t* params, int m_active, const void* q, c
     return GSA_OK;
 }
 
-gsa_status_t bwd_impl(const gsa_params_t* params, const void* q, const void* k, const void* v,
+gsa_status_t bwd_impl(const CallParams* params, const void* q, const void* k, const void* v,
                       const float* gate, const float* K0, const float* V0, const float* ok_saved,
                       const void* dO, const float* dKT, const float* dVT, void* dq, void* dk,
                       void* dv, float* dgate, float* dK0, float* dV0, bool gate_is_saved, const void* gate_saved,
@@ -840,7 +917,7 @@ gsa_status_t bwd_impl(const gsa_params_t* params, const void* q, const void* k, 
     const void *q_raw = q, *k_raw = k, *v_raw = v;
     float *dgate_row = nullptr, *colsum = nullptr;
     {
-        const gsa_params_t pi0 = internal_params(*params);
+        const CallParams pi0 = internal_params(*params);
         const size_t before = carve(pi0, GSA_WS_BWD, nullptr).bytes + pad_bytes(*params, GSA_WS_BWD);
         rc = gate_as_f32(*params, GSA_WS_BWD, gate, ws, ws_bytes, before, static_cast<cudaStream_t>(stream), &gate);
         if (rc != GSA_OK) return rc;
@@ -871,8 +948,8 @@ gsa_status_t bwd_impl(const gsa_params_t* params, const void* q, const void* k, 
     if (!pads_slots(*params))
         return finish(bwd_core(params, 0, q, k, v, gate, K0, V0, ok_saved, dO, dKT, dVT, dq, dk, dv, dgate, dK0, dV0,
                                gate_is_saved, gate_saved, gate_saved_bytes, ws, ws_bytes, stream, dev_status));
-    const gsa_params_t& p = *params;
-    const gsa_params_t pi = internal_params(p);
+    const CallParams& p = *params;
+    const CallParams pi = internal_params(p);
     if (ws == nullptr || (reinterpret_cast<uintptr_t>(ws) & 255u) != 0) return GSA_ERR_WORKSPACE;
     const size_t core = carve(pi, GSA_WS_BWD, nullptr).bytes;
     const PadBuffers pb = carve_pad(p, GSA_WS_BWD, static_cast<char*>(ws) + core);
@@ -903,7 +980,9 @@ gsa_status_t gsa_bwd(const gsa_params_t* params, const void* q, const void* k, c
                      const void* dO, const float* dKT, const float* dVT, void* dq, void* dk,
                      void* dv, float* dgate, float* dK0, float* dV0, void* ws, size_t ws_bytes,
                      void* stream, int32_t* dev_status) {
-    return bwd_impl(params, q, k, v, gate, K0, V0, ok_saved, dO, dKT, dVT, dq, dk, dv, dgate, dK0, dV0, false,
+    if (params == nullptr) return GSA_ERR_INVALID_ARG;
+    const CallParams cp(*params);
+    return bwd_impl(&cp, q, k, v, gate, K0, V0, ok_saved, dO, dKT, dVT, dq, dk, dv, dgate, dK0, dV0, false,
                     nullptr, 0, ws, ws_bytes, stream, dev_status);
 }
 
@@ -913,7 +992,9 @@ gsa_status_t gsa_bwd_saved_gate(const gsa_params_t* params, const void* q, const
                                 void* dv, float* dgate, float* dK0, float* dV0, const void* gate_saved,
                                 size_t gate_saved_bytes, void* ws, size_t ws_bytes, void* stream,
                                 int32_t* dev_status) {
-    return bwd_impl(params, q, k, v, gate, K0, V0, ok_saved, dO, dKT, dVT, dq, dk, dv, dgate, dK0, dV0, true,
+    if (params == nullptr) return GSA_ERR_INVALID_ARG;
+    const CallParams cp(*params);
+    return bwd_impl(&cp, q, k, v, gate, K0, V0, ok_saved, dO, dKT, dVT, dq, dk, dv, dgate, dK0, dV0, true,
                     gate_saved, gate_saved_bytes, ws, ws_bytes, stream, dev_status);
 }
 
@@ -950,10 +1031,10 @@ gsa_status_t gsa_shard_states(const gsa_params_t* params, const void* k, const v
     void* oscratch = static_cast<char*>(ws) + w.bytes;      // the scans' token outputs are not wanted: they land here
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // one "segment" per batch element: the whole shard from empty memories, end memories only
-    GSA_CUDA(cudaMemsetAsync(w.strong, 0, sizeof(int) * (size_t)p.B * p.H * segments_of(p), st));
+    GSA_CUDA(cudaMemsetAsync(w.strong, 0, sizeof(int) * (size_t)p.B * p.H, st));
     GSA_LAUNCH("gate_cumsum", launch_gate_cumsum(gate, p.gate_kind, inv_tau(p), w.G, w.I, p.B, p.T, p.H, p.m, chunk_of(p),
-                                                 w.strong, 1, w.Id, p.io == GSA_BF16, st));
-    GSA_LAUNCH("segment_logdecay", launch_segment_logdecay(w.G, logdecay, p.B, p.T, p.H, p.m, 1, chunk_of(p), st));
+                                                 w.strong, 1, p.T, w.Id, p.io == GSA_BF16, st));
+    GSA_LAUNCH("segment_logdecay", launch_segment_logdecay(w.G, logdecay, p.B, p.T, p.H, p.m, 1, p.T, chunk_of(p), st));
     ValueSideArgs s1{k, k, w.I, w.G, nullptr, KT, w.okpart, p.B, p.T, p.H, p.d_k, w.Id, 1};
     GSA_LAUNCH("segment_pass1_states", value_side(p, s1, 0, w.strong, st, dev_status));
     KeySideArgs s2{w.I, w.I, w.G, v, nullptr, VT, oscratch, p.B, p.T, p.H, p.d_v, w.Id, w.Id, 1};

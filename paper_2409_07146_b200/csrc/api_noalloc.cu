@@ -49,15 +49,13 @@ extern "C" GSA_API gsa_status_t gsa_fwd_noalloc(const gsa_params_t* params, cons
                                                 const void* v, const float* gate, const float* K0,
                                                 const float* V0, void* o, float* ok_save, float* KT,
                                                 float* VT, void* stream, int32_t* dev_status) {
-    const size_t need = gsa_workspace_bytes(params, GSA_WS_FWD);
-    if (need == 0) {
+    if (gsa_workspace_bytes(params, GSA_WS_FWD) == 0) {
         // invalid or unsupported params: let the regular entry point name the error
         return gsa_fwd(params, q, k, v, gate, K0, V0, o, ok_save, KT, VT, nullptr, 0, stream, dev_status);
     }
-    if (need > kScratchBytes) return GSA_ERR_WORKSPACE;    // shape too large for the built-in scratch
     void* scratch = nullptr;
     if (scratch_address(&scratch) != cudaSuccess) return GSA_ERR_CUDA;
     // Nothing in the scratch has to start at zero: the forward writes every scratch tensor
     // (G, 1-a, partial logits, logits, p) in full before it reads it.
-    return gsa_fwd(params, q, k, v, gate, K0, V0, o, ok_save, KT, VT, scratch, kScratchBytes, stream, dev_status);
+    return gsa::fwd_within(params, q, k, v, gate, K0, V0, o, ok_save, KT, VT, scratch, kScratchBytes, stream, dev_status);
 }

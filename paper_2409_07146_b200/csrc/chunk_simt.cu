@@ -157,7 +157,8 @@ __global__ void __launch_bounds__(256) value_side_simt_kernel(ValueSideArgs a) {
     __shared__ int s_flag;
 
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-    const int slice = blockIdx.y, bh = blockIdx.x, b = bh / a.H, h = bh % a.H;
+    const ScanSpan span = scan_span(blockIdx.x, a.H, a.T, a.nseg, a.tseg);
+    const int slice = blockIdx.y, bh = blockIdx.x, b = span.b, h = span.h;
     const int d0 = slice * kDS;
     const size_t strideD = (size_t)a.H * a.D, strideM = (size_t)a.H * M;
     const IO* xq = (const IO*)a.xq + ((size_t)b * a.T * a.H + h) * a.D + d0;
@@ -171,13 +172,13 @@ __global__ void __launch_bounds__(256) value_side_simt_kernel(ValueSideArgs a) {
         const int s = idx / kDS, c = idx % kDS;
         sS[c * LM + s] = a.S0 ? a.S0[((size_t)bh * M + s) * a.D + d0 + c] : 0.f;
     }
-    const int nchunks = (a.T + kC - 1) / kC;
+    const int nchunks = (span.t_end - span.t0 + kC - 1) / kC;
     for (int it = 0; it < nchunks; ++it) {
         const int n = REV ? nchunks - 1 - it : it;
-        const int t0 = n * kC;
-        const int valid = min(kC, a.T - t0);
+        const int t0 = span.t0 + n * kC;
+        const int valid = min(kC, span.t_end - t0);
         __syncthreads();
-        load_io_tile<IO>(sXq, xq + (size_t)t0 * strideD, strideD, valid);
+        if (!a.state_only) load_io_tile<IO>(sXq, xq + (size_t)t0 * strideD, strideD, valid);
         load_io_tile<IO>(sXk, xk + (size_t)t0 * strideD, strideD, valid);
         load_slot_tile<M, false>(sW, w + (size_t)t0 * strideM, strideM, valid);
         load_slot_tile<M, true>(sG, G + (size_t)t0 * strideM, strideM, valid);
@@ -192,7 +193,7 @@ __global__ void __launch_bounds__(256) value_side_simt_kernel(ValueSideArgs a) {
             }
         }
         // P = Xq Xk^T, masked to the causal (forward) or anti-causal (reverse) triangle
-        {
+        if (!a.state_only) {
             float acc[4][4] = {};
             mm_nt(sXq, kLd, sXk, kLd, kDS, ty, tx, acc);
 #pragma unroll
@@ -206,7 +207,7 @@ __global__ void __launch_bounds__(256) value_side_simt_kernel(ValueSideArgs a) {
         }
         __syncthreads();
         // out = rowscale * ( colscale * (Xq S) + P W' )
-        {
+        if (!a.state_only) {
             float acc[4][NJ] = {};
             mm_nn<NJ>(sXq, kLd, sS, LM, kDS, ty, tx, acc);
             if (moderate) {
@@ -306,7 +307,8 @@ __global__ void __launch_bounds__(256) key_side_simt_kernel(KeySideArgs a) {
     __shared__ int s_flag;
 
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-    const int slice = blockIdx.y, bh = blockIdx.x, b = bh / a.H, h = bh % a.H;
+    const ScanSpan span = scan_span(blockIdx.x, a.H, a.T, a.nseg, a.tseg);
+    const int slice = blockIdx.y, bh = blockIdx.x, b = span.b, h = span.h;
     const int d0 = slice * kDS;
     const size_t strideD = (size_t)a.H * a.D, strideM = (size_t)a.H * M;
     const float* uq = a.uq + ((size_t)b * a.T * a.H + h) * M;
@@ -319,13 +321,13 @@ __global__ void __launch_bounds__(256) key_side_simt_kernel(KeySideArgs a) {
         const int s = idx / kDS, c = idx % kDS;
         sS[s * kLd + c] = a.S0 ? a.S0[((size_t)bh * M + s) * a.D + d0 + c] : 0.f;
     }
-    const int nchunks = (a.T + kC - 1) / kC;
+    const int nchunks = (span.t_end - span.t0 + kC - 1) / kC;
     for (int it = 0; it < nchunks; ++it) {
         const int n = REV ? nchunks - 1 - it : it;
-        const int t0 = n * kC;
-        const int valid = min(kC, a.T - t0);
+        const int t0 = span.t0 + n * kC;
+        const int valid = min(kC, span.t_end - t0);
         __syncthreads();
-        load_slot_tile<M, false>(sQ, uq + (size_t)t0 * strideM, strideM, valid);
+        if (!a.state_only) load_slot_tile<M, false>(sQ, uq + (size_t)t0 * strideM, strideM, valid);
         load_slot_tile<M, false>(sK, uk + (size_t)t0 * strideM, strideM, valid);
         load_slot_tile<M, true>(sG, G + (size_t)t0 * strideM, strideM, valid);
         load_io_tile<IO>(sV, xv + (size_t)t0 * strideD, strideD, valid);
@@ -342,7 +344,7 @@ __global__ void __launch_bounds__(256) key_side_simt_kernel(KeySideArgs a) {
             }
             __syncthreads();
             float acc[4][4] = {};
-            mm_nt(sQ, LM, sK, LM, M, ty, tx, acc);
+            if (!a.state_only) mm_nt(sQ, LM, sK, LM, M, ty, tx, acc);
 #pragma unroll
             for (int ii = 0; ii < 4; ++ii)
 #pragma unroll
@@ -351,7 +353,7 @@ __global__ void __launch_bounds__(256) key_side_simt_kernel(KeySideArgs a) {
                     const bool keep = REV ? (j >= i) : (j <= i);
                     sA[i * kLd + j] = keep ? acc[ii][jj] : 0.f;
                 }
-        } else {
+        } else if (!a.state_only) {
             float acc[4][4] = {};
             for (int s = 0; s < M; ++s) {
                 float qi[4], gi[4], kj[4], gj[4];
@@ -396,7 +398,7 @@ __global__ void __launch_bounds__(256) key_side_simt_kernel(KeySideArgs a) {
         }
         __syncthreads();
         // out = Q- S + A Xv
-        {
+        if (!a.state_only) {
             float acc[4][4] = {};
             mm_nn<4>(sQ, LM, sS, kLd, M, ty, tx, acc);
             mm_nn<4>(sA, kLd, sV, kLd, kC, ty, tx, acc);
@@ -442,7 +444,7 @@ cudaError_t launch_vs(const ValueSideArgs& a, cudaStream_t st) {
     const size_t smem = sizeof(float) * (3 * kC * kLd + (kDS + 2 * kC) * (M + 4));
     cudaError_t e = set_smem(value_side_simt_kernel<IO, M, REV>, smem);
     if (e != cudaSuccess) return e;
-    dim3 grid(a.B * a.H, a.D / kDS);
+    dim3 grid(a.B * a.nseg * a.H, a.D / kDS);
     value_side_simt_kernel<IO, M, REV><<<grid, 256, smem, st>>>(a);
     return cudaGetLastError();
 }
@@ -451,7 +453,7 @@ cudaError_t launch_ks(const KeySideArgs& a, cudaStream_t st) {
     const size_t smem = sizeof(float) * (3 * kC * (M + 4) + 2 * kC * kLd + M * kLd);
     cudaError_t e = set_smem(key_side_simt_kernel<IO, M, REV>, smem);
     if (e != cudaSuccess) return e;
-    dim3 grid(a.B * a.H, a.D / kDS);
+    dim3 grid(a.B * a.nseg * a.H, a.D / kDS);
     key_side_simt_kernel<IO, M, REV><<<grid, 256, smem, st>>>(a);
     return cudaGetLastError();
 }

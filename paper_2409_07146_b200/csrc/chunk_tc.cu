@@ -226,15 +226,16 @@ value_side_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_cons
 
     const int tid = threadIdx.x, warp = tid >> 5, wq = warp & 3, half = (tid >> 7) & 1, row = tid & 127;
     const int sb = kHS * half;          // this thread's first slot
-    const int bh = blockIdx.x, slice = blockIdx.y, b = bh / a.H, h = bh % a.H;
+    const ScanSpan span = scan_span(blockIdx.x, a.H, a.T, a.nseg, a.tseg);
+    const int bh = blockIdx.x, slice = blockIdx.y, b = span.b, h = span.h;
     const int d0 = slice * kDST;
     const size_t strideM = (size_t)a.H * kM;
     float* obase = a.out + (size_t)slice * a.B * a.T * a.H * kM + ((size_t)b * a.T * a.H + h) * kM;
 
     ctl_init(ctl, tid, warp);
     const uint32_t tmem = ctl->tmem_slot;
-    const int nchunks = (a.T + kCT - 1) / kCT;
-    auto chunk_t0 = [&](int it) { return (REV ? nchunks - 1 - it : it) * kCT; };
+    const int nchunks = (span.t_end - span.t0 + kCT - 1) / kCT;
+    auto chunk_t0 = [&](int it) { return span.t0 + (REV ? nchunks - 1 - it : it) * kCT; };
 
     if (warp == kComputeThreads / 32) {
         // =============================== issuing warp: TMA loads / stores and all MMAs
@@ -371,7 +372,7 @@ value_side_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_cons
         PROF_DECL
         for (int it = 0; it < nchunks; ++it) {
             const int t0 = chunk_t0(it);
-            const int valid = min(kCT, a.T - t0);
+            const int valid = min(kCT, span.t_end - t0);
             PROF_MARK();
             const unsigned char* gt = sG + (2 * (it & 1)) * kPanelB;
             WAIT_OR_ABORT(&ctl->bar_g[it & 1], (it >> 1) & 1);
@@ -632,13 +633,14 @@ key_side_tc_kernel(const __grid_constant__ CUtensorMap mapV, const __grid_consta
 
     const int tid = threadIdx.x, warp = tid >> 5, wq = warp & 3, half = (tid >> 7) & 1, row = tid & 127;
     const int sb = kHS * half;          // this thread's first slot
-    const int bh = blockIdx.x, slice = blockIdx.y, b = bh / a.H, h = bh % a.H;
+    const ScanSpan span = scan_span(blockIdx.x, a.H, a.T, a.nseg, a.tseg);
+    const int bh = blockIdx.x, slice = blockIdx.y, b = span.b, h = span.h;
     const int d0 = slice * kDST;
 
     ctl_init(ctl, tid, warp);
     const uint32_t tmem = ctl->tmem_slot;
-    const int nchunks = (a.T + kCT - 1) / kCT;
-    auto chunk_t0 = [&](int it) { return (REV ? nchunks - 1 - it : it) * kCT; };
+    const int nchunks = (span.t_end - span.t0 + kCT - 1) / kCT;
+    auto chunk_t0 = [&](int it) { return span.t0 + (REV ? nchunks - 1 - it : it) * kCT; };
 
     if (warp == kComputeThreads / 32) {
         // =============================== issuing warp: TMA loads / stores and all MMAs
@@ -755,7 +757,7 @@ key_side_tc_kernel(const __grid_constant__ CUtensorMap mapV, const __grid_consta
         PROF_DECL
         for (int it = 0; it < nchunks; ++it) {
             const int t0 = chunk_t0(it);
-            const int valid = min(kCT, a.T - t0);
+            const int valid = min(kCT, span.t_end - t0);
             (void)t0;
             PROF_MARK();
             WAIT_OR_ABORT(&ctl->bar_g[0], it & 1);
@@ -961,7 +963,7 @@ cudaError_t launch_value_side_tc(const ValueSideArgs& a, int M, int reverse, con
     if (e == cudaSuccess) e = make_tensor_map_bthd(&mw, a.w, a.B, a.T, a.H, kM, kCT, 4);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&mg, a.G, a.B, a.T, a.H, kM, kCT, 4);
     if (e != cudaSuccess) return e;
-    dim3 grid(a.B * a.H, tc_value_side_slices(a.D));
+    dim3 grid(a.B * a.nseg * a.H, tc_value_side_slices(a.D));
 #define GSA_LAUNCH_VS(REVV, FLAGS)                                                                       \
     e = prepare(value_side_tc_kernel<REVV, true>, kSmemValueSide);                                       \
     if (e != cudaSuccess) return e;                                                                      \
@@ -995,7 +997,7 @@ cudaError_t launch_value_side_general(const ValueSideArgs& a, int M, int reverse
     if (e == cudaSuccess) e = make_tensor_map_bthd(&mw, a.w, a.B, a.T, a.H, kM, kCT, 4);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&mg, a.G, a.B, a.T, a.H, kM, kCT, 4);
     if (e != cudaSuccess) return e;
-    dim3 grid(a.B * a.H, tc_value_side_slices(a.D));
+    dim3 grid(a.B * a.nseg * a.H, tc_value_side_slices(a.D));
     if (reverse) {
         e = prepare(value_side_tc_kernel<true, true>, kSmemValueSide);
         if (e != cudaSuccess) return e;
@@ -1018,7 +1020,7 @@ cudaError_t launch_key_side_general(const KeySideArgs& a, int M, int reverse, co
     if (e == cudaSuccess) e = make_tensor_map_bthd(&muk, a.uk, a.B, a.T, a.H, kM, kCT, 4);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&mg, a.G, a.B, a.T, a.H, kM, kCT, 4);
     if (e != cudaSuccess) return e;
-    dim3 grid(a.B * a.H, tc_value_side_slices(a.D));
+    dim3 grid(a.B * a.nseg * a.H, tc_value_side_slices(a.D));
     if (reverse) {
         e = prepare(key_side_tc_kernel<true, true>, kSmemKeySide);
         if (e != cudaSuccess) return e;
@@ -1041,7 +1043,7 @@ cudaError_t launch_key_side_tc(const KeySideArgs& a, int M, int reverse, const i
     if (e == cudaSuccess) e = make_tensor_map_bthd(&muk, a.uk, a.B, a.T, a.H, kM, kCT, 4);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&mg, a.G, a.B, a.T, a.H, kM, kCT, 4);
     if (e != cudaSuccess) return e;
-    dim3 grid(a.B * a.H, tc_value_side_slices(a.D));
+    dim3 grid(a.B * a.nseg * a.H, tc_value_side_slices(a.D));
 #define GSA_LAUNCH_KS(REVV, FLAGS)                                                                       \
     e = prepare(key_side_tc_kernel<REVV, true>, kSmemKeySide);                                           \
     if (e != cudaSuccess) return e;                                                                      \

@@ -132,13 +132,14 @@ value_side_lean_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_co
 
     const int tid = threadIdx.x, warp = tid >> 5, wq = warp & 3, half = (tid >> 7) & 1, row = tid & 127;
     const int sb = kHS * half;          // this thread's first slot
-    const int bh = blockIdx.x, slice = blockIdx.y, b = bh / a.H, h = bh % a.H;
+    const ScanSpan span = scan_span(blockIdx.x, a.H, a.T, a.nseg, a.tseg);
+    const int bh = blockIdx.x, slice = blockIdx.y, b = span.b, h = span.h;
     const int d0 = slice * kDST;
 
     lean_ctl_init(ctl, tid, warp);
     const uint32_t tmem = ctl->tmem_slot;
-    const int nchunks = (a.T + kCT - 1) / kCT;
-    auto chunk_t0 = [&](int n) { return (REV ? nchunks - 1 - n : n) * kCT; };
+    const int nchunks = (span.t_end - span.t0 + kCT - 1) / kCT;
+    auto chunk_t0 = [&](int n) { return span.t0 + (REV ? nchunks - 1 - n : n) * kCT; };
 
     if (warp == kCopyWarp) {
         if (elect_one()) {
@@ -277,7 +278,7 @@ value_side_lean_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_co
 
         // G of the last valid row of chunk n (threads 0..63, one slot each), one chunk ahead
         auto chunk_gc = [&](int n) {
-            const int last = min(chunk_t0(n) + kCT, a.T) - 1;
+            const int last = min(chunk_t0(n) + kCT, span.t_end) - 1;
             return a.G[(((size_t)b * a.T + last) * a.H + h) * kM + tid];
         };
         float g_next = 0.f;
@@ -292,7 +293,6 @@ value_side_lean_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_co
             const int it = n;
             (void)it;
             PROF_MARK();
-            const int valid = min(kCT, a.T - chunk_t0(n));
             const float* egc = ctl->egc[n & 1];
             if (tid < kM && n + 1 < nchunks) {
                 ctl->egc[(n + 1) & 1][tid] = __expf(g_next);
@@ -353,7 +353,6 @@ value_side_lean_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_co
                     *reinterpret_cast<float4*>(panel + swz128(row, c)) =
                         make_float4(vo[4 * c], vo[4 * c + 1], vo[4 * c + 2], vo[4 * c + 3]);
             }
-            (void)valid;
             const bool stop = publish_and_vote(&ctl->bar_out[n & 1], tid, ctl->abort != 0);
             PROF_MARK();
             PROF_DUMP("value_side lean compute");
@@ -392,13 +391,14 @@ key_side_lean_kernel(const __grid_constant__ CUtensorMap mapV, const __grid_cons
 
     const int tid = threadIdx.x, warp = tid >> 5, wq = warp & 3, half = (tid >> 7) & 1, row = tid & 127;
     const int sb = kHS * half;          // this thread's first slot
-    const int bh = blockIdx.x, slice = blockIdx.y, b = bh / a.H, h = bh % a.H;
+    const ScanSpan span = scan_span(blockIdx.x, a.H, a.T, a.nseg, a.tseg);
+    const int bh = blockIdx.x, slice = blockIdx.y, b = span.b, h = span.h;
     const int d0 = slice * kDST;
 
     lean_ctl_init(ctl, tid, warp);
     const uint32_t tmem = ctl->tmem_slot;
-    const int nchunks = (a.T + kCT - 1) / kCT;
-    auto chunk_t0 = [&](int n) { return (REV ? nchunks - 1 - n : n) * kCT; };
+    const int nchunks = (span.t_end - span.t0 + kCT - 1) / kCT;
+    auto chunk_t0 = [&](int n) { return span.t0 + (REV ? nchunks - 1 - n : n) * kCT; };
 
     if (warp == kCopyWarp) {
         if (elect_one()) {
@@ -551,7 +551,7 @@ key_side_lean_kernel(const __grid_constant__ CUtensorMap mapV, const __grid_cons
         // G of the last valid row of chunk n (threads 0..63, one slot each)
         auto chunk_gc = [&](int n) {
             const int t0 = chunk_t0(n);
-            const int last = min(t0 + kCT, a.T) - 1;
+            const int last = min(t0 + kCT, span.t_end) - 1;
             return a.G[(((size_t)b * a.T + last) * a.H + h) * kM + tid];
         };
         float g_next = 0.f;      // gc of chunk n+1, loaded one chunk ahead
@@ -649,7 +649,7 @@ template <bool REV>
 __global__ void __launch_bounds__(kLeanThreads, 1)
 state_scan_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapW,
                   const float* __restrict__ G, const float* __restrict__ S0, float* __restrict__ Send, int T, int H,
-                  int D, const int* __restrict__ strong_flag, int32_t* dev_status) {
+                  int D, int nseg, int tseg, const int* __restrict__ strong_flag, int32_t* dev_status) {
     if (strong_flag[blockIdx.x] != 0) return;       // the general kernel takes this (batch, head)
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -658,7 +658,8 @@ state_scan_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
 
     const int tid = threadIdx.x, warp = tid >> 5, wq = warp & 3, half = (tid >> 7) & 1, row = tid & 127;
     const int sb = kHS * half;          // this thread's first slot
-    const int bh = blockIdx.x, slice = blockIdx.y, b = bh / H, h = bh % H;
+    const ScanSpan span = scan_span(blockIdx.x, H, T, nseg, tseg);
+    const int bh = blockIdx.x, slice = blockIdx.y, b = span.b, h = span.h;
     const int d0 = slice * kDST;
 
     if (tid == 0) {
@@ -681,8 +682,8 @@ state_scan_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem = ctl->tmem_slot;
-    const int nchunks = (T + kCT - 1) / kCT;
-    auto chunk_t0 = [&](int n) { return (REV ? nchunks - 1 - n : n) * kCT; };
+    const int nchunks = (span.t_end - span.t0 + kCT - 1) / kCT;
+    auto chunk_t0 = [&](int n) { return span.t0 + (REV ? nchunks - 1 - n : n) * kCT; };
 
     if (warp == kCopyWarp) {
         if (elect_one()) {
@@ -732,7 +733,7 @@ state_scan_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
         for (int s = 0; s < kHS; ++s) S[s] = (S0 && d0 + row < D) ? S0[((size_t)bh * kM + sb + s) * D + d0 + row] : 0.f;
         // G of the last valid row of chunk n (threads 0..63, one slot each), one chunk ahead
         auto chunk_gc = [&](int n) {
-            const int last = min(chunk_t0(n) + kCT, T) - 1;
+            const int last = min(chunk_t0(n) + kCT, span.t_end) - 1;
             return G[(((size_t)b * T + last) * H + h) * kM + tid];
         };
         float g_next = 0.f;
@@ -784,20 +785,21 @@ constexpr size_t kSmemLeanKey = 1024 + 14 * kPanelB + sizeof(LeanCtl);     // ke
 namespace {
 // X: [B,T,H,D] bf16, the tile that enters the state; W: [B,T,H,2M] bf16 decayed rows [hi | lo]
 cudaError_t launch_state_scan(const void* X, const void* W, const float* G, const float* S0, float* Send, int B, int T,
-                              int H, int D, int reverse, const int* strong_flag, cudaStream_t st, int32_t* dev_status) {
+                              int H, int D, int nseg, int tseg, int reverse, const int* strong_flag, cudaStream_t st,
+                              int32_t* dev_status) {
     CUtensorMap mx, mw;
     cudaError_t e = make_tensor_map_bthd(&mx, X, B, T, H, D, kCT, 2);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&mw, W, B, T, H, 2 * kM, kCT, 2);
     if (e != cudaSuccess) return e;
-    dim3 grid(B * H, tc_value_side_slices(D));
+    dim3 grid(B * nseg * H, tc_value_side_slices(D));
     if (reverse) {
         e = prepare(state_scan_kernel<true>, kSmemStateScan, kLeanThreads);
         if (e != cudaSuccess) return e;
-        state_scan_kernel<true><<<grid, kLeanThreads, kSmemStateScan, st>>>(mx, mw, G, S0, Send, T, H, D, strong_flag, dev_status);
+        state_scan_kernel<true><<<grid, kLeanThreads, kSmemStateScan, st>>>(mx, mw, G, S0, Send, T, H, D, nseg, tseg, strong_flag, dev_status);
     } else {
         e = prepare(state_scan_kernel<false>, kSmemStateScan, kLeanThreads);
         if (e != cudaSuccess) return e;
-        state_scan_kernel<false><<<grid, kLeanThreads, kSmemStateScan, st>>>(mx, mw, G, S0, Send, T, H, D, strong_flag, dev_status);
+        state_scan_kernel<false><<<grid, kLeanThreads, kSmemStateScan, st>>>(mx, mw, G, S0, Send, T, H, D, nseg, tseg, strong_flag, dev_status);
     }
     return cudaGetLastError();
 }
@@ -806,14 +808,15 @@ cudaError_t launch_state_scan(const void* X, const void* W, const float* G, cons
 cudaError_t launch_value_side_lean(const ValueSideArgs& a, int reverse, const int* strong_flag, cudaStream_t st,
                                    int32_t* dev_status) {
     if (a.state_only)
-        return launch_state_scan(a.xk, a.wd, a.G, a.S0, a.Send, a.B, a.T, a.H, a.D, reverse, strong_flag, st, dev_status);
+        return launch_state_scan(a.xk, a.wd, a.G, a.S0, a.Send, a.B, a.T, a.H, a.D, a.nseg, a.tseg, reverse, strong_flag, st,
+                                 dev_status);
     CUtensorMap mq, mk, mw, mo;
     cudaError_t e = make_tensor_map_bthd(&mq, a.xq, a.B, a.T, a.H, a.D, kCT, 2);
     if (e == cudaSuccess) e = make_tensor_map_sliced(&mo, a.out, tc_value_side_slices(a.D), a.B, a.T, a.H, kM, kCT, 4);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&mk, a.xk, a.B, a.T, a.H, a.D, kCT, 2);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&mw, a.wd, a.B, a.T, a.H, 2 * kM, kCT, 2);
     if (e != cudaSuccess) return e;
-    dim3 grid(a.B * a.H, tc_value_side_slices(a.D));
+    dim3 grid(a.B * a.nseg * a.H, tc_value_side_slices(a.D));
     auto launch = [&](auto kernel) {
         cudaError_t e2 = prepare(kernel, kSmemLeanValue, kLeanThreads);
         if (e2 != cudaSuccess) return e2;
@@ -827,14 +830,15 @@ cudaError_t launch_value_side_lean(const ValueSideArgs& a, int reverse, const in
 cudaError_t launch_key_side_lean(const KeySideArgs& a, int reverse, const int* strong_flag, cudaStream_t st,
                                  int32_t* dev_status) {
     if (a.state_only)
-        return launch_state_scan(a.xv, a.uk_d, a.G, a.S0, a.Send, a.B, a.T, a.H, a.D, reverse, strong_flag, st, dev_status);
+        return launch_state_scan(a.xv, a.uk_d, a.G, a.S0, a.Send, a.B, a.T, a.H, a.D, a.nseg, a.tseg, reverse, strong_flag, st,
+                                 dev_status);
     CUtensorMap mv, muq, muk, mo;
     cudaError_t e = make_tensor_map_bthd(&mv, a.xv, a.B, a.T, a.H, a.D, kCT, 2);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&mo, a.out, a.B, a.T, a.H, a.D, kCT, 2);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&muq, a.uq_d, a.B, a.T, a.H, 2 * kM, kCT, 2);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&muk, a.uk_d, a.B, a.T, a.H, 2 * kM, kCT, 2);
     if (e != cudaSuccess) return e;
-    dim3 grid(a.B * a.H, tc_value_side_slices(a.D));
+    dim3 grid(a.B * a.nseg * a.H, tc_value_side_slices(a.D));
     auto launch = [&](auto kernel) {
         cudaError_t e2 = prepare(kernel, kSmemLeanKey, kLeanThreads);
         if (e2 != cudaSuccess) return e2;

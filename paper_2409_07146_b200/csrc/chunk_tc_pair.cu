@@ -67,7 +67,7 @@ rev_pair_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
                 const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapQ,
                 const __grid_constant__ CUtensorMap mapOv, const __grid_constant__ CUtensorMap mapOk,
                 const float* __restrict__ G, const float* __restrict__ S0, float* __restrict__ Send, int T, int H,
-                int D, const int* __restrict__ strong_flag, int32_t* dev_status) {
+                int D, int nseg, int tseg, const int* __restrict__ strong_flag, int32_t* dev_status) {
     if (strong_flag[blockIdx.x] != 0) return;       // the general kernels take this (batch, head)
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -83,7 +83,8 @@ rev_pair_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
 
     const int tid = threadIdx.x, warp = tid >> 5, wq = warp & 3, half = (tid >> 7) & 1, row = tid & 127;
     const int sb = kHS * half;          // this thread's first slot
-    const int bh = blockIdx.x, slice = blockIdx.y, b = bh / H, h = bh % H;
+    const ScanSpan span = scan_span(blockIdx.x, H, T, nseg, tseg);
+    const int bh = blockIdx.x, slice = blockIdx.y, b = span.b, h = span.h;
     const int d0 = slice * kDST;
 
     if (tid == 0) {
@@ -107,8 +108,8 @@ rev_pair_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem = ctl->tmem_slot;
-    const int nchunks = (T + kCT - 1) / kCT;
-    auto chunk_t0 = [&](int n) { return (nchunks - 1 - n) * kCT; };     // from the last chunk down
+    const int nchunks = (span.t_end - span.t0 + kCT - 1) / kCT;
+    auto chunk_t0 = [&](int n) { return span.t0 + (nchunks - 1 - n) * kCT; };     // from the last chunk down
 
     if (warp == kCopyWarp) {
         if (elect_one()) {
@@ -328,7 +329,7 @@ rev_pair_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
 
         // G of the last valid row of chunk n (threads 0..63, one slot each), one chunk ahead
         auto chunk_gc = [&](int n) {
-            const int last = min(chunk_t0(n) + kCT, T) - 1;
+            const int last = min(chunk_t0(n) + kCT, span.t_end) - 1;
             return G[(((size_t)b * T + last) * H + h) * kM + tid];
         };
         float g_next = 0.f;
@@ -444,7 +445,7 @@ constexpr size_t kSmemPair = 1024 + 14 * kPanelB + sizeof(PairCtl);
 }  // namespace
 
 bool rev_pair_supported(const ValueSideArgs& av, const KeySideArgs& ak, int M) {
-    return M == kM && tc_dim_ok(av.D) && av.D == ak.D && av.B == ak.B && av.T == ak.T && av.H == ak.H &&
+    return M == kM && tc_dim_ok(av.D) && av.D == ak.D && av.B == ak.B && av.T == ak.T && av.H == ak.H && av.nseg == ak.nseg && av.tseg == ak.tseg &&
            av.xk == ak.xv && av.wd != nullptr && av.wd == ak.uk_d && ak.uq_d != nullptr && av.G == ak.G &&
            av.S0 == ak.S0 && av.Send == nullptr && !av.state_only && !ak.state_only && av.single == ak.single;
 }
@@ -466,12 +467,12 @@ cudaError_t launch_rev_pair_tc(const ValueSideArgs& av, const KeySideArgs& ak, i
     if (e == cudaSuccess) e = cudaEventRecord(side->fork, st);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(side->stream, side->fork, 0);
     if (e != cudaSuccess) return e;
-    const dim3 grid(av.B * av.H, tc_value_side_slices(av.D));
+    const dim3 grid(av.B * av.nseg * av.H, tc_value_side_slices(av.D));
     auto launch = [&](auto kernel) {
         cudaError_t e2 = prepare(kernel, kSmemPair, kPairThreads);
         if (e2 != cudaSuccess) return e2;
         kernel<<<grid, kPairThreads, kSmemPair, st>>>(mx, my, mw, mq, mov, mok, ak.G, ak.S0, ak.Send, ak.T, ak.H, ak.D,
-                                                      strong_flag, dev_status);
+                                                      ak.nseg, ak.tseg, strong_flag, dev_status);
         return cudaGetLastError();
     };
     e = av.single ? launch(rev_pair_kernel<false>) : launch(rev_pair_kernel<true>);

@@ -87,6 +87,9 @@ struct ValueSideArgs {
     // may leave `out` unwritten where computing it is expensive
     int state_only;
     int single;                       // tensor-core kernels: derived operands as one bf16 value (GSA_TC_SINGLE)
+    // T runs as nseg segments of tseg tokens (the last one shorter), each an independent scan: S0, Send and the
+    // strong-decay flags are then [B, nseg, H, ..]
+    int nseg = 1, tseg = 0;
 };
 struct KeySideArgs {
     const float* uq; const float* uk; const float* G;
@@ -100,7 +103,15 @@ struct KeySideArgs {
     const void* uq_d; const void* uk_d;
     int state_only;                   // as in ValueSideArgs
     int single;                       // as in ValueSideArgs
+    int nseg = 1, tseg = 0;           // likewise
 };
+
+// What scan `bhs` of a launch over B * nseg * H scans works on: batch element, head and the tokens [t0, t_end).
+struct ScanSpan { int b, h, t0, t_end; };
+__host__ __device__ inline ScanSpan scan_span(int bhs, int H, int T, int nseg, int tseg) {
+    const int bs = bhs / H, b = bs / nseg, t0 = (bs - b * nseg) * tseg;
+    return {b, bhs - bs * H, t0, nseg == 1 ? T : (t0 + tseg < T ? t0 + tseg : T)};
+}
 
 // Element-wise replacements of the slot softmax (gsa_act_t other than GSA_ACT_SOFTMAX): f(z) and f'(z).
 __device__ __forceinline__ float slot_act_value(float z, int act) {
@@ -137,7 +148,7 @@ __device__ __forceinline__ float dlog_gate_dlogit(float x, float inv_tau) {
 struct PendingDecay {
     const float* G;
     const int* strong;
-    int T, H, nseg;
+    int T, H, nseg, tseg;             // (tseg: tokens per segment, see ValueSideArgs)
     // != 0: the slot kernel serves ONLY the pairs flagged in `strong` (the fused chunk kernel has done
     // the others on chip): rows with a pending factor are skipped
     int strong_only;
@@ -145,7 +156,7 @@ struct PendingDecay {
     __host__ __device__ bool pending(int b, int r) const {
         if (G == nullptr) return false;
         const int t = r / H, h = r - t * H;
-        const int seg = nseg == 1 ? 0 : t / (T / nseg);
+        const int seg = nseg == 1 ? 0 : t / tseg;
         return strong[(b * nseg + seg) * H + h] == 0;
     }
 };
@@ -158,7 +169,7 @@ struct PendingDecay {
 // hardware base-2 logarithm (absolute error 2^-21.4 for a in [0.5, 1], 3 ulp below), for bf16 io.
 // gate_kind: gsa_gate_t (a, log a, or logits with inv_tau = 1/tau)
 cudaError_t launch_gate_cumsum(const float* gate, int gate_kind, float inv_tau, float* G, float* I,
-                               int B, int T, int H, int M, int chunk, int* strong_flag, int nseg,
+                               int B, int T, int H, int M, int chunk, int* strong_flag, int nseg, int tseg,
                                void* decayed, int fast_log, cudaStream_t st, const int* cu_seqlens = nullptr,
                                int nseq = 0);
 // ABC (Eq. 3-4): write weights phi (cumulative softmax over time of the scores) into I, zeros into G, phi as the
@@ -176,7 +187,7 @@ cudaError_t launch_widen_bf16(const void* in, float* out, size_t n, cudaStream_t
 // log-decay [B,nseg,H,M] from G, and the start memories [B,nseg,H,M,D] of every segment from the
 // end memories of the segments run from empty memories.
 cudaError_t launch_segment_logdecay(const float* G, float* seg_logdecay, int B, int T, int H, int M, int nseg,
-                                    int chunk, cudaStream_t st);
+                                    int tseg, int chunk, cudaStream_t st);
 cudaError_t launch_segment_combine(const float* seg_logdecay, const float* local_end, const float* S0,
                                    float* start, float* final_state, int B, int H, int M, int D, int nseg,
                                    int reverse, cudaStream_t st);
@@ -258,6 +269,10 @@ cudaError_t launch_out_norm_fwd(const void* o, const float* weight, float eps, v
                                 cudaStream_t st);
 cudaError_t launch_out_norm_bwd(const void* o, const void* dy, const float* weight, float eps, void* d_o, float* dw_part,
                                 float* dweight, size_t rows, int N, int io, cudaStream_t st);
+// gsa_fwd in a scratch memory of a fixed size (api.cu)
+gsa_status_t fwd_within(const gsa_params_t* params, const void* q, const void* k, const void* v, const float* gate,
+                        const float* K0, const float* V0, void* o, float* ok_save, float* KT, float* VT, void* ws,
+                        size_t ws_bytes, void* stream, int32_t* dev_status);
 cudaError_t launch_decode(const gsa_params_t& p, const void* q, const void* k, const void* v,
                           const float* gate, float* Ks, float* Vs, void* o, cudaStream_t st);
 

@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
                                                             int gate_kind, float inv_tau,
                                                             float* __restrict__ G,
                                                             float* __restrict__ I, int T, int H,
-                                                            int chunk, int* __restrict__ strong_flag, int nseg,
+                                                            int chunk, int* __restrict__ strong_flag, int nseg, int tseg,
                                                             __nv_bfloat16* __restrict__ decayed, int fast_log,
                                                             const int* __restrict__ cu_seqlens, int nseq) {
     __shared__ double group_sum[16][M];
@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
     // (with segment-parallel scheduling the flags are per (batch, segment, head))
     if (strong_flag != nullptr && grp == (int)blockDim.y - 1 &&
         fmin(before0 + acc0, before1 + acc1) < (double)kFactorisedDecayMin) {
-        const int seg = (int)(((long long)n * chunk) / (T / nseg));
+        const int seg = nseg == 1 ? 0 : n * chunk / tseg;
         strong_flag[(b * nseg + seg) * H + h] = 1;
     }
     // second pass over the same rows: the sums of the groups before as a float pair (value, rest)
@@ -121,20 +121,20 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
 }
 
 cudaError_t launch_gate_cumsum(const float* gate, int gate_kind, float inv_tau, float* G, float* I, int B,
-                               int T, int H, int M, int chunk, int* strong_flag, int nseg, void* decayed, int fast_log,
+                               int T, int H, int M, int chunk, int* strong_flag, int nseg, int tseg, void* decayed, int fast_log,
                                cudaStream_t st, const int* cu_seqlens, int nseq) {
     if (chunk % kCumRows != 0 || chunk / kCumRows > 16 || (M / 2) * (chunk / kCumRows) > 1024) return cudaErrorInvalidValue;
     const int nchunks = (T + chunk - 1) / chunk;
     dim3 block(M / 2, chunk / kCumRows);
     dim3 grid(B * H, nchunks);
     if (M == 128)
-        gate_cumsum_kernel<128><<<grid, block, 0, st>>>(gate, gate_kind, inv_tau, G, I, T, H, chunk, strong_flag, nseg < 1 ? 1 : nseg,
+        gate_cumsum_kernel<128><<<grid, block, 0, st>>>(gate, gate_kind, inv_tau, G, I, T, H, chunk, strong_flag, nseg, tseg,
                                                         static_cast<__nv_bfloat16*>(decayed), fast_log, cu_seqlens, nseq);
     else if (M == 64)
-        gate_cumsum_kernel<64><<<grid, block, 0, st>>>(gate, gate_kind, inv_tau, G, I, T, H, chunk, strong_flag, nseg < 1 ? 1 : nseg,
+        gate_cumsum_kernel<64><<<grid, block, 0, st>>>(gate, gate_kind, inv_tau, G, I, T, H, chunk, strong_flag, nseg, tseg,
                                                        static_cast<__nv_bfloat16*>(decayed), fast_log, cu_seqlens, nseq);
     else
-        gate_cumsum_kernel<32><<<grid, block, 0, st>>>(gate, gate_kind, inv_tau, G, I, T, H, chunk, strong_flag, nseg < 1 ? 1 : nseg,
+        gate_cumsum_kernel<32><<<grid, block, 0, st>>>(gate, gate_kind, inv_tau, G, I, T, H, chunk, strong_flag, nseg, tseg,
                                                        static_cast<__nv_bfloat16*>(decayed), fast_log, cu_seqlens, nseq);
     return cudaGetLastError();
 }
@@ -488,7 +488,7 @@ __global__ void __launch_bounds__(128) gate_grad_local_kernel(
     };
     float2 x[kGG], dI[kGG], gt[kGG];
     load_dI(dIk, nsk, dIv, nsv, base, stride, total, rows, dI);
-    if (pend.G != nullptr && pend.strong[(b * pend.nseg + t0 / (T / pend.nseg)) * H + h] == 0) {
+    if (pend.pending(b, t0 * H + h)) {
         // the time-reversed value_side runs left their row factor exp(-G_i) to this kernel
 #pragma unroll
         for (int i = 0; i < kGG; ++i) gt[i] = ld2(pend.G, i, 0.f);
@@ -533,7 +533,7 @@ __global__ void __launch_bounds__(256) gate_grad_local_tma_kernel(
     const __grid_constant__ CUtensorMap mapGate, const __grid_constant__ CUtensorMap mapG,
     const __grid_constant__ CUtensorMap mapDIk, const __grid_constant__ CUtensorMap mapDIv, int nsk, int nsv,
     int gate_kind, float inv_tau, float* __restrict__ blk_tot, float* __restrict__ dgate, int T, int H, int nblk,
-    const int* __restrict__ strong, int nseg, int32_t* dev_status) {
+    const int* __restrict__ strong, int nseg, int tseg, int32_t* dev_status) {
     using namespace tc;
     constexpr int M = 64;
     extern __shared__ unsigned char gg_smem_raw[];
@@ -588,7 +588,7 @@ __global__ void __launch_bounds__(256) gate_grad_local_tma_kernel(
 #pragma unroll
         for (int i = 0; i < kHalf; ++i) dI[i] += at(4 + sl, i);
     }
-    if (strong != nullptr && strong[(b * nseg + t0 / (T / nseg)) * H + h] == 0) {
+    if (strong != nullptr && strong[(b * nseg + (nseg == 1 ? 0 : t0 / tseg)) * H + h] == 0) {
         // the time-reversed value_side runs left their row factor exp(-G_i) to this kernel
 #pragma unroll
         for (int i = 0; i < kHalf; ++i) dI[i] *= __expf(-at(3, i));
@@ -632,7 +632,7 @@ __global__ void __launch_bounds__(kGGComputeThreads + 32) gate_grad_local_ring_k
     const __grid_constant__ CUtensorMap mapGate, const __grid_constant__ CUtensorMap mapG,
     const __grid_constant__ CUtensorMap mapDIk, const __grid_constant__ CUtensorMap mapDIv, int nsk, int nsv,
     int gate_kind, float inv_tau, float* __restrict__ blk_tot, float* __restrict__ dgate, int T, int H, int BH,
-    int ntile, int nstage, int nblk, const int* __restrict__ strong, int nseg, int32_t* dev_status) {
+    int ntile, int nstage, int nblk, const int* __restrict__ strong, int nseg, int tseg, int32_t* dev_status) {
     using namespace tc;
     constexpr int M = 64;
     extern __shared__ unsigned char gg_smem_raw[];
@@ -713,7 +713,7 @@ __global__ void __launch_bounds__(kGGComputeThreads + 32) gate_grad_local_ring_k
 #pragma unroll
                     for (int i = 0; i < kHalf; ++i) dI[i] += at(4 + sl, i);
                 }
-                if (strong != nullptr && strong[(b * nseg + t0 / (T / nseg)) * H + h] == 0) {
+                if (strong != nullptr && strong[(b * nseg + (nseg == 1 ? 0 : t0 / tseg)) * H + h] == 0) {
                     // the time-reversed value_side runs left their row factor exp(-G_i) to this kernel
 #pragma unroll
                     for (int i = 0; i < kHalf; ++i) dI[i] *= __expf(-at(3, i));
@@ -833,7 +833,7 @@ cudaError_t launch_gate_grad(const float* u, const float* I, const float* dIk_pa
             const int ctas = (int)(total < sm_count ? total : sm_count);      // one persistent CTA per SM
             gate_grad_local_ring_kernel<<<ctas, kGGComputeThreads + 32, smem, st>>>(
                 mu, mi, mg, mG, mk, mv, nsk, nsv, gate_kind, inv_tau, blk_tot, dgate, T, H, BH, ntile, nstage, nblk,
-                pend.G != nullptr ? pend.strong : nullptr, pend.nseg, dev_status);
+                pend.G != nullptr ? pend.strong : nullptr, pend.nseg, pend.tseg, dev_status);
         } else if (staged) {
             const size_t smem = 1024 + (size_t)(4 + nsl) * kGGTileB;
             cudaError_t e = cudaFuncSetAttribute(gate_grad_local_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -842,7 +842,7 @@ cudaError_t launch_gate_grad(const float* u, const float* I, const float* dIk_pa
             dim3 tgrid(B * H, (T + kGGTmaRows - 1) / kGGTmaRows);
             gate_grad_local_tma_kernel<<<tgrid, 256, smem, st>>>(mu, mi, mg, mG, mk, mv, nsk, nsv, gate_kind, inv_tau, blk_tot,
                                                                 dgate, T, H, nblk, pend.G != nullptr ? pend.strong : nullptr,
-                                                                pend.nseg, dev_status);
+                                                                pend.nseg, pend.tseg, dev_status);
         } else {
             gate_grad_local_kernel<64><<<grid, block, 0, st>>>(u, I, dIk_part, nsk, dIv_part, nsv, gate, gate_kind, inv_tau,
                                                                blk_tot, dgate, B, T, H, nblk, pend);
@@ -1045,15 +1045,13 @@ cudaError_t launch_resize_rows(const float* in, float* out, size_t rows, int n_i
 // seg_logdecay[b][r][h][s] = sum over the chunks of segment r of G at the chunk's last row.
 template <int M>
 __global__ void segment_logdecay_kernel(const float* __restrict__ G, float* __restrict__ seg_logdecay, int T, int H,
-                                        int nseg, int chunk) {
+                                        int nseg, int tseg, int chunk) {
     const int s = threadIdx.x, h = blockIdx.y;
     const int b = blockIdx.x / nseg, r = blockIdx.x % nseg;
-    const int Tseg = T / nseg;
+    const int t_begin = r * tseg, t_end = min(T, t_begin + tseg);
     double acc = 0.0;
-    for (int t = r * Tseg + chunk - 1; t < (r + 1) * Tseg; t += chunk)
-        acc += (double)G[(((size_t)b * T + t) * H + h) * M + s];
-    // (a ragged last chunk, possible only when the whole sequence is one segment)
-    if (((r + 1) * Tseg) % chunk != 0) acc += (double)G[(((size_t)b * T + (r + 1) * Tseg - 1) * H + h) * M + s];
+    for (int t = t_begin; t < t_end; t += chunk)      // (the last chunk of the sequence may be a ragged one)
+        acc += (double)G[(((size_t)b * T + min(t + chunk, t_end) - 1) * H + h) * M + s];
     seg_logdecay[(((size_t)b * nseg + r) * H + h) * M + s] = (float)acc;
 }
 
@@ -1074,7 +1072,7 @@ __global__ void segment_combine_kernel(const float* __restrict__ seg_logdecay, c
             const int r = reverse ? nseg - 1 - i : i;
             const size_t pair = ((size_t)b * nseg + r) * H + h;
             start[pair * M * D + idx] = cur;
-            cur = fmaf(cur, __expf(seg_logdecay[pair * M + s]), local_end[pair * M * D + idx]);
+            cur = fmaf(cur, expf(seg_logdecay[pair * M + s]), local_end[pair * M * D + idx]);
         }
         if (final_state) final_state[((size_t)(b * H + h)) * M * D + idx] = cur;
     }
@@ -1109,18 +1107,20 @@ cudaError_t launch_shard_combine(const float* logdecay_all, const float* local_a
 }
 
 cudaError_t launch_segment_logdecay(const float* G, float* seg_logdecay, int B, int T, int H, int M, int nseg,
-                                    int chunk, cudaStream_t st) {
+                                    int tseg, int chunk, cudaStream_t st) {
     dim3 grid(B * nseg, H);
-    if (M == 128) segment_logdecay_kernel<128><<<grid, 128, 0, st>>>(G, seg_logdecay, T, H, nseg, chunk);
-    else if (M == 64) segment_logdecay_kernel<64><<<grid, 64, 0, st>>>(G, seg_logdecay, T, H, nseg, chunk);
-    else segment_logdecay_kernel<32><<<grid, 32, 0, st>>>(G, seg_logdecay, T, H, nseg, chunk);
+    if (M == 128) segment_logdecay_kernel<128><<<grid, 128, 0, st>>>(G, seg_logdecay, T, H, nseg, tseg, chunk);
+    else if (M == 64) segment_logdecay_kernel<64><<<grid, 64, 0, st>>>(G, seg_logdecay, T, H, nseg, tseg, chunk);
+    else segment_logdecay_kernel<32><<<grid, 32, 0, st>>>(G, seg_logdecay, T, H, nseg, tseg, chunk);
     return cudaGetLastError();
 }
 
 cudaError_t launch_segment_combine(const float* seg_logdecay, const float* local_end, const float* S0, float* start,
                                    float* final_state, int B, int H, int M, int D, int nseg, int reverse, cudaStream_t st) {
     dim3 grid(B * H, (M * D + 255) / 256);
-    if (M == 64)
+    if (M == 128)
+        segment_combine_kernel<128><<<grid, 256, 0, st>>>(seg_logdecay, local_end, S0, start, final_state, H, D, nseg, reverse);
+    else if (M == 64)
         segment_combine_kernel<64><<<grid, 256, 0, st>>>(seg_logdecay, local_end, S0, start, final_state, H, D, nseg, reverse);
     else
         segment_combine_kernel<32><<<grid, 256, 0, st>>>(seg_logdecay, local_end, S0, start, final_state, H, D, nseg, reverse);

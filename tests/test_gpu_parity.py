@@ -322,6 +322,18 @@ def test_fwd_tc_segment_parallel_schedule(gate, init):
     print("segment-parallel fwd", errs)
 
 
+@pytest.mark.parametrize("io,T,H,d,m", [("bf16", 2817, 2, 128, 64), ("bf16", 3071, 1, 256, 32), ("f32", 130, 2, 64, 32),
+                                        ("f32", 449, 1, 128, 64), ("f32", 321, 1, 64, 128)])
+def test_segments_of_a_ragged_sequence(io, T, H, d, m):
+    # lengths that no number of segments divides: the last segment is shorter and ends in a ragged chunk (one row
+    # of it at 2817, 449 and 321), everything that crosses a segment boundary in either direction matters
+    data = rand_inputs(T, 1, T, H, d, d, m, io, init=True, final_grads=True)
+    got, gate = run_fwd(data, 1, T, H, d, d, m, io, scale=0.9)
+    check_fwd(data, got, gate, io, scale=0.9, storage=False)
+    gb, rb = run_bwd(data, 1, T, H, d, d, m, io, scale=0.9)
+    check_bwd(gb, rb, TOL[io], tc=io == "bf16")
+
+
 @pytest.mark.parametrize("strong_segment", [False, True])
 @pytest.mark.parametrize("saved", [False, True])
 def test_bwd_tc_segment_parallel_schedule(strong_segment, saved):

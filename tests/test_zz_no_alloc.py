@@ -49,6 +49,21 @@ def test_noalloc_forward_matches_gsa_fwd_twice_in_a_row():
     _run_both(903, 2, 300, 2, 128, 128, 64, "bf16")
 
 
+def test_noalloc_takes_fewer_segments_where_its_scratch_ends():
+    # unsegmented, this shape fits the built-in scratch; the memories of the segments that gsa_fwd cuts it into do not
+    shape = (1, 2900, 4, 512, 512, 64)
+    p = gsa.Params(*shape, io="bf16")
+    assert gsa.gsa_workspace_bytes(p, 0) > gsa.GSA_NOALLOC_MAX_WORKSPACE_BYTES
+    d = rand_inputs(905, *shape, "bf16")
+    q, k, v, gate = to_dev(d["q"], "bf16"), to_dev(d["k"], "bf16"), to_dev(d["v"], "bf16"), to_dev(d["gate"])
+    a = gsa.gsa_fwd(p, q, k, v, gate)
+    b = torch.empty_like(a)
+    gsa.gsa_fwd_noalloc(p, q, k, v, gate, o=b)
+    # two orders of the same fp32 sums, each rounded once to bfloat16: neighbouring values at most (2^-7 of the value)
+    diff = (a.float() - b.float()).abs()
+    assert bool((diff <= 2.0 ** -7 * a.float().abs() + 1e-3 * a.float().std()).all())
+
+
 def test_noalloc_steady_state_call_leaves_device_memory_alone():
     # after the first call on this device (symbol lookup, the library's side stream and events) a
     # call must not change the amount of free device memory
