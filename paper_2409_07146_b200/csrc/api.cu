@@ -897,7 +897,7 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
     // forget-gate gradient: reversed cumulative sum over the whole sequence
     GSA_LAUNCH("gate_grad", launch_gate_grad(w.u, w.I, w.dIk, s.k, w.dIv, s.v, gate, p.gate_kind, inv_tau(p),
                               dKT, w.KT, dVT, w.VT, p.d_k, p.d_v, w.chunk_tot, dgate, p.B, p.T,
-                              p.H, p.m, pend, st, dev_status));
+                              p.H, p.m, pend, st, dev_status, p.cu_seqlens, p.nseq));
     return GSA_OK;
 }
 

@@ -213,7 +213,8 @@ cudaError_t launch_gate_grad(const float* u, const float* I, const float* dIk_pa
                              int gate_kind, float inv_tau, const float* dKT, const float* KT,
                              const float* dVT, const float* VT, int d_k, int d_v,
                              float* chunk_tot, float* dgate, int B, int T, int H, int M,
-                             PendingDecay pend, cudaStream_t st, int32_t* dev_status);
+                             PendingDecay pend, cudaStream_t st, int32_t* dev_status, const int* cu_seqlens = nullptr,
+                             int nseq = 0);
 int gate_grad_blocks(int T);       // entries per (b,h,slot) of launch_gate_grad's scratch
 cudaError_t launch_value_side_simt(const ValueSideArgs& a, int io, int M, int reverse,
                                    cudaStream_t st);

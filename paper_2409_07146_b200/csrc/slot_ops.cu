@@ -42,6 +42,17 @@ __device__ __forceinline__ bool sequence_starts_at(const int* __restrict__ cu, i
     return false;
 }
 
+// What the first token of a packed sequence does to the running log gate.  The memories must lose all they carried
+// there.  With a log gate of -100 (a = 0 in fp32) the chunk's total falls below what the factorised decay can
+// represent and the whole (batch, head, segment) goes to the strong-decay kernels: 1490 us for a training step on 8K
+// tokens of 13 sequences.  A drop of kReset does the same work -- e^-28 is below the 2^-40 at which those kernels
+// leave a sum -- and the chunk stays on the pipelined kernels: 381 us.  Where the chunk's own decay leaves less than
+// that of the factorised range to each of the sequences that begin in it, they share what it leaves, down to
+// kLeastReset each (e^-20 = 2e-9 of the old memories, a thirtieth of an fp32 rounding; more than two sequences in a
+// chunk); below that the chunk takes -100 and the strong-decay kernels.
+constexpr float kReset = 28.f;
+constexpr float kLeastReset = 20.f;
+
 template <int M>
 __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) gate_cumsum_kernel(const float* __restrict__ gate,
                                                             int gate_kind, float inv_tau,
@@ -59,6 +70,16 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
     const size_t stride = (size_t)H * M;
     const size_t base = (((size_t)b * T + t0) * H + h) * M + s;
     float2 g[kCumRows], inps[kCumRows];
+    __shared__ float least_of[M / 2];
+    __shared__ uint32_t starts[4];                // rows of the chunk that begin a packed sequence, one bit each
+    if (cu_seqlens != nullptr) {
+        const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+        if (tid < 4) starts[tid] = 0;
+        __syncthreads();
+        for (int r = tid; r < min(chunk, T - n * chunk); r += blockDim.x * blockDim.y)
+            if (sequence_starts_at(cu_seqlens, nseq, n * chunk + r)) atomicOr(&starts[r >> 5], 1u << (r & 31));
+        __syncthreads();
+    }
 #pragma unroll
     for (int i = 0; i < kCumRows; ++i) {
         // (rows past the end: a = 1, log a = 0)
@@ -75,10 +96,36 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
         }
         g[i].x = fmaxf(g[i].x, kLogGateMin);
         g[i].y = fmaxf(g[i].y, kLogGateMin);
-        // the first token of a packed sequence drops what the memories carried (its decay is exp(-100) = 0 in
-        // fp32); its own write, 1 - a, is untouched.  The chunk is then flagged for the strong-decay kernels.
-        if (sequence_starts_at(cu_seqlens, nseq, t0 + i)) g[i] = make_float2(kLogGateMin, kLogGateMin);
         if (i < rows) *reinterpret_cast<float2*>(I + base + (size_t)i * stride) = inps[i];
+    }
+    // the first token of a packed sequence drops what the memories carried; its own write, 1 - a, is untouched
+    if (cu_seqlens != nullptr && (starts[0] | starts[1] | starts[2] | starts[3]) != 0) {
+        const uint32_t mine = (starts[(grp * kCumRows) >> 5] >> ((grp * kCumRows) & 31)) & ((1u << kCumRows) - 1);
+        float reset = kLogGateMin;
+        if (strong_flag != nullptr) {
+            // the rest of the chunk's decay, of the slot that decays most
+            float own0 = 0.f, own1 = 0.f;
+#pragma unroll
+            for (int i = 0; i < kCumRows; ++i)
+                if (i < rows && !((mine >> i) & 1)) { own0 += g[i].x; own1 += g[i].y; }
+            group_sum[grp][s] = own0;
+            group_sum[grp][s + 1] = own1;
+            __syncthreads();
+            if (grp == 0) {
+                double all0 = 0.0, all1 = 0.0;
+                for (int q = 0; q < (int)blockDim.y; ++q) { all0 += group_sum[q][s]; all1 += group_sum[q][s + 1]; }
+                least_of[threadIdx.x] = fminf((float)all0, (float)all1);
+            }
+            __syncthreads();
+            float least = 0.f;
+            for (int c = 0; c < M / 2; ++c) least = fminf(least, least_of[c]);
+            const int count = __popc(starts[0]) + __popc(starts[1]) + __popc(starts[2]) + __popc(starts[3]);
+            const float each = (least - kFactorisedDecayMin) * 0.999f / (float)count;
+            if (each >= kLeastReset) reset = -fminf(each, kReset);
+        }
+#pragma unroll
+        for (int i = 0; i < kCumRows; ++i)
+            if ((mine >> i) & 1) g[i] = make_float2(reset, reset);
     }
     // running sums: fp32 inside the thread's 8 rows (g becomes the running sum), fp64 across the
     // row groups -- G stays within an ulp of the exact cumulative sum also where strong decay
@@ -386,6 +433,21 @@ cudaError_t launch_slot_softmax_bwd(const float* ok, const float* dp_part, int n
 
 constexpr int kGG = 16;   // rows per thread of the gate-gradient kernels
 
+// Packed sequences: nothing of a later sequence reaches an earlier one, so the running sum restarts at every token
+// that begins a sequence.  (The totals of the later sequences vanish exactly, their roundings do not: without the
+// restart they are all added to every token before.)  Which of the rows [t0, t0 + rows) begin one, a bit each.
+__device__ __forceinline__ uint32_t starts_among(const int* __restrict__ cu, int nseq, int t0, int rows) {
+    uint32_t mask = 0;
+    if (cu == nullptr) return mask;
+    int lo = 1, hi = nseq;                       // the first offset >= max(t0, 1) among cu[1 .. nseq - 1]
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (cu[mid] < max(t0, 1)) lo = mid + 1; else hi = mid;
+    }
+    for (; lo < nseq && cu[lo] < t0 + rows; ++lo) mask |= 1u << (cu[lo] - t0);
+    return mask;
+}
+
 // From the decay-path gradient d(log a) (`run`: what this block knows of it) and the input-gate
 // gradient dI to the gradient with respect to the gate tensor as passed (`gt`):
 //   a       : run / a - dI            (a == 0 leaves no way back from d(log a): only -dI is kept)
@@ -428,14 +490,26 @@ __device__ __forceinline__ void load_dI(const float* __restrict__ dIk, int nsk, 
 template <int M>
 __global__ void __launch_bounds__(M * (M > 64 ? 8 : 16)) gate_grad_scan_kernel(
     float* __restrict__ blk_tot, const float* __restrict__ dKT, const float* __restrict__ KT,
-    const float* __restrict__ dVT, const float* __restrict__ VT, int d_k, int d_v, int nblk) {
+    const float* __restrict__ dVT, const float* __restrict__ VT, int d_k, int d_v, int nblk,
+    const int* __restrict__ cu, int nseq) {
     constexpr int kSeg = M > 64 ? 8 : 16;       // segments of consecutive blocks (threads: M slots x kSeg)
     __shared__ double seg_sum[kSeg][M];
     const int s = threadIdx.x, seg = threadIdx.y, bh = blockIdx.x;
     const int per = (nblk + kSeg - 1) / kSeg;
     const int lo = seg * per, hi = min(nblk, lo + per);
     double sum = 0.0;
-    for (int n = lo; n < hi; ++n) sum += (double)blk_tot[((size_t)bh * nblk + n) * M + s];
+    __shared__ bool restarts[kSeg];              // does a packed sequence begin in the segment?
+    if (cu == nullptr) {
+        for (int n = lo; n < hi; ++n) sum += (double)blk_tot[((size_t)bh * nblk + n) * M + s];
+    } else {
+        bool any = false;
+        for (int n = hi - 1; n >= lo; --n) {
+            const bool here = starts_among(cu, nseq, n * kGG, kGG) != 0;
+            sum = (here ? 0.0 : sum) + (double)blk_tot[((size_t)bh * nblk + n) * M + s];
+            any = any || here;
+        }
+        if (s == 0) restarts[seg] = any;
+    }
     seg_sum[seg][s] = sum;
     // final-memory term <dK~_T[s], K~_T[s]> + <dV~_T[s], V~_T[s]>: a warp per slot, lanes along the row
     __shared__ double final_term[M];
@@ -458,11 +532,16 @@ __global__ void __launch_bounds__(M * (M > 64 ? 8 : 16)) gate_grad_scan_kernel(
     }
     __syncthreads();
     double carry = final_term[s];
-    for (int g = seg + 1; g < kSeg; ++g) carry += seg_sum[g][s];
+    if (cu == nullptr) {
+        for (int g = seg + 1; g < kSeg; ++g) carry += seg_sum[g][s];
+    } else {
+        for (int g = kSeg - 1; g > seg; --g) carry = (restarts[g] ? 0.0 : carry) + seg_sum[g][s];
+    }
     for (int n = hi - 1; n >= lo; --n) {
         const size_t idx = ((size_t)bh * nblk + n) * M + s;
         const float t = blk_tot[idx];
         blk_tot[idx] = (float)carry;
+        if (starts_among(cu, nseq, n * kGG, kGG) != 0) carry = 0.0;
         carry += (double)t;
     }
 }
@@ -474,7 +553,8 @@ template <int M>
 __global__ void __launch_bounds__(128) gate_grad_local_kernel(
     const float* __restrict__ u, const float* __restrict__ I, const float* __restrict__ dIk, int nsk,
     const float* __restrict__ dIv, int nsv, const float* __restrict__ gate, int gate_kind, float inv_tau,
-    float* __restrict__ blk_tot, float* __restrict__ dgate, int B, int T, int H, int nblk, PendingDecay pend) {
+    float* __restrict__ blk_tot, float* __restrict__ dgate, int B, int T, int H, int nblk, PendingDecay pend,
+    const int* __restrict__ cu, int nseq) {
     const int s = 2 * threadIdx.x;                       // this thread's two slots
     const int n = blockIdx.y * blockDim.y + threadIdx.y;
     if (n >= nblk) return;
@@ -506,10 +586,12 @@ __global__ void __launch_bounds__(128) gate_grad_local_kernel(
 #pragma unroll
     for (int i = 0; i < kGG; ++i) gt[i] = ld2(gate, i, 1.f);
     float run0 = 0.f, run1 = 0.f;
+    const uint32_t starts = starts_among(cu, nseq, t0, rows);
 #pragma unroll
     for (int i = kGG - 1; i >= 0; --i) {
         run0 += x[i].x;
         run1 += x[i].y;
+        if ((starts >> i) & 1) run0 = run1 = 0.f;
         if (i < rows) {
             const float2 out = make_float2(gate_grad_out(run0, dI[i].x, gt[i].x, gate_kind, inv_tau),
                                            gate_grad_out(run1, dI[i].y, gt[i].y, gate_kind, inv_tau));
@@ -533,7 +615,7 @@ __global__ void __launch_bounds__(256) gate_grad_local_tma_kernel(
     const __grid_constant__ CUtensorMap mapGate, const __grid_constant__ CUtensorMap mapG,
     const __grid_constant__ CUtensorMap mapDIk, const __grid_constant__ CUtensorMap mapDIv, int nsk, int nsv,
     int gate_kind, float inv_tau, float* __restrict__ blk_tot, float* __restrict__ dgate, int T, int H, int nblk,
-    const int* __restrict__ strong, int nseg, int tseg, int32_t* dev_status) {
+    const int* __restrict__ strong, int nseg, int tseg, const int* __restrict__ cu, int nseq, int32_t* dev_status) {
     using namespace tc;
     constexpr int M = 64;
     extern __shared__ unsigned char gg_smem_raw[];
@@ -601,15 +683,18 @@ __global__ void __launch_bounds__(256) gate_grad_local_tma_kernel(
     const size_t stride = (size_t)H * M;
     const size_t base = (((size_t)b * T + n * kGG + hh * kHalf) * H + h) * M + tx;
     // the early half starts from the total of the late half of its group
+    const uint32_t starts = starts_among(cu, nseq, n * kGG + hh * kHalf, kHalf);
     float tot = 0.f;
 #pragma unroll
-    for (int i = 0; i < kHalf; ++i) tot += x[i];
+    for (int i = 0; i < kHalf; ++i)
+        if ((starts & ((2u << i) - 1)) == 0) tot += x[i];         // (up to the first token that begins a sequence)
     if (hh == 1) late_half[ty][tx] = tot;
     __syncthreads();
     float run = hh == 0 ? late_half[ty][tx] : 0.f;
 #pragma unroll
     for (int i = kHalf - 1; i >= 0; --i) {
         run += x[i];
+        if ((starts >> i) & 1) run = 0.f;
         if (hh * kHalf + i < rows)
             dgate[base + (size_t)i * stride] = gate_grad_out(run, dI[i], at(2, i), gate_kind, inv_tau);
     }
@@ -632,7 +717,7 @@ __global__ void __launch_bounds__(kGGComputeThreads + 32) gate_grad_local_ring_k
     const __grid_constant__ CUtensorMap mapGate, const __grid_constant__ CUtensorMap mapG,
     const __grid_constant__ CUtensorMap mapDIk, const __grid_constant__ CUtensorMap mapDIv, int nsk, int nsv,
     int gate_kind, float inv_tau, float* __restrict__ blk_tot, float* __restrict__ dgate, int T, int H, int BH,
-    int ntile, int nstage, int nblk, const int* __restrict__ strong, int nseg, int tseg, int32_t* dev_status) {
+    int ntile, int nstage, int nblk, const int* __restrict__ strong, int nseg, int tseg, const int* __restrict__ cu, int nseq, int32_t* dev_status) {
     using namespace tc;
     constexpr int M = 64;
     extern __shared__ unsigned char gg_smem_raw[];
@@ -726,9 +811,11 @@ __global__ void __launch_bounds__(kGGComputeThreads + 32) gate_grad_local_ring_k
                 }
             }
             // the early half starts from the total of the late half of its group
+            const uint32_t starts = starts_among(cu, nseq, n * kGG + hh * kHalf, kHalf);
             float tot = 0.f;
 #pragma unroll
-            for (int i = 0; i < kHalf; ++i) tot += x[i];
+            for (int i = 0; i < kHalf; ++i)
+                if ((starts & ((2u << i) - 1)) == 0) tot += x[i];         // (up to the first token that begins a sequence)
             if (hh == 1) late_half[ty][tx] = tot;
             csync();                              // (also: every thread has read its part of the stage)
             if (threadIdx.x == 0)
@@ -738,6 +825,7 @@ __global__ void __launch_bounds__(kGGComputeThreads + 32) gate_grad_local_ring_k
 #pragma unroll
             for (int i = kHalf - 1; i >= 0; --i) {
                 run += x[i];
+                if ((starts >> i) & 1) run = 0.f;
                 if (hh * kHalf + i < rows)
                     dgate[base + (size_t)i * stride] = gate_grad_out(run, dI[i], gt[i], gate_kind, inv_tau);
             }
@@ -761,7 +849,7 @@ __global__ void __launch_bounds__(kGGComputeThreads + 32) gate_grad_local_ring_k
 template <int M>
 __global__ void __launch_bounds__(256) gate_grad_carry_kernel(
     const float* __restrict__ gate, int gate_kind, float inv_tau, const float* __restrict__ blk_carry,
-    float* __restrict__ dgate, int T, int H, int nblk) {
+    float* __restrict__ dgate, int T, int H, int nblk, const int* __restrict__ cu, int nseq) {
     constexpr int kRows = kGG / 2;
     const int s = 2 * threadIdx.x;
     const int n = blockIdx.y * blockDim.y + threadIdx.y;
@@ -771,6 +859,8 @@ __global__ void __launch_bounds__(256) gate_grad_carry_kernel(
     const int rows = max(0, min(kRows, T - t0));
     const size_t stride = (size_t)H * M;
     const size_t base = (((size_t)b * T + t0) * H + h) * M + s;
+    // (what follows the block reaches the rows after its last token that begins a sequence)
+    const int from = 32 - __clz(starts_among(cu, nseq, n * kGG, kGG)) - (int)threadIdx.z * kRows;
     const float2 carry = *reinterpret_cast<const float2*>(blk_carry + ((size_t)bh * nblk + n) * M + s);
     float2 d[kRows], gt[kRows];
 #pragma unroll
@@ -781,7 +871,7 @@ __global__ void __launch_bounds__(256) gate_grad_carry_kernel(
     }
 #pragma unroll
     for (int i = 0; i < kRows; ++i)
-        if (i < rows) {
+        if (i < rows && i >= from) {
             float2 out;
             out.x = d[i].x + gate_grad_carry(carry.x, gt[i].x, gate_kind, inv_tau);
             out.y = d[i].y + gate_grad_carry(carry.y, gt[i].y, gate_kind, inv_tau);
@@ -796,7 +886,7 @@ cudaError_t launch_gate_grad(const float* u, const float* I, const float* dIk_pa
                              int gate_kind, float inv_tau, const float* dKT, const float* KT,
                              const float* dVT, const float* VT, int d_k, int d_v,
                              float* blk_tot, float* dgate, int B, int T, int H, int M,
-                             PendingDecay pend, cudaStream_t st, int32_t* dev_status) {
+                             PendingDecay pend, cudaStream_t st, int32_t* dev_status, const int* cu_seqlens, int nseq) {
     const int nblk = gate_grad_blocks(T);
     dim3 block(M / 2, 256 / M);      // 128 threads: M/2 slot pairs x 16-row blocks
     dim3 grid(B * H, (nblk + block.y - 1) / block.y);
@@ -833,7 +923,7 @@ cudaError_t launch_gate_grad(const float* u, const float* I, const float* dIk_pa
             const int ctas = (int)(total < sm_count ? total : sm_count);      // one persistent CTA per SM
             gate_grad_local_ring_kernel<<<ctas, kGGComputeThreads + 32, smem, st>>>(
                 mu, mi, mg, mG, mk, mv, nsk, nsv, gate_kind, inv_tau, blk_tot, dgate, T, H, BH, ntile, nstage, nblk,
-                pend.G != nullptr ? pend.strong : nullptr, pend.nseg, pend.tseg, dev_status);
+                pend.G != nullptr ? pend.strong : nullptr, pend.nseg, pend.tseg, cu_seqlens, nseq, dev_status);
         } else if (staged) {
             const size_t smem = 1024 + (size_t)(4 + nsl) * kGGTileB;
             cudaError_t e = cudaFuncSetAttribute(gate_grad_local_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -842,23 +932,23 @@ cudaError_t launch_gate_grad(const float* u, const float* I, const float* dIk_pa
             dim3 tgrid(B * H, (T + kGGTmaRows - 1) / kGGTmaRows);
             gate_grad_local_tma_kernel<<<tgrid, 256, smem, st>>>(mu, mi, mg, mG, mk, mv, nsk, nsv, gate_kind, inv_tau, blk_tot,
                                                                 dgate, T, H, nblk, pend.G != nullptr ? pend.strong : nullptr,
-                                                                pend.nseg, pend.tseg, dev_status);
+                                                                pend.nseg, pend.tseg, cu_seqlens, nseq, dev_status);
         } else {
             gate_grad_local_kernel<64><<<grid, block, 0, st>>>(u, I, dIk_part, nsk, dIv_part, nsv, gate, gate_kind, inv_tau,
-                                                               blk_tot, dgate, B, T, H, nblk, pend);
+                                                               blk_tot, dgate, B, T, H, nblk, pend, cu_seqlens, nseq);
         }
-        gate_grad_scan_kernel<64><<<B * H, dim3(64, 16), 0, st>>>(blk_tot, dKT, KT, dVT, VT, d_k, d_v, nblk);
-        gate_grad_carry_kernel<64><<<grid, dim3(block.x, block.y, 2), 0, st>>>(gate, gate_kind, inv_tau, blk_tot, dgate, T, H, nblk);
+        gate_grad_scan_kernel<64><<<B * H, dim3(64, 16), 0, st>>>(blk_tot, dKT, KT, dVT, VT, d_k, d_v, nblk, cu_seqlens, nseq);
+        gate_grad_carry_kernel<64><<<grid, dim3(block.x, block.y, 2), 0, st>>>(gate, gate_kind, inv_tau, blk_tot, dgate, T, H, nblk, cu_seqlens, nseq);
     } else if (M == 128) {
         gate_grad_local_kernel<128><<<grid, block, 0, st>>>(u, I, dIk_part, nsk, dIv_part, nsv, gate, gate_kind, inv_tau,
-                                                            blk_tot, dgate, B, T, H, nblk, pend);
-        gate_grad_scan_kernel<128><<<B * H, dim3(128, 8), 0, st>>>(blk_tot, dKT, KT, dVT, VT, d_k, d_v, nblk);
-        gate_grad_carry_kernel<128><<<grid, dim3(block.x, block.y, 2), 0, st>>>(gate, gate_kind, inv_tau, blk_tot, dgate, T, H, nblk);
+                                                            blk_tot, dgate, B, T, H, nblk, pend, cu_seqlens, nseq);
+        gate_grad_scan_kernel<128><<<B * H, dim3(128, 8), 0, st>>>(blk_tot, dKT, KT, dVT, VT, d_k, d_v, nblk, cu_seqlens, nseq);
+        gate_grad_carry_kernel<128><<<grid, dim3(block.x, block.y, 2), 0, st>>>(gate, gate_kind, inv_tau, blk_tot, dgate, T, H, nblk, cu_seqlens, nseq);
     } else {
         gate_grad_local_kernel<32><<<grid, block, 0, st>>>(u, I, dIk_part, nsk, dIv_part, nsv, gate, gate_kind, inv_tau,
-                                                           blk_tot, dgate, B, T, H, nblk, pend);
-        gate_grad_scan_kernel<32><<<B * H, dim3(32, 16), 0, st>>>(blk_tot, dKT, KT, dVT, VT, d_k, d_v, nblk);
-        gate_grad_carry_kernel<32><<<grid, dim3(block.x, block.y, 2), 0, st>>>(gate, gate_kind, inv_tau, blk_tot, dgate, T, H, nblk);
+                                                           blk_tot, dgate, B, T, H, nblk, pend, cu_seqlens, nseq);
+        gate_grad_scan_kernel<32><<<B * H, dim3(32, 16), 0, st>>>(blk_tot, dKT, KT, dVT, VT, d_k, d_v, nblk, cu_seqlens, nseq);
+        gate_grad_carry_kernel<32><<<grid, dim3(block.x, block.y, 2), 0, st>>>(gate, gate_kind, inv_tau, blk_tot, dgate, T, H, nblk, cu_seqlens, nseq);
     }
     return cudaGetLastError();
 }
