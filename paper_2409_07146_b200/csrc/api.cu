@@ -99,12 +99,14 @@ Slices slices(const gsa_params_t& p) {
 // from empty memories, for their end memories only.  n = 1: off.
 //
 // The rule: the n with the smallest time by this model of a forward, one wave of CTAs at most,
-//     n = 1:  2 (chunks * scan + launch)        n > 1:  2 (chunks / n * (scan + state) + 2 launch) + combine
-// (two scans, two state-only runs, the scans over the segments), if it saves a sixth of the time.  The times per
-// chunk and launch, in tenths of a microsecond, are measured ones.  Forward, us: B = 1, T = 4096, 32 heads of 128 as
-// one segment 227, two 218, four (the rule's) 185; T = 1431, 4 heads of 512 as one (the rule's) 86, six 105 (the
-// launches); training steps: T = 5001, 4 heads of 512: one 500, four 321, nine (the rule's) 289; fp32, B = 2,
-// T = 1024, 4 heads of 256: one 2030, four 782, eight (the rule's) 618.
+//     n = 1:  2 chunks * scan        n > 1:  2 chunks / n * (scan + state) + fixed + each * CTAs
+// (two scans; two state-only runs, the scans over the segments).  Its times, in tenths of a microsecond, are fitted to
+// measured ones; us, forward / training step: T = 1431, 4 heads of 512: one segment 83 / 196, four (the rule's) 72 / 157;
+// T = 2040: 99 / 239 and 70 / 172 (four to nine alike); B = 2, T = 1024, 16 heads of 128: one (the rule's) 73 / 185, four
+// 80 / 207; T = 4096, 32 heads of 128: one 226 / 547, four (the rule's) 176 / 479.  Two segments do not pay on the
+// tensor-core kernels, nor do segments of less than three chunks: B = 4, T = 2047, 4 heads of 512: one 115 / 295, two
+// 126 / 348 (the backward's scans fill the GPU side by side).  CUDA-core kernels: fp32 step, B = 2, T = 1024, 4 heads
+// of 256: one 2030, four 782, eight (the rule's) 618.
 struct Segments { int n, t; };
 Segments segments_of(const CallParams& p) {
     const bool tc = use_tc(p);
@@ -117,18 +119,16 @@ Segments segments_of(const CallParams& p) {
         return {n, p.T / n};
     }
     const int slots = tc || p.m > 64 ? kSMs : 2 * kSMs;       // CTAs of a scan that the GPU holds at a time
-    const int scan = tc ? 27 : (p.m > 64 ? 280 : 150), state = tc ? 10 : scan / 3, launch = tc ? 100 : 50,
-              combine = tc ? 200 : 110;
+    const int scan = tc ? 20 : (p.m > 64 ? 280 : 150), state = tc ? 8 : scan / 3, fixed = tc ? 60 : 210;
     long long most = slots / ctas;
     if (most > p.max_segments) most = p.max_segments;
     if (most > chunks) most = chunks;
-    const long long alone = 2LL * ((long long)chunks * scan + launch);
     int best = chunks;
-    long long best_cost = alone - alone / 6;
-    for (int n = 2; n <= most; ++n) {
+    long long best_cost = 2LL * chunks * scan;
+    for (int n = tc ? 3 : 2; n <= most; ++n) {
         const int per = (chunks + n - 1) / n;
-        const long long cost = 2LL * ((long long)per * (scan + state) + 2 * launch) + combine;
-        if (cost < best_cost) { best = per; best_cost = cost; }
+        const long long cost = 2LL * per * (scan + state) + fixed + (tc ? 3 * ctas * n / 2 : 0);
+        if (cost < best_cost && (per >= 3 || !tc)) { best = per; best_cost = cost; }
     }
     return {(chunks + best - 1) / best, best * chunk};
 }
@@ -263,6 +263,19 @@ cudaError_t key_side(const gsa_params_t& p, const KeySideArgs& a, int reverse, c
         return launch_key_side_tc(b, p.m, reverse, strong, st, dev_status);
     }
     return launch_key_side_simt(a, p.io, p.m, reverse, st);
+}
+
+// End memories (reverse: the gradients entering from the right) of every segment run from empty memories, K and V side.
+// Both primitives update their state alike, S <- decay (S + X^T W), so value_side's arguments serve both.
+struct StateSet { const void* x; const float* w; const void* wd; float* end; };
+cudaError_t state_scans(const gsa_params_t& p, Segments segs, StateSet ks, StateSet vs, const Workspace& w, int reverse,
+                        cudaStream_t st, int32_t* dev_status) {
+    ValueSideArgs a[2] = {{ks.x, ks.x, ks.w, w.G, nullptr, ks.end, nullptr, p.B, p.T, p.H, p.d_k, ks.wd, 1},
+                          {vs.x, vs.x, vs.w, w.G, nullptr, vs.end, nullptr, p.B, p.T, p.H, p.d_v, vs.wd, 1}};
+    for (ValueSideArgs& x : a) { x.nseg = segs.n; x.tseg = segs.t; }
+    if (use_tc(p)) return launch_state_scan_tc(a[0], a[1], reverse, w.strong, st, dev_status);
+    cudaError_t e = launch_value_side_simt(a[0], p.io, p.m, reverse, st);
+    return e == cudaSuccess ? launch_value_side_simt(a[1], p.io, p.m, reverse, st) : e;
 }
 
 // ---- optional per-kernel timing (benchmarks only): while a sink is active on the calling
@@ -547,19 +560,13 @@ gsa_status_t fwd_core(const CallParams* params, int m_active, const void* q, con
         // segments, and the final memories, by a scan over the segments
         GSA_LAUNCH("segment_logdecay", launch_segment_logdecay(w.G, w.seg_decay, p.B, p.T, p.H, p.m, nseg,
                                                                tseg, chunk_of(p), st));
-        ValueSideArgs s1{q, k, w.I, w.G, nullptr, w.Kloc, w.okpart, p.B, p.T, p.H, p.d_k, w.Id, 1};
-        s1.nseg = nseg; s1.tseg = tseg;
-        GSA_LAUNCH("segment_pass1_states", value_side(p, s1, 0, w.strong, st, dev_status));
-        KeySideArgs s2{w.I, w.I, w.G, v, nullptr, w.Vloc, o, p.B, p.T, p.H, p.d_v, w.Id, w.Id, 1};
-        s2.nseg = nseg; s2.tseg = tseg;
-        GSA_LAUNCH("segment_pass2_states", key_side(p, s2, 0, w.strong, st, dev_status));
+        GSA_LAUNCH("segment_states", state_scans(p, segs, StateSet{k, w.I, w.Id, w.Kloc}, StateSet{v, w.I, w.Id, w.Vloc}, w, 0,
+                                                  st, dev_status));
         // (when the backward is to reuse them, the final memories land in the saved block first)
         float* KTc = save_gate ? w.KT : KT;
         float* VTc = save_gate ? w.VT : VT;
-        GSA_LAUNCH("segment_combine", launch_segment_combine(w.seg_decay, w.Kloc, K0, w.Kstart, KTc, p.B, p.H, p.m,
-                                                             p.d_k, nseg, 0, st));
-        GSA_LAUNCH("segment_combine", launch_segment_combine(w.seg_decay, w.Vloc, V0, w.Vstart, VTc, p.B, p.H, p.m,
-                                                             p.d_v, nseg, 0, st));
+        GSA_LAUNCH("segment_combine", launch_segment_combine(w.seg_decay, {w.Kloc, K0, w.Kstart, KTc, p.d_k}, {w.Vloc, V0, w.Vstart, VTc, p.d_v}, p.B,
+                                                             p.H, p.m, nseg, 0, st));
         if (save_gate && KT != nullptr)
             GSA_CUDA(cudaMemcpyAsync(KT, w.KT, sizeof(float) * (size_t)p.B * p.H * p.m * p.d_k, cudaMemcpyDeviceToDevice, st));
         if (save_gate && VT != nullptr)
@@ -589,9 +596,9 @@ gsa_status_t fwd_core(const CallParams* params, int m_active, const void* q, con
         GSA_LAUNCH("fused_fwd", launch_fused_pair(0, q, k, w.Id, v, o, w.G, Kin, Vin, Kout, Vout, p.B * nseg, tseg, p.H, p.d_k,
                                                   p.d_v, p.scale, p.slot_act, ok_save, nullptr, nullptr, nullptr, w.strong,
                                                   st, dev_status));
-        GSA_CUDA(launch_value_side_general(a1, p.m, 0, w.strong, ss, dev_status));
+        GSA_CUDA(launch_value_side_general(a1, w.strong, ss, dev_status));
         GSA_CUDA(launch_slot_softmax_fwd(w.okpart, s.k, p.scale, p.slot_act, ok, w.p, p.B, p.T * p.H, p.m, pend.G, w.Pd, only, ss, m_active));
-        GSA_CUDA(launch_key_side_general(a2, p.m, 0, w.strong, ss, dev_status));
+        GSA_CUDA(launch_key_side_general(a2, w.strong, ss, dev_status));
         if (!g_sink.active) {
             GSA_CUDA(cudaEventRecord(side->join, ss));
             GSA_CUDA(cudaStreamWaitEvent(st, side->join, 0));
@@ -730,16 +737,10 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
     } else if (nseg > 1) {
         GSA_LAUNCH("segment_logdecay", launch_segment_logdecay(w.G, w.seg_decay, p.B, p.T, p.H, p.m, nseg,
                                                                tseg, chunk_of(p), st));
-        ValueSideArgs s1{q, k, w.I, w.G, nullptr, w.Kloc, w.okpart, p.B, p.T, p.H, p.d_k, w.Id, 1};
-        s1.nseg = nseg; s1.tseg = tseg;
-        GSA_LAUNCH("segment_pass1_states", value_side(p, s1, 0, w.strong, st, dev_status));
-        KeySideArgs s2{w.I, w.I, w.G, v, nullptr, w.Vloc, dv, p.B, p.T, p.H, p.d_v, w.Id, w.Id, 1};
-        s2.nseg = nseg; s2.tseg = tseg;
-        GSA_LAUNCH("segment_pass2_states", key_side(p, s2, 0, w.strong, st, dev_status));
-        GSA_LAUNCH("segment_combine", launch_segment_combine(w.seg_decay, w.Kloc, K0, w.Kstart, KTout, p.B, p.H, p.m,
-                                                             p.d_k, nseg, 0, st));
-        GSA_LAUNCH("segment_combine", launch_segment_combine(w.seg_decay, w.Vloc, V0, w.Vstart, VTout, p.B, p.H, p.m,
-                                                             p.d_v, nseg, 0, st));
+        GSA_LAUNCH("segment_states", state_scans(p, segs, StateSet{k, w.I, w.Id, w.Kloc}, StateSet{v, w.I, w.Id, w.Vloc}, w, 0,
+                                                  st, dev_status));
+        GSA_LAUNCH("segment_combine", launch_segment_combine(w.seg_decay, {w.Kloc, K0, w.Kstart, KTout, p.d_k}, {w.Vloc, V0, w.Vstart, VTout, p.d_v}, p.B,
+                                                             p.H, p.m, nseg, 0, st));
         Kin = w.Kstart; Vin = w.Vstart;
         KTout = nullptr; VTout = nullptr;
     }
@@ -787,10 +788,10 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
         GSA_LAUNCH("fused_bwd", launch_fused_pair(1, dO, v, w.Id, k, dq, w.G, Vin, Kin, VTout, KTout, p.B * nseg, tseg, p.H, p.d_v,
                                                   p.d_k, p.scale, p.slot_act, const_cast<float*>(ok), w.u, w.Pd, w.Zd,
                                                   w.strong, st, dev_status));
-        GSA_CUDA(launch_value_side_general(adp, p.m, 0, w.strong, ss, dev_status));
+        GSA_CUDA(launch_value_side_general(adp, w.strong, ss, dev_status));
         GSA_CUDA(launch_slot_softmax_bwd(ok, w.dppart, s.v, p.scale, p.slot_act, w.p, w.dz, w.u, p.B, p.T * p.H, p.m, pend.G,
                                          w.Pd, w.Zd, only, ss, m_active));
-        GSA_CUDA(launch_key_side_general(adq, p.m, 0, w.strong, ss, dev_status));
+        GSA_CUDA(launch_key_side_general(adq, w.strong, ss, dev_status));
         if (!g_sink.active) {
             GSA_CUDA(cudaEventRecord(side->join, ss));
             GSA_CUDA(cudaStreamWaitEvent(st, side->join, 0));
@@ -825,16 +826,10 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
         // reversed scans of every segment from empty states, for their end states only (the outputs
         // land in dk / dv, which the real scans overwrite); then the states entering every segment,
         // and dK0 / dV0, by a scan over the segments from the last one down
-        KeySideArgs r1{w.I, w.dz, w.G, q, nullptr, w.Kloc, dk, p.B, p.T, p.H, p.d_k, w.Id, w.Zd, 1};
-        r1.nseg = nseg; r1.tseg = tseg;
-        GSA_LAUNCH("segment_dk_states", key_side(p, r1, 1, w.strong, st, dev_status));
-        KeySideArgs r2{w.I, w.p, w.G, dO, nullptr, w.Vloc, dv, p.B, p.T, p.H, p.d_v, w.Id, w.Pd, 1};
-        r2.nseg = nseg; r2.tseg = tseg;
-        GSA_LAUNCH("segment_dv_states", key_side(p, r2, 1, w.strong, st, dev_status));
-        GSA_LAUNCH("segment_combine", launch_segment_combine(w.seg_decay, w.Kloc, dKT, w.dKend, dK0, p.B, p.H, p.m,
-                                                             p.d_k, nseg, 1, st));
-        GSA_LAUNCH("segment_combine", launch_segment_combine(w.seg_decay, w.Vloc, dVT, w.dVend, dV0, p.B, p.H, p.m,
-                                                             p.d_v, nseg, 1, st));
+        GSA_LAUNCH("segment_rev_states", state_scans(p, segs, StateSet{q, w.dz, w.Zd, w.Kloc}, StateSet{dO, w.p, w.Pd, w.Vloc}, w,
+                                                      1, st, dev_status));
+        GSA_LAUNCH("segment_combine", launch_segment_combine(w.seg_decay, {w.Kloc, dKT, w.dKend, dK0, p.d_k}, {w.Vloc, dVT, w.dVend, dV0, p.d_v}, p.B,
+                                                             p.H, p.m, nseg, 1, st));
         dKin = w.dKend; dVin = w.dVend;
         dK0out = nullptr; dV0out = nullptr;
     }
@@ -1025,20 +1020,15 @@ gsa_status_t gsa_shard_states(const gsa_params_t* params, const void* k, const v
     const gsa_params_t& p = *params;
     if (ws == nullptr || (reinterpret_cast<uintptr_t>(ws) & 255u) != 0) return GSA_ERR_WORKSPACE;
     Workspace w = carve(p, GSA_WS_FWD, ws);
-    const size_t esz = p.io == GSA_BF16 ? 2 : 4;
-    const size_t obytes = align_up((size_t)p.B * p.T * p.H * p.d_v * esz, 256);
-    if (ws_bytes < w.bytes + obytes) return GSA_ERR_WORKSPACE;
-    void* oscratch = static_cast<char*>(ws) + w.bytes;      // the scans' token outputs are not wanted: they land here
+    if (ws_bytes < gsa_workspace_bytes(params, GSA_WS_SHARD)) return GSA_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // one "segment" per batch element: the whole shard from empty memories, end memories only
     GSA_CUDA(cudaMemsetAsync(w.strong, 0, sizeof(int) * (size_t)p.B * p.H, st));
     GSA_LAUNCH("gate_cumsum", launch_gate_cumsum(gate, p.gate_kind, inv_tau(p), w.G, w.I, p.B, p.T, p.H, p.m, chunk_of(p),
                                                  w.strong, 1, p.T, w.Id, p.io == GSA_BF16, st));
     GSA_LAUNCH("segment_logdecay", launch_segment_logdecay(w.G, logdecay, p.B, p.T, p.H, p.m, 1, p.T, chunk_of(p), st));
-    ValueSideArgs s1{k, k, w.I, w.G, nullptr, KT, w.okpart, p.B, p.T, p.H, p.d_k, w.Id, 1};
-    GSA_LAUNCH("segment_pass1_states", value_side(p, s1, 0, w.strong, st, dev_status));
-    KeySideArgs s2{w.I, w.I, w.G, v, nullptr, VT, oscratch, p.B, p.T, p.H, p.d_v, w.Id, w.Id, 1};
-    GSA_LAUNCH("segment_pass2_states", key_side(p, s2, 0, w.strong, st, dev_status));
+    GSA_LAUNCH("segment_states", state_scans(p, Segments{1, p.T}, StateSet{k, w.I, w.Id, KT}, StateSet{v, w.I, w.Id, VT}, w, 0, st,
+                                              dev_status));
     return GSA_OK;
 }
 

@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(256) key_side_simt_kernel(KeySideArgs a) {
         const int t0 = span.t0 + n * kC;
         const int valid = min(kC, span.t_end - t0);
         __syncthreads();
-        if (!a.state_only) load_slot_tile<M, false>(sQ, uq + (size_t)t0 * strideM, strideM, valid);
+        load_slot_tile<M, false>(sQ, uq + (size_t)t0 * strideM, strideM, valid);
         load_slot_tile<M, false>(sK, uk + (size_t)t0 * strideM, strideM, valid);
         load_slot_tile<M, true>(sG, G + (size_t)t0 * strideM, strideM, valid);
         load_io_tile<IO>(sV, xv + (size_t)t0 * strideD, strideD, valid);
@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(256) key_side_simt_kernel(KeySideArgs a) {
             }
             __syncthreads();
             float acc[4][4] = {};
-            if (!a.state_only) mm_nt(sQ, LM, sK, LM, M, ty, tx, acc);
+            mm_nt(sQ, LM, sK, LM, M, ty, tx, acc);
 #pragma unroll
             for (int ii = 0; ii < 4; ++ii)
 #pragma unroll
@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(256) key_side_simt_kernel(KeySideArgs a) {
                     const bool keep = REV ? (j >= i) : (j <= i);
                     sA[i * kLd + j] = keep ? acc[ii][jj] : 0.f;
                 }
-        } else if (!a.state_only) {
+        } else {
             float acc[4][4] = {};
             for (int s = 0; s < M; ++s) {
                 float qi[4], gi[4], kj[4], gj[4];
@@ -398,7 +398,7 @@ __global__ void __launch_bounds__(256) key_side_simt_kernel(KeySideArgs a) {
         }
         __syncthreads();
         // out = Q- S + A Xv
-        if (!a.state_only) {
+        {
             float acc[4][4] = {};
             mm_nn<4>(sQ, LM, sS, kLd, M, ty, tx, acc);
             mm_nn<4>(sA, kLd, sV, kLd, kC, ty, tx, acc);

@@ -33,7 +33,6 @@ namespace {
 using namespace tc;
 using namespace tcchunk;
 
-constexpr int kFThreads = kComputeThreads + 64;
 constexpr int kFMma = kComputeThreads, kFCopy = kComputeThreads + 32;
 // accumulator columns: first product of either pass (P, then A), state update of either pass (U),
 // first-pass rows (inter + intra, [high | low] weight parts), second-pass rows (inter + intra)
@@ -144,7 +143,7 @@ __device__ __forceinline__ void split2(float x0, float x1, uint32_t& hi, uint32_
 // MODE 0: forward (softmax between the passes); MODE 1: backward (dsoftmax between the passes).
 // NSL: CTAs per cluster = 128-wide slices of either head dimension.
 template <int MODE, int NSL>
-__global__ void __launch_bounds__(kFThreads, 1)
+__global__ void __launch_bounds__(kScanThreads, 1)
 fused_pair_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
                   const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapV,
                   const __grid_constant__ CUtensorMap mapO, FusedArgs a, const int* __restrict__ strong_flag,
@@ -730,12 +729,12 @@ template <int MODE, int NSL>
 cudaError_t launch_one(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mw, const CUtensorMap& mv,
                        const CUtensorMap& mo, const FusedArgs& a, const int* strong, cudaStream_t st, int32_t* dev_status) {
     auto kernel = fused_pair_kernel<MODE, NSL>;
-    cudaError_t e = prepare(kernel, kSmemFused, kFThreads);
+    cudaError_t e = prepare<fused_pair_kernel<MODE, NSL>>(kSmemFused);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3((unsigned)(a.B * a.H * NSL));
-    cfg.blockDim = dim3(kFThreads);
+    cfg.blockDim = dim3(kScanThreads);
     cfg.dynamicSmemBytes = kSmemFused;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];

@@ -17,7 +17,7 @@
 // Tile geometry and the bounded waits are those of the general kernels.
 // The file also holds the state-only scan that segment-parallel scheduling uses for the end
 // memories of every segment (state_scan_kernel, below the two chunk kernels).
-#include "chunk_tc_shared.cuh"
+#include "chunk_tc_general.cuh"
 
 namespace gsa {
 namespace {
@@ -25,8 +25,8 @@ using namespace tc;
 using namespace tcchunk;
 
 // 8 compute warps, one warp whose lane 0 issues every MMA, one warp whose lane 0 requests every
-// tile copy (loads and stores)
-constexpr int kLeanThreads = kComputeThreads + 64;
+// tile copy (loads and stores).  A CTA whose (batch, head) pair holds a strong-decay chunk runs the
+// general scan instead (chunk_tc_general.cuh); w, uq, uk and G as fp32 tiles (mapW32 ..) are for that.
 constexpr int kMmaWarp = kComputeThreads / 32, kCopyWarp = kMmaWarp + 1;   // (entered by one elected lane, see elect_one)
 
 struct LeanCtl {
@@ -116,11 +116,15 @@ constexpr int kLkA = 0, kLkO = 128 /* two buffers of 128 */, kLkU = 384;        
 //   sums the slices of `out` multiplies it in (see PendingDecay), so this kernel needs no G tile.
 // ======================================================================================
 template <bool REV, bool PAIRS>
-__global__ void __launch_bounds__(kLeanThreads, 1)
+__global__ void __launch_bounds__(kScanThreads, 1)
 value_side_lean_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
                        const __grid_constant__ CUtensorMap mapWd, const __grid_constant__ CUtensorMap mapO,
-                       ValueSideArgs a, const int* __restrict__ strong_flag, int32_t* dev_status) {
-    if (strong_flag[blockIdx.x] != 0) return;       // the general kernel takes this (batch, head)
+                       const __grid_constant__ CUtensorMap mapW32, const __grid_constant__ CUtensorMap mapG32,
+                       const __grid_constant__ ValueSideArgs a, const int* __restrict__ strong_flag, int32_t* dev_status) {
+    if (strong_flag[blockIdx.x] != 0) {
+        value_side_general<REV>(mapQ, mapK, mapW32, mapG32, mapO, a, dev_status, blockIdx.y);
+        return;
+    }
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     unsigned char* sX = smem;                        // xq, xk tiles: 2 stages x (2 + 2 panels)  (128 KB)
@@ -372,11 +376,16 @@ value_side_lean_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_co
 //   reverse uq exp(-G), uk exp(G).
 // ======================================================================================
 template <bool REV, bool PAIRS>
-__global__ void __launch_bounds__(kLeanThreads, 1)
+__global__ void __launch_bounds__(kScanThreads, 1)
 key_side_lean_kernel(const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapUq,
                      const __grid_constant__ CUtensorMap mapUk, const __grid_constant__ CUtensorMap mapO,
-                     KeySideArgs a, const int* __restrict__ strong_flag, int32_t* dev_status) {
-    if (strong_flag[blockIdx.x] != 0) return;       // the general kernel takes this (batch, head)
+                     const __grid_constant__ CUtensorMap mapUq32, const __grid_constant__ CUtensorMap mapUk32,
+                     const __grid_constant__ CUtensorMap mapG32, const __grid_constant__ KeySideArgs a,
+                     const int* __restrict__ strong_flag, int32_t* dev_status) {
+    if (strong_flag[blockIdx.x] != 0) {
+        key_side_general<REV>(mapV, mapUq32, mapUk32, mapG32, mapO, a, dev_status);
+        return;
+    }
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     unsigned char* sXv = smem;                       // xv tile, 2 stages of 2 panels              (64 KB)
@@ -645,12 +654,30 @@ struct ScanCtl {
     alignas(16) float egc[2][kM];     // exp(G of the chunk's last valid row), by chunk parity
 };
 
+// The K and the V memories (or their gradients) of a call go in one launch: the first `slices0` slices of the grid are
+// those of set 0, the rest those of set 1.
+struct StateScanArgs {
+    ValueSideArgs set[2];             // (xk, w and wd: the tile that enters the state and its weights; Send)
+    int slices0;
+};
+
 template <bool REV>
-__global__ void __launch_bounds__(kLeanThreads, 1)
-state_scan_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapW,
-                  const float* __restrict__ G, const float* __restrict__ S0, float* __restrict__ Send, int T, int H,
-                  int D, int nseg, int tseg, const int* __restrict__ strong_flag, int32_t* dev_status) {
-    if (strong_flag[blockIdx.x] != 0) return;       // the general kernel takes this (batch, head)
+__global__ void __launch_bounds__(kScanThreads, 1)
+state_scan_kernel(const __grid_constant__ CUtensorMap mapX0, const __grid_constant__ CUtensorMap mapW0,
+                  const __grid_constant__ CUtensorMap mapW32_0, const __grid_constant__ CUtensorMap mapX1,
+                  const __grid_constant__ CUtensorMap mapW1, const __grid_constant__ CUtensorMap mapW32_1,
+                  const __grid_constant__ CUtensorMap mapG32, const __grid_constant__ StateScanArgs sets,
+                  const int* __restrict__ strong_flag, int32_t* dev_status) {
+    const bool second = (int)blockIdx.y >= sets.slices0;
+    const CUtensorMap &mapX = second ? mapX1 : mapX0, &mapW = second ? mapW1 : mapW0;
+    const ValueSideArgs& a = sets.set[second];
+    const int slice = second ? blockIdx.y - sets.slices0 : blockIdx.y;
+    if (strong_flag[blockIdx.x] != 0) {
+        value_side_general<REV>(mapX, mapX, second ? mapW32_1 : mapW32_0, mapG32, mapG32, a, dev_status, slice);
+        return;
+    }
+    const float* __restrict__ G = a.G;
+    const int T = a.T, H = a.H, D = a.D;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     // a stage: X tile (2 panels of 64 channels) and the decayed rows [hi 64 | lo 64] (2 panels)
@@ -658,8 +685,8 @@ state_scan_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
 
     const int tid = threadIdx.x, warp = tid >> 5, wq = warp & 3, half = (tid >> 7) & 1, row = tid & 127;
     const int sb = kHS * half;          // this thread's first slot
-    const ScanSpan span = scan_span(blockIdx.x, H, T, nseg, tseg);
-    const int bh = blockIdx.x, slice = blockIdx.y, b = span.b, h = span.h;
+    const ScanSpan span = scan_span(blockIdx.x, H, T, a.nseg, a.tseg);
+    const int bh = blockIdx.x, b = span.b, h = span.h;
     const int d0 = slice * kDST;
 
     if (tid == 0) {
@@ -730,7 +757,7 @@ state_scan_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
         // =============================== compute threads: S[c = row][s], slots sb .. sb+31
         float S[kHS];
 #pragma unroll
-        for (int s = 0; s < kHS; ++s) S[s] = (S0 && d0 + row < D) ? S0[((size_t)bh * kM + sb + s) * D + d0 + row] : 0.f;
+        for (int s = 0; s < kHS; ++s) S[s] = 0.f;
         // G of the last valid row of chunk n (threads 0..63, one slot each), one chunk ahead
         auto chunk_gc = [&](int n) {
             const int last = min(chunk_t0(n) + kCT, span.t_end) - 1;
@@ -768,9 +795,9 @@ state_scan_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
             // (the barrier inside also publishes the next chunk's egc)
             if (publish_and_vote(&ctl->bar_acc[n & 1], tid, ctl->abort != 0)) break;
         }
-        if (!ctl->abort && Send && d0 + row < D) {
+        if (!ctl->abort && d0 + row < D) {
 #pragma unroll
-            for (int s = 0; s < kHS; ++s) Send[((size_t)bh * kM + sb + s) * D + d0 + row] = S[s];
+            for (int s = 0; s < kHS; ++s) a.Send[((size_t)bh * kM + sb + s) * D + d0 + row] = S[s];
         }
     }
     lean_finish(ctl, tid, warp, tmem, dev_status);
@@ -782,71 +809,90 @@ constexpr size_t kSmemLeanKey = 1024 + 14 * kPanelB + sizeof(LeanCtl);     // ke
 
 }  // namespace
 
-namespace {
-// X: [B,T,H,D] bf16, the tile that enters the state; W: [B,T,H,2M] bf16 decayed rows [hi | lo]
-cudaError_t launch_state_scan(const void* X, const void* W, const float* G, const float* S0, float* Send, int B, int T,
-                              int H, int D, int nseg, int tseg, int reverse, const int* strong_flag, cudaStream_t st,
-                              int32_t* dev_status) {
-    CUtensorMap mx, mw;
-    cudaError_t e = make_tensor_map_bthd(&mx, X, B, T, H, D, kCT, 2);
-    if (e == cudaSuccess) e = make_tensor_map_bthd(&mw, W, B, T, H, 2 * kM, kCT, 2);
+cudaError_t launch_state_scan_tc(const ValueSideArgs& k, const ValueSideArgs& v, int reverse, const int* strong_flag,
+                                 cudaStream_t st, int32_t* dev_status) {
+    StateScanArgs sets{{k, v}, tc_value_side_slices(k.D)};
+    CUtensorMap mx[2], mw[2], mw32[2], mg;
+    cudaError_t e = make_tensor_map_bthd(&mg, k.G, k.B, k.T, k.H, kM, kCT, 4);
+    for (int i = 0; i < 2; ++i) {
+        ValueSideArgs& a = sets.set[i];
+        a.xq = a.xk;
+        a.S0 = nullptr;
+        a.out = nullptr;
+        a.state_only = 1;
+        if (e == cudaSuccess) e = make_tensor_map_bthd(&mx[i], a.xk, a.B, a.T, a.H, a.D, kCT, 2);
+        if (e == cudaSuccess) e = make_tensor_map_bthd(&mw[i], a.wd, a.B, a.T, a.H, 2 * kM, kCT, 2);
+        if (e == cudaSuccess) e = make_tensor_map_bthd(&mw32[i], a.w, a.B, a.T, a.H, kM, kCT, 4);
+    }
     if (e != cudaSuccess) return e;
-    dim3 grid(B * nseg * H, tc_value_side_slices(D));
+    dim3 grid(k.B * k.nseg * k.H, sets.slices0 + tc_value_side_slices(v.D));
+    constexpr size_t smem = kSmemStateScan > kSmemGeneral ? kSmemStateScan : kSmemGeneral;
     if (reverse) {
-        e = prepare(state_scan_kernel<true>, kSmemStateScan, kLeanThreads);
+        e = prepare<state_scan_kernel<true>>(smem);
         if (e != cudaSuccess) return e;
-        state_scan_kernel<true><<<grid, kLeanThreads, kSmemStateScan, st>>>(mx, mw, G, S0, Send, T, H, D, nseg, tseg, strong_flag, dev_status);
+        state_scan_kernel<true><<<grid, kScanThreads, smem, st>>>(mx[0], mw[0], mw32[0], mx[1], mw[1], mw32[1], mg, sets,
+                                                                  strong_flag, dev_status);
     } else {
-        e = prepare(state_scan_kernel<false>, kSmemStateScan, kLeanThreads);
+        e = prepare<state_scan_kernel<false>>(smem);
         if (e != cudaSuccess) return e;
-        state_scan_kernel<false><<<grid, kLeanThreads, kSmemStateScan, st>>>(mx, mw, G, S0, Send, T, H, D, nseg, tseg, strong_flag, dev_status);
+        state_scan_kernel<false><<<grid, kScanThreads, smem, st>>>(mx[0], mw[0], mw32[0], mx[1], mw[1], mw32[1], mg, sets,
+                                                                   strong_flag, dev_status);
     }
     return cudaGetLastError();
 }
-}  // namespace
 
-cudaError_t launch_value_side_lean(const ValueSideArgs& a, int reverse, const int* strong_flag, cudaStream_t st,
-                                   int32_t* dev_status) {
-    if (a.state_only)
-        return launch_state_scan(a.xk, a.wd, a.G, a.S0, a.Send, a.B, a.T, a.H, a.D, a.nseg, a.tseg, reverse, strong_flag, st,
-                                 dev_status);
-    CUtensorMap mq, mk, mw, mo;
+// Is there a kernel for these shapes and operands?
+static bool tc_operands_ok(int M, int D, const void* wd, const void* uq_d, const int* strong_flag) {
+    return M == kM && tc_dim_ok(D) && wd != nullptr && uq_d != nullptr && strong_flag != nullptr;
+}
+
+cudaError_t launch_value_side_tc(const ValueSideArgs& a, int M, int reverse, const int* strong_flag, cudaStream_t st,
+                                 int32_t* dev_status) {
+    if (!tc_operands_ok(M, a.D, a.wd, a.wd, strong_flag)) return cudaErrorNotSupported;
+    CUtensorMap mq, mk, mw, mo, mw32, mg32;
     cudaError_t e = make_tensor_map_bthd(&mq, a.xq, a.B, a.T, a.H, a.D, kCT, 2);
     if (e == cudaSuccess) e = make_tensor_map_sliced(&mo, a.out, tc_value_side_slices(a.D), a.B, a.T, a.H, kM, kCT, 4);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&mk, a.xk, a.B, a.T, a.H, a.D, kCT, 2);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&mw, a.wd, a.B, a.T, a.H, 2 * kM, kCT, 2);
+    if (e == cudaSuccess) e = make_tensor_map_bthd(&mw32, a.w, a.B, a.T, a.H, kM, kCT, 4);
+    if (e == cudaSuccess) e = make_tensor_map_bthd(&mg32, a.G, a.B, a.T, a.H, kM, kCT, 4);
     if (e != cudaSuccess) return e;
     dim3 grid(a.B * a.nseg * a.H, tc_value_side_slices(a.D));
-    auto launch = [&](auto kernel) {
-        cudaError_t e2 = prepare(kernel, kSmemLeanValue, kLeanThreads);
-        if (e2 != cudaSuccess) return e2;
-        kernel<<<grid, kLeanThreads, kSmemLeanValue, st>>>(mq, mk, mw, mo, a, strong_flag, dev_status);
+    constexpr size_t smem = kSmemLeanValue > kSmemGeneral ? kSmemLeanValue : kSmemGeneral;
+    auto launch = [&](auto kernel, cudaError_t ready) {
+        if (ready != cudaSuccess) return ready;
+        kernel<<<grid, kScanThreads, smem, st>>>(mq, mk, mw, mo, mw32, mg32, a, strong_flag, dev_status);
         return cudaGetLastError();
     };
-    if (reverse) return a.single ? launch(value_side_lean_kernel<true, false>) : launch(value_side_lean_kernel<true, true>);
-    return a.single ? launch(value_side_lean_kernel<false, false>) : launch(value_side_lean_kernel<false, true>);
+#define GSA_VALUE(REV, PAIRS) launch(value_side_lean_kernel<REV, PAIRS>, prepare<value_side_lean_kernel<REV, PAIRS>>(smem))
+    if (reverse) return a.single ? GSA_VALUE(true, false) : GSA_VALUE(true, true);
+    return a.single ? GSA_VALUE(false, false) : GSA_VALUE(false, true);
+#undef GSA_VALUE
 }
 
-cudaError_t launch_key_side_lean(const KeySideArgs& a, int reverse, const int* strong_flag, cudaStream_t st,
-                                 int32_t* dev_status) {
-    if (a.state_only)
-        return launch_state_scan(a.xv, a.uk_d, a.G, a.S0, a.Send, a.B, a.T, a.H, a.D, a.nseg, a.tseg, reverse, strong_flag, st,
-                                 dev_status);
-    CUtensorMap mv, muq, muk, mo;
+cudaError_t launch_key_side_tc(const KeySideArgs& a, int M, int reverse, const int* strong_flag, cudaStream_t st,
+                               int32_t* dev_status) {
+    if (!tc_operands_ok(M, a.D, a.uk_d, a.uq_d, strong_flag)) return cudaErrorNotSupported;
+    CUtensorMap mv, muq, muk, mo, muq32, muk32, mg32;
     cudaError_t e = make_tensor_map_bthd(&mv, a.xv, a.B, a.T, a.H, a.D, kCT, 2);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&mo, a.out, a.B, a.T, a.H, a.D, kCT, 2);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&muq, a.uq_d, a.B, a.T, a.H, 2 * kM, kCT, 2);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&muk, a.uk_d, a.B, a.T, a.H, 2 * kM, kCT, 2);
+    if (e == cudaSuccess) e = make_tensor_map_bthd(&muq32, a.uq, a.B, a.T, a.H, kM, kCT, 4);
+    if (e == cudaSuccess) e = make_tensor_map_bthd(&muk32, a.uk, a.B, a.T, a.H, kM, kCT, 4);
+    if (e == cudaSuccess) e = make_tensor_map_bthd(&mg32, a.G, a.B, a.T, a.H, kM, kCT, 4);
     if (e != cudaSuccess) return e;
     dim3 grid(a.B * a.nseg * a.H, tc_value_side_slices(a.D));
-    auto launch = [&](auto kernel) {
-        cudaError_t e2 = prepare(kernel, kSmemLeanKey, kLeanThreads);
-        if (e2 != cudaSuccess) return e2;
-        kernel<<<grid, kLeanThreads, kSmemLeanKey, st>>>(mv, muq, muk, mo, a, strong_flag, dev_status);
+    constexpr size_t smem = kSmemLeanKey > kSmemGeneral ? kSmemLeanKey : kSmemGeneral;
+    auto launch = [&](auto kernel, cudaError_t ready) {
+        if (ready != cudaSuccess) return ready;
+        kernel<<<grid, kScanThreads, smem, st>>>(mv, muq, muk, mo, muq32, muk32, mg32, a, strong_flag, dev_status);
         return cudaGetLastError();
     };
-    if (reverse) return a.single ? launch(key_side_lean_kernel<true, false>) : launch(key_side_lean_kernel<true, true>);
-    return a.single ? launch(key_side_lean_kernel<false, false>) : launch(key_side_lean_kernel<false, true>);
+#define GSA_KEY(REV, PAIRS) launch(key_side_lean_kernel<REV, PAIRS>, prepare<key_side_lean_kernel<REV, PAIRS>>(smem))
+    if (reverse) return a.single ? GSA_KEY(true, false) : GSA_KEY(true, true);
+    return a.single ? GSA_KEY(false, false) : GSA_KEY(false, true);
+#undef GSA_KEY
 }
 
 }  // namespace gsa

@@ -18,14 +18,14 @@
 // Only for (batch, head) pairs without a strong-decay chunk; the flagged ones take the two general
 // kernels.  Geometry, operand pairs (bf16 value + rounding residual) and bounded waits are those
 // of the pipelined single kernels.
-#include "chunk_tc_shared.cuh"
+#include "chunk_tc_general.cuh"
 
 namespace gsa {
 namespace {
 using namespace tc;
 using namespace tcchunk;
 
-constexpr int kPairThreads = kComputeThreads + 64;   // 8 compute warps, an MMA lane, a copy lane
+// 8 compute warps, an MMA lane, a copy lane
 constexpr int kMmaWarp = kComputeThreads / 32, kCopyWarp = kMmaWarp + 1;
 
 struct PairCtl {
@@ -62,13 +62,22 @@ struct PairCtl {
 constexpr int kPcP = 0, kPcA = 128, kPcO2 = 256, kPcU = 384, kPcOI = 448;
 
 template <bool PAIRS>
-__global__ void __launch_bounds__(kPairThreads, 1)
+__global__ void __launch_bounds__(kScanThreads, 1)
 rev_pair_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapY,
                 const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapQ,
                 const __grid_constant__ CUtensorMap mapOv, const __grid_constant__ CUtensorMap mapOk,
-                const float* __restrict__ G, const float* __restrict__ S0, float* __restrict__ Send, int T, int H,
-                int D, int nseg, int tseg, const int* __restrict__ strong_flag, int32_t* dev_status) {
-    if (strong_flag[blockIdx.x] != 0) return;       // the general kernels take this (batch, head)
+                const __grid_constant__ CUtensorMap mapW32, const __grid_constant__ CUtensorMap mapQ32,
+                const __grid_constant__ CUtensorMap mapG32, const __grid_constant__ ValueSideArgs av,
+                const __grid_constant__ KeySideArgs ak, const int* __restrict__ strong_flag, int32_t* dev_status) {
+    if (strong_flag[blockIdx.x] != 0) {             // the two general scans, one after the other
+        if (value_side_general<true, false>(mapY, mapX, mapW32, mapG32, mapOv, av, dev_status, blockIdx.y))
+            key_side_general<true, false>(mapX, mapQ32, mapW32, mapG32, mapOk, ak, dev_status);
+        return;
+    }
+    const float* __restrict__ G = ak.G;
+    const float* __restrict__ S0 = ak.S0;
+    float* __restrict__ Send = ak.Send;
+    const int T = ak.T, H = ak.H, D = ak.D, nseg = ak.nseg, tseg = ak.tseg;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     unsigned char* sX = smem;                        // X tile, 2 stages of 2 panels (64 KB); a stage also holds the
@@ -446,41 +455,33 @@ constexpr size_t kSmemPair = 1024 + 14 * kPanelB + sizeof(PairCtl);
 
 bool rev_pair_supported(const ValueSideArgs& av, const KeySideArgs& ak, int M) {
     return M == kM && tc_dim_ok(av.D) && av.D == ak.D && av.B == ak.B && av.T == ak.T && av.H == ak.H && av.nseg == ak.nseg && av.tseg == ak.tseg &&
-           av.xk == ak.xv && av.wd != nullptr && av.wd == ak.uk_d && ak.uq_d != nullptr && av.G == ak.G &&
-           av.S0 == ak.S0 && av.Send == nullptr && !av.state_only && !ak.state_only && av.single == ak.single;
+           av.xk == ak.xv && av.wd != nullptr && av.wd == ak.uk_d && av.w == ak.uk && ak.uq_d != nullptr && av.G == ak.G &&
+           av.S0 == ak.S0 && av.Send == nullptr && !av.state_only && av.single == ak.single;
 }
 
 cudaError_t launch_rev_pair_tc(const ValueSideArgs& av, const KeySideArgs& ak, int M, const int* strong_flag,
                                cudaStream_t st, int32_t* dev_status) {
     if (!rev_pair_supported(av, ak, M) || strong_flag == nullptr) return cudaErrorNotSupported;
-    CUtensorMap mx, my, mw, mq, mov, mok;
+    CUtensorMap mx, my, mw, mq, mov, mok, mw32, mq32, mg32;
     cudaError_t e = make_tensor_map_bthd(&mx, ak.xv, ak.B, ak.T, ak.H, ak.D, kCT, 2);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&my, av.xq, av.B, av.T, av.H, av.D, kCT, 2);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&mw, av.wd, av.B, av.T, av.H, 2 * kM, kCT, 2);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&mq, ak.uq_d, ak.B, ak.T, ak.H, 2 * kM, kCT, 2);
     if (e == cudaSuccess) e = make_tensor_map_sliced(&mov, av.out, tc_value_side_slices(av.D), av.B, av.T, av.H, kM, kCT, 4);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&mok, ak.out, ak.B, ak.T, ak.H, ak.D, kCT, 2);
-    if (e != cudaSuccess) return e;
-    // the flagged (batch, head) pairs: the two general kernels on the side stream, beside the pair kernel
-    SideLane* side = nullptr;
-    e = side_lane(&side);
-    if (e == cudaSuccess) e = cudaEventRecord(side->fork, st);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(side->stream, side->fork, 0);
+    if (e == cudaSuccess) e = make_tensor_map_bthd(&mw32, av.w, av.B, av.T, av.H, kM, kCT, 4);
+    if (e == cudaSuccess) e = make_tensor_map_bthd(&mq32, ak.uq, ak.B, ak.T, ak.H, kM, kCT, 4);
+    if (e == cudaSuccess) e = make_tensor_map_bthd(&mg32, ak.G, ak.B, ak.T, ak.H, kM, kCT, 4);
     if (e != cudaSuccess) return e;
     const dim3 grid(av.B * av.nseg * av.H, tc_value_side_slices(av.D));
-    auto launch = [&](auto kernel) {
-        cudaError_t e2 = prepare(kernel, kSmemPair, kPairThreads);
-        if (e2 != cudaSuccess) return e2;
-        kernel<<<grid, kPairThreads, kSmemPair, st>>>(mx, my, mw, mq, mov, mok, ak.G, ak.S0, ak.Send, ak.T, ak.H, ak.D,
-                                                      ak.nseg, ak.tseg, strong_flag, dev_status);
+    constexpr size_t smem = kSmemPair > kSmemGeneral ? kSmemPair : kSmemGeneral;
+    auto launch = [&](auto kernel, cudaError_t ready) {
+        if (ready != cudaSuccess) return ready;
+        kernel<<<grid, kScanThreads, smem, st>>>(mx, my, mw, mq, mov, mok, mw32, mq32, mg32, av, ak, strong_flag, dev_status);
         return cudaGetLastError();
     };
-    e = av.single ? launch(rev_pair_kernel<false>) : launch(rev_pair_kernel<true>);
-    if (e == cudaSuccess) e = launch_value_side_general(av, M, 1, strong_flag, side->stream, dev_status);
-    if (e == cudaSuccess) e = launch_key_side_general(ak, M, 1, strong_flag, side->stream, dev_status);
-    if (e == cudaSuccess) e = cudaEventRecord(side->join, side->stream);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, side->join, 0);
-    return e;
+    return av.single ? launch(rev_pair_kernel<false>, prepare<rev_pair_kernel<false>>(smem))
+                     : launch(rev_pair_kernel<true>, prepare<rev_pair_kernel<true>>(smem));
 }
 
 }  // namespace gsa

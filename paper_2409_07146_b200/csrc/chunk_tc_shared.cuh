@@ -4,6 +4,8 @@
 #pragma once
 #include <stdio.h>
 
+#include <atomic>
+
 #include "common.cuh"
 #include "tc_common.cuh"
 
@@ -17,7 +19,8 @@ constexpr int kM = 64;                 // slots
 constexpr int kPanelB = 128 * 128;     // bytes of a 128-row operand panel
 constexpr uint32_t kTmemCols = 512;
 constexpr int kComputeThreads = 256;   // 8 warps: two threads per chunk row
-constexpr int kThreads = kComputeThreads + 32;   // + the issuing warp (TMA and MMA), one lane active
+// + two warps of one active lane each: MMA issue and tile copies (the general scans use the first for both)
+constexpr int kScanThreads = kComputeThreads + 64;
 constexpr int kHS = kM / 2;            // slots per thread
 
 // accumulator columns
@@ -218,15 +221,24 @@ __device__ __forceinline__ void mask_row_in_tmem(uint32_t tmem, int wq, int row,
         if (!mbar_wait(bar, parity)) ctl->abort = 1;        \
     } while (0)
 
-template <typename K>
-cudaError_t prepare(K kernel, size_t smem, int threads = kThreads) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+// What a kernel needs once per device before its first launch: its shared memory, and the check that no second CTA
+// fits beside it -- each CTA takes the whole tensor memory of its SM.
+template <auto kernel>
+cudaError_t prepare(size_t smem) {
+    static std::atomic<uint64_t> done{0};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    // each CTA takes the whole tensor memory of its SM: make sure no second CTA can be co-resident
+    const uint64_t bit = dev < 64 ? 1ull << dev : 0;
+    if ((done.load(std::memory_order_acquire) & bit) != 0) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kScanThreads, smem);
     if (e != cudaSuccess) return e;
-    return per_sm == 1 ? cudaSuccess : cudaErrorLaunchOutOfResources;
+    if (per_sm != 1) return cudaErrorLaunchOutOfResources;
+    done.fetch_or(bit, std::memory_order_release);
+    return cudaSuccess;
 }
 
 }  // namespace tcchunk

@@ -83,8 +83,7 @@ struct ValueSideArgs {
     // tensor-core path: the weights already multiplied by their decay factor, bf16 rows of 2M
     // [high part | rounding residual] of w exp(-G) (forward) or w exp(G) (reverse); nullable
     const void* wd;
-    // only the end state matters to the caller (first run of the segment-parallel forward): kernels
-    // may leave `out` unwritten where computing it is expensive
+    // only the end state matters to the caller (the state runs of segment-parallel scheduling): `out` is not written
     int state_only;
     int single;                       // tensor-core kernels: derived operands as one bf16 value (GSA_TC_SINGLE)
     // T runs as nseg segments of tseg tokens (the last one shorter), each an independent scan: S0, Send and the
@@ -101,7 +100,6 @@ struct KeySideArgs {
     // tensor-core path: decayed bf16 rows of 2M (the first M are used): forward uq exp(G) and
     // uk exp(-G), reverse uq exp(-G) and uk exp(G); nullable (both or neither)
     const void* uq_d; const void* uk_d;
-    int state_only;                   // as in ValueSideArgs
     int single;                       // as in ValueSideArgs
     int nseg = 1, tseg = 0;           // likewise
 };
@@ -188,8 +186,9 @@ cudaError_t launch_widen_bf16(const void* in, float* out, size_t n, cudaStream_t
 // end memories of the segments run from empty memories.
 cudaError_t launch_segment_logdecay(const float* G, float* seg_logdecay, int B, int T, int H, int M, int nseg,
                                     int tseg, int chunk, cudaStream_t st);
-cudaError_t launch_segment_combine(const float* seg_logdecay, const float* local_end, const float* S0,
-                                   float* start, float* final_state, int B, int H, int M, int D, int nseg,
+// one side's memories in launch_segment_combine (S0 and final_state nullable); the K and the V side go in one launch
+struct CombineSet { const float* local_end; const float* S0; float* start; float* final_state; int D; };
+cudaError_t launch_segment_combine(const float* seg_logdecay, CombineSet k, CombineSet v, int B, int H, int M, int nseg,
                                    int reverse, cudaStream_t st);
 cudaError_t launch_shard_combine(const float* logdecay_all, const float* local_all, const float* S0, float* start,
                                  float* final_state, int B, int H, int M, int D, int nshard, int rank, int reverse,
@@ -229,17 +228,13 @@ cudaError_t launch_value_side_tc(const ValueSideArgs& a, int M, int reverse, con
                                  cudaStream_t st, int32_t* dev_status);
 cudaError_t launch_key_side_tc(const KeySideArgs& a, int M, int reverse, const int* strong_flag,
                                cudaStream_t st, int32_t* dev_status);
-// the pipelined kernels for the (batch, head) pairs without a strong-decay chunk (strong_flag 0);
-// they need the pre-decayed operands of the argument structs
-cudaError_t launch_value_side_lean(const ValueSideArgs& a, int reverse, const int* strong_flag, cudaStream_t st,
-                                   int32_t* dev_status);
-cudaError_t launch_key_side_lean(const KeySideArgs& a, int reverse, const int* strong_flag, cudaStream_t st,
-                                 int32_t* dev_status);
-// only the general kernel of a scan (the flagged pairs), on the given stream
-cudaError_t launch_value_side_general(const ValueSideArgs& a, int M, int reverse, const int* strong_flag,
-                                      cudaStream_t st, int32_t* dev_status);
-cudaError_t launch_key_side_general(const KeySideArgs& a, int M, int reverse, const int* strong_flag,
-                                    cudaStream_t st, int32_t* dev_status);
+// the general scan as a launch of its own, for the flagged pairs (beside the fused kernel; forward direction)
+cudaError_t launch_value_side_general(const ValueSideArgs& a, const int* strong_flag, cudaStream_t st, int32_t* dev_status);
+cudaError_t launch_key_side_general(const KeySideArgs& a, const int* strong_flag, cudaStream_t st, int32_t* dev_status);
+// end memories only, from empty ones, of the K and the V side in one launch: xk, w and wd of each set are the tile that
+// enters the state and its weights (key_side: xv, uk, uk_d)
+cudaError_t launch_state_scan_tc(const ValueSideArgs& k, const ValueSideArgs& v, int reverse, const int* strong_flag,
+                                 cudaStream_t st, int32_t* dev_status);
 // The two reversed scans that share a state (dv with dI^v, dk with dI^k) as one kernel
 // (chunk_tc_pair.cu): av / ak are the arguments the single reversed scans would get.
 bool rev_pair_supported(const ValueSideArgs& av, const KeySideArgs& ak, int M);

@@ -1150,21 +1150,24 @@ __global__ void segment_logdecay_kernel(const float* __restrict__ G, float* __re
 // reverse: the same from the last segment down (time-reversed scans: start[r] is the state that
 // enters segment r from the right, S0 the one after the last token, final the one before the first).
 template <int M>
-__global__ void segment_combine_kernel(const float* __restrict__ seg_logdecay, const float* __restrict__ local_end,
-                                       const float* __restrict__ S0, float* __restrict__ start,
-                                       float* __restrict__ final_state, int H, int D, int nseg, int reverse) {
+__global__ void segment_combine_kernel(const float* __restrict__ seg_logdecay, CombineSet k, CombineSet v, int H, int nseg,
+                                       int reverse) {
     const int b = blockIdx.x / H, h = blockIdx.x % H;
-    const int idx = blockIdx.y * blockDim.x + threadIdx.x;
-    if (idx < M * D) {
-        const int s = idx / D;
-        float cur = S0 ? S0[((size_t)(b * H + h)) * M * D + idx] : 0.f;
+    int idx = blockIdx.y * blockDim.x + threadIdx.x;
+    const bool second = idx >= M * k.D;
+    if (second) idx -= M * k.D;
+    const CombineSet& a = second ? v : k;
+    if (idx < M * a.D) {
+        const int s = idx / a.D;
+        float cur = a.S0 ? a.S0[((size_t)(b * H + h)) * M * a.D + idx] : 0.f;
+#pragma unroll 4
         for (int i = 0; i < nseg; ++i) {
             const int r = reverse ? nseg - 1 - i : i;
             const size_t pair = ((size_t)b * nseg + r) * H + h;
-            start[pair * M * D + idx] = cur;
-            cur = fmaf(cur, expf(seg_logdecay[pair * M + s]), local_end[pair * M * D + idx]);
+            a.start[pair * M * a.D + idx] = cur;
+            cur = fmaf(cur, expf(seg_logdecay[pair * M + s]), a.local_end[pair * M * a.D + idx]);
         }
-        if (final_state) final_state[((size_t)(b * H + h)) * M * D + idx] = cur;
+        if (a.final_state) a.final_state[((size_t)(b * H + h)) * M * a.D + idx] = cur;
     }
 }
 
@@ -1205,15 +1208,12 @@ cudaError_t launch_segment_logdecay(const float* G, float* seg_logdecay, int B, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_segment_combine(const float* seg_logdecay, const float* local_end, const float* S0, float* start,
-                                   float* final_state, int B, int H, int M, int D, int nseg, int reverse, cudaStream_t st) {
-    dim3 grid(B * H, (M * D + 255) / 256);
-    if (M == 128)
-        segment_combine_kernel<128><<<grid, 256, 0, st>>>(seg_logdecay, local_end, S0, start, final_state, H, D, nseg, reverse);
-    else if (M == 64)
-        segment_combine_kernel<64><<<grid, 256, 0, st>>>(seg_logdecay, local_end, S0, start, final_state, H, D, nseg, reverse);
-    else
-        segment_combine_kernel<32><<<grid, 256, 0, st>>>(seg_logdecay, local_end, S0, start, final_state, H, D, nseg, reverse);
+cudaError_t launch_segment_combine(const float* seg_logdecay, CombineSet k, CombineSet v, int B, int H, int M, int nseg,
+                                   int reverse, cudaStream_t st) {
+    dim3 grid(B * H, (M * (k.D + v.D) + 255) / 256);
+    if (M == 128) segment_combine_kernel<128><<<grid, 256, 0, st>>>(seg_logdecay, k, v, H, nseg, reverse);
+    else if (M == 64) segment_combine_kernel<64><<<grid, 256, 0, st>>>(seg_logdecay, k, v, H, nseg, reverse);
+    else segment_combine_kernel<32><<<grid, 256, 0, st>>>(seg_logdecay, k, v, H, nseg, reverse);
     return cudaGetLastError();
 }
 
