@@ -37,9 +37,10 @@
  *     workspaces.
  *   - Supported: d_k, d_v in {64,128,256,512}; m in {32,64,128}; B,T,H >= 1
  *     (T need not be a multiple of the chunk; the tail chunk is masked).  bf16 io
- *     with m in {32,64} runs on the tensor-core kernels (m = 32 on their 64-slot
- *     tiles with the upper half padded; d = 64 on half a 128-wide slice); fp32 io
- *     and m = 128 run on the fp32 CUDA-core kernels.
+ *     runs on the tensor-core kernels (m = 32 on 64-slot tiles with the upper half
+ *     padded; m = 128 on kernels of its own, not with GSA_GATE_ABC nor by name with
+ *     GSA_IMPL_TC; d = 64 on half a 128-wide slice); fp32 io runs on the fp32
+ *     CUDA-core kernels.
  *   - Errors are return codes; arguments are validated before anything is
  *     launched and outputs are untouched when a call fails validation.
  *     No entry point throws, aborts or prints.

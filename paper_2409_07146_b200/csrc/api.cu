@@ -52,6 +52,11 @@ gsa_status_t check_params(const gsa_params_t* p, bool need_T) {
 
 // Does this call run the tensor-core chunk kernels?
 bool use_tc(const gsa_params_t& p);
+// ... those for 128 slots (chunk_tc_wide.cu)?
+bool use_wide(const gsa_params_t& p) {
+    return p.m == 128 && p.impl == GSA_IMPL_AUTO && p.io == GSA_BF16 && p.gate_kind != GSA_GATE_ABC && tc_dim_ok(p.d_k) &&
+           tc_dim_ok(p.d_v);
+}
 // The parameters of a call as the host code passes them on: the caller's, and how many segments its scans may be
 // cut into (see segments_of; less than that rule would take only where the scratch memory is a fixed one).
 struct CallParams : gsa_params_t {
@@ -59,8 +64,8 @@ struct CallParams : gsa_params_t {
     CallParams(const gsa_params_t& p, int max_seg = 1 << 30) : gsa_params_t(p), max_segments(max_seg) {}
 };
 bool use_tc(const gsa_params_t& p) {
-    if (p.impl == GSA_IMPL_SIMT) return false;
-    return p.io == GSA_BF16 && tc_supported(p.d_k, p.d_v, p.m);
+    if (p.impl == GSA_IMPL_SIMT || p.io != GSA_BF16) return false;
+    return tc_supported(p.d_k, p.d_v, p.m) || use_wide(p);
 }
 
 // A bf16 layer with 32 slots runs on the tensor-core kernels too: their tiles are 64 slots wide, so the
@@ -86,6 +91,8 @@ bool use_fused(const gsa_params_t& p) {
 float inv_tau(const gsa_params_t& p) { return p.tau > 0.f ? 1.f / p.tau : 0.f; }
 
 int chunk_of(const gsa_params_t& p) { return use_tc(p) ? tc_chunk() : kChunk; }
+// ... that the running log gates G are local to (gsa_gate_cumsum's, too)
+int log_gate_chunk(const gsa_params_t& p) { return p.m == 128 ? kChunk : chunk_of(p); }
 
 struct Slices { int k, v; };
 Slices slices(const gsa_params_t& p) {
@@ -112,7 +119,7 @@ Segments segments_of(const CallParams& p) {
     const bool tc = use_tc(p);
     const int chunk = chunk_of(p), chunks = (p.T + chunk - 1) / chunk;
     const Slices sl = slices(p);
-    const long long ctas = (long long)p.B * p.H * (sl.k < sl.v ? sl.k : sl.v);
+    const long long ctas = (long long)p.B * p.H * (sl.k < sl.v ? sl.k : sl.v) * (use_wide(p) ? 2 : 1);
     if (use_fused(p)) {       // (the fused kernel sees segments as batch elements: equal ones)
         int n = 1;
         while (ctas * n * 2 <= 160 && p.T % (n * 2 * chunk) == 0 && p.T / (n * 2) >= 8 * chunk && n * 2 <= p.max_segments) n *= 2;
@@ -143,7 +150,7 @@ struct Carver {
 };
 
 struct Workspace {
-    float *G, *I, *okpart, *ok, *p, *dz, *u, *dppart, *dIk, *dIv, *chunk_tot, *KT, *VT;
+    float *G, *I, *E, *okpart, *ok, *p, *dz, *u, *dppart, *dIk, *dIv, *chunk_tot, *KT, *VT;
     int* strong;     // [B*nseg*H] flags: this (b,h) has a chunk that decays too hard for the factorised form
     float *seg_decay, *Kloc, *Vloc, *Kstart, *Vstart;   // segment-parallel scheduling only
     float *dKend, *dVend;                               // ... backward: states entering each segment from the right
@@ -151,6 +158,12 @@ struct Workspace {
     void *Id, *Pd, *Zd;
     size_t bytes;
 };
+
+// a decayed operand in floats: 2 bf16 values for every slot, 3 with 128 slots
+size_t decayed_floats(const gsa_params_t& p) {
+    const size_t mt = (size_t)p.B * p.T * p.H * p.m;
+    return use_wide(p) ? mt / 2 * 3 : mt;
+}
 
 Workspace carve(const CallParams& p, int which, void* ws) {
     Workspace w;
@@ -178,9 +191,10 @@ Workspace carve(const CallParams& p, int which, void* ws) {
     w.ok = c.take(mt);
     w.p = c.take(mt);
     if (use_tc(p)) {           // 2m bf16 per row = m floats
-        w.Id = c.take(mt);
-        w.Pd = c.take(mt);
-        if (which == GSA_WS_BWD) w.Zd = c.take(mt);
+        w.Id = c.take(decayed_floats(p));
+        w.Pd = c.take(decayed_floats(p));
+        if (which == GSA_WS_BWD) w.Zd = c.take(decayed_floats(p));
+        if (use_wide(p)) w.E = c.take(mt);
     }
     if (which == GSA_WS_BWD) {
         w.dz = c.take(mt);
@@ -201,7 +215,7 @@ Workspace carve(const CallParams& p, int which, void* ws) {
 // With segment-parallel scheduling the block also carries what the forward's first run found: the
 // segments' decay, the memories entering every segment and the final memories.
 struct GateSums {
-    int* strong; float *G, *I; void* Id;
+    int* strong; float *G, *I, *E; void* Id;
     float* p; void* Pd;                               // slot weights of the forward (tensor-core path)
     float *seg_decay, *Kstart, *Vstart, *KT, *VT;     // nseg > 1 only
     size_t bytes;
@@ -215,12 +229,13 @@ GateSums carve_gate(const CallParams& p, void* base) {
     g.strong = reinterpret_cast<int*>(c.take((size_t)p.B * p.H * nseg));
     g.G = c.take(mt);
     g.I = c.take(mt);
-    g.Id = use_tc(p) ? c.take(mt) : nullptr;
+    g.E = use_wide(p) ? c.take(mt) : nullptr;
+    g.Id = use_tc(p) ? c.take(decayed_floats(p)) : nullptr;
     // the slot weights p (fp32 for the pairs flagged for strong decay, the decayed operand pair for
     // the others) depend on the forward's logits only: kept, they let the backward's dv and dI^v
     // scans start before the softmax gradient is known
     g.p = use_tc(p) ? c.take(mt) : nullptr;
-    g.Pd = use_tc(p) ? c.take(mt) : nullptr;
+    g.Pd = use_tc(p) ? c.take(decayed_floats(p)) : nullptr;
     if (nseg > 1) {
         const size_t pairs = (size_t)p.B * nseg * p.H;
         g.seg_decay = c.take(pairs * p.m);
@@ -237,7 +252,7 @@ bool use_gate_block(const CallParams& p, Workspace* w, void* block, size_t block
     if (block == nullptr || (reinterpret_cast<uintptr_t>(block) & 255u) != 0) return false;
     const GateSums g = carve_gate(p, block);
     if (block_bytes < g.bytes) return false;
-    w->strong = g.strong; w->G = g.G; w->I = g.I; w->Id = g.Id;
+    w->strong = g.strong; w->G = g.G; w->I = g.I; w->E = g.E; w->Id = g.Id;
     if (g.p != nullptr) { w->p = g.p; w->Pd = g.Pd; }
     if (g.seg_decay != nullptr) {
         w->seg_decay = g.seg_decay; w->Kstart = g.Kstart; w->Vstart = g.Vstart;
@@ -248,6 +263,7 @@ bool use_gate_block(const CallParams& p, Workspace* w, void* block, size_t block
 
 cudaError_t value_side(const gsa_params_t& p, const ValueSideArgs& a, int reverse, const int* strong,
                        cudaStream_t st, int32_t* dev_status) {
+    if (use_wide(p)) return launch_value_side_wide(a, reverse, strong, st, dev_status);
     if (use_tc(p)) {
         ValueSideArgs b = a;
         b.single = p.tc_operands == GSA_TC_SINGLE;
@@ -257,12 +273,29 @@ cudaError_t value_side(const gsa_params_t& p, const ValueSideArgs& a, int revers
 }
 cudaError_t key_side(const gsa_params_t& p, const KeySideArgs& a, int reverse, const int* strong,
                      cudaStream_t st, int32_t* dev_status) {
+    if (use_wide(p)) return launch_key_side_wide(a, reverse, strong, st, dev_status);
     if (use_tc(p)) {
         KeySideArgs b = a;
         b.single = p.tc_operands == GSA_TC_SINGLE;
         return launch_key_side_tc(b, p.m, reverse, strong, st, dev_status);
     }
     return launch_key_side_simt(a, p.io, p.m, reverse, st);
+}
+
+// the gate kernel: G, 1 - a, the decayed rows and the strong-decay flags (cleared by the caller)
+cudaError_t gate_products(const gsa_params_t& p, Segments segs, const float* gate, const Workspace& w, cudaStream_t st) {
+    if (use_wide(p))
+        return launch_gate_cumsum_wide(gate, p.gate_kind, inv_tau(p), w.G, w.I, w.E, p.B, p.T, p.H, w.strong, segs.n, segs.t,
+                                       w.Id, st, p.cu_seqlens, p.nseq);
+    return launch_gate_cumsum(gate, p.gate_kind, inv_tau(p), w.G, w.I, p.B, p.T, p.H, p.m, chunk_of(p), w.strong, segs.n,
+                              segs.t, w.Id, p.io == GSA_BF16, st, p.cu_seqlens, p.nseq);
+}
+// the row factors that the tensor-core value_side scans leave to the slot kernels
+PendingDecay pending_decay(const gsa_params_t& p, Segments segs, const Workspace& w) {
+    if (!use_tc(p)) return {nullptr, nullptr, 1, 1, 1, 1, 0};
+    PendingDecay d{use_wide(p) ? w.E : w.G, w.strong, p.T, p.H, segs.n, segs.t, 0};
+    d.wide = use_wide(p);
+    return d;
 }
 
 // End memories (reverse: the gradients entering from the right) of every segment run from empty memories, K and V side.
@@ -272,7 +305,8 @@ cudaError_t state_scans(const gsa_params_t& p, Segments segs, StateSet ks, State
                         cudaStream_t st, int32_t* dev_status) {
     ValueSideArgs a[2] = {{ks.x, ks.x, ks.w, w.G, nullptr, ks.end, nullptr, p.B, p.T, p.H, p.d_k, ks.wd, 1},
                           {vs.x, vs.x, vs.w, w.G, nullptr, vs.end, nullptr, p.B, p.T, p.H, p.d_v, vs.wd, 1}};
-    for (ValueSideArgs& x : a) { x.nseg = segs.n; x.tseg = segs.t; }
+    for (ValueSideArgs& x : a) { x.nseg = segs.n; x.tseg = segs.t; x.E = w.E; }
+    if (use_wide(p)) return launch_state_scans_wide(a[0], a[1], reverse, w.strong, st, dev_status);
     if (use_tc(p)) return launch_state_scan_tc(a[0], a[1], reverse, w.strong, st, dev_status);
     cudaError_t e = launch_value_side_simt(a[0], p.io, p.m, reverse, st);
     return e == cudaSuccess ? launch_value_side_simt(a[1], p.io, p.m, reverse, st) : e;
@@ -475,7 +509,7 @@ extern "C" {
 
 int32_t gsa_chunk_size(const gsa_params_t* params) {
     if (check_params(params, false) != GSA_OK) return 0;
-    return chunk_of(internal_params(*params));
+    return log_gate_chunk(internal_params(*params));
 }
 
 const char* gsa_status_string(gsa_status_t status) {
@@ -521,7 +555,7 @@ gsa_status_t gsa_gate_cumsum(const gsa_params_t* params, const float* gate, floa
     const gsa_params_t& p = *params;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     GSA_LAUNCH("gate_cumsum", launch_gate_cumsum(gate, p.gate_kind, inv_tau(p), G, I, p.B, p.T,
-                                                 p.H, p.m, chunk_of(internal_params(p)), nullptr, 1, p.T, nullptr, 0, st,
+                                                 p.H, p.m, log_gate_chunk(internal_params(p)), nullptr, 1, p.T, nullptr, 0, st,
                                                  p.cu_seqlens, p.nseq));
     return GSA_OK;
 }
@@ -546,12 +580,10 @@ gsa_status_t fwd_core(const CallParams* params, int m_active, const void* q, con
     if (p.gate_kind == GSA_GATE_ABC)      // no decay, write weights from the cumulative softmax of the scores
         GSA_LAUNCH("abc_write", launch_abc_write(gate, w.G, w.I, w.Id, p.B, p.T, p.H, p.m, st));
     else
-        GSA_LAUNCH("gate_cumsum", launch_gate_cumsum(gate, p.gate_kind, inv_tau(p), w.G, w.I, p.B, p.T,
-                                                     p.H, p.m, chunk_of(p), w.strong, nseg, tseg, w.Id, p.io == GSA_BF16, st,
-                                                     p.cu_seqlens, p.nseq));
+        GSA_LAUNCH("gate_cumsum", gate_products(p, segs, gate, w, st));
     float* ok = ok_save;      // the scaled logits leave the softmax kernel only if the caller keeps them
     // the pipelined kernels leave the row factor of the pass-1 sums to the softmax kernel
-    const PendingDecay pend = use_tc(p) ? PendingDecay{w.G, w.strong, p.T, p.H, nseg, tseg, 0} : PendingDecay{nullptr, nullptr, 1, 1, 1, 1, 0};
+    const PendingDecay pend = pending_decay(p, segs, w);
     const float *Kin = K0, *Vin = V0;
     float *Kout = KT, *Vout = VT;
     if (nseg > 1) {
@@ -559,7 +591,7 @@ gsa_status_t fwd_core(const CallParams* params, int m_active, const void* q, con
         // land in buffers that the second pass overwrites); then the start memories of all
         // segments, and the final memories, by a scan over the segments
         GSA_LAUNCH("segment_logdecay", launch_segment_logdecay(w.G, w.seg_decay, p.B, p.T, p.H, p.m, nseg,
-                                                               tseg, chunk_of(p), st));
+                                                               tseg, log_gate_chunk(p), st));
         GSA_LAUNCH("segment_states", state_scans(p, segs, StateSet{k, w.I, w.Id, w.Kloc}, StateSet{v, w.I, w.Id, w.Vloc}, w, 0,
                                                   st, dev_status));
         // (when the backward is to reuse them, the final memories land in the saved block first)
@@ -576,10 +608,10 @@ gsa_status_t fwd_core(const CallParams* params, int m_active, const void* q, con
     }
     // pass 1: o' = GLA(q, k, 1-a) with the decay on the slot (value) side
     ValueSideArgs a1{q, k, w.I, w.G, Kin, Kout, w.okpart, p.B, p.T, p.H, p.d_k, w.Id};
-    a1.nseg = nseg; a1.tseg = tseg;
+    a1.nseg = nseg; a1.tseg = tseg; a1.E = w.E;
     // pass 2: o = GLA(softmax(o'), 1-a, v) with the decay on the slot (key) side
     KeySideArgs a2{w.p, w.I, w.G, v, Vin, Vout, o, p.B, p.T, p.H, p.d_v, w.Pd, w.Id};
-    a2.nseg = nseg; a2.tseg = tseg;
+    a2.nseg = nseg; a2.tseg = tseg; a2.E = w.E;
     if (use_fused(p)) {
         // One kernel for pass 1 -> softmax -> pass 2; the logits are written only if the caller wants
         // them.  The (batch, head) pairs flagged for strong decay take the general kernels and the
@@ -690,6 +722,12 @@ gsa_status_t gsa::fwd_within(const gsa_params_t* params, const void* q, const vo
     CallParams cp(*params);
     cp.max_segments = segments_of(internal_params(cp)).n;
     while (cp.max_segments > 1 && workspace_bytes(cp, GSA_WS_FWD) > ws_bytes) --cp.max_segments;
+    if (use_wide(cp) && workspace_bytes(cp, GSA_WS_FWD) > ws_bytes) {       // (the CUDA-core kernels need less for narrow heads)
+        cp.impl = GSA_IMPL_SIMT;
+        cp.max_segments = 1 << 30;
+        cp.max_segments = segments_of(cp).n;
+        while (cp.max_segments > 1 && workspace_bytes(cp, GSA_WS_FWD) > ws_bytes) --cp.max_segments;
+    }
     if (workspace_bytes(cp, GSA_WS_FWD) > ws_bytes) return GSA_ERR_WORKSPACE;
     return fwd_impl(&cp, q, k, v, gate, K0, V0, o, ok_save, KT, VT, false, nullptr, 0, ws, ws_bytes, stream, dev_status);
 }
@@ -720,12 +758,10 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
         if (p.gate_kind == GSA_GATE_ABC)
             GSA_LAUNCH("abc_write", launch_abc_write(gate, w.G, w.I, w.Id, p.B, p.T, p.H, p.m, st));
         else
-            GSA_LAUNCH("gate_cumsum", launch_gate_cumsum(gate, p.gate_kind, inv_tau(p), w.G, w.I, p.B, p.T,
-                                                         p.H, p.m, chunk_of(p), w.strong, nseg, tseg, w.Id, p.io == GSA_BF16, st,
-                                                         p.cu_seqlens, p.nseq));
+            GSA_LAUNCH("gate_cumsum", gate_products(p, segs, gate, w, st));
     }
     const float* ok = ok_saved;
-    const PendingDecay pend = use_tc(p) ? PendingDecay{w.G, w.strong, p.T, p.H, nseg, tseg, 0} : PendingDecay{nullptr, nullptr, 1, 1, 1, 1, 0};
+    const PendingDecay pend = pending_decay(p, segs, w);
     const float *Kin = K0, *Vin = V0;        // states entering the forward-direction scans
     float* KTout = dKT ? w.KT : nullptr;     // final memories, for the gate gradient's final-memory term
     float* VTout = dVT ? w.VT : nullptr;
@@ -736,7 +772,7 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
         KTout = nullptr; VTout = nullptr;
     } else if (nseg > 1) {
         GSA_LAUNCH("segment_logdecay", launch_segment_logdecay(w.G, w.seg_decay, p.B, p.T, p.H, p.m, nseg,
-                                                               tseg, chunk_of(p), st));
+                                                               tseg, log_gate_chunk(p), st));
         GSA_LAUNCH("segment_states", state_scans(p, segs, StateSet{k, w.I, w.Id, w.Kloc}, StateSet{v, w.I, w.Id, w.Vloc}, w, 0,
                                                   st, dev_status));
         GSA_LAUNCH("segment_combine", launch_segment_combine(w.seg_decay, {w.Kloc, K0, w.Kstart, KTout, p.d_k}, {w.Vloc, V0, w.Vstart, VTout, p.d_v}, p.B,
@@ -746,7 +782,7 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
     }
     if (ok == nullptr) {  // recompute pass 1 and its logits
         ValueSideArgs a1{q, k, w.I, w.G, Kin, nullptr, w.okpart, p.B, p.T, p.H, p.d_k, w.Id};
-        a1.nseg = nseg; a1.tseg = tseg;
+        a1.nseg = nseg; a1.tseg = tseg; a1.E = w.E;
         GSA_LAUNCH("pass1_value_side", value_side(p, a1, 0, w.strong, st, dev_status));
         GSA_LAUNCH("slot_softmax", launch_slot_softmax_fwd(w.okpart, s.k, p.scale, p.slot_act, w.ok, w.p, p.B, p.T * p.H, p.m, pend.G,
                                                            nullptr, pend, st, m_active));
@@ -754,10 +790,10 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
     }
     // gradient w.r.t. the pass-2 queries p: the pass-1 form on (dO, v, 1-a); carries V~
     ValueSideArgs adp{dO, v, w.I, w.G, Vin, VTout, w.dppart, p.B, p.T, p.H, p.d_v, w.Id};
-    adp.nseg = nseg; adp.tseg = tseg;
+    adp.nseg = nseg; adp.tseg = tseg; adp.E = w.E;
     // dq: the pass-2 form on (dz, 1-a, k); carries K~
     KeySideArgs adq{w.dz, w.I, w.G, k, Kin, KTout, dq, p.B, p.T, p.H, p.d_k, w.Zd, w.Id};
-    adq.nseg = nseg; adq.tseg = tseg;
+    adq.nseg = nseg; adq.tseg = tseg; adq.E = w.E;
     const bool fused = use_fused(p);
     // With the forward's slot weights in the saved block (and the logits saved, so that nothing here
     // rewrites them), the dv and dI^v scans depend on nothing this call computes: they start at once,
@@ -800,9 +836,9 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
         GSA_LAUNCH("bwd_dp_value_side", value_side(p, adp, 0, w.strong, sc, dev_status));
         if (early) {
             KeySideArgs adv{w.I, w.p, w.G, dO, dVT, dV0, dv, p.B, p.T, p.H, p.d_v, w.Id, w.Pd};
-            adv.nseg = nseg; adv.tseg = tseg;
+            adv.nseg = nseg; adv.tseg = tseg; adv.E = w.E;
             ValueSideArgs adIv{v, dO, w.p, w.G, dVT, nullptr, w.dIv, p.B, p.T, p.H, p.d_v, w.Pd};
-            adIv.nseg = nseg; adIv.tseg = tseg;
+            adIv.nseg = nseg; adIv.tseg = tseg; adIv.E = w.E;
             adv.single = adIv.single = p.tc_operands == GSA_TC_SINGLE;
             if (g_pair_scans.load(std::memory_order_relaxed) != 0 && rev_pair_supported(adIv, adv, p.m)) {
                 GSA_CUDA(launch_rev_pair_tc(adIv, adv, p.m, w.strong, lanes->stream[0], dev_status));
@@ -835,13 +871,13 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
     }
     // time-reversed runs: dv and dI^v share the state dV~; dk and dI^k share dK~
     KeySideArgs adv{w.I, w.p, w.G, dO, dVin, dV0out, dv, p.B, p.T, p.H, p.d_v, w.Id, w.Pd};
-    adv.nseg = nseg; adv.tseg = tseg;
+    adv.nseg = nseg; adv.tseg = tseg; adv.E = w.E;
     ValueSideArgs adIv{v, dO, w.p, w.G, dVin, nullptr, w.dIv, p.B, p.T, p.H, p.d_v, w.Pd};
-    adIv.nseg = nseg; adIv.tseg = tseg;
+    adIv.nseg = nseg; adIv.tseg = tseg; adIv.E = w.E;
     KeySideArgs adk{w.I, w.dz, w.G, q, dKin, dK0out, dk, p.B, p.T, p.H, p.d_k, w.Id, w.Zd};
-    adk.nseg = nseg; adk.tseg = tseg;
+    adk.nseg = nseg; adk.tseg = tseg; adk.E = w.E;
     ValueSideArgs adIk{k, q, w.dz, w.G, dKin, nullptr, w.dIk, p.B, p.T, p.H, p.d_k, w.Zd};
-    adIk.nseg = nseg; adIk.tseg = tseg;
+    adIk.nseg = nseg; adIk.tseg = tseg; adIk.E = w.E;
     // the reversed scans that share a state run as one kernel each (dv with dI^v, dk with dI^k)
     ValueSideArgs pIv = adIv, pIk = adIk;
     KeySideArgs pv = adv, pk = adk;
@@ -1024,9 +1060,8 @@ gsa_status_t gsa_shard_states(const gsa_params_t* params, const void* k, const v
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // one "segment" per batch element: the whole shard from empty memories, end memories only
     GSA_CUDA(cudaMemsetAsync(w.strong, 0, sizeof(int) * (size_t)p.B * p.H, st));
-    GSA_LAUNCH("gate_cumsum", launch_gate_cumsum(gate, p.gate_kind, inv_tau(p), w.G, w.I, p.B, p.T, p.H, p.m, chunk_of(p),
-                                                 w.strong, 1, p.T, w.Id, p.io == GSA_BF16, st));
-    GSA_LAUNCH("segment_logdecay", launch_segment_logdecay(w.G, logdecay, p.B, p.T, p.H, p.m, 1, p.T, chunk_of(p), st));
+    GSA_LAUNCH("gate_cumsum", gate_products(p, Segments{1, p.T}, gate, w, st));
+    GSA_LAUNCH("segment_logdecay", launch_segment_logdecay(w.G, logdecay, p.B, p.T, p.H, p.m, 1, p.T, log_gate_chunk(p), st));
     GSA_LAUNCH("segment_states", state_scans(p, Segments{1, p.T}, StateSet{k, w.I, w.Id, KT}, StateSet{v, w.I, w.Id, VT}, w, 0, st,
                                               dev_status));
     return GSA_OK;

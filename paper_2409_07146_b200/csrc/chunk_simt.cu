@@ -143,8 +143,11 @@ __device__ __forceinline__ bool chunk_is_moderate(const float* sG, int* flag) {
 }
 
 // =============================================================== value_side (pass-1 form)
-template <typename IO, int M, bool REV>
-__global__ void __launch_bounds__(256) value_side_simt_kernel(ValueSideArgs a) {
+// FLAGGED: the flagged pairs of a tensor-core scan alone (see launch_value_side_simt); a CTA then takes both 64-wide
+// halves of a 128-wide slice, one after the other.
+template <typename IO, int M, bool REV, bool FLAGGED>
+__global__ void __launch_bounds__(256) value_side_simt_kernel(ValueSideArgs a, const int* __restrict__ strong_flag) {
+    if (FLAGGED && strong_flag[blockIdx.x] == 0) return;
     constexpr int NJ = M / 16;
     constexpr int LM = M + 4;
     extern __shared__ __align__(16) float smem[];
@@ -159,7 +162,9 @@ __global__ void __launch_bounds__(256) value_side_simt_kernel(ValueSideArgs a) {
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
     const ScanSpan span = scan_span(blockIdx.x, a.H, a.T, a.nseg, a.tseg);
     const int slice = blockIdx.y, bh = blockIdx.x, b = span.b, h = span.h;
-    const int d0 = slice * kDS;
+    const int subs = FLAGGED ? min(2, (a.D - slice * 2 * kDS) / kDS) : 1;
+    for (int sub = 0; sub < subs; ++sub) {
+    const int d0 = slice * (FLAGGED ? 2 : 1) * kDS + sub * kDS;
     const size_t strideD = (size_t)a.H * a.D, strideM = (size_t)a.H * M;
     const IO* xq = (const IO*)a.xq + ((size_t)b * a.T * a.H + h) * a.D + d0;
     const IO* xk = (const IO*)a.xk + ((size_t)b * a.T * a.H + h) * a.D + d0;
@@ -256,7 +261,10 @@ __global__ void __launch_bounds__(256) value_side_simt_kernel(ValueSideArgs a) {
                 const int i = 4 * ty + ii;
                 if (i < valid) {
 #pragma unroll
-                    for (int jj = 0; jj < NJ; ++jj) out[(size_t)(t0 + i) * strideM + NJ * tx + jj] = acc[ii][jj];
+                    for (int jj = 0; jj < NJ; ++jj) {
+                        float* o = out + (size_t)(t0 + i) * strideM + NJ * tx + jj;
+                        *o = FLAGGED && sub > 0 ? *o + acc[ii][jj] : acc[ii][jj];
+                    }
                 }
             }
         }
@@ -291,11 +299,14 @@ __global__ void __launch_bounds__(256) value_side_simt_kernel(ValueSideArgs a) {
             a.Send[((size_t)bh * M + s) * a.D + d0 + c] = sS[c * LM + s];
         }
     }
+    if (FLAGGED) __syncthreads();
+    }
 }
 
 // =============================================================== key_side (pass-2 form)
-template <typename IO, int M, bool REV>
-__global__ void __launch_bounds__(256) key_side_simt_kernel(KeySideArgs a) {
+template <typename IO, int M, bool REV, bool FLAGGED>
+__global__ void __launch_bounds__(256) key_side_simt_kernel(KeySideArgs a, const int* __restrict__ strong_flag) {
+    if (FLAGGED && strong_flag[blockIdx.x] == 0) return;
     constexpr int LM = M + 4;
     extern __shared__ __align__(16) float smem[];
     float* sQ = smem;                  // [64][LM]  uq (scaled in place)
@@ -439,28 +450,33 @@ cudaError_t set_smem(K kernel, size_t bytes) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
-template <typename IO, int M, bool REV>
-cudaError_t launch_vs(const ValueSideArgs& a, cudaStream_t st) {
+template <typename IO, int M, bool REV, bool FLAGGED = false>
+cudaError_t launch_vs(const ValueSideArgs& a, cudaStream_t st, const int* strong_flag = nullptr) {
     const size_t smem = sizeof(float) * (3 * kC * kLd + (kDS + 2 * kC) * (M + 4));
-    cudaError_t e = set_smem(value_side_simt_kernel<IO, M, REV>, smem);
+    cudaError_t e = set_smem(value_side_simt_kernel<IO, M, REV, FLAGGED>, smem);
     if (e != cudaSuccess) return e;
-    dim3 grid(a.B * a.nseg * a.H, a.D / kDS);
-    value_side_simt_kernel<IO, M, REV><<<grid, 256, smem, st>>>(a);
+    dim3 grid(a.B * a.nseg * a.H, FLAGGED ? (a.D + 2 * kDS - 1) / (2 * kDS) : a.D / kDS);
+    value_side_simt_kernel<IO, M, REV, FLAGGED><<<grid, 256, smem, st>>>(a, strong_flag);
     return cudaGetLastError();
 }
-template <typename IO, int M, bool REV>
-cudaError_t launch_ks(const KeySideArgs& a, cudaStream_t st) {
+template <typename IO, int M, bool REV, bool FLAGGED = false>
+cudaError_t launch_ks(const KeySideArgs& a, cudaStream_t st, const int* strong_flag = nullptr) {
     const size_t smem = sizeof(float) * (3 * kC * (M + 4) + 2 * kC * kLd + M * kLd);
-    cudaError_t e = set_smem(key_side_simt_kernel<IO, M, REV>, smem);
+    cudaError_t e = set_smem(key_side_simt_kernel<IO, M, REV, FLAGGED>, smem);
     if (e != cudaSuccess) return e;
     dim3 grid(a.B * a.nseg * a.H, a.D / kDS);
-    key_side_simt_kernel<IO, M, REV><<<grid, 256, smem, st>>>(a);
+    key_side_simt_kernel<IO, M, REV, FLAGGED><<<grid, 256, smem, st>>>(a, strong_flag);
     return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t launch_value_side_simt(const ValueSideArgs& a, int io, int M, int reverse, cudaStream_t st) {
+cudaError_t launch_value_side_simt(const ValueSideArgs& a, int io, int M, int reverse, cudaStream_t st, const int* strong_flag) {
+    if (strong_flag != nullptr) {        // (beside the kernels for 128 slots)
+        if (io != GSA_BF16 || M != 128) return cudaErrorNotSupported;
+        return reverse ? launch_vs<__nv_bfloat16, 128, true, true>(a, st, strong_flag)
+                       : launch_vs<__nv_bfloat16, 128, false, true>(a, st, strong_flag);
+    }
 #define GSA_VS(IO, MM)                                                                   \
     return reverse ? launch_vs<IO, MM, true>(a, st) : launch_vs<IO, MM, false>(a, st)
     if (io == GSA_BF16) {
@@ -471,7 +487,12 @@ cudaError_t launch_value_side_simt(const ValueSideArgs& a, int io, int M, int re
 #undef GSA_VS
 }
 
-cudaError_t launch_key_side_simt(const KeySideArgs& a, int io, int M, int reverse, cudaStream_t st) {
+cudaError_t launch_key_side_simt(const KeySideArgs& a, int io, int M, int reverse, cudaStream_t st, const int* strong_flag) {
+    if (strong_flag != nullptr) {
+        if (io != GSA_BF16 || M != 128) return cudaErrorNotSupported;
+        return reverse ? launch_ks<__nv_bfloat16, 128, true, true>(a, st, strong_flag)
+                       : launch_ks<__nv_bfloat16, 128, false, true>(a, st, strong_flag);
+    }
 #define GSA_KS(IO, MM)                                                                   \
     return reverse ? launch_ks<IO, MM, true>(a, st) : launch_ks<IO, MM, false>(a, st)
     if (io == GSA_BF16) {

@@ -1,0 +1,772 @@
+// Tensor-core chunk kernels for 128 slots (bf16 io), for the (batch, head) pairs whose chunks all decay moderately; the
+// flagged pairs take the CUDA-core kernels (chunk_simt.cu).
+//
+// A layer with 128 slots ran on the fp32 CUDA-core kernels alone: 14.4 ms for a training step at B = 8, T = 2048, 4 heads
+// of 512, 26% of the fp32 rate, where 64 slots take 0.5 ms.  What the caller gets in fp32 (logits, memories, gate
+// gradient) keeps that accuracy here: the operands the kernels derive on the way to those -- decayed weights, masked
+// first product, state copy -- enter the products as THREE bfloat16 parts (24 bits), all products down to 2^-24 of the
+// leading one are formed, and decay factors come as exp(G) formed from the exact sums (`E`) instead of exp of a rounded
+// G.  What only leads to an output that is rounded to bfloat16 (key_side: o, dq, dk, dv) takes two parts, as with 64
+// slots.
+//
+// The 128 slots are two halves of 64: a [.., H, 128] slot tensor is a [.., 2 H, 64] one, decayed rows are [.., 2 H, 192]
+// ([high | middle | low] of 64 slots).
+//   value_side  the halves are independent, each CTA takes one: the pipelined kernel of chunk_tc_lean.cu with 64-column
+//               accumulators that collect all parts.  14 panels of shared memory: two stages of xq and xk, one of the
+//               weights, one state copy; the output rows are staged where xq was.
+//   key_side    the halves add up in A = Q K^T, so a CTA takes both, one as each stage of the decayed rows; the xv tile is
+//               single-staged (14 panels), the next one asked into L2 ahead.
+// B200, B = 8, T = 2048, 4 heads of 512, training step: 14400 us on the CUDA cores, 1145 here; error of the gate gradient
+// against 64 bits 9.0e-7 there (2-norm), 8.3e-7 here.
+#include "chunk_tc_shared.cuh"
+
+namespace gsa {
+namespace {
+using namespace tc;
+using namespace tcchunk;
+
+constexpr int kMmaWarp = kComputeThreads / 32, kCopyWarp = kMmaWarp + 1;
+constexpr int kWide = 2 * kM;          // slots
+constexpr int kParts = 3 * kM;         // columns of a decayed row of one half
+
+struct WideCtl {
+    // filled by TMA
+    uint64_t bar_x[2];     // value_side: xq, xk (two stages); key_side: [0] = xv
+    uint64_t bar_w[2];     // value_side: [0] = weights; key_side: decayed rows of a half
+    // signalled by tcgen05.commit
+    uint64_t bar_p;        // first product of a chunk
+    uint64_t bar_mma1;     // state and inter-chunk products
+    uint64_t bar_mma2[2];  // intra-chunk product, for the compute threads (value_side: by chunk parity)
+    uint64_t bar_free[2];  // value_side: [0] = the weights are consumed; key_side: the rows of a half are
+    // signalled by the compute threads
+    uint64_t bar_pm;       // masked rows are in tensor memory
+    uint64_t bar_sb;       // state copy for the next chunk is written
+    uint64_t bar_out[2];   // output rows are staged, their accumulator is free (value_side: by chunk parity)
+    uint32_t tmem_slot;
+    volatile int abort;
+    alignas(16) float egc[2][kWide];   // exp(G) of the chunk's last valid row, by chunk parity
+};
+
+#define WIDE_WAIT(bar, parity)                                              \
+    do {                                                                    \
+        if (!ctl->abort && !mbar_wait(bar, parity)) ctl->abort = 1;         \
+    } while (0)
+
+__device__ __forceinline__ void wide_begin(WideCtl* ctl, int tid, int warp) {
+    if (tid == 0) {
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&ctl->bar_x[i], 1);
+            mbar_init(&ctl->bar_w[i], 1);
+            mbar_init(&ctl->bar_mma2[i], 1);
+            mbar_init(&ctl->bar_free[i], 1);
+            mbar_init(&ctl->bar_out[i], 1);
+        }
+        mbar_init(&ctl->bar_p, 1);
+        mbar_init(&ctl->bar_mma1, 1);
+        mbar_init(&ctl->bar_pm, 1);
+        mbar_init(&ctl->bar_sb, 1);
+        ctl->abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        __syncwarp();
+        tmem_alloc(&ctl->tmem_slot, kTmemCols);
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+}
+
+__device__ __forceinline__ void wide_end(WideCtl* ctl, int tid, int warp, uint32_t tmem, int32_t* dev_status) {
+    tc_fence_before_sync();
+    __syncthreads();
+    if (ctl->abort) {
+        if (tid == 0 && dev_status != nullptr) *dev_status = GSA_ERR_TIMEOUT;
+        // bounded grace period for tile copies still in flight before shared memory goes away
+        for (int i = 0; i < 200; ++i) __nanosleep(1000);
+    }
+    __syncthreads();
+    if (warp == 0) {
+        __syncwarp();
+        tmem_dealloc(tmem, kTmemCols);
+    }
+}
+
+// x = high + middle + low as bfloat16 parts of two values, packed
+__device__ __forceinline__ void split3(float x0, float x1, uint32_t& h, uint32_t& m, uint32_t& l) {
+    h = pack_bf16(x0, x1);
+    const float r0 = x0 - __uint_as_float(h << 16), r1 = x1 - __uint_as_float(h & 0xffff0000u);
+    m = pack_bf16(r0, r1);
+    l = pack_bf16(r0 - __uint_as_float(m << 16), r1 - __uint_as_float(m & 0xffff0000u));
+}
+
+// The masked first product as three bfloat16 parts: high and middle part in place (the layout of mask_row_in_tmem), the low
+// part in 64 columns of their own from col_lo on (K step kk at col_lo + 32 (kk >> 2) + 8 (kk & 3)).
+template <bool REV>
+__device__ __forceinline__ void mask_row_split3(uint32_t tmem, int wq, int row, int half, int col0, int col_lo) {
+    const int base = col0 + 64 * half;
+    uint32_t mid[32];
+#pragma unroll
+    for (int c0 = 0; c0 < 64; c0 += 32) {
+        float v[32];
+        uint32_t hi[16], lo[16];
+        tmem_ld32(tmem_row_addr(tmem, wq, base + c0), v);
+#pragma unroll
+        for (int e = 0; e < 32; e += 2) {
+            const int j = 64 * half + c0 + e;
+            const float x0 = (REV ? (j >= row) : (j <= row)) ? v[e] : 0.f;
+            const float x1 = (REV ? (j + 1 >= row) : (j + 1 <= row)) ? v[e + 1] : 0.f;
+            split3(x0, x1, hi[e >> 1], mid[(c0 + e) >> 1], lo[e >> 1]);
+        }
+        tmem_st16(tmem_row_addr(tmem, wq, base + (c0 >> 1)), hi);            // (onto columns already read)
+        tmem_st16(tmem_row_addr(tmem, wq, col_lo + 32 * half + (c0 >> 1)), lo);
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+        tmem_st16(tmem_row_addr(tmem, wq, base + 32 + 16 * q), *reinterpret_cast<const uint32_t (*)[16]>(&mid[16 * q]));
+    tmem_st_wait();
+}
+
+// this thread's half state row (32 slots from sb on, times scale[sb ..]) as three bfloat16 panels
+template <bool SCALE>
+__device__ __forceinline__ void store_state_split3(unsigned char* panels, int row, int sb, const float (&S)[kHS],
+                                                   const float* scale) {
+#pragma unroll
+    for (int c = 0; c < kHS / 8; ++c) {
+        uint32_t h[4], m[4], l[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float x0 = S[8 * c + 2 * e], x1 = S[8 * c + 2 * e + 1];
+            split3(SCALE ? x0 * scale[sb + 8 * c + 2 * e] : x0, SCALE ? x1 * scale[sb + 8 * c + 2 * e + 1] : x1, h[e], m[e], l[e]);
+        }
+        const uint32_t at = swz128(row, (sb >> 3) + c);
+        *reinterpret_cast<uint4*>(panels + at) = make_uint4(h[0], h[1], h[2], h[3]);
+        *reinterpret_cast<uint4*>(panels + kPanelB + at) = make_uint4(m[0], m[1], m[2], m[3]);
+        *reinterpret_cast<uint4*>(panels + 2 * kPanelB + at) = make_uint4(l[0], l[1], l[2], l[3]);
+    }
+}
+
+__device__ __forceinline__ uint32_t step_kmaj(int kk) { return (uint32_t)((kk >> 2) * kPanelB + (kk & 3) * 32); }
+__device__ __forceinline__ uint32_t step_mnmaj(int kk) { return (uint32_t)(kk * 2048); }
+
+// ======================================================================================
+// value_side of one half: out_i[s] = sum_{j<=i} <xq_i, xk_j> w_j[s] decay_ij[s] + decayed (xq_i S)[s], without the row
+// factor (see PendingDecay).  Accumulator columns: first product 128 (+ 64 for its low part), state product 64, inter- and
+// intra-chunk output 2 x 64 each by chunk parity.  An accumulation drops what falls below the accumulator's last bit, so
+// the smallest parts are summed first and only the eight products of the leading parts meet a full-sized accumulator
+// (leading parts first, inter- and intra-chunk products in one accumulator: logits off by 5e-6 of their rms, not 2.5e-6).
+// In the reverse direction the state copy carries the total decay of the chunk it is used in.
+// ======================================================================================
+constexpr int kWvP = 0, kWvPlow = 128, kWvU = 192, kWvO = 256, kWvI = 384;
+
+template <bool REV>
+__global__ void __launch_bounds__(kScanThreads, 1)
+value_side_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
+                       const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapO,
+                       const __grid_constant__ ValueSideArgs a, const int* __restrict__ strong_flag, int32_t* dev_status) {
+    const int H2 = 2 * a.H;
+    const ScanSpan span = scan_span(blockIdx.x, H2, a.T, a.nseg, a.tseg);
+    const int bh = blockIdx.x, slice = blockIdx.y, b = span.b, h2 = span.h, h = h2 >> 1;
+    if (strong_flag[(bh / H2) * a.H + h] != 0) return;       // the CUDA-core kernel takes this (batch, head)
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    unsigned char* sX = smem;                        // xq, xk tiles: 2 stages x (2 + 2 panels); the output rows (fp32, 2
+                                                     //   panels of 32 slots) are staged where the chunk's xq was
+    unsigned char* sW = sX + 8 * kPanelB;            // weights [high | middle | low], MN-major B, 3 panels
+    unsigned char* sSb = sW + 3 * kPanelB;           // state copy, likewise, 3 panels
+    WideCtl* ctl = reinterpret_cast<WideCtl*>(sSb + 3 * kPanelB);
+
+    const int tid = threadIdx.x, warp = tid >> 5, wq = warp & 3, half = (tid >> 7) & 1, row = tid & 127;
+    const int sb = kHS * half;          // this thread's first slot of the half
+    const int d0 = slice * kDST;
+
+    wide_begin(ctl, tid, warp);
+    const uint32_t tmem = ctl->tmem_slot;
+    const int nchunks = (span.t_end - span.t0 + kCT - 1) / kCT;
+    auto chunk_t0 = [&](int n) { return span.t0 + (REV ? nchunks - 1 - n : n) * kCT; };
+
+    if (warp == kCopyWarp) {
+        if (elect_one()) {
+            // =============================== copy lane
+            auto load_x = [&](int n) {
+                const int t = chunk_t0(n), st = n & 1;
+                unsigned char* sXq = sX + 4 * st * kPanelB;
+                mbar_expect_tx(&ctl->bar_x[st], 4 * kPanelB);
+                tma_load_4d(sXq, &mapQ, &ctl->bar_x[st], d0, h, t, b);
+                tma_load_4d(sXq + kPanelB, &mapQ, &ctl->bar_x[st], d0 + 64, h, t, b);
+                tma_load_4d(sXq + 2 * kPanelB, &mapK, &ctl->bar_x[st], d0, h, t, b);
+                tma_load_4d(sXq + 3 * kPanelB, &mapK, &ctl->bar_x[st], d0 + 64, h, t, b);
+            };
+            auto load_w = [&](int n) {
+                const int t = chunk_t0(n);
+                mbar_expect_tx(&ctl->bar_w[0], 3 * kPanelB);
+                for (int i = 0; i < 3; ++i) tma_load_4d(sW + i * kPanelB, &mapW, &ctl->bar_w[0], 64 * i, h2, t, b);
+            };
+            prefetch_tmap(&mapQ); prefetch_tmap(&mapK); prefetch_tmap(&mapW); prefetch_tmap(&mapO);
+            load_x(0);
+            load_w(0);
+            if (nchunks > 1) load_x(1);
+            for (int n = 0; n < nchunks && !ctl->abort; ++n) {
+                WIDE_WAIT(&ctl->bar_free[0], n & 1);
+                if (ctl->abort) break;
+                if (n + 1 < nchunks) load_w(n + 1);
+                WIDE_WAIT(&ctl->bar_out[n & 1], (n >> 1) & 1);
+                if (ctl->abort) break;
+                const unsigned char* sOut = sX + 4 * (n & 1) * kPanelB;
+                tma_store_5d(&mapO, sOut, 0, h2, chunk_t0(n), b, slice);
+                tma_store_5d(&mapO, sOut + kPanelB, 32, h2, chunk_t0(n), b, slice);
+                bulk_commit();
+                bulk_wait_read();
+                if (n + 2 < nchunks) load_x(n + 2);
+            }
+        }
+    } else if (warp == kMmaWarp) {
+        if (elect_one()) {
+            // =============================== MMA lane
+            constexpr uint32_t idescP = make_idesc(128, 128, false, false);    // xq xk^T
+            constexpr uint32_t idescO = make_idesc(128, kM, false, true);      // xq or masked P x part (MN-major B)
+            constexpr uint32_t idescU = make_idesc(128, kM, true, true);       // xk^T (MN-major A) x part (MN-major B)
+            uint64_t dW[3], dS[3];
+            for (int i = 0; i < 3; ++i) {
+                dW[i] = desc_mnmajor(smem_u32(sW + i * kPanelB), 0, kPanelB);
+                dS[i] = desc_mnmajor(smem_u32(sSb + i * kPanelB), 0, kPanelB);
+            }
+            auto issue_p = [&](int n) {
+                const uint32_t xq = smem_u32(sX + 4 * (n & 1) * kPanelB);
+                const uint64_t dQk = desc_kmajor(xq, 0), dKk = desc_kmajor(xq + 2 * kPanelB, 0);
+#pragma unroll
+                for (int kk = 0; kk < kDST / 16; ++kk)
+                    mma_bf16(tmem + kWvP, desc_advance(dQk, step_kmaj(kk)), desc_advance(dKk, step_kmaj(kk)), idescP, kk > 0);
+                mma_commit(&ctl->bar_p);
+            };
+            WIDE_WAIT(&ctl->bar_x[0], 0);
+            tc_fence_after_sync();
+            if (!ctl->abort) issue_p(0);
+            for (int n = 0; n < nchunks && !ctl->abort; ++n) {
+                const uint32_t xq = smem_u32(sX + 4 * (n & 1) * kPanelB);
+                const uint64_t dQk = desc_kmajor(xq, 0), dKm = desc_mnmajor(xq + 2 * kPanelB, 0, kPanelB);
+                const uint32_t accO = tmem + kWvO + kM * (n & 1), accI = tmem + kWvI + kM * (n & 1);
+                // state and inter-chunk products (the state copy was written in chunk n-1, the output accumulators of
+                // this parity read out in chunk n-2)
+                WIDE_WAIT(&ctl->bar_w[0], n & 1);
+                WIDE_WAIT(&ctl->bar_sb, n & 1);
+                if (n >= 2) WIDE_WAIT(&ctl->bar_out[n & 1], ((n - 2) >> 1) & 1);
+                if (ctl->abort) break;
+                tc_fence_after_sync();
+#pragma unroll
+                for (int i = 2; i >= 0; --i)
+#pragma unroll
+                    for (int kk = 0; kk < kCT / 16; ++kk)
+                        mma_bf16(tmem + kWvU, desc_advance(dKm, step_mnmaj(kk)), desc_advance(dW[i], step_mnmaj(kk)), idescU,
+                                 i < 2 || kk > 0);
+#pragma unroll
+                for (int i = 2; i >= 0; --i)
+#pragma unroll
+                    for (int kk = 0; kk < kDST / 16; ++kk)
+                        mma_bf16(accO, desc_advance(dQk, step_kmaj(kk)), desc_advance(dS[i], step_mnmaj(kk)), idescO,
+                                 i < 2 || kk > 0);
+                mma_commit(&ctl->bar_mma1);
+                // intra-chunk product: the parts of the masked P times those of the weights, from 2^-24 up
+                WIDE_WAIT(&ctl->bar_pm, n & 1);
+                if (ctl->abort) break;
+                tc_fence_after_sync();
+#pragma unroll
+                for (int order = 2; order >= 0; --order)
+#pragma unroll
+                    for (int ip = 0; ip <= order; ++ip)
+#pragma unroll
+                        for (int kk = 0; kk < kCT / 16; ++kk)
+                            mma_bf16_ta(accI,
+                                        ip < 2 ? tmem + kWvP + 64 * (kk >> 2) + 32 * ip + 8 * (kk & 3)
+                                               : tmem + kWvPlow + 32 * (kk >> 2) + 8 * (kk & 3),
+                                        desc_advance(dW[order - ip], step_mnmaj(kk)), idescO, order < 2 || ip + kk > 0);
+                mma_commit(&ctl->bar_mma2[n & 1]);
+                mma_commit(&ctl->bar_free[0]);
+                if (n + 1 < nchunks) {
+                    WIDE_WAIT(&ctl->bar_x[(n + 1) & 1], ((n + 1) >> 1) & 1);
+                    if (ctl->abort) break;
+                    tc_fence_after_sync();
+                    issue_p(n + 1);
+                }
+            }
+        }
+    } else if (tid < kComputeThreads) {
+        // =============================== compute threads: state slice S[c = row][s], slots sb .. sb+31 of the half
+        float S[kHS];
+#pragma unroll
+        for (int s = 0; s < kHS; ++s) S[s] = (a.S0 && d0 + row < a.D) ? a.S0[((size_t)bh * kM + sb + s) * a.D + d0 + row] : 0.f;
+        auto chunk_e = [&](int n) {
+            const int last = min(chunk_t0(n) + kCT, span.t_end) - 1;
+            return a.E[(((size_t)b * a.T + last) * H2 + h2) * kM + tid];
+        };
+        float e_next = 0.f;
+        if (tid < kM) {
+            ctl->egc[0][tid] = chunk_e(0);
+            if (nchunks > 1) e_next = chunk_e(1);
+        }
+        compute_sync();
+        store_state_split3<REV>(sSb, row, sb, S, ctl->egc[0]);
+        publish(&ctl->bar_sb, tid);
+        for (int n = 0; n < nchunks; ++n) {
+            const float* egc = ctl->egc[n & 1];
+            if (tid < kM && n + 1 < nchunks) {
+                ctl->egc[(n + 1) & 1][tid] = e_next;
+                if (n + 2 < nchunks) e_next = chunk_e(n + 2);
+            }
+            WIDE_WAIT(&ctl->bar_p, n & 1);
+            tc_fence_after_sync();
+            mask_row_split3<REV>(tmem, wq, row, half, kWvP, kWvPlow);
+            publish(&ctl->bar_pm, tid);
+
+            // state update: forward S <- exp(G_C) (S + U), reverse S <- exp(G_C) S + U
+            WIDE_WAIT(&ctl->bar_mma1, n & 1);
+            tc_fence_after_sync();
+            {
+                float v[kHS];
+                tmem_ld32(tmem_row_addr(tmem, wq, kWvU + sb), v);
+#pragma unroll
+                for (int e = 0; e < kHS; ++e) S[e] = REV ? fmaf(S[e], egc[sb + e], v[e]) : (S[e] + v[e]) * egc[sb + e];
+            }
+            store_state_split3<REV>(sSb, row, sb, S, ctl->egc[(n + 1) & 1]);
+            publish(&ctl->bar_sb, tid);
+
+            WIDE_WAIT(&ctl->bar_mma2[n & 1], (n >> 1) & 1);
+            tc_fence_after_sync();
+            {
+                float vo[kHS], vi[kHS];
+                tmem_ld32(tmem_row_addr(tmem, wq, kWvO + kM * (n & 1) + sb), vo);
+                tmem_ld32(tmem_row_addr(tmem, wq, kWvI + kM * (n & 1) + sb), vi);
+#pragma unroll
+                for (int e = 0; e < kHS; ++e) vo[e] += vi[e];
+                unsigned char* panel = sX + (4 * (n & 1) + half) * kPanelB;
+#pragma unroll
+                for (int c = 0; c < kHS / 4; ++c)
+                    *reinterpret_cast<float4*>(panel + swz128(row, c)) =
+                        make_float4(vo[4 * c], vo[4 * c + 1], vo[4 * c + 2], vo[4 * c + 3]);
+            }
+            if (publish_and_vote(&ctl->bar_out[n & 1], tid, ctl->abort != 0)) break;
+        }
+        if (!ctl->abort && a.Send && d0 + row < a.D) {
+#pragma unroll
+            for (int s = 0; s < kHS; ++s) a.Send[((size_t)bh * kM + sb + s) * a.D + d0 + row] = S[s];
+        }
+    }
+    wide_end(ctl, tid, warp, tmem, dev_status);
+}
+
+// ======================================================================================
+// key_side: out_i = (uq_i scaled) S + sum_j A_ij xv_j,  A_ij = sum over both halves of uq_i[s] uk_j[s] decay_ij[s].
+// Two parts of every derived operand.  Accumulator columns: A 128, output 128, state product 128 for each half
+// (high | low part).  End states are not given out (their accuracy would be that of two parts): state_scan_wide.
+// ======================================================================================
+constexpr int kWkA = 0, kWkO = 128, kWkU = 256;
+
+template <bool REV>
+__global__ void __launch_bounds__(kScanThreads, 1)
+key_side_wide_kernel(const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapUq,
+                     const __grid_constant__ CUtensorMap mapUk, const __grid_constant__ CUtensorMap mapO,
+                     const __grid_constant__ KeySideArgs a, const int* __restrict__ strong_flag, int32_t* dev_status) {
+    if (strong_flag[blockIdx.x] != 0) return;       // the CUDA-core kernel takes this (batch, head)
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    unsigned char* sXv = smem;                       // xv tile, 2 panels; ... the output rows once it is consumed
+    unsigned char* sQK = sXv + 2 * kPanelB;          // half 0, half 1: [uq_hi, uk_hi, uq_lo, uk_lo], 8 panels
+    unsigned char* sSb = sQK + 8 * kPanelB;          // state copy, K-major B: half 0 hi, lo, half 1 hi, lo, 4 panels
+    WideCtl* ctl = reinterpret_cast<WideCtl*>(sSb + 4 * kPanelB);
+
+    const int tid = threadIdx.x, warp = tid >> 5, wq = warp & 3, half = (tid >> 7) & 1, row = tid & 127;
+    const ScanSpan span = scan_span(blockIdx.x, a.H, a.T, a.nseg, a.tseg);
+    const int bh = blockIdx.x, slice = blockIdx.y, b = span.b, h = span.h;
+    const int d0 = slice * kDST;
+
+    wide_begin(ctl, tid, warp);
+    const uint32_t tmem = ctl->tmem_slot;
+    const int nchunks = (span.t_end - span.t0 + kCT - 1) / kCT;
+    auto chunk_t0 = [&](int n) { return span.t0 + (REV ? nchunks - 1 - n : n) * kCT; };
+
+    if (warp == kCopyWarp) {
+        if (elect_one()) {
+            // =============================== copy lane
+            auto load_v = [&](int n) {
+                mbar_expect_tx(&ctl->bar_x[0], 2 * kPanelB);
+                tma_load_4d(sXv, &mapV, &ctl->bar_x[0], d0, h, chunk_t0(n), b);
+                tma_load_4d(sXv + kPanelB, &mapV, &ctl->bar_x[0], d0 + 64, h, chunk_t0(n), b);
+            };
+            auto load_qk = [&](int n, int hf) {
+                const int t = chunk_t0(n);
+                unsigned char* s = sQK + 4 * hf * kPanelB;
+                mbar_expect_tx(&ctl->bar_w[hf], 4 * kPanelB);
+                tma_load_4d(s, &mapUq, &ctl->bar_w[hf], 0, 2 * h + hf, t, b);
+                tma_load_4d(s + kPanelB, &mapUk, &ctl->bar_w[hf], 0, 2 * h + hf, t, b);
+                tma_load_4d(s + 2 * kPanelB, &mapUq, &ctl->bar_w[hf], 64, 2 * h + hf, t, b);
+                tma_load_4d(s + 3 * kPanelB, &mapUk, &ctl->bar_w[hf], 64, 2 * h + hf, t, b);
+            };
+            prefetch_tmap(&mapV); prefetch_tmap(&mapUq); prefetch_tmap(&mapUk); prefetch_tmap(&mapO);
+            load_qk(0, 0);
+            load_qk(0, 1);
+            load_v(0);
+            for (int n = 0; n < nchunks && !ctl->abort; ++n) {
+                if (n + 1 < nchunks) {
+                    tma_prefetch_4d(&mapV, d0, h, chunk_t0(n + 1), b);
+                    if (d0 + 64 < a.D) tma_prefetch_4d(&mapV, d0 + 64, h, chunk_t0(n + 1), b);
+                }
+                for (int hf = 0; hf < 2; ++hf) {
+                    WIDE_WAIT(&ctl->bar_free[hf], n & 1);
+                    if (ctl->abort) break;
+                    if (n + 1 < nchunks) load_qk(n + 1, hf);
+                }
+                WIDE_WAIT(&ctl->bar_out[0], n & 1);
+                if (ctl->abort) break;
+                tma_store_4d(&mapO, sXv, d0, h, chunk_t0(n), b);
+                if (d0 + 64 < a.D) tma_store_4d(&mapO, sXv + kPanelB, d0 + 64, h, chunk_t0(n), b);
+                bulk_commit();
+                bulk_wait_read();
+                if (n + 1 < nchunks) load_v(n + 1);
+            }
+        }
+    } else if (warp == kMmaWarp) {
+        if (elect_one()) {
+            // =============================== MMA lane
+            constexpr uint32_t idescA = make_idesc(128, 128, false, false);   // Q~ K~^T
+            constexpr uint32_t idescO = make_idesc(128, kDST, false, false);  // Q~ x state copy (K-major B)
+            constexpr uint32_t idescU = make_idesc(128, 2 * kM, true, true);  // xv^T (MN-major A) x [K~_hi | K~_lo] (MN-major B)
+            constexpr uint32_t idescV = make_idesc(128, kDST, false, true);   // masked A x xv (MN-major B)
+            const uint64_t dV = desc_mnmajor(smem_u32(sXv), 0, kPanelB);
+            auto issue_a = [&](int n) {
+                for (int hf = 0; hf < 2; ++hf) {
+                    WIDE_WAIT(&ctl->bar_w[hf], n & 1);
+                    if (ctl->abort) return;
+                    tc_fence_after_sync();
+                    const uint32_t qk = smem_u32(sQK + 4 * hf * kPanelB);
+                    const uint64_t dQh = desc_kmajor(qk, 0), dKh = desc_kmajor(qk + kPanelB, 0);
+                    const uint64_t dQl = desc_kmajor(qk + 2 * kPanelB, 0), dKl = desc_kmajor(qk + 3 * kPanelB, 0);
+#pragma unroll
+                    for (int kk = 0; kk < kM / 16; ++kk)
+                        mma_bf16(tmem + kWkA, desc_advance(dQh, step_kmaj(kk)), desc_advance(dKh, step_kmaj(kk)), idescA, hf + kk > 0);
+#pragma unroll
+                    for (int kk = 0; kk < kM / 16; ++kk)
+                        mma_bf16(tmem + kWkA, desc_advance(dQl, step_kmaj(kk)), desc_advance(dKh, step_kmaj(kk)), idescA, true);
+#pragma unroll
+                    for (int kk = 0; kk < kM / 16; ++kk)
+                        mma_bf16(tmem + kWkA, desc_advance(dQh, step_kmaj(kk)), desc_advance(dKl, step_kmaj(kk)), idescA, true);
+                }
+                mma_commit(&ctl->bar_p);
+            };
+            issue_a(0);
+            for (int n = 0; n < nchunks && !ctl->abort; ++n) {
+                WIDE_WAIT(&ctl->bar_x[0], n & 1);
+                WIDE_WAIT(&ctl->bar_sb, n & 1);
+                if (ctl->abort) break;
+                tc_fence_after_sync();
+                for (int hf = 0; hf < 2; ++hf) {
+                    // the decayed uk read MN-major, its high and low parts as one N = 128 operand (two panels apart)
+                    const uint64_t dKm = desc_mnmajor(smem_u32(sQK + (4 * hf + 1) * kPanelB), 0, 2 * kPanelB);
+#pragma unroll
+                    for (int kk = 0; kk < kCT / 16; ++kk)
+                        mma_bf16(tmem + kWkU + 2 * kM * hf, desc_advance(dV, step_mnmaj(kk)), desc_advance(dKm, step_mnmaj(kk)),
+                                 idescU, kk > 0);
+                }
+                // the output accumulator: the rows of chunk n-1 have been read out
+                if (n >= 1) WIDE_WAIT(&ctl->bar_out[0], (n - 1) & 1);
+                if (ctl->abort) break;
+                tc_fence_after_sync();
+                for (int hf = 0; hf < 2; ++hf) {
+                    const uint32_t qk = smem_u32(sQK + 4 * hf * kPanelB), sp = smem_u32(sSb + 2 * hf * kPanelB);
+                    const uint64_t dQh = desc_kmajor(qk, 0), dQl = desc_kmajor(qk + 2 * kPanelB, 0);
+                    const uint64_t dSh = desc_kmajor(sp, 0), dSl = desc_kmajor(sp + kPanelB, 0);
+#pragma unroll
+                    for (int kk = 0; kk < kM / 16; ++kk)
+                        mma_bf16(tmem + kWkO, desc_advance(dQh, step_kmaj(kk)), desc_advance(dSh, step_kmaj(kk)), idescO, hf + kk > 0);
+#pragma unroll
+                    for (int kk = 0; kk < kM / 16; ++kk)
+                        mma_bf16(tmem + kWkO, desc_advance(dQl, step_kmaj(kk)), desc_advance(dSh, step_kmaj(kk)), idescO, true);
+#pragma unroll
+                    for (int kk = 0; kk < kM / 16; ++kk)
+                        mma_bf16(tmem + kWkO, desc_advance(dQh, step_kmaj(kk)), desc_advance(dSl, step_kmaj(kk)), idescO, true);
+                    mma_commit(&ctl->bar_free[hf]);
+                }
+                mma_commit(&ctl->bar_mma1);
+                // intra-chunk product (masked A and its rounding residual) on top of the inter-chunk one
+                WIDE_WAIT(&ctl->bar_pm, n & 1);
+                if (ctl->abort) break;
+                tc_fence_after_sync();
+#pragma unroll
+                for (int ip = 0; ip < 2; ++ip)
+#pragma unroll
+                    for (int kk = 0; kk < kCT / 16; ++kk)
+                        mma_bf16_ta(tmem + kWkO, tmem + kWkA + 64 * (kk >> 2) + 32 * ip + 8 * (kk & 3),
+                                    desc_advance(dV, step_mnmaj(kk)), idescV, true);
+                mma_commit(&ctl->bar_mma2[0]);
+                if (n + 1 < nchunks) issue_a(n + 1);
+            }
+        }
+    } else if (tid < kComputeThreads) {
+        // =============================== compute threads: S[c = row][s] of the slots of half `half`, in two groups of 32
+        float S[2][kHS];
+        const float* S0 = a.S0 ? a.S0 + ((size_t)bh * kWide + kM * half) * a.D + d0 + row : nullptr;
+#pragma unroll
+        for (int g = 0; g < 2; ++g)
+#pragma unroll
+            for (int s = 0; s < kHS; ++s) S[g][s] = (S0 && d0 + row < a.D) ? S0[(size_t)(kHS * g + s) * a.D] : 0.f;
+        auto chunk_e = [&](int n) {
+            const int last = min(chunk_t0(n) + kCT, span.t_end) - 1;
+            return a.E[(((size_t)b * a.T + last) * a.H + h) * kWide + tid];
+        };
+        float e_next = 0.f;
+        if (tid < kWide) {
+            ctl->egc[0][tid] = chunk_e(0);
+            if (nchunks > 1) e_next = chunk_e(1);
+        }
+        compute_sync();
+        unsigned char* panels = sSb + 2 * half * kPanelB;
+#pragma unroll
+        for (int g = 0; g < 2; ++g)
+            store_state_row_split<REV>(panels, panels + kPanelB, row, kHS * g, S[g], ctl->egc[0] + kM * half);
+        publish(&ctl->bar_sb, tid);
+        for (int n = 0; n < nchunks; ++n) {
+            const float* egc = ctl->egc[n & 1] + kM * half;
+            if (tid < kWide && n + 1 < nchunks) {
+                ctl->egc[(n + 1) & 1][tid] = e_next;
+                if (n + 2 < nchunks) e_next = chunk_e(n + 2);
+            }
+            WIDE_WAIT(&ctl->bar_p, n & 1);
+            tc_fence_after_sync();
+            mask_row_in_tmem<REV, true>(tmem, wq, row, half, kWkA);
+            publish(&ctl->bar_pm, tid);
+
+            // state update: forward S <- exp(G_C) (S + U), reverse S <- exp(G_C) S + U
+            WIDE_WAIT(&ctl->bar_mma1, n & 1);
+            tc_fence_after_sync();
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+                float v[kHS], vl[kHS];
+                tmem_ld32(tmem_row_addr(tmem, wq, kWkU + 2 * kM * half + kHS * g), v);
+                tmem_ld32(tmem_row_addr(tmem, wq, kWkU + 2 * kM * half + kM + kHS * g), vl);
+#pragma unroll
+                for (int e = 0; e < kHS; ++e) {
+                    const float u = v[e] + vl[e], c = egc[kHS * g + e];
+                    S[g][e] = REV ? fmaf(S[g][e], c, u) : (S[g][e] + u) * c;
+                }
+                store_state_row_split<REV>(panels, panels + kPanelB, row, kHS * g, S[g], ctl->egc[(n + 1) & 1] + kM * half);
+            }
+            publish(&ctl->bar_sb, tid);
+
+            WIDE_WAIT(&ctl->bar_mma2[0], n & 1);
+            tc_fence_after_sync();
+#pragma unroll 1
+            for (int c0 = 0; c0 < 64; c0 += 32) {
+                float v[32];
+                tmem_ld32(tmem_row_addr(tmem, wq, kWkO + 64 * half + c0), v);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const float x[8] = {v[8 * c], v[8 * c + 1], v[8 * c + 2], v[8 * c + 3],
+                                        v[8 * c + 4], v[8 * c + 5], v[8 * c + 6], v[8 * c + 7]};
+                    store_chunk(sXv + half * kPanelB, row, (c0 >> 3) + c, x);
+                }
+            }
+            if (publish_and_vote(&ctl->bar_out[0], tid, ctl->abort != 0)) break;
+        }
+    }
+    wide_end(ctl, tid, warp, tmem, dev_status);
+}
+
+// ======================================================================================
+// End states only (and those that key_side does not give out): U = X^T W of every chunk with all three parts, no product
+// depends on the state.  The sets of one launch as in state_scan_kernel (chunk_tc_lean.cu): two stages of [X | W] (10
+// panels), the accumulator by chunk parity.
+// ======================================================================================
+struct WideScanArgs {
+    ValueSideArgs set[2];
+    int slices0;
+};
+
+template <bool REV>
+__global__ void __launch_bounds__(kScanThreads, 1)
+state_scan_wide_kernel(const __grid_constant__ CUtensorMap mapX0, const __grid_constant__ CUtensorMap mapW0,
+                       const __grid_constant__ CUtensorMap mapX1, const __grid_constant__ CUtensorMap mapW1,
+                       const __grid_constant__ WideScanArgs sets, const int* __restrict__ strong_flag, int32_t* dev_status) {
+    const bool second = (int)blockIdx.y >= sets.slices0;
+    const CUtensorMap &mapX = second ? mapX1 : mapX0, &mapW = second ? mapW1 : mapW0;
+    const ValueSideArgs& a = sets.set[second];
+    const int slice = second ? blockIdx.y - sets.slices0 : blockIdx.y;
+    const int H2 = 2 * a.H;
+    const ScanSpan span = scan_span(blockIdx.x, H2, a.T, a.nseg, a.tseg);
+    const int bh = blockIdx.x, b = span.b, h2 = span.h, h = h2 >> 1;
+    if (strong_flag[(bh / H2) * a.H + h] != 0) return;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    WideCtl* ctl = reinterpret_cast<WideCtl*>(smem + 10 * kPanelB);
+    const int tid = threadIdx.x, warp = tid >> 5, wq = warp & 3, half = (tid >> 7) & 1, row = tid & 127;
+    const int sb = kHS * half, d0 = slice * kDST;
+    wide_begin(ctl, tid, warp);
+    const uint32_t tmem = ctl->tmem_slot;
+    const int nchunks = (span.t_end - span.t0 + kCT - 1) / kCT;
+    auto chunk_t0 = [&](int n) { return span.t0 + (REV ? nchunks - 1 - n : n) * kCT; };
+
+    // bar_x: a stage has landed; bar_free: ... is consumed; bar_mma2: the product of a chunk is complete; bar_out: ... has
+    // been read out -- all by chunk parity
+    if (warp == kCopyWarp) {
+        if (elect_one()) {
+            auto load = [&](int n) {
+                const int t = chunk_t0(n), st = n & 1;
+                unsigned char* s = smem + 5 * st * kPanelB;
+                mbar_expect_tx(&ctl->bar_x[st], 5 * kPanelB);
+                tma_load_4d(s, &mapX, &ctl->bar_x[st], d0, h, t, b);
+                tma_load_4d(s + kPanelB, &mapX, &ctl->bar_x[st], d0 + 64, h, t, b);
+                for (int i = 0; i < 3; ++i) tma_load_4d(s + (2 + i) * kPanelB, &mapW, &ctl->bar_x[st], 64 * i, h2, t, b);
+            };
+            prefetch_tmap(&mapX); prefetch_tmap(&mapW);
+            for (int n = 0; n < 2 && n < nchunks; ++n) load(n);
+            for (int n = 0; n + 2 < nchunks && !ctl->abort; ++n) {
+                WIDE_WAIT(&ctl->bar_free[n & 1], (n >> 1) & 1);
+                if (ctl->abort) break;
+                load(n + 2);
+            }
+        }
+    } else if (warp == kMmaWarp) {
+        if (elect_one()) {
+            constexpr uint32_t idescU = make_idesc(128, kM, true, true);   // X^T (MN-major A) x part (MN-major B)
+            for (int n = 0; n < nchunks && !ctl->abort; ++n) {
+                const uint32_t s = smem_u32(smem + 5 * (n & 1) * kPanelB);
+                const uint64_t dX = desc_mnmajor(s, 0, kPanelB);
+                WIDE_WAIT(&ctl->bar_x[n & 1], (n >> 1) & 1);
+                if (n >= 2) WIDE_WAIT(&ctl->bar_out[n & 1], ((n - 2) >> 1) & 1);
+                if (ctl->abort) break;
+                tc_fence_after_sync();
+#pragma unroll
+                for (int i = 2; i >= 0; --i) {
+                    const uint64_t dW = desc_mnmajor(s + (2 + i) * kPanelB, 0, kPanelB);
+#pragma unroll
+                    for (int kk = 0; kk < kCT / 16; ++kk)
+                        mma_bf16(tmem + kM * (n & 1), desc_advance(dX, step_mnmaj(kk)), desc_advance(dW, step_mnmaj(kk)), idescU,
+                                 i < 2 || kk > 0);
+                }
+                mma_commit(&ctl->bar_mma2[n & 1]);
+                mma_commit(&ctl->bar_free[n & 1]);
+            }
+        }
+    } else if (tid < kComputeThreads) {
+        float S[kHS];
+#pragma unroll
+        for (int s = 0; s < kHS; ++s) S[s] = (a.S0 && d0 + row < a.D) ? a.S0[((size_t)bh * kM + sb + s) * a.D + d0 + row] : 0.f;
+        auto chunk_e = [&](int n) {
+            const int last = min(chunk_t0(n) + kCT, span.t_end) - 1;
+            return a.E[(((size_t)b * a.T + last) * H2 + h2) * kM + tid];
+        };
+        float e_next = 0.f;
+        if (tid < kM) {
+            ctl->egc[0][tid] = chunk_e(0);
+            if (nchunks > 1) e_next = chunk_e(1);
+        }
+        compute_sync();
+        for (int n = 0; n < nchunks; ++n) {
+            const float* egc = ctl->egc[n & 1];
+            if (tid < kM && n + 1 < nchunks) {
+                ctl->egc[(n + 1) & 1][tid] = e_next;
+                if (n + 2 < nchunks) e_next = chunk_e(n + 2);
+            }
+            WIDE_WAIT(&ctl->bar_mma2[n & 1], (n >> 1) & 1);
+            tc_fence_after_sync();
+            float v[kHS];
+            tmem_ld32(tmem_row_addr(tmem, wq, kM * (n & 1) + sb), v);
+#pragma unroll
+            for (int e = 0; e < kHS; ++e) S[e] = REV ? fmaf(S[e], egc[sb + e], v[e]) : (S[e] + v[e]) * egc[sb + e];
+            if (publish_and_vote(&ctl->bar_out[n & 1], tid, ctl->abort != 0)) break;
+        }
+        if (!ctl->abort && d0 + row < a.D) {
+#pragma unroll
+            for (int s = 0; s < kHS; ++s) a.Send[((size_t)bh * kM + sb + s) * a.D + d0 + row] = S[s];
+        }
+    }
+    wide_end(ctl, tid, warp, tmem, dev_status);
+}
+
+constexpr size_t kSmemWide = 1024 + 14 * kPanelB + sizeof(WideCtl);      // all three: the largest is 14 panels
+
+// one set, or two in one launch
+cudaError_t launch_state_scan_wide(const ValueSideArgs& k, const ValueSideArgs* v, int reverse, const int* strong_flag,
+                                   cudaStream_t st, int32_t* dev_status) {
+    WideScanArgs sets{{k, v != nullptr ? *v : k}, tc_value_side_slices(k.D)};
+    CUtensorMap mx[2], mw[2];
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < 2; ++i) {
+        const ValueSideArgs& a = sets.set[i];
+        if (e == cudaSuccess) e = make_tensor_map_bthd(&mx[i], a.xk, a.B, a.T, a.H, a.D, kCT, 2);
+        if (e == cudaSuccess) e = make_tensor_map_bthd(&mw[i], a.wd, a.B, a.T, 2 * a.H, kParts, kCT, 2);
+    }
+    if (e != cudaSuccess) return e;
+    dim3 grid(k.B * k.nseg * 2 * k.H, sets.slices0 + (v != nullptr ? tc_value_side_slices(v->D) : 0));
+    if (reverse) {
+        e = prepare<state_scan_wide_kernel<true>>(kSmemWide);
+        if (e != cudaSuccess) return e;
+        state_scan_wide_kernel<true><<<grid, kScanThreads, kSmemWide, st>>>(mx[0], mw[0], mx[1], mw[1], sets, strong_flag, dev_status);
+    } else {
+        e = prepare<state_scan_wide_kernel<false>>(kSmemWide);
+        if (e != cudaSuccess) return e;
+        state_scan_wide_kernel<false><<<grid, kScanThreads, kSmemWide, st>>>(mx[0], mw[0], mx[1], mw[1], sets, strong_flag, dev_status);
+    }
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_value_side_wide(const ValueSideArgs& a, int reverse, const int* strong_flag, cudaStream_t st,
+                                   int32_t* dev_status) {
+    if (!tc_dim_ok(a.D) || a.wd == nullptr || a.E == nullptr || strong_flag == nullptr) return cudaErrorNotSupported;
+    CUtensorMap mq, mk, mw, mo;
+    cudaError_t e = make_tensor_map_bthd(&mq, a.xq, a.B, a.T, a.H, a.D, kCT, 2);
+    if (e == cudaSuccess) e = make_tensor_map_bthd(&mk, a.xk, a.B, a.T, a.H, a.D, kCT, 2);
+    if (e == cudaSuccess) e = make_tensor_map_bthd(&mw, a.wd, a.B, a.T, 2 * a.H, kParts, kCT, 2);
+    if (e == cudaSuccess) e = make_tensor_map_sliced(&mo, a.out, tc_value_side_slices(a.D), a.B, a.T, 2 * a.H, kM, kCT, 4);
+    if (e != cudaSuccess) return e;
+    dim3 grid(a.B * a.nseg * 2 * a.H, tc_value_side_slices(a.D));
+    if (reverse) {
+        e = prepare<value_side_wide_kernel<true>>(kSmemWide);
+        if (e != cudaSuccess) return e;
+        value_side_wide_kernel<true><<<grid, kScanThreads, kSmemWide, st>>>(mq, mk, mw, mo, a, strong_flag, dev_status);
+    } else {
+        e = prepare<value_side_wide_kernel<false>>(kSmemWide);
+        if (e != cudaSuccess) return e;
+        value_side_wide_kernel<false><<<grid, kScanThreads, kSmemWide, st>>>(mq, mk, mw, mo, a, strong_flag, dev_status);
+    }
+    e = cudaGetLastError();
+    return e == cudaSuccess ? launch_value_side_simt(a, GSA_BF16, kWide, reverse, st, strong_flag) : e;
+}
+
+cudaError_t launch_key_side_wide(const KeySideArgs& a, int reverse, const int* strong_flag, cudaStream_t st,
+                                 int32_t* dev_status) {
+    if (!tc_dim_ok(a.D) || a.uq_d == nullptr || a.uk_d == nullptr || a.E == nullptr || strong_flag == nullptr)
+        return cudaErrorNotSupported;
+    CUtensorMap mv, muq, muk, mo;
+    cudaError_t e = make_tensor_map_bthd(&mv, a.xv, a.B, a.T, a.H, a.D, kCT, 2);
+    if (e == cudaSuccess) e = make_tensor_map_bthd(&muq, a.uq_d, a.B, a.T, 2 * a.H, kParts, kCT, 2);
+    if (e == cudaSuccess) e = make_tensor_map_bthd(&muk, a.uk_d, a.B, a.T, 2 * a.H, kParts, kCT, 2);
+    if (e == cudaSuccess) e = make_tensor_map_bthd(&mo, a.out, a.B, a.T, a.H, a.D, kCT, 2);
+    if (e != cudaSuccess) return e;
+    dim3 grid(a.B * a.nseg * a.H, tc_value_side_slices(a.D));
+    if (reverse) {
+        e = prepare<key_side_wide_kernel<true>>(kSmemWide);
+        if (e != cudaSuccess) return e;
+        key_side_wide_kernel<true><<<grid, kScanThreads, kSmemWide, st>>>(mv, muq, muk, mo, a, strong_flag, dev_status);
+    } else {
+        e = prepare<key_side_wide_kernel<false>>(kSmemWide);
+        if (e != cudaSuccess) return e;
+        key_side_wide_kernel<false><<<grid, kScanThreads, kSmemWide, st>>>(mv, muq, muk, mo, a, strong_flag, dev_status);
+    }
+    e = cudaGetLastError();
+    if (e == cudaSuccess && a.Send != nullptr) {
+        ValueSideArgs s{a.xv, a.xv, a.uk, a.G, a.S0, a.Send, nullptr, a.B, a.T, a.H, a.D, a.uk_d, 1};
+        s.nseg = a.nseg; s.tseg = a.tseg; s.E = a.E;
+        e = launch_state_scan_wide(s, nullptr, reverse, strong_flag, st, dev_status);
+    }
+    return e == cudaSuccess ? launch_key_side_simt(a, GSA_BF16, kWide, reverse, st, strong_flag) : e;
+}
+
+cudaError_t launch_state_scans_wide(const ValueSideArgs& k, const ValueSideArgs& v, int reverse, const int* strong_flag,
+                                    cudaStream_t st, int32_t* dev_status) {
+    cudaError_t e = launch_state_scan_wide(k, &v, reverse, strong_flag, st, dev_status);
+    if (e == cudaSuccess) e = launch_value_side_simt(k, GSA_BF16, kWide, reverse, st, strong_flag);
+    return e == cudaSuccess ? launch_value_side_simt(v, GSA_BF16, kWide, reverse, st, strong_flag) : e;
+}
+
+}  // namespace gsa

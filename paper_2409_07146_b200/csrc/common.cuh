@@ -89,6 +89,7 @@ struct ValueSideArgs {
     // T runs as nseg segments of tseg tokens (the last one shorter), each an independent scan: S0, Send and the
     // strong-decay flags are then [B, nseg, H, ..]
     int nseg = 1, tseg = 0;
+    const float* E = nullptr;         // kernels for 128 slots: exp(G), see launch_gate_cumsum_wide
 };
 struct KeySideArgs {
     const float* uq; const float* uk; const float* G;
@@ -102,6 +103,7 @@ struct KeySideArgs {
     const void* uq_d; const void* uk_d;
     int single;                       // as in ValueSideArgs
     int nseg = 1, tseg = 0;           // likewise
+    const float* E = nullptr;         // likewise
 };
 
 // What scan `bhs` of a launch over B * nseg * H scans works on: batch element, head and the tokens [t0, t_end).
@@ -150,13 +152,21 @@ struct PendingDecay {
     // != 0: the slot kernel serves ONLY the pairs flagged in `strong` (the fused chunk kernel has done
     // the others on chip): rows with a pending factor are skipped
     int strong_only;
+    // 128 slots on the tensor-core kernels: G holds exp(G) itself, and a kernel may see the tensors as H = 2 x heads of
+    // 64 slots (half_heads), both of which have the flag of their head
+    int wide = 0, half_heads = 0;
+    __host__ __device__ bool pending_at(int b, int t, int h) const {
+        if (G == nullptr) return false;
+        const int seg = nseg == 1 ? 0 : t / tseg;
+        return strong[(b * nseg + seg) * (H >> half_heads) + (h >> half_heads)] == 0;
+    }
     // row r = t * H + h of batch element b of a [B,T,H,M] tensor (32-bit arithmetic: T * H < 2^31)
     __host__ __device__ bool pending(int b, int r) const {
-        if (G == nullptr) return false;
-        const int t = r / H, h = r - t * H;
-        const int seg = nseg == 1 ? 0 : t / tseg;
-        return strong[(b * nseg + seg) * H + h] == 0;
+        const int t = r / H;
+        return pending_at(b, t, r - t * H);
     }
+    // the factor exp(-G_i) left out of the time-reversed partial sums, from an element of G (0 past the sequence end)
+    __device__ float reverse_factor(float g) const { return wide ? (g > 0.f ? 1.f / g : 0.f) : __expf(-g); }
 };
 
 // launchers (definitions in the .cu files); all return cudaGetLastError() of the launch
@@ -170,6 +180,12 @@ cudaError_t launch_gate_cumsum(const float* gate, int gate_kind, float inv_tau, 
                                int B, int T, int H, int M, int chunk, int* strong_flag, int nseg, int tseg,
                                void* decayed, int fast_log, cudaStream_t st, const int* cu_seqlens = nullptr,
                                int nseq = 0);
+// The same for the tensor-core kernels with 128 slots, M = 2 x 64: `decayed` are bf16 [B,T,2H,192] rows [high | middle |
+// low part] of I exp(-G), E = exp(G), local to chunks of 128 tokens; both, and log a, to fp32 accuracy whatever the io
+// type.  G is local to 64 tokens, the chunks of the CUDA-core kernels that take the flagged pairs.
+cudaError_t launch_gate_cumsum_wide(const float* gate, int gate_kind, float inv_tau, float* G, float* I, float* E, int B, int T,
+                                    int H, int* strong_flag, int nseg, int tseg, void* decayed, cudaStream_t st,
+                                    const int* cu_seqlens, int nseq);
 // ABC (Eq. 3-4): write weights phi (cumulative softmax over time of the scores) into I, zeros into G, phi as the
 // decayed bf16 rows; and the gradient w.r.t. the scores from phi and the input-gate gradient partial sums
 cudaError_t launch_abc_write(const float* s_in, float* G, float* I, void* decayed, int B, int T, int H, int M, cudaStream_t st);
@@ -215,10 +231,12 @@ cudaError_t launch_gate_grad(const float* u, const float* I, const float* dIk_pa
                              PendingDecay pend, cudaStream_t st, int32_t* dev_status, const int* cu_seqlens = nullptr,
                              int nseq = 0);
 int gate_grad_blocks(int T);       // entries per (b,h,slot) of launch_gate_grad's scratch
+// strong_flag != NULL: beside the tensor-core kernels, for the flagged (batch, head) pairs alone; value_side then sums its
+// slices to their 128-wide ones
 cudaError_t launch_value_side_simt(const ValueSideArgs& a, int io, int M, int reverse,
-                                   cudaStream_t st);
+                                   cudaStream_t st, const int* strong_flag = nullptr);
 cudaError_t launch_key_side_simt(const KeySideArgs& a, int io, int M, int reverse,
-                                 cudaStream_t st);
+                                 cudaStream_t st, const int* strong_flag = nullptr);
 // tcgen05 (bf16 tensor-core) versions of the two primitives; bf16 io only.
 bool tc_supported(int d_k, int d_v, int M);
 bool tc_dim_ok(int D);
@@ -228,6 +246,13 @@ cudaError_t launch_value_side_tc(const ValueSideArgs& a, int M, int reverse, con
                                  cudaStream_t st, int32_t* dev_status);
 cudaError_t launch_key_side_tc(const KeySideArgs& a, int M, int reverse, const int* strong_flag,
                                cudaStream_t st, int32_t* dev_status);
+// 128 slots (chunk_tc_wide.cu): the slot tensors as above, the decayed rows as launch_gate_cumsum_wide writes them
+cudaError_t launch_value_side_wide(const ValueSideArgs& a, int reverse, const int* strong_flag, cudaStream_t st,
+                                   int32_t* dev_status);
+cudaError_t launch_key_side_wide(const KeySideArgs& a, int reverse, const int* strong_flag, cudaStream_t st,
+                                 int32_t* dev_status);
+cudaError_t launch_state_scans_wide(const ValueSideArgs& k, const ValueSideArgs& v, int reverse, const int* strong_flag,
+                                    cudaStream_t st, int32_t* dev_status);
 // the general scan as a launch of its own, for the flagged pairs (beside the fused kernel; forward direction)
 cudaError_t launch_value_side_general(const ValueSideArgs& a, const int* strong_flag, cudaStream_t st, int32_t* dev_status);
 cudaError_t launch_key_side_general(const KeySideArgs& a, const int* strong_flag, cudaStream_t st, int32_t* dev_status);

@@ -21,6 +21,12 @@ __device__ __forceinline__ void split_bf16x2(float x0, float x1, uint32_t& hi, u
     const __nv_bfloat162 l = __floats2bfloat162_rn(x0 - __uint_as_float(hi << 16), x1 - __uint_as_float(hi & 0xffff0000u));
     lo = *reinterpret_cast<const uint32_t*>(&l);
 }
+// ... as three parts: bits 0-7, 8-15 and 16-23 of the mantissas
+__device__ __forceinline__ void split_bf16x3(float x0, float x1, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
+    hi = *reinterpret_cast<const uint32_t*>(&h);
+    split_bf16x2(x0 - __uint_as_float(hi << 16), x1 - __uint_as_float(hi & 0xffff0000u), mid, lo);
+}
 template <int M>
 __device__ __forceinline__ void store_split2(__nv_bfloat16* row, int c, float x0, float x1) {
     uint32_t hi, lo;
@@ -53,14 +59,16 @@ __device__ __forceinline__ bool sequence_starts_at(const int* __restrict__ cu, i
 constexpr float kReset = 28.f;
 constexpr float kLeastReset = 20.f;
 
-template <int M>
+// WIDE: the halves of 128 slots as 2 H heads of 64 (see launch_gate_cumsum_wide), which share their head's flag.
+template <int M, bool WIDE = false>
 __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) gate_cumsum_kernel(const float* __restrict__ gate,
                                                             int gate_kind, float inv_tau,
                                                             float* __restrict__ G,
                                                             float* __restrict__ I, int T, int H,
                                                             int chunk, int* __restrict__ strong_flag, int nseg, int tseg,
                                                             __nv_bfloat16* __restrict__ decayed, int fast_log,
-                                                            const int* __restrict__ cu_seqlens, int nseq) {
+                                                            const int* __restrict__ cu_seqlens, int nseq,
+                                                            float* __restrict__ E = nullptr) {
     __shared__ double group_sum[16][M];
     const int s = 2 * threadIdx.x, grp = threadIdx.y;          // blockDim.y = chunk / 8 <= 16
     const int n = blockIdx.y;
@@ -139,17 +147,21 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
     group_sum[grp][s] = acc0;
     group_sum[grp][s + 1] = acc1;
     __syncthreads();
-    double before0 = 0.0, before1 = 0.0;
+    double before0 = 0.0, before1 = 0.0, half0 = 0.0, half1 = 0.0;       // (half: since the last multiple of 64 tokens)
     for (int q = 0; q < grp; ++q) {
+        if (WIDE && q == 64 / kCumRows) half0 = half1 = 0.0;
         before0 += group_sum[q][s];
         before1 += group_sum[q][s + 1];
+        half0 += group_sum[q][s];
+        half1 += group_sum[q][s + 1];
     }
+    if (WIDE && grp == 64 / kCumRows) half0 = half1 = 0.0;
     // the chunk's total log-decay decides which of the chunk kernels takes this (b,h)
     // (with segment-parallel scheduling the flags are per (batch, segment, head))
     if (strong_flag != nullptr && grp == (int)blockDim.y - 1 &&
         fmin(before0 + acc0, before1 + acc1) < (double)kFactorisedDecayMin) {
         const int seg = nseg == 1 ? 0 : n * chunk / tseg;
-        strong_flag[(b * nseg + seg) * H + h] = 1;
+        strong_flag[WIDE ? (b * nseg + seg) * (H / 2) + h / 2 : (b * nseg + seg) * H + h] = 1;
     }
     // second pass over the same rows: the sums of the groups before as a float pair (value, rest)
     const float b0h = (float)before0, b0l = (float)(before0 - (double)b0h);
@@ -158,8 +170,22 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
     for (int i = 0; i < kCumRows; ++i)
         if (i < rows) {
             const float G0 = b0h + (b0l + g[i].x), G1 = b1h + (b1l + g[i].y);
-            *reinterpret_cast<float2*>(G + base + (size_t)i * stride) = make_float2(G0, G1);
-            if (decayed != nullptr) {
+            if (!WIDE) *reinterpret_cast<float2*>(G + base + (size_t)i * stride) = make_float2(G0, G1);
+            if (WIDE) {
+                // G itself is for the CUDA-core kernels, whose chunks have 64 tokens
+                *reinterpret_cast<float2*>(G + base + (size_t)i * stride) =
+                    make_float2((float)(half0 + (double)g[i].x), (float)(half1 + (double)g[i].y));
+                // exp(+-G) from the sum before its rounding to G: G0 + r0 is the sum of the pair and the thread's rows
+                const float r0 = (b0l + g[i].x) - (G0 - b0h), r1 = (b1l + g[i].y) - (G1 - b1h);
+                const float e0 = expf(G0), e1 = expf(G1), d0 = expf(-G0), d1 = expf(-G1);
+                *reinterpret_cast<float2*>(E + base + (size_t)i * stride) = make_float2(fmaf(e0, r0, e0), fmaf(e1, r1, e1));
+                uint32_t hi, mid, lo;
+                split_bf16x3(inps[i].x * fmaf(d0, -r0, d0), inps[i].y * fmaf(d1, -r1, d1), hi, mid, lo);
+                uint32_t* row = reinterpret_cast<uint32_t*>(decayed + 3 * (base + (size_t)i * stride - s) + s);
+                row[0] = hi;
+                row[M / 2] = mid;
+                row[M] = lo;
+            } else if (decayed != nullptr) {
                 // (meaningful for moderate decay only; pairs with a strong-decay chunk do not read it)
                 store_split2<M>(decayed + 2 * (base + (size_t)i * stride - s), s, inps[i].x * __expf(-G0),
                                 inps[i].y * __expf(-G1));
@@ -186,6 +212,16 @@ cudaError_t launch_gate_cumsum(const float* gate, int gate_kind, float inv_tau, 
     return cudaGetLastError();
 }
 
+cudaError_t launch_gate_cumsum_wide(const float* gate, int gate_kind, float inv_tau, float* G, float* I, float* E, int B, int T,
+                                    int H, int* strong_flag, int nseg, int tseg, void* decayed, cudaStream_t st,
+                                    const int* cu_seqlens, int nseq) {
+    constexpr int chunk = 128;
+    gate_cumsum_kernel<64, true><<<dim3(2 * B * H, (T + chunk - 1) / chunk), dim3(32, chunk / kCumRows), 0, st>>>(
+        gate, gate_kind, inv_tau, G, I, T, 2 * H, chunk, strong_flag, nseg, tseg, static_cast<__nv_bfloat16*>(decayed), 0,
+        cu_seqlens, nseq, E);
+    return cudaGetLastError();
+}
+
 // ------------------------------------------------------------------ slot softmax
 // M/4 lanes per token-head row of M slots, four adjacent slots per lane (one 16-byte access per
 // tensor and lane), 128/M rows per warp; reductions run over the lanes of a row.
@@ -205,6 +241,16 @@ __device__ __forceinline__ void st_split(__nv_bfloat16* row, int c, const float 
     split_bf16x2(x[2], x[3], h1, l1);
     *reinterpret_cast<uint2*>(row + c) = make_uint2(h0, h1);
     *reinterpret_cast<uint2*>(row + M + c) = make_uint2(l0, l1);
+}
+// ... as that of the operands with 128 slots: [half][high | middle | low] of 64 slots each
+__device__ __forceinline__ void st_split3(__nv_bfloat16* row, int c, const float (&x)[kSmR]) {
+    uint32_t h0, h1, m0, m1, l0, l1;
+    split_bf16x3(x[0], x[1], h0, m0, l0);
+    split_bf16x3(x[2], x[3], h1, m1, l1);
+    __nv_bfloat16* at = row + 192 * (c >> 6) + (c & 63);
+    *reinterpret_cast<uint2*>(at) = make_uint2(h0, h1);
+    *reinterpret_cast<uint2*>(at + 64) = make_uint2(m0, m1);
+    *reinterpret_cast<uint2*>(at + 128) = make_uint2(l0, l1);
 }
 template <int LPR>
 __device__ __forceinline__ float row_max(float x) {
@@ -254,7 +300,7 @@ __global__ void __launch_bounds__(256) slot_softmax_fwd_kernel(const float* __re
     if (G != nullptr) {
         ld_vec(G + idx, eg);
 #pragma unroll
-        for (int r = 0; r < R; ++r) eg[r] = __expf(eg[r]);
+        for (int r = 0; r < R; ++r) eg[r] = M == 128 ? eg[r] : __expf(eg[r]);      // (128 slots: G holds exp(G) itself)
     }
     float zmax = -INFINITY;
 #pragma unroll
@@ -285,7 +331,8 @@ __global__ void __launch_bounds__(256) slot_softmax_fwd_kernel(const float* __re
     if (p_decayed != nullptr) {
 #pragma unroll
         for (int r = 0; r < R; ++r) e[r] *= eg[r];
-        st_split<M>(p_decayed + row * 2 * M, l * R, e);
+        if (M == 128) st_split3(p_decayed + row * 3 * M, l * R, e);
+        else st_split<M>(p_decayed + row * 2 * M, l * R, e);
     }
 }
 
@@ -350,7 +397,7 @@ __global__ void __launch_bounds__(256) slot_softmax_bwd_kernel(const float* __re
     if (G != nullptr) {
         ld_vec(G + idx, eg);
 #pragma unroll
-        for (int r = 0; r < R; ++r) eg[r] = __expf(eg[r]);
+        for (int r = 0; r < R; ++r) eg[r] = M == 128 ? eg[r] : __expf(eg[r]);      // (128 slots: G holds exp(G) itself)
     }
     float zmax = -INFINITY;
 #pragma unroll
@@ -395,8 +442,13 @@ __global__ void __launch_bounds__(256) slot_softmax_bwd_kernel(const float* __re
     if (dz_decayed != nullptr) {
 #pragma unroll
         for (int r = 0; r < R; ++r) { e[r] *= eg[r]; dzv[r] *= eg[r]; }
-        if (p_decayed != nullptr) st_split<M>(p_decayed + row * 2 * M, l * R, e);
-        st_split<M>(dz_decayed + row * 2 * M, l * R, dzv);
+        if (M == 128) {
+            if (p_decayed != nullptr) st_split3(p_decayed + row * 3 * M, l * R, e);
+            st_split3(dz_decayed + row * 3 * M, l * R, dzv);
+        } else {
+            if (p_decayed != nullptr) st_split<M>(p_decayed + row * 2 * M, l * R, e);
+            st_split<M>(dz_decayed + row * 2 * M, l * R, dzv);
+        }
     }
 }
 
@@ -573,7 +625,7 @@ __global__ void __launch_bounds__(128) gate_grad_local_kernel(
 #pragma unroll
         for (int i = 0; i < kGG; ++i) gt[i] = ld2(pend.G, i, 0.f);
 #pragma unroll
-        for (int i = 0; i < kGG; ++i) { dI[i].x *= __expf(-gt[i].x); dI[i].y *= __expf(-gt[i].y); }
+        for (int i = 0; i < kGG; ++i) { dI[i].x *= pend.reverse_factor(gt[i].x); dI[i].y *= pend.reverse_factor(gt[i].y); }
     }
 #pragma unroll
     for (int i = 0; i < kGG; ++i) gt[i] = ld2(I, i, 0.f);
@@ -615,7 +667,7 @@ __global__ void __launch_bounds__(256) gate_grad_local_tma_kernel(
     const __grid_constant__ CUtensorMap mapGate, const __grid_constant__ CUtensorMap mapG,
     const __grid_constant__ CUtensorMap mapDIk, const __grid_constant__ CUtensorMap mapDIv, int nsk, int nsv,
     int gate_kind, float inv_tau, float* __restrict__ blk_tot, float* __restrict__ dgate, int T, int H, int nblk,
-    const int* __restrict__ strong, int nseg, int tseg, const int* __restrict__ cu, int nseq, int32_t* dev_status) {
+    PendingDecay pend, const int* __restrict__ cu, int nseq, int32_t* dev_status) {
     using namespace tc;
     constexpr int M = 64;
     extern __shared__ unsigned char gg_smem_raw[];
@@ -632,7 +684,7 @@ __global__ void __launch_bounds__(256) gate_grad_local_tma_kernel(
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         // tiles 0..3 = u, I, gate, G; I is not read when the gate tensor holds a itself (1 - a is one
         // subtraction), G only when a row factor is pending
-        const bool need[4] = {true, gate_kind != GSA_GATE_A, true, strong != nullptr};
+        const bool need[4] = {true, gate_kind != GSA_GATE_A, true, pend.G != nullptr};
         int ntiles = nslices;
         for (int i = 0; i < 4; ++i) ntiles += need[i] ? 1 : 0;
         mbar_expect_tx(&bar, (uint32_t)(ntiles * kGGTileB));
@@ -670,10 +722,10 @@ __global__ void __launch_bounds__(256) gate_grad_local_tma_kernel(
 #pragma unroll
         for (int i = 0; i < kHalf; ++i) dI[i] += at(4 + sl, i);
     }
-    if (strong != nullptr && strong[(b * nseg + (nseg == 1 ? 0 : t0 / tseg)) * H + h] == 0) {
+    if (pend.pending_at(b, t0, h)) {
         // the time-reversed value_side runs left their row factor exp(-G_i) to this kernel
 #pragma unroll
-        for (int i = 0; i < kHalf; ++i) dI[i] *= __expf(-at(3, i));
+        for (int i = 0; i < kHalf; ++i) dI[i] *= pend.reverse_factor(at(3, i));
     }
 #pragma unroll
     for (int i = 0; i < kHalf; ++i) {
@@ -717,7 +769,7 @@ __global__ void __launch_bounds__(kGGComputeThreads + 32) gate_grad_local_ring_k
     const __grid_constant__ CUtensorMap mapGate, const __grid_constant__ CUtensorMap mapG,
     const __grid_constant__ CUtensorMap mapDIk, const __grid_constant__ CUtensorMap mapDIv, int nsk, int nsv,
     int gate_kind, float inv_tau, float* __restrict__ blk_tot, float* __restrict__ dgate, int T, int H, int BH,
-    int ntile, int nstage, int nblk, const int* __restrict__ strong, int nseg, int tseg, const int* __restrict__ cu, int nseq, int32_t* dev_status) {
+    int ntile, int nstage, int nblk, PendingDecay pend, const int* __restrict__ cu, int nseq, int32_t* dev_status) {
     using namespace tc;
     constexpr int M = 64;
     extern __shared__ unsigned char gg_smem_raw[];
@@ -742,7 +794,7 @@ __global__ void __launch_bounds__(kGGComputeThreads + 32) gate_grad_local_ring_k
         // =============================== copy lane
         // tiles 0..3 = u, I, gate, G; I is not read when the gate tensor holds a itself (1 - a is one
         // subtraction), G only when a row factor is pending
-        const bool need[4] = {true, gate_kind != GSA_GATE_A, true, strong != nullptr};
+        const bool need[4] = {true, gate_kind != GSA_GATE_A, true, pend.G != nullptr};
         int ntiles = nslices;
         for (int i = 0; i < 4; ++i) ntiles += need[i] ? 1 : 0;
         const CUtensorMap* maps[4] = {&mapU, &mapI, &mapGate, &mapG};
@@ -798,10 +850,10 @@ __global__ void __launch_bounds__(kGGComputeThreads + 32) gate_grad_local_ring_k
 #pragma unroll
                     for (int i = 0; i < kHalf; ++i) dI[i] += at(4 + sl, i);
                 }
-                if (strong != nullptr && strong[(b * nseg + (nseg == 1 ? 0 : t0 / tseg)) * H + h] == 0) {
+                if (pend.pending_at(b, t0, h)) {
                     // the time-reversed value_side runs left their row factor exp(-G_i) to this kernel
 #pragma unroll
-                    for (int i = 0; i < kHalf; ++i) dI[i] *= __expf(-at(3, i));
+                    for (int i = 0; i < kHalf; ++i) dI[i] *= pend.reverse_factor(at(3, i));
                 }
 #pragma unroll
                 for (int i = 0; i < kHalf; ++i) {
@@ -887,6 +939,12 @@ cudaError_t launch_gate_grad(const float* u, const float* I, const float* dIk_pa
                              const float* dVT, const float* VT, int d_k, int d_v,
                              float* blk_tot, float* dgate, int B, int T, int H, int M,
                              PendingDecay pend, cudaStream_t st, int32_t* dev_status, const int* cu_seqlens, int nseq) {
+    if (pend.wide && M == 128) {       // as 2 H heads of 64 slots: the kernels that stage their tiles
+        pend.half_heads = 1;
+        pend.H = 2 * H;
+        return launch_gate_grad(u, I, dIk_part, nsk, dIv_part, nsv, gate, gate_kind, inv_tau, dKT, KT, dVT, VT, d_k, d_v, blk_tot,
+                                dgate, B, T, 2 * H, 64, pend, st, dev_status, cu_seqlens, nseq);
+    }
     const int nblk = gate_grad_blocks(T);
     dim3 block(M / 2, 256 / M);      // 128 threads: M/2 slot pairs x 16-row blocks
     dim3 grid(B * H, (nblk + block.y - 1) / block.y);
@@ -923,7 +981,7 @@ cudaError_t launch_gate_grad(const float* u, const float* I, const float* dIk_pa
             const int ctas = (int)(total < sm_count ? total : sm_count);      // one persistent CTA per SM
             gate_grad_local_ring_kernel<<<ctas, kGGComputeThreads + 32, smem, st>>>(
                 mu, mi, mg, mG, mk, mv, nsk, nsv, gate_kind, inv_tau, blk_tot, dgate, T, H, BH, ntile, nstage, nblk,
-                pend.G != nullptr ? pend.strong : nullptr, pend.nseg, pend.tseg, cu_seqlens, nseq, dev_status);
+                pend, cu_seqlens, nseq, dev_status);
         } else if (staged) {
             const size_t smem = 1024 + (size_t)(4 + nsl) * kGGTileB;
             cudaError_t e = cudaFuncSetAttribute(gate_grad_local_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -931,8 +989,7 @@ cudaError_t launch_gate_grad(const float* u, const float* I, const float* dIk_pa
             if (e != cudaSuccess) return e;
             dim3 tgrid(B * H, (T + kGGTmaRows - 1) / kGGTmaRows);
             gate_grad_local_tma_kernel<<<tgrid, 256, smem, st>>>(mu, mi, mg, mG, mk, mv, nsk, nsv, gate_kind, inv_tau, blk_tot,
-                                                                dgate, T, H, nblk, pend.G != nullptr ? pend.strong : nullptr,
-                                                                pend.nseg, pend.tseg, cu_seqlens, nseq, dev_status);
+                                                                dgate, T, H, nblk, pend, cu_seqlens, nseq, dev_status);
         } else {
             gate_grad_local_kernel<64><<<grid, block, 0, st>>>(u, I, dIk_part, nsk, dIv_part, nsv, gate, gate_kind, inv_tau,
                                                                blk_tot, dgate, B, T, H, nblk, pend, cu_seqlens, nseq);

@@ -212,6 +212,31 @@ def test_128_slots_fwd_bwd(io):
         check_bwd(gb, rb, TOL[io])
 
 
+@pytest.mark.parametrize("T,H,dk,dv,gate", [(1, 1, 64, 64, "tau8"), (127, 1, 128, 64, "tau8"), (128, 2, 64, 128, "tau8"),
+                                            (129, 2, 256, 128, "mixed"), (385, 3, 128, 512, "tau8"), (1153, 1, 128, 256, "mixed"),
+                                            (1700, 1, 256, 256, "tau8")])
+def test_128_slots_on_tensor_cores(T, H, dk, dv, gate):
+    """bf16 io: edges of the 128-token chunks, half-filled slices, several segments, and (mixed gates) pairs that go to the
+    CUDA-core kernels beside the others.  What comes out in fp32 is held to fp32 accuracy, not to that of bf16 products:
+    three bfloat16 parts carry 24 bits and the accumulators are fp32, so sums of a few hundred terms are off by a few
+    2^-21 = 5e-7 of their rms on average, ten times that at the worst of 1e5 elements; the gate gradient is a difference
+    of such sums, up to ten times as large as itself."""
+    B, m = 2, 128
+    d = rand_inputs(1280 + T, B, T, H, dk, dv, m, "bf16", init=True, final_grads=True)
+    if gate == "mixed":          # one head of one batch element forgets hard
+        d["gate"][0, :, 0] = d["gate"][0, :, 0] ** 8.0
+    got, g = run_fwd(d, B, T, H, dk, dv, m, "bf16", scale=0.9, log=True)
+    ref = oracle.fwd(d["q"], d["k"], d["v"], g, gate_is_log=True, scale=0.9, K0=d["K0"], V0=d["V0"])
+    gb, rb = run_bwd(d, B, T, H, dk, dv, m, "bf16", scale=0.9, log=True, saved=T % 2 == 0)
+    check_bwd(gb, rb, TOL["bf16"], tc=True)
+    errs = {n: rel_err(got[n], ref[n], n == "o") for n in ("o", "ok", "KT", "VT")}
+    errs.update({n: rel_err(gb[n], rb[n]) for n in ("dgate", "dK0", "dV0")})
+    print("128 slots", T, gate, {n: float("%.2g" % e) for n, e in errs.items()})
+    # (log gates of a hard-forgetting chunk sum to 100 and more: see test_bwd_strong_forgetting)
+    assert all(e <= (5e-5 if n == "dgate" else 1e-5) * (3 if gate == "mixed" else 1) for n, e in errs.items() if n != "o"), errs
+    assert errs["o"] <= TOL["bf16"]
+
+
 # ------------------------------------------------------------------ decode
 @pytest.mark.parametrize("io", ["f32", "bf16"])
 @pytest.mark.parametrize("dk,dv,m", [(64, 64, 32), (128, 128, 64), (256, 512, 64), (512, 64, 32), (128, 256, 128)])
