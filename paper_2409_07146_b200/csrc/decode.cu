@@ -69,6 +69,16 @@ struct RowVec {
     }
 };
 
+// a and 1 - a from element gi of the gate tensor
+__device__ __forceinline__ void decode_gate(const void* gate_raw, size_t gi, int gate_bf16, int gate_kind, float inv_tau,
+                                            float& a, float& ia) {
+    float gt = gate_bf16 ? __bfloat162float(static_cast<const __nv_bfloat16*>(gate_raw)[gi])
+                         : static_cast<const float*>(gate_raw)[gi];
+    if (gate_kind == GSA_GATE_LOGITS) gt = log_gate_from_logit(gt, inv_tau);
+    if (gate_kind != GSA_GATE_A) { a = __expf(gt); ia = -expm1f(gt); }
+    else { a = gt; ia = 1.f - gt; }
+}
+
 template <typename IO, int DK, int DV, int M>
 __global__ void __launch_bounds__(kDecodeWarps * 32)
 decode_step_kernel(const IO* __restrict__ q, const IO* __restrict__ k, const IO* __restrict__ v,
@@ -95,11 +105,7 @@ decode_step_kernel(const IO* __restrict__ q, const IO* __restrict__ k, const IO*
     for (int r = 0; r < RPW; ++r) {
         // (data-independent decay: one gate row per head, shared by all sequences; gate_row_of_head = H then)
         const size_t gi = (gate_row_of_head ? pair % gate_row_of_head : pair) * M + warp * RPW + r;
-        float gt = gate_bf16 ? __bfloat162float(static_cast<const __nv_bfloat16*>(gate_raw)[gi])
-                             : static_cast<const float*>(gate_raw)[gi];
-        if (gate_kind == GSA_GATE_LOGITS) gt = log_gate_from_logit(gt, inv_tau);
-        if (gate_kind != GSA_GATE_A) { a[r] = __expf(gt); ia[r] = -expm1f(gt); }
-        else { a[r] = gt; ia[r] = 1.f - gt; }
+        decode_gate(gate_raw, gi, gate_bf16, gate_kind, inv_tau, a[r], ia[r]);
     }
 
     // K~ <- a K~ + (1-a) k ; z = scale * K~ q.  Rows go through registers in batches whose
@@ -185,10 +191,165 @@ decode_step_kernel(const IO* __restrict__ q, const IO* __restrict__ k, const IO*
     }
 }
 
+// Few (sequence, head) pairs: a pair is dealt out over a cluster of M / (8 RPW) CTAs, RPW rows of each memory to a warp, so
+// that one sequence uses more than H SMs.  A step of one CTA per pair is bound by the latency of its chain -- K rows in
+// batches, logits, softmax, V rows in batches, sums -- and by what one SM can pull: 512 KB at d = 512, 9.6 us a launch
+// where 4 pairs keep 4 SMs busy.  Here every row of both memories is requested at once, before anything is used; the CTAs
+// exchange the M logits and the partial output rows through distributed shared memory (two cluster barriers).
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// the word at the same place of CTA `rank`'s shared memory <- x
+__device__ __forceinline__ void store_to_rank(float* local, unsigned rank, float x) {
+    uint32_t at, remote;
+    at = (uint32_t)__cvta_generic_to_shared(local);
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(at), "r"(rank));
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(x) : "memory");
+}
+
+template <typename IO, int DK, int DV, int RPW>
+__global__ void __launch_bounds__(kDecodeWarps * 32)
+decode_split_kernel(const IO* __restrict__ q, const IO* __restrict__ k, const IO* __restrict__ v,
+                    const void* __restrict__ gate_raw, int M, int gate_bf16, int gate_row_of_head, int feature_map,
+                    int gate_kind, float inv_tau, float scale, int act, float* __restrict__ Ks, float* __restrict__ Vs,
+                    IO* __restrict__ o) {
+    const int C = M / (kDecodeWarps * RPW);                     // CTAs of the cluster, M <= 128, C <= 8
+    const size_t pair = blockIdx.x / C;
+    const int rank = blockIdx.x % C, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int row0 = (rank * kDecodeWarps + warp) * RPW;        // this warp's memory rows
+    __shared__ float s_z[128];
+    __shared__ float s_o[kDecodeWarps][DV];
+    __shared__ float s_part[8][DV];         // partial sums of this CTA's DV / C output channels, from every rank
+    cluster_arrive();                       // (every CTA runs before another one writes to it)
+
+    float* Kp = Ks + (pair * M + row0) * DK;
+    float* Vp = Vs + (pair * M + row0) * DV;
+    RowVec<DK> kr[RPW], qv, kv;
+    RowVec<DV> vr[RPW], vv;
+#pragma unroll
+    for (int r = 0; r < RPW; ++r) kr[r].load(Kp + (size_t)r * DK, lane);
+#pragma unroll
+    for (int r = 0; r < RPW; ++r) vr[r].load(Vp + (size_t)r * DV, lane);
+    qv.load_io(q + pair * DK, lane);
+    kv.load_io(k + pair * DK, lane);
+    vv.load_io(v + pair * DV, lane);
+    float a[RPW], ia[RPW];
+#pragma unroll
+    for (int r = 0; r < RPW; ++r) {
+        const size_t gi = (gate_row_of_head ? pair % gate_row_of_head : pair) * M + row0 + r;
+        decode_gate(gate_raw, gi, gate_bf16, gate_kind, inv_tau, a[r], ia[r]);
+    }
+    if (feature_map == GSA_FEAT_SWISH) { qv.swish(); kv.swish(); vv.swish(); }
+    float z[RPW];
+#pragma unroll
+    for (int r = 0; r < RPW; ++r) {
+        float dot = 0.f;
+#pragma unroll
+        for (int i = 0; i < RowVec<DK>::kN; ++i)
+#pragma unroll
+            for (int w = 0; w < RowVec<DK>::kW; ++w) {
+                const float x = fmaf(a[r], kr[r].v[i][w], ia[r] * kv.v[i][w]);
+                kr[r].v[i][w] = x;
+                dot = fmaf(x, qv.v[i][w], dot);
+            }
+#pragma unroll
+        for (int off = 16; off; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
+        z[r] = dot * scale;
+    }
+    cluster_wait();
+#pragma unroll
+    for (int r = 0; r < RPW; ++r)
+        if (lane < C) store_to_rank(&s_z[row0 + r], lane, z[r]);
+    cluster_arrive();
+    // (the memories leave while the logits travel)
+#pragma unroll
+    for (int r = 0; r < RPW; ++r) {
+        kr[r].store(Kp + (size_t)r * DK, lane);
+#pragma unroll
+        for (int i = 0; i < RowVec<DV>::kN; ++i)
+#pragma unroll
+            for (int w = 0; w < RowVec<DV>::kW; ++w) vr[r].v[i][w] = fmaf(a[r], vr[r].v[i][w], ia[r] * vv.v[i][w]);
+        vr[r].store(Vp + (size_t)r * DV, lane);
+    }
+    cluster_wait();
+    // slot weights of this warp's rows, each warp by itself
+    float p[RPW];
+    if (act != GSA_ACT_SOFTMAX) {
+#pragma unroll
+        for (int r = 0; r < RPW; ++r) p[r] = slot_act_value(z[r], act);
+    } else {
+        float zmax = -INFINITY, den = 0.f;
+        for (int s = lane; s < M; s += 32) zmax = fmaxf(zmax, s_z[s]);
+#pragma unroll
+        for (int off = 16; off; off >>= 1) zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, off));
+        for (int s = lane; s < M; s += 32) den += __expf(s_z[s] - zmax);
+#pragma unroll
+        for (int off = 16; off; off >>= 1) den += __shfl_xor_sync(0xffffffffu, den, off);
+        const float inv = 1.f / den;
+#pragma unroll
+        for (int r = 0; r < RPW; ++r) p[r] = __expf(z[r] - zmax) * inv;
+    }
+    RowVec<DV> acc;
+#pragma unroll
+    for (int i = 0; i < RowVec<DV>::kN; ++i)
+#pragma unroll
+        for (int w = 0; w < RowVec<DV>::kW; ++w) {
+            acc.v[i][w] = 0.f;
+#pragma unroll
+            for (int r = 0; r < RPW; ++r) acc.v[i][w] = fmaf(p[r], vr[r].v[i][w], acc.v[i][w]);
+        }
+    acc.store(&s_o[warp][0], lane);
+    __syncthreads();
+    // the CTA's partial sum of channel c goes to the CTA that owns the channel
+    const int own = DV / C;
+    for (int c = threadIdx.x; c < DV; c += kDecodeWarps * 32) {
+        float sum = 0.f;
+#pragma unroll
+        for (int w = 0; w < kDecodeWarps; ++w) sum += s_o[w][c];
+        store_to_rank(&s_part[rank][c % own], c / own, sum);
+    }
+    cluster_arrive();
+    cluster_wait();
+    for (int c = threadIdx.x; c < own; c += kDecodeWarps * 32) {
+        float sum = 0.f;
+        for (int r = 0; r < C; ++r) sum += s_part[r][c];
+        o[pair * DV + rank * own + c] = float_to_io<IO>(sum);
+    }
+}
+
+template <typename IO, int DK, int DV, int RPW>
+static cudaError_t launch_decode_split(const gsa_params_t& p, const IO* q, const IO* k, const IO* v, const float* gate,
+                                       float* Ks, float* Vs, IO* o, cudaStream_t st) {
+    const unsigned C = (unsigned)(p.m / (kDecodeWarps * RPW));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)p.B * (unsigned)p.H * C);
+    cfg.blockDim = dim3(kDecodeWarps * 32);
+    cfg.stream = st;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = C;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, decode_split_kernel<IO, DK, DV, RPW>, q, k, v, static_cast<const void*>(gate), (int)p.m,
+                              (int)(p.gate_dtype == GSA_BF16), (int)(p.gate_broadcast ? p.H : 0), (int)p.feature_map,
+                              (int)p.gate_kind, p.tau > 0.f ? 1.f / p.tau : 0.f, p.scale, (int)p.slot_act, Ks, Vs, o);
+}
+
 template <typename IO, int DK, int DV>
 static cudaError_t launch_decode_m(const gsa_params_t& p, const IO* q, const IO* k, const IO* v,
                                    const float* gate, float* Ks, float* Vs, IO* o, cudaStream_t st) {
     const unsigned pairs = (unsigned)p.B * (unsigned)p.H;
+    // The line between the kernels, us a step of one layer (64 slots) with one CTA a pair / a row a warp / two: 4 pairs of
+    // d = 512: 10.3 / 4.8 / 5.6, 16: 15.3 / 6.6 / 7.0, 64: 19.5 / 14.3 / 14.5, 80: 20.1 / 19.2 / 19.9, 128: 22.8 / 26.8 / 27.1;
+    // d = 256: 8 pairs 5.9 / 4.0 / 4.6, 64: 10.8 / 11.5 / 7.8; d = 128: 32 pairs 4.4 / 4.3 / 4.2, 128: 7.5 / 11.9 / 7.9 (a pair
+    // is little enough for one SM).  So: heads of 256 and more, a row a warp while no SM has two CTAs, two rows a warp
+    // while none has more than two.
+    if constexpr (DK + DV >= 512) {
+        const long long ctas = (long long)pairs * (p.m / kDecodeWarps);
+        if (p.m <= 64 && ctas <= 148) return launch_decode_split<IO, DK, DV, 1>(p, q, k, v, gate, Ks, Vs, o, st);
+        if (ctas / 2 <= 2 * 148) return launch_decode_split<IO, DK, DV, 2>(p, q, k, v, gate, Ks, Vs, o, st);
+    }
     const int is_log = p.gate_kind;
     const float inv_tau = p.tau > 0.f ? 1.f / p.tau : 0.f;
     if (p.m == 128)

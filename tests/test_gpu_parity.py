@@ -778,3 +778,28 @@ def test_data_independent_decay_one_gate_row_for_all_tokens(io, impl, kind):
     od = gsa.gsa_decode_step(pd, q[:, 0].contiguous(), k[:, 0].contiguous(), v[:, 0].contiguous(), to_dev(row), Ks, Vs)
     ro = oracle.decode_step(x["q"][:, 0], x["k"][:, 0], x["v"][:, 0], full[:, 0], Kr, Vr, **kw)
     assert rel_err(to_np(od), ro, io == "bf16") <= TOL[io] and rel_err(to_np(Ks), Kr) <= 1e-5
+
+
+@pytest.mark.parametrize("io,B,H,dk,dv,m", [("bf16", 1, 4, 512, 512, 64), ("f32", 2, 9, 256, 256, 64), ("bf16", 2, 10, 256, 256, 64),
+                                            ("bf16", 37, 2, 512, 64, 64), ("bf16", 75, 1, 512, 512, 64), ("f32", 3, 12, 64, 512, 32),
+                                            ("f32", 37, 4, 256, 512, 32), ("bf16", 2, 3, 256, 256, 128), ("f32", 37, 1, 512, 128, 128),
+                                            ("bf16", 38, 1, 512, 256, 128)])
+@pytest.mark.parametrize("act", ["softmax", "swish"])
+def test_decode_over_clusters(io, B, H, dk, dv, m, act):
+    """A pair dealt out over the CTAs of a cluster, one and two memory rows to a warp, on both sides of the lines between
+    those and the kernel of one CTA a pair: two steps, the second one from the memories that the first one left."""
+    r = np.random.default_rng(B * H + m)
+    f = lambda *s: r.standard_normal(s).astype(np.float32)
+    K, V = f(B, H, m, dk) * np.float32(0.3), f(B, H, m, dv) * np.float32(0.3)
+    p = gsa.Params(B, 1, H, dk, dv, m, io=io, scale=0.8, slot_act=act)
+    Ks, Vs = to_dev(K), to_dev(V)
+    for _ in range(2):
+        q, k, v = f(B, 1, H, dk) * np.float32(dk ** -0.5), f(B, 1, H, dk), f(B, 1, H, dv)
+        if io == "bf16":
+            q, k, v = (W.round_to_bf16(x) for x in (q, k, v))
+        gate = ((1 / (1 + np.exp(-f(B, 1, H, m)))) ** 0.125).astype(np.float32)
+        o = gsa.gsa_decode_step(p, *(to_dev(x[:, 0], io) for x in (q, k, v)), to_dev(gate[:, 0]), Ks, Vs)
+        ref = oracle.fwd(q, k, v, gate, scale=0.8, K0=K, V0=V, act=act)
+        assert rel_err(to_np(o), ref["o"][:, 0], io == "bf16") <= TOL[io]
+        assert rel_err(to_np(Ks), ref["KT"]) <= 1e-5 and rel_err(to_np(Vs), ref["VT"]) <= 1e-5
+        K, V = ref["KT"], ref["VT"]
