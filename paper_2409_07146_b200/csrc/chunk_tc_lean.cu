@@ -121,6 +121,7 @@ value_side_lean_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_co
                        const __grid_constant__ CUtensorMap mapWd, const __grid_constant__ CUtensorMap mapO,
                        const __grid_constant__ CUtensorMap mapW32, const __grid_constant__ CUtensorMap mapG32,
                        const __grid_constant__ ValueSideArgs a, const int* __restrict__ strong_flag, int32_t* dev_status) {
+    follow_previous_grid();
     if (strong_flag[blockIdx.x] != 0) {
         value_side_general<REV>(mapQ, mapK, mapW32, mapG32, mapO, a, dev_status, blockIdx.y);
         return;
@@ -382,6 +383,7 @@ key_side_lean_kernel(const __grid_constant__ CUtensorMap mapV, const __grid_cons
                      const __grid_constant__ CUtensorMap mapUq32, const __grid_constant__ CUtensorMap mapUk32,
                      const __grid_constant__ CUtensorMap mapG32, const __grid_constant__ KeySideArgs a,
                      const int* __restrict__ strong_flag, int32_t* dev_status) {
+    follow_previous_grid();
     if (strong_flag[blockIdx.x] != 0) {
         key_side_general<REV>(mapV, mapUq32, mapUk32, mapG32, mapO, a, dev_status);
         return;
@@ -668,6 +670,7 @@ state_scan_kernel(const __grid_constant__ CUtensorMap mapX0, const __grid_consta
                   const __grid_constant__ CUtensorMap mapW1, const __grid_constant__ CUtensorMap mapW32_1,
                   const __grid_constant__ CUtensorMap mapG32, const __grid_constant__ StateScanArgs sets,
                   const int* __restrict__ strong_flag, int32_t* dev_status) {
+    follow_previous_grid();
     const bool second = (int)blockIdx.y >= sets.slices0;
     const CUtensorMap &mapX = second ? mapX1 : mapX0, &mapW = second ? mapW1 : mapW0;
     const ValueSideArgs& a = sets.set[second];
@@ -830,12 +833,12 @@ cudaError_t launch_state_scan_tc(const ValueSideArgs& k, const ValueSideArgs& v,
     if (reverse) {
         e = prepare<state_scan_kernel<true>>(smem);
         if (e != cudaSuccess) return e;
-        state_scan_kernel<true><<<grid, kScanThreads, smem, st>>>(mx[0], mw[0], mw32[0], mx[1], mw[1], mw32[1], mg, sets,
+        launch_after(state_scan_kernel<true>, grid, kScanThreads, smem, st, mx[0], mw[0], mw32[0], mx[1], mw[1], mw32[1], mg, sets,
                                                                   strong_flag, dev_status);
     } else {
         e = prepare<state_scan_kernel<false>>(smem);
         if (e != cudaSuccess) return e;
-        state_scan_kernel<false><<<grid, kScanThreads, smem, st>>>(mx[0], mw[0], mw32[0], mx[1], mw[1], mw32[1], mg, sets,
+        launch_after(state_scan_kernel<false>, grid, kScanThreads, smem, st, mx[0], mw[0], mw32[0], mx[1], mw[1], mw32[1], mg, sets,
                                                                    strong_flag, dev_status);
     }
     return cudaGetLastError();
@@ -861,7 +864,7 @@ cudaError_t launch_value_side_tc(const ValueSideArgs& a, int M, int reverse, con
     constexpr size_t smem = kSmemLeanValue > kSmemGeneral ? kSmemLeanValue : kSmemGeneral;
     auto launch = [&](auto kernel, cudaError_t ready) {
         if (ready != cudaSuccess) return ready;
-        kernel<<<grid, kScanThreads, smem, st>>>(mq, mk, mw, mo, mw32, mg32, a, strong_flag, dev_status);
+        launch_after(kernel, grid, kScanThreads, smem, st, mq, mk, mw, mo, mw32, mg32, a, strong_flag, dev_status);
         return cudaGetLastError();
     };
 #define GSA_VALUE(REV, PAIRS) launch(value_side_lean_kernel<REV, PAIRS>, prepare<value_side_lean_kernel<REV, PAIRS>>(smem))
@@ -886,7 +889,7 @@ cudaError_t launch_key_side_tc(const KeySideArgs& a, int M, int reverse, const i
     constexpr size_t smem = kSmemLeanKey > kSmemGeneral ? kSmemLeanKey : kSmemGeneral;
     auto launch = [&](auto kernel, cudaError_t ready) {
         if (ready != cudaSuccess) return ready;
-        kernel<<<grid, kScanThreads, smem, st>>>(mv, muq, muk, mo, muq32, muk32, mg32, a, strong_flag, dev_status);
+        launch_after(kernel, grid, kScanThreads, smem, st, mv, muq, muk, mo, muq32, muk32, mg32, a, strong_flag, dev_status);
         return cudaGetLastError();
     };
 #define GSA_KEY(REV, PAIRS) launch(key_side_lean_kernel<REV, PAIRS>, prepare<key_side_lean_kernel<REV, PAIRS>>(smem))

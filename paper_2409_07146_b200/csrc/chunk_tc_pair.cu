@@ -69,6 +69,7 @@ rev_pair_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
                 const __grid_constant__ CUtensorMap mapW32, const __grid_constant__ CUtensorMap mapQ32,
                 const __grid_constant__ CUtensorMap mapG32, const __grid_constant__ ValueSideArgs av,
                 const __grid_constant__ KeySideArgs ak, const int* __restrict__ strong_flag, int32_t* dev_status) {
+    follow_previous_grid();
     if (strong_flag[blockIdx.x] != 0) {             // the two general scans, one after the other
         if (value_side_general<true, false>(mapY, mapX, mapW32, mapG32, mapOv, av, dev_status, blockIdx.y))
             key_side_general<true, false>(mapX, mapQ32, mapW32, mapG32, mapOk, ak, dev_status);
@@ -477,7 +478,7 @@ cudaError_t launch_rev_pair_tc(const ValueSideArgs& av, const KeySideArgs& ak, i
     constexpr size_t smem = kSmemPair > kSmemGeneral ? kSmemPair : kSmemGeneral;
     auto launch = [&](auto kernel, cudaError_t ready) {
         if (ready != cudaSuccess) return ready;
-        kernel<<<grid, kScanThreads, smem, st>>>(mx, my, mw, mq, mov, mok, mw32, mq32, mg32, av, ak, strong_flag, dev_status);
+        launch_after(kernel, grid, kScanThreads, smem, st, mx, my, mw, mq, mov, mok, mw32, mq32, mg32, av, ak, strong_flag, dev_status);
         return cudaGetLastError();
     };
     return av.single ? launch(rev_pair_kernel<false>, prepare<rev_pair_kernel<false>>(smem))

@@ -164,6 +164,7 @@ __global__ void __launch_bounds__(kScanThreads, 1)
 value_side_wide_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
                        const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapO,
                        const __grid_constant__ ValueSideArgs a, const int* __restrict__ strong_flag, int32_t* dev_status) {
+    follow_previous_grid();
     const int H2 = 2 * a.H;
     const ScanSpan span = scan_span(blockIdx.x, H2, a.T, a.nseg, a.tseg);
     const int bh = blockIdx.x, slice = blockIdx.y, b = span.b, h2 = span.h, h = h2 >> 1;
@@ -366,6 +367,7 @@ __global__ void __launch_bounds__(kScanThreads, 1)
 key_side_wide_kernel(const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapUq,
                      const __grid_constant__ CUtensorMap mapUk, const __grid_constant__ CUtensorMap mapO,
                      const __grid_constant__ KeySideArgs a, const int* __restrict__ strong_flag, int32_t* dev_status) {
+    follow_previous_grid();
     if (strong_flag[blockIdx.x] != 0) return;       // the CUDA-core kernel takes this (batch, head)
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -585,6 +587,7 @@ __global__ void __launch_bounds__(kScanThreads, 1)
 state_scan_wide_kernel(const __grid_constant__ CUtensorMap mapX0, const __grid_constant__ CUtensorMap mapW0,
                        const __grid_constant__ CUtensorMap mapX1, const __grid_constant__ CUtensorMap mapW1,
                        const __grid_constant__ WideScanArgs sets, const int* __restrict__ strong_flag, int32_t* dev_status) {
+    follow_previous_grid();
     const bool second = (int)blockIdx.y >= sets.slices0;
     const CUtensorMap &mapX = second ? mapX1 : mapX0, &mapW = second ? mapW1 : mapW0;
     const ValueSideArgs& a = sets.set[second];
@@ -699,11 +702,11 @@ cudaError_t launch_state_scan_wide(const ValueSideArgs& k, const ValueSideArgs* 
     if (reverse) {
         e = prepare<state_scan_wide_kernel<true>>(kSmemWide);
         if (e != cudaSuccess) return e;
-        state_scan_wide_kernel<true><<<grid, kScanThreads, kSmemWide, st>>>(mx[0], mw[0], mx[1], mw[1], sets, strong_flag, dev_status);
+        launch_after(state_scan_wide_kernel<true>, grid, kScanThreads, kSmemWide, st, mx[0], mw[0], mx[1], mw[1], sets, strong_flag, dev_status);
     } else {
         e = prepare<state_scan_wide_kernel<false>>(kSmemWide);
         if (e != cudaSuccess) return e;
-        state_scan_wide_kernel<false><<<grid, kScanThreads, kSmemWide, st>>>(mx[0], mw[0], mx[1], mw[1], sets, strong_flag, dev_status);
+        launch_after(state_scan_wide_kernel<false>, grid, kScanThreads, kSmemWide, st, mx[0], mw[0], mx[1], mw[1], sets, strong_flag, dev_status);
     }
     return cudaGetLastError();
 }
@@ -723,11 +726,11 @@ cudaError_t launch_value_side_wide(const ValueSideArgs& a, int reverse, const in
     if (reverse) {
         e = prepare<value_side_wide_kernel<true>>(kSmemWide);
         if (e != cudaSuccess) return e;
-        value_side_wide_kernel<true><<<grid, kScanThreads, kSmemWide, st>>>(mq, mk, mw, mo, a, strong_flag, dev_status);
+        launch_after(value_side_wide_kernel<true>, grid, kScanThreads, kSmemWide, st, mq, mk, mw, mo, a, strong_flag, dev_status);
     } else {
         e = prepare<value_side_wide_kernel<false>>(kSmemWide);
         if (e != cudaSuccess) return e;
-        value_side_wide_kernel<false><<<grid, kScanThreads, kSmemWide, st>>>(mq, mk, mw, mo, a, strong_flag, dev_status);
+        launch_after(value_side_wide_kernel<false>, grid, kScanThreads, kSmemWide, st, mq, mk, mw, mo, a, strong_flag, dev_status);
     }
     e = cudaGetLastError();
     return e == cudaSuccess ? launch_value_side_simt(a, GSA_BF16, kWide, reverse, st, strong_flag) : e;
@@ -747,11 +750,11 @@ cudaError_t launch_key_side_wide(const KeySideArgs& a, int reverse, const int* s
     if (reverse) {
         e = prepare<key_side_wide_kernel<true>>(kSmemWide);
         if (e != cudaSuccess) return e;
-        key_side_wide_kernel<true><<<grid, kScanThreads, kSmemWide, st>>>(mv, muq, muk, mo, a, strong_flag, dev_status);
+        launch_after(key_side_wide_kernel<true>, grid, kScanThreads, kSmemWide, st, mv, muq, muk, mo, a, strong_flag, dev_status);
     } else {
         e = prepare<key_side_wide_kernel<false>>(kSmemWide);
         if (e != cudaSuccess) return e;
-        key_side_wide_kernel<false><<<grid, kScanThreads, kSmemWide, st>>>(mv, muq, muk, mo, a, strong_flag, dev_status);
+        launch_after(key_side_wide_kernel<false>, grid, kScanThreads, kSmemWide, st, mv, muq, muk, mo, a, strong_flag, dev_status);
     }
     e = cudaGetLastError();
     if (e == cudaSuccess && a.Send != nullptr) {

@@ -59,6 +59,30 @@ __device__ __forceinline__ void store_vec4(__nv_bfloat16* p, const float (&in)[4
     *reinterpret_cast<uint2*>(p) = v;
 }
 
+// Kernels of a call follow one another closely: each is launched with launch_after, may be placed on the GPU as soon as
+// every CTA of the kernel before it in the stream has started, and waits, first thing, until that kernel is complete and its
+// memory is visible (follow_previous_grid).  As every kernel waits, what is complete for one is complete for all after it.
+// The gaps between the 8 kernels of a forward over 1431 tokens, 2.4 us each, take 17 of its 67 us without; 56 us with it.
+// (A CTA that waits holds its SM's resources: not for kernels whose CTAs usually leave at once while another stream works.)
+__device__ __forceinline__ void follow_previous_grid() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // ---- arguments of the two chunk primitives (both passes, forward and time-reversed) ----
 //
 // value_side ("gsa_fwd" of Algorithm 1 with GATE_K = False, the pass-1 form):

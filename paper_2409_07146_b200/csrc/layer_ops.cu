@@ -23,6 +23,7 @@ __device__ __forceinline__ float swish_gradf(float x) {
 
 template <typename IO>
 __global__ void __launch_bounds__(256) swish_fwd_kernel(const IO* __restrict__ in, IO* __restrict__ out, size_t nvec) {
+    follow_previous_grid();
     constexpr int V = IoTraits<IO>::kVec;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nvec; i += (size_t)gridDim.x * blockDim.x) {
         float x[V];
@@ -35,6 +36,7 @@ __global__ void __launch_bounds__(256) swish_fwd_kernel(const IO* __restrict__ i
 // d <- d * Swish'(x), in place on the gradient
 template <typename IO>
 __global__ void __launch_bounds__(256) swish_bwd_kernel(const IO* __restrict__ x_in, IO* __restrict__ d, size_t nvec) {
+    follow_previous_grid();
     constexpr int V = IoTraits<IO>::kVec;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nvec; i += (size_t)gridDim.x * blockDim.x) {
         float x[V], g[V];
@@ -64,6 +66,7 @@ constexpr int kMaxVecPerThread = 2;
 template <typename IO>
 __global__ void __launch_bounds__(256) out_norm_fwd_kernel(const IO* __restrict__ o, const float* __restrict__ weight,
                                                            float eps, IO* __restrict__ y, int N) {
+    follow_previous_grid();
     constexpr int V = IoTraits<IO>::kVec;
     __shared__ float scratch[8];
     const size_t row = blockIdx.x;
@@ -98,6 +101,7 @@ template <typename IO>
 __global__ void __launch_bounds__(256) out_norm_bwd_kernel(const IO* __restrict__ o, const IO* __restrict__ dy,
                                                            const float* __restrict__ weight, float eps, IO* __restrict__ d_o,
                                                            float* __restrict__ dw_part, int N, size_t rows) {
+    follow_previous_grid();
     constexpr int V = IoTraits<IO>::kVec;
     __shared__ float scratch[8];
     const int nvec = N / V;
@@ -159,6 +163,7 @@ __global__ void __launch_bounds__(256) out_norm_bwd_kernel(const IO* __restrict_
     }
 }
 __global__ void out_norm_dw_kernel(const float* __restrict__ dw_part, float* __restrict__ dweight, int N, int nparts) {
+    follow_previous_grid();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= N) return;
     double acc = 0.0;
@@ -177,20 +182,20 @@ unsigned stream_blocks(size_t nvec) {
 cudaError_t launch_swish_fwd(const void* in, void* out, size_t n, int io, cudaStream_t st) {
     if (io == GSA_BF16) {
         const size_t nv = n / 8;
-        swish_fwd_kernel<__nv_bfloat16><<<stream_blocks(nv), 256, 0, st>>>((const __nv_bfloat16*)in, (__nv_bfloat16*)out, nv);
+        launch_after(swish_fwd_kernel<__nv_bfloat16>, stream_blocks(nv), 256, 0, st, (const __nv_bfloat16*)in, (__nv_bfloat16*)out, nv);
     } else {
         const size_t nv = n / 4;
-        swish_fwd_kernel<float><<<stream_blocks(nv), 256, 0, st>>>((const float*)in, (float*)out, nv);
+        launch_after(swish_fwd_kernel<float>, stream_blocks(nv), 256, 0, st, (const float*)in, (float*)out, nv);
     }
     return cudaGetLastError();
 }
 cudaError_t launch_swish_bwd(const void* x, void* d, size_t n, int io, cudaStream_t st) {
     if (io == GSA_BF16) {
         const size_t nv = n / 8;
-        swish_bwd_kernel<__nv_bfloat16><<<stream_blocks(nv), 256, 0, st>>>((const __nv_bfloat16*)x, (__nv_bfloat16*)d, nv);
+        launch_after(swish_bwd_kernel<__nv_bfloat16>, stream_blocks(nv), 256, 0, st, (const __nv_bfloat16*)x, (__nv_bfloat16*)d, nv);
     } else {
         const size_t nv = n / 4;
-        swish_bwd_kernel<float><<<stream_blocks(nv), 256, 0, st>>>((const float*)x, (float*)d, nv);
+        launch_after(swish_bwd_kernel<float>, stream_blocks(nv), 256, 0, st, (const float*)x, (float*)d, nv);
     }
     return cudaGetLastError();
 }
@@ -198,20 +203,20 @@ int out_norm_max_width(int io) { return 256 * kMaxVecPerThread * (io == GSA_BF16
 size_t out_norm_bwd_parts(size_t rows) { return (rows + kRowsPerCta - 1) / kRowsPerCta; }
 cudaError_t launch_out_norm_fwd(const void* o, const float* weight, float eps, void* y, size_t rows, int N, int io,
                                 cudaStream_t st) {
-    if (io == GSA_BF16) out_norm_fwd_kernel<__nv_bfloat16><<<(unsigned)rows, 256, 0, st>>>((const __nv_bfloat16*)o, weight, eps, (__nv_bfloat16*)y, N);
-    else out_norm_fwd_kernel<float><<<(unsigned)rows, 256, 0, st>>>((const float*)o, weight, eps, (float*)y, N);
+    if (io == GSA_BF16) launch_after(out_norm_fwd_kernel<__nv_bfloat16>, (unsigned)rows, 256, 0, st, (const __nv_bfloat16*)o, weight, eps, (__nv_bfloat16*)y, N);
+    else launch_after(out_norm_fwd_kernel<float>, (unsigned)rows, 256, 0, st, (const float*)o, weight, eps, (float*)y, N);
     return cudaGetLastError();
 }
 cudaError_t launch_out_norm_bwd(const void* o, const void* dy, const float* weight, float eps, void* d_o, float* dw_part,
                                 float* dweight, size_t rows, int N, int io, cudaStream_t st) {
     const unsigned parts = (unsigned)out_norm_bwd_parts(rows);
     if (io == GSA_BF16)
-        out_norm_bwd_kernel<__nv_bfloat16><<<parts, 256, 0, st>>>((const __nv_bfloat16*)o, (const __nv_bfloat16*)dy, weight, eps,
+        launch_after(out_norm_bwd_kernel<__nv_bfloat16>, parts, 256, 0, st, (const __nv_bfloat16*)o, (const __nv_bfloat16*)dy, weight, eps,
                                                                 (__nv_bfloat16*)d_o, dweight ? dw_part : nullptr, N, rows);
     else
-        out_norm_bwd_kernel<float><<<parts, 256, 0, st>>>((const float*)o, (const float*)dy, weight, eps, (float*)d_o,
+        launch_after(out_norm_bwd_kernel<float>, parts, 256, 0, st, (const float*)o, (const float*)dy, weight, eps, (float*)d_o,
                                                         dweight ? dw_part : nullptr, N, rows);
-    if (dweight != nullptr) out_norm_dw_kernel<<<(N + 255) / 256, 256, 0, st>>>(dw_part, dweight, N, (int)parts);
+    if (dweight != nullptr) launch_after(out_norm_dw_kernel, (N + 255) / 256, 256, 0, st, dw_part, dweight, N, (int)parts);
     return cudaGetLastError();
 }
 

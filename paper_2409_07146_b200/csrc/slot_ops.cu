@@ -68,7 +68,8 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
                                                             int chunk, int* __restrict__ strong_flag, int nseg, int tseg,
                                                             __nv_bfloat16* __restrict__ decayed, int fast_log,
                                                             const int* __restrict__ cu_seqlens, int nseq,
-                                                            float* __restrict__ E = nullptr) {
+                                                            float* __restrict__ E) {
+    follow_previous_grid();
     __shared__ double group_sum[16][M];
     const int s = 2 * threadIdx.x, grp = threadIdx.y;          // blockDim.y = chunk / 8 <= 16
     const int n = blockIdx.y;
@@ -201,14 +202,14 @@ cudaError_t launch_gate_cumsum(const float* gate, int gate_kind, float inv_tau, 
     dim3 block(M / 2, chunk / kCumRows);
     dim3 grid(B * H, nchunks);
     if (M == 128)
-        gate_cumsum_kernel<128><<<grid, block, 0, st>>>(gate, gate_kind, inv_tau, G, I, T, H, chunk, strong_flag, nseg, tseg,
-                                                        static_cast<__nv_bfloat16*>(decayed), fast_log, cu_seqlens, nseq);
+        launch_after(gate_cumsum_kernel<128>, grid, block, 0, st, gate, gate_kind, inv_tau, G, I, T, H, chunk, strong_flag, nseg, tseg,
+                                                        static_cast<__nv_bfloat16*>(decayed), fast_log, cu_seqlens, nseq, nullptr);
     else if (M == 64)
-        gate_cumsum_kernel<64><<<grid, block, 0, st>>>(gate, gate_kind, inv_tau, G, I, T, H, chunk, strong_flag, nseg, tseg,
-                                                       static_cast<__nv_bfloat16*>(decayed), fast_log, cu_seqlens, nseq);
+        launch_after(gate_cumsum_kernel<64>, grid, block, 0, st, gate, gate_kind, inv_tau, G, I, T, H, chunk, strong_flag, nseg, tseg,
+                                                       static_cast<__nv_bfloat16*>(decayed), fast_log, cu_seqlens, nseq, nullptr);
     else
-        gate_cumsum_kernel<32><<<grid, block, 0, st>>>(gate, gate_kind, inv_tau, G, I, T, H, chunk, strong_flag, nseg, tseg,
-                                                       static_cast<__nv_bfloat16*>(decayed), fast_log, cu_seqlens, nseq);
+        launch_after(gate_cumsum_kernel<32>, grid, block, 0, st, gate, gate_kind, inv_tau, G, I, T, H, chunk, strong_flag, nseg, tseg,
+                                                       static_cast<__nv_bfloat16*>(decayed), fast_log, cu_seqlens, nseq, nullptr);
     return cudaGetLastError();
 }
 
@@ -216,8 +217,7 @@ cudaError_t launch_gate_cumsum_wide(const float* gate, int gate_kind, float inv_
                                     int H, int* strong_flag, int nseg, int tseg, void* decayed, cudaStream_t st,
                                     const int* cu_seqlens, int nseq) {
     constexpr int chunk = 128;
-    gate_cumsum_kernel<64, true><<<dim3(2 * B * H, (T + chunk - 1) / chunk), dim3(32, chunk / kCumRows), 0, st>>>(
-        gate, gate_kind, inv_tau, G, I, T, 2 * H, chunk, strong_flag, nseg, tseg, static_cast<__nv_bfloat16*>(decayed), 0,
+    launch_after(gate_cumsum_kernel<64, true>, dim3(2 * B * H, (T + chunk - 1) / chunk), dim3(32, chunk / kCumRows), 0, st, gate, gate_kind, inv_tau, G, I, T, 2 * H, chunk, strong_flag, nseg, tseg, static_cast<__nv_bfloat16*>(decayed), 0,
         cu_seqlens, nseq, E);
     return cudaGetLastError();
 }
@@ -273,6 +273,7 @@ __global__ void __launch_bounds__(256) slot_softmax_fwd_kernel(const float* __re
                                                                int rows_per_batch, const float* __restrict__ G,
                                                                __nv_bfloat16* __restrict__ p_decayed,
                                                                PendingDecay pend, int m_active) {
+    follow_previous_grid();
     constexpr int R = kSmR, LPR = M / R, RPW = 32 / LPR;       // lanes per row, rows per warp
     const int lane = threadIdx.x & 31, sub = lane / LPR, l = lane % LPR;
     const int r_in_b = (blockIdx.x * 8 + (threadIdx.x >> 5)) * RPW + sub, b = blockIdx.y;
@@ -344,13 +345,13 @@ cudaError_t launch_slot_softmax_fwd(const float* part, int nslice, float scale, 
     const dim3 grid((unsigned)((rows_per_batch + rpb - 1) / rpb), (unsigned)B);
     const int rows = rows_per_batch;
     if (M == 128)
-        slot_softmax_fwd_kernel<128><<<grid, 256, 0, st>>>(part, nslice, scale, act, ok, p, rows, G,
+        launch_after(slot_softmax_fwd_kernel<128>, grid, 256, 0, st, part, nslice, scale, act, ok, p, rows, G,
                                                            static_cast<__nv_bfloat16*>(p_decayed), pend, m_active);
     else if (M == 64)
-        slot_softmax_fwd_kernel<64><<<grid, 256, 0, st>>>(part, nslice, scale, act, ok, p, rows, G,
+        launch_after(slot_softmax_fwd_kernel<64>, grid, 256, 0, st, part, nslice, scale, act, ok, p, rows, G,
                                                           static_cast<__nv_bfloat16*>(p_decayed), pend, m_active);
     else
-        slot_softmax_fwd_kernel<32><<<grid, 256, 0, st>>>(part, nslice, scale, act, ok, p, rows, G,
+        launch_after(slot_softmax_fwd_kernel<32>, grid, 256, 0, st, part, nslice, scale, act, ok, p, rows, G,
                                                           static_cast<__nv_bfloat16*>(p_decayed), pend, m_active);
     return cudaGetLastError();
 }
@@ -371,6 +372,7 @@ __global__ void __launch_bounds__(256) slot_softmax_bwd_kernel(const float* __re
                                                                __nv_bfloat16* __restrict__ p_decayed,
                                                                __nv_bfloat16* __restrict__ dz_decayed,
                                                                PendingDecay pend, int m_active) {
+    follow_previous_grid();
     constexpr int R = kSmR, LPR = M / R, RPW = 32 / LPR;       // lanes per row, rows per warp
     const int lane = threadIdx.x & 31, sub = lane / LPR, l = lane % LPR;
     const int r_in_b = (blockIdx.x * 8 + (threadIdx.x >> 5)) * RPW + sub, b = blockIdx.y;
@@ -461,15 +463,15 @@ cudaError_t launch_slot_softmax_bwd(const float* ok, const float* dp_part, int n
     const dim3 grid((unsigned)((rows_per_batch + rpb - 1) / rpb), (unsigned)B);
     const int rows = rows_per_batch;
     if (M == 128)
-        slot_softmax_bwd_kernel<128><<<grid, 256, 0, st>>>(ok, dp_part, nslice, scale, act, p, dz, u, rows, G,
+        launch_after(slot_softmax_bwd_kernel<128>, grid, 256, 0, st, ok, dp_part, nslice, scale, act, p, dz, u, rows, G,
                                                            static_cast<__nv_bfloat16*>(p_decayed),
                                                            static_cast<__nv_bfloat16*>(dz_decayed), pend, m_active);
     else if (M == 64)
-        slot_softmax_bwd_kernel<64><<<grid, 256, 0, st>>>(ok, dp_part, nslice, scale, act, p, dz, u, rows, G,
+        launch_after(slot_softmax_bwd_kernel<64>, grid, 256, 0, st, ok, dp_part, nslice, scale, act, p, dz, u, rows, G,
                                                           static_cast<__nv_bfloat16*>(p_decayed),
                                                           static_cast<__nv_bfloat16*>(dz_decayed), pend, m_active);
     else
-        slot_softmax_bwd_kernel<32><<<grid, 256, 0, st>>>(ok, dp_part, nslice, scale, act, p, dz, u, rows, G,
+        launch_after(slot_softmax_bwd_kernel<32>, grid, 256, 0, st, ok, dp_part, nslice, scale, act, p, dz, u, rows, G,
                                                           static_cast<__nv_bfloat16*>(p_decayed),
                                                           static_cast<__nv_bfloat16*>(dz_decayed), pend, m_active);
     return cudaGetLastError();
@@ -544,6 +546,7 @@ __global__ void __launch_bounds__(M * (M > 64 ? 8 : 16)) gate_grad_scan_kernel(
     float* __restrict__ blk_tot, const float* __restrict__ dKT, const float* __restrict__ KT,
     const float* __restrict__ dVT, const float* __restrict__ VT, int d_k, int d_v, int nblk,
     const int* __restrict__ cu, int nseq) {
+    follow_previous_grid();
     constexpr int kSeg = M > 64 ? 8 : 16;       // segments of consecutive blocks (threads: M slots x kSeg)
     __shared__ double seg_sum[kSeg][M];
     const int s = threadIdx.x, seg = threadIdx.y, bh = blockIdx.x;
@@ -607,6 +610,7 @@ __global__ void __launch_bounds__(128) gate_grad_local_kernel(
     const float* __restrict__ dIv, int nsv, const float* __restrict__ gate, int gate_kind, float inv_tau,
     float* __restrict__ blk_tot, float* __restrict__ dgate, int B, int T, int H, int nblk, PendingDecay pend,
     const int* __restrict__ cu, int nseq) {
+    follow_previous_grid();
     const int s = 2 * threadIdx.x;                       // this thread's two slots
     const int n = blockIdx.y * blockDim.y + threadIdx.y;
     if (n >= nblk) return;
@@ -668,6 +672,7 @@ __global__ void __launch_bounds__(256) gate_grad_local_tma_kernel(
     const __grid_constant__ CUtensorMap mapDIk, const __grid_constant__ CUtensorMap mapDIv, int nsk, int nsv,
     int gate_kind, float inv_tau, float* __restrict__ blk_tot, float* __restrict__ dgate, int T, int H, int nblk,
     PendingDecay pend, const int* __restrict__ cu, int nseq, int32_t* dev_status) {
+    follow_previous_grid();
     using namespace tc;
     constexpr int M = 64;
     extern __shared__ unsigned char gg_smem_raw[];
@@ -770,6 +775,7 @@ __global__ void __launch_bounds__(kGGComputeThreads + 32) gate_grad_local_ring_k
     const __grid_constant__ CUtensorMap mapDIk, const __grid_constant__ CUtensorMap mapDIv, int nsk, int nsv,
     int gate_kind, float inv_tau, float* __restrict__ blk_tot, float* __restrict__ dgate, int T, int H, int BH,
     int ntile, int nstage, int nblk, PendingDecay pend, const int* __restrict__ cu, int nseq, int32_t* dev_status) {
+    follow_previous_grid();
     using namespace tc;
     constexpr int M = 64;
     extern __shared__ unsigned char gg_smem_raw[];
@@ -902,6 +908,7 @@ template <int M>
 __global__ void __launch_bounds__(256) gate_grad_carry_kernel(
     const float* __restrict__ gate, int gate_kind, float inv_tau, const float* __restrict__ blk_carry,
     float* __restrict__ dgate, int T, int H, int nblk, const int* __restrict__ cu, int nseq) {
+    follow_previous_grid();
     constexpr int kRows = kGG / 2;
     const int s = 2 * threadIdx.x;
     const int n = blockIdx.y * blockDim.y + threadIdx.y;
@@ -979,8 +986,7 @@ cudaError_t launch_gate_grad(const float* u, const float* I, const float* dIk_pa
             const int BH = B * H, ntile = (T + kGGTmaRows - 1) / kGGTmaRows;
             const long long total = (long long)BH * ntile;
             const int ctas = (int)(total < sm_count ? total : sm_count);      // one persistent CTA per SM
-            gate_grad_local_ring_kernel<<<ctas, kGGComputeThreads + 32, smem, st>>>(
-                mu, mi, mg, mG, mk, mv, nsk, nsv, gate_kind, inv_tau, blk_tot, dgate, T, H, BH, ntile, nstage, nblk,
+            launch_after(gate_grad_local_ring_kernel, ctas, kGGComputeThreads + 32, smem, st, mu, mi, mg, mG, mk, mv, nsk, nsv, gate_kind, inv_tau, blk_tot, dgate, T, H, BH, ntile, nstage, nblk,
                 pend, cu_seqlens, nseq, dev_status);
         } else if (staged) {
             const size_t smem = 1024 + (size_t)(4 + nsl) * kGGTileB;
@@ -988,24 +994,24 @@ cudaError_t launch_gate_grad(const float* u, const float* I, const float* dIk_pa
                                                  (int)smem);
             if (e != cudaSuccess) return e;
             dim3 tgrid(B * H, (T + kGGTmaRows - 1) / kGGTmaRows);
-            gate_grad_local_tma_kernel<<<tgrid, 256, smem, st>>>(mu, mi, mg, mG, mk, mv, nsk, nsv, gate_kind, inv_tau, blk_tot,
+            launch_after(gate_grad_local_tma_kernel, tgrid, 256, smem, st, mu, mi, mg, mG, mk, mv, nsk, nsv, gate_kind, inv_tau, blk_tot,
                                                                 dgate, T, H, nblk, pend, cu_seqlens, nseq, dev_status);
         } else {
-            gate_grad_local_kernel<64><<<grid, block, 0, st>>>(u, I, dIk_part, nsk, dIv_part, nsv, gate, gate_kind, inv_tau,
+            launch_after(gate_grad_local_kernel<64>, grid, block, 0, st, u, I, dIk_part, nsk, dIv_part, nsv, gate, gate_kind, inv_tau,
                                                                blk_tot, dgate, B, T, H, nblk, pend, cu_seqlens, nseq);
         }
-        gate_grad_scan_kernel<64><<<B * H, dim3(64, 16), 0, st>>>(blk_tot, dKT, KT, dVT, VT, d_k, d_v, nblk, cu_seqlens, nseq);
-        gate_grad_carry_kernel<64><<<grid, dim3(block.x, block.y, 2), 0, st>>>(gate, gate_kind, inv_tau, blk_tot, dgate, T, H, nblk, cu_seqlens, nseq);
+        launch_after(gate_grad_scan_kernel<64>, B * H, dim3(64, 16), 0, st, blk_tot, dKT, KT, dVT, VT, d_k, d_v, nblk, cu_seqlens, nseq);
+        launch_after(gate_grad_carry_kernel<64>, grid, dim3(block.x, block.y, 2), 0, st, gate, gate_kind, inv_tau, blk_tot, dgate, T, H, nblk, cu_seqlens, nseq);
     } else if (M == 128) {
-        gate_grad_local_kernel<128><<<grid, block, 0, st>>>(u, I, dIk_part, nsk, dIv_part, nsv, gate, gate_kind, inv_tau,
+        launch_after(gate_grad_local_kernel<128>, grid, block, 0, st, u, I, dIk_part, nsk, dIv_part, nsv, gate, gate_kind, inv_tau,
                                                             blk_tot, dgate, B, T, H, nblk, pend, cu_seqlens, nseq);
-        gate_grad_scan_kernel<128><<<B * H, dim3(128, 8), 0, st>>>(blk_tot, dKT, KT, dVT, VT, d_k, d_v, nblk, cu_seqlens, nseq);
-        gate_grad_carry_kernel<128><<<grid, dim3(block.x, block.y, 2), 0, st>>>(gate, gate_kind, inv_tau, blk_tot, dgate, T, H, nblk, cu_seqlens, nseq);
+        launch_after(gate_grad_scan_kernel<128>, B * H, dim3(128, 8), 0, st, blk_tot, dKT, KT, dVT, VT, d_k, d_v, nblk, cu_seqlens, nseq);
+        launch_after(gate_grad_carry_kernel<128>, grid, dim3(block.x, block.y, 2), 0, st, gate, gate_kind, inv_tau, blk_tot, dgate, T, H, nblk, cu_seqlens, nseq);
     } else {
-        gate_grad_local_kernel<32><<<grid, block, 0, st>>>(u, I, dIk_part, nsk, dIv_part, nsv, gate, gate_kind, inv_tau,
+        launch_after(gate_grad_local_kernel<32>, grid, block, 0, st, u, I, dIk_part, nsk, dIv_part, nsv, gate, gate_kind, inv_tau,
                                                            blk_tot, dgate, B, T, H, nblk, pend, cu_seqlens, nseq);
-        gate_grad_scan_kernel<32><<<B * H, dim3(32, 16), 0, st>>>(blk_tot, dKT, KT, dVT, VT, d_k, d_v, nblk, cu_seqlens, nseq);
-        gate_grad_carry_kernel<32><<<grid, dim3(block.x, block.y, 2), 0, st>>>(gate, gate_kind, inv_tau, blk_tot, dgate, T, H, nblk, cu_seqlens, nseq);
+        launch_after(gate_grad_scan_kernel<32>, B * H, dim3(32, 16), 0, st, blk_tot, dKT, KT, dVT, VT, d_k, d_v, nblk, cu_seqlens, nseq);
+        launch_after(gate_grad_carry_kernel<32>, grid, dim3(block.x, block.y, 2), 0, st, gate, gate_kind, inv_tau, blk_tot, dgate, T, H, nblk, cu_seqlens, nseq);
     }
     return cudaGetLastError();
 }
@@ -1023,6 +1029,7 @@ template <int M>
 __global__ void __launch_bounds__(M) abc_write_kernel(const float* __restrict__ s_in, float* __restrict__ G,
                                                       float* __restrict__ I, __nv_bfloat16* __restrict__ decayed, int T,
                                                       int H) {
+    follow_previous_grid();
     const int bh = blockIdx.x, b = bh / H, h = bh % H, s = threadIdx.x;
     const size_t stride = (size_t)H * M;
     size_t idx = ((size_t)b * T * H + h) * M + s;
@@ -1061,6 +1068,7 @@ template <int M>
 __global__ void __launch_bounds__(M) abc_grad_kernel(const float* __restrict__ phi_in, const float* __restrict__ dIk, int nsk,
                                                      const float* __restrict__ dIv, int nsv, float* __restrict__ ds, int T,
                                                      int H, size_t total) {
+    follow_previous_grid();
     const int bh = blockIdx.x, b = bh / H, h = bh % H, s = threadIdx.x;
     const size_t stride = (size_t)H * M;
     const size_t base = ((size_t)b * T * H + h) * M + s;
@@ -1090,17 +1098,17 @@ __global__ void __launch_bounds__(M) abc_grad_kernel(const float* __restrict__ p
 }
 
 cudaError_t launch_abc_write(const float* s_in, float* G, float* I, void* decayed, int B, int T, int H, int M, cudaStream_t st) {
-    if (M == 128) abc_write_kernel<128><<<B * H, 128, 0, st>>>(s_in, G, I, static_cast<__nv_bfloat16*>(decayed), T, H);
-    else if (M == 64) abc_write_kernel<64><<<B * H, 64, 0, st>>>(s_in, G, I, static_cast<__nv_bfloat16*>(decayed), T, H);
-    else abc_write_kernel<32><<<B * H, 32, 0, st>>>(s_in, G, I, static_cast<__nv_bfloat16*>(decayed), T, H);
+    if (M == 128) launch_after(abc_write_kernel<128>, B * H, 128, 0, st, s_in, G, I, static_cast<__nv_bfloat16*>(decayed), T, H);
+    else if (M == 64) launch_after(abc_write_kernel<64>, B * H, 64, 0, st, s_in, G, I, static_cast<__nv_bfloat16*>(decayed), T, H);
+    else launch_after(abc_write_kernel<32>, B * H, 32, 0, st, s_in, G, I, static_cast<__nv_bfloat16*>(decayed), T, H);
     return cudaGetLastError();
 }
 cudaError_t launch_abc_grad(const float* phi, const float* dIk, int nsk, const float* dIv, int nsv, float* ds, int B, int T,
                             int H, int M, cudaStream_t st) {
     const size_t total = (size_t)B * T * H * M;
-    if (M == 128) abc_grad_kernel<128><<<B * H, 128, 0, st>>>(phi, dIk, nsk, dIv, nsv, ds, T, H, total);
-    else if (M == 64) abc_grad_kernel<64><<<B * H, 64, 0, st>>>(phi, dIk, nsk, dIv, nsv, ds, T, H, total);
-    else abc_grad_kernel<32><<<B * H, 32, 0, st>>>(phi, dIk, nsk, dIv, nsv, ds, T, H, total);
+    if (M == 128) launch_after(abc_grad_kernel<128>, B * H, 128, 0, st, phi, dIk, nsk, dIv, nsv, ds, T, H, total);
+    else if (M == 64) launch_after(abc_grad_kernel<64>, B * H, 64, 0, st, phi, dIk, nsk, dIv, nsv, ds, T, H, total);
+    else launch_after(abc_grad_kernel<32>, B * H, 32, 0, st, phi, dIk, nsk, dIv, nsv, ds, T, H, total);
     return cudaGetLastError();
 }
 
@@ -1109,12 +1117,14 @@ cudaError_t launch_abc_grad(const float* phi, const float* dIk, int nsk, const f
 // row [H, M] for all tokens: it is spread over [B,T,H,M] on the way in, and the gate gradient is
 // summed over the tokens on the way out (partial sums per block of rows, added in order).
 __global__ void broadcast_rows_kernel(const float* __restrict__ row, float* __restrict__ out, size_t rows, int n) {
+    follow_previous_grid();
     const size_t total = rows * (size_t)n;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x)
         out[i] = row[i % n];
 }
 constexpr int kColSumRows = 256;
 __global__ void column_partial_kernel(const float* __restrict__ in, float* __restrict__ part, size_t rows, int n) {
+    follow_previous_grid();
     const int c = blockIdx.y * blockDim.x + threadIdx.x;
     if (c >= n) return;
     const size_t r0 = (size_t)blockIdx.x * kColSumRows;
@@ -1124,6 +1134,7 @@ __global__ void column_partial_kernel(const float* __restrict__ in, float* __res
     part[(size_t)blockIdx.x * n + c] = acc;
 }
 __global__ void column_final_kernel(const float* __restrict__ part, float* __restrict__ out, int nparts, int n) {
+    follow_previous_grid();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= n) return;
     double acc = 0.0;
@@ -1133,20 +1144,21 @@ __global__ void column_final_kernel(const float* __restrict__ part, float* __res
 cudaError_t launch_broadcast_rows(const float* row, float* out, size_t rows, int n, cudaStream_t st) {
     const size_t total = rows * (size_t)n;
     const unsigned blocks = (unsigned)((total + 255) / 256 < 148 * 32 ? (total + 255) / 256 : 148 * 32);
-    broadcast_rows_kernel<<<blocks ? blocks : 1, 256, 0, st>>>(row, out, rows, n);
+    launch_after(broadcast_rows_kernel, blocks ? blocks : 1, 256, 0, st, row, out, rows, n);
     return cudaGetLastError();
 }
 size_t column_sum_parts(size_t rows) { return (rows + kColSumRows - 1) / kColSumRows; }
 // out[c] = sum over rows of in[r][c]; part: column_sum_parts(rows) * n floats of scratch
 cudaError_t launch_column_sum(const float* in, float* part, float* out, size_t rows, int n, cudaStream_t st) {
     const unsigned parts = (unsigned)column_sum_parts(rows);
-    column_partial_kernel<<<dim3(parts, (n + 127) / 128), 128, 0, st>>>(in, part, rows, n);
-    column_final_kernel<<<(n + 127) / 128, 128, 0, st>>>(part, out, (int)parts, n);
+    launch_after(column_partial_kernel, dim3(parts, (n + 127) / 128), 128, 0, st, in, part, rows, n);
+    launch_after(column_final_kernel, (n + 127) / 128, 128, 0, st, part, out, (int)parts, n);
     return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ gate tensor in bfloat16
 __global__ void widen_bf16_kernel(const __nv_bfloat16* __restrict__ in, float* __restrict__ out, size_t n) {
+    follow_previous_grid();
     for (size_t i = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * 2; i < n; i += (size_t)gridDim.x * blockDim.x * 2) {
         if (i + 1 < n) {
             const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(in + i));
@@ -1159,7 +1171,7 @@ __global__ void widen_bf16_kernel(const __nv_bfloat16* __restrict__ in, float* _
 cudaError_t launch_widen_bf16(const void* in, float* out, size_t n, cudaStream_t st) {
     const size_t pairs = (n + 1) / 2;
     const unsigned blocks = (unsigned)((pairs + 255) / 256 < 148 * 32 ? (pairs + 255) / 256 : 148 * 32);
-    widen_bf16_kernel<<<blocks ? blocks : 1, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(in), out, n);
+    launch_after(widen_bf16_kernel, blocks ? blocks : 1, 256, 0, st, static_cast<const __nv_bfloat16*>(in), out, n);
     return cudaGetLastError();
 }
 
@@ -1169,6 +1181,7 @@ cudaError_t launch_widen_bf16(const void* in, float* out, size_t n, cudaStream_t
 // tensor-core kernels: gate rows are widened with a neutral gate, memories with empty slots.
 __global__ void resize_rows_kernel(const float* __restrict__ in, float* __restrict__ out, size_t rows, int n_in, int n_out,
                                    float fill) {
+    follow_previous_grid();
     const size_t total = rows * (size_t)n_out;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         const size_t r = i / n_out;
@@ -1179,7 +1192,7 @@ __global__ void resize_rows_kernel(const float* __restrict__ in, float* __restri
 cudaError_t launch_resize_rows(const float* in, float* out, size_t rows, int n_in, int n_out, float fill, cudaStream_t st) {
     const size_t total = rows * (size_t)n_out;
     const unsigned blocks = (unsigned)((total + 255) / 256 < 148 * 32 ? (total + 255) / 256 : 148 * 32);
-    resize_rows_kernel<<<blocks ? blocks : 1, 256, 0, st>>>(in, out, rows, n_in, n_out, fill);
+    launch_after(resize_rows_kernel, blocks ? blocks : 1, 256, 0, st, in, out, rows, n_in, n_out, fill);
     return cudaGetLastError();
 }
 
@@ -1193,6 +1206,7 @@ cudaError_t launch_resize_rows(const float* in, float* out, size_t rows, int n_i
 template <int M>
 __global__ void segment_logdecay_kernel(const float* __restrict__ G, float* __restrict__ seg_logdecay, int T, int H,
                                         int nseg, int tseg, int chunk) {
+    follow_previous_grid();
     const int s = threadIdx.x, h = blockIdx.y;
     const int b = blockIdx.x / nseg, r = blockIdx.x % nseg;
     const int t_begin = r * tseg, t_end = min(T, t_begin + tseg);
@@ -1209,6 +1223,7 @@ __global__ void segment_logdecay_kernel(const float* __restrict__ G, float* __re
 template <int M>
 __global__ void segment_combine_kernel(const float* __restrict__ seg_logdecay, CombineSet k, CombineSet v, int H, int nseg,
                                        int reverse) {
+    follow_previous_grid();
     const int b = blockIdx.x / H, h = blockIdx.x % H;
     int idx = blockIdx.y * blockDim.x + threadIdx.x;
     const bool second = idx >= M * k.D;
@@ -1235,6 +1250,7 @@ __global__ void segment_combine_kernel(const float* __restrict__ seg_logdecay, C
 __global__ void shard_combine_kernel(const float* __restrict__ logdecay_all, const float* __restrict__ local_all,
                                      const float* __restrict__ S0, float* __restrict__ start, float* __restrict__ final_state,
                                      int BH, int M, int D, int nshard, int rank, int reverse) {
+    follow_previous_grid();
     const int bh = blockIdx.x;
     const int idx = blockIdx.y * blockDim.x + threadIdx.x;
     if (idx >= M * D) return;
@@ -1252,25 +1268,25 @@ cudaError_t launch_shard_combine(const float* logdecay_all, const float* local_a
                                  float* final_state, int B, int H, int M, int D, int nshard, int rank, int reverse,
                                  cudaStream_t st) {
     dim3 grid(B * H, (M * D + 255) / 256);
-    shard_combine_kernel<<<grid, 256, 0, st>>>(logdecay_all, local_all, S0, start, final_state, B * H, M, D, nshard, rank, reverse);
+    launch_after(shard_combine_kernel, grid, 256, 0, st, logdecay_all, local_all, S0, start, final_state, B * H, M, D, nshard, rank, reverse);
     return cudaGetLastError();
 }
 
 cudaError_t launch_segment_logdecay(const float* G, float* seg_logdecay, int B, int T, int H, int M, int nseg,
                                     int tseg, int chunk, cudaStream_t st) {
     dim3 grid(B * nseg, H);
-    if (M == 128) segment_logdecay_kernel<128><<<grid, 128, 0, st>>>(G, seg_logdecay, T, H, nseg, tseg, chunk);
-    else if (M == 64) segment_logdecay_kernel<64><<<grid, 64, 0, st>>>(G, seg_logdecay, T, H, nseg, tseg, chunk);
-    else segment_logdecay_kernel<32><<<grid, 32, 0, st>>>(G, seg_logdecay, T, H, nseg, tseg, chunk);
+    if (M == 128) launch_after(segment_logdecay_kernel<128>, grid, 128, 0, st, G, seg_logdecay, T, H, nseg, tseg, chunk);
+    else if (M == 64) launch_after(segment_logdecay_kernel<64>, grid, 64, 0, st, G, seg_logdecay, T, H, nseg, tseg, chunk);
+    else launch_after(segment_logdecay_kernel<32>, grid, 32, 0, st, G, seg_logdecay, T, H, nseg, tseg, chunk);
     return cudaGetLastError();
 }
 
 cudaError_t launch_segment_combine(const float* seg_logdecay, CombineSet k, CombineSet v, int B, int H, int M, int nseg,
                                    int reverse, cudaStream_t st) {
     dim3 grid(B * H, (M * (k.D + v.D) + 255) / 256);
-    if (M == 128) segment_combine_kernel<128><<<grid, 256, 0, st>>>(seg_logdecay, k, v, H, nseg, reverse);
-    else if (M == 64) segment_combine_kernel<64><<<grid, 256, 0, st>>>(seg_logdecay, k, v, H, nseg, reverse);
-    else segment_combine_kernel<32><<<grid, 256, 0, st>>>(seg_logdecay, k, v, H, nseg, reverse);
+    if (M == 128) launch_after(segment_combine_kernel<128>, grid, 256, 0, st, seg_logdecay, k, v, H, nseg, reverse);
+    else if (M == 64) launch_after(segment_combine_kernel<64>, grid, 256, 0, st, seg_logdecay, k, v, H, nseg, reverse);
+    else launch_after(segment_combine_kernel<32>, grid, 256, 0, st, seg_logdecay, k, v, H, nseg, reverse);
     return cudaGetLastError();
 }
 
