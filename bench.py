@@ -457,14 +457,12 @@ def run_ours(args):
         per = {}
         for lab, ms in recs:
             per.setdefault(lab, []).append(ms)
-        # kernels behind one label: gate_grad is three; every chunk pass is two (the lean and the
-        # general variant of the kernel are both launched, each CTA runs in one of them)
-        two = sum(len(v) for lab, v in per.items() if lab.endswith("_side") or lab.endswith("_side_rev"))
+        # kernels behind one label: gate_grad is three; a chunk pass is one, with 128 slots two (the flagged pairs
+        # have a launch of their own there)
+        two = sum(len(v) for lab, v in per.items() if lab.endswith("_side") or lab.endswith("_side_rev")) if w.m == 128 else 0
         # a fused label is the fused kernel plus the three kernels that serve the flagged pairs
         fusedl = sum(len(v) for lab, v in per.items() if lab.startswith("fused"))
-        # a pair label is the pair kernel plus the two general kernels that serve the flagged pairs
-        pairl = sum(len(v) for lab, v in per.items() if "pair_rev" in lab)
-        launches = (len(recs) + 2 * len(per.get("gate_grad", [])) + two + 3 * fusedl + 2 * pairl) // reps
+        launches = (len(recs) + 2 * len(per.get("gate_grad", [])) + two + 3 * fusedl) // reps
         kernels = []
         tot = sum(sum(v) for v in per.values())
         for lab, v in per.items():
@@ -848,7 +846,7 @@ def main():
                          "seq (every rank a T-shard of the same sequences, one all-gather of shard memories)")
     ap.add_argument("--m", type=int, default=0, choices=[0, 32, 64, 128],
                     help="slot count on the benchmark shape (default: the workload's 64); 32 runs on the tensor-core "
-                         "kernels' 64-slot tiles, 128 on the fp32 CUDA-core kernels")
+                         "kernels' 64-slot tiles, 128 on kernels of their own")
     ap.add_argument("--fuse", action="store_true",
                     help="the fused chunk kernel (pass 1 -> slot softmax -> pass 2 in one kernel, and its backward "
                          "twin) instead of the separate kernels; slower as measured, not the default")

@@ -147,15 +147,14 @@ typedef struct {
                          * cu_seqlens[nseq] = T, or NULL.  Every batch row then holds nseq sequences back
                          * to back (variable-length batches packed as B = 1): the memories are emptied at
                          * every offset, so each sequence is an independent recurrence; K0 / V0 enter the
-                         * first sequence, KT / VT leave the last.  gsa_fwd and gsa_bwd only.  The chunks
-                         * that hold an offset run on the strong-decay kernels. */
+                         * first sequence, KT / VT leave the last.  gsa_fwd and gsa_bwd only. */
 } gsa_params_t;
 
 enum { GSA_WS_FWD = 0, GSA_WS_BWD = 1, GSA_WS_DECODE = 2, GSA_WS_GATE = 3, GSA_WS_SHARD = 4 };
 
 /* Chunk length C of the chunkwise form that these params select (Algorithm 1 leaves C
- * open): 128 for the tensor-core kernels, 64 for the fp32 CUDA-core kernels; 0 for
- * invalid params. */
+ * open), as gsa_gate_cumsum sums by it: 128 for the tensor-core kernels, 64 for the fp32
+ * CUDA-core kernels and for 128 slots; 0 for invalid params. */
 GSA_API int32_t gsa_chunk_size(const gsa_params_t* params);
 
 /* Bytes of scratch `which` (GSA_WS_*) needs for these params; 0 for decode and

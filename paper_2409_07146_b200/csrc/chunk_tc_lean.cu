@@ -3,7 +3,7 @@
 // kFactorisedDecayMin), which is every pair of the paper's workloads except the strong-forgetting
 // stress case.
 //
-// Differences from the general kernels (chunk_tc.cu):
+// Differences from the general scans (chunk_tc_general.cuh), which a CTA whose pair is flagged runs instead:
 //   * the slot-sized operands arrive by TMA already multiplied by their decay factor and already
 //     in bfloat16 -- w exp(-G) or w exp(G) as a high/low pair, written once per (batch, head) by
 //     the element-wise kernels that produce w (gate kernel, slot softmax forward / backward)
@@ -14,7 +14,7 @@
 //     threads find their next accumulator ready when they finish a chunk.
 //   * tile copies and MMA issue are two lanes of two warps, so that a wait of one (for a store to
 //     drain, for a tile to land) never delays the other.
-// Tile geometry and the bounded waits are those of the general kernels.
+// Tile geometry and the bounded waits are those of the general scans.
 // The file also holds the state-only scan that segment-parallel scheduling uses for the end
 // memories of every segment (state_scan_kernel, below the two chunk kernels).
 #include "chunk_tc_general.cuh"

@@ -201,8 +201,7 @@ def test_bwd_strong_forgetting():
 
 @pytest.mark.parametrize("io", ["f32", "bf16"])
 def test_128_slots_fwd_bwd(io):
-    """m = 128 (the largest slot count of the paper's ablation on the number of slots) runs on the
-    CUDA-core kernels for either io type."""
+    """m = 128, the largest slot count of the paper's ablation on the number of slots, for either io type."""
     B, T, H, dk, dv, m = 2, 150, 2, 128, 64, 128
     d = rand_inputs(128 + len(io), B, T, H, dk, dv, m, io, init=True, final_grads=True)
     got, gate = run_fwd(d, B, T, H, dk, dv, m, io, scale=0.9)
