@@ -461,9 +461,10 @@ gsa_status_t apply_feature_map(const CallParams& p, int which, const void** q, c
     const FeatureBuffers f = carve_features(p, static_cast<char*>(ws) + before);
     if (ws_bytes < before + f.bytes) return GSA_ERR_WORKSPACE;
     const size_t R = (size_t)p.B * p.T * p.H;
-    if (launch_swish_fwd(*q, f.q, R * p.d_k, p.io, st) != cudaSuccess) return GSA_ERR_CUDA;
-    if (launch_swish_fwd(*k, f.k, R * p.d_k, p.io, st) != cudaSuccess) return GSA_ERR_CUDA;
-    if (launch_swish_fwd(*v, f.v, R * p.d_v, p.io, st) != cudaSuccess) return GSA_ERR_CUDA;
+    const void* const in[3] = {*q, *k, *v};
+    void* const out[3] = {f.q, f.k, f.v};
+    const size_t n[3] = {R * p.d_k, R * p.d_k, R * p.d_v};
+    if (launch_swish_fwd(in, out, n, p.io, st) != cudaSuccess) return GSA_ERR_CUDA;
     *q = f.q; *k = f.k; *v = f.v;
     return GSA_OK;
 }
@@ -971,10 +972,10 @@ gsa_status_t bwd_impl(const CallParams* params, const void* q, const void* k, co
             return GSA_ERR_CUDA;
         if (params->feature_map != GSA_FEAT_SWISH) return GSA_OK;
         const size_t R = (size_t)params->B * params->T * params->H;
-        if (launch_swish_bwd(q_raw, dq, R * params->d_k, params->io, s2) != cudaSuccess) return GSA_ERR_CUDA;
-        if (launch_swish_bwd(k_raw, dk, R * params->d_k, params->io, s2) != cudaSuccess) return GSA_ERR_CUDA;
-        if (launch_swish_bwd(v_raw, dv, R * params->d_v, params->io, s2) != cudaSuccess) return GSA_ERR_CUDA;
-        return GSA_OK;
+        const void* const x[3] = {q_raw, k_raw, v_raw};
+        void* const d[3] = {dq, dk, dv};
+        const size_t n[3] = {R * params->d_k, R * params->d_k, R * params->d_v};
+        return launch_swish_bwd(x, d, n, params->io, s2) == cudaSuccess ? GSA_OK : GSA_ERR_CUDA;
     };
     if (!pads_slots(*params))
         return finish(bwd_core(params, 0, q, k, v, gate, K0, V0, ok_saved, dO, dKT, dVT, dq, dk, dv, dgate, dK0, dV0,

@@ -306,8 +306,9 @@ cudaError_t launch_fused_pair(int mode, const void* xq1, const void* xk1, const 
                               int T, int H, int D1, int D2, float scale, int act, float* ok, float* u, void* Pd,
                               void* Zd, const int* strong_flag, cudaStream_t st, int32_t* dev_status);
 // layer pre- and post-operations (layer_ops.cu)
-cudaError_t launch_swish_fwd(const void* in, void* out, size_t n, int io, cudaStream_t st);
-cudaError_t launch_swish_bwd(const void* x, void* d, size_t n, int io, cudaStream_t st);
+// (q, k and v, or their gradients, in one launch)
+cudaError_t launch_swish_fwd(const void* const in[3], void* const out[3], const size_t n[3], int io, cudaStream_t st);
+cudaError_t launch_swish_bwd(const void* const x[3], void* const d[3], const size_t n[3], int io, cudaStream_t st);
 int out_norm_max_width(int io);
 size_t out_norm_bwd_parts(size_t rows);
 cudaError_t launch_out_norm_fwd(const void* o, const float* weight, float eps, void* y, size_t rows, int N, int io,

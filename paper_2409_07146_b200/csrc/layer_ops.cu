@@ -15,208 +15,252 @@
 namespace gsa {
 namespace {
 
-__device__ __forceinline__ float swishf(float x) { return x / (1.f + __expf(-x)); }
-__device__ __forceinline__ float swish_gradf(float x) {
-    const float s = 1.f / (1.f + __expf(-x));
-    return s * (1.f + x * (1.f - s));
-}
-
+// 1 / (1 + exp(-x)); where the results are rounded to bfloat16, by the approximate reciprocal (2 ulp of fp32): the IEEE
+// division is half of all instructions of these kernels
 template <typename IO>
-__global__ void __launch_bounds__(256) swish_fwd_kernel(const IO* __restrict__ in, IO* __restrict__ out, size_t nvec) {
+__device__ __forceinline__ float sigmoidf(float x);
+template <>
+__device__ __forceinline__ float sigmoidf<float>(float x) { return 1.f / (1.f + __expf(-x)); }
+template <>
+__device__ __forceinline__ float sigmoidf<__nv_bfloat16>(float x) { return __fdividef(1.f, 1.f + __expf(-x)); }
+__device__ __forceinline__ float swish_slope(float x, float sigmoid) { return sigmoid * (1.f + x * (1.f - sigmoid)); }
+
+// The feature map of q, k and v in one launch: blocks of kStream vectors a thread, all requested before the first is used
+// (one at a time, in a launch per tensor: 20 us for 41 MB in and out, 4.1 TB/s).
+constexpr int kStream = 4;
+struct SwishSet { const void* in; void* out; size_t nvec; };
+struct SwishSets { SwishSet t[3]; };
+template <typename IO, bool BWD>
+__global__ void __launch_bounds__(256) swish_kernel(const SwishSets sets) {
     follow_previous_grid();
     constexpr int V = IoTraits<IO>::kVec;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nvec; i += (size_t)gridDim.x * blockDim.x) {
-        float x[V];
-        load_vec(in + i * V, x);
+    const SwishSet& t = sets.t[blockIdx.y];
+    const IO* in = static_cast<const IO*>(t.in);
+    IO* out = static_cast<IO*>(t.out);
+    const size_t i0 = (size_t)blockIdx.x * (kStream * 256) + threadIdx.x;
+    float x[kStream][V], g[BWD ? kStream : 1][V];
 #pragma unroll
-        for (int e = 0; e < V; ++e) x[e] = swishf(x[e]);
-        store_vec(out + i * V, x);
-    }
-}
-// d <- d * Swish'(x), in place on the gradient
-template <typename IO>
-__global__ void __launch_bounds__(256) swish_bwd_kernel(const IO* __restrict__ x_in, IO* __restrict__ d, size_t nvec) {
-    follow_previous_grid();
-    constexpr int V = IoTraits<IO>::kVec;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nvec; i += (size_t)gridDim.x * blockDim.x) {
-        float x[V], g[V];
-        load_vec(x_in + i * V, x);
-        load_vec(d + i * V, g);
+    for (int j = 0; j < kStream; ++j)
+        if (i0 + j * 256 < t.nvec) {
+            load_vec(in + (i0 + j * 256) * V, x[j]);
+            if (BWD) load_vec(out + (i0 + j * 256) * V, g[BWD ? j : 0]);
+        }
 #pragma unroll
-        for (int e = 0; e < V; ++e) g[e] *= swish_gradf(x[e]);
-        store_vec(d + i * V, g);
-    }
+    for (int j = 0; j < kStream; ++j)
+        if (i0 + j * 256 < t.nvec) {
+#pragma unroll
+            for (int e = 0; e < V; ++e) {
+                const float s = sigmoidf<IO>(x[j][e]);
+                x[j][e] = BWD ? g[BWD ? j : 0][e] * swish_slope(x[j][e], s) : x[j][e] * s;
+            }
+            store_vec(out + (i0 + j * 256) * V, x[j]);
+        }
 }
 
-__device__ __forceinline__ float block_sum(float v, float* scratch) {
+// ---- the output path.  N = H d_v values of a token make up to 512 vectors of 16 bytes: a thread of the CTA owns one of
+// them, and kTokens tokens are in flight together, so that their loads overlap and one barrier serves their sums.
+constexpr int kTokens = 4;
+
+// sums over the CTA of n values per thread, the same in every thread and run; `scratch` (16 x n floats) is free again at
+// the next but one barrier
+template <int n>
+__device__ __forceinline__ void cta_sums(float (&v)[n], float (*scratch)[n]) {
 #pragma unroll
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    for (int i = 0; i < n; ++i)
+#pragma unroll
+        for (int o = 16; o; o >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    __syncthreads();                      // scratch may still be read from a previous call
-    if (lane == 0) scratch[warp] = v;
+    if (lane == 0) {
+#pragma unroll
+        for (int i = 0; i < n; ++i) scratch[warp][i] = v[i];
+    }
     __syncthreads();
-    float t = 0.f;
-    for (int w = 0; w < nw; ++w) t += scratch[w];     // same order in every thread: deterministic
-    return t;
+#pragma unroll
+    for (int i = 0; i < n; ++i) v[i] = 0.f;
+    for (int w = 0; w < nw; ++w) {
+#pragma unroll
+        for (int i = 0; i < n; ++i) v[i] += scratch[w][i];
+    }
 }
 
-// One CTA per token: y = w * Swish(o) / sqrt(mean(Swish(o)^2) + eps) over the N = H d_v values of the token.
-// A thread keeps up to kMaxVecPerThread vectors of the row in registers (N <= 256 threads * that * V).
-constexpr int kMaxVecPerThread = 2;
+// y = w * Swish(o) / sqrt(mean(Swish(o)^2) + eps), kTokens tokens a CTA.  Bound by memory: 82 MB at 8 K tokens of 2560
+// values; a CTA of 256 threads a token, two barriers each, took 39 us.
 template <typename IO>
-__global__ void __launch_bounds__(256) out_norm_fwd_kernel(const IO* __restrict__ o, const float* __restrict__ weight,
-                                                           float eps, IO* __restrict__ y, int N) {
+__global__ void __launch_bounds__(512) out_norm_fwd_kernel(const IO* __restrict__ o, const float* __restrict__ weight,
+                                                           float eps, IO* __restrict__ y, int N, size_t rows) {
     follow_previous_grid();
     constexpr int V = IoTraits<IO>::kVec;
-    __shared__ float scratch[8];
-    const size_t row = blockIdx.x;
-    const int nvec = N / V;
-    float x[kMaxVecPerThread][V];
-    float ss = 0.f;
+    __shared__ float scratch[16][kTokens];
+    const size_t row0 = (size_t)blockIdx.x * kTokens;
+    const int c = threadIdx.x * V;
+    const bool own = c < N;
+    float x[kTokens][V], ss[kTokens];
 #pragma unroll
-    for (int j = 0; j < kMaxVecPerThread; ++j) {
-        const int c = threadIdx.x + j * 256;
-        if (c < nvec) {
-            load_vec(o + row * N + (size_t)c * V, x[j]);
+    for (int r = 0; r < kTokens; ++r)
+        if (own && row0 + r < rows) load_vec(o + (row0 + r) * N + c, x[r]);
 #pragma unroll
-            for (int e = 0; e < V; ++e) { x[j][e] = swishf(x[j][e]); ss += x[j][e] * x[j][e]; }
+    for (int r = 0; r < kTokens; ++r) {
+        ss[r] = 0.f;
+        if (own && row0 + r < rows) {
+#pragma unroll
+            for (int e = 0; e < V; ++e) { x[r][e] *= sigmoidf<IO>(x[r][e]); ss[r] += x[r][e] * x[r][e]; }
         }
     }
-    const float inv = rsqrtf(block_sum(ss, scratch) / (float)N + eps);
+    cta_sums(ss, scratch);
+    if (!own) return;
+    float w[V];
 #pragma unroll
-    for (int j = 0; j < kMaxVecPerThread; ++j) {
-        const int c = threadIdx.x + j * 256;
-        if (c < nvec) {
+    for (int e = 0; e < V; ++e) w[e] = weight ? weight[c + e] : 1.f;
 #pragma unroll
-            for (int e = 0; e < V; ++e) x[j][e] *= inv * (weight ? weight[c * V + e] : 1.f);
-            store_vec(y + row * N + (size_t)c * V, x[j]);
+    for (int r = 0; r < kTokens; ++r)
+        if (row0 + r < rows) {
+            const float inv = rsqrtf(ss[r] / (float)N + eps);
+#pragma unroll
+            for (int e = 0; e < V; ++e) x[r][e] *= inv * w[e];
+            store_vec(y + (row0 + r) * N + c, x[r]);
         }
-    }
 }
 
-// Backward: a CTA takes kRowsPerCta consecutive tokens (so that the weight gradient can be summed
-// over them in registers, one partial row per CTA; a second kernel adds the partial rows in order).
+// Backward: a CTA takes kRowsPerCta consecutive tokens, kTokens at a time (so that the weight gradient can be summed over
+// them in registers, one partial row per CTA; a second kernel adds the partial rows in order).  With x = Swish(o), g = w dy
+// and r = 1 / sqrt(mean(x^2) + eps):  d_o = r (g - x r^2 mean(g x)) Swish'(o) -- both means in one pass over the tokens'
+// values, which stay in registers as they came.  One token at a time, two means after one another: 143 us at 8 K tokens
+// of 2560 values (123 MB).
 constexpr int kRowsPerCta = 16;
 template <typename IO>
-__global__ void __launch_bounds__(256) out_norm_bwd_kernel(const IO* __restrict__ o, const IO* __restrict__ dy,
+__global__ void __launch_bounds__(512) out_norm_bwd_kernel(const IO* __restrict__ o, const IO* __restrict__ dy,
                                                            const float* __restrict__ weight, float eps, IO* __restrict__ d_o,
                                                            float* __restrict__ dw_part, int N, size_t rows) {
     follow_previous_grid();
     constexpr int V = IoTraits<IO>::kVec;
-    __shared__ float scratch[8];
-    const int nvec = N / V;
-    float dw[kMaxVecPerThread][V];
+    __shared__ float scratch[2][16][2 * kTokens];
+    const int c = threadIdx.x * V;
+    const bool own = c < N;
+    float dw[V], w[V];
 #pragma unroll
-    for (int j = 0; j < kMaxVecPerThread; ++j)
+    for (int e = 0; e < V; ++e) {
+        dw[e] = 0.f;
+        w[e] = weight && own ? weight[c + e] : 1.f;
+    }
+    for (int r0 = 0; r0 < kRowsPerCta; r0 += kTokens) {
+        const size_t row0 = (size_t)blockIdx.x * kRowsPerCta + r0;
+        if (row0 >= rows) break;
+        uint4 ov[kTokens], gv[kTokens];
 #pragma unroll
-        for (int e = 0; e < V; ++e) dw[j][e] = 0.f;
-    for (int r = 0; r < kRowsPerCta; ++r) {
-        const size_t row = (size_t)blockIdx.x * kRowsPerCta + r;
-        if (row >= rows) break;
-        float ov[kMaxVecPerThread][V], x[kMaxVecPerThread][V], g[kMaxVecPerThread][V];
-        float ss = 0.f;
-#pragma unroll
-        for (int j = 0; j < kMaxVecPerThread; ++j) {
-            const int c = threadIdx.x + j * 256;
-            if (c < nvec) {
-                load_vec(o + row * N + (size_t)c * V, ov[j]);
-                load_vec(dy + row * N + (size_t)c * V, g[j]);
-#pragma unroll
-                for (int e = 0; e < V; ++e) { x[j][e] = swishf(ov[j][e]); ss += x[j][e] * x[j][e]; }
+        for (int r = 0; r < kTokens; ++r)
+            if (own && row0 + r < rows) {
+                ov[r] = *reinterpret_cast<const uint4*>(o + (row0 + r) * N + c);
+                gv[r] = *reinterpret_cast<const uint4*>(dy + (row0 + r) * N + c);
             }
-        }
-        const float inv = rsqrtf(block_sum(ss, scratch) / (float)N + eps);
-        float dot = 0.f;
+        float sums[2 * kTokens];
 #pragma unroll
-        for (int j = 0; j < kMaxVecPerThread; ++j) {
-            const int c = threadIdx.x + j * 256;
-            if (c < nvec) {
+        for (int r = 0; r < kTokens; ++r) {
+            float ss = 0.f, dot = 0.f;
+            if (own && row0 + r < rows) {
+                float x[V], g[V];
+                load_vec(reinterpret_cast<const IO*>(&ov[r]), x);
+                load_vec(reinterpret_cast<const IO*>(&gv[r]), g);
 #pragma unroll
                 for (int e = 0; e < V; ++e) {
-                    x[j][e] *= inv;                                         // xhat
-                    dw[j][e] += g[j][e] * x[j][e];
-                    g[j][e] *= weight ? weight[c * V + e] : 1.f;           // gradient w.r.t. xhat
-                    dot += g[j][e] * x[j][e];
+                    x[e] *= sigmoidf<IO>(x[e]);
+                    ss += x[e] * x[e];
+                    dot += g[e] * w[e] * x[e];
                 }
             }
+            sums[2 * r] = ss;
+            sums[2 * r + 1] = dot;
         }
-        const float mean = block_sum(dot, scratch) / (float)N;
+        cta_sums(sums, scratch[(r0 / kTokens) & 1]);
 #pragma unroll
-        for (int j = 0; j < kMaxVecPerThread; ++j) {
-            const int c = threadIdx.x + j * 256;
-            if (c < nvec) {
+        for (int r = 0; r < kTokens; ++r)
+            if (own && row0 + r < rows) {
+                const float inv = rsqrtf(sums[2 * r] / (float)N + eps);
+                const float mean = sums[2 * r + 1] * inv / (float)N;          // mean of g times x inv
+                float x[V], g[V];
+                load_vec(reinterpret_cast<const IO*>(&ov[r]), x);
+                load_vec(reinterpret_cast<const IO*>(&gv[r]), g);
 #pragma unroll
-                for (int e = 0; e < V; ++e) g[j][e] = (g[j][e] - x[j][e] * mean) * inv * swish_gradf(ov[j][e]);
-                store_vec(d_o + row * N + (size_t)c * V, g[j]);
+                for (int e = 0; e < V; ++e) {
+                    const float s = sigmoidf<IO>(x[e]), xhat = x[e] * s * inv;
+                    dw[e] += g[e] * xhat;
+                    g[e] = (g[e] * w[e] - xhat * mean) * inv * swish_slope(x[e], s);
+                }
+                store_vec(d_o + (row0 + r) * N + c, g);
             }
-        }
     }
-    if (dw_part != nullptr) {
+    if (dw_part != nullptr && own) {
 #pragma unroll
-        for (int j = 0; j < kMaxVecPerThread; ++j) {
-            const int c = threadIdx.x + j * 256;
-            if (c < nvec) {
-#pragma unroll
-                for (int e = 0; e < V; ++e) dw_part[(size_t)blockIdx.x * N + c * V + e] = dw[j][e];
-            }
-        }
+        for (int e = 0; e < V; e += 4)
+            *reinterpret_cast<float4*>(dw_part + (size_t)blockIdx.x * N + c + e) = make_float4(dw[e], dw[e + 1], dw[e + 2], dw[e + 3]);
     }
 }
-__global__ void out_norm_dw_kernel(const float* __restrict__ dw_part, float* __restrict__ dweight, int N, int nparts) {
+// 32 columns a CTA, the partial rows dealt out over 16 groups of threads, in a fixed order (a thread a column: 26 us for 500
+// partial rows of 2560, all of it latency)
+__global__ void __launch_bounds__(512) out_norm_dw_kernel(const float* __restrict__ dw_part, float* __restrict__ dweight, int N,
+                                                          int nparts) {
     follow_previous_grid();
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= N) return;
+    __shared__ double group[16][32];
+    const int c = blockIdx.x * 32 + threadIdx.x;
     double acc = 0.0;
-    for (int p = 0; p < nparts; ++p) acc += (double)dw_part[(size_t)p * N + c];
+    if (c < N) {
+#pragma unroll 8
+        for (int p = threadIdx.y; p < nparts; p += 16) acc += (double)dw_part[(size_t)p * N + c];
+    }
+    group[threadIdx.y][threadIdx.x] = acc;
+    __syncthreads();
+    if (threadIdx.y != 0 || c >= N) return;
+    for (int i = 1; i < 16; ++i) acc += group[i][threadIdx.x];
     dweight[c] = (float)acc;
 }
 
-unsigned stream_blocks(size_t nvec) {
-    const size_t want = (nvec + 255) / 256;
-    return (unsigned)(want < 148 * 16 ? (want ? want : 1) : 148 * 16);
+// threads of a CTA of the output path: one for each vector of a token
+unsigned token_threads(int N, int io) { return (unsigned)((N / (io == GSA_BF16 ? 8 : 4) + 31) / 32 * 32); }
+
+template <bool BWD>
+cudaError_t launch_swish(SwishSets sets, int io, cudaStream_t st) {
+    size_t most = 0;
+    for (SwishSet& t : sets.t) {
+        t.nvec /= io == GSA_BF16 ? 8 : 4;
+        if (t.nvec > most) most = t.nvec;
+    }
+    const dim3 grid((unsigned)((most + kStream * 256 - 1) / (kStream * 256)), 3);
+    if (io == GSA_BF16) launch_after(swish_kernel<__nv_bfloat16, BWD>, grid, 256, 0, st, sets);
+    else launch_after(swish_kernel<float, BWD>, grid, 256, 0, st, sets);
+    return cudaGetLastError();
 }
 
 }  // namespace
 
-// n elements (a multiple of the 16-byte vector) of io type
-cudaError_t launch_swish_fwd(const void* in, void* out, size_t n, int io, cudaStream_t st) {
-    if (io == GSA_BF16) {
-        const size_t nv = n / 8;
-        launch_after(swish_fwd_kernel<__nv_bfloat16>, stream_blocks(nv), 256, 0, st, (const __nv_bfloat16*)in, (__nv_bfloat16*)out, nv);
-    } else {
-        const size_t nv = n / 4;
-        launch_after(swish_fwd_kernel<float>, stream_blocks(nv), 256, 0, st, (const float*)in, (float*)out, nv);
-    }
-    return cudaGetLastError();
+// n elements (a multiple of the 16-byte vector) of io type each
+cudaError_t launch_swish_fwd(const void* const in[3], void* const out[3], const size_t n[3], int io, cudaStream_t st) {
+    return launch_swish<false>({{{in[0], out[0], n[0]}, {in[1], out[1], n[1]}, {in[2], out[2], n[2]}}}, io, st);
 }
-cudaError_t launch_swish_bwd(const void* x, void* d, size_t n, int io, cudaStream_t st) {
-    if (io == GSA_BF16) {
-        const size_t nv = n / 8;
-        launch_after(swish_bwd_kernel<__nv_bfloat16>, stream_blocks(nv), 256, 0, st, (const __nv_bfloat16*)x, (__nv_bfloat16*)d, nv);
-    } else {
-        const size_t nv = n / 4;
-        launch_after(swish_bwd_kernel<float>, stream_blocks(nv), 256, 0, st, (const float*)x, (float*)d, nv);
-    }
-    return cudaGetLastError();
+// d <- d * Swish'(x), in place on the gradients
+cudaError_t launch_swish_bwd(const void* const x[3], void* const d[3], const size_t n[3], int io, cudaStream_t st) {
+    return launch_swish<true>({{{x[0], d[0], n[0]}, {x[1], d[1], n[1]}, {x[2], d[2], n[2]}}}, io, st);
 }
-int out_norm_max_width(int io) { return 256 * kMaxVecPerThread * (io == GSA_BF16 ? 8 : 4); }
+int out_norm_max_width(int io) { return 512 * (io == GSA_BF16 ? 8 : 4); }
 size_t out_norm_bwd_parts(size_t rows) { return (rows + kRowsPerCta - 1) / kRowsPerCta; }
 cudaError_t launch_out_norm_fwd(const void* o, const float* weight, float eps, void* y, size_t rows, int N, int io,
                                 cudaStream_t st) {
-    if (io == GSA_BF16) launch_after(out_norm_fwd_kernel<__nv_bfloat16>, (unsigned)rows, 256, 0, st, (const __nv_bfloat16*)o, weight, eps, (__nv_bfloat16*)y, N);
-    else launch_after(out_norm_fwd_kernel<float>, (unsigned)rows, 256, 0, st, (const float*)o, weight, eps, (float*)y, N);
+    const unsigned ctas = (unsigned)((rows + kTokens - 1) / kTokens), threads = token_threads(N, io);
+    if (io == GSA_BF16)
+        launch_after(out_norm_fwd_kernel<__nv_bfloat16>, ctas, threads, 0, st, (const __nv_bfloat16*)o, weight, eps,
+                     (__nv_bfloat16*)y, N, rows);
+    else
+        launch_after(out_norm_fwd_kernel<float>, ctas, threads, 0, st, (const float*)o, weight, eps, (float*)y, N, rows);
     return cudaGetLastError();
 }
 cudaError_t launch_out_norm_bwd(const void* o, const void* dy, const float* weight, float eps, void* d_o, float* dw_part,
                                 float* dweight, size_t rows, int N, int io, cudaStream_t st) {
-    const unsigned parts = (unsigned)out_norm_bwd_parts(rows);
+    const unsigned parts = (unsigned)out_norm_bwd_parts(rows), threads = token_threads(N, io);
     if (io == GSA_BF16)
-        launch_after(out_norm_bwd_kernel<__nv_bfloat16>, parts, 256, 0, st, (const __nv_bfloat16*)o, (const __nv_bfloat16*)dy, weight, eps,
-                                                                (__nv_bfloat16*)d_o, dweight ? dw_part : nullptr, N, rows);
+        launch_after(out_norm_bwd_kernel<__nv_bfloat16>, parts, threads, 0, st, (const __nv_bfloat16*)o, (const __nv_bfloat16*)dy,
+                     weight, eps, (__nv_bfloat16*)d_o, dweight ? dw_part : nullptr, N, rows);
     else
-        launch_after(out_norm_bwd_kernel<float>, parts, 256, 0, st, (const float*)o, (const float*)dy, weight, eps, (float*)d_o,
-                                                        dweight ? dw_part : nullptr, N, rows);
-    if (dweight != nullptr) launch_after(out_norm_dw_kernel, (N + 255) / 256, 256, 0, st, dw_part, dweight, N, (int)parts);
+        launch_after(out_norm_bwd_kernel<float>, parts, threads, 0, st, (const float*)o, (const float*)dy, weight, eps, (float*)d_o,
+                     dweight ? dw_part : nullptr, N, rows);
+    if (dweight != nullptr) launch_after(out_norm_dw_kernel, (N + 31) / 32, dim3(32, 16), 0, st, dw_part, dweight, N, (int)parts);
     return cudaGetLastError();
 }
 

@@ -95,3 +95,31 @@ def test_output_norm_fwd_bwd(io, H, dv, T, with_weight):
     d2, dw2 = gsa.gsa_out_norm_bwd(p, od, dyd, wd, eps)
     torch.cuda.synchronize()
     assert torch.equal(d_o, d2) and torch.equal(dw, dw2)
+
+
+@pytest.mark.parametrize("io,H,dv,T", [("bf16", 1, 64, 1), ("f32", 3, 64, 7), ("bf16", 8, 512, 9), ("f32", 4, 512, 5), ("bf16", 7, 64, 17)])
+def test_output_norm_edges(io, H, dv, T):
+    # tokens that do not fill the four and sixteen of a CTA, rows from 8 vectors to the widest, a CTA of a partial last warp
+    test_output_norm_fwd_bwd(io, H, dv, T, True)
+
+
+@pytest.mark.parametrize("io,T,dk,dv", [("bf16", 1, 64, 512), ("f32", 33, 128, 64), ("bf16", 67, 256, 64)])
+def test_feature_map_of_unequal_widths(io, T, dk, dv):
+    # q, k and v share a launch: a short tensor beside a long one, sizes that do not fill the last block
+    B, H, m = 1, 1, 64
+    d = rand_inputs(5 + T, B, T, H, dk, dv, m, io)
+    q, k, v, dO = (to_dev(d[n], io) for n in ("q", "k", "v", "dO"))
+    p = gsa.Params(B, T, H, dk, dv, m, io=io, feature_map="swish")
+    pn = gsa.Params(B, T, H, dk, dv, m, io=io)
+    g = to_dev(d["gate"])
+    sq, sk, sv = (torch.nn.functional.silu(x.float()).to(x.dtype) for x in (q, k, v))
+    # the same kernels on features made by torch.  fp32: the two Swish differ by 2^-22 of the value, the gradients w.r.t. q
+    # and k are differences of terms that many times larger (dq ~ p (dp - <p, dp>)), at the worst of all elements by rms a
+    # hundredfold: 2.4e-5.  bf16: features and gradients are rounded to 8 bits on either side.
+    tol = 1e-4 if io == "f32" else 2e-2
+    assert rel_err(to_np(gsa.gsa_fwd(p, q, k, v, g)), to_np(gsa.gsa_fwd(pn, sq, sk, sv, g)), io == "bf16") <= tol
+    got = gsa.gsa_bwd(p, q, k, v, g, dO)
+    want = gsa.gsa_bwd(pn, sq, sk, sv, g, dO)
+    for x, a, b in zip((q, k, v), got[:3], want[:3]):
+        s = torch.sigmoid(x.double())
+        assert rel_err(to_np(a), to_np((b.double() * s * (1 + x.double() * (1 - s))).float()), io == "bf16") <= tol
