@@ -25,6 +25,7 @@ constexpr int kLd = 68;         // shared-memory pitch of a 64-wide fp32 tile (1
 template <int NJ>
 __device__ __forceinline__ void mm_nn(const float* A, int lda, const float* B, int ldb, int K,
                                       int ty, int tx, float (&acc)[4][NJ]) {
+#pragma unroll 2
     for (int k = 0; k < K; k += 4) {
         float a[4][4];
 #pragma unroll
@@ -82,6 +83,7 @@ __device__ __forceinline__ void mm_tn(const float* A, int lda, const float* B, i
 // NT: acc[ii][jj] += sum_k A[4 ty + ii][k] * B[tx + 16 jj][k]      (64 columns: jj < 4)
 __device__ __forceinline__ void mm_nt(const float* A, int lda, const float* B, int ldb, int K,
                                       int ty, int tx, float (&acc)[4][4]) {
+#pragma unroll 2
     for (int k = 0; k < K; k += 4) {
         float4 a[4], b[4];
 #pragma unroll
@@ -100,35 +102,53 @@ __device__ __forceinline__ void mm_nt(const float* A, int lda, const float* B, i
     }
 }
 
-// ---- tile loads: 64 rows x 64 columns of io type -> fp32 shared (rows >= valid are zero)
+// ---- tile loads.  fp32 tiles go to shared memory by asynchronous copies: all tiles of a chunk are requested before the
+// first is waited for (through registers a tile's copies waited for those of the tile before it: four to five latencies of
+// memory a chunk, a third of the kernels' stalls).  With the second scaling pass of a moderate chunk gone, too: a fp32
+// training step, B = 2, T = 1024, 4 heads of 256, 586 -> 439 us, a forward over T = 256 53 -> 41 us.
+__device__ __forceinline__ void copy16_async(float* dst, const float* src, bool live) {      // (!live: zeros)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+                 "r"(live ? 16 : 0)
+                 : "memory");
+}
+__device__ __forceinline__ void copies_landed() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// 64 rows x 64 columns of io type -> fp32 shared (rows >= valid are zero)
 template <typename IO>
 __device__ __forceinline__ void load_io_tile(float* dst, const IO* src, size_t row_stride, int valid) {
     constexpr int V = IoTraits<IO>::kVec;
     constexpr int PER_ROW = kDS / V;
-    for (int idx = threadIdx.x; idx < kC * PER_ROW; idx += 256) {
-        const int r = idx / PER_ROW, c = (idx % PER_ROW) * V;
-        float x[V];
-        if (r < valid) {
-            load_vec(src + (size_t)r * row_stride + c, x);
-        } else {
+    if constexpr (V == 4) {
 #pragma unroll
-            for (int e = 0; e < V; ++e) x[e] = 0.f;
+        for (int idx = threadIdx.x; idx < kC * PER_ROW; idx += 256) {
+            const int r = idx / PER_ROW, c = (idx % PER_ROW) * V;
+            copy16_async(dst + r * kLd + c, src + (size_t)min(r, valid - 1) * row_stride + c, r < valid);
         }
+    } else {
 #pragma unroll
-        for (int e = 0; e < V; e += 4)
-            *reinterpret_cast<float4*>(dst + r * kLd + c + e) = make_float4(x[e], x[e + 1], x[e + 2], x[e + 3]);
+        for (int idx = threadIdx.x; idx < kC * PER_ROW; idx += 256) {
+            const int r = idx / PER_ROW, c = (idx % PER_ROW) * V;
+            float x[V];
+            if (r < valid) {
+                load_vec(src + (size_t)r * row_stride + c, x);
+            } else {
+#pragma unroll
+                for (int e = 0; e < V; ++e) x[e] = 0.f;
+            }
+#pragma unroll
+            for (int e = 0; e < V; e += 4)
+                *reinterpret_cast<float4*>(dst + r * kLd + c + e) = make_float4(x[e], x[e + 1], x[e + 2], x[e + 3]);
+        }
     }
 }
 // 64 rows x M fp32; rows >= valid get `fill` (0 for weights) or replicate the last valid row (G)
 template <int M, bool REPLICATE_LAST>
 __device__ __forceinline__ void load_slot_tile(float* dst, const float* src, size_t row_stride, int valid) {
     constexpr int PER_ROW = M / 4;
+#pragma unroll
     for (int idx = threadIdx.x; idx < kC * PER_ROW; idx += 256) {
         const int r = idx / PER_ROW, c = (idx % PER_ROW) * 4;
-        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (r < valid) x = *reinterpret_cast<const float4*>(src + (size_t)r * row_stride + c);
-        else if (REPLICATE_LAST) x = *reinterpret_cast<const float4*>(src + (size_t)(valid - 1) * row_stride + c);
-        *reinterpret_cast<float4*>(dst + r * (M + 4) + c) = x;
+        copy16_async(dst + r * (M + 4) + c, src + (size_t)min(r, valid - 1) * row_stride + c, REPLICATE_LAST || r < valid);
     }
 }
 
@@ -146,7 +166,7 @@ __device__ __forceinline__ bool chunk_is_moderate(const float* sG, int* flag) {
 // FLAGGED: the flagged pairs of a tensor-core scan alone (see launch_value_side_simt); a CTA then takes both 64-wide
 // halves of a 128-wide slice, one after the other.
 template <typename IO, int M, bool REV, bool FLAGGED>
-__global__ void __launch_bounds__(256) value_side_simt_kernel(ValueSideArgs a, const int* __restrict__ strong_flag) {
+__global__ void __launch_bounds__(256, M > 64 ? 1 : 2) value_side_simt_kernel(ValueSideArgs a, const int* __restrict__ strong_flag) {
     follow_previous_grid();
     if (FLAGGED && strong_flag[blockIdx.x] == 0) return;
     constexpr int NJ = M / 16;
@@ -174,6 +194,7 @@ __global__ void __launch_bounds__(256) value_side_simt_kernel(ValueSideArgs a, c
     float* out = a.out + (size_t)slice * a.B * a.T * a.H * M + ((size_t)b * a.T * a.H + h) * M;
 
     // state slice S[c][s] <- S0[bh][s][d0 + c]
+#pragma unroll
     for (int idx = tid; idx < kDS * M; idx += 256) {
         const int s = idx / kDS, c = idx % kDS;
         sS[c * LM + s] = a.S0 ? a.S0[((size_t)bh * M + s) * a.D + d0 + c] : 0.f;
@@ -188,6 +209,7 @@ __global__ void __launch_bounds__(256) value_side_simt_kernel(ValueSideArgs a, c
         load_io_tile<IO>(sXk, xk + (size_t)t0 * strideD, strideD, valid);
         load_slot_tile<M, false>(sW, w + (size_t)t0 * strideM, strideM, valid);
         load_slot_tile<M, true>(sG, G + (size_t)t0 * strideM, strideM, valid);
+        copies_landed();
         __syncthreads();
         const bool moderate = chunk_is_moderate<M>(sG, &s_flag);
         if (moderate) {
@@ -270,27 +292,29 @@ __global__ void __launch_bounds__(256) value_side_simt_kernel(ValueSideArgs a, c
             }
         }
         __syncthreads();
-        // W~ for the state update: forward W exp(G_C - G), reverse W exp(G)
-        for (int idx = tid; idx < kC * M; idx += 256) {
-            const int r = idx / M, s = idx % M;
-            const float gc = sG[(kC - 1) * LM + s];
-            float f;
-            if (moderate) f = REV ? 1.f : __expf(gc);
-            else f = __expf(REV ? sG[r * LM + s] : gc - sG[r * LM + s]);
-            sW[r * LM + s] *= f;
+        // W~ for the state update: forward W exp(G_C - G), reverse W exp(G).  A moderate chunk's weights are W exp(-G) and
+        // W exp(G): the forward update takes its exp(G_C) with the state, S <- exp(G_C) (S + Xk^T W')
+        if (!moderate) {
+            for (int idx = tid; idx < kC * M; idx += 256) {
+                const int r = idx / M, s = idx % M;
+                sW[r * LM + s] *= __expf(REV ? sG[r * LM + s] : sG[(kC - 1) * LM + s] - sG[r * LM + s]);
+            }
+            __syncthreads();
         }
-        __syncthreads();
         // S <- S * exp(G_C) + Xk^T W~
         {
             float acc[4][NJ] = {};
             mm_tn<NJ>(sXk, kLd, sW, LM, kC, ty, tx, acc);
 #pragma unroll
-            for (int ii = 0; ii < 4; ++ii)
+            for (int jj = 0; jj < NJ; ++jj) {
+                const int s = NJ * tx + jj;
+                const float egc = __expf(sG[(kC - 1) * LM + s]);
 #pragma unroll
-                for (int jj = 0; jj < NJ; ++jj) {
-                    const int c = 4 * ty + ii, s = NJ * tx + jj;
-                    sS[c * LM + s] = fmaf(sS[c * LM + s], __expf(sG[(kC - 1) * LM + s]), acc[ii][jj]);
+                for (int ii = 0; ii < 4; ++ii) {
+                    float& S = sS[(4 * ty + ii) * LM + s];
+                    S = !REV && moderate ? (S + acc[ii][jj]) * egc : fmaf(S, egc, acc[ii][jj]);
                 }
+            }
         }
     }
     __syncthreads();
@@ -306,7 +330,7 @@ __global__ void __launch_bounds__(256) value_side_simt_kernel(ValueSideArgs a, c
 
 // =============================================================== key_side (pass-2 form)
 template <typename IO, int M, bool REV, bool FLAGGED>
-__global__ void __launch_bounds__(256) key_side_simt_kernel(KeySideArgs a, const int* __restrict__ strong_flag) {
+__global__ void __launch_bounds__(256, M > 64 ? 1 : 2) key_side_simt_kernel(KeySideArgs a, const int* __restrict__ strong_flag) {
     follow_previous_grid();
     if (FLAGGED && strong_flag[blockIdx.x] == 0) return;
     constexpr int LM = M + 4;
@@ -330,6 +354,7 @@ __global__ void __launch_bounds__(256) key_side_simt_kernel(KeySideArgs a, const
     const IO* xv = (const IO*)a.xv + ((size_t)b * a.T * a.H + h) * a.D + d0;
     IO* out = (IO*)a.out + ((size_t)b * a.T * a.H + h) * a.D + d0;
 
+#pragma unroll
     for (int idx = tid; idx < M * kDS; idx += 256) {
         const int s = idx / kDS, c = idx % kDS;
         sS[s * kLd + c] = a.S0 ? a.S0[((size_t)bh * M + s) * a.D + d0 + c] : 0.f;
@@ -344,6 +369,7 @@ __global__ void __launch_bounds__(256) key_side_simt_kernel(KeySideArgs a, const
         load_slot_tile<M, false>(sK, uk + (size_t)t0 * strideM, strideM, valid);
         load_slot_tile<M, true>(sG, G + (size_t)t0 * strideM, strideM, valid);
         load_io_tile<IO>(sV, xv + (size_t)t0 * strideD, strideD, valid);
+        copies_landed();
         __syncthreads();
         const bool moderate = chunk_is_moderate<M>(sG, &s_flag);
         // A_ij = sum_s uq_i[s] uk_j[s] exp(+-(G_i[s] - G_j[s])) on the kept triangle
@@ -395,21 +421,17 @@ __global__ void __launch_bounds__(256) key_side_simt_kernel(KeySideArgs a, const
         // bring uq, uk to the scalings of the state terms:
         //   forward: Q- = uq exp(G),        K- = uk exp(G_C - G)
         //   reverse: Q- = uq exp(G_C - G),  K- = uk exp(G)
-        for (int idx = tid; idx < kC * M; idx += 256) {
-            const int r = idx / M, s = idx % M;
-            const float g = sG[r * LM + s], gc = sG[(kC - 1) * LM + s];
-            float fq, fk;
-            if (moderate) {
-                fq = REV ? __expf(gc) : 1.f;
-                fk = REV ? 1.f : __expf(gc);
-            } else {
-                fq = __expf(REV ? gc - g : g);
-                fk = __expf(REV ? g : gc - g);
+        // (a moderate chunk has uq exp(G) and uk exp(-G), reversed uq exp(-G) and uk exp(G): forward, the state takes the
+        // exp(G_C) of its update, S <- exp(G_C) (S + K-^T Xv))
+        if (!moderate || REV) {
+            for (int idx = tid; idx < kC * M; idx += 256) {
+                const int r = idx / M, s = idx % M;
+                const float g = sG[r * LM + s], gc = sG[(kC - 1) * LM + s];
+                sQ[r * LM + s] *= __expf(REV ? (moderate ? gc : gc - g) : g);
+                if (!moderate) sK[r * LM + s] *= __expf(REV ? g : gc - g);
             }
-            sQ[r * LM + s] *= fq;
-            sK[r * LM + s] *= fk;
+            __syncthreads();
         }
-        __syncthreads();
         // out = Q- S + A Xv
         {
             float acc[4][4] = {};
@@ -433,8 +455,10 @@ __global__ void __launch_bounds__(256) key_side_simt_kernel(KeySideArgs a, const
                 const int s = s0 + 4 * ty + ii;
                 const float e = __expf(sG[(kC - 1) * LM + s]);
 #pragma unroll
-                for (int jj = 0; jj < 4; ++jj)
-                    sS[s * kLd + 4 * tx + jj] = fmaf(sS[s * kLd + 4 * tx + jj], e, acc[ii][jj]);
+                for (int jj = 0; jj < 4; ++jj) {
+                    float& S = sS[s * kLd + 4 * tx + jj];
+                    S = !REV && moderate ? (S + acc[ii][jj]) * e : fmaf(S, e, acc[ii][jj]);
+                }
             }
         }
     }
