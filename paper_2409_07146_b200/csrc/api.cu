@@ -300,15 +300,22 @@ PendingDecay pending_decay(const gsa_params_t& p, Segments segs, const Workspace
 // End memories (reverse: the gradients entering from the right) of every segment run from empty memories, K and V side.
 // Both primitives update their state alike, S <- decay (S + X^T W), so value_side's arguments serve both.
 struct StateSet { const void* x; const float* w; const void* wd; float* end; };
+// logdecay (nullable; forward runs): receives the segments' log-decay [B,nseg,H,m].
 cudaError_t state_scans(const gsa_params_t& p, Segments segs, StateSet ks, StateSet vs, const Workspace& w, int reverse,
-                        cudaStream_t st, int32_t* dev_status) {
+                        float* logdecay, cudaStream_t st, int32_t* dev_status) {
     ValueSideArgs a[2] = {{ks.x, ks.x, ks.w, w.G, nullptr, ks.end, nullptr, p.B, p.T, p.H, p.d_k, ks.wd, 1},
                           {vs.x, vs.x, vs.w, w.G, nullptr, vs.end, nullptr, p.B, p.T, p.H, p.d_v, vs.wd, 1}};
     for (ValueSideArgs& x : a) { x.nseg = segs.n; x.tseg = segs.t; x.E = w.E; }
-    if (use_wide(p)) return launch_state_scans_wide(a[0], a[1], reverse, w.strong, st, dev_status);
+    if (use_wide(p)) {
+        if (logdecay != nullptr) {
+            const cudaError_t e = launch_segment_logdecay(w.G, logdecay, p.B, p.T, p.H, p.m, segs.n, segs.t, log_gate_chunk(p), st);
+            if (e != cudaSuccess) return e;
+        }
+        return launch_state_scans_wide(a[0], a[1], reverse, w.strong, st, dev_status);
+    }
+    a[0].seg_logdecay = logdecay;
     if (use_tc(p)) return launch_state_scan_tc(a[0], a[1], reverse, w.strong, st, dev_status);
-    cudaError_t e = launch_value_side_simt(a[0], p.io, p.m, reverse, st);
-    return e == cudaSuccess ? launch_value_side_simt(a[1], p.io, p.m, reverse, st) : e;
+    return launch_state_scan_simt(a[0], a[1], p.io, p.m, reverse, st);
 }
 
 // ---- optional per-kernel timing (benchmarks only): while a sink is active on the calling
@@ -584,10 +591,8 @@ gsa_status_t fwd_core(const CallParams* params, int m_active, const void* q, con
     if (nseg > 1) {
         // first pass: every segment from empty memories, for its end memories alone; then the start
         // memories of all segments, and the final memories, by a scan over the segments
-        GSA_LAUNCH("segment_logdecay", launch_segment_logdecay(w.G, w.seg_decay, p.B, p.T, p.H, p.m, nseg,
-                                                               tseg, log_gate_chunk(p), st));
         GSA_LAUNCH("segment_states", state_scans(p, segs, StateSet{k, w.I, w.Id, w.Kloc}, StateSet{v, w.I, w.Id, w.Vloc}, w, 0,
-                                                  st, dev_status));
+                                                  w.seg_decay, st, dev_status));
         // (when the backward is to reuse them, the final memories land in the saved block first)
         float* KTc = save_gate ? w.KT : KT;
         float* VTc = save_gate ? w.VT : VT;
@@ -765,10 +770,8 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
         Kin = w.Kstart; Vin = w.Vstart;
         KTout = nullptr; VTout = nullptr;
     } else if (nseg > 1) {
-        GSA_LAUNCH("segment_logdecay", launch_segment_logdecay(w.G, w.seg_decay, p.B, p.T, p.H, p.m, nseg,
-                                                               tseg, log_gate_chunk(p), st));
         GSA_LAUNCH("segment_states", state_scans(p, segs, StateSet{k, w.I, w.Id, w.Kloc}, StateSet{v, w.I, w.Id, w.Vloc}, w, 0,
-                                                  st, dev_status));
+                                                  w.seg_decay, st, dev_status));
         GSA_LAUNCH("segment_combine", launch_segment_combine(w.seg_decay, {w.Kloc, K0, w.Kstart, KTout, p.d_k}, {w.Vloc, V0, w.Vstart, VTout, p.d_v}, p.B,
                                                              p.H, p.m, nseg, 0, st));
         Kin = w.Kstart; Vin = w.Vstart;
@@ -856,7 +859,7 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
         // reversed scans of every segment from empty states, for their end states alone; then the states
         // entering every segment, and dK0 / dV0, by a scan over the segments from the last one down
         GSA_LAUNCH("segment_rev_states", state_scans(p, segs, StateSet{q, w.dz, w.Zd, w.Kloc}, StateSet{dO, w.p, w.Pd, w.Vloc}, w,
-                                                      1, st, dev_status));
+                                                      1, nullptr, st, dev_status));
         GSA_LAUNCH("segment_combine", launch_segment_combine(w.seg_decay, {w.Kloc, dKT, w.dKend, dK0, p.d_k}, {w.Vloc, dVT, w.dVend, dV0, p.d_v}, p.B,
                                                              p.H, p.m, nseg, 1, st));
         dKin = w.dKend; dVin = w.dVend;
@@ -1054,8 +1057,7 @@ gsa_status_t gsa_shard_states(const gsa_params_t* params, const void* k, const v
     // one "segment" per batch element: the whole shard from empty memories, end memories only
     GSA_CUDA(cudaMemsetAsync(w.strong, 0, sizeof(int) * (size_t)p.B * p.H, st));
     GSA_LAUNCH("gate_cumsum", gate_products(p, Segments{1, p.T}, gate, w, st));
-    GSA_LAUNCH("segment_logdecay", launch_segment_logdecay(w.G, logdecay, p.B, p.T, p.H, p.m, 1, p.T, log_gate_chunk(p), st));
-    GSA_LAUNCH("segment_states", state_scans(p, Segments{1, p.T}, StateSet{k, w.I, w.Id, KT}, StateSet{v, w.I, w.Id, VT}, w, 0, st,
+    GSA_LAUNCH("segment_states", state_scans(p, Segments{1, p.T}, StateSet{k, w.I, w.Id, KT}, StateSet{v, w.I, w.Id, VT}, w, 0, logdecay, st,
                                               dev_status));
     return GSA_OK;
 }

@@ -675,7 +675,15 @@ state_scan_kernel(const __grid_constant__ CUtensorMap mapX0, const __grid_consta
     const CUtensorMap &mapX = second ? mapX1 : mapX0, &mapW = second ? mapW1 : mapW0;
     const ValueSideArgs& a = sets.set[second];
     const int slice = second ? blockIdx.y - sets.slices0 : blockIdx.y;
+    float* seg_logdecay = slice == 0 && !REV ? a.seg_logdecay : nullptr;
     if (strong_flag[blockIdx.x] != 0) {
+        if (seg_logdecay != nullptr && threadIdx.x < kM) {
+            const ScanSpan span = scan_span(blockIdx.x, a.H, a.T, a.nseg, a.tseg);
+            double sum = 0.0;
+            for (int t = span.t0; t < span.t_end; t += kCT)
+                sum += (double)a.G[(((size_t)span.b * a.T + min(t + kCT, span.t_end) - 1) * a.H + span.h) * kM + threadIdx.x];
+            seg_logdecay[(size_t)blockIdx.x * kM + threadIdx.x] = (float)sum;
+        }
         value_side_general<REV>(mapX, mapX, second ? mapW32_1 : mapW32_0, mapG32, mapG32, a, dev_status, slice);
         return;
     }
@@ -767,8 +775,11 @@ state_scan_kernel(const __grid_constant__ CUtensorMap mapX0, const __grid_consta
             return G[(((size_t)b * T + last) * H + h) * kM + tid];
         };
         float g_next = 0.f;
+        double decay = 0.0;                // the segment's log-decay
         if (tid < kM) {
-            ctl->egc[0][tid] = __expf(chunk_gc(0));
+            const float g = chunk_gc(0);
+            decay = (double)g;
+            ctl->egc[0][tid] = __expf(g);
             if (nchunks > 1) g_next = chunk_gc(1);
         }
         compute_sync();
@@ -776,6 +787,7 @@ state_scan_kernel(const __grid_constant__ CUtensorMap mapX0, const __grid_consta
             const float* egc = ctl->egc[n & 1];
             if (tid < kM && n + 1 < nchunks) {
                 ctl->egc[(n + 1) & 1][tid] = __expf(g_next);
+                decay += (double)g_next;
                 if (n + 2 < nchunks) g_next = chunk_gc(n + 2);
             }
             LEAN_WAIT(&ctl->bar_u[n & 1], (n >> 1) & 1);
@@ -802,6 +814,7 @@ state_scan_kernel(const __grid_constant__ CUtensorMap mapX0, const __grid_consta
 #pragma unroll
             for (int s = 0; s < kHS; ++s) a.Send[((size_t)bh * kM + sb + s) * D + d0 + row] = S[s];
         }
+        if (seg_logdecay != nullptr && tid < kM) seg_logdecay[(size_t)bh * kM + tid] = (float)decay;
     }
     lean_finish(ctl, tid, warp, tmem, dev_status);
 }

@@ -119,6 +119,7 @@ struct ValueSideArgs {
     // strong-decay flags are then [B, nseg, H, ..]
     int nseg = 1, tseg = 0;
     const float* E = nullptr;         // kernels for 128 slots: exp(G), see launch_gate_cumsum_wide
+    float* seg_logdecay = nullptr;    // state runs, forward, K side: receives the segments' log-decay (launch_segment_logdecay)
 };
 struct KeySideArgs {
     const float* uq; const float* uk; const float* G;
@@ -227,7 +228,8 @@ cudaError_t launch_column_sum(const float* in, float* part, float* out, size_t r
 // n bfloat16 values -> fp32 (a gate tensor given in bfloat16)
 cudaError_t launch_widen_bf16(const void* in, float* out, size_t n, cudaStream_t st);
 // Segment-parallel scheduling (T cut into nseg segments run as independent sequences): per-segment
-// log-decay [B,nseg,H,M] from G, and the start memories [B,nseg,H,M,D] of every segment from the
+// log-decay [B,nseg,H,M] from G (128 slots on the tensor cores; the other state runs leave it themselves, which spares
+// every segmented call a launch), and the start memories [B,nseg,H,M,D] of every segment from the
 // end memories of the segments run from empty memories.
 cudaError_t launch_segment_logdecay(const float* G, float* seg_logdecay, int B, int T, int H, int M, int nseg,
                                     int tseg, int chunk, cudaStream_t st);
@@ -264,6 +266,8 @@ int gate_grad_blocks(int T);       // entries per (b,h,slot) of launch_gate_grad
 // slices to their 128-wide ones, which those have zeroed
 cudaError_t launch_value_side_simt(const ValueSideArgs& a, int io, int M, int reverse,
                                    cudaStream_t st, const int* strong_flag = nullptr);
+// state runs (end memories only, from empty ones) of the K and the V side in one launch; k also takes seg_logdecay
+cudaError_t launch_state_scan_simt(const ValueSideArgs& k, const ValueSideArgs& v, int io, int M, int reverse, cudaStream_t st);
 cudaError_t launch_key_side_simt(const KeySideArgs& a, int io, int M, int reverse,
                                  cudaStream_t st, const int* strong_flag = nullptr);
 // tcgen05 (bf16 tensor-core) versions of the two primitives; bf16 io only.
