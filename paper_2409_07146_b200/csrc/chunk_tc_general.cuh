@@ -112,9 +112,8 @@ __device__ __forceinline__ void ctl_init(Ctl* ctl, int tid, int warp) {
 // The per-step gates a_j = exp(G_j - G_{j-1}) are formed once per chunk, in place of the G tile.
 constexpr float kDecayFloor = 9.094947e-13f;      // 2^-40
 
-// Replace the G tile by the per-step gates (rows past the end: 1).  gi receives this thread's own
-// G row (slots sb .. sb+31) first.  Two compute-thread barriers inside.
-__device__ __forceinline__ void gates_in_place(unsigned char* gt, int row, int half, int sb, int valid, float (&gi)[kHS]) {
+// Replace the G tile by the per-step gates (rows past the end: 1).  Two compute-thread barriers inside.
+__device__ __forceinline__ void gates_in_place(unsigned char* gt, int row, int half, int sb, int valid) {
     const int grow = min(row, valid - 1);
     float aj[kHS];
 #pragma unroll
@@ -124,7 +123,6 @@ __device__ __forceinline__ void gates_in_place(unsigned char* gt, int row, int h
         if (row > 0 && row < valid) tile_row8(gt, row - 1, sb + 8 * c, gp);
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-            gi[8 * c + e] = g[e];
             aj[8 * c + e] = row >= valid ? 1.f : __expf(row > 0 ? g[e] - gp[e] : g[e]);
         }
     }
@@ -136,75 +134,104 @@ __device__ __forceinline__ void gates_in_place(unsigned char* gt, int row, int h
     compute_sync();
 }
 
-// 16 consecutive fp32 values (s0 % 16 == 0) of row `row` of a slot-sized fp32 tile
-__device__ __forceinline__ void tile_row16(const unsigned char* tile, int row, int s0, float (&x)[16]) {
-    const unsigned char* panel = tile + (s0 >> 5) * kPanelB;
-    const int c = (s0 & 31) >> 2;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const float4 t = *reinterpret_cast<const float4*>(panel + swz128(row, c + q));
-        x[4 * q] = t.x; x[4 * q + 1] = t.y; x[4 * q + 2] = t.z; x[4 * q + 3] = t.w;
-    }
+// The walks go by distance: at step d every row i of the chunk is at j = i - d (time-reversed: i + d), so that all lanes of a
+// warp are at work until their products have died out.  (By absolute columns, as the accumulator is read, a warp repeats
+// the walk for the different rows of its lanes, a third of them live at a time.  32 K tokens, 16 heads of 128, gates that forget
+// within a dozen tokens: value_side 615 -> 488 us, key_side 678 -> 408.  What is left is the shared memory's rate: two rows of
+// 64 slots a step for each of 128 rows, 8 k cycles a chunk at a dozen steps, beside 8 k of the scan around it.)  The
+// accumulator's columns are turned into distances through a band in shared memory, kBand distances at a time, stored
+// [distance][row]: the chunk's 128 rows are then 128 consecutive words.
+constexpr int kBand = 32;
+static_assert(kBand * kCT * 4 == kPanelB, "a band is one operand panel");
+
+// Which 32 accumulator columns of the warp's rows the threads of `half` turn into distances of band k: a row's band lies in
+// two adjacent blocks of 32 columns.  (-1: outside the chunk)
+template <bool REV> __device__ __forceinline__ int band_block(int wq, int half, int k) {
+    const int blk = REV ? wq + k + half : wq - k - half;
+    return blk >= 0 && blk < kCT / 32 ? blk : -1;
 }
+// The gate between j and the next row of the walk: prod_{r=j+1..i} becomes prod_{r=j..i}, reversed prod_{r=i+1..j}
+// prod_{r=i+1..j+1}.
+template <bool REV> __device__ __forceinline__ int next_gate_row(int j) { return REV ? min(j + 1, kCT - 1) : j; }
+template <bool REV> __device__ __forceinline__ int distance(int row, int j) { return REV ? j - row : row - j; }
 
 // Strong-decay chunk of value_side: this thread's 32 output slots of row `row`,
 //   out[s] = exp(+-..) * inter[s] + sum_j P_ij w_j[s] prod a_r[s]   (j <= i forward, j >= i reverse),
 // P and the inter-chunk product are read from the accumulators; the row goes straight to global
-// memory.  `gt` holds the per-step gates (gates_in_place), gi this thread's G row.
+// memory.  `gt` holds the per-step gates (gates_in_place), g_row this row's G; `band`: a panel nobody else uses.  Sixteen slots
+// at a time: with 32 at a time the scan around the walk spills, and every chunk of a flagged pair pays for it (the state
+// runs of 32 K tokens of strong gates 222 -> 277 us).
 template <bool REV>
-__device__ __forceinline__ void value_side_explicit_rows(const unsigned char* gt, const unsigned char* sW,
-                                                      const float* gc, const float (&gi)[kHS], uint32_t tmem, int wq,
-                                                      int row, int sb, int valid, float* out_row) {
-    // the accumulator loads are warp-collective: the 16-column segments are those of the whole warp,
-    // walked away from the diagonal
-    const int first = REV ? wq * 32 : wq * 32 + 16, last = REV ? kCT - 16 : 0, step = REV ? 16 : -16;
+__device__ __forceinline__ void value_side_explicit_rows(const unsigned char* gt, const unsigned char* sW, float* band,
+                                                      const float* gc, const float* g_row, uint32_t tmem, int wq,
+                                                      int row, int half, int sb, int valid, float* out_row) {
+    const unsigned char* ga = gt + half * kPanelB;           // this thread's 32 slots of the gates and of the weights
+    const unsigned char* wa = sW + half * kPanelB;
 #pragma unroll 1
-    for (int s0 = sb; s0 < sb + kHS; s0 += 16) {
+    for (int c0 = 0; c0 < kHS / 4; c0 += 4) {
         float acc[16], dec[16];
 #pragma unroll
         for (int e = 0; e < 16; ++e) { acc[e] = 0.f; dec[e] = 1.f; }
-        bool live = true;
+        bool live = row < valid;
 #pragma unroll 1
-        for (int c0 = first; REV ? c0 <= last : c0 >= last; c0 += step) {
-            float v[16];
-            tmem_ld16(tmem_row_addr(tmem, wq, kColP + c0), v);
-            if (live) {
+        for (int k = 0; k < kCT / kBand; ++k) {
+            const int blk = band_block<REV>(wq, half, k);
+            if (blk >= 0) {
 #pragma unroll
-                for (int ee = 0; ee < 16; ++ee) {
-                    const int e = REV ? ee : 15 - ee;
-                    const int j = c0 + e;
-                    if ((REV ? j < row : j > row) || !live) continue;
-                    float aj[16], wj[16];
-                    tile_row16(gt, j, s0, aj);
-                    tile_row16(sW, j, s0, wj);
+                for (int q = 0; q < 32; q += 16) {
+                    float v[16];
+                    tmem_ld16(tmem_row_addr(tmem, wq, kColP + 32 * blk + q), v);
 #pragma unroll
-                    for (int u = 0; u < 16; ++u) {
-                        if (REV && j > row) dec[u] *= aj[u];            // prod_{r=i+1..j}
-                        acc[u] = fmaf(v[e] * wj[u], dec[u], acc[u]);
-                        if (!REV) dec[u] *= aj[u];                      // prod_{r=j..i} for the next (earlier) row
-                    }
-                    if ((ee & 3) == 3) {
-                        float top = 0.f;
-#pragma unroll
-                        for (int u = 0; u < 16; ++u) top = fmaxf(top, dec[u]);
-                        live = top >= kDecayFloor;
+                    for (int e = 0; e < 16; ++e) {
+                        const int d = distance<REV>(row, 32 * blk + q + e) - kBand * k;
+                        if (d >= 0 && d < kBand) band[d * kCT + row] = v[e];
                     }
                 }
             }
-            if (!__any_sync(0xffffffffu, live)) break;
+            compute_sync();
+#pragma unroll 1
+            for (int d0 = 0; d0 < kBand; d0 += 4) {
+                if (!__any_sync(0xffffffffu, live)) break;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int d = kBand * k + d0 + u, j = REV ? row + d : row - d;
+                    live = live && (REV ? j < valid : j >= 0);
+                    if (!live) continue;
+                    const float p = band[(d0 + u) * kCT + row];
+                    const int jg = next_gate_row<REV>(j);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        const float4 a4 = *reinterpret_cast<const float4*>(ga + swz128(jg, c0 + c));
+                        const float4 w4 = *reinterpret_cast<const float4*>(wa + swz128(j, c0 + c));
+                        const float aj[4] = {a4.x, a4.y, a4.z, a4.w}, wj[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            float& x = dec[4 * c + e];
+                            acc[4 * c + e] = fmaf(p * wj[e], x, acc[4 * c + e]);
+                            x *= aj[e];
+                        }
+                    }
+                }
+                float top = 0.f;
+#pragma unroll
+                for (int e = 0; e < 16; ++e) top = fmaxf(top, dec[e]);
+                live = live && top >= kDecayFloor;
+            }
+            if (!compute_sync_or(live)) break;       // (the barrier also covers: the band may be written again)
         }
         float vi[16], vj[16];
+        const int s0 = sb + 4 * c0;
         tmem_ld16(tmem_row_addr(tmem, wq, kColO + s0), vi);
         tmem_ld16(tmem_row_addr(tmem, wq, kColO + kM + s0), vj);       // (the state copy is a high/low pair)
-#pragma unroll
-        for (int e = 0; e < 16; ++e) vi[e] += vj[e];
         if (row < valid) {
 #pragma unroll
             for (int e = 0; e < 16; e += 4) {
+                const float4 g4 = *reinterpret_cast<const float4*>(g_row + s0 + e);
+                const float g[4] = {g4.x, g4.y, g4.z, g4.w};
                 float r[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
-                    r[u] = fmaf(vi[e + u], __expf(REV ? gc[s0 + e + u] - gi[s0 - sb + e + u] : gi[s0 - sb + e + u]), acc[e + u]);
+                    r[u] = fmaf(vi[e + u] + vj[e + u], __expf(REV ? gc[s0 + e + u] - g[u] : g[u]), acc[e + u]);
                 *reinterpret_cast<float4*>(out_row + s0 + e) = make_float4(r[0], r[1], r[2], r[3]);
             }
         }
@@ -216,7 +243,8 @@ __device__ __forceinline__ void value_side_explicit_rows(const unsigned char* gt
 // ======================================================================================
 // LAST = false: another scan of this CTA follows, which takes over the tensor memory.  Returns whether all went well
 // (the same for every thread); otherwise the tensor memory is freed and nothing may follow.
-template <bool REV, bool LAST = true>
+// STATES: end memories only; of a chunk's products the state's alone is formed.
+template <bool REV, bool LAST = true, bool STATES = false>
 __device__ __noinline__ bool value_side_general(const CUtensorMap& mapQ, const CUtensorMap& mapK,
                        const CUtensorMap& mapW, const CUtensorMap& mapG,
                        const CUtensorMap& mapO, const ValueSideArgs& args,
@@ -256,9 +284,11 @@ __device__ __noinline__ bool value_side_general(const CUtensorMap& mapQ, const C
         if (elect_one()) {
             auto load_x = [&](int it) {
                 const int t = chunk_t0(it);
-                mbar_expect_tx(&ctl->bar_x, 4 * kPanelB);
-                tma_load_4d(sXq, &mapQ, &ctl->bar_x, d0, h, t, b);
-                tma_load_4d(sXq + kPanelB, &mapQ, &ctl->bar_x, d0 + 64, h, t, b);
+                mbar_expect_tx(&ctl->bar_x, (STATES ? 2 : 4) * kPanelB);
+                if (!STATES) {
+                    tma_load_4d(sXq, &mapQ, &ctl->bar_x, d0, h, t, b);
+                    tma_load_4d(sXq + kPanelB, &mapQ, &ctl->bar_x, d0 + 64, h, t, b);
+                }
                 tma_load_4d(sXk, &mapK, &ctl->bar_x, d0, h, t, b);
                 tma_load_4d(sXk + kPanelB, &mapK, &ctl->bar_x, d0 + 64, h, t, b);
             };
@@ -302,17 +332,21 @@ __device__ __noinline__ bool value_side_general(const CUtensorMap& mapQ, const C
                 WAIT_OR_ABORT(&ctl->bar_x, it & 1);
                 tc_fence_after_sync();
                 PROF_MARK();
+                if (!STATES) {
 #pragma unroll
-                for (int kk = 0; kk < kDST / 16; ++kk)
-                    mma_bf16(tmem + kColP, desc_advance(dQk, kmaj(kk)), desc_advance(dKk, kmaj(kk)), idescP, kk > 0);
-                mma_commit(&ctl->bar_p);
+                    for (int kk = 0; kk < kDST / 16; ++kk)
+                        mma_bf16(tmem + kColP, desc_advance(dQk, kmaj(kk)), desc_advance(dKk, kmaj(kk)), idescP, kk > 0);
+                    mma_commit(&ctl->bar_p);
+                }
                 // so does the inter-chunk product O = xq S: the state copy was written at the end
                 // of the previous chunk
                 WAIT_OR_ABORT(&ctl->bar_sb, it & 1);
                 tc_fence_after_sync();
+                if (!STATES) {
 #pragma unroll
-                for (int kk = 0; kk < kDST / 16; ++kk)
-                    mma_bf16(tmem + kColO, desc_advance(dQk, kmaj(kk)), desc_advance(dS, mnmaj(kk)), idescO, kk > 0);
+                    for (int kk = 0; kk < kDST / 16; ++kk)
+                        mma_bf16(tmem + kColO, desc_advance(dQk, kmaj(kk)), desc_advance(dS, mnmaj(kk)), idescO, kk > 0);
+                }
                 PROF_MARK();
                 if (it + 1 < nchunks) {
                     bulk_wait_read();     // the output rows staged in that G buffer one chunk ago have left
@@ -323,7 +357,7 @@ __device__ __noinline__ bool value_side_general(const CUtensorMap& mapQ, const C
                 WAIT_OR_ABORT(&ctl->bar_ops, it & 1);
                 tc_fence_after_sync();
                 PROF_MARK();
-                const bool moderate = ctl->moderate[it & 1] != 0;
+                const bool moderate = !STATES && ctl->moderate[it & 1] != 0;       // (... has an intra-chunk product)
 #pragma unroll
                 for (int kk = 0; kk < kCT / 16; ++kk)
                     mma_bf16(tmem + kColU, desc_advance(dKm, mnmaj(kk)), desc_advance(dWa, mnmaj(kk)), idescU, kk > 0);
@@ -359,7 +393,7 @@ __device__ __noinline__ bool value_side_general(const CUtensorMap& mapQ, const C
                 PROF_MARK();
                 PROF_DUMP("value_side issue");
                 if (ctl->abort) break;
-                if (moderate && !a.state_only) {
+                if (moderate) {
                     tma_store_5d(&mapO, gt, 0, h, t0, b, slice);
                     tma_store_5d(&mapO, gt + kPanelB, 32, h, t0, b, slice);
                     bulk_commit();
@@ -425,10 +459,13 @@ __device__ __noinline__ bool value_side_general(const CUtensorMap& mapQ, const C
             if (tid == 0) mbar_arrive(&ctl->bar_ops);
             PROF_MARK();
 
-            WAIT_OR_ABORT(&ctl->bar_p, it & 1);
-            tc_fence_after_sync();
+            if (!STATES) {
+                WAIT_OR_ABORT(&ctl->bar_p, it & 1);
+                tc_fence_after_sync();
+            }
             PROF_MARK();
-            if (moderate) {
+            if (STATES) {
+            } else if (moderate) {
                 mask_row_in_tmem<REV, true>(tmem, wq, row, half, kColP);
                 tc_fence_before_sync();
                 compute_sync();
@@ -437,10 +474,11 @@ __device__ __noinline__ bool value_side_general(const CUtensorMap& mapQ, const C
                 // strong decay: the intra-chunk term by the walk over the per-step gates
                 WAIT_OR_ABORT(&ctl->bar_mma1, it & 1);    // the inter-chunk product
                 tc_fence_after_sync();
-                if (!a.state_only) {
-                    float gi[kHS];
-                    gates_in_place(const_cast<unsigned char*>(gt), row, half, sb, valid, gi);
-                    value_side_explicit_rows<REV>(gt, sW, ctl->gc, gi, tmem, wq, row, sb, valid,
+                {
+                    gates_in_place(const_cast<unsigned char*>(gt), row, half, sb, valid);
+                    // (the band: the weights' operand rows, which the state product, complete, was the last to read)
+                    value_side_explicit_rows<REV>(gt, sW, reinterpret_cast<float*>(sWa), ctl->gc,
+                                                  a.G + (((size_t)b * a.T + t0 + row) * a.H + h) * kM, tmem, wq, row, half, sb, valid,
                                                   obase + (size_t)(t0 + row) * strideM);
                 }
             }
@@ -467,11 +505,11 @@ __device__ __noinline__ bool value_side_general(const CUtensorMap& mapQ, const C
             }
             // its bf16 copy feeds the next chunk's inter-chunk product (issued as soon as the next
             // tiles are there); the product of this chunk that read the old copy is complete
-            store_state_row_split<false>(sSb, sSb + kPanelB, row, sb, S, nullptr);
+            if (!STATES) store_state_row_split<false>(sSb, sSb + kPanelB, row, sb, S, nullptr);
 
             // ---- output rows of a moderate chunk: exp(+-G_i) * (inter + intra)
             PROF_MARK();
-            if (moderate) {
+            if (!STATES && moderate) {
                 WAIT_OR_ABORT(&ctl->bar_mma2, n_mod & 1);
                 ++n_mod;
                 tc_fence_after_sync();
@@ -538,86 +576,96 @@ __device__ __noinline__ bool value_side_general(const CUtensorMap& mapQ, const C
 }
 
 // Strong-decay chunk of key_side: A_ij = sum_s uq_i[s] uk_j[s] prod a_r[s] on the kept triangle, by
-// the same walk: the thread carries uq_i[s] times the running decay product for its 64 slots, one
-// multiplication per step and slot, and stops once every product is below 2^-40.  Written into tensor
-// memory as the bf16 high/low operand rows of the masked matrix, in the layout mask_row_in_tmem leaves
-// (this thread's 64 columns: 32 packed high parts, then 32 packed residuals).  `sG` is replaced by the
-// per-step gates on the way.
+// the same walk: the thread carries uq_i[s] times the running decay product for its 32 slots, one
+// multiplication per step and slot, and stops once every product is below 2^-40 of the largest it began with.  The two
+// threads of a row meet in two bands (over the uq rows, which are in registers by then); the sums go to the
+// accumulator's fp32 columns and from there, like those of a moderate chunk, into the masked bf16 operand rows.
+// `sG` is replaced by the per-step gates on the way.
 template <bool REV>
-__device__ __forceinline__ void key_side_explicit_rows(unsigned char* sG, const unsigned char* sUq,
+__device__ __forceinline__ void key_side_explicit_rows(unsigned char* sG, unsigned char* sUq,
                                                     const unsigned char* sUk, uint32_t tmem, int wq, int row, int half,
-                                                    int sb, int grow, int valid) {
-    // thread (row, half) fills columns j in [64 half, 64 half + 63]; its walk starts at the column nearest to
-    // the diagonal: j0 = min(row, 64 half + 63) forward, max(row, 64 half) reverse
-    const int jlo = 64 * half, jhi = jlo + 63;
-    const bool any = REV ? row <= jhi : row >= jlo;
-    const int j0 = REV ? max(row, jlo) : min(row, jhi);
-    float qd[kM];
+                                                    int sb, int valid) {
+    float qd[kHS];
+#pragma unroll
+    for (int s0 = 0; s0 < kHS; s0 += 8) {
+        float uq[8];
+        tile_row8(sUq, row, sb + s0, uq);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) qd[s0 + e] = uq[e];
+    }
+    gates_in_place(sG, row, half, sb, valid);       // (its barriers also cover: every uq row is in registers)
     {
-        // uq_i[s] exp(G_i[s] - G_j0[s]) (reverse: G_j0 - G_i): the product of the gates between the row and the
-        // start of the walk, 64 exponentials once (zero exponent when the walk starts on the diagonal)
-        const int g0 = min(j0, valid - 1);
+        uint32_t zero[16];
 #pragma unroll
-        for (int s0 = 0; s0 < kM; s0 += 8) {
-            float g[8], gj[8], uq[8];
-            tile_row8(sG, grow, s0, g);
-            tile_row8(sG, g0, s0, gj);
-            tile_row8(sUq, row, s0, uq);
+        for (int e = 0; e < 16; ++e) zero[e] = 0u;
 #pragma unroll
-            for (int e = 0; e < 8; ++e) qd[s0 + e] = uq[e] * __expf(fminf(REV ? gj[e] - g[e] : g[e] - gj[e], 0.f));
-        }
+        for (int q = 0; q < 4; ++q) tmem_st16(tmem_row_addr(tmem, wq, kColP + 64 * half + 16 * q), zero);
+        tmem_st_wait();
+        tc_fence_before_sync();
     }
-    float gi[kHS];
-    gates_in_place(sG, row, half, sb, valid, gi);       // (its barriers also cover: every uq row is in registers)
-    (void)gi;
-    float x[64];
+    float* band = reinterpret_cast<float*>(sUq + half * kPanelB);
+    const float *band0 = reinterpret_cast<const float*>(sUq), *band1 = reinterpret_cast<const float*>(sUq + kPanelB);
+    const unsigned char* ga = sG + half * kPanelB;
+    const unsigned char* ka = sUk + half * kPanelB;
+    float start = 0.f;
 #pragma unroll
-    for (int e = 0; e < 64; ++e) x[e] = 0.f;
-    if (any) {
-        float start = 0.f;
-#pragma unroll
-        for (int s = 0; s < kM; ++s) start = fmaxf(start, fabsf(qd[s]));
-        const float floor_ = start * kDecayFloor;
+    for (int e = 0; e < kHS; ++e) start = fmaxf(start, fabsf(qd[e]));
+    const float floor_ = start * kDecayFloor;
+    bool live = start > 0.f;
 #pragma unroll 1
-        for (int j = j0; REV ? j <= jhi : j >= jlo; j += REV ? 1 : -1) {
-            // reverse: the product up to column j includes a_j (prod_{r=i+1..j}); j0 itself is already covered
-            float acc = 0.f;
+    for (int k = 0; k < kCT / kBand; ++k) {
+#pragma unroll 1
+        for (int d0 = 0; d0 < kBand; d0 += 4) {
 #pragma unroll
-            for (int s0 = 0; s0 < kM; s0 += 16) {
-                float aj[16], uk[16];
-                tile_row16(sG, j, s0, aj);
-                tile_row16(sUk, j, s0, uk);
+            for (int u = 0; u < 4; ++u) {
+                const int d = kBand * k + d0 + u, j = REV ? row + d : row - d;
+                live = live && (REV ? j < valid : j >= 0);
+                float sum[4] = {0.f, 0.f, 0.f, 0.f};
+                if (live) {
+                    const int jg = next_gate_row<REV>(j);
 #pragma unroll
-                for (int u = 0; u < 16; ++u) {
-                    if (REV && j > j0) qd[s0 + u] *= aj[u];
-                    acc = fmaf(qd[s0 + u], uk[u], acc);
-                    if (!REV) qd[s0 + u] *= aj[u];
+                    for (int c = 0; c < kHS / 4; ++c) {
+                        const float4 a4 = *reinterpret_cast<const float4*>(ga + swz128(jg, c));
+                        const float4 k4 = *reinterpret_cast<const float4*>(ka + swz128(j, c));
+                        const float aj[4] = {a4.x, a4.y, a4.z, a4.w}, uk[4] = {k4.x, k4.y, k4.z, k4.w};
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            float& x = qd[4 * c + e];
+                            sum[e] = fmaf(x, uk[e], sum[e]);
+                            x *= aj[e];
+                        }
+                    }
                 }
+                band[(d0 + u) * kCT + row] = (sum[0] + sum[1]) + (sum[2] + sum[3]);
             }
-            x[j - jlo] = acc;
-            if (((j - j0) & 3) == 0) {        // every fourth step: has every product fallen below 2^-40 of the start?
-                float top = 0.f;
+            float top = 0.f;
 #pragma unroll
-                for (int s = 0; s < kM; ++s) top = fmaxf(top, fabsf(qd[s]));
-                if (top <= floor_) break;
+            for (int e = 0; e < kHS; ++e) top = fmaxf(top, fabsf(qd[e]));
+            live = live && top > floor_;
+        }
+        compute_sync();
+        tc_fence_after_sync();
+        const int blk = band_block<REV>(wq, half, k);
+        if (blk >= 0) {
+            float v[32];
+            tmem_ld32(tmem_row_addr(tmem, wq, kColP + 32 * blk), v);
+            uint32_t out[2][16];
+#pragma unroll
+            for (int e = 0; e < 32; ++e) {
+                const int d = distance<REV>(row, 32 * blk + e) - kBand * k;
+                if (d >= 0 && d < kBand) v[e] = band0[d * kCT + row] + band1[d * kCT + row];
+                out[e >> 4][e & 15] = __float_as_uint(v[e]);
             }
+            tmem_st16(tmem_row_addr(tmem, wq, kColP + 32 * blk), out[0]);
+            tmem_st16(tmem_row_addr(tmem, wq, kColP + 32 * blk + 16), out[1]);
+            tmem_st_wait();
         }
+        tc_fence_before_sync();
+        const bool more = compute_sync_or(live);     // (the barrier also covers: the bands may be written again)
+        tc_fence_after_sync();
+        if (!more) break;
     }
-    const int base = kColP + 64 * half;
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        uint32_t hi[16], lo[16];
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            const float x0 = x[32 * q + 2 * e], x1 = x[32 * q + 2 * e + 1];
-            hi[e] = pack_bf16(x0, x1);
-            const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162*>(&hi[e]);
-            lo[e] = pack_bf16(x0 - __bfloat162float(h.x), x1 - __bfloat162float(h.y));
-        }
-        tmem_st16(tmem_row_addr(tmem, wq, base + 16 * q), hi);
-        tmem_st16(tmem_row_addr(tmem, wq, base + 32 + 16 * q), lo);
-    }
-    tmem_st_wait();
+    mask_row_in_tmem<REV, true>(tmem, wq, row, half, kColP);
 }
 
 // ======================================================================================
@@ -839,7 +887,8 @@ __device__ __noinline__ void key_side_general(const CUtensorMap& mapV, const CUt
                 mask_row_in_tmem<REV, true>(tmem, wq, row, half, kColP);
             } else {
                 // strong decay: A_ij by the walk over the per-step gates
-                key_side_explicit_rows<REV>(sG, sUq, sUk, tmem, wq, row, half, sb, grow, valid);
+                key_side_explicit_rows<REV>(sG, sUq, sUk, tmem, wq, row, half, sb, valid);
+                fence_async_smem();     // (gates and bands were written where the next tiles land)
             }
             tc_fence_before_sync();
             compute_sync();

@@ -684,7 +684,7 @@ state_scan_kernel(const __grid_constant__ CUtensorMap mapX0, const __grid_consta
                 sum += (double)a.G[(((size_t)span.b * a.T + min(t + kCT, span.t_end) - 1) * a.H + span.h) * kM + threadIdx.x];
             seg_logdecay[(size_t)blockIdx.x * kM + threadIdx.x] = (float)sum;
         }
-        value_side_general<REV>(mapX, mapX, second ? mapW32_1 : mapW32_0, mapG32, mapG32, a, dev_status, slice);
+        value_side_general<REV, true, true>(mapX, mapX, second ? mapW32_1 : mapW32_0, mapG32, mapG32, a, dev_status, slice);
         return;
     }
     const float* G = a.G;
@@ -835,7 +835,6 @@ cudaError_t launch_state_scan_tc(const ValueSideArgs& k, const ValueSideArgs& v,
         a.xq = a.xk;
         a.S0 = nullptr;
         a.out = nullptr;
-        a.state_only = 1;
         if (e == cudaSuccess) e = make_tensor_map_bthd(&mx[i], a.xk, a.B, a.T, a.H, a.D, kCT, 2);
         if (e == cudaSuccess) e = make_tensor_map_bthd(&mw[i], a.wd, a.B, a.T, a.H, 2 * kM, kCT, 2);
         if (e == cudaSuccess) e = make_tensor_map_bthd(&mw32[i], a.w, a.B, a.T, a.H, kM, kCT, 4);

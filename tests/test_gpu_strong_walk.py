@@ -1,0 +1,26 @@
+"""Chunks of strong decay on the tensor-core kernels: the walk away from the diagonal takes 32 distances at a time.  One slot
+that forgets hard sends the pair there, the others' memory decides how far the walk goes: a few steps, past the first band,
+through all four; ragged chunks; both directions."""
+import numpy as np
+import pytest
+
+from test_gpu_parity import check_bwd, check_fwd, run_bwd, run_fwd
+from util import TOL, rand_inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("T", [1, 33, 128, 161, 300])
+@pytest.mark.parametrize("keep", [0.2, 0.55, 0.999])     # 2^-40 is below 0.2^18, 0.55^47 and 0.999^27000
+def test_strong_decay_walk(T, keep):
+    B, H, dk, dv, m = 1, 2, 128, 64, 64
+    d = rand_inputs(900 + T, B, T, H, dk, dv, m, "bf16", init=True, final_grads=True)
+    r = np.random.default_rng(T)
+    a = keep ** r.uniform(0.5, 1.5, d["gate"].shape)
+    a[..., 5] = 0.2                                       # e^-206 over a chunk of 128 tokens
+    a[..., 40] = 0.3
+    d["gate"] = a.astype(np.float32)
+    got, g = run_fwd(d, B, T, H, dk, dv, m, "bf16", impl="tc", log=True)
+    check_fwd(d, got, g, "bf16", log=True, tc=True)
+    gb, rb = run_bwd(d, B, T, H, dk, dv, m, "bf16", impl="tc", log=True)
+    check_bwd(gb, rb, TOL["bf16"], tc=True)
