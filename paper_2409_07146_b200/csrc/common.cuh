@@ -190,11 +190,6 @@ struct PendingDecay {
         const int seg = nseg == 1 ? 0 : t / tseg;
         return strong[(b * nseg + seg) * (H >> half_heads) + (h >> half_heads)] == 0;
     }
-    // row r = t * H + h of batch element b of a [B,T,H,M] tensor (32-bit arithmetic: T * H < 2^31)
-    __host__ __device__ bool pending(int b, int r) const {
-        const int t = r / H;
-        return pending_at(b, t, r - t * H);
-    }
     // the factor exp(-G_i) left out of the time-reversed partial sums, from an element of G (0 past the sequence end)
     __device__ float reverse_factor(float g) const { return wide ? (g > 0.f ? 1.f / g : 0.f) : __expf(-g); }
 };

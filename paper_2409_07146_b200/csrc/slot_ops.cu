@@ -256,6 +256,63 @@ __device__ __forceinline__ float row_sum(float x) {
     return x;
 }
 
+// A CTA's 256 threads hold 1024 consecutive values, 1024 / M rows.  These kernels move 16 bytes per thread and stream, so the
+// instructions around a row count (302 a thread forward, a third of them integer, kept the issue slots busy for 35 of 57 us;
+// 64 MB streams): everything that is the same for the CTA is formed from blockIdx alone, a thread adds a 32-bit offset, and
+// the row's token and head come from a multiplication (FastDiv).  B = 4, T = 4096, 32 heads of 128: 113 -> 96 us, backward
+// 154 -> 138; T = 32768, 16 heads: 113 -> 88.  (Two or four rows a thread instead, to have the same instructions serve more,
+// costs occupancy: 127 .. 131 us and 162 .. 199.)
+// x / d for x < 2^31: with mul = floor(2^shift / d) + 1, shift = 31 + ceil(log2 d), mul d exceeds 2^shift by at most d, and
+// x d < 2^shift, so the quotient is exact; mul < 2^32.
+struct FastDiv {
+    uint32_t mul, shift;
+    FastDiv() = default;
+    explicit FastDiv(uint32_t d) : shift(31) {
+        while ((1u << (shift - 31)) < d) ++shift;
+        mul = (uint32_t)((1ull << shift) / d + 1);
+    }
+    __device__ __forceinline__ uint32_t operator()(uint32_t x) const { return (uint32_t)(((uint64_t)x * mul) >> shift); }
+};
+struct RowDivs { FastDiv heads, segment; };       // by H and by the tokens of a segment
+
+template <int M> struct SlotPlace {
+    static constexpr int kRows = 256 * kSmR / M;
+    size_t cta;            // the CTA's first element
+    uint32_t off;          // this thread's first element from there (a row past the end repeats the last one: full-warp shuffles)
+    int col;               // ... and in its row
+    int rows;              // of a batch element
+    bool live, pending;
+    __device__ __forceinline__ SlotPlace(int rows_per_batch, const PendingDecay& pend, const RowDivs& div) {
+        const uint32_t row0 = blockIdx.x * kRows, left = rows_per_batch - row0, sub = threadIdx.x / (M / kSmR);
+        rows = rows_per_batch;
+        live = sub < left;
+        const uint32_t r = min(sub, left - 1);
+        col = (threadIdx.x % (M / kSmR)) * kSmR;
+        cta = ((size_t)blockIdx.y * rows_per_batch + row0) * M;
+        off = r * M + col;
+        pending = false;
+        if (pend.G != nullptr) {
+            const uint32_t t = div.heads(row0 + r), h = row0 + r - t * pend.H, seg = pend.nseg == 1 ? 0 : div.segment(t);
+            pending = pend.strong[(blockIdx.y * pend.nseg + seg) * (uint32_t)(pend.H >> pend.half_heads) + (h >> pend.half_heads)] == 0;
+        }
+    }
+    // of the decayed operand rows, which hold 2 bf16 a slot (128 slots: 3)
+    __device__ __forceinline__ size_t decayed() const { return (M == 128 ? 3 : 2) * (cta + (off - col)); }
+};
+template <int M>
+__device__ __forceinline__ void slot_sums(const float* part, int nslice, const SlotPlace<M>& at, float (&x)[kSmR]) {
+    ld_vec(part + at.cta + at.off, x);
+    if (nslice == 1) return;
+    const size_t total = (size_t)gridDim.y * (uint32_t)at.rows * M;
+#pragma unroll 3
+    for (int sl = 1; sl < nslice; ++sl) {
+        float t[kSmR];
+        ld_vec(part + (at.cta + sl * total) + at.off, t);
+#pragma unroll
+        for (int r = 0; r < kSmR; ++r) x[r] += t[r];
+    }
+}
+
 template <int M>
 __global__ void __launch_bounds__(256) slot_softmax_fwd_kernel(const float* part,
                                                                int nslice, float scale, int act,
@@ -263,34 +320,22 @@ __global__ void __launch_bounds__(256) slot_softmax_fwd_kernel(const float* part
                                                                float* __restrict__ p,
                                                                int rows_per_batch, const float* G,
                                                                __nv_bfloat16* __restrict__ p_decayed,
-                                                               PendingDecay pend, int m_active) {
+                                                               PendingDecay pend, int m_active, RowDivs div) {
     follow_previous_grid();
-    constexpr int R = kSmR, LPR = M / R, RPW = 32 / LPR;       // lanes per row, rows per warp
-    const int lane = threadIdx.x & 31, sub = lane / LPR, l = lane % LPR;
-    const int r_in_b = (blockIdx.x * 8 + (threadIdx.x >> 5)) * RPW + sub, b = blockIdx.y;
-    const bool live = r_in_b < rows_per_batch;       // a row past the end repeats the last one (full-warp shuffles)
-    const int rr = live ? r_in_b : rows_per_batch - 1;
-    const size_t row = (size_t)b * rows_per_batch + rr;
-    const size_t total = (size_t)gridDim.y * rows_per_batch * M;
-    const size_t idx = row * M + l * R;
-    const bool pending = pend.pending(b, rr);
+    constexpr int R = kSmR, LPR = M / R;       // lanes per row
+    const SlotPlace<M> at(rows_per_batch, pend, div);
+    const bool live = at.live, pending = at.pending;
     // slots from m_active on are padding (a layer with fewer slots than the kernels' tile): they take no part
-    const bool padded = l * R >= m_active;
+    const bool padded = at.col >= m_active;
     // serving the flagged pairs only: a warp none of whose rows is flagged has nothing to do
     const bool skip = pend.strong_only != 0 && pending;
     if (__all_sync(0xffffffffu, skip)) return;
     float z[R], eg[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) { z[r] = 0.f; eg[r] = 1.f; }
-#pragma unroll 4
-    for (int sl = 0; sl < nslice; ++sl) {
-        float t[R];
-        ld_vec(part + idx + (size_t)sl * total, t);
-#pragma unroll
-        for (int r = 0; r < R; ++r) z[r] += t[r];
-    }
+    for (int r = 0; r < R; ++r) eg[r] = 1.f;
+    slot_sums<M>(part, nslice, at, z);
     if (G != nullptr) {
-        ld_vec(G + idx, eg);
+        ld_vec(G + at.cta + at.off, eg);
 #pragma unroll
         for (int r = 0; r < R; ++r) eg[r] = M == 128 ? eg[r] : __expf(eg[r]);      // (128 slots: G holds exp(G) itself)
     }
@@ -316,15 +361,15 @@ __global__ void __launch_bounds__(256) slot_softmax_fwd_kernel(const float* part
         for (int r = 0; r < R; ++r) e[r] = padded ? 0.f : slot_act_value(z[r], act);
     }
     if (!live || skip) return;
-    if (ok != nullptr) st_vec(ok + idx, z);
+    if (ok != nullptr) st_vec(ok + at.cta + at.off, z);
     // fp32 p is read by the general chunk kernels and the CUDA-core kernels only: rows of a pair
     // that the pipelined kernels serve (pending) get the decayed bf16 rows alone
-    if (!pending) st_vec(p + idx, e);
+    if (!pending) st_vec(p + at.cta + at.off, e);
     if (p_decayed != nullptr) {
 #pragma unroll
         for (int r = 0; r < R; ++r) e[r] *= eg[r];
-        if (M == 128) st_split3(p_decayed + row * 3 * M, l * R, e);
-        else st_split<M>(p_decayed + row * 2 * M, l * R, e);
+        if (M == 128) st_split3(p_decayed + at.decayed(), at.col, e);
+        else st_split<M>(p_decayed + at.decayed(), at.col, e);
     }
 }
 
@@ -335,15 +380,16 @@ cudaError_t launch_slot_softmax_fwd(const float* part, int nslice, float scale, 
     const int rpb = 8 * (128 / M);       // rows per block: 8 warps x 128/M rows
     const dim3 grid((unsigned)((rows_per_batch + rpb - 1) / rpb), (unsigned)B);
     const int rows = rows_per_batch;
+    const RowDivs div{FastDiv(pend.H), FastDiv(pend.tseg)};
     if (M == 128)
         launch_after(slot_softmax_fwd_kernel<128>, grid, 256, 0, st, part, nslice, scale, act, ok, p, rows, G,
-                                                           static_cast<__nv_bfloat16*>(p_decayed), pend, m_active);
+                                                           static_cast<__nv_bfloat16*>(p_decayed), pend, m_active, div);
     else if (M == 64)
         launch_after(slot_softmax_fwd_kernel<64>, grid, 256, 0, st, part, nslice, scale, act, ok, p, rows, G,
-                                                          static_cast<__nv_bfloat16*>(p_decayed), pend, m_active);
+                                                          static_cast<__nv_bfloat16*>(p_decayed), pend, m_active, div);
     else
         launch_after(slot_softmax_fwd_kernel<32>, grid, 256, 0, st, part, nslice, scale, act, ok, p, rows, G,
-                                                          static_cast<__nv_bfloat16*>(p_decayed), pend, m_active);
+                                                          static_cast<__nv_bfloat16*>(p_decayed), pend, m_active, div);
     return cudaGetLastError();
 }
 
@@ -362,33 +408,21 @@ __global__ void __launch_bounds__(256) slot_softmax_bwd_kernel(const float* ok,
                                                                int rows_per_batch, const float* G,
                                                                __nv_bfloat16* __restrict__ p_decayed,
                                                                __nv_bfloat16* __restrict__ dz_decayed,
-                                                               PendingDecay pend, int m_active) {
+                                                               PendingDecay pend, int m_active, RowDivs div) {
     follow_previous_grid();
-    constexpr int R = kSmR, LPR = M / R, RPW = 32 / LPR;       // lanes per row, rows per warp
-    const int lane = threadIdx.x & 31, sub = lane / LPR, l = lane % LPR;
-    const int r_in_b = (blockIdx.x * 8 + (threadIdx.x >> 5)) * RPW + sub, b = blockIdx.y;
-    const bool live = r_in_b < rows_per_batch;       // a row past the end repeats the last one (full-warp shuffles)
-    const int rr = live ? r_in_b : rows_per_batch - 1;
-    const size_t row = (size_t)b * rows_per_batch + rr;
-    const size_t total = (size_t)gridDim.y * rows_per_batch * M;
-    const size_t idx = row * M + l * R;
-    const bool pending = pend.pending(b, rr);
+    constexpr int R = kSmR, LPR = M / R;       // lanes per row
+    const SlotPlace<M> at(rows_per_batch, pend, div);
+    const bool live = at.live, pending = at.pending;
     const bool skip = pend.strong_only != 0 && pending;      // (as in the forward kernel)
-    const bool padded = l * R >= m_active;                   // (likewise)
+    const bool padded = at.col >= m_active;                  // (likewise)
     if (__all_sync(0xffffffffu, skip)) return;
     float z[R], dpv[R], eg[R];
-    ld_vec(ok + idx, z);
+    ld_vec(ok + at.cta + at.off, z);
 #pragma unroll
-    for (int r = 0; r < R; ++r) { dpv[r] = 0.f; eg[r] = 1.f; }
-#pragma unroll 4
-    for (int sl = 0; sl < nslice; ++sl) {
-        float t[R];
-        ld_vec(dp_part + idx + (size_t)sl * total, t);
-#pragma unroll
-        for (int r = 0; r < R; ++r) dpv[r] += t[r];
-    }
+    for (int r = 0; r < R; ++r) eg[r] = 1.f;
+    slot_sums<M>(dp_part, nslice, at, dpv);
     if (G != nullptr) {
-        ld_vec(G + idx, eg);
+        ld_vec(G + at.cta + at.off, eg);
 #pragma unroll
         for (int r = 0; r < R; ++r) eg[r] = M == 128 ? eg[r] : __expf(eg[r]);      // (128 slots: G holds exp(G) itself)
     }
@@ -428,19 +462,19 @@ __global__ void __launch_bounds__(256) slot_softmax_bwd_kernel(const float* ok,
     }
     if (!live || skip) return;
     if (!pending) {       // (as in the forward: fp32 p and dz only where a non-pipelined kernel reads them)
-        if (p != nullptr) st_vec(p + idx, e);      // (p == NULL: the forward's p is kept and in use)
-        st_vec(dz + idx, dzv);
+        if (p != nullptr) st_vec(p + at.cta + at.off, e);      // (p == NULL: the forward's p is kept and in use)
+        st_vec(dz + at.cta + at.off, dzv);
     }
-    st_vec(u + idx, uv);
+    st_vec(u + at.cta + at.off, uv);
     if (dz_decayed != nullptr) {
 #pragma unroll
         for (int r = 0; r < R; ++r) { e[r] *= eg[r]; dzv[r] *= eg[r]; }
         if (M == 128) {
-            if (p_decayed != nullptr) st_split3(p_decayed + row * 3 * M, l * R, e);
-            st_split3(dz_decayed + row * 3 * M, l * R, dzv);
+            if (p_decayed != nullptr) st_split3(p_decayed + at.decayed(), at.col, e);
+            st_split3(dz_decayed + at.decayed(), at.col, dzv);
         } else {
-            if (p_decayed != nullptr) st_split<M>(p_decayed + row * 2 * M, l * R, e);
-            st_split<M>(dz_decayed + row * 2 * M, l * R, dzv);
+            if (p_decayed != nullptr) st_split<M>(p_decayed + at.decayed(), at.col, e);
+            st_split<M>(dz_decayed + at.decayed(), at.col, dzv);
         }
     }
 }
@@ -453,18 +487,19 @@ cudaError_t launch_slot_softmax_bwd(const float* ok, const float* dp_part, int n
     const int rpb = 8 * (128 / M);       // rows per block: 8 warps x 128/M rows
     const dim3 grid((unsigned)((rows_per_batch + rpb - 1) / rpb), (unsigned)B);
     const int rows = rows_per_batch;
+    const RowDivs div{FastDiv(pend.H), FastDiv(pend.tseg)};
     if (M == 128)
         launch_after(slot_softmax_bwd_kernel<128>, grid, 256, 0, st, ok, dp_part, nslice, scale, act, p, dz, u, rows, G,
                                                            static_cast<__nv_bfloat16*>(p_decayed),
-                                                           static_cast<__nv_bfloat16*>(dz_decayed), pend, m_active);
+                                                           static_cast<__nv_bfloat16*>(dz_decayed), pend, m_active, div);
     else if (M == 64)
         launch_after(slot_softmax_bwd_kernel<64>, grid, 256, 0, st, ok, dp_part, nslice, scale, act, p, dz, u, rows, G,
                                                           static_cast<__nv_bfloat16*>(p_decayed),
-                                                          static_cast<__nv_bfloat16*>(dz_decayed), pend, m_active);
+                                                          static_cast<__nv_bfloat16*>(dz_decayed), pend, m_active, div);
     else
         launch_after(slot_softmax_bwd_kernel<32>, grid, 256, 0, st, ok, dp_part, nslice, scale, act, p, dz, u, rows, G,
                                                           static_cast<__nv_bfloat16*>(p_decayed),
-                                                          static_cast<__nv_bfloat16*>(dz_decayed), pend, m_active);
+                                                          static_cast<__nv_bfloat16*>(dz_decayed), pend, m_active, div);
     return cudaGetLastError();
 }
 
@@ -617,7 +652,7 @@ __global__ void __launch_bounds__(128) gate_grad_local_kernel(
     };
     float2 x[kGG], dI[kGG], gt[kGG];
     load_dI(dIk, nsk, dIv, nsv, base, stride, total, rows, dI);
-    if (pend.pending(b, t0 * H + h)) {
+    if (pend.pending_at(b, t0, h)) {
         // the time-reversed value_side runs left their row factor exp(-G_i) to this kernel
 #pragma unroll
         for (int i = 0; i < kGG; ++i) gt[i] = ld2(pend.G, i, 0.f);
