@@ -2,6 +2,8 @@
 // (chunk_cumsum of Algorithm 1), the slot softmax between the two passes and its
 // backward, and the forget-gate gradient (reversed cumulative sum, App. B).
 // All of them stream [B,T,H,m] fp32 tensors once: they are HBM-bound.
+#include <type_traits>
+
 #include "common.cuh"
 #include "tc_common.cuh"
 
@@ -58,10 +60,21 @@ __device__ __forceinline__ bool sequence_starts_at(const int* cu, int nseq, int 
 // a chunk down to a chunk's own decay of e^-20.  Everywhere else the chunk takes -100 and the strong-decay kernels.
 constexpr float kReset = 40.f;
 
-// WIDE: the halves of 128 slots as 2 H heads of 64 (see launch_gate_cumsum_wide), which share their head's flag.
-template <int M, bool WIDE = false>
+// exp(-G), 2^-126 and below as zero, of a moderate chunk's sum (at least -60: the plain exponential)
+__device__ __forceinline__ float exp_minus(float g) {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(g * -1.4426950408889634f));
+    return r;
+}
+
+// KIND: gate_kind.  WIDE: the halves of 128 slots as 2 H heads of 64 (see launch_gate_cumsum_wide), which share their
+// head's flag.  907 instructions a thread -- the kind asked for at every element, a predicate at every row, a 64-bit address
+// for every access -- kept the issue slots as busy as the memory; with the kind a template argument, whole chunks apart from
+// ragged ones and 32-bit offsets from the chunk's first element: B = 4, T = 4096, 32 heads, 64 slots (0.54 GB) 137 -> 95 us,
+// 5.7 TB/s; 128 slots, B = 8, T = 2048, 4 heads 48 -> 39.
+template <int M, bool WIDE, int KIND>
 __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) gate_cumsum_kernel(const float* gate,
-                                                            int gate_kind, float inv_tau,
+                                                            float inv_tau,
                                                             float* __restrict__ G,
                                                             float* __restrict__ I, int T, int H,
                                                             int chunk, int* __restrict__ strong_flag, int nseg, int tseg,
@@ -69,41 +82,49 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
                                                             const int* cu_seqlens, int nseq,
                                                             float* __restrict__ E) {
     follow_previous_grid();
-    __shared__ double group_sum[16][M];
-    const int s = 2 * threadIdx.x, grp = threadIdx.y;          // blockDim.y = chunk / 8 <= 16
+    __shared__ double2 group_sum[16][M / 2];
+    const int grp = threadIdx.y, s = 2 * threadIdx.x;          // blockDim.y = chunk / 8 <= 16
     const int n = blockIdx.y;
     const int bh = blockIdx.x, b = bh / H, h = bh % H;
-    const int t0 = n * chunk + grp * kCumRows;
-    const int rows = max(0, min(kCumRows, min(T, (n + 1) * chunk) - t0));
-    const size_t stride = (size_t)H * M;
-    const size_t base = (((size_t)b * T + t0) * H + h) * M + s;
+    const int t_chunk = n * chunk, rows_here = min(T - t_chunk, chunk);
+    const int rows = max(0, min(kCumRows, rows_here - grp * kCumRows));
+    // (a CTA's first element, and 32-bit offsets from there: a chunk's rows reach 128 H M < 2^31 elements)
+    const size_t first = (((size_t)b * T + t_chunk) * H + h) * M;
+    const uint32_t stride = (uint32_t)H * M, off = grp * kCumRows * stride + s;
     float2 g[kCumRows], inps[kCumRows];
     __shared__ uint32_t starts[4];                // rows of the chunk that begin a packed sequence, one bit each
     if (cu_seqlens != nullptr) {
         const int tid = threadIdx.y * blockDim.x + threadIdx.x;
         if (tid < 4) starts[tid] = 0;
         __syncthreads();
-        for (int r = tid; r < min(chunk, T - n * chunk); r += blockDim.x * blockDim.y)
-            if (sequence_starts_at(cu_seqlens, nseq, n * chunk + r)) atomicOr(&starts[r >> 5], 1u << (r & 31));
+        for (int r = tid; r < rows_here; r += blockDim.x * blockDim.y)
+            if (sequence_starts_at(cu_seqlens, nseq, t_chunk + r)) atomicOr(&starts[r >> 5], 1u << (r & 31));
         __syncthreads();
+    }
+    {
+        // (rows past the end: a = 1, log a = 0)
+        const float neutral = KIND == GSA_GATE_LOG_A ? 0.f : (KIND == GSA_GATE_LOGITS ? 80.f : 1.f);
+        const float* src = gate + first;
+        if (rows == kCumRows) {
+#pragma unroll
+            for (int i = 0; i < kCumRows; ++i) g[i] = *reinterpret_cast<const float2*>(src + (off + i * stride));
+        } else {
+#pragma unroll
+            for (int i = 0; i < kCumRows; ++i)
+                g[i] = i < rows ? *reinterpret_cast<const float2*>(src + (off + i * stride)) : make_float2(neutral, neutral);
+        }
     }
 #pragma unroll
     for (int i = 0; i < kCumRows; ++i) {
-        // (rows past the end: a = 1, log a = 0)
-        const float neutral = gate_kind == GSA_GATE_LOG_A ? 0.f : (gate_kind == GSA_GATE_LOGITS ? 80.f : 1.f);
-        float2 x = make_float2(neutral, neutral);
-        if (i < rows) x = *reinterpret_cast<const float2*>(gate + base + (size_t)i * stride);
-        if (gate_kind == GSA_GATE_LOGITS) x = make_float2(log_gate_from_logit(x.x, inv_tau), log_gate_from_logit(x.y, inv_tau));
-        if (gate_kind != GSA_GATE_A) {
-            g[i] = x;
+        float2 x = g[i];
+        if (KIND == GSA_GATE_LOGITS) x = make_float2(log_gate_from_logit(x.x, inv_tau), log_gate_from_logit(x.y, inv_tau));
+        if (KIND != GSA_GATE_A) {
             inps[i] = make_float2(-expm1f(x.x), -expm1f(x.y));
         } else {
-            g[i] = fast_log ? make_float2(__logf(x.x), __logf(x.y)) : make_float2(logf(x.x), logf(x.y));
             inps[i] = make_float2(1.f - x.x, 1.f - x.y);
+            x = fast_log ? make_float2(__logf(x.x), __logf(x.y)) : make_float2(logf(x.x), logf(x.y));
         }
-        g[i].x = fmaxf(g[i].x, kLogGateMin);
-        g[i].y = fmaxf(g[i].y, kLogGateMin);
-        if (i < rows) *reinterpret_cast<float2*>(I + base + (size_t)i * stride) = inps[i];
+        g[i] = make_float2(fmaxf(x.x, kLogGateMin), fmaxf(x.y, kLogGateMin));
     }
     // the first token of a packed sequence drops what the memories carried; its own write, 1 - a, is untouched
     if (cu_seqlens != nullptr && (starts[0] | starts[1] | starts[2] | starts[3]) != 0) {
@@ -115,11 +136,10 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
 #pragma unroll
             for (int i = 0; i < kCumRows; ++i)
                 if (i < rows && !((mine >> i) & 1)) { own0 += g[i].x; own1 += g[i].y; }
-            group_sum[grp][s] = own0;
-            group_sum[grp][s + 1] = own1;
+            group_sum[grp][threadIdx.x] = make_double2(own0, own1);
             __syncthreads();
             double all0 = 0.0, all1 = 0.0;
-            for (int q = 0; q < (int)blockDim.y; ++q) { all0 += group_sum[q][s]; all1 += group_sum[q][s + 1]; }
+            for (int q = 0; q < (int)blockDim.y; ++q) { all0 += group_sum[q][threadIdx.x].x; all1 += group_sum[q][threadIdx.x].y; }
             const int count = __popc(starts[0]) + __popc(starts[1]) + __popc(starts[2]) + __popc(starts[3]);
             if (__syncthreads_and(fmin(all0, all1) - kReset * count >= (double)kFactorisedDecayMin)) reset = -kReset;
         }
@@ -132,57 +152,76 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
     // makes |G| reach the hundreds, without a conversion per element
 #pragma unroll
     for (int i = 1; i < kCumRows; ++i) {
-        g[i].x = (i < rows) ? g[i - 1].x + g[i].x : g[i - 1].x;
-        g[i].y = (i < rows) ? g[i - 1].y + g[i].y : g[i - 1].y;
+        // (a row past the end adds its log a of 0)
+        g[i].x += g[i - 1].x;
+        g[i].y += g[i - 1].y;
     }
-    const double acc0 = rows > 0 ? (double)g[kCumRows - 1].x : 0.0, acc1 = rows > 0 ? (double)g[kCumRows - 1].y : 0.0;
-    group_sum[grp][s] = acc0;
-    group_sum[grp][s + 1] = acc1;
+    const double acc0 = (double)g[kCumRows - 1].x, acc1 = (double)g[kCumRows - 1].y;
+    group_sum[grp][threadIdx.x] = make_double2(acc0, acc1);
     __syncthreads();
     double before0 = 0.0, before1 = 0.0, half0 = 0.0, half1 = 0.0;       // (half: since the last multiple of 64 tokens)
+#pragma unroll 5
     for (int q = 0; q < grp; ++q) {
+        const double2 t = group_sum[q][threadIdx.x];
         if (WIDE && q == 64 / kCumRows) half0 = half1 = 0.0;
-        before0 += group_sum[q][s];
-        before1 += group_sum[q][s + 1];
-        half0 += group_sum[q][s];
-        half1 += group_sum[q][s + 1];
+        before0 += t.x;
+        before1 += t.y;
+        if (WIDE) {
+            half0 += t.x;
+            half1 += t.y;
+        }
     }
     if (WIDE && grp == 64 / kCumRows) half0 = half1 = 0.0;
     // the chunk's total log-decay decides which of the chunk kernels takes this (b,h)
     // (with segment-parallel scheduling the flags are per (batch, segment, head))
     if (strong_flag != nullptr && grp == (int)blockDim.y - 1 &&
         fmin(before0 + acc0, before1 + acc1) < (double)kFactorisedDecayMin) {
-        const int seg = nseg == 1 ? 0 : n * chunk / tseg;
+        const int seg = nseg == 1 ? 0 : t_chunk / tseg;
         strong_flag[WIDE ? (b * nseg + seg) * (H / 2) + h / 2 : (b * nseg + seg) * H + h] = 1;
     }
     // second pass over the same rows: the sums of the groups before as a float pair (value, rest)
     const float b0h = (float)before0, b0l = (float)(before0 - (double)b0h);
     const float b1h = (float)before1, b1l = (float)(before1 - (double)b1h);
-#pragma unroll
-    for (int i = 0; i < kCumRows; ++i)
-        if (i < rows) {
-            const float G0 = b0h + (b0l + g[i].x), G1 = b1h + (b1l + g[i].y);
-            if (!WIDE) *reinterpret_cast<float2*>(G + base + (size_t)i * stride) = make_float2(G0, G1);
-            if (WIDE) {
-                // G itself is for the CUDA-core kernels, whose chunks have 64 tokens
-                *reinterpret_cast<float2*>(G + base + (size_t)i * stride) =
-                    make_float2((float)(half0 + (double)g[i].x), (float)(half1 + (double)g[i].y));
-                // exp(+-G) from the sum before its rounding to G: G0 + r0 is the sum of the pair and the thread's rows
-                const float r0 = (b0l + g[i].x) - (G0 - b0h), r1 = (b1l + g[i].y) - (G1 - b1h);
-                const float e0 = expf(G0), e1 = expf(G1), d0 = expf(-G0), d1 = expf(-G1);
-                *reinterpret_cast<float2*>(E + base + (size_t)i * stride) = make_float2(fmaf(e0, r0, e0), fmaf(e1, r1, e1));
-                uint32_t hi, mid, lo;
-                split_bf16x3(inps[i].x * fmaf(d0, -r0, d0), inps[i].y * fmaf(d1, -r1, d1), hi, mid, lo);
-                uint32_t* row = reinterpret_cast<uint32_t*>(decayed + 3 * (base + (size_t)i * stride - s) + s);
-                row[0] = hi;
-                row[M / 2] = mid;
-                row[M] = lo;
-            } else if (decayed != nullptr) {
-                // (meaningful for moderate decay only; pairs with a strong-decay chunk do not read it)
-                store_split2<M>(decayed + 2 * (base + (size_t)i * stride - s), s, inps[i].x * __expf(-G0),
-                                inps[i].y * __expf(-G1));
-            }
+    auto write_row = [&](int i) {
+        const uint32_t at = off + i * stride;
+        *reinterpret_cast<float2*>(I + first + at) = inps[i];
+        const float G0 = b0h + (b0l + g[i].x), G1 = b1h + (b1l + g[i].y);
+        if (!WIDE) {
+            *reinterpret_cast<float2*>(G + first + at) = make_float2(G0, G1);
+            // (meaningful for moderate decay only; pairs with a strong-decay chunk do not read it)
+            if (decayed != nullptr)
+                store_split2<M>(decayed + 2 * first + (2 * at - 2 * s), s, inps[i].x * exp_minus(G0), inps[i].y * exp_minus(G1));
+        } else {
+            // G itself is for the CUDA-core kernels, whose chunks have 64 tokens
+            *reinterpret_cast<float2*>(G + first + at) =
+                make_float2((float)(half0 + (double)g[i].x), (float)(half1 + (double)g[i].y));
+            // exp(+-G) from the sum before its rounding to G: G0 + r0 is the sum of the pair and the thread's rows
+            const float r0 = (b0l + g[i].x) - (G0 - b0h), r1 = (b1l + g[i].y) - (G1 - b1h);
+            const float e0 = expf(G0), e1 = expf(G1), d0 = expf(-G0), d1 = expf(-G1);
+            *reinterpret_cast<float2*>(E + first + at) = make_float2(fmaf(e0, r0, e0), fmaf(e1, r1, e1));
+            uint32_t hi, mid, lo;
+            split_bf16x3(inps[i].x * fmaf(d0, -r0, d0), inps[i].y * fmaf(d1, -r1, d1), hi, mid, lo);
+            uint32_t* row = reinterpret_cast<uint32_t*>(decayed + 3 * first + (3 * (at - s) + s));
+            row[0] = hi;
+            row[M / 2] = mid;
+            row[M] = lo;
         }
+    };
+    if (rows == kCumRows) {
+#pragma unroll
+        for (int i = 0; i < kCumRows; ++i) write_row(i);
+    } else {
+#pragma unroll
+        for (int i = 0; i < kCumRows; ++i)
+            if (i < rows) write_row(i);
+    }
+}
+
+template <int M, bool WIDE, class... A>
+void launch_gate_kind(int gate_kind, dim3 grid, dim3 block, cudaStream_t st, const float* gate, A... rest) {
+    if (gate_kind == GSA_GATE_A) launch_after(gate_cumsum_kernel<M, WIDE, GSA_GATE_A>, grid, block, 0, st, gate, rest...);
+    else if (gate_kind == GSA_GATE_LOG_A) launch_after(gate_cumsum_kernel<M, WIDE, GSA_GATE_LOG_A>, grid, block, 0, st, gate, rest...);
+    else launch_after(gate_cumsum_kernel<M, WIDE, GSA_GATE_LOGITS>, grid, block, 0, st, gate, rest...);
 }
 
 cudaError_t launch_gate_cumsum(const float* gate, int gate_kind, float inv_tau, float* G, float* I, int B,
@@ -192,15 +231,13 @@ cudaError_t launch_gate_cumsum(const float* gate, int gate_kind, float inv_tau, 
     const int nchunks = (T + chunk - 1) / chunk;
     dim3 block(M / 2, chunk / kCumRows);
     dim3 grid(B * H, nchunks);
-    if (M == 128)
-        launch_after(gate_cumsum_kernel<128>, grid, block, 0, st, gate, gate_kind, inv_tau, G, I, T, H, chunk, strong_flag, nseg, tseg,
-                                                        static_cast<__nv_bfloat16*>(decayed), fast_log, cu_seqlens, nseq, nullptr);
-    else if (M == 64)
-        launch_after(gate_cumsum_kernel<64>, grid, block, 0, st, gate, gate_kind, inv_tau, G, I, T, H, chunk, strong_flag, nseg, tseg,
-                                                       static_cast<__nv_bfloat16*>(decayed), fast_log, cu_seqlens, nseq, nullptr);
-    else
-        launch_after(gate_cumsum_kernel<32>, grid, block, 0, st, gate, gate_kind, inv_tau, G, I, T, H, chunk, strong_flag, nseg, tseg,
-                                                       static_cast<__nv_bfloat16*>(decayed), fast_log, cu_seqlens, nseq, nullptr);
+    auto launch = [&](auto m) {
+        launch_gate_kind<decltype(m)::value, false>(gate_kind, grid, block, st, gate, inv_tau, G, I, T, H, chunk, strong_flag, nseg, tseg,
+                                                    static_cast<__nv_bfloat16*>(decayed), fast_log, cu_seqlens, nseq, (float*)nullptr);
+    };
+    if (M == 128) launch(std::integral_constant<int, 128>{});
+    else if (M == 64) launch(std::integral_constant<int, 64>{});
+    else launch(std::integral_constant<int, 32>{});
     return cudaGetLastError();
 }
 
@@ -208,8 +245,8 @@ cudaError_t launch_gate_cumsum_wide(const float* gate, int gate_kind, float inv_
                                     int H, int* strong_flag, int nseg, int tseg, void* decayed, cudaStream_t st,
                                     const int* cu_seqlens, int nseq) {
     constexpr int chunk = 128;
-    launch_after(gate_cumsum_kernel<64, true>, dim3(2 * B * H, (T + chunk - 1) / chunk), dim3(32, chunk / kCumRows), 0, st, gate, gate_kind, inv_tau, G, I, T, 2 * H, chunk, strong_flag, nseg, tseg, static_cast<__nv_bfloat16*>(decayed), 0,
-        cu_seqlens, nseq, E);
+    launch_gate_kind<64, true>(gate_kind, dim3(2 * B * H, (T + chunk - 1) / chunk), dim3(32, chunk / kCumRows), st, gate, inv_tau, G, I, T,
+                               2 * H, chunk, strong_flag, nseg, tseg, static_cast<__nv_bfloat16*>(decayed), 0, cu_seqlens, nseq, E);
     return cudaGetLastError();
 }
 
