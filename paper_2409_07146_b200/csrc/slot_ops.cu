@@ -731,11 +731,84 @@ constexpr int kGGTmaRows = 32;
 constexpr int kGGTmaMaxSlices = 8;
 constexpr int kGGTileB = kGGTmaRows * 64 * 4;      // bytes of one [32 x 64] fp32 tile (two swizzled panels)
 
+// A thread's eight rows of a staged tile -- slot tx, 16-row group ty, early (0) or late (1) half hh of it -- and their output.
+// The kind of gate is a template argument, every shared-memory address an offset of the row plus a constant of the stream,
+// and whole halves are apart from ragged ones: 802 instructions a thread kept the issue slots busy for 47 of 81 us.  With the
+// carry kernel treated alike, the gate gradient of B = 4, T = 4096, 32 heads of 128: 231 -> 211 us; B = 8, T = 2048, 4 heads of
+// 512: 61 -> 57, with 128 slots 110 -> 96.
+constexpr int kGGHalf = kGG / 2;
+template <int KIND, bool WIDE> struct GateGradRows {
+    float x[kGGHalf], dI[kGGHalf], gt[kGGHalf];       // u - I dI; dI; the gate as passed
+    // tiles 0..3 = u, I, gate, G, then the slices of dI; a swizzled panel of 32 slots is half a tile
+    __device__ __forceinline__ void read(const unsigned char* tiles, int nslices, int tx, int ty, int hh, bool pending) {
+        const unsigned char* row = tiles + (tx >> 5) * (kGGTileB / 2) + (ty * kGG + hh * kGGHalf) * 128 + (tx & 3) * 4;
+        const int q = (tx & 31) >> 2;
+        int off[kGGHalf];
+#pragma unroll
+        for (int i = 0; i < kGGHalf; ++i) off[i] = i * 128 + ((q ^ i) << 4);          // (row & 7 == i)
+        auto at = [&](int tile, int i) { return *reinterpret_cast<const float*>(row + off[i] + tile * kGGTileB); };
+#pragma unroll
+        for (int i = 0; i < kGGHalf; ++i) dI[i] = 0.f;
+#pragma unroll
+        for (int sl = 0; sl < kGGTmaMaxSlices; ++sl) {
+            if (sl >= nslices) break;
+#pragma unroll
+            for (int i = 0; i < kGGHalf; ++i) dI[i] += at(4 + sl, i);
+        }
+        if (pending) {
+            // the time-reversed value_side runs left their row factor exp(-G_i) to this kernel
+#pragma unroll
+            for (int i = 0; i < kGGHalf; ++i) {
+                const float g = at(3, i);      // (128 slots: exp(G), 0 past the sequence end)
+                dI[i] *= WIDE ? (g > 0.f ? 1.f / g : 0.f) : exp_minus(g);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < kGGHalf; ++i) {
+            gt[i] = at(2, i);
+            const float ii = KIND == GSA_GATE_A ? 1.f - gt[i] : at(1, i);      // 1 - a as the gate kernel formed it
+            x[i] = at(0, i) - ii * dI[i];                                      // rows past the end: u = dI = 0
+        }
+    }
+    // sum over the rows, up to the first token that begins a sequence
+    __device__ __forceinline__ float total(uint32_t starts) const {
+        float tot = 0.f;
+        if (starts == 0) {
+#pragma unroll
+            for (int i = 0; i < kGGHalf; ++i) tot += x[i];
+        } else {
+#pragma unroll
+            for (int i = 0; i < kGGHalf; ++i)
+                if ((starts & ((2u << i) - 1)) == 0) tot += x[i];
+        }
+        return tot;
+    }
+    // the rows' gradients from the sum `run` of the rows behind them in the group, which becomes theirs too
+    __device__ __forceinline__ float write(float run, uint32_t starts, int rows, float* out, uint32_t stride, float inv_tau) const {
+        if (starts == 0 && rows >= kGGHalf) {
+#pragma unroll
+            for (int i = kGGHalf - 1; i >= 0; --i) {
+                run += x[i];
+                out[i * stride] = gate_grad_out(run, dI[i], gt[i], KIND, inv_tau);
+            }
+        } else {
+#pragma unroll
+            for (int i = kGGHalf - 1; i >= 0; --i) {
+                run += x[i];
+                if ((starts >> i) & 1) run = 0.f;
+                if (i < rows) out[i * stride] = gate_grad_out(run, dI[i], gt[i], KIND, inv_tau);
+            }
+        }
+        return run;
+    }
+};
+
+template <int KIND, bool WIDE>
 __global__ void __launch_bounds__(256) gate_grad_local_tma_kernel(
     const __grid_constant__ CUtensorMap mapU, const __grid_constant__ CUtensorMap mapI,
     const __grid_constant__ CUtensorMap mapGate, const __grid_constant__ CUtensorMap mapG,
     const __grid_constant__ CUtensorMap mapDIk, const __grid_constant__ CUtensorMap mapDIv, int nsk, int nsv,
-    int gate_kind, float inv_tau, float* __restrict__ blk_tot, float* __restrict__ dgate, int T, int H, int nblk,
+    float inv_tau, float* __restrict__ blk_tot, float* __restrict__ dgate, int T, int H, int nblk,
     PendingDecay pend, const int* cu, int nseq, int32_t* dev_status) {
     follow_previous_grid();
     using namespace tc;
@@ -754,7 +827,7 @@ __global__ void __launch_bounds__(256) gate_grad_local_tma_kernel(
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         // tiles 0..3 = u, I, gate, G; I is not read when the gate tensor holds a itself (1 - a is one
         // subtraction), G only when a row factor is pending
-        const bool need[4] = {true, gate_kind != GSA_GATE_A, true, pend.G != nullptr};
+        const bool need[4] = {true, KIND != GSA_GATE_A, true, pend.G != nullptr};
         int ntiles = nslices;
         for (int i = 0; i < 4; ++i) ntiles += need[i] ? 1 : 0;
         mbar_expect_tx(&bar, (uint32_t)(ntiles * kGGTileB));
@@ -776,50 +849,16 @@ __global__ void __launch_bounds__(256) gate_grad_local_tma_kernel(
     if (!landed && threadIdx.x == 0 && dev_status != nullptr) *dev_status = GSA_ERR_TIMEOUT;
     if (__syncthreads_or(!landed)) return;
 
-    constexpr int kHalf = kGG / 2;
     const int n = blockIdx.y * (kGGTmaRows / kGG) + ty;           // 16-row block of the sequence
-    const int rows = n < nblk ? min(kGG, T - n * kGG) : 0;
-    // row r (of this thread's 16), this thread's slot, of tile `tile`
-    auto at = [&](int tile, int r) {
-        const int row = ty * kGG + hh * kHalf + r, c = tx;
-        const unsigned char* p = smem + tile * kGGTileB + (c >> 5) * (kGGTileB / 2) + swz128(row, (c & 31) >> 2) + (c & 3) * 4;
-        return *reinterpret_cast<const float*>(p);
-    };
-    float x[kHalf], dI[kHalf];
-#pragma unroll
-    for (int i = 0; i < kHalf; ++i) dI[i] = 0.f;
-    for (int sl = 0; sl < nslices; ++sl) {
-#pragma unroll
-        for (int i = 0; i < kHalf; ++i) dI[i] += at(4 + sl, i);
-    }
-    if (pend.pending_at(b, t0, h)) {
-        // the time-reversed value_side runs left their row factor exp(-G_i) to this kernel
-#pragma unroll
-        for (int i = 0; i < kHalf; ++i) dI[i] *= pend.reverse_factor(at(3, i));
-    }
-#pragma unroll
-    for (int i = 0; i < kHalf; ++i) {
-        const float ii = gate_kind == GSA_GATE_A ? 1.f - at(2, i) : at(1, i);      // 1 - a as the gate kernel formed it
-        x[i] = at(0, i) - ii * dI[i];                                              // rows past the end: u = dI = 0
-    }
-    const size_t stride = (size_t)H * M;
-    const size_t base = (((size_t)b * T + n * kGG + hh * kHalf) * H + h) * M + tx;
+    const int rows = n < nblk ? T - n * kGG - hh * kGGHalf : 0;   // ... from this thread's first row on
+    GateGradRows<KIND, WIDE> r;
+    r.read(smem, nslices, tx, ty, hh, pend.pending_at(b, t0, h));
     // the early half starts from the total of the late half of its group
-    const uint32_t starts = starts_among(cu, nseq, n * kGG + hh * kHalf, kHalf);
-    float tot = 0.f;
-#pragma unroll
-    for (int i = 0; i < kHalf; ++i)
-        if ((starts & ((2u << i) - 1)) == 0) tot += x[i];         // (up to the first token that begins a sequence)
-    if (hh == 1) late_half[ty][tx] = tot;
+    const uint32_t starts = starts_among(cu, nseq, n * kGG + hh * kGGHalf, kGGHalf);
+    if (hh == 1) late_half[ty][tx] = r.total(starts);
     __syncthreads();
-    float run = hh == 0 ? late_half[ty][tx] : 0.f;
-#pragma unroll
-    for (int i = kHalf - 1; i >= 0; --i) {
-        run += x[i];
-        if ((starts >> i) & 1) run = 0.f;
-        if (hh * kHalf + i < rows)
-            dgate[base + (size_t)i * stride] = gate_grad_out(run, dI[i], at(2, i), gate_kind, inv_tau);
-    }
+    float* out = dgate + (((size_t)b * T + t0) * H + h) * M + (uint32_t)((ty * kGG + hh * kGGHalf) * H * M + tx);
+    const float run = r.write(hh == 0 ? late_half[ty][tx] : 0.f, starts, rows, out, (uint32_t)H * M, inv_tau);
     if (hh == 0 && n < nblk) blk_tot[((size_t)bh * nblk + n) * M + tx] = run;
 }
 
@@ -834,11 +873,12 @@ constexpr int kGGMaxStages = 4;
 constexpr int kGGRingMinSlices = 6;
 constexpr int kGGComputeThreads = 256;
 
+template <int KIND, bool WIDE>
 __global__ void __launch_bounds__(kGGComputeThreads + 32) gate_grad_local_ring_kernel(
     const __grid_constant__ CUtensorMap mapU, const __grid_constant__ CUtensorMap mapI,
     const __grid_constant__ CUtensorMap mapGate, const __grid_constant__ CUtensorMap mapG,
     const __grid_constant__ CUtensorMap mapDIk, const __grid_constant__ CUtensorMap mapDIv, int nsk, int nsv,
-    int gate_kind, float inv_tau, float* __restrict__ blk_tot, float* __restrict__ dgate, int T, int H, int BH,
+    float inv_tau, float* __restrict__ blk_tot, float* __restrict__ dgate, int T, int H, int BH,
     int ntile, int nstage, int nblk, PendingDecay pend, const int* cu, int nseq, int32_t* dev_status) {
     follow_previous_grid();
     using namespace tc;
@@ -865,7 +905,7 @@ __global__ void __launch_bounds__(kGGComputeThreads + 32) gate_grad_local_ring_k
         // =============================== copy lane
         // tiles 0..3 = u, I, gate, G; I is not read when the gate tensor holds a itself (1 - a is one
         // subtraction), G only when a row factor is pending
-        const bool need[4] = {true, gate_kind != GSA_GATE_A, true, pend.G != nullptr};
+        const bool need[4] = {true, KIND != GSA_GATE_A, true, pend.G != nullptr};
         int ntiles = nslices;
         for (int i = 0; i < 4; ++i) ntiles += need[i] ? 1 : 0;
         const CUtensorMap* maps[4] = {&mapU, &mapI, &mapGate, &mapG};
@@ -895,63 +935,25 @@ __global__ void __launch_bounds__(kGGComputeThreads + 32) gate_grad_local_ring_k
         // =============================== compute warps
         // slot, 16-row group, early (0) or late (1) 8 rows of the group
         const int tx = threadIdx.x & 63, ty = (threadIdx.x >> 6) & 1, hh = threadIdx.x >> 7;
-        constexpr int kHalf = kGG / 2;
-        const size_t stride = (size_t)H * M;
         auto csync = [] { asm volatile("bar.sync 1, 256;" ::: "memory"); };
         int it = 0;
         for (int t = blockIdx.x; t < total; t += gridDim.x, ++it) {
             const int s = it % nstage;
             const int bh = t % BH, b = bh / H, h = bh % H, ty0 = t / BH, t0 = ty0 * kGGTmaRows;
             const unsigned char* smem = smem0 + (size_t)s * stage_bytes;
-            const bool landed = mbar_wait(&bar_full[s], (it / nstage) & 1);
-            if (!landed) failed_s = 1;
+            if (!mbar_wait(&bar_full[s], (it / nstage) & 1)) failed_s = 1;     // (what is read then means nothing)
             const int n = ty0 * (kGGTmaRows / kGG) + ty;           // 16-row block of the sequence
-            const int rows = n < nblk ? min(kGG, T - n * kGG) : 0;
-            // row r (of this thread's 8), this thread's slot, of tile `tile`
-            auto at = [&](int tile, int r) {
-                const int row = ty * kGG + hh * kHalf + r, c = tx;
-                const unsigned char* p = smem + tile * kGGTileB + (c >> 5) * (kGGTileB / 2) + swz128(row, (c & 31) >> 2) + (c & 3) * 4;
-                return *reinterpret_cast<const float*>(p);
-            };
-            float x[kHalf], dI[kHalf], gt[kHalf];
-#pragma unroll
-            for (int i = 0; i < kHalf; ++i) { dI[i] = 0.f; x[i] = 0.f; gt[i] = 1.f; }
-            if (landed) {
-                for (int sl = 0; sl < nslices; ++sl) {
-#pragma unroll
-                    for (int i = 0; i < kHalf; ++i) dI[i] += at(4 + sl, i);
-                }
-                if (pend.pending_at(b, t0, h)) {
-                    // the time-reversed value_side runs left their row factor exp(-G_i) to this kernel
-#pragma unroll
-                    for (int i = 0; i < kHalf; ++i) dI[i] *= pend.reverse_factor(at(3, i));
-                }
-#pragma unroll
-                for (int i = 0; i < kHalf; ++i) {
-                    gt[i] = at(2, i);
-                    const float ii = gate_kind == GSA_GATE_A ? 1.f - gt[i] : at(1, i);      // 1 - a as the gate kernel formed it
-                    x[i] = at(0, i) - ii * dI[i];                                          // rows past the end: u = dI = 0
-                }
-            }
+            const int rows = n < nblk ? T - n * kGG - hh * kGGHalf : 0;
+            GateGradRows<KIND, WIDE> r;
+            r.read(smem, nslices, tx, ty, hh, pend.pending_at(b, t0, h));
             // the early half starts from the total of the late half of its group
-            const uint32_t starts = starts_among(cu, nseq, n * kGG + hh * kHalf, kHalf);
-            float tot = 0.f;
-#pragma unroll
-            for (int i = 0; i < kHalf; ++i)
-                if ((starts & ((2u << i) - 1)) == 0) tot += x[i];         // (up to the first token that begins a sequence)
-            if (hh == 1) late_half[ty][tx] = tot;
+            const uint32_t starts = starts_among(cu, nseq, n * kGG + hh * kGGHalf, kGGHalf);
+            if (hh == 1) late_half[ty][tx] = r.total(starts);
             csync();                              // (also: every thread has read its part of the stage)
             if (threadIdx.x == 0)
                 asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar_empty[s])) : "memory");
-            float run = hh == 0 ? late_half[ty][tx] : 0.f;
-            const size_t base = (((size_t)b * T + n * kGG + hh * kHalf) * H + h) * M + tx;
-#pragma unroll
-            for (int i = kHalf - 1; i >= 0; --i) {
-                run += x[i];
-                if ((starts >> i) & 1) run = 0.f;
-                if (hh * kHalf + i < rows)
-                    dgate[base + (size_t)i * stride] = gate_grad_out(run, dI[i], gt[i], gate_kind, inv_tau);
-            }
+            float* out = dgate + (((size_t)b * T + t0) * H + h) * M + (uint32_t)((ty * kGG + hh * kGGHalf) * H * M + tx);
+            const float run = r.write(hh == 0 ? late_half[ty][tx] : 0.f, starts, rows, out, (uint32_t)H * M, inv_tau);
             if (hh == 0 && n < nblk) blk_tot[((size_t)bh * nblk + n) * M + tx] = run;
             // (one thread reads the flag that the copy lane may raise at any time, so that all leave together)
             if (threadIdx.x == 0) stop_s = failed_s;
@@ -969,9 +971,9 @@ __global__ void __launch_bounds__(kGGComputeThreads + 32) gate_grad_local_ring_k
 
 // Adds what follows the block: dgate += carry (log gate) or carry / a (linear gate).  A thread
 // takes two slots of eight rows (half a block): threadIdx = (slot pair, block, half).
-template <int M>
+template <int M, int KIND>
 __global__ void __launch_bounds__(256) gate_grad_carry_kernel(
-    const float* gate, int gate_kind, float inv_tau, const float* blk_carry,
+    const float* gate, float inv_tau, const float* blk_carry,
     float* dgate, int T, int H, int nblk, const int* cu, int nseq) {
     follow_previous_grid();
     constexpr int kRows = kGG / 2;
@@ -979,28 +981,54 @@ __global__ void __launch_bounds__(256) gate_grad_carry_kernel(
     const int n = blockIdx.y * blockDim.y + threadIdx.y;
     if (n >= nblk) return;
     const int bh = blockIdx.x, b = bh / H, h = bh % H;
-    const int t0 = n * kGG + threadIdx.z * kRows;
-    const int rows = max(0, min(kRows, T - t0));
-    const size_t stride = (size_t)H * M;
-    const size_t base = (((size_t)b * T + t0) * H + h) * M + s;
+    // (a CTA's first element, and 32-bit offsets from there)
+    const int t_cta = blockIdx.y * blockDim.y * kGG, t0 = n * kGG + threadIdx.z * kRows;
+    const size_t first = (((size_t)b * T + t_cta) * H + h) * M;
+    const uint32_t stride = (uint32_t)H * M, off = (t0 - t_cta) * stride + s;
+    const int rows = T - t0;
     // (what follows the block reaches the rows after its last token that begins a sequence)
-    const int from = 32 - __clz(starts_among(cu, nseq, n * kGG, min(kGG, T - n * kGG))) - (int)threadIdx.z * kRows;
+    const int from = cu == nullptr ? 0 : 32 - __clz(starts_among(cu, nseq, n * kGG, min(kGG, T - n * kGG))) - (int)threadIdx.z * kRows;
     const float2 carry = *reinterpret_cast<const float2*>(blk_carry + ((size_t)bh * nblk + n) * M + s);
     float2 d[kRows], gt[kRows];
+    float* out = dgate + first;
+    const float* in = gate + first;
+    auto row = [&](int i) {
+        *reinterpret_cast<float2*>(out + (off + i * stride)) =
+            make_float2(d[i].x + gate_grad_carry(carry.x, gt[i].x, KIND, inv_tau), d[i].y + gate_grad_carry(carry.y, gt[i].y, KIND, inv_tau));
+    };
+    if (rows >= kRows && from <= 0) {
 #pragma unroll
-    for (int i = 0; i < kRows; ++i) {
-        d[i] = (i < rows) ? *reinterpret_cast<const float2*>(dgate + base + (size_t)i * stride) : make_float2(0.f, 0.f);
-        gt[i] = (i < rows && gate_kind != GSA_GATE_LOG_A) ? *reinterpret_cast<const float2*>(gate + base + (size_t)i * stride)
-                                                          : make_float2(1.f, 1.f);
+        for (int i = 0; i < kRows; ++i) {
+            d[i] = *reinterpret_cast<const float2*>(out + (off + i * stride));
+            if (KIND != GSA_GATE_LOG_A) gt[i] = *reinterpret_cast<const float2*>(in + (off + i * stride));
+        }
+#pragma unroll
+        for (int i = 0; i < kRows; ++i) row(i);
+        return;
     }
 #pragma unroll
     for (int i = 0; i < kRows; ++i)
         if (i < rows && i >= from) {
-            float2 out;
-            out.x = d[i].x + gate_grad_carry(carry.x, gt[i].x, gate_kind, inv_tau);
-            out.y = d[i].y + gate_grad_carry(carry.y, gt[i].y, gate_kind, inv_tau);
-            *reinterpret_cast<float2*>(dgate + base + (size_t)i * stride) = out;
+            d[i] = *reinterpret_cast<const float2*>(out + (off + i * stride));
+            gt[i] = KIND != GSA_GATE_LOG_A ? *reinterpret_cast<const float2*>(in + (off + i * stride)) : make_float2(1.f, 1.f);
+            row(i);
         }
+}
+template <int M, class... A>
+void launch_gate_carry(int gate_kind, dim3 grid, dim3 block, cudaStream_t st, const float* gate, A... rest) {
+    if (gate_kind == GSA_GATE_A) launch_after(gate_grad_carry_kernel<M, GSA_GATE_A>, grid, block, 0, st, gate, rest...);
+    else if (gate_kind == GSA_GATE_LOG_A) launch_after(gate_grad_carry_kernel<M, GSA_GATE_LOG_A>, grid, block, 0, st, gate, rest...);
+    else launch_after(gate_grad_carry_kernel<M, GSA_GATE_LOGITS>, grid, block, 0, st, gate, rest...);
+}
+// f(kind, wide) with both as types
+template <class F>
+cudaError_t with_gate_kind(int gate_kind, int wide, F&& f) {
+    auto kind = [&](auto w) {
+        if (gate_kind == GSA_GATE_A) return f(std::integral_constant<int, GSA_GATE_A>{}, w);
+        if (gate_kind == GSA_GATE_LOG_A) return f(std::integral_constant<int, GSA_GATE_LOG_A>{}, w);
+        return f(std::integral_constant<int, GSA_GATE_LOGITS>{}, w);
+    };
+    return wide ? kind(std::true_type{}) : kind(std::false_type{});
 }
 
 int gate_grad_blocks(int T) { return (T + kGG - 1) / kGG; }
@@ -1038,9 +1066,6 @@ cudaError_t launch_gate_grad(const float* u, const float* I, const float* dIk_pa
             const int stage_bytes = (4 + nsl) * kGGTileB;
             const int nstage = 2;
             const size_t smem = 1024 + (size_t)nstage * stage_bytes;
-            cudaError_t e = cudaFuncSetAttribute(gate_grad_local_ring_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)smem);
-            if (e != cudaSuccess) return e;
             static int sm_count = 0;
             if (sm_count == 0) {
                 int dev = 0;
@@ -1051,32 +1076,41 @@ cudaError_t launch_gate_grad(const float* u, const float* I, const float* dIk_pa
             const int BH = B * H, ntile = (T + kGGTmaRows - 1) / kGGTmaRows;
             const long long total = (long long)BH * ntile;
             const int ctas = (int)(total < sm_count ? total : sm_count);      // one persistent CTA per SM
-            launch_after(gate_grad_local_ring_kernel, ctas, kGGComputeThreads + 32, smem, st, mu, mi, mg, mG, mk, mv, nsk, nsv, gate_kind, inv_tau, blk_tot, dgate, T, H, BH, ntile, nstage, nblk,
-                pend, cu_seqlens, nseq, dev_status);
+            const cudaError_t e = with_gate_kind(gate_kind, pend.wide, [&](auto k, auto w) {
+                constexpr auto kernel = gate_grad_local_ring_kernel<decltype(k)::value, decltype(w)::value>;
+                const cudaError_t ready = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                if (ready != cudaSuccess) return ready;
+                return launch_after(gate_grad_local_ring_kernel<decltype(k)::value, decltype(w)::value>, ctas, kGGComputeThreads + 32, smem, st, mu, mi, mg, mG, mk, mv, nsk, nsv, inv_tau, blk_tot, dgate,
+                                    T, H, BH, ntile, nstage, nblk, pend, cu_seqlens, nseq, dev_status);
+            });
+            if (e != cudaSuccess) return e;
         } else if (staged) {
             const size_t smem = 1024 + (size_t)(4 + nsl) * kGGTileB;
-            cudaError_t e = cudaFuncSetAttribute(gate_grad_local_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)smem);
-            if (e != cudaSuccess) return e;
             dim3 tgrid(B * H, (T + kGGTmaRows - 1) / kGGTmaRows);
-            launch_after(gate_grad_local_tma_kernel, tgrid, 256, smem, st, mu, mi, mg, mG, mk, mv, nsk, nsv, gate_kind, inv_tau, blk_tot,
-                                                                dgate, T, H, nblk, pend, cu_seqlens, nseq, dev_status);
+            const cudaError_t e = with_gate_kind(gate_kind, pend.wide, [&](auto k, auto w) {
+                constexpr auto kernel = gate_grad_local_tma_kernel<decltype(k)::value, decltype(w)::value>;
+                const cudaError_t ready = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                if (ready != cudaSuccess) return ready;
+                return launch_after(gate_grad_local_tma_kernel<decltype(k)::value, decltype(w)::value>, tgrid, 256, smem, st, mu, mi, mg, mG, mk, mv, nsk, nsv, inv_tau, blk_tot, dgate, T, H, nblk, pend,
+                                    cu_seqlens, nseq, dev_status);
+            });
+            if (e != cudaSuccess) return e;
         } else {
             launch_after(gate_grad_local_kernel<64>, grid, block, 0, st, u, I, dIk_part, nsk, dIv_part, nsv, gate, gate_kind, inv_tau,
                                                                blk_tot, dgate, B, T, H, nblk, pend, cu_seqlens, nseq);
         }
         launch_after(gate_grad_scan_kernel<64>, B * H, dim3(64, 16), 0, st, blk_tot, dKT, KT, dVT, VT, d_k, d_v, nblk, T, cu_seqlens, nseq);
-        launch_after(gate_grad_carry_kernel<64>, grid, dim3(block.x, block.y, 2), 0, st, gate, gate_kind, inv_tau, blk_tot, dgate, T, H, nblk, cu_seqlens, nseq);
+        launch_gate_carry<64>(gate_kind, grid, dim3(block.x, block.y, 2), st, gate, inv_tau, blk_tot, dgate, T, H, nblk, cu_seqlens, nseq);
     } else if (M == 128) {
         launch_after(gate_grad_local_kernel<128>, grid, block, 0, st, u, I, dIk_part, nsk, dIv_part, nsv, gate, gate_kind, inv_tau,
                                                             blk_tot, dgate, B, T, H, nblk, pend, cu_seqlens, nseq);
         launch_after(gate_grad_scan_kernel<128>, B * H, dim3(128, 8), 0, st, blk_tot, dKT, KT, dVT, VT, d_k, d_v, nblk, T, cu_seqlens, nseq);
-        launch_after(gate_grad_carry_kernel<128>, grid, dim3(block.x, block.y, 2), 0, st, gate, gate_kind, inv_tau, blk_tot, dgate, T, H, nblk, cu_seqlens, nseq);
+        launch_gate_carry<128>(gate_kind, grid, dim3(block.x, block.y, 2), st, gate, inv_tau, blk_tot, dgate, T, H, nblk, cu_seqlens, nseq);
     } else {
         launch_after(gate_grad_local_kernel<32>, grid, block, 0, st, u, I, dIk_part, nsk, dIv_part, nsv, gate, gate_kind, inv_tau,
                                                            blk_tot, dgate, B, T, H, nblk, pend, cu_seqlens, nseq);
         launch_after(gate_grad_scan_kernel<32>, B * H, dim3(32, 16), 0, st, blk_tot, dKT, KT, dVT, VT, d_k, d_v, nblk, T, cu_seqlens, nseq);
-        launch_after(gate_grad_carry_kernel<32>, grid, dim3(block.x, block.y, 2), 0, st, gate, gate_kind, inv_tau, blk_tot, dgate, T, H, nblk, cu_seqlens, nseq);
+        launch_gate_carry<32>(gate_kind, grid, dim3(block.x, block.y, 2), st, gate, inv_tau, blk_tot, dgate, T, H, nblk, cu_seqlens, nseq);
     }
     return cudaGetLastError();
 }
