@@ -1009,30 +1009,26 @@ __global__ void __launch_bounds__(256) gate_grad_carry_kernel(
     // (what follows the block reaches the rows after its last token that begins a sequence)
     const int from = cu == nullptr ? 0 : 32 - __clz(starts_among(cu, nseq, n * kGG, min(kGG, T - n * kGG))) - (int)threadIdx.z * kRows;
     const float2 carry = *reinterpret_cast<const float2*>(blk_carry + ((size_t)bh * nblk + n) * M + s);
-    float2 d[kRows], gt[kRows];
     float* out = dgate + first;
     const float* in = gate + first;
-    auto row = [&](int i) {
+    auto load = [&](const float* p, int i) { return *reinterpret_cast<const float2*>(p + (off + i * stride)); };
+    auto add = [&](int i, float2 d, float2 gt) {
         *reinterpret_cast<float2*>(out + (off + i * stride)) =
-            make_float2(d[i].x + gate_grad_carry(carry.x, gt[i].x, KIND, inv_tau), d[i].y + gate_grad_carry(carry.y, gt[i].y, KIND, inv_tau));
+            make_float2(d.x + gate_grad_carry(carry.x, gt.x, KIND, inv_tau), d.y + gate_grad_carry(carry.y, gt.y, KIND, inv_tau));
     };
+    const float2 unused = make_float2(1.f, 1.f);           // (log gates: the carry goes as it is)
     if (rows >= kRows && from <= 0) {
+        float2 d[kRows], gt[kRows];
 #pragma unroll
         for (int i = 0; i < kRows; ++i) {
-            d[i] = *reinterpret_cast<const float2*>(out + (off + i * stride));
-            if (KIND != GSA_GATE_LOG_A) gt[i] = *reinterpret_cast<const float2*>(in + (off + i * stride));
+            d[i] = load(out, i);
+            gt[i] = KIND != GSA_GATE_LOG_A ? load(in, i) : unused;
         }
 #pragma unroll
-        for (int i = 0; i < kRows; ++i) row(i);
+        for (int i = 0; i < kRows; ++i) add(i, d[i], gt[i]);
         return;
     }
-#pragma unroll
-    for (int i = 0; i < kRows; ++i)
-        if (i < rows && i >= from) {
-            d[i] = *reinterpret_cast<const float2*>(out + (off + i * stride));
-            gt[i] = KIND != GSA_GATE_LOG_A ? *reinterpret_cast<const float2*>(in + (off + i * stride)) : make_float2(1.f, 1.f);
-            row(i);
-        }
+    for (int i = max(from, 0); i < min(rows, kRows); ++i) add(i, load(out, i), KIND != GSA_GATE_LOG_A ? load(in, i) : unused);
 }
 template <int M, class... A>
 void launch_gate_carry(int gate_kind, dim3 grid, dim3 block, cudaStream_t st, const float* gate, A... rest) {
