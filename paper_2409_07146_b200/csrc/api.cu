@@ -1091,7 +1091,7 @@ gsa_status_t gsa_out_norm_fwd(const gsa_params_t* params, const void* o, const f
 
 size_t gsa_out_norm_workspace_bytes(const gsa_params_t* params) {
     if (check_params(params, true) != GSA_OK) return 0;
-    return align_up(out_norm_bwd_parts((size_t)params->B * params->T) * params->H * params->d_v * sizeof(float), 256);
+    return align_up(out_norm_bwd_parts((size_t)params->B * params->T, params->H * params->d_v, params->io) * params->H * params->d_v * sizeof(float), 256);
 }
 
 gsa_status_t gsa_out_norm_bwd(const gsa_params_t* params, const void* o, const void* dy, const float* weight, float eps,

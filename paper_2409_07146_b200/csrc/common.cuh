@@ -314,7 +314,7 @@ cudaError_t launch_fused_pair(int mode, const void* xq1, const void* xk1, const 
 cudaError_t launch_swish_fwd(const void* const in[3], void* const out[3], const size_t n[3], int io, cudaStream_t st);
 cudaError_t launch_swish_bwd(const void* const x[3], void* const d[3], const size_t n[3], int io, cudaStream_t st);
 int out_norm_max_width(int io);
-size_t out_norm_bwd_parts(size_t rows);
+size_t out_norm_bwd_parts(size_t rows, int N, int io);
 cudaError_t launch_out_norm_fwd(const void* o, const float* weight, float eps, void* y, size_t rows, int N, int io,
                                 cudaStream_t st);
 cudaError_t launch_out_norm_bwd(const void* o, const void* dy, const float* weight, float eps, void* d_o, float* dw_part,

@@ -15,21 +15,34 @@
 namespace gsa {
 namespace {
 
-// 1 / (1 + exp(-x)); where all results are rounded to bfloat16, by the approximate reciprocal (2 ulp of fp32): the IEEE
+// exp(-x) by the hardware's base-2 exponential, as __expf, without its care for results below 2^-126: 1 is added to them
+__device__ __forceinline__ float exp_neg(float x) {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x * -1.4426950408889634f));
+    return r;
+}
+__device__ __forceinline__ float reciprocal_approx(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+// 1 / (1 + exp(-x)); where all results are rounded to bfloat16, by the approximate reciprocal (1 ulp of fp32): the IEEE
 // division is half of all instructions of these kernels (training step of the 2.7B model's layer, 4 x 1999 tokens: 736 us
 // with it in all of them, 652 without)
 template <typename IO>
 __device__ __forceinline__ float sigmoidf(float x);
 template <>
-__device__ __forceinline__ float sigmoidf<float>(float x) { return 1.f / (1.f + __expf(-x)); }
+__device__ __forceinline__ float sigmoidf<float>(float x) { return 1.f / (1.f + exp_neg(x)); }
 template <>
-__device__ __forceinline__ float sigmoidf<__nv_bfloat16>(float x) { return __fdividef(1.f, 1.f + __expf(-x)); }
-__device__ __forceinline__ float sigmoid_exact(float x) { return 1.f / (1.f + __expf(-x)); }
+__device__ __forceinline__ float sigmoidf<__nv_bfloat16>(float x) { return reciprocal_approx(1.f + exp_neg(x)); }
+__device__ __forceinline__ float sigmoid_exact(float x) { return 1.f / (1.f + exp_neg(x)); }
 __device__ __forceinline__ float swish_slope(float x, float sigmoid) { return sigmoid * (1.f + x * (1.f - sigmoid)); }
 
 // The feature map of q, k and v in one launch: blocks of kStream vectors a thread, all requested before the first is used
-// (one at a time, in a launch per tensor: 20 us for 41 MB in and out, 4.1 TB/s).
-constexpr int kStream = 4;
+// (one at a time, in a launch per tensor: 20 us for 41 MB in and out, 4.1 TB/s; three tensors of 41 MB, four vectors a thread held
+// as fp32 values, 47 us and 83 backward; held as they come, with the sigmoid in four instructions, 44 and 55; eight vectors, a
+// training step of the layer 604 -> 592).
+constexpr int kStream = 8;
 struct SwishSet { const void* in; void* out; size_t nvec; };
 struct SwishSets { SwishSet t[3]; };
 template <typename IO, bool BWD>
@@ -40,22 +53,25 @@ __global__ void __launch_bounds__(256) swish_kernel(const SwishSets sets) {
     const IO* in = static_cast<const IO*>(t.in);
     IO* out = static_cast<IO*>(t.out);
     const size_t i0 = (size_t)blockIdx.x * (kStream * 256) + threadIdx.x;
-    float x[kStream][V], g[BWD ? kStream : 1][V];
+    uint4 xv[kStream], gv[BWD ? kStream : 1];         // (as they come: half the registers of their values in fp32)
 #pragma unroll
     for (int j = 0; j < kStream; ++j)
         if (i0 + j * 256 < t.nvec) {
-            load_vec(in + (i0 + j * 256) * V, x[j]);
-            if (BWD) load_vec(out + (i0 + j * 256) * V, g[BWD ? j : 0]);
+            xv[j] = reinterpret_cast<const uint4*>(in)[i0 + j * 256];
+            if (BWD) gv[BWD ? j : 0] = reinterpret_cast<const uint4*>(out)[i0 + j * 256];
         }
 #pragma unroll
     for (int j = 0; j < kStream; ++j)
         if (i0 + j * 256 < t.nvec) {
+            float x[V], g[V];
+            load_vec(reinterpret_cast<const IO*>(&xv[j]), x);
+            if (BWD) load_vec(reinterpret_cast<const IO*>(&gv[BWD ? j : 0]), g);
 #pragma unroll
             for (int e = 0; e < V; ++e) {
-                const float s = sigmoidf<IO>(x[j][e]);
-                x[j][e] = BWD ? g[BWD ? j : 0][e] * swish_slope(x[j][e], s) : x[j][e] * s;
+                const float s = sigmoidf<IO>(x[e]);
+                x[e] = BWD ? g[e] * swish_slope(x[e], s) : x[e] * s;
             }
-            store_vec(out + (i0 + j * 256) * V, x[j]);
+            store_vec(out + (i0 + j * 256) * V, x);
         }
 }
 
@@ -123,20 +139,22 @@ __global__ void __launch_bounds__(512) out_norm_fwd_kernel(const IO* o, const fl
         }
 }
 
-// Backward: a CTA takes kRowsPerCta consecutive tokens, kTokens at a time (so that the weight gradient can be summed over
+// Backward: a CTA takes every gridDim.x-th pair of tokens (so that the weight gradient can be summed over
 // them in registers, one partial row per CTA; a second kernel adds the partial rows in order).  With x = Swish(o), g = w dy
 // and r = 1 / sqrt(mean(x^2) + eps):  d_o = r (g - x r^2 mean(g x)) Swish'(o) -- both means in one pass over the tokens'
-// values, which stay in registers as they came; sigmoids by the exact reciprocal whatever the io type, since the weight
-// gradient leaves in fp32.  One token at a time, two means after one another: 143 us at 8 K tokens of 2560
-// values (123 MB).
-constexpr int kRowsPerCta = 16;
+// values, which stay in registers as they came, with their sigmoids; these by the exact reciprocal whatever the io type, since
+// the weight gradient leaves in fp32.  Bound by instructions and the latency of a pair (loads, sums, barrier): two tokens in 64
+// registers let three CTAs of 320 threads share an SM.  8 K tokens of 2560 values (123 MB): one token at a time, two means after
+// one another 143 us; four tokens of one CTA per SM, each sigmoid formed twice, 86;
+// so, 60 (both kernels).
+constexpr int kBwdTokens = 2;
 template <typename IO>
-__global__ void __launch_bounds__(512) out_norm_bwd_kernel(const IO* o, const IO* dy,
+__global__ void __launch_bounds__(512, 2) out_norm_bwd_kernel(const IO* o, const IO* dy,
                                                            const float* weight, float eps, IO* d_o,
                                                            float* __restrict__ dw_part, int N, size_t rows) {
     follow_previous_grid();
     constexpr int V = IoTraits<IO>::kVec;
-    __shared__ float scratch[2][16][2 * kTokens];
+    __shared__ float scratch[2][16][2 * kBwdTokens];
     const int c = threadIdx.x * V;
     const bool own = c < N;
     float dw[V], w[V];
@@ -145,19 +163,18 @@ __global__ void __launch_bounds__(512) out_norm_bwd_kernel(const IO* o, const IO
         dw[e] = 0.f;
         w[e] = weight && own ? weight[c + e] : 1.f;
     }
-    for (int r0 = 0; r0 < kRowsPerCta; r0 += kTokens) {
-        const size_t row0 = (size_t)blockIdx.x * kRowsPerCta + r0;
-        if (row0 >= rows) break;
-        uint4 ov[kTokens], gv[kTokens];
+    int it = 0;
+    for (size_t row0 = (size_t)blockIdx.x * kBwdTokens; row0 < rows; row0 += (size_t)gridDim.x * kBwdTokens, ++it) {
+        uint4 ov[kBwdTokens], gv[kBwdTokens];
 #pragma unroll
-        for (int r = 0; r < kTokens; ++r)
+        for (int r = 0; r < kBwdTokens; ++r)
             if (own && row0 + r < rows) {
                 ov[r] = *reinterpret_cast<const uint4*>(o + (row0 + r) * N + c);
                 gv[r] = *reinterpret_cast<const uint4*>(dy + (row0 + r) * N + c);
             }
-        float sums[2 * kTokens];
+        float sums[2 * kBwdTokens], sg[kBwdTokens][V];
 #pragma unroll
-        for (int r = 0; r < kTokens; ++r) {
+        for (int r = 0; r < kBwdTokens; ++r) {
             float ss = 0.f, dot = 0.f;
             if (own && row0 + r < rows) {
                 float x[V], g[V];
@@ -165,7 +182,8 @@ __global__ void __launch_bounds__(512) out_norm_bwd_kernel(const IO* o, const IO
                 load_vec(reinterpret_cast<const IO*>(&gv[r]), g);
 #pragma unroll
                 for (int e = 0; e < V; ++e) {
-                    x[e] *= sigmoid_exact(x[e]);
+                    sg[r][e] = sigmoid_exact(x[e]);
+                    x[e] *= sg[r][e];
                     ss += x[e] * x[e];
                     dot += g[e] * w[e] * x[e];
                 }
@@ -173,9 +191,9 @@ __global__ void __launch_bounds__(512) out_norm_bwd_kernel(const IO* o, const IO
             sums[2 * r] = ss;
             sums[2 * r + 1] = dot;
         }
-        cta_sums(sums, scratch[(r0 / kTokens) & 1]);
+        cta_sums(sums, scratch[it & 1]);
 #pragma unroll
-        for (int r = 0; r < kTokens; ++r)
+        for (int r = 0; r < kBwdTokens; ++r)
             if (own && row0 + r < rows) {
                 const float inv = rsqrtf(sums[2 * r] / (float)N + eps);
                 const float mean = sums[2 * r + 1] * inv / (float)N;          // mean of g times x inv
@@ -184,7 +202,7 @@ __global__ void __launch_bounds__(512) out_norm_bwd_kernel(const IO* o, const IO
                 load_vec(reinterpret_cast<const IO*>(&gv[r]), g);
 #pragma unroll
                 for (int e = 0; e < V; ++e) {
-                    const float s = sigmoid_exact(x[e]), xhat = x[e] * s * inv;
+                    const float s = sg[r][e], xhat = x[e] * s * inv;
                     dw[e] += g[e] * xhat;
                     g[e] = (g[e] * w[e] - xhat * mean) * inv * swish_slope(x[e], s);
                 }
@@ -197,22 +215,24 @@ __global__ void __launch_bounds__(512) out_norm_bwd_kernel(const IO* o, const IO
             *reinterpret_cast<float4*>(dw_part + (size_t)blockIdx.x * N + c + e) = make_float4(dw[e], dw[e + 1], dw[e + 2], dw[e + 3]);
     }
 }
-// 32 columns a CTA, the partial rows dealt out over 16 groups of threads, in a fixed order (a thread a column: 26 us for 500
-// partial rows of 2560, all of it latency)
-__global__ void __launch_bounds__(512) out_norm_dw_kernel(const float* dw_part, float* __restrict__ dweight, int N,
+// 32 columns a CTA, the partial rows dealt out over 32 groups of threads, in a fixed order (all of it latency: a thread a
+// column 26 us for 500 partial rows of 2560, 16 groups 17, 32
+// groups 10)
+constexpr int kDwGroups = 32;
+__global__ void __launch_bounds__(32 * kDwGroups) out_norm_dw_kernel(const float* dw_part, float* __restrict__ dweight, int N,
                                                           int nparts) {
     follow_previous_grid();
-    __shared__ double group[16][32];
+    __shared__ double group[kDwGroups][32];
     const int c = blockIdx.x * 32 + threadIdx.x;
     double acc = 0.0;
     if (c < N) {
-#pragma unroll 8
-        for (int p = threadIdx.y; p < nparts; p += 16) acc += (double)dw_part[(size_t)p * N + c];
+#pragma unroll 16
+        for (int p = threadIdx.y; p < nparts; p += kDwGroups) acc += (double)dw_part[(size_t)p * N + c];
     }
     group[threadIdx.y][threadIdx.x] = acc;
     __syncthreads();
     if (threadIdx.y != 0 || c >= N) return;
-    for (int i = 1; i < 16; ++i) acc += group[i][threadIdx.x];
+    for (int i = 1; i < kDwGroups; ++i) acc += group[i][threadIdx.x];
     dweight[c] = (float)acc;
 }
 
@@ -243,7 +263,14 @@ cudaError_t launch_swish_bwd(const void* const x[3], void* const d[3], const siz
     return launch_swish<true>({{{x[0], d[0], n[0]}, {x[1], d[1], n[1]}, {x[2], d[2], n[2]}}}, io, st);
 }
 int out_norm_max_width(int io) { return 512 * (io == GSA_BF16 ? 8 : 4); }
-size_t out_norm_bwd_parts(size_t rows) { return (rows + kRowsPerCta - 1) / kRowsPerCta; }
+// CTAs of the backward, a partial row of the weight gradient each: as many as the GPU holds at 64 registers a thread, up to
+// eight per SM, and no more than there are pairs of tokens
+size_t out_norm_bwd_parts(size_t rows, int N, int io) {
+    const size_t pairs = (rows + kBwdTokens - 1) / kBwdTokens;
+    size_t per_sm = 1024 / token_threads(N, io);
+    per_sm = per_sm < 1 ? 1 : (per_sm > 8 ? 8 : per_sm);
+    return pairs < kSMs * per_sm ? pairs : kSMs * per_sm;
+}
 cudaError_t launch_out_norm_fwd(const void* o, const float* weight, float eps, void* y, size_t rows, int N, int io,
                                 cudaStream_t st) {
     const unsigned ctas = (unsigned)((rows + kTokens - 1) / kTokens), threads = token_threads(N, io);
@@ -256,14 +283,14 @@ cudaError_t launch_out_norm_fwd(const void* o, const float* weight, float eps, v
 }
 cudaError_t launch_out_norm_bwd(const void* o, const void* dy, const float* weight, float eps, void* d_o, float* dw_part,
                                 float* dweight, size_t rows, int N, int io, cudaStream_t st) {
-    const unsigned parts = (unsigned)out_norm_bwd_parts(rows), threads = token_threads(N, io);
+    const unsigned parts = (unsigned)out_norm_bwd_parts(rows, N, io), threads = token_threads(N, io);
     if (io == GSA_BF16)
         launch_after(out_norm_bwd_kernel<__nv_bfloat16>, parts, threads, 0, st, (const __nv_bfloat16*)o, (const __nv_bfloat16*)dy,
                      weight, eps, (__nv_bfloat16*)d_o, dweight ? dw_part : nullptr, N, rows);
     else
         launch_after(out_norm_bwd_kernel<float>, parts, threads, 0, st, (const float*)o, (const float*)dy, weight, eps, (float*)d_o,
                      dweight ? dw_part : nullptr, N, rows);
-    if (dweight != nullptr) launch_after(out_norm_dw_kernel, (N + 31) / 32, dim3(32, 16), 0, st, dw_part, dweight, N, (int)parts);
+    if (dweight != nullptr) launch_after(out_norm_dw_kernel, (N + 31) / 32, dim3(32, kDwGroups), 0, st, dw_part, dweight, N, (int)parts);
     return cudaGetLastError();
 }
 
