@@ -73,9 +73,17 @@ class Params:
             object.__setattr__(self, "_c", made)
         return made
 
+    def _made_at(self) -> int:
+        """The address of that struct where it is made once (0 otherwise)."""
+        at = self.__dict__.get("_at")
+        if at is None:
+            at = 0 if self.cu_seqlens is not None else ctypes.addressof(self._made_c())
+            object.__setattr__(self, "_at", at)
+        return at
+
     def __getstate__(self):
         # (the C struct neither travels nor is copied)
-        return {n: x for n, x in self.__dict__.items() if n != "_c"}
+        return {n: x for n, x in self.__dict__.items() if n not in ("_c", "_at")}
 
     def c(self) -> _CParams:
         return _CParams(self.B, self.T, self.H, self.d_k, self.d_v, self.m,
@@ -169,8 +177,18 @@ def load_library():
     lib.gsa_out_norm_bwd.restype = ctypes.c_int
     lib.gsa_release_streams.argtypes = []
     lib.gsa_release_streams.restype = ctypes.c_int
+    from . import _native
+    _native.set_library(ctypes.cast(lib.gsa_decode_step, vp).value)
+    global _decode_step
+    _decode_step = _native.decode_step
     _lib = lib
     return lib
+
+
+def _decode_step(*args):
+    """Replaced by _native.decode_step when the library is loaded."""
+    load_library()
+    return _decode_step(*args)
 
 
 def _ptr(t, dtype=None, shape=None, name="tensor"):
@@ -287,6 +305,14 @@ def gsa_bwd(p: Params, q, k, v, gate, dO, K0=None, V0=None, ok_saved=None, dKT=N
 
 def gsa_decode_step(p: Params, q, k, v, gate, Kstate, Vstate, o=None):
     """One recurrent step for p.B sequences; Kstate/Vstate are updated in place.  Returns o."""
+    if o is not None:
+        at = p._made_at()
+        code = _decode_step(at, q, k, v, gate, Kstate, Vstate, o) if at else None
+        if code == 0:
+            return o
+        if code is not None:
+            raise GsaError(code, "gsa_decode_step")
+    # (not a plain call, or one that allocates: checked and worded here)
     io = p.io_dtype
     qk, vv, mm = (p.B, p.H, p.d_k), (p.B, p.H, p.d_v), (p.B, p.H, p.m)
     if o is None:

@@ -1,4 +1,5 @@
-"""Builds libgsa.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a.
+"""Builds libgsa.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and _native.so, through which the binding takes
+torch tensors into its decode step.
 
     python -m paper_2409_07146_b200.build [--force] [--verbose]
 
@@ -17,6 +18,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libgsa.so")
+NATIVE = os.path.join(HERE, "_native.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -29,11 +31,26 @@ def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
+def _build_native() -> None:
+    import sysconfig
+
+    import torch
+    from torch.utils import cpp_extension
+    tmp = NATIVE + ".tmp.%d" % os.getpid()
+    include = [os.path.join(ROOT, "include"), sysconfig.get_paths()["include"], "/usr/local/cuda/include", *cpp_extension.include_paths()]
+    lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
+                           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI), *["-I" + d for d in include],
+                           os.path.join(CSRC, "binding_native.cpp"), "-o", tmp, "-L" + lib, "-ltorch_python", "-ltorch_cpu", "-lc10_cuda",
+                           "-lc10"])
+    os.replace(tmp, NATIVE)
+
+
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(NATIVE):
         return True
-    t = os.path.getmtime(LIB)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + \
+    t = min(os.path.getmtime(LIB), os.path.getmtime(NATIVE))
+    deps = sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.cpp")) + \
         glob.glob(os.path.join(ROOT, "include", "*.h")) + [os.path.abspath(__file__)]
     return any(os.path.getmtime(d) > t for d in deps)
 
@@ -54,6 +71,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
             cmd.insert(1, "-Xptxas=-v")
         procs.append((src, subprocess.Popen(cmd)))
         objs.append(obj)
+    _build_native()
     for src, pr in procs:
         if pr.wait() != 0:
             raise RuntimeError(f"nvcc failed on {src}")
