@@ -73,19 +73,28 @@ __device__ __forceinline__ void follow_previous_grid() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+struct ClusterGrid { dim3 grid, cluster; };
 template <typename... P, typename... A>
-cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+cudaError_t launch_after(void (*kernel)(P...), ClusterGrid in, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
+    cfg.gridDim = in.grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = in.cluster.x;
+    attr[1].val.clusterDim.y = in.cluster.y;
+    attr[1].val.clusterDim.z = in.cluster.z;
+    cfg.attrs = attr;
+    cfg.numAttrs = in.cluster.x * in.cluster.y * in.cluster.z > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+    return launch_after(kernel, ClusterGrid{grid, dim3(1, 1, 1)}, block, smem, st, static_cast<A&&>(args)...);
 }
 
 // ---- arguments of the two chunk primitives (both passes, forward and time-reversed) ----

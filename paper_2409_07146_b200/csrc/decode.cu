@@ -195,7 +195,9 @@ decode_step_kernel(const IO* __restrict__ q, const IO* __restrict__ k, const IO*
 // that one sequence uses more than H SMs.  A step of one CTA per pair is bound by the latency of its chain -- K rows in
 // batches, logits, softmax, V rows in batches, sums -- and by what one SM can pull: 512 KB at d = 512, 9.6 us a launch
 // where 4 pairs keep 4 SMs busy.  Here every row of both memories is requested at once, before anything is used; the CTAs
-// exchange the M logits and the partial output rows through distributed shared memory (two cluster barriers).
+// exchange the M logits and the partial output rows through distributed shared memory (two cluster barriers).  The steps
+// of a stack of layers follow one another: each is placed while the one before it drains (24 layers of 4 pairs
+// of d = 512: 150 -> 118 us as calls, 111 -> 107 in a graph).
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 // the word at the same place of CTA `rank`'s shared memory <- x
@@ -208,10 +210,11 @@ __device__ __forceinline__ void store_to_rank(float* local, unsigned rank, float
 
 template <typename IO, int DK, int DV, int RPW>
 __global__ void __launch_bounds__(kDecodeWarps * 32)
-decode_split_kernel(const IO* __restrict__ q, const IO* __restrict__ k, const IO* __restrict__ v,
-                    const void* __restrict__ gate_raw, int M, int gate_bf16, int gate_row_of_head, int feature_map,
-                    int gate_kind, float inv_tau, float scale, int act, float* __restrict__ Ks, float* __restrict__ Vs,
+decode_split_kernel(const IO* q, const IO* k, const IO* v,
+                    const void* gate_raw, int M, int gate_bf16, int gate_row_of_head, int feature_map,
+                    int gate_kind, float inv_tau, float scale, int act, float* Ks, float* Vs,
                     IO* __restrict__ o) {
+    follow_previous_grid();
     const int C = M / (kDecodeWarps * RPW);                     // CTAs of the cluster, M <= 128, C <= 8
     const size_t pair = blockIdx.x / C;
     const int rank = blockIdx.x % C, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -320,18 +323,8 @@ template <typename IO, int DK, int DV, int RPW>
 static cudaError_t launch_decode_split(const gsa_params_t& p, const IO* q, const IO* k, const IO* v, const float* gate,
                                        float* Ks, float* Vs, IO* o, cudaStream_t st) {
     const unsigned C = (unsigned)(p.m / (kDecodeWarps * RPW));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)p.B * (unsigned)p.H * C);
-    cfg.blockDim = dim3(kDecodeWarps * 32);
-    cfg.stream = st;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = C;
-    attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, decode_split_kernel<IO, DK, DV, RPW>, q, k, v, static_cast<const void*>(gate), (int)p.m,
+    return launch_after(decode_split_kernel<IO, DK, DV, RPW>, ClusterGrid{dim3((unsigned)p.B * (unsigned)p.H * C), dim3(C, 1, 1)},
+                        dim3(kDecodeWarps * 32), 0, st, q, k, v, static_cast<const void*>(gate), (int)p.m,
                               (int)(p.gate_dtype == GSA_BF16), (int)(p.gate_broadcast ? p.H : 0), (int)p.feature_map,
                               (int)p.gate_kind, p.tau > 0.f ? 1.f / p.tau : 0.f, p.scale, (int)p.slot_act, Ks, Vs, o);
 }
