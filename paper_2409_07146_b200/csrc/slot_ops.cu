@@ -1272,21 +1272,21 @@ cudaError_t launch_column_sum(const float* in, float* part, float* out, size_t r
 }
 
 // ------------------------------------------------------------------ gate tensor in bfloat16
-__global__ void widen_bf16_kernel(const __nv_bfloat16* in, float* __restrict__ out, size_t n) {
+// eight values a thread (both tensors start on 16 bytes); two at a time, 15 MB took 8.7 us
+__global__ void __launch_bounds__(256) widen_bf16_kernel(const __nv_bfloat16* in, float* __restrict__ out, size_t n) {
     follow_previous_grid();
-    for (size_t i = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * 2; i < n; i += (size_t)gridDim.x * blockDim.x * 2) {
-        if (i + 1 < n) {
-            const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(in + i));
-            *reinterpret_cast<float2*>(out + i) = f;
-        } else {
-            out[i] = __bfloat162float(in[i]);
-        }
+    const size_t i = ((size_t)blockIdx.x * 256 + threadIdx.x) * 8;
+    if (i + 8 <= n) {
+        float x[8];
+        load_vec(in + i, x);
+        *reinterpret_cast<float4*>(out + i) = make_float4(x[0], x[1], x[2], x[3]);
+        *reinterpret_cast<float4*>(out + i + 4) = make_float4(x[4], x[5], x[6], x[7]);
+    } else {
+        for (size_t j = i; j < n; ++j) out[j] = __bfloat162float(in[j]);
     }
 }
 cudaError_t launch_widen_bf16(const void* in, float* out, size_t n, cudaStream_t st) {
-    const size_t pairs = (n + 1) / 2;
-    const unsigned blocks = (unsigned)((pairs + 255) / 256 < 148 * 32 ? (pairs + 255) / 256 : 148 * 32);
-    launch_after(widen_bf16_kernel, blocks ? blocks : 1, 256, 0, st, static_cast<const __nv_bfloat16*>(in), out, n);
+    launch_after(widen_bf16_kernel, (unsigned)((n + 2047) / 2048), 256, 0, st, static_cast<const __nv_bfloat16*>(in), out, n);
     return cudaGetLastError();
 }
 
