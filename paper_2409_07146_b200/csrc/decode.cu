@@ -5,7 +5,8 @@
 // 8 warps owns one pair; a warp owns a memory row at a time, with 16-byte accesses that
 // cover the row contiguously (coalesced); rows are loaded in batches before any is used so
 // that several 512-byte requests per warp are in flight.  The key memory is updated and
-// read first (slot logits), then the softmax, then the value memory is updated and summed.
+// read first (slot logits), then the softmax, then the value memory is updated and summed.  A step is placed while the launch
+// before it drains: 24 layers of one sequence, 32 heads of 128, 148 -> 105 us as calls; 256 sequences, one layer 165.5 -> 163.1.
 #include "common.cuh"
 
 namespace gsa {
@@ -81,9 +82,10 @@ __device__ __forceinline__ void decode_gate(const void* gate_raw, size_t gi, int
 
 template <typename IO, int DK, int DV, int M>
 __global__ void __launch_bounds__(kDecodeWarps * 32)
-decode_step_kernel(const IO* __restrict__ q, const IO* __restrict__ k, const IO* __restrict__ v,
-                   const void* __restrict__ gate_raw, int gate_bf16, int gate_row_of_head, int feature_map, int gate_kind, float inv_tau, float scale, int act,
-                   float* __restrict__ Ks, float* __restrict__ Vs, IO* __restrict__ o) {
+decode_step_kernel(const IO* q, const IO* k, const IO* v,
+                   const void* gate_raw, int gate_bf16, int gate_row_of_head, int feature_map, int gate_kind, float inv_tau, float scale, int act,
+                   float* Ks, float* Vs, IO* __restrict__ o) {
+    follow_previous_grid();
     constexpr int RPW = M / kDecodeWarps;  // memory rows per warp
     const size_t pair = blockIdx.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -348,11 +350,11 @@ static cudaError_t launch_decode_m(const gsa_params_t& p, const IO* q, const IO*
     const int is_log = p.gate_kind;
     const float inv_tau = p.tau > 0.f ? 1.f / p.tau : 0.f;
     if (p.m == 128)
-        decode_step_kernel<IO, DK, DV, 128><<<pairs, kDecodeWarps * 32, 0, st>>>(q, k, v, gate, p.gate_dtype == GSA_BF16, p.gate_broadcast ? p.H : 0, p.feature_map, is_log, inv_tau, p.scale, p.slot_act, Ks, Vs, o);
+        launch_after(decode_step_kernel<IO, DK, DV, 128>, pairs, kDecodeWarps * 32, 0, st, q, k, v, gate, p.gate_dtype == GSA_BF16, p.gate_broadcast ? p.H : 0, p.feature_map, is_log, inv_tau, p.scale, p.slot_act, Ks, Vs, o);
     else if (p.m == 64)
-        decode_step_kernel<IO, DK, DV, 64><<<pairs, kDecodeWarps * 32, 0, st>>>(q, k, v, gate, p.gate_dtype == GSA_BF16, p.gate_broadcast ? p.H : 0, p.feature_map, is_log, inv_tau, p.scale, p.slot_act, Ks, Vs, o);
+        launch_after(decode_step_kernel<IO, DK, DV, 64>, pairs, kDecodeWarps * 32, 0, st, q, k, v, gate, p.gate_dtype == GSA_BF16, p.gate_broadcast ? p.H : 0, p.feature_map, is_log, inv_tau, p.scale, p.slot_act, Ks, Vs, o);
     else
-        decode_step_kernel<IO, DK, DV, 32><<<pairs, kDecodeWarps * 32, 0, st>>>(q, k, v, gate, p.gate_dtype == GSA_BF16, p.gate_broadcast ? p.H : 0, p.feature_map, is_log, inv_tau, p.scale, p.slot_act, Ks, Vs, o);
+        launch_after(decode_step_kernel<IO, DK, DV, 32>, pairs, kDecodeWarps * 32, 0, st, q, k, v, gate, p.gate_dtype == GSA_BF16, p.gate_broadcast ? p.H : 0, p.feature_map, is_log, inv_tau, p.scale, p.slot_act, Ks, Vs, o);
     return cudaGetLastError();
 }
 
