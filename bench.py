@@ -78,7 +78,7 @@ def kernel_algorithmic_bytes(label: str, w: W.Workload) -> int:
     # bytes per token-head row on the tensor-core path: fp32 [.., m] tensors are 4m, a decayed
     # bf16 operand row [high | residual] is 4m too
     table = {
-        "gate_cumsum": 16 * m,                                       # gate -> G, I, I exp(-G)
+        "gate_cumsum": 12 * m,                                       # gate -> G, I exp(-G)
         "pass1_value_side": 2 * w.d_k * e + 4 * m + 4 * m * nsk,     # q, k, I exp(-G) -> slices of o'
         "slot_softmax": 4 * m * nsk + 12 * m,                        # slices, G -> o', p exp(G)
         "pass2_key_side": 2 * w.d_v * e + 8 * m,                     # v, two decayed rows -> o

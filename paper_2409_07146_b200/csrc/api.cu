@@ -281,13 +281,25 @@ cudaError_t key_side(const gsa_params_t& p, const KeySideArgs& a, int reverse, c
     return launch_key_side_simt(a, p.io, p.m, reverse, st);
 }
 
+// Is 1 - a, in fp32, left out of the gate kernel's products?  On the tensor cores with 64 slots only the general scans read it,
+// which form the rows of their pairs themselves -- and the gate gradient, but where the gate tensor holds a it takes 1 - a
+// from there.  A quarter of the kernel's bytes: B = 4, T = 4096, 32 heads 95 -> 78 us, T = 32768, 16 heads 94 -> 78.
+bool leaves_input_gate(const gsa_params_t& p, bool gate_gradient_follows) {
+    return use_tc(p) && !use_wide(p) && p.gate_kind != GSA_GATE_ABC && (p.gate_kind == GSA_GATE_A || !gate_gradient_follows);
+}
+InputGate input_gate_of(const gsa_params_t& p, const float* gate, bool left_out) {
+    return left_out ? InputGate{gate, p.gate_kind, inv_tau(p)} : InputGate{};
+}
+
 // the gate kernel: G, 1 - a, the decayed rows and the strong-decay flags (cleared by the caller)
-cudaError_t gate_products(const gsa_params_t& p, Segments segs, const float* gate, const Workspace& w, cudaStream_t st) {
+// (input_gate = false: 1 - a is left out, see leaves_input_gate)
+cudaError_t gate_products(const gsa_params_t& p, Segments segs, const float* gate, const Workspace& w, bool input_gate,
+                          cudaStream_t st) {
     if (use_wide(p))
         return launch_gate_cumsum_wide(gate, p.gate_kind, inv_tau(p), w.G, w.I, w.E, p.B, p.T, p.H, w.strong, segs.n, segs.t,
                                        w.Id, st, p.cu_seqlens, p.nseq);
     return launch_gate_cumsum(gate, p.gate_kind, inv_tau(p), w.G, w.I, p.B, p.T, p.H, p.m, chunk_of(p), w.strong, segs.n,
-                              segs.t, w.Id, p.io == GSA_BF16, st, p.cu_seqlens, p.nseq);
+                              segs.t, w.Id, p.io == GSA_BF16, st, p.cu_seqlens, p.nseq, input_gate ? 0 : 1);
 }
 // the row factors that the tensor-core value_side scans leave to the slot kernels
 PendingDecay pending_decay(const gsa_params_t& p, Segments segs, const Workspace& w) {
@@ -302,10 +314,10 @@ PendingDecay pending_decay(const gsa_params_t& p, Segments segs, const Workspace
 struct StateSet { const void* x; const float* w; const void* wd; float* end; };
 // logdecay (nullable; forward runs): receives the segments' log-decay [B,nseg,H,m].
 cudaError_t state_scans(const gsa_params_t& p, Segments segs, StateSet ks, StateSet vs, const Workspace& w, int reverse,
-                        float* logdecay, cudaStream_t st, int32_t* dev_status) {
+                        float* logdecay, InputGate input_gate, cudaStream_t st, int32_t* dev_status) {
     ValueSideArgs a[2] = {{ks.x, ks.x, ks.w, w.G, nullptr, ks.end, nullptr, p.B, p.T, p.H, p.d_k, ks.wd, 1},
                           {vs.x, vs.x, vs.w, w.G, nullptr, vs.end, nullptr, p.B, p.T, p.H, p.d_v, vs.wd, 1}};
-    for (ValueSideArgs& x : a) { x.nseg = segs.n; x.tseg = segs.t; x.E = w.E; }
+    for (ValueSideArgs& x : a) { x.nseg = segs.n; x.tseg = segs.t; x.E = w.E; x.input_gate = input_gate; }
     if (use_wide(p)) {
         if (logdecay != nullptr) {
             const cudaError_t e = launch_segment_logdecay(w.G, logdecay, p.B, p.T, p.H, p.m, segs.n, segs.t, log_gate_chunk(p), st);
@@ -578,11 +590,13 @@ gsa_status_t fwd_core(const CallParams* params, int m_active, const void* q, con
 
     const Segments segs = segments_of(p);
     const int nseg = segs.n, tseg = segs.t;
+    const bool left_out = leaves_input_gate(p, save_gate);
+    const InputGate input_gate = input_gate_of(p, gate, left_out);
     GSA_CUDA(cudaMemsetAsync(w.strong, 0, sizeof(int) * (size_t)p.B * p.H * nseg, st));
     if (p.gate_kind == GSA_GATE_ABC)      // no decay, write weights from the cumulative softmax of the scores
         GSA_LAUNCH("abc_write", launch_abc_write(gate, w.G, w.I, w.Id, p.B, p.T, p.H, p.m, st));
     else
-        GSA_LAUNCH("gate_cumsum", gate_products(p, segs, gate, w, st));
+        GSA_LAUNCH("gate_cumsum", gate_products(p, segs, gate, w, !left_out, st));
     float* ok = ok_save;      // the scaled logits leave the softmax kernel only if the caller keeps them
     // the pipelined kernels leave the row factor of the pass-1 sums to the softmax kernel
     const PendingDecay pend = pending_decay(p, segs, w);
@@ -592,7 +606,7 @@ gsa_status_t fwd_core(const CallParams* params, int m_active, const void* q, con
         // first pass: every segment from empty memories, for its end memories alone; then the start
         // memories of all segments, and the final memories, by a scan over the segments
         GSA_LAUNCH("segment_states", state_scans(p, segs, StateSet{k, w.I, w.Id, w.Kloc}, StateSet{v, w.I, w.Id, w.Vloc}, w, 0,
-                                                  w.seg_decay, st, dev_status));
+                                                  w.seg_decay, input_gate, st, dev_status));
         // (when the backward is to reuse them, the final memories land in the saved block first)
         float* KTc = save_gate ? w.KT : KT;
         float* VTc = save_gate ? w.VT : VT;
@@ -608,6 +622,7 @@ gsa_status_t fwd_core(const CallParams* params, int m_active, const void* q, con
     // pass 1: o' = GLA(q, k, 1-a) with the decay on the slot (value) side
     ValueSideArgs a1{q, k, w.I, w.G, Kin, Kout, w.okpart, p.B, p.T, p.H, p.d_k, w.Id};
     a1.nseg = nseg; a1.tseg = tseg; a1.E = w.E;
+    if (nseg == 1) a1.input_gate = input_gate;       // (several segments: the state runs have been there)
     // pass 2: o = GLA(softmax(o'), 1-a, v) with the decay on the slot (key) side
     KeySideArgs a2{w.p, w.I, w.G, v, Vin, Vout, o, p.B, p.T, p.H, p.d_v, w.Pd, w.Id};
     a2.nseg = nseg; a2.tseg = tseg; a2.E = w.E;
@@ -752,12 +767,14 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
     // the right for the reversed ones.
     const Segments segs = segments_of(p);
     const int nseg = segs.n, tseg = segs.t;
+    const bool left_out = !gate_is_saved && leaves_input_gate(p, true);
+    const InputGate input_gate = input_gate_of(p, gate, left_out);
     if (!gate_is_saved) {      // (a forward of the same call left the gate kernel's products otherwise)
         GSA_CUDA(cudaMemsetAsync(w.strong, 0, sizeof(int) * (size_t)p.B * p.H * nseg, st));
         if (p.gate_kind == GSA_GATE_ABC)
             GSA_LAUNCH("abc_write", launch_abc_write(gate, w.G, w.I, w.Id, p.B, p.T, p.H, p.m, st));
         else
-            GSA_LAUNCH("gate_cumsum", gate_products(p, segs, gate, w, st));
+            GSA_LAUNCH("gate_cumsum", gate_products(p, segs, gate, w, !left_out, st));
     }
     const float* ok = ok_saved;
     const PendingDecay pend = pending_decay(p, segs, w);
@@ -771,7 +788,7 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
         KTout = nullptr; VTout = nullptr;
     } else if (nseg > 1) {
         GSA_LAUNCH("segment_states", state_scans(p, segs, StateSet{k, w.I, w.Id, w.Kloc}, StateSet{v, w.I, w.Id, w.Vloc}, w, 0,
-                                                  w.seg_decay, st, dev_status));
+                                                  w.seg_decay, input_gate, st, dev_status));
         GSA_LAUNCH("segment_combine", launch_segment_combine(w.seg_decay, {w.Kloc, K0, w.Kstart, KTout, p.d_k}, {w.Vloc, V0, w.Vstart, VTout, p.d_v}, p.B,
                                                              p.H, p.m, nseg, 0, st));
         Kin = w.Kstart; Vin = w.Vstart;
@@ -780,6 +797,7 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
     if (ok == nullptr) {  // recompute pass 1 and its logits
         ValueSideArgs a1{q, k, w.I, w.G, Kin, nullptr, w.okpart, p.B, p.T, p.H, p.d_k, w.Id};
         a1.nseg = nseg; a1.tseg = tseg; a1.E = w.E;
+        if (nseg == 1) a1.input_gate = input_gate;
         GSA_LAUNCH("pass1_value_side", value_side(p, a1, 0, w.strong, st, dev_status));
         GSA_LAUNCH("slot_softmax", launch_slot_softmax_fwd(w.okpart, s.k, p.scale, p.slot_act, w.ok, w.p, p.B, p.T * p.H, p.m, pend.G,
                                                            nullptr, pend, st, m_active));
@@ -788,6 +806,7 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
     // gradient w.r.t. the pass-2 queries p: the pass-1 form on (dO, v, 1-a); carries V~
     ValueSideArgs adp{dO, v, w.I, w.G, Vin, VTout, w.dppart, p.B, p.T, p.H, p.d_v, w.Id};
     adp.nseg = nseg; adp.tseg = tseg; adp.E = w.E;
+    if (nseg == 1 && ok_saved != nullptr) adp.input_gate = input_gate;      // (otherwise the scans before it have been there)
     // dq: the pass-2 form on (dz, 1-a, k); carries K~
     KeySideArgs adq{w.dz, w.I, w.G, k, Kin, KTout, dq, p.B, p.T, p.H, p.d_k, w.Zd, w.Id};
     adq.nseg = nseg; adq.tseg = tseg; adq.E = w.E;
@@ -859,7 +878,7 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
         // reversed scans of every segment from empty states, for their end states alone; then the states
         // entering every segment, and dK0 / dV0, by a scan over the segments from the last one down
         GSA_LAUNCH("segment_rev_states", state_scans(p, segs, StateSet{q, w.dz, w.Zd, w.Kloc}, StateSet{dO, w.p, w.Pd, w.Vloc}, w,
-                                                      1, nullptr, st, dev_status));
+                                                      1, nullptr, InputGate{}, st, dev_status));
         GSA_LAUNCH("segment_combine", launch_segment_combine(w.seg_decay, {w.Kloc, dKT, w.dKend, dK0, p.d_k}, {w.Vloc, dVT, w.dVend, dV0, p.d_v}, p.B,
                                                              p.H, p.m, nseg, 1, st));
         dKin = w.dKend; dVin = w.dVend;
@@ -1056,8 +1075,9 @@ gsa_status_t gsa_shard_states(const gsa_params_t* params, const void* k, const v
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // one "segment" per batch element: the whole shard from empty memories, end memories only
     GSA_CUDA(cudaMemsetAsync(w.strong, 0, sizeof(int) * (size_t)p.B * p.H, st));
-    GSA_LAUNCH("gate_cumsum", gate_products(p, Segments{1, p.T}, gate, w, st));
-    GSA_LAUNCH("segment_states", state_scans(p, Segments{1, p.T}, StateSet{k, w.I, w.Id, KT}, StateSet{v, w.I, w.Id, VT}, w, 0, logdecay, st,
+    GSA_LAUNCH("gate_cumsum", gate_products(p, Segments{1, p.T}, gate, w, !leaves_input_gate(p, false), st));
+    GSA_LAUNCH("segment_states", state_scans(p, Segments{1, p.T}, StateSet{k, w.I, w.Id, KT}, StateSet{v, w.I, w.Id, VT}, w, 0, logdecay,
+                                              input_gate_of(p, gate, leaves_input_gate(p, false)), st,
                                               dev_status));
     return GSA_OK;
 }

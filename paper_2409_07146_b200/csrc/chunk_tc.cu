@@ -11,7 +11,9 @@ value_side_general_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid
                           const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapG,
                           const __grid_constant__ CUtensorMap mapO, const __grid_constant__ ValueSideArgs a,
                           const int* __restrict__ strong_flag, int32_t* dev_status) {
-    if (strong_flag[blockIdx.x] != 0) value_side_general<REV>(mapQ, mapK, mapW, mapG, mapO, a, dev_status, blockIdx.y);
+    if (strong_flag[blockIdx.x] == 0) return;
+    if (!REV) write_input_gate(a);
+    value_side_general<REV>(mapQ, mapK, mapW, mapG, mapO, a, dev_status, blockIdx.y);
 }
 template <bool REV>
 __global__ void __launch_bounds__(kScanThreads, 1)

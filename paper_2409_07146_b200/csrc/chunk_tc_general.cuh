@@ -35,6 +35,47 @@ namespace {
 using namespace tc;
 using namespace tcchunk;
 
+// The rows of 1 - a of a flagged pair's moderate chunks, as the gate kernel forms them, where it has left them out
+// (InputGate).  Every CTA that is about to read them writes them all -- the same values -- and reads its own.  A warp a chunk.
+// (All chunks, strong ones too: 32 K tokens of strong gates, 16 heads, 1279 -> 1517 us.)
+__device__ __forceinline__ void write_input_gate(const ValueSideArgs& a) {
+    if (a.input_gate.gate == nullptr) return;
+    constexpr int kBatch = 8;
+    const ScanSpan span = scan_span(blockIdx.x, a.H, a.T, a.nseg, a.tseg);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const size_t stride = (size_t)a.H * kM;
+    for (int t0 = span.t0 + warp * kCT; t0 < span.t_end; t0 += (int)(blockDim.x >> 5) * kCT) {
+        const int rows = min(kCT, span.t_end - t0);
+        const size_t first = (((size_t)span.b * a.T + t0) * a.H + span.h) * kM;
+        // (clearly below the bound that the gate kernel compared the exact sum with: G is that sum to an ulp)
+        const float2 g = *reinterpret_cast<const float2*>(a.G + first + (rows - 1) * stride + 2 * lane);
+        if (__any_sync(0xffffffffu, fminf(g.x, g.y) < kFactorisedDecayMin - 0.01f)) continue;
+        const float* gate = a.input_gate.gate + first + (lane & 15) * 4;
+        float* out = const_cast<float*>(a.w) + first + (lane & 15) * 4;
+        for (int r0 = lane >> 4; r0 < rows; r0 += 2 * kBatch) {
+            float4 x[kBatch];
+#pragma unroll
+            for (int q = 0; q < kBatch; ++q)
+                if (r0 + 2 * q < rows) x[q] = *reinterpret_cast<const float4*>(gate + (r0 + 2 * q) * stride);
+#pragma unroll
+            for (int q = 0; q < kBatch; ++q) {
+                if (r0 + 2 * q >= rows) break;
+                float y[4] = {x[q].x, x[q].y, x[q].z, x[q].w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    if (a.input_gate.kind == GSA_GATE_A) { y[e] = 1.f - y[e]; continue; }
+                    if (a.input_gate.kind == GSA_GATE_LOGITS) y[e] = log_gate_from_logit(y[e], a.input_gate.inv_tau);
+                    y[e] = -expm1f(y[e]);
+                }
+                *reinterpret_cast<float4*>(out + (r0 + 2 * q) * stride) = make_float4(y[0], y[1], y[2], y[3]);
+            }
+        }
+    }
+    __threadfence();
+    asm volatile("fence.proxy.async;" ::: "memory");      // (the copy engine reads them next)
+    __syncthreads();
+}
+
 struct Ctl {
     // filled by TMA
     uint64_t bar_x;        // d-sized tiles of the current chunk

@@ -123,6 +123,7 @@ value_side_lean_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_co
                        const __grid_constant__ ValueSideArgs a, const int* strong_flag, int32_t* dev_status) {
     follow_previous_grid();
     if (strong_flag[blockIdx.x] != 0) {
+        if (!REV) write_input_gate(a);
         value_side_general<REV>(mapQ, mapK, mapW32, mapG32, mapO, a, dev_status, blockIdx.y);
         return;
     }
@@ -684,6 +685,7 @@ state_scan_kernel(const __grid_constant__ CUtensorMap mapX0, const __grid_consta
                 sum += (double)a.G[(((size_t)span.b * a.T + min(t + kCT, span.t_end) - 1) * a.H + span.h) * kM + threadIdx.x];
             seg_logdecay[(size_t)blockIdx.x * kM + threadIdx.x] = (float)sum;
         }
+        if (!REV) write_input_gate(a);
         value_side_general<REV, true, true>(mapX, mapX, second ? mapW32_1 : mapW32_0, mapG32, mapG32, a, dev_status, slice);
         return;
     }

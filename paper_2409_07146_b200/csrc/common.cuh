@@ -111,6 +111,10 @@ cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t sme
 //
 // reverse = 1 sums over i >= j instead (same decay product): the gradients w.r.t. keys,
 // values and the input gate are such time-reversed runs.
+// Where w is the input gate 1 - a and only the flagged pairs read it in fp32 (the general scans): the gate kernel leaves it
+// out but of the chunks that flag their pair, and the scans form the other rows of a flagged pair from the gate before they go
+// on (write_input_gate).
+struct InputGate { const float* gate = nullptr; int kind = 0; float inv_tau = 0.f; };
 struct ValueSideArgs {
     const void* xq; const void* xk;   // io
     const float* w; const float* G;
@@ -128,6 +132,7 @@ struct ValueSideArgs {
     // strong-decay flags are then [B, nseg, H, ..]
     int nseg = 1, tseg = 0;
     const float* E = nullptr;         // kernels for 128 slots: exp(G), see launch_gate_cumsum_wide
+    InputGate input_gate;             // forward-direction runs on the tensor cores; gate null: w is there
     float* seg_logdecay = nullptr;    // state runs, forward, K side: receives the segments' log-decay (launch_segment_logdecay)
 };
 struct KeySideArgs {
@@ -207,13 +212,14 @@ struct PendingDecay {
 // strong_flag (nullable, [B*H] ints, zeroed by the caller): set to 1 for every (b,h) that has a
 // chunk whose total log-decay is below kFactorisedDecayMin (nseg > 1: [B*nseg*H], per segment).
 // decayed (nullable, bf16 [B,T,H,2M]): rows [high part | rounding residual] of I exp(-G), the
-// input-gate operand of the pipelined tensor-core kernels.  fast_log: take log a with the
+// input-gate operand of the pipelined tensor-core kernels.  leave_out: I only of the chunks that decay
+// below kFactorisedDecayMin (see InputGate).  fast_log: take log a with the
 // hardware base-2 logarithm (absolute error 2^-21.4 for a in [0.5, 1], 3 ulp below), for bf16 io.
 // gate_kind: gsa_gate_t (a, log a, or logits with inv_tau = 1/tau)
 cudaError_t launch_gate_cumsum(const float* gate, int gate_kind, float inv_tau, float* G, float* I,
                                int B, int T, int H, int M, int chunk, int* strong_flag, int nseg, int tseg,
                                void* decayed, int fast_log, cudaStream_t st, const int* cu_seqlens = nullptr,
-                               int nseq = 0);
+                               int nseq = 0, int leave_out = 0);
 // The same for the tensor-core kernels with 128 slots, M = 2 x 64: `decayed` are bf16 [B,T,2H,192] rows [high | middle |
 // low part] of I exp(-G), E = exp(G), local to chunks of 128 tokens; both, and log a, to fp32 accuracy whatever the io
 // type.  G is local to 64 tokens, the chunks of the CUDA-core kernels that take the flagged pairs.

@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
                                                             int chunk, int* __restrict__ strong_flag, int nseg, int tseg,
                                                             __nv_bfloat16* __restrict__ decayed, int fast_log,
                                                             const int* cu_seqlens, int nseq,
-                                                            float* __restrict__ E) {
+                                                            float* __restrict__ E, int leave_out) {
     follow_previous_grid();
     __shared__ double2 group_sum[16][M / 2];
     const int grp = threadIdx.y, s = 2 * threadIdx.x;          // blockDim.y = chunk / 8 <= 16
@@ -174,8 +174,11 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
     if (WIDE && grp == 64 / kCumRows) half0 = half1 = 0.0;
     // the chunk's total log-decay decides which of the chunk kernels takes this (b,h)
     // (with segment-parallel scheduling the flags are per (batch, segment, head))
-    if (strong_flag != nullptr && grp == (int)blockDim.y - 1 &&
-        fmin(before0 + acc0, before1 + acc1) < (double)kFactorisedDecayMin) {
+    const bool strong = strong_flag != nullptr && grp == (int)blockDim.y - 1 &&
+                        fmin(before0 + acc0, before1 + acc1) < (double)kFactorisedDecayMin;
+    // (1 - a left out: of the chunks that do not decide on the general scans by themselves, see InputGate)
+    const bool put_I = leave_out == 0 || __syncthreads_or(strong);
+    if (strong) {
         const int seg = nseg == 1 ? 0 : t_chunk / tseg;
         strong_flag[WIDE ? (b * nseg + seg) * (H / 2) + h / 2 : (b * nseg + seg) * H + h] = 1;
     }
@@ -184,7 +187,7 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
     const float b1h = (float)before1, b1l = (float)(before1 - (double)b1h);
     auto write_row = [&](int i) {
         const uint32_t at = off + i * stride;
-        *reinterpret_cast<float2*>(I + first + at) = inps[i];
+        if (put_I) *reinterpret_cast<float2*>(I + first + at) = inps[i];
         const float G0 = b0h + (b0l + g[i].x), G1 = b1h + (b1l + g[i].y);
         if (!WIDE) {
             *reinterpret_cast<float2*>(G + first + at) = make_float2(G0, G1);
@@ -226,14 +229,14 @@ void launch_gate_kind(int gate_kind, dim3 grid, dim3 block, cudaStream_t st, con
 
 cudaError_t launch_gate_cumsum(const float* gate, int gate_kind, float inv_tau, float* G, float* I, int B,
                                int T, int H, int M, int chunk, int* strong_flag, int nseg, int tseg, void* decayed, int fast_log,
-                               cudaStream_t st, const int* cu_seqlens, int nseq) {
+                               cudaStream_t st, const int* cu_seqlens, int nseq, int leave_out) {
     if (chunk % kCumRows != 0 || chunk / kCumRows > 16 || (M / 2) * (chunk / kCumRows) > 1024) return cudaErrorInvalidValue;
     const int nchunks = (T + chunk - 1) / chunk;
     dim3 block(M / 2, chunk / kCumRows);
     dim3 grid(B * H, nchunks);
     auto launch = [&](auto m) {
         launch_gate_kind<decltype(m)::value, false>(gate_kind, grid, block, st, gate, inv_tau, G, I, T, H, chunk, strong_flag, nseg, tseg,
-                                                    static_cast<__nv_bfloat16*>(decayed), fast_log, cu_seqlens, nseq, (float*)nullptr);
+                                                    static_cast<__nv_bfloat16*>(decayed), fast_log, cu_seqlens, nseq, (float*)nullptr, leave_out);
     };
     if (M == 128) launch(std::integral_constant<int, 128>{});
     else if (M == 64) launch(std::integral_constant<int, 64>{});
@@ -246,7 +249,7 @@ cudaError_t launch_gate_cumsum_wide(const float* gate, int gate_kind, float inv_
                                     const int* cu_seqlens, int nseq) {
     constexpr int chunk = 128;
     launch_gate_kind<64, true>(gate_kind, dim3(2 * B * H, (T + chunk - 1) / chunk), dim3(32, chunk / kCumRows), st, gate, inv_tau, G, I, T,
-                               2 * H, chunk, strong_flag, nseg, tseg, static_cast<__nv_bfloat16*>(decayed), 0, cu_seqlens, nseq, E);
+                               2 * H, chunk, strong_flag, nseg, tseg, static_cast<__nv_bfloat16*>(decayed), 0, cu_seqlens, nseq, E, 0);
     return cudaGetLastError();
 }
 
@@ -717,7 +720,11 @@ __global__ void __launch_bounds__(128) gate_grad_local_kernel(
         for (int i = 0; i < kGG; ++i) { dI[i].x *= pend.reverse_factor(gt[i].x); dI[i].y *= pend.reverse_factor(gt[i].y); }
     }
 #pragma unroll
-    for (int i = 0; i < kGG; ++i) gt[i] = ld2(I, i, 0.f);
+    for (int i = 0; i < kGG; ++i) {
+        // (a gate tensor that holds a gives 1 - a as the gate kernel forms it, which may have left it out)
+        gt[i] = gate_kind == GSA_GATE_A ? ld2(gate, i, 1.f) : ld2(I, i, 0.f);
+        if (gate_kind == GSA_GATE_A) gt[i] = make_float2(1.f - gt[i].x, 1.f - gt[i].y);
+    }
 #pragma unroll
     for (int i = 0; i < kGG; ++i) x[i] = make_float2(-gt[i].x * dI[i].x, -gt[i].y * dI[i].y);
 #pragma unroll
