@@ -38,7 +38,9 @@ using namespace tcchunk;
 // The rows of 1 - a of a flagged pair's moderate chunks, as the gate kernel forms them, where it has left them out
 // (InputGate).  Every CTA that is about to read them writes them all -- the same values -- and reads its own.  A warp a chunk.
 // (All chunks, strong ones too: 32 K tokens of strong gates, 16 heads, 1279 -> 1517 us.)
-__device__ __forceinline__ void write_input_gate(const ValueSideArgs& a) {
+// Not inlined: within the pipelined kernels it costs the scan beside it registers (value_side of B = 8, T = 2048, 4 heads of 512,
+// 55 -> 64 us).
+__device__ __noinline__ void write_input_gate(const ValueSideArgs& a) {
     if (a.input_gate.gate == nullptr) return;
     constexpr int kBatch = 8;
     const ScanSpan span = scan_span(blockIdx.x, a.H, a.T, a.nseg, a.tseg);
