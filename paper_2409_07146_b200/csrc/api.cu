@@ -355,10 +355,11 @@ void timing_after(const char* label, cudaStream_t st) {
     }
 }
 
-// ---- the five scans of the backward that follow the softmax gradient are independent: on the
-// tensor-core path they run on five streams of the calling host thread (the caller's and four
+// ---- the five scans of the backward that follow the softmax gradient are independent: they run
+// on five streams of the calling host thread (the caller's and four
 // of the library's), so that the CTAs of one start as those of another finish and the SMs that
-// one scan's 128 CTAs leave idle take CTAs of the next.  Forked and joined by events; with a
+// one scan's 128 CTAs leave idle take CTAs of the next.  (fp32 steps: B = 2, T = 1024, 4 heads of 256 423 -> 396 us; B = 8, 8 heads
+// of 128 1487 -> 1407; T = 130, 2 heads of 64 142 -> 96.)  Forked and joined by events; with a
 // timing sink active they run one after the other instead, so that each is timed alone.
 struct ScanLanes {
     cudaStream_t stream[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -816,7 +817,7 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
     // on two of the library's streams, beside the dp scan and the softmax gradient.
     const bool early = gate_is_saved && ok_saved != nullptr && use_tc(p) && !fused && nseg == 1 && !g_sink.active;
     ScanLanes* lanes = nullptr;
-    if (use_tc(p) && !g_sink.active) GSA_CUDA(scan_lanes(&lanes));
+    if (!g_sink.active) GSA_CUDA(scan_lanes(&lanes));
     if (early) {
         GSA_CUDA(cudaEventRecord(lanes->fork_early, st));
         for (int i = 0; i < 2; ++i) GSA_CUDA(cudaStreamWaitEvent(lanes->stream[i], lanes->fork_early, 0));
@@ -913,7 +914,7 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
         if (!fused) GSA_LAUNCH("bwd_dq_key_side", key_side(p, adq, 0, w.strong, st, dev_status));
         GSA_LAUNCH("bwd_dv_dIv_pair_rev", launch_rev_pair_tc(pIv, pv, p.m, w.strong, st, dev_status));
         GSA_LAUNCH("bwd_dk_dIk_pair_rev", launch_rev_pair_tc(pIk, pk, p.m, w.strong, st, dev_status));
-    } else if (use_tc(p) && !g_sink.active) {
+    } else if (!g_sink.active) {
         // the five scans side by side (see ScanLanes)
         GSA_CUDA(cudaEventRecord(lanes->fork, st));
         for (int i = early ? 2 : 0; i < 4; ++i) GSA_CUDA(cudaStreamWaitEvent(lanes->stream[i], lanes->fork, 0));
