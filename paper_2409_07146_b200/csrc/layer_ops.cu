@@ -147,7 +147,11 @@ __global__ void __launch_bounds__(512) out_norm_fwd_kernel(const IO* o, const fl
 // registers let three CTAs of 320 threads share an SM.  8 K tokens of 2560 values (123 MB): one token at a time, two means after
 // one another 143 us; four tokens of one CTA per SM, each sigmoid formed twice, 86;
 // so, 60 (both kernels).
+// A CTA's tokens are as many as the call has for it, so a run of fp32 additions ends after kRunPairs pairs, in an fp64 sum of
+// the thread's own: the rounding of 16 additions whatever the batch.  Run and sum stand in shared memory -- in registers the run
+// spills the loop (64 K tokens of 4096 values 600 -> 695 us; so, 590; a partial row for every 16 tokens 630).
 constexpr int kBwdTokens = 2;
+constexpr int kRunPairs = 8;
 template <typename IO>
 __global__ void __launch_bounds__(512, 2) out_norm_bwd_kernel(const IO* o, const IO* dy,
                                                            const float* weight, float eps, IO* d_o,
@@ -155,12 +159,19 @@ __global__ void __launch_bounds__(512, 2) out_norm_bwd_kernel(const IO* o, const
     follow_previous_grid();
     constexpr int V = IoTraits<IO>::kVec;
     __shared__ float scratch[2][16][2 * kBwdTokens];
+    extern __shared__ double sums_of_runs[];          // [V][threads], where the weight gradient is wanted
+    float4* run = reinterpret_cast<float4*>(sums_of_runs + V * blockDim.x) + threadIdx.x;      // [V / 4][threads]
     const int c = threadIdx.x * V;
     const bool own = c < N;
-    float dw[V], w[V];
+    if (dw_part != nullptr) {
+#pragma unroll
+        for (int e = 0; e < V; ++e) sums_of_runs[e * blockDim.x + threadIdx.x] = 0.0;
+#pragma unroll
+        for (int e = 0; e < V / 4; ++e) run[e * blockDim.x] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    float w[V];
 #pragma unroll
     for (int e = 0; e < V; ++e) {
-        dw[e] = 0.f;
         w[e] = weight && own ? weight[c + e] : 1.f;
     }
     int it = 0;
@@ -192,6 +203,9 @@ __global__ void __launch_bounds__(512, 2) out_norm_bwd_kernel(const IO* o, const
             sums[2 * r + 1] = dot;
         }
         cta_sums(sums, scratch[it & 1]);
+        float dw[V];
+#pragma unroll
+        for (int e = 0; e < V; ++e) dw[e] = 0.f;
 #pragma unroll
         for (int r = 0; r < kBwdTokens; ++r)
             if (own && row0 + r < rows) {
@@ -208,11 +222,31 @@ __global__ void __launch_bounds__(512, 2) out_norm_bwd_kernel(const IO* o, const
                 }
                 store_vec(d_o + (row0 + r) * N + c, g);
             }
+        if (dw_part != nullptr) {
+            const bool last = it % kRunPairs == kRunPairs - 1;
+#pragma unroll
+            for (int e = 0; e < V; e += 4) {
+                float4 t = run[e / 4 * blockDim.x];
+                t.x += dw[e]; t.y += dw[e + 1]; t.z += dw[e + 2]; t.w += dw[e + 3];
+                if (last) {
+                    double* sum = sums_of_runs + e * blockDim.x + threadIdx.x;
+                    sum[0] += (double)t.x; sum[blockDim.x] += (double)t.y;
+                    sum[2 * blockDim.x] += (double)t.z; sum[3 * blockDim.x] += (double)t.w;
+                    t = make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+                run[e / 4 * blockDim.x] = t;
+            }
+        }
     }
     if (dw_part != nullptr && own) {
 #pragma unroll
-        for (int e = 0; e < V; e += 4)
-            *reinterpret_cast<float4*>(dw_part + (size_t)blockIdx.x * N + c + e) = make_float4(dw[e], dw[e + 1], dw[e + 2], dw[e + 3]);
+        for (int e = 0; e < V; e += 4) {
+            const float4 t = run[e / 4 * blockDim.x];
+            const double* sum = sums_of_runs + e * blockDim.x + threadIdx.x;
+            *reinterpret_cast<float4*>(dw_part + (size_t)blockIdx.x * N + c + e) =
+                make_float4((float)(sum[0] + (double)t.x), (float)(sum[blockDim.x] + (double)t.y),
+                            (float)(sum[2 * blockDim.x] + (double)t.z), (float)(sum[3 * blockDim.x] + (double)t.w));
+        }
     }
 }
 // 32 columns a CTA, the partial rows dealt out over 32 groups of threads, in a fixed order (all of it latency: a thread a
@@ -284,11 +318,18 @@ cudaError_t launch_out_norm_fwd(const void* o, const float* weight, float eps, v
 cudaError_t launch_out_norm_bwd(const void* o, const void* dy, const float* weight, float eps, void* d_o, float* dw_part,
                                 float* dweight, size_t rows, int N, int io, cudaStream_t st) {
     const unsigned parts = (unsigned)out_norm_bwd_parts(rows, N, io), threads = token_threads(N, io);
+    constexpr int kSumBytes = sizeof(double) + sizeof(float);        // of a value: the sum of its runs and the run
+    const size_t smem = dweight ? (size_t)kSumBytes * threads * (io == GSA_BF16 ? 8 : 4) : 0;
+    const cudaError_t ready =
+        io == GSA_BF16
+            ? cudaFuncSetAttribute(out_norm_bwd_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSumBytes * 512 * 8)
+            : cudaFuncSetAttribute(out_norm_bwd_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSumBytes * 512 * 4);
+    if (ready != cudaSuccess) return ready;
     if (io == GSA_BF16)
-        launch_after(out_norm_bwd_kernel<__nv_bfloat16>, parts, threads, 0, st, (const __nv_bfloat16*)o, (const __nv_bfloat16*)dy,
+        launch_after(out_norm_bwd_kernel<__nv_bfloat16>, parts, threads, smem, st, (const __nv_bfloat16*)o, (const __nv_bfloat16*)dy,
                      weight, eps, (__nv_bfloat16*)d_o, dweight ? dw_part : nullptr, N, rows);
     else
-        launch_after(out_norm_bwd_kernel<float>, parts, threads, 0, st, (const float*)o, (const float*)dy, weight, eps, (float*)d_o,
+        launch_after(out_norm_bwd_kernel<float>, parts, threads, smem, st, (const float*)o, (const float*)dy, weight, eps, (float*)d_o,
                      dweight ? dw_part : nullptr, N, rows);
     if (dweight != nullptr) launch_after(out_norm_dw_kernel, (N + 31) / 32, dim3(32, kDwGroups), 0, st, dw_part, dweight, N, (int)parts);
     return cudaGetLastError();

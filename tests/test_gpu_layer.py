@@ -99,7 +99,7 @@ def test_output_norm_fwd_bwd(io, H, dv, T, with_weight):
 
 @pytest.mark.parametrize("io,H,dv,T", [("bf16", 1, 64, 1), ("f32", 3, 64, 7), ("bf16", 8, 512, 9), ("f32", 4, 512, 5), ("bf16", 7, 64, 17)])
 def test_output_norm_edges(io, H, dv, T):
-    # tokens that do not fill the four and sixteen of a CTA, rows from 8 vectors to the widest, a CTA of a partial last warp
+    # tokens that do not fill the four of a forward CTA or the pair of a backward one, rows from 8 vectors to the widest, a CTA of a partial last warp
     test_output_norm_fwd_bwd(io, H, dv, T, True)
 
 
@@ -137,3 +137,39 @@ def test_output_norm_weight_gradient_of_tiny_activations(io):
     x, g = o.double().flatten(), dy.to(p.io_dtype).double().flatten()
     want = g * x * torch.sigmoid(x) * 1e3
     assert float(((dw.double() - want) / want).abs().max()) <= 2e-5
+
+
+@pytest.mark.parametrize("io,H,dv,T", [("bf16", 8, 512, 1301), ("bf16", 1, 64, 5003), ("f32", 1, 64, 5003)])
+def test_output_norm_bwd_of_more_tokens_than_ctas(io, H, dv, T):
+    # at most 148 * (2 .. 8) CTAs: each takes several pairs of tokens here, the last pair has one
+    r = np.random.default_rng(T)
+    o, dy = r.standard_normal((1, T, H, dv)).astype(np.float32), r.standard_normal((1, T, H, dv)).astype(np.float32)
+    if io == "bf16":
+        o, dy = W.round_to_bf16(o), W.round_to_bf16(dy)
+    wgt = (1.0 + 0.3 * r.standard_normal(H * dv)).astype(np.float32)
+    p = gsa.Params(1, T, H, 64, dv, 64, io=io)
+    d_o, dw = gsa.gsa_out_norm_bwd(p, to_dev(o, io), to_dev(dy, io), to_dev(wgt), 1e-5)
+    again = gsa.gsa_out_norm_bwd(p, to_dev(o, io), to_dev(dy, io), to_dev(wgt), 1e-5)
+    without = gsa.gsa_out_norm_bwd(p, to_dev(o, io), to_dev(dy, io), to_dev(wgt), 1e-5, want_dweight=False)[0]
+    rdo, rdw = layer.out_norm_bwd(o, dy, wgt, 1e-5)
+    assert rel_err(to_np(d_o), rdo, io == "bf16") <= TOL[io]
+    # terms of N(0, 1) size with 2^-21 from the exponential and the divisions, the worst of 4096 sums of them
+    assert rel_err(to_np(dw), rdw) <= 5e-6
+    assert torch.equal(d_o, again[0]) and torch.equal(dw, again[1]) and torch.equal(d_o, without)
+
+
+@pytest.mark.parametrize("io,H,dv,T", [("bf16", 8, 512, 37889), ("f32", 4, 512, 37889)])
+def test_output_norm_weight_gradient_does_not_drift(io, H, dv, T):
+    # All tokens alike, so that every addition to a CTA's sum (128 tokens of it) rounds the same way.  Against T times the
+    # gradient of one token: a run of 16 equal fp32 terms, (2 + .. + 16) / 16 half-ulps at the most; three roundings of sums.
+    # (128 in one run: 1.9e-6.)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    row = torch.randn(2, 1, 1, H, dv, generator=g, device="cuda").to(torch.bfloat16 if io == "bf16" else torch.float32)
+    one = gsa.Params(1, 1, H, 64, dv, 64, io=io)
+    d_one, dw_one = gsa.gsa_out_norm_bwd(one, row[0], row[1])
+    p = gsa.Params(1, T, H, 64, dv, 64, io=io)
+    o, dy = (x.expand(1, T, H, dv).contiguous() for x in row)
+    d_o, dw = gsa.gsa_out_norm_bwd(p, o, dy)
+    want = dw_one.double() * T
+    assert float(((dw.double() - want) / want).abs().max()) <= (135 / 16 + 3) * 2.0 ** -24
+    assert bool((d_o == d_one).all())
