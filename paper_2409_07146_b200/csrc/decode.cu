@@ -331,6 +331,35 @@ static cudaError_t launch_decode_split(const gsa_params_t& p, const IO* q, const
                               (int)p.gate_kind, p.tau > 0.f ? 1.f / p.tau : 0.f, p.scale, (int)p.slot_act, Ks, Vs, o);
 }
 
+// One CTA a pair.  A step placed while the one before it runs takes what that leaves: where the GPU holds one step's CTAs but not
+// two steps', the CTAs left over come last, to whichever SMs are free first, five to some while others have one.  With three a
+// balanced share and five held, that costs more than the early launch gives: shared memory then limits an SM to three.  384
+// pairs of d = 64, us a step of one layer / of 8 layers, logits: early 9.3 / 11.1, plain 8.2 / 11.1, so 7.2 / 9.8; 444 pairs alike;
+// at four a balanced share early 8.7 (456 pairs, 8 layers), so 9.6.  Four held (d = 128, 304 pairs): early 8.9 / 10.4, plain 8.2 /
+// 12.3, so 8.6 / 11.9: left as it is.
+constexpr int kShare = 3, kHeldMin = 5;
+template <auto kernel, typename... A>
+static cudaError_t launch_step(unsigned pairs, cudaStream_t st, A&&... args) {
+    size_t smem = 0;
+    if (pairs > 2 * kSMs && pairs <= kShare * kSMs) {
+        struct Held { int ctas; size_t smem; };
+        static const Held held = [] {
+            Held h{0, 0};
+            cudaFuncAttributes at;
+            // (an SM has 228 KB, a CTA takes 1 KB beside its own)
+            if (cudaFuncGetAttributes(&at, kernel) == cudaSuccess) h.smem = ((228 << 10) / kShare - (1 << 10) - at.sharedSizeBytes) & ~(size_t)127;
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&h.ctas, kernel, kDecodeWarps * 32, 0) != cudaSuccess) h.ctas = 0;
+            return h;
+        }();
+        if (held.ctas >= kHeldMin && 2 * (long long)pairs > (long long)held.ctas * kSMs) {
+            smem = held.smem;
+            const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+        }
+    }
+    return launch_after(kernel, pairs, kDecodeWarps * 32, smem, st, static_cast<A&&>(args)...);
+}
+
 template <typename IO, int DK, int DV>
 static cudaError_t launch_decode_m(const gsa_params_t& p, const IO* q, const IO* k, const IO* v,
                                    const float* gate, float* Ks, float* Vs, IO* o, cudaStream_t st) {
@@ -350,12 +379,10 @@ static cudaError_t launch_decode_m(const gsa_params_t& p, const IO* q, const IO*
     const int is_log = p.gate_kind;
     const float inv_tau = p.tau > 0.f ? 1.f / p.tau : 0.f;
     if (p.m == 128)
-        launch_after(decode_step_kernel<IO, DK, DV, 128>, pairs, kDecodeWarps * 32, 0, st, q, k, v, gate, p.gate_dtype == GSA_BF16, p.gate_broadcast ? p.H : 0, p.feature_map, is_log, inv_tau, p.scale, p.slot_act, Ks, Vs, o);
-    else if (p.m == 64)
-        launch_after(decode_step_kernel<IO, DK, DV, 64>, pairs, kDecodeWarps * 32, 0, st, q, k, v, gate, p.gate_dtype == GSA_BF16, p.gate_broadcast ? p.H : 0, p.feature_map, is_log, inv_tau, p.scale, p.slot_act, Ks, Vs, o);
-    else
-        launch_after(decode_step_kernel<IO, DK, DV, 32>, pairs, kDecodeWarps * 32, 0, st, q, k, v, gate, p.gate_dtype == GSA_BF16, p.gate_broadcast ? p.H : 0, p.feature_map, is_log, inv_tau, p.scale, p.slot_act, Ks, Vs, o);
-    return cudaGetLastError();
+        return launch_step<decode_step_kernel<IO, DK, DV, 128>>(pairs, st, q, k, v, gate, p.gate_dtype == GSA_BF16, p.gate_broadcast ? p.H : 0, p.feature_map, is_log, inv_tau, p.scale, p.slot_act, Ks, Vs, o);
+    if (p.m == 64)
+        return launch_step<decode_step_kernel<IO, DK, DV, 64>>(pairs, st, q, k, v, gate, p.gate_dtype == GSA_BF16, p.gate_broadcast ? p.H : 0, p.feature_map, is_log, inv_tau, p.scale, p.slot_act, Ks, Vs, o);
+    return launch_step<decode_step_kernel<IO, DK, DV, 32>>(pairs, st, q, k, v, gate, p.gate_dtype == GSA_BF16, p.gate_broadcast ? p.H : 0, p.feature_map, is_log, inv_tau, p.scale, p.slot_act, Ks, Vs, o);
 }
 
 template <typename IO, int DK>

@@ -50,3 +50,24 @@ def test_what_is_refused(at, bad, error):
     with pytest.raises(gsa.GsaError):
         gsa.gsa_decode_step(gsa.Params(2, 1, 3, 96, 128, 64), *[t.new_empty(2, 3, 96) for t in x[:2]], *x[2:4], x[4].new_empty(2, 3, 64, 96),
                             x[5], o=x[6])
+
+
+@pytest.mark.parametrize("B", [30, 31, 37, 38])
+def test_steps_of_a_little_more_than_half_of_what_the_gpu_holds(B):
+    # 360 .. 456 pairs of d = 64: 31 and 37 on either edge of the steps that leave an SM three CTAs.  Two steps, one placed
+    # while the other runs, against the same pairs in calls of 24.
+    H, d, m = 12, 64, 64
+    g = torch.Generator(device="cuda").manual_seed(B)
+    r = lambda *s, dt=torch.float32: torch.randn(*s, generator=g, device="cuda").to(dt)
+    x = [r(B, H, d, dt=torch.bfloat16) for _ in range(3)] + [r(B, H, m), r(B, H, m, d), r(B, H, m, d)]
+    y = [t.clone() for t in x]
+    p = gsa.Params(B, 1, H, d, d, m, gate_is_logits=True)
+    o = torch.empty(2, B, H, d, dtype=torch.bfloat16, device="cuda")
+    for i in range(2):
+        gsa.gsa_decode_step(p, *x, o=o[i])
+    for b in range(0, B, 2):
+        n = min(2, B - b)
+        part = gsa.Params(n, 1, H, d, d, m, gate_is_logits=True)
+        for i in range(2):
+            assert torch.equal(gsa.gsa_decode_step(part, *[t[b:b + n] for t in y]), o[i, b:b + n])
+    assert torch.equal(x[4], y[4]) and torch.equal(x[5], y[5])
