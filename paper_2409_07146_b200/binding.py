@@ -2,7 +2,9 @@
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
+import sysconfig
 from dataclasses import dataclass
 
 import torch
@@ -115,6 +117,11 @@ def lib_path() -> str:
     return _LIB_PATH
 
 
+def native_path() -> str:
+    """The extension module for this interpreter and torch (two builds of torch share no C++ interface)."""
+    return os.path.join(_HERE, "_native.%s.torch-%s.so" % (sysconfig.get_config_var("SOABI"), torch.__version__))
+
+
 def exported_symbols():
     return ["gsa_chunk_size", "gsa_workspace_bytes", "gsa_status_string", "gsa_gate_cumsum",
             "gsa_fwd", "gsa_bwd", "gsa_decode_step", "gsa_tc_selftest", "gsa_timing_begin",
@@ -177,16 +184,28 @@ def load_library():
     lib.gsa_out_norm_bwd.restype = ctypes.c_int
     lib.gsa_release_streams.argtypes = []
     lib.gsa_release_streams.restype = ctypes.c_int
-    from . import _native
-    _native.set_library(ctypes.cast(lib.gsa_decode_step, vp).value)
     global _decode_step
-    _decode_step = _native.decode_step
+    _decode_step = _native_decode_step(ctypes.cast(lib.gsa_decode_step, vp).value)
     _lib = lib
     return lib
 
 
+def _native_decode_step(address: int):
+    """decode_step of the extension module built for this interpreter and torch.  The Python path serves every call where
+    there is none, or one that does not load: nothing else of the library depends on it."""
+    path = native_path()
+    try:
+        spec = importlib.util.spec_from_file_location(__package__ + "._native", path)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+    except (ImportError, OSError):
+        return lambda *args: None
+    module.set_library(address)
+    return module.decode_step
+
+
 def _decode_step(*args):
-    """Replaced by _native.decode_step when the library is loaded."""
+    """Replaced when the library is loaded."""
     load_library()
     return _decode_step(*args)
 

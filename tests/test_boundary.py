@@ -135,3 +135,31 @@ def test_shard_states_ask_for_no_more_than_a_forward(lib, io, m):
     # the state runs write no token outputs: the workspace is the forward's without room for any
     p = gsa.Params(1, 4096, 4, 512, 512, m, io=io)
     assert 0 < gsa.gsa_workspace_bytes(p, binding.GSA_WS_SHARD) <= gsa.gsa_workspace_bytes(p, binding.GSA_WS_FWD)
+
+
+def test_everything_but_the_native_decode_call_does_without_the_extension(lib, monkeypatch, tmp_path):
+    """The extension module is compiled against torch's C++ interface; the library is not, and serves without it."""
+    for there in (None, b"not a shared object"):
+        path = tmp_path / "_native.so"
+        if there is not None:
+            path.write_bytes(there)
+        monkeypatch.setattr(binding, "native_path", lambda: str(path))
+        monkeypatch.setattr(binding, "_lib", None)
+        monkeypatch.setattr(binding, "_decode_step", binding._decode_step)
+        fresh = binding.load_library()
+        assert fresh.gsa_status_string(0) == b"ok" and binding._decode_step(1, *[None] * 7) is None
+        p = gsa.Params(B=2, T=100, H=3, d_k=64, d_v=128, m=32)
+        assert gsa.gsa_workspace_bytes(p, binding.GSA_WS_FWD) > 0
+    monkeypatch.undo()
+    assert binding._native_decode_step(ctypes.cast(lib.gsa_decode_step, ctypes.c_void_p).value).__name__ == "decode_step"
+
+
+def test_a_build_without_the_extension_says_so_and_goes_on(monkeypatch, capsys):
+    from paper_2409_07146_b200 import build
+
+    def refuse():
+        raise OSError("no g++")
+    monkeypatch.setattr(build, "_build_native", refuse)
+    monkeypatch.setattr(build, "native_path", lambda: os.path.join(build.HERE, "_native.of-another-torch.so"))
+    assert build.build() == build.LIB
+    assert "not built" in capsys.readouterr().err
