@@ -70,10 +70,8 @@ class Params:
         if self.cu_seqlens is not None:
             return self.c()
         made = self.__dict__.get("_c")
-        if made is None:
-            made = self.c()
-            object.__setattr__(self, "_c", made)
-        return made
+        # (of several threads that make one, the first one's stays: its address may be in use)
+        return self.__dict__.setdefault("_c", self.c()) if made is None else made
 
     def _made_at(self) -> int:
         """The address of that struct where it is made once (0 otherwise)."""

@@ -137,6 +137,30 @@ def test_shard_states_ask_for_no_more_than_a_forward(lib, io, m):
     assert 0 < gsa.gsa_workspace_bytes(p, binding.GSA_WS_SHARD) <= gsa.gsa_workspace_bytes(p, binding.GSA_WS_FWD)
 
 
+def test_the_address_of_a_struct_holds_whatever_thread_made_it(lib, monkeypatch):
+    """Two threads' first calls with one Params: a thread is held while it makes the C struct, another makes one meanwhile and
+    hands its address to the library."""
+    import threading
+    p = gsa.Params(2, 1, 3, 64, 64, 32, io="f32")
+    began, go = threading.Event(), threading.Event()
+    make = gsa.Params.c
+
+    def c(self):
+        made = make(self)
+        if threading.current_thread() is slow:
+            began.set()
+            assert go.wait(10)
+        return made
+    slow = threading.Thread(target=lambda: gsa.gsa_chunk_size(p))
+    monkeypatch.setattr(gsa.Params, "c", c)
+    slow.start()
+    assert began.wait(10)
+    at = p._made_at()
+    go.set()
+    slow.join()
+    assert at == p._made_at() == ctypes.addressof(p._made_c())
+
+
 def test_everything_but_the_native_decode_call_does_without_the_extension(lib, monkeypatch, tmp_path):
     """The extension module is compiled against torch's C++ interface; the library is not, and serves without it."""
     for there in (None, b"not a shared object"):
