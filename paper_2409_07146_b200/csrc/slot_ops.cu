@@ -70,7 +70,7 @@ __device__ __forceinline__ float exp_minus(float g) {
 // KIND: gate_kind.  WIDE: the halves of 128 slots as 2 H heads of 64 (see launch_gate_cumsum_wide), which share their
 // head's flag.  907 instructions a thread -- the kind asked for at every element, a predicate at every row, a 64-bit address
 // for every access -- kept the issue slots as busy as the memory; with the kind a template argument, whole chunks apart from
-// ragged ones and 32-bit offsets from the chunk's first element: B = 4, T = 4096, 32 heads, 64 slots (0.54 GB) 137 -> 95 us,
+// ragged ones and 32-bit offsets from a thread's first element: B = 4, T = 4096, 32 heads, 64 slots (0.54 GB) 137 -> 95 us,
 // 5.7 TB/s; 128 slots, B = 8, T = 2048, 4 heads 48 -> 39.
 template <int M, bool WIDE, int KIND>
 __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) gate_cumsum_kernel(const float* gate,
@@ -88,9 +88,10 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
     const int bh = blockIdx.x, b = bh / H, h = bh % H;
     const int t_chunk = n * chunk, rows_here = min(T - t_chunk, chunk);
     const int rows = max(0, min(kCumRows, rows_here - grp * kCumRows));
-    // (a CTA's first element, and 32-bit offsets from there: a chunk's rows reach 128 H M < 2^31 elements)
-    const size_t first = (((size_t)b * T + t_chunk) * H + h) * M;
-    const uint32_t stride = (uint32_t)H * M, off = grp * kCumRows * stride + s;
+    // (a thread's first element, and 32-bit offsets from there: eight rows hold less than 2^32 elements, 16 GB of gates; a
+    // chunk's 128 need not)
+    const size_t first = (((size_t)b * T + t_chunk + grp * kCumRows) * H + h) * M + s;
+    const uint32_t stride = (uint32_t)H * M;
     float2 g[kCumRows], inps[kCumRows];
     __shared__ uint32_t starts[4];                // rows of the chunk that begin a packed sequence, one bit each
     if (cu_seqlens != nullptr) {
@@ -107,11 +108,11 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
         const float* src = gate + first;
         if (rows == kCumRows) {
 #pragma unroll
-            for (int i = 0; i < kCumRows; ++i) g[i] = *reinterpret_cast<const float2*>(src + (off + i * stride));
+            for (int i = 0; i < kCumRows; ++i) g[i] = *reinterpret_cast<const float2*>(src + i * stride);
         } else {
 #pragma unroll
             for (int i = 0; i < kCumRows; ++i)
-                g[i] = i < rows ? *reinterpret_cast<const float2*>(src + (off + i * stride)) : make_float2(neutral, neutral);
+                g[i] = i < rows ? *reinterpret_cast<const float2*>(src + i * stride) : make_float2(neutral, neutral);
         }
     }
 #pragma unroll
@@ -186,14 +187,14 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
     const float b0h = (float)before0, b0l = (float)(before0 - (double)b0h);
     const float b1h = (float)before1, b1l = (float)(before1 - (double)b1h);
     auto write_row = [&](int i) {
-        const uint32_t at = off + i * stride;
+        const uint32_t at = i * stride;
         if (put_I) *reinterpret_cast<float2*>(I + first + at) = inps[i];
         const float G0 = b0h + (b0l + g[i].x), G1 = b1h + (b1l + g[i].y);
         if (!WIDE) {
             *reinterpret_cast<float2*>(G + first + at) = make_float2(G0, G1);
             // (meaningful for moderate decay only; pairs with a strong-decay chunk do not read it)
             if (decayed != nullptr)
-                store_split2<M>(decayed + 2 * first + (2 * at - 2 * s), s, inps[i].x * exp_minus(G0), inps[i].y * exp_minus(G1));
+                store_split2<M>(decayed + 2 * (first - s) + 2 * (size_t)at, s, inps[i].x * exp_minus(G0), inps[i].y * exp_minus(G1));
         } else {
             // G itself is for the CUDA-core kernels, whose chunks have 64 tokens
             *reinterpret_cast<float2*>(G + first + at) =
@@ -204,7 +205,7 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
             *reinterpret_cast<float2*>(E + first + at) = make_float2(fmaf(e0, r0, e0), fmaf(e1, r1, e1));
             uint32_t hi, mid, lo;
             split_bf16x3(inps[i].x * fmaf(d0, -r0, d0), inps[i].y * fmaf(d1, -r1, d1), hi, mid, lo);
-            uint32_t* row = reinterpret_cast<uint32_t*>(decayed + 3 * first + (3 * (at - s) + s));
+            uint32_t* row = reinterpret_cast<uint32_t*>(decayed + 3 * (first - s) + s + 3 * (size_t)at);
             row[0] = hi;
             row[M / 2] = mid;
             row[M] = lo;
@@ -884,7 +885,7 @@ __global__ void __launch_bounds__(256) gate_grad_local_tma_kernel(
     const uint32_t starts = starts_among(cu, nseq, n * kGG + hh * kGGHalf, kGGHalf);
     if (hh == 1) late_half[ty][tx] = r.total(starts);
     __syncthreads();
-    float* out = dgate + (((size_t)b * T + t0) * H + h) * M + (uint32_t)((ty * kGG + hh * kGGHalf) * H * M + tx);
+    float* out = dgate + (((size_t)b * T + t0 + ty * kGG + hh * kGGHalf) * H + h) * M + tx;
     const float run = r.write(hh == 0 ? late_half[ty][tx] : 0.f, starts, rows, out, (uint32_t)H * M, inv_tau);
     if (hh == 0 && n < nblk) blk_tot[((size_t)bh * nblk + n) * M + tx] = run;
 }
@@ -979,7 +980,7 @@ __global__ void __launch_bounds__(kGGComputeThreads + 32) gate_grad_local_ring_k
             csync();                              // (also: every thread has read its part of the stage)
             if (threadIdx.x == 0)
                 asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar_empty[s])) : "memory");
-            float* out = dgate + (((size_t)b * T + t0) * H + h) * M + (uint32_t)((ty * kGG + hh * kGGHalf) * H * M + tx);
+            float* out = dgate + (((size_t)b * T + t0 + ty * kGG + hh * kGGHalf) * H + h) * M + tx;
             const float run = r.write(hh == 0 ? late_half[ty][tx] : 0.f, starts, rows, out, (uint32_t)H * M, inv_tau);
             if (hh == 0 && n < nblk) blk_tot[((size_t)bh * nblk + n) * M + tx] = run;
             // (one thread reads the flag that the copy lane may raise at any time, so that all leave together)
@@ -1008,19 +1009,19 @@ __global__ void __launch_bounds__(256) gate_grad_carry_kernel(
     const int n = blockIdx.y * blockDim.y + threadIdx.y;
     if (n >= nblk) return;
     const int bh = blockIdx.x, b = bh / H, h = bh % H;
-    // (a CTA's first element, and 32-bit offsets from there)
-    const int t_cta = blockIdx.y * blockDim.y * kGG, t0 = n * kGG + threadIdx.z * kRows;
-    const size_t first = (((size_t)b * T + t_cta) * H + h) * M;
-    const uint32_t stride = (uint32_t)H * M, off = (t0 - t_cta) * stride + s;
+    // (a thread's first element, and 32-bit offsets from there)
+    const int t0 = n * kGG + threadIdx.z * kRows;
+    const size_t first = (((size_t)b * T + t0) * H + h) * M + s;
+    const uint32_t stride = (uint32_t)H * M;
     const int rows = T - t0;
     // (what follows the block reaches the rows after its last token that begins a sequence)
     const int from = cu == nullptr ? 0 : 32 - __clz(starts_among(cu, nseq, n * kGG, min(kGG, T - n * kGG))) - (int)threadIdx.z * kRows;
     const float2 carry = *reinterpret_cast<const float2*>(blk_carry + ((size_t)bh * nblk + n) * M + s);
     float* out = dgate + first;
     const float* in = gate + first;
-    auto load = [&](const float* p, int i) { return *reinterpret_cast<const float2*>(p + (off + i * stride)); };
+    auto load = [&](const float* p, int i) { return *reinterpret_cast<const float2*>(p + i * stride); };
     auto add = [&](int i, float2 d, float2 gt) {
-        *reinterpret_cast<float2*>(out + (off + i * stride)) =
+        *reinterpret_cast<float2*>(out + i * stride) =
             make_float2(d.x + gate_grad_carry(carry.x, gt.x, KIND, inv_tau), d.y + gate_grad_carry(carry.y, gt.y, KIND, inv_tau));
     };
     const float2 unused = make_float2(1.f, 1.f);           // (log gates: the carry goes as it is)

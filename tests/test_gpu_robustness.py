@@ -128,3 +128,26 @@ def test_internal_streams_can_be_released_and_come_back():
     b = gsa.gsa_fwd(p, *args)
     torch.cuda.synchronize()
     assert torch.equal(a, b)
+
+
+def test_gate_kernel_of_a_chunk_of_more_than_2_32_elements():
+    # 64 tokens (a chunk) of 533000 heads of 128 slots: 17.5 GB a tensor.  The last heads' last tokens lie past 2^32
+    # elements from the chunk's first; the same heads alone give the same.
+    T, H, m, few = 64, 533000, 128, 2
+    if torch.cuda.mem_get_info()[0] < 60 << 30:
+        pytest.skip("needs 60 GB")
+    g = torch.Generator(device="cuda").manual_seed(1)
+    tail = torch.rand(1, T, few, m, generator=g, device="cuda") * 0.5 + 0.5
+    gate = torch.ones(1, T, H, m, device="cuda")
+    gate[:, :, -few:] = tail
+    G, I = torch.full_like(gate, 7.0), torch.full_like(gate, 7.0)
+    gsa.gsa_gate_cumsum(gsa.Params(1, T, H, 64, 64, m, io="f32"), gate, G, I)
+    want_G, want_I = torch.empty_like(tail), torch.empty_like(tail)
+    gsa.gsa_gate_cumsum(gsa.Params(1, T, few, 64, 64, m, io="f32"), tail, want_G, want_I)
+    try:
+        assert torch.equal(G[:, :, -few:], want_G) and torch.equal(I[:, :, -few:], want_I)
+        for t in range(0, T, 8):
+            assert not bool(G[:, t:t + 8, :-few].any()) and not bool(I[:, t:t + 8, :-few].any())
+    finally:
+        del gate, G, I
+        torch.cuda.empty_cache()
