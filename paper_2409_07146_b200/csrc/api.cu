@@ -393,6 +393,15 @@ cudaError_t scan_lanes(ScanLanes** out) {
     return cudaSuccess;
 }
 
+// Are the lanes in a capture that `st` is no part of?  (A call captured by this thread takes them into the capture until that
+// ends; a call on another stream meanwhile, plain or of another capture, runs its scans one after the other.)
+bool lanes_taken(const ScanLanes& l, cudaStream_t st) {
+    cudaStreamCaptureStatus lane = cudaStreamCaptureStatusNone, own = cudaStreamCaptureStatusNone;
+    unsigned long long lane_id = 0, own_id = 0;
+    if (cudaStreamGetCaptureInfo(l.stream[0], &lane, &lane_id) != cudaSuccess || lane == cudaStreamCaptureStatusNone) return false;
+    return cudaStreamGetCaptureInfo(st, &own, &own_id) != cudaSuccess || own == cudaStreamCaptureStatusNone || own_id != lane_id;
+}
+
 cudaError_t scan_lanes_release() {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -815,9 +824,10 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
     // With the forward's slot weights in the saved block (and the logits saved, so that nothing here
     // rewrites them), the dv and dI^v scans depend on nothing this call computes: they start at once,
     // on two of the library's streams, beside the dp scan and the softmax gradient.
-    const bool early = gate_is_saved && ok_saved != nullptr && use_tc(p) && !fused && nseg == 1 && !g_sink.active;
     ScanLanes* lanes = nullptr;
     if (!g_sink.active) GSA_CUDA(scan_lanes(&lanes));
+    const bool side_by_side = !g_sink.active && !lanes_taken(*lanes, st);
+    const bool early = gate_is_saved && ok_saved != nullptr && use_tc(p) && !fused && nseg == 1 && side_by_side;
     if (early) {
         GSA_CUDA(cudaEventRecord(lanes->fork_early, st));
         for (int i = 0; i < 2; ++i) GSA_CUDA(cudaStreamWaitEvent(lanes->stream[i], lanes->fork_early, 0));
@@ -900,7 +910,7 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
     pIv.single = pIk.single = pv.single = pk.single = p.tc_operands == GSA_TC_SINGLE;
     const bool paired = use_tc(p) && g_pair_scans.load(std::memory_order_relaxed) != 0 &&
                         rev_pair_supported(pIv, pv, p.m) && rev_pair_supported(pIk, pk, p.m);
-    if (paired && !g_sink.active) {
+    if (paired && side_by_side) {
         GSA_CUDA(cudaEventRecord(lanes->fork, st));
         for (int i = early ? 1 : 0; i < 2; ++i) GSA_CUDA(cudaStreamWaitEvent(lanes->stream[i], lanes->fork, 0));
         if (!fused) GSA_CUDA(key_side(p, adq, 0, w.strong, st, dev_status));
@@ -914,7 +924,7 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
         if (!fused) GSA_LAUNCH("bwd_dq_key_side", key_side(p, adq, 0, w.strong, st, dev_status));
         GSA_LAUNCH("bwd_dv_dIv_pair_rev", launch_rev_pair_tc(pIv, pv, p.m, w.strong, st, dev_status));
         GSA_LAUNCH("bwd_dk_dIk_pair_rev", launch_rev_pair_tc(pIk, pk, p.m, w.strong, st, dev_status));
-    } else if (!g_sink.active) {
+    } else if (side_by_side) {
         // the five scans side by side (see ScanLanes)
         GSA_CUDA(cudaEventRecord(lanes->fork, st));
         for (int i = early ? 2 : 0; i < 4; ++i) GSA_CUDA(cudaStreamWaitEvent(lanes->stream[i], lanes->fork, 0));

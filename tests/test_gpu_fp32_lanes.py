@@ -48,3 +48,44 @@ print("same")
 def test_captured_and_plain_steps_agree(T, m):
     done = subprocess.run([sys.executable, "-c", PROGRAM.format(T=T, m=m)], capture_output=True, text=True, timeout=300)
     assert done.returncode == 0 and "same" in done.stdout, done.stderr[-2000:]
+
+
+BESIDE = """
+import torch
+import paper_2409_07146_b200 as gsa
+g = torch.Generator(device="cuda").manual_seed(2)
+r = lambda *s: torch.randn(*s, generator=g, device="cuda").to(torch.{dtype})
+p = gsa.Params(2, 130, 2, 128, 64, 64, io="{io}", gate_is_logits=True)
+q, k, v, dO = r(2, 130, 2, 128) * 0.09, r(2, 130, 2, 128), r(2, 130, 2, 64), r(2, 130, 2, 64)
+gate = r(2, 130, 2, 64).float()
+ws = [torch.empty(gsa.gsa_workspace_bytes(p, 1), dtype=torch.uint8, device="cuda") for _ in range(2)]
+out = [[torch.empty_like(t) for t in (q, k, v, gate)] for _ in range(2)]
+def step(i):
+    gsa.gsa_bwd(p, q, k, v, gate, dO, dq=out[i][0], dk=out[i][1], dv=out[i][2], dgate=out[i][3], ws=ws[i])
+step(0)
+torch.cuda.synchronize()
+want = [t.clone() for t in out[0]]
+graph, other = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+with torch.cuda.graph(graph, capture_error_mode="relaxed"):
+    step(0)
+    with torch.cuda.stream(other):
+        step(1)
+    step(0)
+torch.cuda.synchronize()
+assert all(torch.equal(a, b) for a, b in zip(out[1], want))
+for t in out[0]:
+    t.fill_(7.0)
+graph.replay()
+torch.cuda.synchronize()
+assert all(torch.equal(a, b) for a, b in zip(out[0], want))
+step(1)
+torch.cuda.synchronize()
+print("same")
+"""
+
+
+@pytest.mark.parametrize("io,dtype", [("f32", "float32"), ("bf16", "bfloat16")])
+def test_a_plain_call_between_two_captured_ones(io, dtype):
+    # the captured calls hold the thread's lanes until the capture ends: a call on another stream does without
+    done = subprocess.run([sys.executable, "-c", BESIDE.format(io=io, dtype=dtype)], capture_output=True, text=True, timeout=300)
+    assert done.returncode == 0 and "same" in done.stdout, done.stderr[-2000:]
