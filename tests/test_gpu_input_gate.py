@@ -2,8 +2,11 @@
 side, every way a call comes to its first scan, every kind of gate."""
 import numpy as np
 import pytest
+import torch
 
+import oracle
 import paper_2409_07146_b200 as gsa
+import test_gpu_fused as fused
 from test_gpu_parity import check_bwd, check_fwd, run_bwd, run_fwd
 from util import TOL, rand_inputs, rel_err, to_dev, to_np
 
@@ -40,7 +43,6 @@ def test_the_forwards_block_serves_the_backward(T):
     p = gsa.Params(1, T, 2, 128, 64, 64, io="bf16")
     q, k, v, dO = (to_dev(d[n], "bf16") for n in ("q", "k", "v", "dO"))
     gate, K0, V0 = (to_dev(d[n]) for n in ("gate", "K0", "V0"))
-    import torch
     ok, block = torch.empty(1, T, 2, 64, device="cuda"), gsa.gate_block(p, "cuda")
     block.fill_(0x7f)                            # (what is left out is nowhere taken for something)
     gsa.gsa_fwd(p, q, k, v, gate, K0, V0, ok_save=ok, gate_save=block)
@@ -49,3 +51,48 @@ def test_the_forwards_block_serves_the_backward(T):
     torch.cuda.synchronize()
     for a, b in zip(x, y):
         assert rel_err(to_np(a), to_np(b)) <= 1e-6
+
+
+@pytest.mark.parametrize("T,H", [(139, 1), (523, 3), (2700, 1)])
+@pytest.mark.parametrize("bf16_gate", [False, True])
+def test_logits(T, H, bf16_gate):
+    # (forwards alone: where a backward follows, the gate kernel writes all of 1 - a for this kind)
+    d = inputs(T, H, T + 1)
+    a = d["gate"].astype(np.float64)
+    x = (np.log(a) - np.log1p(-a)).astype(np.float32)            # a = sigmoid(x)
+    xd = to_dev(x).to(torch.bfloat16) if bf16_gate else to_dev(x)
+    a = 1.0 / (1.0 + np.exp(-to_np(xd)))
+    ref = oracle.fwd(d["q"], d["k"], d["v"], a, K0=d["K0"], V0=d["V0"])
+    p = gsa.Params(1, T, H, 128, 64, 64, io="bf16", impl="tc", gate_is_logits=True, tau=1.0, gate_bf16=bf16_gate)
+    q, k, v = (to_dev(d[n], "bf16") for n in ("q", "k", "v"))
+    KT, VT, ok = torch.empty(1, H, 64, 128, device="cuda"), torch.empty(1, H, 64, 64, device="cuda"), torch.empty(1, T, H, 64, device="cuda")
+    ws = torch.full((gsa.gsa_workspace_bytes(p, 0),), 0x7f, dtype=torch.uint8, device="cuda")       # (3.4e38)
+    o = gsa.gsa_fwd(p, q, k, v, xd, to_dev(d["K0"]), to_dev(d["V0"]), ok_save=ok, KT=KT, VT=VT, ws=ws)
+    for n, t in (("o", o), ("ok", ok), ("KT", KT), ("VT", VT)):
+        assert rel_err(to_np(t), ref[n], n == "o") <= TOL["bf16"], n
+
+
+@pytest.mark.parametrize("T", [384, 523, 2048])
+@pytest.mark.parametrize("saved", [False, True])
+def test_the_fused_kernels_flagged_pairs(T, saved):
+    B, H, w, m = 1, 3, 128, 64
+    d = rand_inputs(T, B, T, H, w, w, m, "bf16", init=True)
+    a = d["gate"]
+    a[:, 130:200, 0, 7] = 0.3                    # the first and the last pair, each with chunks of both kinds
+    a[:, 300:340, H - 1, :] = 0.05
+    fused.check(fused.run(d, B, T, H, w, w, m, fuse=True, saved=saved), fused.reference(d))
+
+
+@pytest.mark.parametrize("T,H", [(139, 1), (523, 3)])
+@pytest.mark.parametrize("log", [False, True])
+def test_shard_states(T, H, log):
+    d = inputs(T, H, T + 2)
+    p = gsa.Params(1, T, H, 128, 64, 64, io="bf16", impl="tc", gate_is_log=log)
+    g = np.log(d["gate"].astype(np.float64)).astype(np.float32) if log else d["gate"]
+    ws = torch.full((gsa.gsa_workspace_bytes(p, 4),), 0x7f, dtype=torch.uint8, device="cuda")
+    KT, VT, decay = gsa.gsa_shard_states(p, to_dev(d["k"], "bf16"), to_dev(d["v"], "bf16"), to_dev(g), ws=ws)
+    ref = oracle.fwd(d["q"], d["k"], d["v"], g, gate_is_log=log)
+    assert rel_err(to_np(KT), ref["KT"]) <= TOL["bf16"] and rel_err(to_np(VT), ref["VT"]) <= TOL["bf16"]
+    want = (g.astype(np.float64) if log else np.log(d["gate"].astype(np.float64))).sum(1)
+    # log a to 2^-21 each (the hardware's logarithm), the sum of a chunk to 2^-24 of it
+    assert np.abs(to_np(decay) - want).max() <= T * 2.0 ** -21 + 2.0 ** -23 * np.abs(want).max()
