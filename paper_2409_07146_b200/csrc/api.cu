@@ -320,7 +320,7 @@ cudaError_t state_scans(const gsa_params_t& p, Segments segs, StateSet ks, State
     for (ValueSideArgs& x : a) { x.nseg = segs.n; x.tseg = segs.t; x.E = w.E; x.input_gate = input_gate; }
     if (use_wide(p)) {
         if (logdecay != nullptr) {
-            const cudaError_t e = launch_segment_logdecay(w.G, logdecay, p.B, p.T, p.H, p.m, segs.n, segs.t, log_gate_chunk(p), st);
+            const cudaError_t e = launch_segment_logdecay(w.G, logdecay, p.B, p.T, p.H, segs.n, segs.t, log_gate_chunk(p), st);
             if (e != cudaSuccess) return e;
         }
         return launch_state_scans_wide(a[0], a[1], reverse, w.strong, st, dev_status);

@@ -200,12 +200,13 @@ __global__ void __launch_bounds__(256, M > 64 ? 1 : 2) value_side_simt_kernel(Va
         sS[c * LM + s] = a.S0 ? a.S0[((size_t)bh * M + s) * a.D + d0 + c] : 0.f;
     }
     const int nchunks = (span.t_end - span.t0 + kC - 1) / kC;
+    const bool states_only = FLAGGED && a.state_only;          // (beside the kernels for 128 slots; other state runs: state_simt_kernel)
     for (int it = 0; it < nchunks; ++it) {
         const int n = REV ? nchunks - 1 - it : it;
         const int t0 = span.t0 + n * kC;
         const int valid = min(kC, span.t_end - t0);
         __syncthreads();
-        if (!a.state_only) load_io_tile<IO>(sXq, xq + (size_t)t0 * strideD, strideD, valid);
+        if (!states_only) load_io_tile<IO>(sXq, xq + (size_t)t0 * strideD, strideD, valid);
         load_io_tile<IO>(sXk, xk + (size_t)t0 * strideD, strideD, valid);
         load_slot_tile<M, false>(sW, w + (size_t)t0 * strideM, strideM, valid);
         load_slot_tile<M, true>(sG, G + (size_t)t0 * strideM, strideM, valid);
@@ -221,7 +222,7 @@ __global__ void __launch_bounds__(256, M > 64 ? 1 : 2) value_side_simt_kernel(Va
             }
         }
         // P = Xq Xk^T, masked to the causal (forward) or anti-causal (reverse) triangle
-        if (!a.state_only) {
+        if (!states_only) {
             float acc[4][4] = {};
             mm_nt(sXq, kLd, sXk, kLd, kDS, ty, tx, acc);
 #pragma unroll
@@ -235,7 +236,7 @@ __global__ void __launch_bounds__(256, M > 64 ? 1 : 2) value_side_simt_kernel(Va
         }
         __syncthreads();
         // out = rowscale * ( colscale * (Xq S) + P W' )
-        if (!a.state_only) {
+        if (!states_only) {
             float acc[4][NJ] = {};
             mm_nn<NJ>(sXq, kLd, sS, LM, kDS, ty, tx, acc);
             if (moderate) {

@@ -175,6 +175,14 @@ __device__ __forceinline__ float slot_act_slope(float z, int act) {
     return 2.f * fmaxf(z, 0.f);
 }
 
+// exp(-x) = 2^(-x log2 e) in two instructions, zero where that is below 2^-126; infinite x give 0 and infinity.  Relative
+// error: 2^-21 and, for the rounding of the exponent, |x| 2^-23.
+__device__ __forceinline__ float exp_neg(float x) {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x * -1.4426950408889634f));
+    return r;
+}
+
 // GSA_GATE_LOGITS: log a = -softplus(-x) / tau (a = sigmoid(x)^(1/tau), Sec. 3.3) and the factor
 // d(log a)/dx = sigmoid(-x) / tau of the gate gradient.
 __device__ __forceinline__ float log_gate_from_logit(float x, float inv_tau) {
@@ -238,11 +246,11 @@ cudaError_t launch_column_sum(const float* in, float* part, float* out, size_t r
 // n bfloat16 values -> fp32 (a gate tensor given in bfloat16)
 cudaError_t launch_widen_bf16(const void* in, float* out, size_t n, cudaStream_t st);
 // Segment-parallel scheduling (T cut into nseg segments run as independent sequences): per-segment
-// log-decay [B,nseg,H,M] from G (128 slots on the tensor cores; the other state runs leave it themselves, which spares
+// log-decay [B,nseg,H,128] from G (128 slots on the tensor cores; the other state runs leave it themselves, which spares
 // every segmented call a launch), and the start memories [B,nseg,H,M,D] of every segment from the
 // end memories of the segments run from empty memories.
-cudaError_t launch_segment_logdecay(const float* G, float* seg_logdecay, int B, int T, int H, int M, int nseg,
-                                    int tseg, int chunk, cudaStream_t st);
+cudaError_t launch_segment_logdecay(const float* G, float* seg_logdecay, int B, int T, int H, int nseg, int tseg, int chunk,
+                                    cudaStream_t st);
 // one side's memories in launch_segment_combine (S0 and final_state nullable); the K and the V side go in one launch
 struct CombineSet { const float* local_end; const float* S0; float* start; float* final_state; int D; };
 cudaError_t launch_segment_combine(const float* seg_logdecay, CombineSet k, CombineSet v, int B, int H, int M, int nseg,

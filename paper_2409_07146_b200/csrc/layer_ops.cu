@@ -15,12 +15,6 @@
 namespace gsa {
 namespace {
 
-// exp(-x) by the hardware's base-2 exponential, as __expf, without its care for results below 2^-126: 1 is added to them
-__device__ __forceinline__ float exp_neg(float x) {
-    float r;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x * -1.4426950408889634f));
-    return r;
-}
 __device__ __forceinline__ float reciprocal_approx(float x) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));

@@ -60,13 +60,6 @@ __device__ __forceinline__ bool sequence_starts_at(const int* cu, int nseq, int 
 // a chunk down to a chunk's own decay of e^-20.  Everywhere else the chunk takes -100 and the strong-decay kernels.
 constexpr float kReset = 40.f;
 
-// exp(-G), 2^-126 and below as zero, of a moderate chunk's sum (at least -60: the plain exponential)
-__device__ __forceinline__ float exp_minus(float g) {
-    float r;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(g * -1.4426950408889634f));
-    return r;
-}
-
 // KIND: gate_kind.  WIDE: the halves of 128 slots as 2 H heads of 64 (see launch_gate_cumsum_wide), which share their
 // head's flag.  907 instructions a thread -- the kind asked for at every element, a predicate at every row, a 64-bit address
 // for every access -- kept the issue slots as busy as the memory; with the kind a template argument, whole chunks apart from
@@ -194,7 +187,7 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
             *reinterpret_cast<float2*>(G + first + at) = make_float2(G0, G1);
             // (meaningful for moderate decay only; pairs with a strong-decay chunk do not read it)
             if (decayed != nullptr)
-                store_split2<M>(decayed + 2 * (first - s) + 2 * (size_t)at, s, inps[i].x * exp_minus(G0), inps[i].y * exp_minus(G1));
+                store_split2<M>(decayed + 2 * (first - s) + 2 * (size_t)at, s, inps[i].x * exp_neg(G0), inps[i].y * exp_neg(G1));
         } else {
             // G itself is for the CUDA-core kernels, whose chunks have 64 tokens
             *reinterpret_cast<float2*>(G + first + at) =
@@ -788,7 +781,7 @@ template <int KIND, bool WIDE> struct GateGradRows {
 #pragma unroll
             for (int i = 0; i < kGGHalf; ++i) {
                 const float g = at(3, i);      // (128 slots: exp(G), 0 past the sequence end)
-                dI[i] *= WIDE ? (g > 0.f ? 1.f / g : 0.f) : exp_minus(g);
+                dI[i] *= WIDE ? (g > 0.f ? 1.f / g : 0.f) : exp_neg(g);
             }
         }
 #pragma unroll
@@ -1326,10 +1319,11 @@ cudaError_t launch_resize_rows(const float* in, float* out, size_t rows, int n_i
 // memories are known.
 //
 // seg_logdecay[b][r][h][s] = sum over the chunks of segment r of G at the chunk's last row.
-template <int M>
+// (128 slots on the tensor cores; other calls have it from their state runs)
 __global__ void segment_logdecay_kernel(const float* G, float* __restrict__ seg_logdecay, int T, int H,
                                         int nseg, int tseg, int chunk) {
     follow_previous_grid();
+    constexpr int M = 128;
     const int s = threadIdx.x, h = blockIdx.y;
     const int b = blockIdx.x / nseg, r = blockIdx.x % nseg;
     const int t_begin = r * tseg, t_end = min(T, t_begin + tseg);
@@ -1395,12 +1389,9 @@ cudaError_t launch_shard_combine(const float* logdecay_all, const float* local_a
     return cudaGetLastError();
 }
 
-cudaError_t launch_segment_logdecay(const float* G, float* seg_logdecay, int B, int T, int H, int M, int nseg,
-                                    int tseg, int chunk, cudaStream_t st) {
-    dim3 grid(B * nseg, H);
-    if (M == 128) launch_after(segment_logdecay_kernel<128>, grid, 128, 0, st, G, seg_logdecay, T, H, nseg, tseg, chunk);
-    else if (M == 64) launch_after(segment_logdecay_kernel<64>, grid, 64, 0, st, G, seg_logdecay, T, H, nseg, tseg, chunk);
-    else launch_after(segment_logdecay_kernel<32>, grid, 32, 0, st, G, seg_logdecay, T, H, nseg, tseg, chunk);
+cudaError_t launch_segment_logdecay(const float* G, float* seg_logdecay, int B, int T, int H, int nseg, int tseg, int chunk,
+                                    cudaStream_t st) {
+    launch_after(segment_logdecay_kernel, dim3(B * nseg, H), 128, 0, st, G, seg_logdecay, T, H, nseg, tseg, chunk);
     return cudaGetLastError();
 }
 

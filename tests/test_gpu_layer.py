@@ -173,3 +173,18 @@ def test_output_norm_weight_gradient_does_not_drift(io, H, dv, T):
     want = dw_one.double() * T
     assert float(((dw.double() - want) / want).abs().max()) <= (135 / 16 + 3) * 2.0 ** -24
     assert bool((d_o == d_one).all())
+
+
+def test_exponential_of_the_sigmoid():
+    # Swish over the range of fp32's exponential, by itself: with a large eps the output path divides by sqrt(eps).
+    # exp(-x): 2^-21 + |x| 2^-23; the addition, two divisions or products, the square root's reciprocal (2 ulp): 8 half-ulps.
+    o = torch.linspace(-70, 80, 32 * 1024 * 64, device="cuda").view(1, 1024, 32, 64)
+    p = gsa.Params(1, 1024, 32, 64, 64, 64, io="f32")
+    y = gsa.gsa_out_norm_fwd(p, o, None, 1e12)
+    x = o.double()
+    want = x * torch.sigmoid(x) * 1e-6
+    bound = 2.0 ** -21 + x.abs() * 2.0 ** -23 + 8 * 2.0 ** -24
+    # (mean(Swish^2) <= 6400 beside 1e12: another 3.2e-9)
+    assert bool(((y.double() - want).abs() <= (bound + 3.2e-9) * want.abs()).all())
+    far = torch.full((1, 1, 1, 64), -200.0, device="cuda")
+    assert bool((gsa.gsa_out_norm_fwd(gsa.Params(1, 1, 1, 64, 64, 64, io="f32"), far, None, 1.0) == 0).all())       # (-3e-85)
