@@ -7,6 +7,7 @@
 
 #include "common.cuh"
 #include "gsa_dev.h"
+#include "tc_common.cuh"
 
 using namespace gsa;
 
@@ -589,6 +590,7 @@ gsa_status_t fwd_core(const CallParams* params, int m_active, const void* q, con
                       const float* gate, const float* K0, const float* V0, void* o,
                       float* ok_save, float* KT, float* VT, bool save_gate, void* gate_save, size_t gate_save_bytes,
                       void* ws, size_t ws_bytes, void* stream, int32_t* dev_status) {
+    TensorMapTable maps;
     const CallParams& p = *params;
     if (ws == nullptr || (reinterpret_cast<uintptr_t>(ws) & 255u) != 0) return GSA_ERR_WORKSPACE;
     Workspace w = carve(p, GSA_WS_FWD, ws);
@@ -764,6 +766,7 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
                       const void* dO, const float* dKT, const float* dVT, void* dq, void* dk,
                       void* dv, float* dgate, float* dK0, float* dV0, bool gate_is_saved, const void* gate_saved,
                       size_t gate_saved_bytes, void* ws, size_t ws_bytes, void* stream, int32_t* dev_status) {
+    TensorMapTable maps;
     const CallParams& p = *params;
     if (ws == nullptr || (reinterpret_cast<uintptr_t>(ws) & 255u) != 0) return GSA_ERR_WORKSPACE;
     Workspace w = carve(p, GSA_WS_BWD, ws);

@@ -5,23 +5,15 @@
 namespace gsa {
 namespace {
 
-template <bool REV>
 __global__ void __launch_bounds__(kScanThreads, 1)
-value_side_general_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
-                          const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapG,
-                          const __grid_constant__ CUtensorMap mapO, const __grid_constant__ ValueSideArgs a,
-                          const int* __restrict__ strong_flag, int32_t* dev_status) {
+value_side_general_kernel(const __grid_constant__ GeneralValueMaps maps, const __grid_constant__ ValueSideArgs a, const int* __restrict__ strong_flag, int32_t* dev_status) {
     if (strong_flag[blockIdx.x] == 0) return;
-    if (!REV) write_input_gate(a);
-    value_side_general<REV>(mapQ, mapK, mapW, mapG, mapO, a, dev_status, blockIdx.y);
+    write_input_gate(a);
+    value_side_general<false>(maps.steps(), a, dev_status, blockIdx.y);
 }
-template <bool REV>
 __global__ void __launch_bounds__(kScanThreads, 1)
-key_side_general_kernel(const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapUq,
-                        const __grid_constant__ CUtensorMap mapUk, const __grid_constant__ CUtensorMap mapG,
-                        const __grid_constant__ CUtensorMap mapO, const __grid_constant__ KeySideArgs a,
-                        const int* __restrict__ strong_flag, int32_t* dev_status) {
-    if (strong_flag[blockIdx.x] != 0) key_side_general<REV>(mapV, mapUq, mapUk, mapG, mapO, a, dev_status);
+key_side_general_kernel(const __grid_constant__ GeneralKeyMaps maps, const __grid_constant__ KeySideArgs a, const int* __restrict__ strong_flag, int32_t* dev_status) {
+    if (strong_flag[blockIdx.x] != 0) key_side_general<false>(maps.steps(), a, dev_status);
 }
 
 }  // namespace
@@ -76,30 +68,22 @@ int tc_value_side_slices(int D) { return (D + kDST - 1) / kDST; }
 int tc_chunk() { return kCT; }
 
 cudaError_t launch_value_side_general(const ValueSideArgs& a, const int* strong_flag, cudaStream_t st, int32_t* dev_status) {
-    CUtensorMap mq, mk, mw, mg, mo;
-    cudaError_t e = make_tensor_map_bthd(&mq, a.xq, a.B, a.T, a.H, a.D, kCT, 2);
-    if (e == cudaSuccess) e = make_tensor_map_sliced(&mo, a.out, tc_value_side_slices(a.D), a.B, a.T, a.H, kM, kCT, 4);
-    if (e == cudaSuccess) e = make_tensor_map_bthd(&mk, a.xk, a.B, a.T, a.H, a.D, kCT, 2);
-    if (e == cudaSuccess) e = make_tensor_map_bthd(&mw, a.w, a.B, a.T, a.H, kM, kCT, 4);
-    if (e == cudaSuccess) e = make_tensor_map_bthd(&mg, a.G, a.B, a.T, a.H, kM, kCT, 4);
-    if (e == cudaSuccess) e = prepare<value_side_general_kernel<false>>(kSmemGeneral);
+    GeneralValueMaps maps;
+    cudaError_t e = make_general_maps(&maps, a);
+    if (e == cudaSuccess) e = prepare<value_side_general_kernel>(kSmemGeneral);
     if (e != cudaSuccess) return e;
-    dim3 grid(a.B * a.nseg * a.H, tc_value_side_slices(a.D));
-    value_side_general_kernel<false><<<grid, kScanThreads, kSmemGeneral, st>>>(mq, mk, mw, mg, mo, a, strong_flag, dev_status);
+    const dim3 grid(a.B * a.nseg * a.H, tc_value_side_slices(a.D));
+    value_side_general_kernel<<<grid, kScanThreads, kSmemGeneral, st>>>(maps, a, strong_flag, dev_status);
     return cudaGetLastError();
 }
 
 cudaError_t launch_key_side_general(const KeySideArgs& a, const int* strong_flag, cudaStream_t st, int32_t* dev_status) {
-    CUtensorMap mv, muq, muk, mg, mo;
-    cudaError_t e = make_tensor_map_bthd(&mv, a.xv, a.B, a.T, a.H, a.D, kCT, 2);
-    if (e == cudaSuccess) e = make_tensor_map_bthd(&mo, a.out, a.B, a.T, a.H, a.D, kCT, 2);
-    if (e == cudaSuccess) e = make_tensor_map_bthd(&muq, a.uq, a.B, a.T, a.H, kM, kCT, 4);
-    if (e == cudaSuccess) e = make_tensor_map_bthd(&muk, a.uk, a.B, a.T, a.H, kM, kCT, 4);
-    if (e == cudaSuccess) e = make_tensor_map_bthd(&mg, a.G, a.B, a.T, a.H, kM, kCT, 4);
-    if (e == cudaSuccess) e = prepare<key_side_general_kernel<false>>(kSmemGeneral);
+    GeneralKeyMaps maps;
+    cudaError_t e = make_general_maps(&maps, a);
+    if (e == cudaSuccess) e = prepare<key_side_general_kernel>(kSmemGeneral);
     if (e != cudaSuccess) return e;
-    dim3 grid(a.B * a.nseg * a.H, tc_value_side_slices(a.D));
-    key_side_general_kernel<false><<<grid, kScanThreads, kSmemGeneral, st>>>(mv, muq, muk, mg, mo, a, strong_flag, dev_status);
+    const dim3 grid(a.B * a.nseg * a.H, tc_value_side_slices(a.D));
+    key_side_general_kernel<<<grid, kScanThreads, kSmemGeneral, st>>>(maps, a, strong_flag, dev_status);
     return cudaGetLastError();
 }
 

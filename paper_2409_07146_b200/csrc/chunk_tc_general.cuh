@@ -1,32 +1,32 @@
-// The general tcgen05 (bf16 tensor-core) versions of the two chunk primitives of Algorithm 1, for the (batch, head)
-// pairs that hold a strong-decay chunk.  They are device functions: every scan is ONE launch of a pipelined kernel
+// The general versions of the two chunk primitives of Algorithm 1, for the (batch, head) pairs that hold a strong-decay
+// chunk: any gates, from a = 1 to a = 0.  They are device functions: every scan is ONE launch of a pipelined kernel
 // (chunk_tc_lean.cu, chunk_tc_pair.cu) whose CTAs come here when their pair is flagged.  As launches of their own
 // they cost every scan a second launch, a side stream and four events, which is what bounded short calls: a forward over
 // T = 300, 16 heads of 128, 59 us with them and 42 without; a training step of the 1.3B model's layer 481 and 466.
 //
-// One CTA owns one (batch, head) and one 128-wide slice of the head dimension and walks the
-// chunks (128 tokens each) in order.  It has 256 compute threads and one issuing warp.
-// Compute threads r and r + 128 share row r of the chunk, which is channel r of the state
-// slice and TMEM lane r of every accumulator; the first works on slots (or columns) 0..31
-// (0..63), the second on the rest.  One lane of the issuing warp requests every tile copy
-// and issues every MMA, running ahead of the compute threads; the two sides meet on
-// mbarriers only.
-// Per chunk:
-//   * every tile -- the d-sized ones (xq, xk / xv, bf16) and the slot-sized ones (weights,
-//     cumulative log gate G, fp32) -- arrives by TMA with the 128-byte swizzle, requested as
-//     soon as the buffer it lands in has been consumed by the previous chunk, so the copy of
-//     chunk n+1 runs under the computation of chunk n;
-//   * each thread reads its own row of the slot-sized tiles (conflict-free under the
-//     swizzle), scales it by the decay factors and writes bf16 operand rows;
-//   * all contractions run as tcgen05.mma (M = 128) with fp32 accumulators in tensor
-//     memory, committed to mbarriers that the compute threads wait on;
-//   * the fp32 master copy of the state slice stays in registers (32 per thread); its bf16
-//     copy for the next chunk's state product is rewritten every chunk.
-// Decay inside a chunk is factorised as exp(G_i) * exp(-G_j) while the chunk's total
-// log-decay stays above kFactorisedDecayMin; a chunk that forgets harder computes its
-// intra-chunk term with explicit exponent differences on the CUDA cores instead.
-// Every wait is bounded: on expiry the CTA flags dev_status, frees its tensor memory and
-// returns.
+// The decay between two tokens of a 128-token chunk does not factorise around one reference point where the chunk forgets
+// more than e^-60 (App. A: secondary chunking).  Here a CTA walks its scan in steps of kSub = 16 tokens, each with the state
+// carried across it, and every decay factor that it forms is at most 1:
+//   value side   out_i = e_i (xq_i S) + sum_j P_ij w_j prod a_r,      S <- e_last S + xk^T (w_j s_j)
+//   key side     out_i = (uq_i e_i) S + sum_j A_ij xv_j,              S <- e_last S + (uk_j s_j)^T xv
+// with e_i the decay from the step's start through token i and s_j that from j to its end (time-reversed: e and s swap).
+// tcgen05, whose products have 128 (64) rows, would do four times the work of a 16-token step and a commit and a wait per
+// step on top, so the products are warp-level ones (mma.sync m16n8k16: 8.3 cycles each; 64 a state warp and step on the value
+// side, 88 on the key side).  What bounds it: one state warp's chain of splits and products (960 cycles a step by itself on the
+// value side, 1300 beside its scheduler's slot warp; the tensor pipe is 33 and 40% active).  32 K tokens, 16 heads of 128,
+// a = sigmoid(N(-2, 1)): pass 1 486 -> 206 us, pass 2 410 -> 236 (HBM's share of either: 105), state runs 205 -> 33, the forward
+// 1283 -> 659 us.  The scans before these took 128-token chunks on tcgen05 and walked the decay row by row, 28 k cycles a chunk.
+//
+// Warps of two roles, meeting on mbarriers only:
+//   * four slot warps take the steps in turn: a step's rows by TMA, asked for one of a warp's steps ahead (by 16-byte asynchronous
+//     copies of all lanes the warps were held up for 40 cycles a copy, 1400 a step); decay factors, a lane two slots; decayed
+//     operand rows as bf16 high/low pairs; the intra-step term (value side: P by mma, then running decay products in fp32; key
+//     side: A by mma); at the end the output rows;
+//   * four state warps take every step: the state (value side: 16 slots x 128 channels a warp, key side: 32 channels x
+//     64 slots) stays in registers in fp32, in the fragment layout that serves as the next product's operand as it stands.
+//     (Eight of them, half the channels each: 209 and 252 us; two to a scheduler wait for the same pipes at the same time.  Splits
+//     and decays moved by hand behind other blocks' products: 209 and 250.)
+// Every wait is bounded: on expiry the CTA flags dev_status, runs out without waiting and returns.
 #pragma once
 #include "chunk_tc_shared.cuh"
 
@@ -78,931 +78,801 @@ __device__ __noinline__ void write_input_gate(const ValueSideArgs& a) {
     __syncthreads();
 }
 
-struct Ctl {
-    // filled by TMA
-    uint64_t bar_x;        // d-sized tiles of the current chunk
-    uint64_t bar_g[2];     // value_side: G tile, two stages; key_side: [0] = uk + G tiles
-    uint64_t bar_w;        // value_side: weight tile; key_side: uq tile
-    // signalled by tcgen05.commit
-    uint64_t bar_p;        // first product of the chunk (P or A) complete
-    uint64_t bar_mma1;     // state and inter-chunk products complete
-    uint64_t bar_mma2;     // intra-chunk product complete
-    // signalled by the compute threads (one arrival after their barrier)
-    uint64_t bar_ops;      // operand rows of the chunk are in shared memory
-    uint64_t bar_pm;       // masked P / A rows are in shared memory
-    uint64_t bar_out;      // output rows are staged (or the chunk is otherwise done)
-    uint64_t bar_sb;       // value_side: the state copy for the next chunk is written
-                           // key_side: (issuing warp ->) the output staging buffer is free again
-    uint32_t tmem_slot;
+constexpr int kSub = 16;               // tokens of a step
+constexpr int kStages = 8;             // steps whose rows are on their way or in use
+constexpr int kStateWarps = 4, kSlotWarps = 4;       // one of each to a scheduler
+static_assert(kScanThreads >= 32 * (kStateWarps + kSlotWarps) && kStages == 2 * kSlotWarps, "");
+// tiles of a step, by TMA: two panels of [16 rows][128 bytes] with the 128-byte swizzle (128 channels in bf16, 64 slots in fp32)
+constexpr int kStepPanel = kSub * 128, kXTile = 2 * kStepPanel, kSlotTile = 2 * kStepPanel;
+// rows that the warps write, in bytes: eight rows 16 bytes apart modulo 128 meet in no bank
+constexpr int kDecRow = 2 * kM + 16;   // 64 slots, bf16
+constexpr int kORow = 4 * kM + 16;     // 64 slots, fp32, written by columns
+constexpr int kOutRow = 2 * kDST + 16; // 128 channels, bf16
+constexpr int kDecTile = kSub * kDecRow;
+constexpr int kPRow = 8 * kSub + 16;   // value side: a row of P, every value twice (both slots of a lane)
+constexpr int kARow = 2 * kSub + 16;   // key side: a row of A, bf16
+
+struct GeneralCtl {
+    uint64_t full[kStages];            // (TMA) the rows of a step have landed
+    uint64_t ready[kSlotWarps];        // (slot warp) decayed rows and total decay of its step are in shared memory, key side: and A
+    uint64_t done[kSlotWarps];         // (state warps) a slot warp's step has been taken: all its rows may be written again,
+                                       // value side: the inter-step product is in shared memory, key side: the output rows
     volatile int abort;
-    volatile int moderate[2];   // decision of the chunk, by chunk parity
-    alignas(16) float gc[kM];    // G of the chunk's last valid row
-    alignas(16) float egc[kM];   // exp(gc)
 };
 
-// Publish the G row of the chunk's last valid token, its exponential and decide whether the
-// chunk's decay is moderate.  One compute-thread barrier inside; the result is uniform.
-__device__ __forceinline__ bool publish_chunk_decay(Ctl* ctl, int tid, const unsigned char* gtile, int last_row) {
-    bool fine = true;
-    if (tid < kM) {
-        const float g = tile_elem(gtile, last_row, tid);
-        ctl->gc[tid] = g;
-        ctl->egc[tid] = __expf(g);
-        fine = g >= kFactorisedDecayMin;
-    }
-    return compute_sync_and(fine);
+// A wait that expires flags the CTA; once flagged, later waits that are not over return at once and the roles run out.
+__device__ __forceinline__ void general_wait(GeneralCtl* ctl, uint64_t* bar, uint32_t parity) {
+    if (!mbar_try(bar, parity) && !ctl->abort && !mbar_wait(bar, parity)) ctl->abort = 1;
+    __syncwarp();
 }
 
-// FIRST: this is the CTA's first scan, which allocates its tensor memory (a CTA may do that once: the allocation gives
-// up the right to another one); a second scan takes over the barriers' memory and tmem_slot of the first.
-template <bool FIRST>
-__device__ __forceinline__ void ctl_init(Ctl* ctl, int tid, int warp) {
+__device__ __forceinline__ void general_ctl_init(GeneralCtl* ctl, int tid) {
     if (tid == 0) {
-        if (!FIRST) {
-            uint64_t* bars[] = {&ctl->bar_x, &ctl->bar_g[0], &ctl->bar_g[1], &ctl->bar_w, &ctl->bar_p, &ctl->bar_mma1,
-                                &ctl->bar_mma2, &ctl->bar_ops, &ctl->bar_pm, &ctl->bar_out, &ctl->bar_sb};
-            for (uint64_t* b : bars) mbar_inval(b);
+        for (int i = 0; i < kStages; ++i) mbar_init(&ctl->full[i], 1);
+        for (int i = 0; i < kSlotWarps; ++i) {
+            mbar_init(&ctl->ready[i], 1);
+            mbar_init(&ctl->done[i], kStateWarps);
         }
-        mbar_init(&ctl->bar_x, 1);
-        mbar_init(&ctl->bar_g[0], 1);
-        mbar_init(&ctl->bar_g[1], 1);
-        mbar_init(&ctl->bar_w, 1);
-        mbar_init(&ctl->bar_p, 1);
-        mbar_init(&ctl->bar_mma1, 1);
-        mbar_init(&ctl->bar_mma2, 1);
-        mbar_init(&ctl->bar_ops, 1);
-        mbar_init(&ctl->bar_pm, 1);
-        mbar_init(&ctl->bar_out, 1);
-        mbar_init(&ctl->bar_sb, 1);
         ctl->abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (FIRST && warp == 0) {
-        __syncwarp();
-        tmem_alloc(&ctl->tmem_slot, kTmemCols);
-    }
-    tc_fence_before_sync();
     __syncthreads();
-    tc_fence_after_sync();
+}
+// Ends a scan: its barriers' memory may be used again.  Returns whether all went well.
+__device__ __forceinline__ bool general_finish(GeneralCtl* ctl, int tid, int32_t* dev_status) {
+    __syncthreads();
+    const bool fine = ctl->abort == 0;
+    if (!fine)         // bounded grace period for tile copies still in flight before shared memory goes away
+        for (int i = 0; i < 200; ++i) __nanosleep(1000);
+    if (tid == 0) {
+        if (!fine && dev_status != nullptr) *dev_status = GSA_ERR_TIMEOUT;
+        for (int i = 0; i < kStages; ++i) mbar_inval(&ctl->full[i]);
+        for (int i = 0; i < kSlotWarps; ++i) { mbar_inval(&ctl->ready[i]); mbar_inval(&ctl->done[i]); }
+    }
+    __syncthreads();
+    return fine;
+}
+__device__ __forceinline__ void warp_arrive(uint64_t* bar, int lane) {
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar);
 }
 
-// Strong-decay chunks (App. A: a decay too strong for one reference point per chunk).  The decay
-// between two rows of a chunk is a product of per-step gates, prod_{r=j+1..i} a_r[s], every factor
-// <= 1: walking j away from the target row i, the product is carried along by ONE multiplication
-// per step and slot -- no exponential in the loop, nothing can overflow -- and the walk stops as
-// soon as the product has fallen below 2^-40 for all slots of the thread (what is left of the sum is
-// then below 1e-12 of its leading terms).  With strong forgetting that is after a dozen steps.
-// The per-step gates a_j = exp(G_j - G_{j-1}) are formed once per chunk, in place of the G tile.
-constexpr float kDecayFloor = 9.094947e-13f;      // 2^-40
+// ---- warp-level building blocks
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+}
+__device__ __forceinline__ void ldsm4_trans(uint32_t (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+}
+__device__ __forceinline__ void stsm4_trans(uint32_t addr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(r0), "r"(r1), "r"(r2), "r"(r3)
+                 : "memory");
+}
+// c += a b: m16n8k16
+__device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// a lane's two slots: packed fp32 arithmetic (half the issue slots)
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float x, float y) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+// two values as a bf16 high/low pair
+__device__ __forceinline__ void split_pair(float x0, float x1, uint32_t& hi, uint32_t& lo) {
+    hi = pack_bf16(x0, x1);
+    const float2 rest = unpack2(sub2(pack2(x0, x1), pack2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u))));
+    lo = pack_bf16(rest.x, rest.y);
+}
+// s = s dec + u of both
+__device__ __forceinline__ void decay_add(float& s0, float& s1, f32x2 dec, float u0, float u1) {
+    const float2 v = unpack2(fma2(pack2(s0, s1), dec, pack2(u0, u1)));
+    s0 = v.x;
+    s1 = v.y;
+}
+// exp of a log-decay difference to - from <= 0 of both slots
+__device__ __forceinline__ f32x2 decay2(float2 from, float2 to) { return pack2(exp_neg(from.x - to.x), exp_neg(from.y - to.y)); }
+// kBatch tokens at a time, operation by operation: the chains of a token then overlap (token by token the compiler leaves
+// them one behind the other, 35 cycles each)
+constexpr int kBatch = 8;
+// two slots of decayed rows row0 .. row0 + kBatch - 1 as a high/low pair
+__device__ __forceinline__ void store_pairs(unsigned char* hi_tile, int row0, int lane, const f32x2 (&v)[kBatch]) {
+    uint32_t hi[kBatch], lo[kBatch];
+    float2 x[kBatch];
+#pragma unroll
+    for (int j = 0; j < kBatch; ++j) x[j] = unpack2(v[j]);
+#pragma unroll
+    for (int j = 0; j < kBatch; ++j) hi[j] = pack_bf16(x[j].x, x[j].y);
+#pragma unroll
+    for (int j = 0; j < kBatch; ++j) x[j] = unpack2(sub2(v[j], pack2(__uint_as_float(hi[j] << 16), __uint_as_float(hi[j] & 0xffff0000u))));
+#pragma unroll
+    for (int j = 0; j < kBatch; ++j) lo[j] = pack_bf16(x[j].x, x[j].y);
+    uint32_t* p = reinterpret_cast<uint32_t*>(hi_tile + row0 * kDecRow) + lane;
+#pragma unroll
+    for (int j = 0; j < kBatch; ++j) {
+        p[j * (kDecRow / 4)] = hi[j];
+        p[j * (kDecRow / 4) + kDecTile / 4] = lo[j];
+    }
+}
+// a lane's two slots of a row of a slot-sized tile
+__device__ __forceinline__ f32x2 slots2(const unsigned char* tile, int row, int lane) {
+    const uint32_t at = (lane >> 4) * kStepPanel + ((lane & 15) >> 1) * 16 + (lane & 1) * 8;
+    return *reinterpret_cast<const f32x2*>(tile + row * 128 + (at ^ ((row & 7) << 4)));
+}
+// where 8 channels of a row of a d-sized tile are: 16-byte piece `piece` of 16
+__device__ __forceinline__ uint32_t x_at(uint32_t tile, int row, int piece) {
+    return tile + (piece >> 3) * kStepPanel + row * 128 + (((piece & 7) ^ (row & 7)) << 4);
+}
 
-// Replace the G tile by the per-step gates (rows past the end: 1).  Two compute-thread barriers inside.
-__device__ __forceinline__ void gates_in_place(unsigned char* gt, int row, int half, int sb, int valid) {
-    const int grow = min(row, valid - 1);
-    float aj[kHS];
+// Which steps a scan takes: step n works on tokens [t, t + 16) from token() on; forward in order, reversed from the last one.
+struct Steps {
+    int t0, t_end, first, count;       // steps first .. first + count - 1 of the span
+    template <bool REV> __device__ __forceinline__ int token(int n) const {
+        return t0 + kSub * (first + (REV ? count - 1 - n : n));
+    }
+    // (a 128-token chunk, which G is local to, begins here)
+    __device__ __forceinline__ bool chunk_start(int t) const { return (t - t0) % kCT == 0; }
+};
+__device__ __forceinline__ Steps all_steps(const ScanSpan& s) { return {s.t0, s.t_end, 0, (s.t_end - s.t0 + kSub - 1) / kSub}; }
+
+// End memories need only the chunks from which anything is left: those that every slot's decay carries below e^-128 on the way
+// to the span's end (reversed: its start) can change nothing in fp32 where the memories are below 1e10 -- with gates that
+// forget within a dozen tokens, all but one chunk of the span.  Every warp comes to the same result by itself.
+constexpr float kForgotten = -128.f;
+template <bool REV> __device__ __forceinline__ Steps remembered_steps(const ValueSideArgs& a, const ScanSpan& span, int lane) {
+    Steps s = all_steps(span);
+    const int chunks = (span.t_end - span.t0 + kCT - 1) / kCT;
+    constexpr int kBatch = 4;
+    float2 sum = make_float2(0.f, 0.f);
+    int kept = 0;
+    for (int c0 = 0; c0 < chunks && kept == 0; c0 += kBatch) {
+        float2 g[kBatch];
 #pragma unroll
-    for (int c = 0; c < kHS / 8; ++c) {
-        float g[8], gp[8];
-        tile_row8(gt, grow, sb + 8 * c, g);
-        if (row > 0 && row < valid) tile_row8(gt, row - 1, sb + 8 * c, gp);
+        for (int q = 0; q < kBatch; ++q) {
+            const int c = min(c0 + q, chunks - 1), n = REV ? c : chunks - 1 - c;
+            const int last = min(span.t0 + (n + 1) * kCT, span.t_end) - 1;
+            g[q] = *reinterpret_cast<const float2*>(a.G + (((size_t)span.b * a.T + last) * a.H + span.h) * kM + 2 * lane);
+        }
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            aj[8 * c + e] = row >= valid ? 1.f : __expf(row > 0 ? g[e] - gp[e] : g[e]);
+        for (int q = 0; q < kBatch; ++q) {
+            if (kept != 0 || c0 + q >= chunks) continue;
+            sum.x += g[q].x;
+            sum.y += g[q].y;
+            if (__all_sync(0xffffffffu, fmaxf(sum.x, sum.y) < kForgotten)) kept = c0 + q + 1;
         }
     }
-    compute_sync();           // every thread has read what it needs of G
-    unsigned char* panel = gt + half * kPanelB;
+    if (kept == 0 || kept == chunks) return s;
+    const int steps = kept * (kCT / kSub);
+    if (REV) {
+        s.count = steps;
+    } else {
+        s.first = (chunks - kept) * (kCT / kSub);
+        s.count -= s.first;
+    }
+    return s;
+}
+
+// A slot warp's copies: the rows of step n into its stage.  A stage's tiles, in this order: NX d-sized ones (128 channels from
+// d0 on, those past D zero), NS slot-sized ones, then G.  Rows past the end of T are zeros (a span ends there or at a whole chunk).
+struct StepMaps { const CUtensorMap *x[2], *s[2], *G; };
+template <bool REV, int NX, int NS>
+__device__ __forceinline__ void load_step(GeneralCtl* ctl, unsigned char* ring, const StepMaps& maps, const Steps& steps,
+                                          const ScanSpan& span, int d0, int n) {
+    if (n >= steps.count) return;
+    if (elect_one()) {
+        const int st = n % kStages, t = steps.token<REV>(n);
+        uint64_t* bar = &ctl->full[st];
+        unsigned char* dst = ring + st * (NX * kXTile + (NS + 1) * kSlotTile);
+        mbar_expect_tx(bar, NX * kXTile + (NS + 1) * kSlotTile);
 #pragma unroll
-    for (int c = 0; c < kHS / 4; ++c)
-        *reinterpret_cast<float4*>(panel + swz128(row, c)) = make_float4(aj[4 * c], aj[4 * c + 1], aj[4 * c + 2], aj[4 * c + 3]);
-    compute_sync();
+        for (int i = 0; i < NX; ++i, dst += kXTile) {
+            tma_load_4d(dst, maps.x[i], bar, d0, span.h, t, span.b);
+            tma_load_4d(dst + kStepPanel, maps.x[i], bar, d0 + 64, span.h, t, span.b);
+        }
+#pragma unroll
+        for (int i = 0; i <= NS; ++i, dst += kSlotTile) {
+            const CUtensorMap* map = i < NS ? maps.s[i] : maps.G;
+            tma_load_4d(dst, map, bar, 0, span.h, t, span.b);
+            tma_load_4d(dst + kStepPanel, map, bar, 32, span.h, t, span.b);
+        }
+    }
+    __syncwarp();
 }
-
-// The walks go by distance: at step d every row i of the chunk is at j = i - d (time-reversed: i + d), so that all lanes of a
-// warp are at work until their products have died out.  (By absolute columns, as the accumulator is read, a warp repeats
-// the walk for the different rows of its lanes, a third of them live at a time.  32 K tokens, 16 heads of 128, gates that forget
-// within a dozen tokens: value_side 615 -> 488 us, key_side 678 -> 408.  What is left is the shared memory's rate: two rows of
-// 64 slots a step for each of 128 rows, 8 k cycles a chunk at a dozen steps, beside 8 k of the scan around it.)  The
-// accumulator's columns are turned into distances through a band in shared memory, kBand distances at a time, stored
-// [distance][row]: the chunk's 128 rows are then 128 consecutive words.
-constexpr int kBand = 32;
-static_assert(kBand * kCT * 4 == kPanelB, "a band is one operand panel");
-
-// Which 32 accumulator columns of the warp's rows the threads of `half` turn into distances of band k: a row's band lies in
-// two adjacent blocks of 32 columns.  (-1: outside the chunk)
-template <bool REV> __device__ __forceinline__ int band_block(int wq, int half, int k) {
-    const int blk = REV ? wq + k + half : wq - k - half;
-    return blk >= 0 && blk < kCT / 32 ? blk : -1;
-}
-// The gate between j and the next row of the walk: prod_{r=j+1..i} becomes prod_{r=j..i}, reversed prod_{r=i+1..j}
-// prod_{r=i+1..j+1}.
-template <bool REV> __device__ __forceinline__ int next_gate_row(int j) { return REV ? min(j + 1, kCT - 1) : j; }
-template <bool REV> __device__ __forceinline__ int distance(int row, int j) { return REV ? j - row : row - j; }
-
-// Strong-decay chunk of value_side: this thread's 32 output slots of row `row`,
-//   out[s] = exp(+-..) * inter[s] + sum_j P_ij w_j[s] prod a_r[s]   (j <= i forward, j >= i reverse),
-// P and the inter-chunk product are read from the accumulators; the row goes straight to global
-// memory.  `gt` holds the per-step gates (gates_in_place), g_row this row's G; `band`: a panel nobody else uses.  Sixteen slots
-// at a time: with 32 at a time the scan around the walk spills, and every chunk of a flagged pair pays for it (the state
-// runs of 32 K tokens of strong gates 222 -> 277 us).
+// G of the token before step n, this lane's two slots (0 before a 128-token chunk, which G is local to)
 template <bool REV>
-__device__ __forceinline__ void value_side_explicit_rows(const unsigned char* gt, const unsigned char* sW, float* band,
-                                                      const float* gc, const float* g_row, uint32_t tmem, int wq,
-                                                      int row, int half, int sb, int valid, float* out_row) {
-    const unsigned char* ga = gt + half * kPanelB;           // this thread's 32 slots of the gates and of the weights
-    const unsigned char* wa = sW + half * kPanelB;
-#pragma unroll 1
-    for (int c0 = 0; c0 < kHS / 4; c0 += 4) {
-        float acc[16], dec[16];
+__device__ __forceinline__ float2 gate_before(const float* G, const Steps& steps, const ScanSpan& span, int T, int H, int n, int lane) {
+    const int t = steps.token<REV>(n);
+    if (n >= steps.count || steps.chunk_start(t)) return make_float2(0.f, 0.f);
+    return *reinterpret_cast<const float2*>(G + (((size_t)span.b * T + t - 1) * H + span.h) * kM + 2 * lane);
+}
+// this lane's two slots of G on the step's rows; past the end as on the last row (a gate of 1)
+__device__ __forceinline__ void step_gates(float2 (&g)[kSub], const unsigned char* tile, int rows, int lane) {
 #pragma unroll
-        for (int e = 0; e < 16; ++e) { acc[e] = 0.f; dec[e] = 1.f; }
-        bool live = row < valid;
-#pragma unroll 1
-        for (int k = 0; k < kCT / kBand; ++k) {
-            const int blk = band_block<REV>(wq, half, k);
-            if (blk >= 0) {
+    for (int j = 0; j < kSub; ++j) g[j] = unpack2(slots2(tile, j, lane));
+    if (rows < kSub) {
 #pragma unroll
-                for (int q = 0; q < 32; q += 16) {
-                    float v[16];
-                    tmem_ld16(tmem_row_addr(tmem, wq, kColP + 32 * blk + q), v);
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        const int d = distance<REV>(row, 32 * blk + q + e) - kBand * k;
-                        if (d >= 0 && d < kBand) band[d * kCT + row] = v[e];
-                    }
-                }
-            }
-            compute_sync();
-#pragma unroll 1
-            for (int d0 = 0; d0 < kBand; d0 += 4) {
-                if (!__any_sync(0xffffffffu, live)) break;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int d = kBand * k + d0 + u, j = REV ? row + d : row - d;
-                    live = live && (REV ? j < valid : j >= 0);
-                    if (!live) continue;
-                    const float p = band[(d0 + u) * kCT + row];
-                    const int jg = next_gate_row<REV>(j);
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const float4 a4 = *reinterpret_cast<const float4*>(ga + swz128(jg, c0 + c));
-                        const float4 w4 = *reinterpret_cast<const float4*>(wa + swz128(j, c0 + c));
-                        const float aj[4] = {a4.x, a4.y, a4.z, a4.w}, wj[4] = {w4.x, w4.y, w4.z, w4.w};
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            float& x = dec[4 * c + e];
-                            acc[4 * c + e] = fmaf(p * wj[e], x, acc[4 * c + e]);
-                            x *= aj[e];
-                        }
-                    }
-                }
-                float top = 0.f;
-#pragma unroll
-                for (int e = 0; e < 16; ++e) top = fmaxf(top, dec[e]);
-                live = live && top >= kDecayFloor;
-            }
-            if (!compute_sync_or(live)) break;       // (the barrier also covers: the band may be written again)
-        }
-        float vi[16], vj[16];
-        const int s0 = sb + 4 * c0;
-        tmem_ld16(tmem_row_addr(tmem, wq, kColO + s0), vi);
-        tmem_ld16(tmem_row_addr(tmem, wq, kColO + kM + s0), vj);       // (the state copy is a high/low pair)
-        if (row < valid) {
-#pragma unroll
-            for (int e = 0; e < 16; e += 4) {
-                const float4 g4 = *reinterpret_cast<const float4*>(g_row + s0 + e);
-                const float g[4] = {g4.x, g4.y, g4.z, g4.w};
-                float r[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    r[u] = fmaf(vi[e + u] + vj[e + u], __expf(REV ? gc[s0 + e + u] - g[u] : g[u]), acc[e + u]);
-                *reinterpret_cast<float4*>(out_row + s0 + e) = make_float4(r[0], r[1], r[2], r[3]);
-            }
-        }
+        for (int j = 1; j < kSub; ++j) g[j] = j < rows ? g[j] : g[j - 1];
     }
 }
 
 // ======================================================================================
 // value_side: out_i[s] = sum_{j<=i} <xq_i, xk_j> w_j[s] decay_ij[s]  + decayed (xq_i S)[s]
 // ======================================================================================
-// LAST = false: another scan of this CTA follows, which takes over the tensor memory.  Returns whether all went well
-// (the same for every thread); otherwise the tensor memory is freed and nothing may follow.
-// STATES: end memories only; of a chunk's products the state's alone is formed.
-template <bool REV, bool LAST = true, bool STATES = false>
-__device__ __noinline__ bool value_side_general(const CUtensorMap& mapQ, const CUtensorMap& mapK,
-                       const CUtensorMap& mapW, const CUtensorMap& mapG,
-                       const CUtensorMap& mapO, const ValueSideArgs& args,
-                       int32_t* dev_status,
-                       int slice) {
+// A slot warp's shared memory: the decayed weights w_j s_j [16][64] as a high/low pair, the step's total decay, the
+// inter-step product [16][64] from the state warps, P
+constexpr int kValueTotal = 2 * kDecTile, kValueO = kValueTotal + 4 * kM, kValueP = kValueO + kSub * kORow;
+constexpr int kValueSlotB = kValueP + kSub * kPRow;
+constexpr int kValueStageB = 2 * kXTile + 2 * kSlotTile, kValueStateStageB = kXTile + 2 * kSlotTile;
+
+// P = xq xk^T of a step, every value twice, into `out` (rows of kPRow bytes)
+__device__ __forceinline__ void step_scores(uint32_t xq, uint32_t xk, unsigned char* out, int lane) {
+    float p[2][2][4] = {};             // [keys 8 n ..][channels: even, odd blocks of 16]
+    const int q = lane >> 3, r = lane & 7;
+#pragma unroll
+    for (int kk = 0; kk < kDST / 16; ++kk) {
+        uint32_t fa[4], fb[4];
+        // A: rows 0-7, 8-15 of both channel halves; B: both channel halves of keys 0-7, 8-15
+        ldsm4(fa, x_at(xq, (q & 1) * 8 + r, 2 * kk + (q >> 1)));
+        ldsm4(fb, x_at(xk, (q >> 1) * 8 + r, 2 * kk + (q & 1)));
+        mma16816(p[0][kk & 1], fa, fb[0], fb[1]);
+        mma16816(p[1][kk & 1], fa, fb[2], fb[3]);
+    }
+    const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+    for (int n = 0; n < 2; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; e += 2) {
+            const float x = p[n][0][e] + p[n][1][e], y = p[n][0][e + 1] + p[n][1][e + 1];
+            *reinterpret_cast<float4*>(out + (g + 4 * e) * kPRow + 64 * n + 16 * t) = make_float4(x, x, y, y);
+        }
+}
+
+// STATES: end memories only (from empty ones).
+template <bool REV, bool STATES = false>
+__device__ __noinline__ bool value_side_general(const StepMaps maps, const ValueSideArgs& args, int32_t* dev_status, int slice) {
     // (a copy: through the reference every field would be read again after each barrier)
     const ValueSideArgs a = args;
     extern __shared__ unsigned char smem_raw[];
-    // align by pointer arithmetic (not an integer round trip) so accesses stay in the shared window
-    unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    unsigned char* sXq = smem;                       // 2 panels                                  (32 KB)
-    unsigned char* sXk = sXq + 2 * kPanelB;          // 2 panels                                  (32 KB)
-    unsigned char* sG = sXk + 2 * kPanelB;           // G tile fp32, [2 stages][2 panels]         (64 KB)
-    unsigned char* sW = sG + 4 * kPanelB;            // weight tile fp32, 2 panels                (32 KB)
-    unsigned char* sWa = sW + 2 * kPanelB;           // decayed weights, bf16 high part, MN-major B [128][64] (16 KB)
-    unsigned char* sWb = sWa + kPanelB;              // ... their bf16 rounding residual (low part)           (16 KB)
-    unsigned char* sSb = sWb + kPanelB;              // state copy, MN-major B [128][hi 64 | lo 64]  (32 KB)
-    Ctl* ctl = reinterpret_cast<Ctl*>(sSb + 2 * kPanelB);
-    // (the masked P never goes through shared memory: it is rewritten in place in tensor memory as a bf16
-    // high/low pair and read from there as the A operand of the intra-chunk product)
+    unsigned char* ring = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    constexpr int kStageB = STATES ? kValueStateStageB : kValueStageB;
+    unsigned char* slots = ring + kStages * kStageB;                  // of the slot warps
+    GeneralCtl* ctl = reinterpret_cast<GeneralCtl*>(slots + kSlotWarps * kValueSlotB);
 
-    const int tid = threadIdx.x, warp = tid >> 5, wq = warp & 3, half = (tid >> 7) & 1, row = tid & 127;
-    const int sb = kHS * half;          // this thread's first slot
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const ScanSpan span = scan_span(blockIdx.x, a.H, a.T, a.nseg, a.tseg);
-    const int bh = blockIdx.x, b = span.b, h = span.h;
     const int d0 = slice * kDST;
-    const size_t strideM = (size_t)a.H * kM;
-    float* obase = a.out + (size_t)slice * a.B * a.T * a.H * kM + ((size_t)b * a.T * a.H + h) * kM;
+    const Steps steps = STATES ? remembered_steps<REV>(a, span, lane) : all_steps(span);
+    general_ctl_init(ctl, tid);
 
-    ctl_init<true>(ctl, tid, warp);
-    const uint32_t tmem = ctl->tmem_slot;
-    const int nchunks = (span.t_end - span.t0 + kCT - 1) / kCT;
-    auto chunk_t0 = [&](int it) { return span.t0 + (REV ? nchunks - 1 - it : it) * kCT; };
-
-    if (warp == kComputeThreads / 32) {
-        // =============================== issuing warp: TMA loads / stores and all MMAs
-        if (elect_one()) {
-            auto load_x = [&](int it) {
-                const int t = chunk_t0(it);
-                mbar_expect_tx(&ctl->bar_x, (STATES ? 2 : 4) * kPanelB);
-                if (!STATES) {
-                    tma_load_4d(sXq, &mapQ, &ctl->bar_x, d0, h, t, b);
-                    tma_load_4d(sXq + kPanelB, &mapQ, &ctl->bar_x, d0 + 64, h, t, b);
-                }
-                tma_load_4d(sXk, &mapK, &ctl->bar_x, d0, h, t, b);
-                tma_load_4d(sXk + kPanelB, &mapK, &ctl->bar_x, d0 + 64, h, t, b);
-            };
-            auto load_g = [&](int it) {
-                const int t = chunk_t0(it), st = it & 1;
-                mbar_expect_tx(&ctl->bar_g[st], 2 * kPanelB);
-                tma_load_4d(sG + (2 * st) * kPanelB, &mapG, &ctl->bar_g[st], 0, h, t, b);
-                tma_load_4d(sG + (2 * st + 1) * kPanelB, &mapG, &ctl->bar_g[st], 32, h, t, b);
-            };
-            auto load_w = [&](int it) {
-                const int t = chunk_t0(it);
-                mbar_expect_tx(&ctl->bar_w, 2 * kPanelB);
-                tma_load_4d(sW, &mapW, &ctl->bar_w, 0, h, t, b);
-                tma_load_4d(sW + kPanelB, &mapW, &ctl->bar_w, 32, h, t, b);
-            };
-            prefetch_tmap(&mapQ); prefetch_tmap(&mapK); prefetch_tmap(&mapW); prefetch_tmap(&mapG); prefetch_tmap(&mapO);
-            load_g(0);
-            load_w(0);
-            load_x(0);
-            constexpr uint32_t idescP = make_idesc(128, 128, false, false);  // xq xk^T
-            constexpr uint32_t idescO = make_idesc(128, 2 * kM, false, true);  // xq x state copy [S_hi | S_lo] (MN-major B)
-            // the high and the low part of the weights are two adjacent 64-column panels of ONE
-            // MN-major B operand (N = 128): one product yields [.. W_hi | .. W_lo]
-            constexpr uint32_t idescU = make_idesc(128, 2 * kM, true, true);   // xk^T (MN-major A) x [W_hi | W_lo]
-            constexpr uint32_t idescI = make_idesc(128, 2 * kM, false, true);  // masked P (tensor memory) x [W_hi | W_lo]
-            // base descriptors of every operand (K step 0); advancing along K is one add each
-            const uint64_t dQk = desc_kmajor(smem_u32(sXq), 0), dKk = desc_kmajor(smem_u32(sXk), 0);
-            const uint64_t dKm = desc_mnmajor(smem_u32(sXk), 0, kPanelB), dWa = desc_mnmajor(smem_u32(sWa), 0, kPanelB);
-            const uint64_t dS = desc_mnmajor(smem_u32(sSb), 0, kPanelB);
-            // byte offset of K step kk: K-major operands walk 32 bytes inside a 64-column panel,
-            // MN-major operands walk 16 rows (2048 bytes)
-            auto kmaj = [](int kk) { return (uint32_t)((kk >> 2) * kPanelB + (kk & 3) * 32); };
-            auto mnmaj = [](int kk) { return (uint32_t)(kk * 2048); };
-            int n_mod = 0;      // moderate chunks so far (phases of bar_pm / bar_mma2)
-            PROF_DECL
-            for (int it = 0; it < nchunks && !ctl->abort; ++it) {
-                const int t0 = chunk_t0(it);
-                PROF_MARK();
-                const unsigned char* gt = sG + (2 * (it & 1)) * kPanelB;
-                // P = xq xk^T needs nothing but the d-sized tiles: it runs under the operand build
-                WAIT_OR_ABORT(&ctl->bar_x, it & 1);
-                tc_fence_after_sync();
-                PROF_MARK();
-                if (!STATES) {
+    if (warp >= kStateWarps && warp < kStateWarps + kSlotWarps) {
+        // =============================== slot warps: lane l has slots 2 l and 2 l + 1
+        const int w = warp - kStateWarps;
+        unsigned char* mine = slots + w * kValueSlotB;
+        float* obase = STATES ? nullptr : a.out + (size_t)slice * a.B * a.T * a.H * kM + 2 * lane;
+        load_step<REV, STATES ? 1 : 2, 1>(ctl, ring, maps, steps, span, d0, w);
+        float2 next = gate_before<REV>(a.G, steps, span, a.T, a.H, w, lane);
+        for (int n = w; n < steps.count; n += kSlotWarps) {
+            const int st = n % kStages, use = n / kSlotWarps;
+            unsigned char* tile = ring + st * kStageB;
+            const unsigned char *weights = tile + (STATES ? 1 : 2) * kXTile, *gates = weights + kSlotTile;
+            general_wait(ctl, &ctl->full[st], (n / kStages) & 1);
+            f32x2 E[kSub];                                           // w_j, later times the decay between j and i
+            float2 g[kSub];
+            const float2 before = next;
+            step_gates(g, gates, span.t_end - steps.token<REV>(n), lane);
 #pragma unroll
-                    for (int kk = 0; kk < kDST / 16; ++kk)
-                        mma_bf16(tmem + kColP, desc_advance(dQk, kmaj(kk)), desc_advance(dKk, kmaj(kk)), idescP, kk > 0);
-                    mma_commit(&ctl->bar_p);
-                }
-                // so does the inter-chunk product O = xq S: the state copy was written at the end
-                // of the previous chunk
-                WAIT_OR_ABORT(&ctl->bar_sb, it & 1);
-                tc_fence_after_sync();
-                if (!STATES) {
+            for (int j = 0; j < kSub; ++j) E[j] = slots2(weights, j, lane);
+            // decayed weights, total decay: what the state warps wait for
 #pragma unroll
-                    for (int kk = 0; kk < kDST / 16; ++kk)
-                        mma_bf16(tmem + kColO, desc_advance(dQk, kmaj(kk)), desc_advance(dS, mnmaj(kk)), idescO, kk > 0);
-                }
-                PROF_MARK();
-                if (it + 1 < nchunks) {
-                    bulk_wait_read();     // the output rows staged in that G buffer one chunk ago have left
-                    load_g(it + 1);
-                }
-                // U = xk^T W (high + low part of the weights) once the operand rows are there
-                PROF_MARK();
-                WAIT_OR_ABORT(&ctl->bar_ops, it & 1);
-                tc_fence_after_sync();
-                PROF_MARK();
-                const bool moderate = !STATES && ctl->moderate[it & 1] != 0;       // (... has an intra-chunk product)
+            for (int j0 = 0; j0 < kSub; j0 += kBatch) {
+                f32x2 f[kBatch];
 #pragma unroll
-                for (int kk = 0; kk < kCT / 16; ++kk)
-                    mma_bf16(tmem + kColU, desc_advance(dKm, mnmaj(kk)), desc_advance(dWa, mnmaj(kk)), idescU, kk > 0);
-                mma_commit(&ctl->bar_mma1);
-                PROF_MARK();
-                if (moderate) {
-                    WAIT_OR_ABORT(&ctl->bar_pm, n_mod & 1);
-                    tc_fence_after_sync();
-                    PROF_MARK();
+                for (int j = 0; j < kBatch; ++j) f[j] = REV ? decay2(before, g[j0 + j]) : decay2(g[j0 + j], g[kSub - 1]);
 #pragma unroll
-                    for (int kk = 0; kk < kCT / 16; ++kk)
-                        mma_bf16_ta(tmem + kColO2, tmem + kColP + 64 * (kk >> 2) + 8 * (kk & 3), desc_advance(dWa, mnmaj(kk)),
-                                    idescI, kk > 0);
-#pragma unroll
-                    for (int kk = 0; kk < kCT / 16; ++kk)      // ... and the rounding residual of the masked P
-                        mma_bf16_ta(tmem + kColO2, tmem + kColP + 64 * (kk >> 2) + 32 + 8 * (kk & 3),
-                                    desc_advance(dWa, mnmaj(kk)), idescI, true);
-                    mma_commit(&ctl->bar_mma2);
-                    PROF_MARK();
-                }
-                // the d-sized tiles are consumed once U and O are done: request the next chunk's
-                WAIT_OR_ABORT(&ctl->bar_mma1, it & 1);
-                PROF_MARK();
-                if (it + 1 < nchunks) load_x(it + 1);
-                if (moderate) {
-                    // the masked P is consumed: its buffer takes the next chunk's weight tile
-                    WAIT_OR_ABORT(&ctl->bar_mma2, n_mod & 1);
-                    ++n_mod;
-                    if (it + 1 < nchunks) load_w(it + 1);
-                }
-                PROF_MARK();
-                WAIT_OR_ABORT(&ctl->bar_out, it & 1);
-                PROF_MARK();
-                PROF_DUMP("value_side issue");
-                if (ctl->abort) break;
-                if (moderate) {
-                    tma_store_5d(&mapO, gt, 0, h, t0, b, slice);
-                    tma_store_5d(&mapO, gt + kPanelB, 32, h, t0, b, slice);
-                    bulk_commit();
-                } else if (!moderate && it + 1 < nchunks) {
-                    load_w(it + 1);       // a strong-decay chunk read the weight tile until now
-                }
+                for (int j = 0; j < kBatch; ++j) f[j] = mul2(E[j0 + j], f[j]);
+                store_pairs(mine, j0, lane, f);
             }
-            bulk_wait_read();      // staged output rows must have left before shared memory goes away
-        }
-    } else if (tid < kComputeThreads) {
-        // =============================== compute threads
-        // state slice: S[c = row][s], slots sb .. sb+31
-        float S[kHS];
-#pragma unroll
-        for (int s = 0; s < kHS; ++s) S[s] = (a.S0 && d0 + row < a.D) ? a.S0[((size_t)bh * kM + sb + s) * a.D + d0 + row] : 0.f;
-
-        // bf16 copy of the state (value + rounding residual) for the first chunk's inter-chunk product
-        store_state_row_split<false>(sSb, sSb + kPanelB, row, sb, S, nullptr);
-        fence_async_smem();
-        compute_sync();
-        if (tid == 0) mbar_arrive(&ctl->bar_sb);
-
-        int n_mod = 0;
-        PROF_DECL
-        for (int it = 0; it < nchunks; ++it) {
-            const int t0 = chunk_t0(it);
-            const int valid = min(kCT, span.t_end - t0);
-            PROF_MARK();
-            const unsigned char* gt = sG + (2 * (it & 1)) * kPanelB;
-            WAIT_OR_ABORT(&ctl->bar_g[it & 1], (it >> 1) & 1);
-            WAIT_OR_ABORT(&ctl->bar_w, it & 1);
-            PROF_MARK();
-            const bool moderate = publish_chunk_decay(ctl, tid, gt, valid - 1);
-            if (ctl->abort) break;
-            PROF_MARK();
-
-            // ---- this token's slot rows -> operand rows (rows past the end: zero weights)
-            const int grow = min(row, valid - 1);
-            const float strong = moderate ? 0.f : 1.f;      // adds G_C to the exponent of a strong-decay chunk
-#pragma unroll
-            for (int s0 = sb; s0 < sb + kHS; s0 += 8) {
-                float g[8], w[8], wd[8];
-                tile_row8(gt, grow, s0, g);
-                tile_row8(sW, row, s0, w);
-                // ONE set of decayed weights serves the intra-chunk product and the state update,
-                // branch-free over the elements (a branch per element would serialise the exps):
-                //   reverse           : w exp(G)
-                //   forward, moderate : w exp(-G); the state update gets its exp(G_C) afterwards,
-                //                       S <- exp(G_C) (S + xk^T W)
-                //   forward, strong   : w exp(G_C - G) (state update only; no intra product)
-                // They are stored as a bf16 pair (value + rounding residual): the weights multiply
-                // sums that cancel in the gate gradient, where a plain bf16 rounding is too coarse.
-                const float4 gc0 = *reinterpret_cast<const float4*>(&ctl->gc[s0]);
-                const float4 gc1 = *reinterpret_cast<const float4*>(&ctl->gc[s0 + 4]);
-                const float gcv[8] = {gc0.x, gc0.y, gc0.z, gc0.w, gc1.x, gc1.y, gc1.z, gc1.w};
-#pragma unroll
-                for (int e = 0; e < 8; ++e) wd[e] = w[e] * __expf(REV ? g[e] : fmaf(strong, gcv[e], -g[e]));
-                store_chunk_split(sWa, sWb, row, s0 >> 3, wd);
-            }
-            fence_async_smem();
-            if (tid == 0) ctl->moderate[it & 1] = moderate;
-            compute_sync();                     // every row is written and the weight tile is read
-            if (tid == 0) mbar_arrive(&ctl->bar_ops);
-            PROF_MARK();
-
-            if (!STATES) {
-                WAIT_OR_ABORT(&ctl->bar_p, it & 1);
-                tc_fence_after_sync();
-            }
-            PROF_MARK();
+            *reinterpret_cast<f32x2*>(mine + kValueTotal + 8 * lane) = decay2(before, g[kSub - 1]);
+            warp_arrive(&ctl->ready[w], lane);
+            // (the stage of this warp's next step: all are done with the step that it held, the one before this)
+            load_step<REV, STATES ? 1 : 2, 1>(ctl, ring, maps, steps, span, d0, n + kSlotWarps);
+            next = gate_before<REV>(a.G, steps, span, a.T, a.H, n + kSlotWarps, lane);
             if (STATES) {
-            } else if (moderate) {
-                mask_row_in_tmem<REV, true>(tmem, wq, row, half, kColP);
-                tc_fence_before_sync();
-                compute_sync();
-                if (tid == 0) mbar_arrive(&ctl->bar_pm);
-            } else {
-                // strong decay: the intra-chunk term by the walk over the per-step gates
-                WAIT_OR_ABORT(&ctl->bar_mma1, it & 1);    // the inter-chunk product
-                tc_fence_after_sync();
-                {
-                    gates_in_place(const_cast<unsigned char*>(gt), row, half, sb, valid);
-                    // (the band: the weights' operand rows, which the state product, complete, was the last to read)
-                    value_side_explicit_rows<REV>(gt, sW, reinterpret_cast<float*>(sWa), ctl->gc,
-                                                  a.G + (((size_t)b * a.T + t0 + row) * a.H + h) * kM, tmem, wq, row, half, sb, valid,
-                                                  obase + (size_t)(t0 + row) * strideM);
-                }
+                general_wait(ctl, &ctl->done[w], use & 1);
+                continue;
             }
-
-            // ---- state update from U: S <- S exp(G_C) + U  (forward moderate chunk: exp(G_C) (S + U))
-            PROF_MARK();
-            WAIT_OR_ABORT(&ctl->bar_mma1, it & 1);
-            tc_fence_after_sync();
-            PROF_MARK();
-            {
-                float v[kHS], vl[kHS];
-                tmem_ld32(tmem_row_addr(tmem, wq, kColU + sb), v);
-                tmem_ld32(tmem_row_addr(tmem, wq, kColU + kM + sb), vl);
+            step_scores(smem_u32(tile), smem_u32(tile + kXTile), mine + kValueP, lane);
+            __syncwarp();
+            f32x2 acc[kSub];
+            // intra-step rows: the products prod a_r are carried along by one multiplication a token, every factor <= 1
+            const unsigned char* scores = mine + kValueP;
 #pragma unroll
-                for (int e = 0; e < kHS; e += 4) {
-                    const float4 ec = *reinterpret_cast<const float4*>(&ctl->egc[sb + e]);
-                    const float ecv[4] = {ec.x, ec.y, ec.z, ec.w};
+            for (int ii = 0; ii < kSub; ++ii) {
+                const int i = REV ? kSub - 1 - ii : ii;
+                if (ii > 0) {
+                    const int at = REV ? i + 1 : i;
+                    const f32x2 x = decay2(g[at - 1], g[at]);
 #pragma unroll
-                    for (int t = 0; t < 4; ++t) {
-                        const float u = v[e + t] + vl[e + t];
-                        S[e + t] = (!REV && moderate) ? (S[e + t] + u) * ecv[t] : fmaf(S[e + t], ecv[t], u);
-                    }
+                    for (int jj = 0; jj < ii; ++jj) E[REV ? kSub - 1 - jj : jj] = mul2(E[REV ? kSub - 1 - jj : jj], x);
                 }
-            }
-            // its bf16 copy feeds the next chunk's inter-chunk product (issued as soon as the next
-            // tiles are there); the product of this chunk that read the old copy is complete
-            if (!STATES) store_state_row_split<false>(sSb, sSb + kPanelB, row, sb, S, nullptr);
-
-            // ---- output rows of a moderate chunk: exp(+-G_i) * (inter + intra)
-            PROF_MARK();
-            if (!STATES && moderate) {
-                WAIT_OR_ABORT(&ctl->bar_mma2, n_mod & 1);
-                ++n_mod;
-                tc_fence_after_sync();
-                PROF_MARK();
-                // the scaled rows replace this chunk's G rows in place (each thread reads and rewrites
-                // only its own 32 slots) and leave as one tiled store, clipped at the sequence end
-                float vo[kHS], vi[kHS];
-                tmem_ld32(tmem_row_addr(tmem, wq, kColO2 + sb), vo);
-                tmem_ld32(tmem_row_addr(tmem, wq, kColO2 + kM + sb), vi);
+                f32x2 sum[4];
 #pragma unroll
-                for (int e = 0; e < kHS; ++e) vo[e] += vi[e];          // high + low weight parts
-                {
-                    float vj[kHS];
-                    tmem_ld32(tmem_row_addr(tmem, wq, kColO + sb), vi);
-                    tmem_ld32(tmem_row_addr(tmem, wq, kColO + kM + sb), vj);
+                for (int u = 0; u < 4; ++u) sum[u] = pack2(0.f, 0.f);
 #pragma unroll
-                    for (int e = 0; e < kHS; ++e) vi[e] += vj[e];      // high + low state parts
+                for (int j0 = 0; j0 < kSub; j0 += 2) {
+                    const bool one = REV ? j0 >= i : j0 <= i, two = REV ? j0 + 1 >= i : j0 + 1 <= i;
+                    if (!one && !two) continue;
+                    const ulonglong2 p = *reinterpret_cast<const ulonglong2*>(scores + i * kPRow + 8 * j0);
+                    if (one) sum[j0 & 2] = fma2(p.x, E[j0], sum[j0 & 2]);
+                    if (two) sum[(j0 & 2) + 1] = fma2(p.y, E[j0 + 1], sum[(j0 & 2) + 1]);
                 }
-                // forward: exp(G) (inter + intra); reverse: exp(-G) (exp(G_C) inter + intra)
-#pragma unroll
-                for (int e = 0; e < kHS; ++e) vo[e] = REV ? fmaf(vi[e], ctl->egc[sb + e], vo[e]) : vo[e] + vi[e];
-                if (row < valid) {
-                    unsigned char* panel = const_cast<unsigned char*>(gt) + half * kPanelB;
-#pragma unroll
-                    for (int c = 0; c < kHS / 4; ++c) {
-                        float4* cell = reinterpret_cast<float4*>(panel + swz128(row, c));
-                        const float4 g = *cell;
-                        *cell = make_float4(vo[4 * c] * __expf(REV ? -g.x : g.x), vo[4 * c + 1] * __expf(REV ? -g.y : g.y),
-                                            vo[4 * c + 2] * __expf(REV ? -g.z : g.z), vo[4 * c + 3] * __expf(REV ? -g.w : g.w));
-                    }
-                }
+                acc[i] = add2(add2(sum[0], sum[1]), add2(sum[2], sum[3]));
             }
-            fence_async_smem();
-            tc_fence_before_sync();
-            compute_sync();                 // rows staged; gc / egc and the accumulators may be reused
-            if (tid == 0) {
-                mbar_arrive(&ctl->bar_sb);
-                mbar_arrive(&ctl->bar_out);
-            }
-            PROF_MARK();
-            PROF_DUMP("value_side compute");
-            if (ctl->abort) break;
+            // + the row factor times the inter-step product
+            f32x2 f[kSub];
+#pragma unroll
+            for (int j = 0; j < kSub; ++j) f[j] = REV ? decay2(g[j], g[kSub - 1]) : decay2(before, g[j]);
+            general_wait(ctl, &ctl->done[w], use & 1);
+            const int t = steps.token<REV>(n);
+            float* row = obase + (((size_t)span.b * a.T + t) * a.H + span.h) * kM;
+            const unsigned char* inter = mine + kValueO + 8 * lane;
+#pragma unroll
+            for (int j = 0; j < kSub; ++j) f[j] = fma2(f[j], *reinterpret_cast<const f32x2*>(inter + j * kORow), acc[j]);
+#pragma unroll
+            for (int j = 0; j < kSub; ++j)
+                if (t + j < span.t_end) *reinterpret_cast<f32x2*>(row + (size_t)j * a.H * kM) = f[j];
+            __syncwarp();
         }
-        if (!ctl->abort && a.Send && d0 + row < a.D) {
+    } else if (warp < kStateWarps) {
+        // =============================== state warps: S^T[16 slots][128 channels] as accumulator tiles [16 slots][8 channels]
+        constexpr int kTiles = kDST / 8;
+        const int s0 = 16 * warp, g = lane >> 2, t = lane & 3, q = lane >> 3, r = lane & 7;
+        const size_t state = ((size_t)blockIdx.x * kM + s0 + g) * a.D + d0 + 2 * t;
+        float S[kTiles][4];
 #pragma unroll
-            for (int s = 0; s < kHS; ++s) a.Send[((size_t)bh * kM + sb + s) * a.D + d0 + row] = S[s];
+        for (int nt = 0; nt < kTiles; ++nt)
+#pragma unroll
+            for (int e = 0; e < 4; e += 2) {
+                float2 x = make_float2(0.f, 0.f);
+                if (!STATES && d0 + 8 * nt < a.D && a.S0 != nullptr) x = *reinterpret_cast<const float2*>(a.S0 + state + (size_t)4 * e * a.D + 8 * nt);
+                S[nt][e] = x.x;
+                S[nt][e + 1] = x.y;
+            }
+        // the fragments' places in the tiles: channels 16 kb, 16 kb + 8
+        uint32_t at_q[kTiles / 2], at_k[kTiles / 2];
+#pragma unroll
+        for (int kb = 0; kb < kTiles / 2; ++kb) {
+            at_q[kb] = x_at(0, (q >> 1) * 8 + r, 2 * kb + (q & 1));
+            at_k[kb] = x_at(0, (q & 1) * 8 + r, 2 * kb + (q >> 1));
         }
-    }
-
-    tc_fence_before_sync();
-    __syncthreads();
-    if (ctl->abort) {
-        if (tid == 0 && dev_status != nullptr) *dev_status = GSA_ERR_TIMEOUT;
-        // bounded grace period for tile copies still in flight before shared memory goes away
-        for (int i = 0; i < 200; ++i) __nanosleep(1000);
-    }
-    const bool fine = ctl->abort == 0;
-    __syncthreads();
-    if ((LAST || !fine) && warp == 0) {
-        __syncwarp();
-        tmem_dealloc(tmem, kTmemCols);
-    }
-    return fine;
-}
-
-// Strong-decay chunk of key_side: A_ij = sum_s uq_i[s] uk_j[s] prod a_r[s] on the kept triangle, by
-// the same walk: the thread carries uq_i[s] times the running decay product for its 32 slots, one
-// multiplication per step and slot, and stops once every product is below 2^-40 of the largest it began with.  The two
-// threads of a row meet in two bands (over the uq rows, which are in registers by then); the sums go to the
-// accumulator's fp32 columns and from there, like those of a moderate chunk, into the masked bf16 operand rows.
-// `sG` is replaced by the per-step gates on the way.
-template <bool REV>
-__device__ __forceinline__ void key_side_explicit_rows(unsigned char* sG, unsigned char* sUq,
-                                                    const unsigned char* sUk, uint32_t tmem, int wq, int row, int half,
-                                                    int sb, int valid) {
-    float qd[kHS];
+        bool ready = false;
+        for (int n = 0; n < steps.count; ++n) {
+            const int st = n % kStages, w = n % kSlotWarps;
+            unsigned char* tile = ring + st * kStageB;
+            unsigned char* theirs = slots + w * kValueSlotB;
+            // (the slot warp has seen the rows land before it says that its own are ready)
+            if (!ready) general_wait(ctl, &ctl->ready[w], (n / kSlotWarps) & 1);
+            // W^T (rows: slots, k: tokens); xq (k: channels, columns: tokens); xk (k: tokens, columns: channels)
+            uint32_t wh[4], wl[4], x[2][4], y[2][4];
+            const uint32_t wa = smem_u32(theirs) + ((q >> 1) * 8 + r) * kDecRow + 2 * (s0 + (q & 1) * 8);
+            const uint32_t qa = smem_u32(tile), ka = smem_u32(tile + (STATES ? 0 : kXTile));
+            if (!STATES) ldsm4(x[0], qa + at_q[0]);
+            ldsm4_trans(y[0], ka + at_k[0]);
+            ldsm4_trans(wl, wa + kDecTile);
+            ldsm4_trans(wh, wa);
+            const float* total = reinterpret_cast<const float*>(theirs + kValueTotal) + s0 + g;
+            const f32x2 dec[2] = {pack2(total[0], total[0]), pack2(total[8], total[8])};
+            float O[2][2][4] = {};     // [tokens 8 n ..][high, low part of the state]
 #pragma unroll
-    for (int s0 = 0; s0 < kHS; s0 += 8) {
-        float uq[8];
-        tile_row8(sUq, row, sb + s0, uq);
+            for (int kb = 0; kb < kTiles / 2; ++kb) {
+                const uint32_t (&xb)[4] = x[kb & 1], (&yb)[4] = y[kb & 1];
+                uint32_t sh[4], sl[4];
+                if (!STATES) {
 #pragma unroll
-        for (int e = 0; e < 8; ++e) qd[s0 + e] = uq[e];
-    }
-    gates_in_place(sG, row, half, sb, valid);       // (its barriers also cover: every uq row is in registers)
-    {
-        uint32_t zero[16];
-#pragma unroll
-        for (int e = 0; e < 16; ++e) zero[e] = 0u;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) tmem_st16(tmem_row_addr(tmem, wq, kColP + 64 * half + 16 * q), zero);
-        tmem_st_wait();
-        tc_fence_before_sync();
-    }
-    float* band = reinterpret_cast<float*>(sUq + half * kPanelB);
-    const float *band0 = reinterpret_cast<const float*>(sUq), *band1 = reinterpret_cast<const float*>(sUq + kPanelB);
-    const unsigned char* ga = sG + half * kPanelB;
-    const unsigned char* ka = sUk + half * kPanelB;
-    float start = 0.f;
-#pragma unroll
-    for (int e = 0; e < kHS; ++e) start = fmaxf(start, fabsf(qd[e]));
-    const float floor_ = start * kDecayFloor;
-    bool live = start > 0.f;
-#pragma unroll 1
-    for (int k = 0; k < kCT / kBand; ++k) {
-#pragma unroll 1
-        for (int d0 = 0; d0 < kBand; d0 += 4) {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int d = kBand * k + d0 + u, j = REV ? row + d : row - d;
-                live = live && (REV ? j < valid : j >= 0);
-                float sum[4] = {0.f, 0.f, 0.f, 0.f};
-                if (live) {
-                    const int jg = next_gate_row<REV>(j);
-#pragma unroll
-                    for (int c = 0; c < kHS / 4; ++c) {
-                        const float4 a4 = *reinterpret_cast<const float4*>(ga + swz128(jg, c));
-                        const float4 k4 = *reinterpret_cast<const float4*>(ka + swz128(j, c));
-                        const float aj[4] = {a4.x, a4.y, a4.z, a4.w}, uk[4] = {k4.x, k4.y, k4.z, k4.w};
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            float& x = qd[4 * c + e];
-                            sum[e] = fmaf(x, uk[e], sum[e]);
-                            x *= aj[e];
-                        }
-                    }
+                    for (int e = 0; e < 4; ++e) split_pair(S[2 * kb + (e >> 1)][2 * (e & 1)], S[2 * kb + (e >> 1)][2 * (e & 1) + 1], sh[e], sl[e]);
                 }
-                band[(d0 + u) * kCT + row] = (sum[0] + sum[1]) + (sum[2] + sum[3]);
-            }
-            float top = 0.f;
+                if (kb + 1 < kTiles / 2) {
+                    if (!STATES) ldsm4(x[(kb + 1) & 1], qa + at_q[kb + 1]);
+                    ldsm4_trans(y[(kb + 1) & 1], ka + at_k[kb + 1]);
+                }
+                float U[2][4] = {};
+                mma16816(U[0], wl, yb[0], yb[1]);
+                mma16816(U[1], wl, yb[2], yb[3]);
+                if (!STATES) {
+                    mma16816(O[0][0], sh, xb[0], xb[1]);
+                    mma16816(O[1][0], sh, xb[2], xb[3]);
+                }
+                mma16816(U[0], wh, yb[0], yb[1]);
+                mma16816(U[1], wh, yb[2], yb[3]);
+                if (!STATES) {
+                    mma16816(O[0][1], sl, xb[0], xb[1]);
+                    mma16816(O[1][1], sl, xb[2], xb[3]);
+                }
+                // (is the next step's there? asked while the products run)
+                if (kb == 2) ready = n + 1 < steps.count && __all_sync(0xffffffffu, mbar_try(&ctl->ready[(n + 1) % kSlotWarps], ((n + 1) / kSlotWarps) & 1));
 #pragma unroll
-            for (int e = 0; e < kHS; ++e) top = fmaxf(top, fabsf(qd[e]));
-            live = live && top > floor_;
-        }
-        compute_sync();
-        tc_fence_after_sync();
-        const int blk = band_block<REV>(wq, half, k);
-        if (blk >= 0) {
-            float v[32];
-            tmem_ld32(tmem_row_addr(tmem, wq, kColP + 32 * blk), v);
-            uint32_t out[2][16];
+                for (int nn = 0; nn < 2; ++nn)
 #pragma unroll
-            for (int e = 0; e < 32; ++e) {
-                const int d = distance<REV>(row, 32 * blk + e) - kBand * k;
-                if (d >= 0 && d < kBand) v[e] = band0[d * kCT + row] + band1[d * kCT + row];
-                out[e >> 4][e & 15] = __float_as_uint(v[e]);
+                    for (int e = 0; e < 4; e += 2) decay_add(S[2 * kb + nn][e], S[2 * kb + nn][e + 1], dec[e >> 1], U[nn][e], U[nn][e + 1]);
             }
-            tmem_st16(tmem_row_addr(tmem, wq, kColP + 32 * blk), out[0]);
-            tmem_st16(tmem_row_addr(tmem, wq, kColP + 32 * blk + 16), out[1]);
-            tmem_st_wait();
+            if (!STATES) {
+                // (columns of the product are tokens: rows of kORow bytes 8 banks apart)
+                float* o = reinterpret_cast<float*>(theirs + kValueO) + s0 + g;
+#pragma unroll
+                for (int nn = 0; nn < 2; ++nn)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        o[(8 * nn + 2 * t + (e & 1)) * (kORow / 4) + 8 * (e >> 1)] = O[nn][0][e] + O[nn][1][e];
+            }
+            warp_arrive(&ctl->done[w], lane);
         }
-        tc_fence_before_sync();
-        const bool more = compute_sync_or(live);     // (the barrier also covers: the bands may be written again)
-        tc_fence_after_sync();
-        if (!more) break;
+        if (!ctl->abort && a.Send != nullptr) {           // (channels past D are zeros throughout and not written)
+#pragma unroll
+            for (int nt = 0; nt < kTiles; ++nt)
+#pragma unroll
+                for (int e = 0; e < 4; e += 2)
+                    if (d0 + 8 * nt < a.D) *reinterpret_cast<float2*>(a.Send + state + (size_t)4 * e * a.D + 8 * nt) = make_float2(S[nt][e], S[nt][e + 1]);
+        }
     }
-    mask_row_in_tmem<REV, true>(tmem, wq, row, half, kColP);
+    return general_finish(ctl, tid, dev_status);
 }
 
 // ======================================================================================
 // key_side: out_i = (uq_i * qscale_i) S + sum_j A_ij xv_j,  A_ij = sum_s uq_i[s] uk_j[s] decay_ij[s]
 // ======================================================================================
-template <bool REV, bool FIRST = true>
-__device__ __noinline__ void key_side_general(const CUtensorMap& mapV, const CUtensorMap& mapUq,
-                       const CUtensorMap& mapUk, const CUtensorMap& mapG,
-                       const CUtensorMap& mapO, const KeySideArgs& args,
-                       int32_t* dev_status) {
-    // (a copy: through the reference every field would be read again after each barrier)
-    const KeySideArgs a = args;
-    extern __shared__ unsigned char smem_raw[];
-    // align by pointer arithmetic (not an integer round trip) so accesses stay in the shared window
-    unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    unsigned char* sXv = smem;                       // 2 panels                                   (32 KB)
-    unsigned char* sUk = sXv + 2 * kPanelB;          // uk tile fp32, 2 panels                     (32 KB)
-    unsigned char* sG = sUk + 2 * kPanelB;           // G tile fp32, 2 panels                      (32 KB)
-    unsigned char* sUq = sG + 2 * kPanelB;           // uq tile fp32, 2 panels                     (32 KB)
-    unsigned char* sQt = sUq + 2 * kPanelB;          // decayed uq, K-major A [128][64]: value, rounding residual (32 KB)
-                                                     //   ... they also stage the output rows
-    unsigned char* sKt = sQt + 2 * kPanelB;          // decayed uk, K-major / MN-major B [128][64]: value, residual (32 KB)
-    unsigned char* sSb = sKt + 2 * kPanelB;          // state copy, K-major B [128 (channel)][64]: value, residual  (32 KB)
-    Ctl* ctl = reinterpret_cast<Ctl*>(sSb + 2 * kPanelB);
-    // (the masked A never goes through shared memory: it is rewritten in place in tensor memory as a bf16
-    // high/low pair and read from there as the A operand of the intra-chunk product)
+// A slot warp's shared memory: decayed uq and uk [16][64], each a high/low pair; a third pair for A (see step_weights); A as
+// a high/low pair [16 (i)][16 (j)]; the step's total decay
+constexpr int kKeyUk = 2 * kDecTile, kKeyZ = 4 * kDecTile, kKeyA = 6 * kDecTile, kKeyTotal = kKeyA + 2 * kSub * kARow;
+constexpr int kKeyOut = kKeyTotal + 4 * kM;          // ... and the output rows [16][128 channels]
+constexpr int kKeySlotB = kKeyOut + kSub * kOutRow;
+constexpr int kKeyStageB = kXTile + 3 * kSlotTile;
 
-    const int tid = threadIdx.x, warp = tid >> 5, wq = warp & 3, half = (tid >> 7) & 1, row = tid & 127;
-    const int sb = kHS * half;          // this thread's first slot
-    const ScanSpan span = scan_span(blockIdx.x, a.H, a.T, a.nseg, a.tseg);
-    const int bh = blockIdx.x, slice = blockIdx.y, b = span.b, h = span.h;
-    const int d0 = slice * kDST;
-
-    ctl_init<FIRST>(ctl, tid, warp);
-    const uint32_t tmem = ctl->tmem_slot;
-    const int nchunks = (span.t_end - span.t0 + kCT - 1) / kCT;
-    auto chunk_t0 = [&](int it) { return span.t0 + (REV ? nchunks - 1 - it : it) * kCT; };
-
-    if (warp == kComputeThreads / 32) {
-        // =============================== issuing warp: TMA loads / stores and all MMAs
-        if (elect_one()) {
-            auto load_v = [&](int it) {
-                const int t = chunk_t0(it);
-                mbar_expect_tx(&ctl->bar_x, 2 * kPanelB);
-                tma_load_4d(sXv, &mapV, &ctl->bar_x, d0, h, t, b);
-                tma_load_4d(sXv + kPanelB, &mapV, &ctl->bar_x, d0 + 64, h, t, b);
-            };
-            auto load_kg = [&](int it) {
-                const int t = chunk_t0(it);
-                mbar_expect_tx(&ctl->bar_g[0], 4 * kPanelB);
-                tma_load_4d(sUk, &mapUk, &ctl->bar_g[0], 0, h, t, b);
-                tma_load_4d(sUk + kPanelB, &mapUk, &ctl->bar_g[0], 32, h, t, b);
-                tma_load_4d(sG, &mapG, &ctl->bar_g[0], 0, h, t, b);
-                tma_load_4d(sG + kPanelB, &mapG, &ctl->bar_g[0], 32, h, t, b);
-            };
-            auto load_q = [&](int it) {
-                const int t = chunk_t0(it);
-                mbar_expect_tx(&ctl->bar_w, 2 * kPanelB);
-                tma_load_4d(sUq, &mapUq, &ctl->bar_w, 0, h, t, b);
-                tma_load_4d(sUq + kPanelB, &mapUq, &ctl->bar_w, 32, h, t, b);
-            };
-            prefetch_tmap(&mapV); prefetch_tmap(&mapUq); prefetch_tmap(&mapUk); prefetch_tmap(&mapG); prefetch_tmap(&mapO);
-            load_kg(0);
-            load_q(0);
-            load_v(0);
-            constexpr uint32_t idescA = make_idesc(128, 128, false, false);   // Q~ K~^T
-            constexpr uint32_t idescO = make_idesc(128, kDST, false, false);  // Q- x state copy (K-major B)
-            constexpr uint32_t idescU = make_idesc(128, 2 * kM, true, true);  // xv^T (MN-major A) x [K-_hi | K-_lo] (MN-major B)
-            constexpr uint32_t idescV = make_idesc(128, kDST, false, true);   // masked A (tensor memory) x xv (MN-major B)
-            // base descriptors of every operand (K step 0); advancing along K is one add each
-            const uint64_t dV = desc_mnmajor(smem_u32(sXv), 0, kPanelB);
-            const uint64_t dQt = desc_kmajor(smem_u32(sQt), 0), dKt = desc_kmajor(smem_u32(sKt), 0);
-            const uint64_t dQl = desc_kmajor(smem_u32(sQt + kPanelB), 0), dKl = desc_kmajor(smem_u32(sKt + kPanelB), 0);
-            const uint64_t dS = desc_kmajor(smem_u32(sSb), 0), dSl = desc_kmajor(smem_u32(sSb + kPanelB), 0);
-            // the decayed uk read MN-major, its value and residual as one N = 128 operand
-            const uint64_t dKtm = desc_mnmajor(smem_u32(sKt), 0, kPanelB);
-            auto kmaj = [](int kk) { return (uint32_t)((kk >> 2) * kPanelB + (kk & 3) * 32); };
-            auto mnmaj = [](int kk) { return (uint32_t)(kk * 2048); };
-            for (int it = 0; it < nchunks && !ctl->abort; ++it) {
-                const int t0 = chunk_t0(it);
-                WAIT_OR_ABORT(&ctl->bar_ops, it & 1);
-                WAIT_OR_ABORT(&ctl->bar_x, it & 1);
-                tc_fence_after_sync();
-                const bool moderate = ctl->moderate[it & 1] != 0;
-                if (moderate) {
-                    // A = Q- K-^T with both factors as bf16 high/low pairs (the low x low term is dropped)
+// c = X Y^T [16 x 16] over the 64 slots, both as high/low pairs (the low x low term is dropped)
+__device__ __forceinline__ void step_product(float (&c)[2][4], uint32_t x, uint32_t y, int lane) {
+    const int q = lane >> 3, r = lane & 7;
+    const uint32_t xa = x + ((q & 1) * 8 + r) * kDecRow + (q >> 1) * 16, ya = y + ((q >> 1) * 8 + r) * kDecRow + (q & 1) * 16;
+    float part[3][2][4] = {};
 #pragma unroll
-                    for (int kk = 0; kk < kM / 16; ++kk)
-                        mma_bf16(tmem + kColP, desc_advance(dQt, kmaj(kk)), desc_advance(dKt, kmaj(kk)), idescA, kk > 0);
+    for (int kk = 0; kk < kM / 16; ++kk) {
+        uint32_t xh[4], xl[4], yh[4], yl[4];
+        ldsm4(xh, xa + 32 * kk);
+        ldsm4(xl, xa + kDecTile + 32 * kk);
+        ldsm4(yh, ya + 32 * kk);
+        ldsm4(yl, ya + kDecTile + 32 * kk);
 #pragma unroll
-                    for (int kk = 0; kk < kM / 16; ++kk)
-                        mma_bf16(tmem + kColP, desc_advance(dQl, kmaj(kk)), desc_advance(dKt, kmaj(kk)), idescA, true);
-#pragma unroll
-                    for (int kk = 0; kk < kM / 16; ++kk)
-                        mma_bf16(tmem + kColP, desc_advance(dQt, kmaj(kk)), desc_advance(dKl, kmaj(kk)), idescA, true);
-                    mma_commit(&ctl->bar_p);     // the state products below run under the read-out of A
-                }
-                // the decayed uk is read K-major by the intra product and MN-major by the state update
-#pragma unroll
-                for (int kk = 0; kk < kCT / 16; ++kk)
-                    mma_bf16(tmem + kColU, desc_advance(dV, mnmaj(kk)), desc_advance(dKtm, mnmaj(kk)), idescU, kk > 0);
-#pragma unroll
-                for (int kk = 0; kk < kM / 16; ++kk)
-                    mma_bf16(tmem + kColO, desc_advance(dQt, kmaj(kk)), desc_advance(dS, kmaj(kk)), idescO, kk > 0);
-#pragma unroll
-                for (int kk = 0; kk < kM / 16; ++kk)
-                    mma_bf16(tmem + kColO, desc_advance(dQl, kmaj(kk)), desc_advance(dS, kmaj(kk)), idescO, true);
-#pragma unroll
-                for (int kk = 0; kk < kM / 16; ++kk)
-                    mma_bf16(tmem + kColO, desc_advance(dQt, kmaj(kk)), desc_advance(dSl, kmaj(kk)), idescO, true);
-                mma_commit(&ctl->bar_mma1);
-                // a moderate chunk is done with the uk and G tiles: request the next chunk's
-                if (moderate && it + 1 < nchunks) load_kg(it + 1);
-                WAIT_OR_ABORT(&ctl->bar_pm, it & 1);
-                tc_fence_after_sync();
-#pragma unroll
-                for (int kk = 0; kk < kCT / 16; ++kk)
-                    mma_bf16_ta(tmem + kColO, tmem + kColP + 64 * (kk >> 2) + 8 * (kk & 3), desc_advance(dV, mnmaj(kk)), idescV,
-                                true);
-#pragma unroll
-                for (int kk = 0; kk < kCT / 16; ++kk)      // ... and the rounding residual of A
-                    mma_bf16_ta(tmem + kColO, tmem + kColP + 64 * (kk >> 2) + 32 + 8 * (kk & 3), desc_advance(dV, mnmaj(kk)),
-                                idescV, true);
-                mma_commit(&ctl->bar_mma2);
-                if (!moderate && it + 1 < nchunks) load_kg(it + 1);
-                // every product of the chunk is done: the uq and xv tiles may be refilled
-                WAIT_OR_ABORT(&ctl->bar_mma2, it & 1);
-                if (it + 1 < nchunks) {
-                    load_q(it + 1);
-                    load_v(it + 1);
-                }
-                // the output rows are staged over the intra operands: store them, then tell the
-                // compute threads that those buffers may be rewritten
-                WAIT_OR_ABORT(&ctl->bar_out, it & 1);
-                if (ctl->abort) break;
-                tma_store_4d(&mapO, sQt, d0, h, t0, b);
-                if (d0 + 64 < a.D) tma_store_4d(&mapO, sQt + kPanelB, d0 + 64, h, t0, b);
-                bulk_commit();
-                bulk_wait_read();
-                mbar_arrive(&ctl->bar_sb);
-            }
-        }
-    } else if (tid < kComputeThreads) {
-        // =============================== compute threads
-        // state slice, transposed: S[c = row][s], slots sb .. sb+31
-        float S[kHS];
-#pragma unroll
-        for (int s = 0; s < kHS; ++s) S[s] = (a.S0 && d0 + row < a.D) ? a.S0[((size_t)bh * kM + sb + s) * a.D + d0 + row] : 0.f;
-
-        int n_mod = 0;     // moderate chunks so far (phases of bar_p)
-        PROF_DECL
-        for (int it = 0; it < nchunks; ++it) {
-            const int t0 = chunk_t0(it);
-            const int valid = min(kCT, span.t_end - t0);
-            (void)t0;
-            PROF_MARK();
-            WAIT_OR_ABORT(&ctl->bar_g[0], it & 1);
-            PROF_MARK();
-            const bool moderate = publish_chunk_decay(ctl, tid, sG, valid - 1);
-            if (ctl->abort) break;
-            PROF_MARK();
-
-            const int grow = min(row, valid - 1);
-            // the previous chunk's output rows must have left sQt / sKt before they are rewritten
-            if (it > 0) WAIT_OR_ABORT(&ctl->bar_sb, (it - 1) & 1);
-            // key side first: it needs the uk and G tiles only; the uq tile (which shares its buffer
-            // with the previous chunk's masked A) arrives last
-#pragma unroll
-            for (int s0 = sb; s0 < sb + kHS; s0 += 8) {
-                float g[8], uk[8], kd[8], gcv[8];
-                tile_row8(sG, grow, s0, g);
-                tile_row8(sUk, row, s0, uk);
-                // ONE decayed copy of uk serves the intra product and the state update, with one
-                // exponential per element (the SFU is the scarce unit here) and no branch:
-                //   reverse           : uk exp(G)
-                //   forward, moderate : uk exp(-G); the state update gets its exp(G_C) afterwards,
-                //                       S <- exp(G_C) (S + xv^T K)
-                //   forward, strong   : uk exp(G_C - G) (state update only)
-#pragma unroll
-                for (int e = 0; e < 8; ++e) gcv[e] = 0.f;
-                if (!REV && !moderate) tile_free_row8(&ctl->gc[s0], gcv);
-#pragma unroll
-                for (int e = 0; e < 8; ++e) kd[e] = uk[e] * __expf(REV ? g[e] : gcv[e] - g[e]);
-                store_chunk_split(sKt, sKt + kPanelB, row, s0 >> 3, kd);
-            }
-            PROF_MARK();
-            WAIT_OR_ABORT(&ctl->bar_w, it & 1);
-            PROF_MARK();
-#pragma unroll
-            for (int s0 = sb; s0 < sb + kHS; s0 += 8) {
-                float g[8], uq[8], qd[8], gcv[8];
-                tile_row8(sG, grow, s0, g);
-                tile_row8(sUq, row, s0, uq);
-                // likewise ONE decayed copy of uq:
-                //   forward           : uq exp(G)
-                //   reverse, moderate : uq exp(-G); the inter-chunk product gets its exp(G_C) through
-                //                       the state copy, which is scaled per slot
-                //   reverse, strong   : uq exp(G_C - G)
-#pragma unroll
-                for (int e = 0; e < 8; ++e) gcv[e] = 0.f;
-                if (REV && !moderate) tile_free_row8(&ctl->gc[s0], gcv);
-#pragma unroll
-                for (int e = 0; e < 8; ++e) qd[e] = uq[e] * __expf(REV ? gcv[e] - g[e] : g[e]);
-                store_chunk_split(sQt, sQt + kPanelB, row, s0 >> 3, qd);
-            }
-            if (REV && moderate) store_state_row_split<true>(sSb, sSb + kPanelB, row, sb, S, ctl->egc);
-            else store_state_row_split<false>(sSb, sSb + kPanelB, row, sb, S, nullptr);
-            fence_async_smem();
-            if (tid == 0) ctl->moderate[it & 1] = moderate;
-            compute_sync();
-            if (tid == 0) mbar_arrive(&ctl->bar_ops);
-            PROF_MARK();
-
-            if (moderate) {
-                WAIT_OR_ABORT(&ctl->bar_p, n_mod & 1);
-                ++n_mod;
-                tc_fence_after_sync();
-                PROF_MARK();
-                mask_row_in_tmem<REV, true>(tmem, wq, row, half, kColP);
-            } else {
-                // strong decay: A_ij by the walk over the per-step gates
-                key_side_explicit_rows<REV>(sG, sUq, sUk, tmem, wq, row, half, sb, valid);
-                fence_async_smem();     // (gates and bands were written where the next tiles land)
-            }
-            tc_fence_before_sync();
-            compute_sync();
-            if (tid == 0) mbar_arrive(&ctl->bar_pm);
-            PROF_MARK();
-
-            // ---- state update from U^T: S <- exp(G_C) S + U^T  (forward moderate chunk: exp(G_C) (S + U^T))
-            WAIT_OR_ABORT(&ctl->bar_mma1, it & 1);
-            tc_fence_after_sync();
-            PROF_MARK();
-            {
-                float v[kHS], vl[kHS];
-                tmem_ld32(tmem_row_addr(tmem, wq, kColU + sb), v);
-                tmem_ld32(tmem_row_addr(tmem, wq, kColU + kM + sb), vl);
-#pragma unroll
-                for (int e = 0; e < kHS; ++e) v[e] += vl[e];          // value + residual of the decayed uk
-#pragma unroll
-                for (int e = 0; e < kHS; e += 4) {
-                    const float4 ec = *reinterpret_cast<const float4*>(&ctl->egc[sb + e]);
-                    const float ecv[4] = {ec.x, ec.y, ec.z, ec.w};
-#pragma unroll
-                    for (int t = 0; t < 4; ++t)
-                        S[e + t] = (!REV && moderate) ? (S[e + t] + v[e + t]) * ecv[t] : fmaf(S[e + t], ecv[t], v[e + t]);
-                }
-            }
-
-            // ---- output rows -> bf16, staged over the intra operands (consumed since bar_p), stored
-            // by the issuing warp, clipped at the sequence end
-            PROF_MARK();
-            WAIT_OR_ABORT(&ctl->bar_mma2, it & 1);
-            tc_fence_after_sync();
-            PROF_MARK();
-#pragma unroll 1
-            for (int c0 = 0; c0 < 64; c0 += 32) {
-                float v[32];
-                tmem_ld32(tmem_row_addr(tmem, wq, kColO + 64 * half + c0), v);
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const float x[8] = {v[8 * c], v[8 * c + 1], v[8 * c + 2], v[8 * c + 3],
-                                        v[8 * c + 4], v[8 * c + 5], v[8 * c + 6], v[8 * c + 7]};
-                    store_chunk(sQt + half * kPanelB, row, (c0 >> 3) + c, x);
-                }
-            }
-            fence_async_smem();
-            tc_fence_before_sync();
-            compute_sync();
-            if (tid == 0) mbar_arrive(&ctl->bar_out);
-            PROF_MARK();
-            PROF_DUMP("key_side compute");
-            if (ctl->abort) break;
-        }
-        if (!ctl->abort && a.Send && d0 + row < a.D) {
-#pragma unroll
-            for (int s = 0; s < kHS; ++s) a.Send[((size_t)bh * kM + sb + s) * a.D + d0 + row] = S[s];
+        for (int nn = 0; nn < 2; ++nn) {
+            mma16816(part[0][nn], xl, yh[2 * nn], yh[2 * nn + 1]);
+            mma16816(part[1][nn], xh, yl[2 * nn], yl[2 * nn + 1]);
+            mma16816(part[2][nn], xh, yh[2 * nn], yh[2 * nn + 1]);
         }
     }
+#pragma unroll
+    for (int nn = 0; nn < 2; ++nn)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) c[nn][e] = part[2][nn][e] + (part[0][nn][e] + part[1][nn][e]);
+}
 
-    tc_fence_before_sync();
-    __syncthreads();
-    if (ctl->abort) {
-        if (tid == 0 && dev_status != nullptr) *dev_status = GSA_ERR_TIMEOUT;
-        for (int i = 0; i < 200; ++i) __nanosleep(1000);
-    }
-    __syncthreads();
-    if (warp == 0) {
+// A_ij = sum_s uq_i[s] uk_j[s] prod a_r[s] of a step, on the kept triangle, as accumulator fragments.  While no slot's decay
+// over the step is below e^-60: the decayed rows' product, its uk divided by the step's total decay (kFactorisedDecayMin is the
+// bound of the pipelined kernels' chunks, too).  Otherwise by halves: i and j in the two halves of a block of 2 L tokens meet
+// at the block's middle, to which both decay by factors <= 1; four levels L = 8, 4, 2, 1, of which a token plays one part in
+// each -- one pair of rows Z serves both sides -- and the diagonal.
+template <bool REV>
+__device__ __forceinline__ void step_weights(float (&c)[2][4], const unsigned char* uq, const unsigned char* uk, const unsigned char* gates,
+                                             const float2 (&g)[kSub], float2 before, int rows, unsigned char* mine, int lane) {
+    unsigned char* Z = mine + kKeyZ;
+    const float2 whole = make_float2(g[kSub - 1].x - before.x, g[kSub - 1].y - before.y);
+    if (__all_sync(0xffffffffu, fminf(whole.x, whole.y) >= kFactorisedDecayMin)) {
+        // forward: (uq_i e_i) (uk_j / e_j);  reversed: (uq_i s_i) (uk_j / s_j)
+#pragma unroll
+        for (int j0 = 0; j0 < kSub; j0 += kBatch) {
+            f32x2 f[kBatch];
+#pragma unroll
+            for (int j = 0; j < kBatch; ++j) f[j] = REV ? decay2(g[kSub - 1], g[j0 + j]) : decay2(g[j0 + j], before);
+#pragma unroll
+            for (int j = 0; j < kBatch; ++j) f[j] = mul2(slots2(uk, j0 + j, lane), f[j]);
+            store_pairs(Z, j0, lane, f);
+        }
         __syncwarp();
-        tmem_dealloc(tmem, kTmemCols);
+        step_product(c, smem_u32(mine), smem_u32(Z), lane);
+        return;
+    }
+    // (rolled loops: few registers, little code beside the usual case)
+    const int gr = lane >> 2, t = lane & 3;
+    auto gate = [&](int j) { return unpack2(slots2(gates, min(j, rows - 1), lane)); };
+#pragma unroll 1
+    for (int L = kSub / 2; L > 0; L >>= 1) {
+#pragma unroll 1
+        for (int j0 = 0; j0 < kSub; j0 += kBatch) {
+            f32x2 f[kBatch];
+#pragma unroll
+            for (int j = 0; j < kBatch; ++j) {
+                const int at = j0 + j, mid = (at & ~(2 * L - 1)) + L;         // the first token of the block's second half
+                const bool later = (at & L) != 0;
+                const float2 g0 = gate(mid - 1), g1 = gate(at);
+                f[j] = mul2(slots2(later != REV ? uq : uk, at, lane), later ? decay2(g0, g1) : decay2(g1, g0));
+            }
+            store_pairs(Z, j0, lane, f);
+        }
+        __syncwarp();
+        float part[2][4];
+        step_product(part, smem_u32(Z), smem_u32(Z), lane);
+        __syncwarp();
+#pragma unroll
+        for (int nn = 0; nn < 2; ++nn)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int d = (gr + 8 * (e >> 1)) ^ (8 * nn + 2 * t + (e & 1));
+                if (L == kSub / 2 || (d >= L && d < 2 * L)) c[nn][e] = part[nn][e];
+            }
+    }
+#pragma unroll 1
+    for (int j = 0; j < kSub; ++j) {
+        const float2 x = unpack2(mul2(slots2(uq, j, lane), slots2(uk, j, lane)));
+        float sum = x.x + x.y;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+#pragma unroll
+        for (int nn = 0; nn < 2; ++nn)
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (gr + 8 * (e >> 1) == j && 8 * nn + 2 * t + (e & 1) == j) c[nn][e] = sum;
     }
 }
 
-constexpr size_t kSmemGeneral = 1024 + 14 * kPanelB + sizeof(Ctl);
+template <bool REV>
+__device__ __noinline__ bool key_side_general(const StepMaps maps, const KeySideArgs& args, int32_t* dev_status) {
+    const KeySideArgs a = args;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* ring = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    unsigned char* slots = ring + kStages * kKeyStageB;
+    GeneralCtl* ctl = reinterpret_cast<GeneralCtl*>(slots + kSlotWarps * kKeySlotB);
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const ScanSpan span = scan_span(blockIdx.x, a.H, a.T, a.nseg, a.tseg);
+    const int d0 = blockIdx.y * kDST;
+    const Steps steps = all_steps(span);
+    general_ctl_init(ctl, tid);
+
+    if (warp >= kStateWarps && warp < kStateWarps + kSlotWarps) {
+        // =============================== slot warps: lane l has slots 2 l and 2 l + 1
+        const int w = warp - kStateWarps, gr = lane >> 2, t = lane & 3;
+        unsigned char* mine = slots + w * kKeySlotB;
+        load_step<REV, 1, 2>(ctl, ring, maps, steps, span, d0, w);
+        float2 next = gate_before<REV>(a.G, steps, span, a.T, a.H, w, lane);
+        for (int n = w; n < steps.count; n += kSlotWarps) {
+            const int st = n % kStages, use = n / kSlotWarps;
+            const unsigned char *queries = ring + st * kKeyStageB + kXTile, *keys = queries + kSlotTile, *gates = keys + kSlotTile;
+            general_wait(ctl, &ctl->full[st], (n / kStages) & 1);
+            float2 g[kSub];
+            const float2 before = next;
+            const int rows = min(kSub, span.t_end - steps.token<REV>(n));
+            step_gates(g, gates, rows, lane);
+            // (the stage of this warp's next step: all are done with the step that it held, the one before this)
+            load_step<REV, 1, 2>(ctl, ring, maps, steps, span, d0, n + kSlotWarps);
+            next = gate_before<REV>(a.G, steps, span, a.T, a.H, n + kSlotWarps, lane);
+#pragma unroll
+            for (int side = 0; side < 2; ++side) {         // uq, then uk
+#pragma unroll
+                for (int j0 = 0; j0 < kSub; j0 += kBatch) {
+                    f32x2 f[kBatch];
+#pragma unroll
+                    for (int j = 0; j < kBatch; ++j)
+                        f[j] = (side != 0) == REV ? decay2(before, g[j0 + j]) : decay2(g[j0 + j], g[kSub - 1]);
+#pragma unroll
+                    for (int j = 0; j < kBatch; ++j) f[j] = mul2(slots2(side != 0 ? keys : queries, j0 + j, lane), f[j]);
+                    store_pairs(mine + (side != 0 ? kKeyUk : 0), j0, lane, f);
+                }
+            }
+            *reinterpret_cast<f32x2*>(mine + kKeyTotal + 8 * lane) = decay2(before, g[kSub - 1]);
+            __syncwarp();
+            float c[2][4];
+            step_weights<REV>(c, queries, keys, gates, g, before, rows, mine, lane);
+            unsigned char* A = mine + kKeyA;
+#pragma unroll
+            for (int nn = 0; nn < 2; ++nn)
+#pragma unroll
+                for (int e = 0; e < 4; e += 2) {
+                    const int i = gr + 4 * e, j = 8 * nn + 2 * t;
+                    uint32_t hi, lo;
+                    split_pair((REV ? j >= i : j <= i) ? c[nn][e] : 0.f, (REV ? j + 1 >= i : j + 1 <= i) ? c[nn][e + 1] : 0.f, hi, lo);
+                    uint32_t* p = reinterpret_cast<uint32_t*>(A + i * kARow + 2 * j);
+                    p[0] = hi;
+                    p[kSub * kARow / 4] = lo;
+                }
+            warp_arrive(&ctl->ready[w], lane);
+            // the step's output rows
+            general_wait(ctl, &ctl->done[w], use & 1);
+            const int tok = steps.token<REV>(n) + (lane >> 4);
+            __nv_bfloat16* out = static_cast<__nv_bfloat16*>(a.out) + (((size_t)span.b * a.T + tok) * a.H + span.h) * a.D + d0 + 8 * (lane & 15);
+            const unsigned char* o_rows = mine + kKeyOut + (lane >> 4) * kOutRow + 16 * (lane & 15);
+            if (d0 + 8 * (lane & 15) < a.D) {
+#pragma unroll
+                for (int j = 0; j < kSub; j += 2)
+                    if (tok + j < span.t_end) *reinterpret_cast<uint4*>(out + (size_t)j * a.H * a.D) = *reinterpret_cast<const uint4*>(o_rows + j * kOutRow);
+            }
+            __syncwarp();
+        }
+    } else if (warp < kStateWarps) {
+        // =============================== state warps: S^T[32 channels][64 slots] as accumulator tiles [16 channels][8 slots]
+        constexpr int kMt = 2;
+        const int c0 = 16 * kMt * warp, g = lane >> 2, t = lane & 3, q = lane >> 3, r = lane & 7;
+        const bool live = d0 + c0 < a.D;           // (channels past D are zeros throughout and not written)
+        const size_t state = ((size_t)blockIdx.x * kM + 2 * t) * a.D + d0 + c0 + g;
+        float S[kMt][kM / 8][4];
+#pragma unroll
+        for (int mt = 0; mt < kMt; ++mt)
+#pragma unroll
+            for (int nt = 0; nt < kM / 8; ++nt)
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    S[mt][nt][e] = live && a.S0 != nullptr ? a.S0[state + (size_t)(8 * nt + (e & 1)) * a.D + 16 * mt + 8 * (e >> 1)] : 0.f;
+        uint32_t at_v[kMt];
+#pragma unroll
+        for (int mt = 0; mt < kMt; ++mt) at_v[mt] = x_at(0, (q >> 1) * 8 + r, c0 / 8 + 2 * mt + (q & 1));
+        bool ready = false;
+        for (int n = 0; n < steps.count; ++n) {
+            const int st = n % kStages, w = n % kSlotWarps;
+            unsigned char* theirs = slots + w * kKeySlotB;
+            // (the slot warp has seen the rows land before it says that its own are ready)
+            if (!ready) general_wait(ctl, &ctl->ready[w], (n / kSlotWarps) & 1);
+            // xv^T (rows: channels, k: tokens); uq (k: slots, columns: tokens); uk (k: tokens, columns: slots)
+            uint32_t x[kMt][4], ah[4], al[4], qh[2][4], ql[2][4], kh[2][4], kl[2][4];
+            const uint32_t va = smem_u32(ring + st * kKeyStageB);
+            const uint32_t qa = smem_u32(theirs) + ((q >> 1) * 8 + r) * kDecRow + (q & 1) * 16;
+            const uint32_t ka = smem_u32(theirs + kKeyUk) + ((q & 1) * 8 + r) * kDecRow + (q >> 1) * 16;
+            const uint32_t aa = smem_u32(theirs + kKeyA) + ((q >> 1) * 8 + r) * kARow + (q & 1) * 16;
+#pragma unroll
+            for (int mt = 0; mt < kMt; ++mt) ldsm4_trans(x[mt], va + at_v[mt]);
+            ldsm4_trans(kl[0], ka + kDecTile);
+            ldsm4(qh[0], qa);
+            ldsm4_trans(kh[0], ka);
+            ldsm4(ql[0], qa + kDecTile);
+            const float* total = reinterpret_cast<const float*>(theirs + kKeyTotal) + 2 * t;
+            float O[kMt][2][4] = {};     // [channels 16 mt ..][tokens 8 nn ..]
+#pragma unroll
+            for (int ks = 0; ks < kM / 16; ++ks) {
+                const int b = ks & 1;
+                uint32_t sh[kMt][4], sl[kMt][4];
+#pragma unroll
+                for (int mt = 0; mt < kMt; ++mt)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float (&f)[4] = S[mt][2 * ks + (e >> 1)];
+                        split_pair(f[2 * (e & 1)], f[2 * (e & 1) + 1], sh[mt][e], sl[mt][e]);
+                    }
+                const f32x2 dec[2] = {*reinterpret_cast<const f32x2*>(total + 16 * ks), *reinterpret_cast<const f32x2*>(total + 16 * ks + 8)};
+                if (ks + 1 < kM / 16) {
+                    ldsm4_trans(kl[b ^ 1], ka + kDecTile + 32 * (ks + 1));
+                    ldsm4(qh[b ^ 1], qa + 32 * (ks + 1));
+                    ldsm4_trans(kh[b ^ 1], ka + 32 * (ks + 1));
+                    ldsm4(ql[b ^ 1], qa + kDecTile + 32 * (ks + 1));
+                } else {
+                    ldsm4(al, aa + kSub * kARow);
+                    ldsm4(ah, aa);
+                }
+                float U[kMt][2][4] = {};
+#pragma unroll
+                for (int mt = 0; mt < kMt; ++mt)
+#pragma unroll
+                    for (int nn = 0; nn < 2; ++nn) mma16816(U[mt][nn], x[mt], kl[b][2 * nn], kl[b][2 * nn + 1]);
+#pragma unroll
+                for (int mt = 0; mt < kMt; ++mt)
+#pragma unroll
+                    for (int nn = 0; nn < 2; ++nn) mma16816(O[mt][nn], sl[mt], qh[b][2 * nn], qh[b][2 * nn + 1]);
+#pragma unroll
+                for (int mt = 0; mt < kMt; ++mt)
+#pragma unroll
+                    for (int nn = 0; nn < 2; ++nn) mma16816(U[mt][nn], x[mt], kh[b][2 * nn], kh[b][2 * nn + 1]);
+#pragma unroll
+                for (int mt = 0; mt < kMt; ++mt)
+#pragma unroll
+                    for (int nn = 0; nn < 2; ++nn) mma16816(O[mt][nn], sh[mt], ql[b][2 * nn], ql[b][2 * nn + 1]);
+#pragma unroll
+                for (int mt = 0; mt < kMt; ++mt)
+#pragma unroll
+                    for (int nn = 0; nn < 2; ++nn) {
+                        float (&f)[4] = S[mt][2 * ks + nn];
+#pragma unroll
+                        for (int e = 0; e < 4; e += 2) decay_add(f[e], f[e + 1], dec[nn], U[mt][nn][e], U[mt][nn][e + 1]);
+                    }
+#pragma unroll
+                for (int mt = 0; mt < kMt; ++mt)
+#pragma unroll
+                    for (int nn = 0; nn < 2; ++nn) mma16816(O[mt][nn], sh[mt], qh[b][2 * nn], qh[b][2 * nn + 1]);
+                // (is the next step's there? asked while the products run)
+                if (ks == 2) ready = n + 1 < steps.count && __all_sync(0xffffffffu, mbar_try(&ctl->ready[(n + 1) % kSlotWarps], ((n + 1) / kSlotWarps) & 1));
+            }
+            // intra-step rows, xv^T A^T
+#pragma unroll
+            for (int mt = 0; mt < kMt; ++mt)
+#pragma unroll
+                for (int nn = 0; nn < 2; ++nn) mma16816(O[mt][nn], x[mt], al[2 * nn], al[2 * nn + 1]);
+#pragma unroll
+            for (int mt = 0; mt < kMt; ++mt)
+#pragma unroll
+                for (int nn = 0; nn < 2; ++nn) mma16816(O[mt][nn], x[mt], ah[2 * nn], ah[2 * nn + 1]);
+            // output rows, token-major, for the slot warp to store
+            const uint32_t oa = smem_u32(theirs + kKeyOut) + ((q >> 1) * 8 + r) * kOutRow + 2 * c0 + (q & 1) * 16;
+#pragma unroll
+            for (int mt = 0; mt < kMt; ++mt)
+                stsm4_trans(oa + 32 * mt, pack_bf16(O[mt][0][0], O[mt][0][1]), pack_bf16(O[mt][0][2], O[mt][0][3]),
+                            pack_bf16(O[mt][1][0], O[mt][1][1]), pack_bf16(O[mt][1][2], O[mt][1][3]));
+            warp_arrive(&ctl->done[w], lane);
+        }
+        if (!ctl->abort && a.Send != nullptr && live) {
+#pragma unroll
+            for (int mt = 0; mt < kMt; ++mt)
+#pragma unroll
+                for (int nt = 0; nt < kM / 8; ++nt)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        a.Send[state + (size_t)(8 * nt + (e & 1)) * a.D + 16 * mt + 8 * (e >> 1)] = S[mt][nt][e];
+        }
+    }
+    return general_finish(ctl, tid, dev_status);
+}
+
+// the tensor maps of the scans' steps
+inline cudaError_t step_map(CUtensorMap* map, const void* base, int B, int T, int H, int D, int elem_bytes) {
+    return make_tensor_map_bthd(map, base, B, T, H, D, kSub, elem_bytes);
+}
+struct GeneralValueMaps {
+    CUtensorMap q, k, w, G;
+    __device__ __forceinline__ StepMaps steps() const { return {{&q, &k}, {&w, nullptr}, &G}; }
+};
+struct GeneralKeyMaps {
+    CUtensorMap v, uq, uk, G;
+    __device__ __forceinline__ StepMaps steps() const { return {{&v, nullptr}, {&uq, &uk}, &G}; }
+};
+inline cudaError_t make_general_maps(GeneralValueMaps* m, const ValueSideArgs& a) {
+    cudaError_t e = step_map(&m->q, a.xq, a.B, a.T, a.H, a.D, 2);
+    if (e == cudaSuccess) e = step_map(&m->k, a.xk, a.B, a.T, a.H, a.D, 2);
+    if (e == cudaSuccess) e = step_map(&m->w, a.w, a.B, a.T, a.H, kM, 4);
+    if (e == cudaSuccess) e = step_map(&m->G, a.G, a.B, a.T, a.H, kM, 4);
+    return e;
+}
+inline cudaError_t make_general_maps(GeneralKeyMaps* m, const KeySideArgs& a) {
+    cudaError_t e = step_map(&m->v, a.xv, a.B, a.T, a.H, a.D, 2);
+    if (e == cudaSuccess) e = step_map(&m->uq, a.uq, a.B, a.T, a.H, kM, 4);
+    if (e == cudaSuccess) e = step_map(&m->uk, a.uk, a.B, a.T, a.H, kM, 4);
+    if (e == cudaSuccess) e = step_map(&m->G, a.G, a.B, a.T, a.H, kM, 4);
+    return e;
+}
+
+constexpr size_t kSmemGeneralValue = kStages * kValueStageB + kSlotWarps * kValueSlotB;
+constexpr size_t kSmemGeneralKey = kStages * kKeyStageB + kSlotWarps * kKeySlotB;
+constexpr size_t kSmemGeneral = 1024 + (kSmemGeneralValue > kSmemGeneralKey ? kSmemGeneralValue : kSmemGeneralKey) + sizeof(GeneralCtl);
 
 }  // namespace
 }  // namespace gsa

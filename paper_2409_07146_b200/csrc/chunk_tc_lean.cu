@@ -14,7 +14,7 @@
 //     threads find their next accumulator ready when they finish a chunk.
 //   * tile copies and MMA issue are two lanes of two warps, so that a wait of one (for a store to
 //     drain, for a tile to land) never delays the other.
-// Tile geometry and the bounded waits are those of the general scans.
+// Every wait is bounded, as in the general scans.
 // The file also holds the state-only scan that segment-parallel scheduling uses for the end
 // memories of every segment (state_scan_kernel, below the two chunk kernels).
 #include "chunk_tc_general.cuh"
@@ -26,7 +26,7 @@ using namespace tcchunk;
 
 // 8 compute warps, one warp whose lane 0 issues every MMA, one warp whose lane 0 requests every
 // tile copy (loads and stores).  A CTA whose (batch, head) pair holds a strong-decay chunk runs the
-// general scan instead (chunk_tc_general.cuh); w, uq, uk and G as fp32 tiles (mapW32 ..) are for that.
+// general scan instead (chunk_tc_general.cuh).
 constexpr int kMmaWarp = kComputeThreads / 32, kCopyWarp = kMmaWarp + 1;   // (entered by one elected lane, see elect_one)
 
 struct LeanCtl {
@@ -119,12 +119,11 @@ template <bool REV, bool PAIRS>
 __global__ void __launch_bounds__(kScanThreads, 1)
 value_side_lean_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
                        const __grid_constant__ CUtensorMap mapWd, const __grid_constant__ CUtensorMap mapO,
-                       const __grid_constant__ CUtensorMap mapW32, const __grid_constant__ CUtensorMap mapG32,
-                       const __grid_constant__ ValueSideArgs a, const int* strong_flag, int32_t* dev_status) {
+                       const __grid_constant__ GeneralValueMaps general, const __grid_constant__ ValueSideArgs a, const int* strong_flag, int32_t* dev_status) {
     follow_previous_grid();
     if (strong_flag[blockIdx.x] != 0) {
         if (!REV) write_input_gate(a);
-        value_side_general<REV>(mapQ, mapK, mapW32, mapG32, mapO, a, dev_status, blockIdx.y);
+        value_side_general<REV>(general.steps(), a, dev_status, blockIdx.y);
         return;
     }
     extern __shared__ unsigned char smem_raw[];
@@ -381,12 +380,11 @@ template <bool REV, bool PAIRS>
 __global__ void __launch_bounds__(kScanThreads, 1)
 key_side_lean_kernel(const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapUq,
                      const __grid_constant__ CUtensorMap mapUk, const __grid_constant__ CUtensorMap mapO,
-                     const __grid_constant__ CUtensorMap mapUq32, const __grid_constant__ CUtensorMap mapUk32,
-                     const __grid_constant__ CUtensorMap mapG32, const __grid_constant__ KeySideArgs a,
+                     const __grid_constant__ GeneralKeyMaps general, const __grid_constant__ KeySideArgs a,
                      const int* strong_flag, int32_t* dev_status) {
     follow_previous_grid();
     if (strong_flag[blockIdx.x] != 0) {
-        key_side_general<REV>(mapV, mapUq32, mapUk32, mapG32, mapO, a, dev_status);
+        key_side_general<REV>(general.steps(), a, dev_status);
         return;
     }
     extern __shared__ unsigned char smem_raw[];
@@ -664,12 +662,13 @@ struct StateScanArgs {
     int slices0;
 };
 
+struct GeneralStateMaps { CUtensorMap x[2], w[2], G; };
+
 template <bool REV>
 __global__ void __launch_bounds__(kScanThreads, 1)
 state_scan_kernel(const __grid_constant__ CUtensorMap mapX0, const __grid_constant__ CUtensorMap mapW0,
-                  const __grid_constant__ CUtensorMap mapW32_0, const __grid_constant__ CUtensorMap mapX1,
-                  const __grid_constant__ CUtensorMap mapW1, const __grid_constant__ CUtensorMap mapW32_1,
-                  const __grid_constant__ CUtensorMap mapG32, const __grid_constant__ StateScanArgs sets,
+                  const __grid_constant__ CUtensorMap mapX1, const __grid_constant__ CUtensorMap mapW1,
+                  const __grid_constant__ GeneralStateMaps general, const __grid_constant__ StateScanArgs sets,
                   const int* strong_flag, int32_t* dev_status) {
     follow_previous_grid();
     const bool second = (int)blockIdx.y >= sets.slices0;
@@ -686,7 +685,8 @@ state_scan_kernel(const __grid_constant__ CUtensorMap mapX0, const __grid_consta
             seg_logdecay[(size_t)blockIdx.x * kM + threadIdx.x] = (float)sum;
         }
         if (!REV) write_input_gate(a);
-        value_side_general<REV, true, true>(mapX, mapX, second ? mapW32_1 : mapW32_0, mapG32, mapG32, a, dev_status, slice);
+        const StepMaps maps{{&general.x[second], nullptr}, {&general.w[second], nullptr}, &general.G};
+        value_side_general<REV, true>(maps, a, dev_status, slice);
         return;
     }
     const float* G = a.G;
@@ -830,8 +830,9 @@ constexpr size_t kSmemLeanKey = 1024 + 14 * kPanelB + sizeof(LeanCtl);     // ke
 cudaError_t launch_state_scan_tc(const ValueSideArgs& k, const ValueSideArgs& v, int reverse, const int* strong_flag,
                                  cudaStream_t st, int32_t* dev_status) {
     StateScanArgs sets{{k, v}, tc_value_side_slices(k.D)};
-    CUtensorMap mx[2], mw[2], mw32[2], mg;
-    cudaError_t e = make_tensor_map_bthd(&mg, k.G, k.B, k.T, k.H, kM, kCT, 4);
+    CUtensorMap mx[2], mw[2];
+    GeneralStateMaps general;
+    cudaError_t e = step_map(&general.G, k.G, k.B, k.T, k.H, kM, 4);
     for (int i = 0; i < 2; ++i) {
         ValueSideArgs& a = sets.set[i];
         a.xq = a.xk;
@@ -839,7 +840,8 @@ cudaError_t launch_state_scan_tc(const ValueSideArgs& k, const ValueSideArgs& v,
         a.out = nullptr;
         if (e == cudaSuccess) e = make_tensor_map_bthd(&mx[i], a.xk, a.B, a.T, a.H, a.D, kCT, 2);
         if (e == cudaSuccess) e = make_tensor_map_bthd(&mw[i], a.wd, a.B, a.T, a.H, 2 * kM, kCT, 2);
-        if (e == cudaSuccess) e = make_tensor_map_bthd(&mw32[i], a.w, a.B, a.T, a.H, kM, kCT, 4);
+        if (e == cudaSuccess) e = step_map(&general.x[i], a.xk, a.B, a.T, a.H, a.D, 2);
+        if (e == cudaSuccess) e = step_map(&general.w[i], a.w, a.B, a.T, a.H, kM, 4);
     }
     if (e != cudaSuccess) return e;
     dim3 grid(k.B * k.nseg * k.H, sets.slices0 + tc_value_side_slices(v.D));
@@ -847,12 +849,12 @@ cudaError_t launch_state_scan_tc(const ValueSideArgs& k, const ValueSideArgs& v,
     if (reverse) {
         e = prepare<state_scan_kernel<true>>(smem);
         if (e != cudaSuccess) return e;
-        launch_after(state_scan_kernel<true>, grid, kScanThreads, smem, st, mx[0], mw[0], mw32[0], mx[1], mw[1], mw32[1], mg, sets,
+        launch_after(state_scan_kernel<true>, grid, kScanThreads, smem, st, mx[0], mw[0], mx[1], mw[1], general, sets,
                                                                   strong_flag, dev_status);
     } else {
         e = prepare<state_scan_kernel<false>>(smem);
         if (e != cudaSuccess) return e;
-        launch_after(state_scan_kernel<false>, grid, kScanThreads, smem, st, mx[0], mw[0], mw32[0], mx[1], mw[1], mw32[1], mg, sets,
+        launch_after(state_scan_kernel<false>, grid, kScanThreads, smem, st, mx[0], mw[0], mx[1], mw[1], general, sets,
                                                                    strong_flag, dev_status);
     }
     return cudaGetLastError();
@@ -866,19 +868,19 @@ static bool tc_operands_ok(int M, int D, const void* wd, const void* uq_d, const
 cudaError_t launch_value_side_tc(const ValueSideArgs& a, int M, int reverse, const int* strong_flag, cudaStream_t st,
                                  int32_t* dev_status) {
     if (!tc_operands_ok(M, a.D, a.wd, a.wd, strong_flag)) return cudaErrorNotSupported;
-    CUtensorMap mq, mk, mw, mo, mw32, mg32;
+    CUtensorMap mq, mk, mw, mo;
+    GeneralValueMaps general;
     cudaError_t e = make_tensor_map_bthd(&mq, a.xq, a.B, a.T, a.H, a.D, kCT, 2);
     if (e == cudaSuccess) e = make_tensor_map_sliced(&mo, a.out, tc_value_side_slices(a.D), a.B, a.T, a.H, kM, kCT, 4);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&mk, a.xk, a.B, a.T, a.H, a.D, kCT, 2);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&mw, a.wd, a.B, a.T, a.H, 2 * kM, kCT, 2);
-    if (e == cudaSuccess) e = make_tensor_map_bthd(&mw32, a.w, a.B, a.T, a.H, kM, kCT, 4);
-    if (e == cudaSuccess) e = make_tensor_map_bthd(&mg32, a.G, a.B, a.T, a.H, kM, kCT, 4);
+    if (e == cudaSuccess) e = make_general_maps(&general, a);
     if (e != cudaSuccess) return e;
     dim3 grid(a.B * a.nseg * a.H, tc_value_side_slices(a.D));
     constexpr size_t smem = kSmemLeanValue > kSmemGeneral ? kSmemLeanValue : kSmemGeneral;
     auto launch = [&](auto kernel, cudaError_t ready) {
         if (ready != cudaSuccess) return ready;
-        launch_after(kernel, grid, kScanThreads, smem, st, mq, mk, mw, mo, mw32, mg32, a, strong_flag, dev_status);
+        launch_after(kernel, grid, kScanThreads, smem, st, mq, mk, mw, mo, general, a, strong_flag, dev_status);
         return cudaGetLastError();
     };
 #define GSA_VALUE(REV, PAIRS) launch(value_side_lean_kernel<REV, PAIRS>, prepare<value_side_lean_kernel<REV, PAIRS>>(smem))
@@ -890,20 +892,19 @@ cudaError_t launch_value_side_tc(const ValueSideArgs& a, int M, int reverse, con
 cudaError_t launch_key_side_tc(const KeySideArgs& a, int M, int reverse, const int* strong_flag, cudaStream_t st,
                                int32_t* dev_status) {
     if (!tc_operands_ok(M, a.D, a.uk_d, a.uq_d, strong_flag)) return cudaErrorNotSupported;
-    CUtensorMap mv, muq, muk, mo, muq32, muk32, mg32;
+    CUtensorMap mv, muq, muk, mo;
+    GeneralKeyMaps general;
     cudaError_t e = make_tensor_map_bthd(&mv, a.xv, a.B, a.T, a.H, a.D, kCT, 2);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&mo, a.out, a.B, a.T, a.H, a.D, kCT, 2);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&muq, a.uq_d, a.B, a.T, a.H, 2 * kM, kCT, 2);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&muk, a.uk_d, a.B, a.T, a.H, 2 * kM, kCT, 2);
-    if (e == cudaSuccess) e = make_tensor_map_bthd(&muq32, a.uq, a.B, a.T, a.H, kM, kCT, 4);
-    if (e == cudaSuccess) e = make_tensor_map_bthd(&muk32, a.uk, a.B, a.T, a.H, kM, kCT, 4);
-    if (e == cudaSuccess) e = make_tensor_map_bthd(&mg32, a.G, a.B, a.T, a.H, kM, kCT, 4);
+    if (e == cudaSuccess) e = make_general_maps(&general, a);
     if (e != cudaSuccess) return e;
     dim3 grid(a.B * a.nseg * a.H, tc_value_side_slices(a.D));
     constexpr size_t smem = kSmemLeanKey > kSmemGeneral ? kSmemLeanKey : kSmemGeneral;
     auto launch = [&](auto kernel, cudaError_t ready) {
         if (ready != cudaSuccess) return ready;
-        launch_after(kernel, grid, kScanThreads, smem, st, mv, muq, muk, mo, muq32, muk32, mg32, a, strong_flag, dev_status);
+        launch_after(kernel, grid, kScanThreads, smem, st, mv, muq, muk, mo, general, a, strong_flag, dev_status);
         return cudaGetLastError();
     };
 #define GSA_KEY(REV, PAIRS) launch(key_side_lean_kernel<REV, PAIRS>, prepare<key_side_lean_kernel<REV, PAIRS>>(smem))

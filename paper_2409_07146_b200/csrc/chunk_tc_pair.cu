@@ -61,18 +61,18 @@ struct PairCtl {
 // value-side output accumulate their high and low operand parts into 64 columns each
 constexpr int kPcP = 0, kPcA = 128, kPcO2 = 256, kPcU = 384, kPcOI = 448;
 
+struct GeneralPairMaps { CUtensorMap x, y, w, q, G; };
+
 template <bool PAIRS>
 __global__ void __launch_bounds__(kScanThreads, 1)
 rev_pair_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapY,
                 const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapQ,
                 const __grid_constant__ CUtensorMap mapOv, const __grid_constant__ CUtensorMap mapOk,
-                const __grid_constant__ CUtensorMap mapW32, const __grid_constant__ CUtensorMap mapQ32,
-                const __grid_constant__ CUtensorMap mapG32, const __grid_constant__ ValueSideArgs av,
-                const __grid_constant__ KeySideArgs ak, const int* strong_flag, int32_t* dev_status) {
+                const __grid_constant__ GeneralPairMaps general, const __grid_constant__ ValueSideArgs av, const __grid_constant__ KeySideArgs ak, const int* strong_flag, int32_t* dev_status) {
     follow_previous_grid();
     if (strong_flag[blockIdx.x] != 0) {             // the two general scans, one after the other
-        if (value_side_general<true, false>(mapY, mapX, mapW32, mapG32, mapOv, av, dev_status, blockIdx.y))
-            key_side_general<true, false>(mapX, mapQ32, mapW32, mapG32, mapOk, ak, dev_status);
+        if (value_side_general<true>(StepMaps{{&general.y, &general.x}, {&general.w, nullptr}, &general.G}, av, dev_status, blockIdx.y))
+            key_side_general<true>(StepMaps{{&general.x, nullptr}, {&general.q, &general.w}, &general.G}, ak, dev_status);
         return;
     }
     const float* G = ak.G;
@@ -463,22 +463,25 @@ bool rev_pair_supported(const ValueSideArgs& av, const KeySideArgs& ak, int M) {
 cudaError_t launch_rev_pair_tc(const ValueSideArgs& av, const KeySideArgs& ak, int M, const int* strong_flag,
                                cudaStream_t st, int32_t* dev_status) {
     if (!rev_pair_supported(av, ak, M) || strong_flag == nullptr) return cudaErrorNotSupported;
-    CUtensorMap mx, my, mw, mq, mov, mok, mw32, mq32, mg32;
+    CUtensorMap mx, my, mw, mq, mov, mok;
+    GeneralPairMaps general;
     cudaError_t e = make_tensor_map_bthd(&mx, ak.xv, ak.B, ak.T, ak.H, ak.D, kCT, 2);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&my, av.xq, av.B, av.T, av.H, av.D, kCT, 2);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&mw, av.wd, av.B, av.T, av.H, 2 * kM, kCT, 2);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&mq, ak.uq_d, ak.B, ak.T, ak.H, 2 * kM, kCT, 2);
     if (e == cudaSuccess) e = make_tensor_map_sliced(&mov, av.out, tc_value_side_slices(av.D), av.B, av.T, av.H, kM, kCT, 4);
     if (e == cudaSuccess) e = make_tensor_map_bthd(&mok, ak.out, ak.B, ak.T, ak.H, ak.D, kCT, 2);
-    if (e == cudaSuccess) e = make_tensor_map_bthd(&mw32, av.w, av.B, av.T, av.H, kM, kCT, 4);
-    if (e == cudaSuccess) e = make_tensor_map_bthd(&mq32, ak.uq, ak.B, ak.T, ak.H, kM, kCT, 4);
-    if (e == cudaSuccess) e = make_tensor_map_bthd(&mg32, ak.G, ak.B, ak.T, ak.H, kM, kCT, 4);
+    if (e == cudaSuccess) e = step_map(&general.x, ak.xv, ak.B, ak.T, ak.H, ak.D, 2);
+    if (e == cudaSuccess) e = step_map(&general.y, av.xq, av.B, av.T, av.H, av.D, 2);
+    if (e == cudaSuccess) e = step_map(&general.w, av.w, av.B, av.T, av.H, kM, 4);
+    if (e == cudaSuccess) e = step_map(&general.q, ak.uq, ak.B, ak.T, ak.H, kM, 4);
+    if (e == cudaSuccess) e = step_map(&general.G, ak.G, ak.B, ak.T, ak.H, kM, 4);
     if (e != cudaSuccess) return e;
     const dim3 grid(av.B * av.nseg * av.H, tc_value_side_slices(av.D));
     constexpr size_t smem = kSmemPair > kSmemGeneral ? kSmemPair : kSmemGeneral;
     auto launch = [&](auto kernel, cudaError_t ready) {
         if (ready != cudaSuccess) return ready;
-        launch_after(kernel, grid, kScanThreads, smem, st, mx, my, mw, mq, mov, mok, mw32, mq32, mg32, av, ak, strong_flag, dev_status);
+        launch_after(kernel, grid, kScanThreads, smem, st, mx, my, mw, mq, mov, mok, general, av, ak, strong_flag, dev_status);
         return cudaGetLastError();
     };
     return av.single ? launch(rev_pair_kernel<false>, prepare<rev_pair_kernel<false>>(smem))

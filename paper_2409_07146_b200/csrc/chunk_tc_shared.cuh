@@ -52,42 +52,8 @@ constexpr int kColO2 = 384;    // value_side: intra-chunk output [128 x 128], hi
 #define PROF_DUMP(name) do {} while (0)
 #endif
 
-// 8 consecutive fp32 values (columns s0 .. s0+7, s0 % 8 == 0) of row `row` of a slot-sized
-// fp32 tile: two panels of 32 columns, 128-byte swizzle.
-__device__ __forceinline__ void tile_row8(const unsigned char* tile, int row, int s0, float (&x)[8]) {
-    const unsigned char* panel = tile + (s0 >> 5) * kPanelB;
-    const int c = (s0 & 31) >> 2;
-    const float4 t0 = *reinterpret_cast<const float4*>(panel + swz128(row, c));
-    const float4 t1 = *reinterpret_cast<const float4*>(panel + swz128(row, c + 1));
-    x[0] = t0.x; x[1] = t0.y; x[2] = t0.z; x[3] = t0.w;
-    x[4] = t1.x; x[5] = t1.y; x[6] = t1.z; x[7] = t1.w;
-}
-// 8 consecutive floats from a 16-byte aligned plain (unswizzled) row
-__device__ __forceinline__ void tile_free_row8(const float* p, float (&x)[8]) {
-    const float4 t0 = *reinterpret_cast<const float4*>(p);
-    const float4 t1 = *reinterpret_cast<const float4*>(p + 4);
-    x[0] = t0.x; x[1] = t0.y; x[2] = t0.z; x[3] = t0.w;
-    x[4] = t1.x; x[5] = t1.y; x[6] = t1.z; x[7] = t1.w;
-}
-__device__ __forceinline__ float tile_elem(const unsigned char* tile, int row, int s) {
-    return *reinterpret_cast<const float*>(tile + (s >> 5) * kPanelB + swz128(row, (s & 31) >> 2) + (s & 3) * 4);
-}
-
-// bf16 copy of this thread's half state row (32 values from slot sb on, optionally scaled
-// per slot) into row `row` of a one-panel operand
-template <bool SCALE>
-__device__ __forceinline__ void store_state_row(unsigned char* panel, int row, int sb, const float (&S)[kHS],
-                                                const float* scale) {
-#pragma unroll
-    for (int c = 0; c < kHS / 8; ++c) {
-        float x[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) x[e] = SCALE ? S[8 * c + e] * scale[sb + 8 * c + e] : S[8 * c + e];
-        store_chunk(panel, row, (sb >> 3) + c, x);
-    }
-}
-
-// The same as a bf16 pair: the rounded copy and its rounding residual, in two panels
+// bf16 copy of this thread's half state row (32 values from slot sb on, optionally scaled per slot) into row `row` of two
+// one-panel operands: the rounded copy and its rounding residual
 template <bool SCALE>
 __device__ __forceinline__ void store_state_row_split(unsigned char* panel_hi, unsigned char* panel_lo, int row, int sb,
                                                       const float (&S)[kHS], const float* scale) {
@@ -102,18 +68,6 @@ __device__ __forceinline__ void store_state_row_split(unsigned char* panel_hi, u
 
 // Barrier over the 256 compute threads only (the issuing warp runs ahead on its own).
 __device__ __forceinline__ void compute_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
-__device__ __forceinline__ bool compute_sync_and(bool pred) {
-    uint32_t out;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.b32 q, %1, 0;\n\t"
-        "bar.red.and.pred p, 1, 256, q;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(out)
-        : "r"((uint32_t)pred)
-        : "memory");
-    return out != 0;
-}
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }

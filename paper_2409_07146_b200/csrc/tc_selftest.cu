@@ -1,6 +1,8 @@
 // Self-test of the tcgen05 building blocks: one 128-row product per operand-layout
 // combination that the chunk kernels use, on caller-provided 128 x 128 bf16 matrices.
 // It exists so that a wrong matrix descriptor or swizzle shows up in isolation.
+#include <string.h>
+
 #include "common.cuh"
 #include "gsa_dev.h"
 #include "tc_common.cuh"
@@ -25,10 +27,10 @@ cudaError_t get_encoder(EncodeFn* out) {
     *out = encode;
     return cudaSuccess;
 }
-}  // namespace
 
-cudaError_t make_tensor_map_sliced(CUtensorMap* map, const void* base, int nslice, int B, int T, int H, int D,
-                                   int box_rows, int elem_bytes) {
+thread_local TensorMapTable* g_maps = nullptr;
+
+cudaError_t encode_map(CUtensorMap* map, const void* base, int nslice, int B, int T, int H, int D, int box_rows, int elem_bytes) {
     EncodeFn encode;
     cudaError_t e = get_encoder(&encode);
     if (e != cudaSuccess) return e;
@@ -44,6 +46,27 @@ cudaError_t make_tensor_map_sliced(CUtensorMap* map, const void* base, int nslic
                         CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+}  // namespace
+
+TensorMapTable::TensorMapTable() : before(g_maps) { g_maps = this; }
+TensorMapTable::~TensorMapTable() { g_maps = before; }
+
+cudaError_t make_tensor_map_sliced(CUtensorMap* map, const void* base, int nslice, int B, int T, int H, int D,
+                                   int box_rows, int elem_bytes) {
+    TensorMapTable* t = g_maps;
+    const TensorMapTable::Key key{base, {nslice, B, T, H, D, box_rows, elem_bytes}};
+    for (int i = 0; t != nullptr && i < t->count; ++i)
+        if (memcmp(&t->keys[i], &key, sizeof(key)) == 0) {
+            *map = t->maps[i];
+            return cudaSuccess;
+        }
+    const cudaError_t e = encode_map(map, base, nslice, B, T, H, D, box_rows, elem_bytes);
+    if (e == cudaSuccess && t != nullptr && t->count < TensorMapTable::kCapacity) {
+        t->keys[t->count] = key;
+        t->maps[t->count++] = *map;
+    }
+    return e;
 }
 
 cudaError_t make_tensor_map_bthd(CUtensorMap* map, const void* base, int B, int T, int H, int D, int box_rows,
