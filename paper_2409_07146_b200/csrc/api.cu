@@ -292,14 +292,18 @@ InputGate input_gate_of(const gsa_params_t& p, const float* gate, bool left_out)
     return left_out ? InputGate{gate, p.gate_kind, inv_tau(p)} : InputGate{};
 }
 
-// the gate kernel: G, 1 - a, the decayed rows and the strong-decay flags (cleared by the caller)
+// the gate kernel: G, 1 - a, the decayed rows and the strong-decay flags, cleared first (which the CUDA-core kernels do without)
 // (input_gate = false: 1 - a is left out, see leaves_input_gate)
 cudaError_t gate_products(const gsa_params_t& p, Segments segs, const float* gate, const Workspace& w, bool input_gate,
                           cudaStream_t st) {
+    if (use_tc(p)) {
+        const cudaError_t e = launch_clear_flags(w.strong, (size_t)p.B * p.H * segs.n, st);
+        if (e != cudaSuccess) return e;
+    }
     if (use_wide(p))
         return launch_gate_cumsum_wide(gate, p.gate_kind, inv_tau(p), w.G, w.I, w.E, p.B, p.T, p.H, w.strong, segs.n, segs.t,
                                        w.Id, st, p.cu_seqlens, p.nseq);
-    return launch_gate_cumsum(gate, p.gate_kind, inv_tau(p), w.G, w.I, p.B, p.T, p.H, p.m, chunk_of(p), w.strong, segs.n,
+    return launch_gate_cumsum(gate, p.gate_kind, inv_tau(p), w.G, w.I, p.B, p.T, p.H, p.m, chunk_of(p), use_tc(p) ? w.strong : nullptr, segs.n,
                               segs.t, w.Id, p.io == GSA_BF16, st, p.cu_seqlens, p.nseq, input_gate ? 0 : 1);
 }
 // the row factors that the tensor-core value_side scans leave to the slot kernels
@@ -604,10 +608,10 @@ gsa_status_t fwd_core(const CallParams* params, int m_active, const void* q, con
     const int nseg = segs.n, tseg = segs.t;
     const bool left_out = leaves_input_gate(p, save_gate);
     const InputGate input_gate = input_gate_of(p, gate, left_out);
-    GSA_CUDA(cudaMemsetAsync(w.strong, 0, sizeof(int) * (size_t)p.B * p.H * nseg, st));
-    if (p.gate_kind == GSA_GATE_ABC)      // no decay, write weights from the cumulative softmax of the scores
+    if (p.gate_kind == GSA_GATE_ABC) {    // no decay, write weights from the cumulative softmax of the scores
+        GSA_CUDA(launch_clear_flags(w.strong, (size_t)p.B * p.H * nseg, st));
         GSA_LAUNCH("abc_write", launch_abc_write(gate, w.G, w.I, w.Id, p.B, p.T, p.H, p.m, st));
-    else
+    } else
         GSA_LAUNCH("gate_cumsum", gate_products(p, segs, gate, w, !left_out, st));
     float* ok = ok_save;      // the scaled logits leave the softmax kernel only if the caller keeps them
     // the pipelined kernels leave the row factor of the pass-1 sums to the softmax kernel
@@ -783,10 +787,10 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
     const bool left_out = !gate_is_saved && leaves_input_gate(p, true);
     const InputGate input_gate = input_gate_of(p, gate, left_out);
     if (!gate_is_saved) {      // (a forward of the same call left the gate kernel's products otherwise)
-        GSA_CUDA(cudaMemsetAsync(w.strong, 0, sizeof(int) * (size_t)p.B * p.H * nseg, st));
-        if (p.gate_kind == GSA_GATE_ABC)
+        if (p.gate_kind == GSA_GATE_ABC) {
+            GSA_CUDA(launch_clear_flags(w.strong, (size_t)p.B * p.H * nseg, st));
             GSA_LAUNCH("abc_write", launch_abc_write(gate, w.G, w.I, w.Id, p.B, p.T, p.H, p.m, st));
-        else
+        } else
             GSA_LAUNCH("gate_cumsum", gate_products(p, segs, gate, w, !left_out, st));
     }
     const float* ok = ok_saved;
@@ -1088,7 +1092,6 @@ gsa_status_t gsa_shard_states(const gsa_params_t* params, const void* k, const v
     if (ws_bytes < w.bytes) return GSA_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // one "segment" per batch element: the whole shard from empty memories, end memories only
-    GSA_CUDA(cudaMemsetAsync(w.strong, 0, sizeof(int) * (size_t)p.B * p.H, st));
     GSA_LAUNCH("gate_cumsum", gate_products(p, Segments{1, p.T}, gate, w, !leaves_input_gate(p, false), st));
     GSA_LAUNCH("segment_states", state_scans(p, Segments{1, p.T}, StateSet{k, w.I, w.Id, KT}, StateSet{v, w.I, w.Id, VT}, w, 0, logdecay,
                                               input_gate_of(p, gate, leaves_input_gate(p, false)), st,

@@ -224,6 +224,7 @@ struct PendingDecay {
 // below kFactorisedDecayMin (see InputGate).  fast_log: take log a with the
 // hardware base-2 logarithm (absolute error 2^-21.4 for a in [0.5, 1], 3 ulp below), for bf16 io.
 // gate_kind: gsa_gate_t (a, log a, or logits with inv_tau = 1/tau)
+cudaError_t launch_clear_flags(int* flags, size_t n, cudaStream_t st);
 cudaError_t launch_gate_cumsum(const float* gate, int gate_kind, float inv_tau, float* G, float* I,
                                int B, int T, int H, int M, int chunk, int* strong_flag, int nseg, int tseg,
                                void* decayed, int fast_log, cudaStream_t st, const int* cu_seqlens = nullptr,
