@@ -54,16 +54,22 @@ struct RowVec {
                 *reinterpret_cast<float2*>(row + (lane + 32 * r) * 2) = make_float2(v[r][0], v[r][1]);
         }
     }
-    // (the token's q, k, v: an access of kW values, as a row's; value by value, 48 loads a warp at D = 512: 24 layers of one sequence, 4 heads,
-    // 119.6 us, so 112.8)
+    // The token's q, k, v.  Heads of 256 and more: an access of kW values, as a row's; value by value they are 48 loads a warp at
+    // D = 512 (24 layers of one sequence, 4 heads of 512, 115 us value by value, so 109; 8 layers of 8, 8 heads of 256, 56 / 51).
+    // Narrow heads value by value: 8 layers of 100, 12 heads of 64, 148 / 161; 24 of one, 16 heads of 128, 104 / 106.
     template <typename IO>
     __device__ __forceinline__ void load_io(const IO* row, int lane) {
 #pragma unroll
         for (int r = 0; r < kN; ++r) {
-            struct alignas(sizeof(IO) * kW) Values { IO x[kW]; };
-            const Values t = *reinterpret_cast<const Values*>(row + (lane + 32 * r) * kW);
+            if constexpr (D >= 256) {
+                struct alignas(sizeof(IO) * kW) Values { IO x[kW]; };
+                const Values t = *reinterpret_cast<const Values*>(row + (lane + 32 * r) * kW);
 #pragma unroll
-            for (int w = 0; w < kW; ++w) v[r][w] = io_to_float<IO>(t.x[w]);
+                for (int w = 0; w < kW; ++w) v[r][w] = io_to_float<IO>(t.x[w]);
+            } else {
+#pragma unroll
+                for (int w = 0; w < kW; ++w) v[r][w] = io_to_float<IO>(row[(lane + 32 * r) * kW + w]);
+            }
         }
     }
     // the layer's feature map (Sec. 3.3), applied as the token's q, k, v are loaded
