@@ -779,7 +779,10 @@ template <int KIND, bool WIDE> struct GateGradRows {
         int off[kGGHalf];
 #pragma unroll
         for (int i = 0; i < kGGHalf; ++i) off[i] = i * 128 + ((q ^ i) << 4);          // (row & 7 == i)
-        auto at = [&](int tile, int i) { return *reinterpret_cast<const float*>(row + off[i] + tile * kGGTileB); };
+        take([&](int tile, int i) { return *reinterpret_cast<const float*>(row + off[i] + tile * kGGTileB); }, nslices, pending);
+    }
+    // at(tile, i): row i of a tile
+    template <class At> __device__ __forceinline__ void take(At&& at, int nslices, bool pending) {
 #pragma unroll
         for (int i = 0; i < kGGHalf; ++i) dI[i] = 0.f;
 #pragma unroll
@@ -1002,6 +1005,135 @@ __global__ void __launch_bounds__(kGGComputeThreads + 32) gate_grad_local_ring_k
     }
 }
 
+// The whole gradient in one pass, where (batch, head) pairs are enough: a CTA takes a pair, or a half or a quarter of its slots,
+// and walks its tiles from the last to the first, the running sum carried along -- a thread keeps its slot's in fp64 -- so that
+// nothing is written twice and no sums of blocks are scanned (3 of 9 streams at one slice a side).  Thread = (slot, group of eight
+// rows); a tile is as many rows as the threads have groups; a warp of one active lane copies the tiles of the stages ahead.
+// Bound by a tile's chain -- copies seen, eight rows of every stream, two barriers around the scan of the groups' sums by
+// shuffles (summed thread by thread it was half of the chain at 32 groups), rows out -- and by HBM where 128 CTAs walk all slots:
+// B = 4, T = 4096, 32 heads of 128 (0.8 GB) 212 -> 146 us, 5.5 TB/s; B = 8, T = 2048, 4 heads of 512 59 -> 47.5, with 128 slots
+// 98 -> 80.  512 threads, 16 KB a tile, where the slices of dI are few (256: 207); the next tile read ahead of the scan: 144 / 49.5.
+template <int KIND, bool WIDE, int NT>
+__global__ void __launch_bounds__(NT + 32) gate_grad_walk_kernel(
+    const __grid_constant__ CUtensorMap mapU, const __grid_constant__ CUtensorMap mapI,
+    const __grid_constant__ CUtensorMap mapGate, const __grid_constant__ CUtensorMap mapG,
+    const __grid_constant__ CUtensorMap mapDIk, const __grid_constant__ CUtensorMap mapDIv, int nsk, int nsv,
+    float inv_tau, float* __restrict__ dgate, int T, int H, int log_slots, int nstage, const float* dKT, const float* KT,
+    const float* dVT, const float* VT, int d_k, int d_v, PendingDecay pend, const int* cu, int nseq, int32_t* dev_status) {
+    follow_previous_grid();
+    using namespace tc;
+    constexpr int M = 64, kTile = NT * kGGHalf;          // elements of a tile
+    extern __shared__ unsigned char gg_smem_raw[];
+    unsigned char* smem0 = gg_smem_raw + ((128u - (smem_u32(gg_smem_raw) & 127u)) & 127u);
+    __shared__ uint64_t bar_full[kGGMaxStages], bar_empty[kGGMaxStages];
+    __shared__ float totals[NT + NT / 16], before[NT + NT / 16];      // [group][slot], rows one word longer than the slots
+    __shared__ int restarts[NT / 16];                    // does a packed sequence begin in the group?
+    __shared__ double final_term[M];
+    __shared__ volatile int failed_s;
+    const int slots = 1 << log_slots, groups = NT >> log_slots, tile_rows = groups * kGGHalf;
+    const int bh = blockIdx.x, b = bh / H, h = bh % H, s0 = blockIdx.y << log_slots;
+    const int ntile = (T + tile_rows - 1) / tile_rows;
+    // tiles: u, gate, G where a row factor is pending, the slices of dI, 1 - a unless the gate tensor gives it
+    const bool factor = pend.G != nullptr;
+    const int nslices = nsk + nsv, first_slice = factor ? 3 : 2, ntiles = first_slice + nslices + (KIND != GSA_GATE_A ? 1 : 0);
+    if (threadIdx.x == 0) {
+        failed_s = 0;
+        for (int s = 0; s < nstage; ++s) {
+            mbar_init(&bar_full[s], 1);
+            mbar_init(&bar_empty[s], NT / 32);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    if (threadIdx.x >= NT) {
+        if (elect_one()) {
+            // =============================== copy lane
+            for (int it = 0; it < ntile; ++it) {
+                const int s = it % nstage, t0 = (ntile - 1 - it) * tile_rows;
+                if (it >= nstage && !mbar_wait(&bar_empty[s], ((it / nstage) - 1) & 1)) {
+                    failed_s = 1;
+                    break;
+                }
+                unsigned char* smem = smem0 + (size_t)s * ntiles * (kTile * 4);
+                uint64_t* bar = &bar_full[s];
+                mbar_expect_tx(bar, (uint32_t)(ntiles * kTile * 4));
+                auto tile = [&](int i) { return smem + i * (kTile * 4); };
+                tma_load_4d(tile(0), &mapU, bar, s0, h, t0, b);
+                tma_load_4d(tile(1), &mapGate, bar, s0, h, t0, b);
+                if (factor) tma_load_4d(tile(2), &mapG, bar, s0, h, t0, b);
+                for (int sl = 0; sl < nslices; ++sl)
+                    tma_load_5d(tile(first_slice + sl), sl < nsk ? &mapDIk : &mapDIv, bar, s0, h, t0, b, sl < nsk ? sl : sl - nsk);
+                if (KIND != GSA_GATE_A) tma_load_4d(tile(ntiles - 1), &mapI, bar, s0, h, t0, b);
+            }
+        }
+    } else {
+        // =============================== compute warps
+        const int tx = threadIdx.x & (slots - 1), grp = threadIdx.x >> log_slots, mine = grp * (slots + 1) + tx;
+        // the groups' sums are scanned by as many lanes to a slot, the last group first: this thread's place there
+        const int rank = threadIdx.x & (groups - 1), scanned = (groups - 1 - rank) * (slots + 1) + threadIdx.x / groups;
+        auto csync = [] { asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory"); };
+        double carry = 0.0;
+        if (dKT != nullptr || dVT != nullptr) {
+            // final-memory term <dK~_T[s], K~_T[s]> + <dV~_T[s], V~_T[s]>: a warp per slot, lanes along the row
+            const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+            for (int slot = warp; slot < slots; slot += NT / 32) {
+                double dot = 0.0;
+                const size_t row = (size_t)bh * M + s0 + slot;
+                if (dKT != nullptr)
+                    for (int c = lane; c < d_k; c += 32) dot += (double)dKT[row * d_k + c] * (double)KT[row * d_k + c];
+                if (dVT != nullptr)
+                    for (int c = lane; c < d_v; c += 32) dot += (double)dVT[row * d_v + c] * (double)VT[row * d_v + c];
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+                if (lane == 0) final_term[slot] = dot;
+            }
+            csync();
+            carry = final_term[threadIdx.x / groups];
+        }
+        for (int it = 0; it < ntile; ++it) {
+            const int s = it % nstage, t0 = (ntile - 1 - it) * tile_rows, row0 = t0 + grp * kGGHalf;
+            const unsigned char* smem = smem0 + (size_t)s * ntiles * (kTile * 4) + (size_t)((grp * kGGHalf << log_slots) + tx) * 4;
+            if (!failed_s && !mbar_wait(&bar_full[s], (it / nstage) & 1)) failed_s = 1;     // (what is read then means nothing)
+            GateGradRows<KIND, WIDE> r;
+            // (in the order that GateGradRows names them: u, 1 - a, the gate, G, the slices)
+            const int place[4] = {0, ntiles - 1, 1, 2};
+            r.take([&](int tile, int i) {
+                return *reinterpret_cast<const float*>(smem + (tile < 4 ? place[tile] : first_slice + tile - 4) * (kTile * 4) + ((i * 4) << log_slots));
+            }, nslices, pend.pending_at(b, t0, h));
+            __syncwarp();
+            if ((threadIdx.x & 31) == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar_empty[s])) : "memory");
+            const uint32_t starts = starts_among(cu, nseq, row0, kGGHalf);
+            totals[mine] = r.total(starts);
+            if (cu != nullptr && tx == 0) restarts[grp] = starts != 0;
+            csync();
+            // a group passes on what it gets and its own sum; if a sequence begins in it, its own sum alone
+            double sum = (double)totals[scanned];
+            int restart = cu != nullptr ? restarts[groups - 1 - rank] : 0;
+            for (int o = 1; o < groups; o <<= 1) {
+                const double later = __shfl_up_sync(0xffffffffu, sum, o, groups);
+                const int later_restart = cu != nullptr ? __shfl_up_sync(0xffffffffu, restart, o, groups) : 0;
+                if (rank >= o) {
+                    if (restart == 0) sum += later;
+                    restart |= later_restart;
+                }
+            }
+            const double passed = (restart != 0 ? 0.0 : carry) + sum, got = __shfl_up_sync(0xffffffffu, passed, 1, groups);
+            before[scanned] = (float)(rank == 0 ? carry : got);
+            carry = __shfl_sync(0xffffffffu, passed, groups - 1, groups);
+            csync();
+            float* out = dgate + (((size_t)b * T + row0) * H + h) * M + s0 + tx;
+            r.write(before[mine], starts, T - row0, out, (uint32_t)H * M, inv_tau);
+        }
+    }
+    __syncthreads();
+    if (failed_s) {
+        if (threadIdx.x == 0 && dev_status != nullptr) *dev_status = GSA_ERR_TIMEOUT;
+        // bounded grace period for tile copies still in flight before shared memory goes away
+        for (int i = 0; i < 200; ++i) __nanosleep(1000);
+    }
+}
+
 // Adds what follows the block: dgate += carry (log gate) or carry / a (linear gate).  A thread
 // takes two slots of eight rows (half a block): threadIdx = (slot pair, block, half).
 template <int M, int KIND>
@@ -1062,6 +1194,25 @@ cudaError_t with_gate_kind(int gate_kind, int wide, F&& f) {
 
 int gate_grad_blocks(int T) { return (T + kGG - 1) / kGG; }
 
+// Does the gradient walk, and with how many slots to a CTA (as a power of two; 0: it takes the three kernels)?  A wave of walks
+// takes the same time however many SMs it fills; at a half and a quarter of the slots 0.57 and 0.39 of it.  The three kernels
+// take a 95th of it for a pair, and 0.12.  us at 2048 tokens, the three kernels / 16 / 32 / 64 slots: 20 pairs
+// (four slices a side) 44 / 44 / 66 / 120, logits 47 / 52 / 82 / 150, 28: 53 / 46 / 66 / 121, 40: 71 / 84 / 68 / 121, logits 75 / 97 /
+// 82 / 152, 72: 108 / 97 / 86 / 138; (one) 28: 36 / 31 / 46 / 80, 48: 53 / 56 / 47 / 80, 80: 75 / 76 / 80 / 76, 112: 100 / 117 / 82 / 78,
+// 160: 133 / 168 / 119 / 148, logits 151 / 199 / 156 / 195, 256: 219 / 256 / 160 / 152.
+constexpr int kWalkWideSlices = 3, kWalkSmem = 200 << 10;
+int walk_slots(int pairs, int nslices) {
+    if (nslices > kGGTmaMaxSlices) return 0;
+    const float wave[3] = {0.39f, 0.57f, 1.f};
+    float best = 0.95f * ((float)pairs / 95.f + 0.12f);
+    int log_slots = 0;
+    for (int i = 0; i < 3; ++i) {
+        const float cost = wave[i] * (float)((((long long)pairs << (2 - i)) + kSMs - 1) / kSMs);
+        if (cost < best) { best = cost; log_slots = 4 + i; }
+    }
+    return log_slots;
+}
+
 cudaError_t launch_gate_grad(const float* u, const float* I, const float* dIk_part, int nsk,
                              const float* dIv_part, int nsv, const float* gate,
                              int gate_kind, float inv_tau, const float* dKT, const float* KT,
@@ -1073,6 +1224,37 @@ cudaError_t launch_gate_grad(const float* u, const float* I, const float* dIk_pa
         pend.H = 2 * H;
         return launch_gate_grad(u, I, dIk_part, nsk, dIv_part, nsv, gate, gate_kind, inv_tau, dKT, KT, dVT, VT, d_k, d_v, blk_tot,
                                 dgate, B, T, 2 * H, 64, pend, st, dev_status, cu_seqlens, nseq);
+    }
+    const int log_slots = M == 64 ? walk_slots(B * H, nsk + nsv) : 0;
+    if (log_slots != 0) {
+        const int BH = B * H, nsl = nsk + nsv, cols = 1 << log_slots;
+        return with_gate_kind(gate_kind, pend.wide, [&](auto kind, auto wide) {
+            auto launch = [&](auto threads) {
+                constexpr int NT = decltype(threads)::value;
+                constexpr auto kernel = gate_grad_walk_kernel<decltype(kind)::value, decltype(wide)::value, NT>;
+                const int rows = NT / cols * kGGHalf;
+                const int ntiles = 2 + (pend.G != nullptr) + nsl + (gate_kind != GSA_GATE_A);
+                const int stage_bytes = ntiles * NT * kGGHalf * 4;
+                int nstage = (kWalkSmem - 128) / stage_bytes;
+                if (nstage > kGGMaxStages) nstage = kGGMaxStages;
+                CUtensorMap mu, mi, mg, mG, mk, mv;
+                const float* Gp = pend.G != nullptr ? pend.G : u;      // (unused without a pending factor)
+                cudaError_t e = make_tensor_map_sliced(&mu, u, 0, B, T, H, M, rows, 4, cols);
+                if (e == cudaSuccess) e = make_tensor_map_sliced(&mi, I, 0, B, T, H, M, rows, 4, cols);
+                if (e == cudaSuccess) e = make_tensor_map_sliced(&mg, gate, 0, B, T, H, M, rows, 4, cols);
+                if (e == cudaSuccess) e = make_tensor_map_sliced(&mG, Gp, 0, B, T, H, M, rows, 4, cols);
+                if (e == cudaSuccess) e = make_tensor_map_sliced(&mk, dIk_part, nsk, B, T, H, M, rows, 4, cols);
+                if (e == cudaSuccess) e = make_tensor_map_sliced(&mv, dIv_part, nsv, B, T, H, M, rows, 4, cols);
+                const size_t smem = 128 + (size_t)nstage * stage_bytes;
+                if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWalkSmem);
+                if (e != cudaSuccess) return e;
+                return launch_after(gate_grad_walk_kernel<decltype(kind)::value, decltype(wide)::value, NT>, dim3(BH, M >> log_slots), NT + 32, smem, st, mu, mi, mg, mG, mk, mv, nsk, nsv,
+                                    inv_tau, dgate, T, H, log_slots, nstage, dKT, KT, dVT, VT, d_k, d_v, pend, cu_seqlens, nseq, dev_status);
+            };
+            // (wide heads: 96 KB of tiles a stage as it is)
+            if (nsl > kWalkWideSlices) return launch(std::integral_constant<int, 256>{});
+            return launch(std::integral_constant<int, 512>{});
+        });
     }
     const int nblk = gate_grad_blocks(T);
     dim3 block(M / 2, 256 / M);      // 128 threads: M/2 slot pairs x 16-row blocks

@@ -318,15 +318,16 @@ __device__ __forceinline__ void store_elem(unsigned char* panel, int row, int co
 // head), 128-byte swizzle, zero fill beyond the tensor.
 cudaError_t make_tensor_map_bthd(CUtensorMap* map, const void* base, int B, int T, int H, int D, int box_rows,
                                  int elem_bytes);
-// The same over `nslice` stacked [B,T,H,D] tensors (a 5-D map; the slice is the last coordinate).
+// The same over `nslice` stacked [B,T,H,D] tensors (a 5-D map; the slice is the last coordinate).  box_cols > 0: a box of that
+// many columns, its rows one behind the other without a swizzle.
 cudaError_t make_tensor_map_sliced(CUtensorMap* map, const void* base, int nslice, int B, int T, int H, int D,
-                                   int box_rows, int elem_bytes);
+                                   int box_rows, int elem_bytes, int box_cols = 0);
 // The maps of one call, on its stack: while one is in scope the two functions above encode a map of a tensor and a box once
 // for all of the calling thread's launches (a map is a function of its arguments alone; a forward in segments asks for 25,
 // 13 different ones, 0.1 us each: T = 1431, 4 heads of 512, 51.1 us without, 50.7 with).
 struct TensorMapTable {
     static constexpr int kCapacity = 32;
-    struct Key { const void* base; int n[8]; };        // (slices, B, T, H, D, rows of the box, bytes of an element, 0)
+    struct Key { const void* base; int n[8]; };        // (slices, B, T, H, D, rows of the box, bytes of an element, columns)
     Key keys[kCapacity];
     CUtensorMap maps[kCapacity];
     int count = 0;

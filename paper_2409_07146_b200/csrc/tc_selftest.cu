@@ -30,7 +30,8 @@ cudaError_t get_encoder(EncodeFn* out) {
 
 thread_local TensorMapTable* g_maps = nullptr;
 
-cudaError_t encode_map(CUtensorMap* map, const void* base, int nslice, int B, int T, int H, int D, int box_rows, int elem_bytes) {
+cudaError_t encode_map(CUtensorMap* map, const void* base, int nslice, int B, int T, int H, int D, int box_rows, int elem_bytes,
+                       int box_cols) {
     EncodeFn encode;
     cudaError_t e = get_encoder(&encode);
     if (e != cudaSuccess) return e;
@@ -38,12 +39,12 @@ cudaError_t encode_map(CUtensorMap* map, const void* base, int nslice, int B, in
     const cuuint64_t dims[5] = {(cuuint64_t)D, (cuuint64_t)H, (cuuint64_t)T, (cuuint64_t)B, (cuuint64_t)nslice};
     const cuuint64_t strides[4] = {(cuuint64_t)D * eb, (cuuint64_t)H * D * eb, (cuuint64_t)T * H * D * eb,
                                    (cuuint64_t)B * T * H * D * eb};
-    const cuuint32_t box[5] = {(cuuint32_t)(128 / elem_bytes), 1, (cuuint32_t)box_rows, 1, 1};
+    const cuuint32_t box[5] = {(cuuint32_t)(box_cols > 0 ? box_cols : 128 / elem_bytes), 1, (cuuint32_t)box_rows, 1, 1};
     const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
     const cuuint32_t rank = nslice > 0 ? 5 : 4;
     CUresult r = encode(map, elem_bytes == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
                         rank, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                        box_cols > 0 ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
@@ -53,15 +54,15 @@ TensorMapTable::TensorMapTable() : before(g_maps) { g_maps = this; }
 TensorMapTable::~TensorMapTable() { g_maps = before; }
 
 cudaError_t make_tensor_map_sliced(CUtensorMap* map, const void* base, int nslice, int B, int T, int H, int D,
-                                   int box_rows, int elem_bytes) {
+                                   int box_rows, int elem_bytes, int box_cols) {
     TensorMapTable* t = g_maps;
-    const TensorMapTable::Key key{base, {nslice, B, T, H, D, box_rows, elem_bytes}};
+    const TensorMapTable::Key key{base, {nslice, B, T, H, D, box_rows, elem_bytes, box_cols}};
     for (int i = 0; t != nullptr && i < t->count; ++i)
         if (memcmp(&t->keys[i], &key, sizeof(key)) == 0) {
             *map = t->maps[i];
             return cudaSuccess;
         }
-    const cudaError_t e = encode_map(map, base, nslice, B, T, H, D, box_rows, elem_bytes);
+    const cudaError_t e = encode_map(map, base, nslice, B, T, H, D, box_rows, elem_bytes, box_cols);
     if (e == cudaSuccess && t != nullptr && t->count < TensorMapTable::kCapacity) {
         t->keys[t->count] = key;
         t->maps[t->count++] = *map;
