@@ -643,7 +643,7 @@ key_side_lean_kernel(const __grid_constant__ CUtensorMap mapV, const __grid_cons
 // chain is copy -> product -> read-out, with three tile stages and two accumulators, and reads
 // each of the two streams once.
 // ======================================================================================
-constexpr int kScanStages = 3;
+constexpr int kScanStages = 3, kBothStages = 2;      // (of 64 and of 96 KB)
 
 struct ScanCtl {
     uint64_t bar_x[kScanStages];      // (TMA) the tiles of a chunk have landed
@@ -656,7 +656,9 @@ struct ScanCtl {
 };
 
 // The K and the V memories (or their gradients) of a call go in one launch: the first `slices0` slices of the grid are
-// those of set 0, the rest those of set 1.
+// those of set 0, the rest those of set 1.  BOTH: a CTA runs both sets' one slice, which have the decayed rows in common: three
+// streams instead of four, where the CTAs are more than SMs anyway (forward over 32 K tokens, 16 heads of 128, 288 CTAs:
+// 98 -> 80 us, the call 489 -> 471).
 struct StateScanArgs {
     ValueSideArgs set[2];             // (xk, w and wd: the tile that enters the state and its weights; Send)
     int slices0;
@@ -664,7 +666,7 @@ struct StateScanArgs {
 
 struct GeneralStateMaps { CUtensorMap x[2], w[2], G; };
 
-template <bool REV>
+template <bool REV, bool BOTH>
 __global__ void __launch_bounds__(kScanThreads, 1)
 state_scan_kernel(const __grid_constant__ CUtensorMap mapX0, const __grid_constant__ CUtensorMap mapW0,
                   const __grid_constant__ CUtensorMap mapX1, const __grid_constant__ CUtensorMap mapW1,
@@ -686,15 +688,17 @@ state_scan_kernel(const __grid_constant__ CUtensorMap mapX0, const __grid_consta
         }
         if (!REV) write_input_gate(a);
         const StepMaps maps{{&general.x[second], nullptr}, {&general.w[second], nullptr}, &general.G};
-        value_side_general<REV, true>(maps, a, dev_status, slice);
+        if (value_side_general<REV, true>(maps, a, dev_status, slice) && BOTH)
+            value_side_general<REV, true>(StepMaps{{&general.x[1], nullptr}, {&general.w[1], nullptr}, &general.G}, sets.set[1], dev_status, 0);
         return;
     }
     const float* G = a.G;
     const int T = a.T, H = a.H, D = a.D;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    // a stage: X tile (2 panels of 64 channels) and the decayed rows [hi 64 | lo 64] (2 panels)
-    ScanCtl* ctl = reinterpret_cast<ScanCtl*>(smem + kScanStages * 4 * kPanelB);
+    // a stage: X tile (2 panels of 64 channels), of both sets, and the decayed rows [hi 64 | lo 64] (2 panels)
+    constexpr int kSets = BOTH ? 2 : 1, kStages_ = BOTH ? kBothStages : kScanStages, kStagePanels = 2 * kSets + 2;
+    ScanCtl* ctl = reinterpret_cast<ScanCtl*>(smem + kStages_ * kStagePanels * kPanelB);
 
     const int tid = threadIdx.x, warp = tid >> 5, wq = warp & 3, half = (tid >> 7) & 1, row = tid & 127;
     const int sb = kHS * half;          // this thread's first slot
@@ -703,7 +707,7 @@ state_scan_kernel(const __grid_constant__ CUtensorMap mapX0, const __grid_consta
     const int d0 = slice * kDST;
 
     if (tid == 0) {
-        for (int i = 0; i < kScanStages; ++i) {
+        for (int i = 0; i < kStages_; ++i) {
             mbar_init(&ctl->bar_x[i], 1);
             mbar_init(&ctl->bar_free[i], 1);
         }
@@ -729,20 +733,24 @@ state_scan_kernel(const __grid_constant__ CUtensorMap mapX0, const __grid_consta
         if (elect_one()) {
             // =============================== copy lane
             auto load = [&](int n) {
-                const int t = chunk_t0(n), st = n % kScanStages;
-                unsigned char* sX = smem + 4 * st * kPanelB;
-                mbar_expect_tx(&ctl->bar_x[st], 4 * kPanelB);
+                const int t = chunk_t0(n), st = n % kStages_;
+                unsigned char* sX = smem + kStagePanels * st * kPanelB;
+                mbar_expect_tx(&ctl->bar_x[st], kStagePanels * kPanelB);
                 tma_load_4d(sX, &mapX, &ctl->bar_x[st], d0, h, t, b);
                 tma_load_4d(sX + kPanelB, &mapX, &ctl->bar_x[st], d0 + 64, h, t, b);
-                tma_load_4d(sX + 2 * kPanelB, &mapW, &ctl->bar_x[st], 0, h, t, b);
-                tma_load_4d(sX + 3 * kPanelB, &mapW, &ctl->bar_x[st], 64, h, t, b);
+                if (BOTH) {
+                    tma_load_4d(sX + 2 * kPanelB, &mapX1, &ctl->bar_x[st], d0, h, t, b);
+                    tma_load_4d(sX + 3 * kPanelB, &mapX1, &ctl->bar_x[st], d0 + 64, h, t, b);
+                }
+                tma_load_4d(sX + 2 * kSets * kPanelB, &mapW, &ctl->bar_x[st], 0, h, t, b);
+                tma_load_4d(sX + (2 * kSets + 1) * kPanelB, &mapW, &ctl->bar_x[st], 64, h, t, b);
             };
             prefetch_tmap(&mapX); prefetch_tmap(&mapW);
-            for (int n = 0; n < kScanStages && n < nchunks; ++n) load(n);
-            for (int n = 0; n + kScanStages < nchunks && !ctl->abort; ++n) {
-                LEAN_WAIT(&ctl->bar_free[n % kScanStages], (n / kScanStages) & 1);
+            for (int n = 0; n < kStages_ && n < nchunks; ++n) load(n);
+            for (int n = 0; n + kStages_ < nchunks && !ctl->abort; ++n) {
+                LEAN_WAIT(&ctl->bar_free[n % kStages_], (n / kStages_) & 1);
                 if (ctl->abort) break;
-                load(n + kScanStages);
+                load(n + kStages_);
             }
         }
     } else if (warp == kMmaWarp) {
@@ -751,26 +759,32 @@ state_scan_kernel(const __grid_constant__ CUtensorMap mapX0, const __grid_consta
             constexpr uint32_t idescU = make_idesc(128, 2 * kM, true, true);   // X^T (MN-major A) x [W_hi | W_lo] (MN-major B)
             auto mnmaj = [](int kk) { return (uint32_t)(kk * 2048); };
             for (int n = 0; n < nchunks && !ctl->abort; ++n) {
-                const int st = n % kScanStages;
-                const uint32_t sX = smem_u32(smem + 4 * st * kPanelB);
-                const uint64_t dX = desc_mnmajor(sX, 0, kPanelB), dW = desc_mnmajor(sX + 2 * kPanelB, 0, kPanelB);
-                LEAN_WAIT(&ctl->bar_x[st], (n / kScanStages) & 1);
+                const int st = n % kStages_;
+                const uint32_t sX = smem_u32(smem + kStagePanels * st * kPanelB);
+                const uint64_t dW = desc_mnmajor(sX + 2 * kSets * kPanelB, 0, kPanelB);
+                LEAN_WAIT(&ctl->bar_x[st], (n / kStages_) & 1);
                 // the accumulator of chunk n-2 must have been read out
                 if (n >= 2) LEAN_WAIT(&ctl->bar_acc[n & 1], ((n - 2) >> 1) & 1);
                 if (ctl->abort) break;
                 tc_fence_after_sync();
 #pragma unroll
-                for (int kk = 0; kk < kCT / 16; ++kk)
-                    mma_bf16(tmem + 128 * (n & 1), desc_advance(dX, mnmaj(kk)), desc_advance(dW, mnmaj(kk)), idescU, kk > 0);
+                for (int set = 0; set < kSets; ++set) {
+                    const uint64_t dX = desc_mnmajor(sX + 2 * set * kPanelB, 0, kPanelB);
+#pragma unroll
+                    for (int kk = 0; kk < kCT / 16; ++kk)
+                        mma_bf16(tmem + 128 * (kSets * (n & 1) + set), desc_advance(dX, mnmaj(kk)), desc_advance(dW, mnmaj(kk)), idescU, kk > 0);
+                }
                 mma_commit(&ctl->bar_u[n & 1]);
                 mma_commit(&ctl->bar_free[st]);
             }
         }
     } else if (tid < kComputeThreads) {
         // =============================== compute threads: S[c = row][s], slots sb .. sb+31
-        float S[kHS];
+        float S[kSets][kHS];
 #pragma unroll
-        for (int s = 0; s < kHS; ++s) S[s] = 0.f;
+        for (int set = 0; set < kSets; ++set)
+#pragma unroll
+            for (int s = 0; s < kHS; ++s) S[set][s] = 0.f;
         // G of the last valid row of chunk n (threads 0..63, one slot each), one chunk ahead
         auto chunk_gc = [&](int n) {
             const int last = min(chunk_t0(n) + kCT, span.t_end) - 1;
@@ -794,10 +808,12 @@ state_scan_kernel(const __grid_constant__ CUtensorMap mapX0, const __grid_consta
             }
             LEAN_WAIT(&ctl->bar_u[n & 1], (n >> 1) & 1);
             tc_fence_after_sync();
-            {
+#pragma unroll
+            for (int set = 0; set < kSets; ++set) {
                 float v[kHS], vl[kHS];
-                tmem_ld32(tmem_row_addr(tmem, wq, 128 * (n & 1) + sb), v);
-                tmem_ld32(tmem_row_addr(tmem, wq, 128 * (n & 1) + kM + sb), vl);
+                const int col = 128 * (kSets * (n & 1) + set);
+                tmem_ld32(tmem_row_addr(tmem, wq, col + sb), v);
+                tmem_ld32(tmem_row_addr(tmem, wq, col + kM + sb), vl);
 #pragma unroll
                 for (int e = 0; e < kHS; e += 4) {
                     const float4 ec = *reinterpret_cast<const float4*>(&egc[sb + e]);
@@ -805,16 +821,24 @@ state_scan_kernel(const __grid_constant__ CUtensorMap mapX0, const __grid_consta
 #pragma unroll
                     for (int t = 0; t < 4; ++t) {
                         const float u = v[e + t] + vl[e + t];
-                        S[e + t] = REV ? fmaf(S[e + t], ecv[t], u) : (S[e + t] + u) * ecv[t];
+                        float& x = S[set][e + t];
+                        x = REV ? fmaf(x, ecv[t], u) : (x + u) * ecv[t];
                     }
                 }
             }
             // (the barrier inside also publishes the next chunk's egc)
             if (publish_and_vote(&ctl->bar_acc[n & 1], tid, ctl->abort != 0)) break;
         }
-        if (!ctl->abort && d0 + row < D) {
+        if (!ctl->abort) {
 #pragma unroll
-            for (int s = 0; s < kHS; ++s) a.Send[((size_t)bh * kM + sb + s) * D + d0 + row] = S[s];
+            for (int set = 0; set < kSets; ++set) {
+                const int width = BOTH ? sets.set[set].D : D;
+                float* end = BOTH ? sets.set[set].Send : a.Send;
+                if (d0 + row < width) {
+#pragma unroll
+                    for (int s = 0; s < kHS; ++s) end[((size_t)bh * kM + sb + s) * width + d0 + row] = S[set][s];
+                }
+            }
         }
         if (seg_logdecay != nullptr && tid < kM) seg_logdecay[(size_t)bh * kM + tid] = (float)decay;
     }
@@ -822,6 +846,7 @@ state_scan_kernel(const __grid_constant__ CUtensorMap mapX0, const __grid_consta
 }
 
 constexpr size_t kSmemStateScan = 1024 + kScanStages * 4 * kPanelB + sizeof(ScanCtl);
+static_assert(kBothStages * 6 == kScanStages * 4, "both in the same memory");
 constexpr size_t kSmemLeanValue = 1024 + 14 * kPanelB + sizeof(LeanCtl);   // value_side: 8 + 4 + 2 panels
 constexpr size_t kSmemLeanKey = 1024 + 14 * kPanelB + sizeof(LeanCtl);     // key_side: 4 + 8 + 2 panels
 
@@ -844,20 +869,18 @@ cudaError_t launch_state_scan_tc(const ValueSideArgs& k, const ValueSideArgs& v,
         if (e == cudaSuccess) e = step_map(&general.w[i], a.w, a.B, a.T, a.H, kM, 4);
     }
     if (e != cudaSuccess) return e;
-    dim3 grid(k.B * k.nseg * k.H, sets.slices0 + tc_value_side_slices(v.D));
+    const int scans = k.B * k.nseg * k.H;
+    const bool both = !reverse && sets.slices0 == 1 && tc_value_side_slices(v.D) == 1 && k.wd == v.wd && 2 * scans > kSMs;
+    const dim3 grid(scans, both ? 1 : sets.slices0 + tc_value_side_slices(v.D));
     constexpr size_t smem = kSmemStateScan > kSmemGeneral ? kSmemStateScan : kSmemGeneral;
-    if (reverse) {
-        e = prepare<state_scan_kernel<true>>(smem);
-        if (e != cudaSuccess) return e;
-        launch_after(state_scan_kernel<true>, grid, kScanThreads, smem, st, mx[0], mw[0], mx[1], mw[1], general, sets,
-                                                                  strong_flag, dev_status);
-    } else {
-        e = prepare<state_scan_kernel<false>>(smem);
-        if (e != cudaSuccess) return e;
-        launch_after(state_scan_kernel<false>, grid, kScanThreads, smem, st, mx[0], mw[0], mx[1], mw[1], general, sets,
-                                                                   strong_flag, dev_status);
-    }
-    return cudaGetLastError();
+    auto launch = [&](auto kernel, cudaError_t ready) {
+        if (ready != cudaSuccess) return ready;
+        launch_after(kernel, grid, kScanThreads, smem, st, mx[0], mw[0], mx[1], mw[1], general, sets, strong_flag, dev_status);
+        return cudaGetLastError();
+    };
+    if (reverse) return launch(state_scan_kernel<true, false>, prepare<state_scan_kernel<true, false>>(smem));
+    return both ? launch(state_scan_kernel<false, true>, prepare<state_scan_kernel<false, true>>(smem))
+                : launch(state_scan_kernel<false, false>, prepare<state_scan_kernel<false, false>>(smem));
 }
 
 // Is there a kernel for these shapes and operands?

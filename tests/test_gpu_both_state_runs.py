@@ -1,0 +1,41 @@
+"""State runs of the K and the V memories by one CTA, which narrow heads take where the pairs' segments are more than half of the
+SMs: ragged last segments and chunks, unequal widths, flagged pairs beside others, offsets of packed sequences."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2409_07146_b200 as gsa
+from test_gpu_parity import check_bwd, check_fwd, run_bwd, run_fwd
+from util import TOL, rand_inputs, rel_err, to_dev, to_np
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,T,H,dk,dv", [(1, 4700, 8, 128, 128), (2, 3300, 6, 64, 128), (1, 4161, 10, 128, 64)])
+@pytest.mark.parametrize("flagged", [False, True])
+def test_both_memories_in_one_run(B, T, H, dk, dv, flagged):
+    m = 64
+    d = rand_inputs(40 + T, B, T, H, dk, dv, m, "bf16", init=True, final_grads=True)
+    if flagged:                                       # one segment of one head forgets everything now and then
+        d["gate"][0, T // 2: T // 2 + 200: 50, 1] = 1e-20
+    got, g = run_fwd(d, B, T, H, dk, dv, m, "bf16", impl="tc", log=True)
+    check_fwd(d, got, g, "bf16", log=True, tc=True)
+    gb, rb = run_bwd(d, B, T, H, dk, dv, m, "bf16", impl="tc", log=True)
+    # (not in units of the last place, of which the check takes two at 2e-2 of the rms, 2.4e-4 of it: among the 5 million elements of
+    # the longest case is one of dk that is 2.25 off, with single runs as well.  The bound is that of the tensor-core kernels.)
+    check_bwd(gb, rb, TOL["bf16"], tc=True, storage=False)
+
+
+def test_packed_sequences():
+    B, T, H, d_, m = 1, 4500, 8, 128, 64
+    d = rand_inputs(3, B, T, H, d_, d_, m, "bf16")
+    cu = [0, 700, 1000, 1010, 2048, 4499, T]
+    p = gsa.Params(B, T, H, d_, d_, m, io="bf16", cu_seqlens=torch.tensor(cu, dtype=torch.int32, device="cuda"))
+    q, k, v = (to_dev(d[n], "bf16") for n in ("q", "k", "v"))
+    logits = torch.empty(B, T, H, m, device="cuda")
+    gsa.gsa_fwd(p, q, k, v, to_dev(d["gate"]), ok_save=logits)
+    for a, b in zip(cu, cu[1:]):
+        part = {n: d[n][:, a:b] for n in ("q", "k", "v", "gate")}
+        ref = oracle.fwd(part["q"], part["k"], part["v"], part["gate"])["ok"]
+        assert rel_err(to_np(logits)[:, a:b], ref) <= TOL["bf16"]
