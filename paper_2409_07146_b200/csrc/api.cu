@@ -288,8 +288,11 @@ cudaError_t key_side(const gsa_params_t& p, const KeySideArgs& a, int reverse, c
 bool leaves_input_gate(const gsa_params_t& p, bool gate_gradient_follows) {
     return use_tc(p) && !use_wide(p) && p.gate_kind != GSA_GATE_ABC && (p.gate_kind == GSA_GATE_A || !gate_gradient_follows);
 }
+// ... and where the gate tensor holds a it is what they read (16 heads, 32 K tokens of strong gates:
+// the gate kernel 94 -> 82 us)
+bool reads_gate(const gsa_params_t& p) { return use_tc(p) && !use_wide(p) && p.gate_kind == GSA_GATE_A; }
 InputGate input_gate_of(const gsa_params_t& p, const float* gate, bool left_out) {
-    return left_out ? InputGate{gate, p.gate_kind, inv_tau(p)} : InputGate{};
+    return left_out && !reads_gate(p) ? InputGate{gate, p.gate_kind, inv_tau(p)} : InputGate{};
 }
 
 // the gate kernel: G, 1 - a, the decayed rows and the strong-decay flags, cleared first (which the CUDA-core kernels do without)
@@ -304,7 +307,7 @@ cudaError_t gate_products(const gsa_params_t& p, Segments segs, const float* gat
         return launch_gate_cumsum_wide(gate, p.gate_kind, inv_tau(p), w.G, w.I, w.E, p.B, p.T, p.H, w.strong, segs.n, segs.t,
                                        w.Id, st, p.cu_seqlens, p.nseq);
     return launch_gate_cumsum(gate, p.gate_kind, inv_tau(p), w.G, w.I, p.B, p.T, p.H, p.m, chunk_of(p), use_tc(p) ? w.strong : nullptr, segs.n,
-                              segs.t, w.Id, p.io == GSA_BF16, st, p.cu_seqlens, p.nseq, input_gate ? 0 : 1);
+                              segs.t, w.Id, p.io == GSA_BF16, st, p.cu_seqlens, p.nseq, reads_gate(p) ? 2 : (input_gate ? 0 : 1));
 }
 // the row factors that the tensor-core value_side scans leave to the slot kernels
 PendingDecay pending_decay(const gsa_params_t& p, Segments segs, const Workspace& w) {
@@ -322,7 +325,7 @@ cudaError_t state_scans(const gsa_params_t& p, Segments segs, StateSet ks, State
                         float* logdecay, InputGate input_gate, cudaStream_t st, int32_t* dev_status) {
     ValueSideArgs a[2] = {{ks.x, ks.x, ks.w, w.G, nullptr, ks.end, nullptr, p.B, p.T, p.H, p.d_k, ks.wd, 1},
                           {vs.x, vs.x, vs.w, w.G, nullptr, vs.end, nullptr, p.B, p.T, p.H, p.d_v, vs.wd, 1}};
-    for (ValueSideArgs& x : a) { x.nseg = segs.n; x.tseg = segs.t; x.E = w.E; x.input_gate = input_gate; }
+    for (ValueSideArgs& x : a) { x.nseg = segs.n; x.tseg = segs.t; x.E = w.E; x.input_gate = input_gate; x.w_keeps = !reverse && reads_gate(p); }
     if (use_wide(p)) {
         if (logdecay != nullptr) {
             const cudaError_t e = launch_segment_logdecay(w.G, logdecay, p.B, p.T, p.H, segs.n, segs.t, log_gate_chunk(p), st);
@@ -616,6 +619,8 @@ gsa_status_t fwd_core(const CallParams* params, int m_active, const void* q, con
     const int nseg = segs.n, tseg = segs.t;
     const bool left_out = leaves_input_gate(p, save_gate);
     const InputGate input_gate = input_gate_of(p, gate, left_out);
+    const float* I = reads_gate(p) ? gate : w.I;          // (of the scans in fp32: the general ones)
+    const int keeps = reads_gate(p);
     if (p.gate_kind == GSA_GATE_ABC) {    // no decay, write weights from the cumulative softmax of the scores
         GSA_CUDA(launch_clear_flags(w.strong, (size_t)p.B * p.H * nseg, st));
         GSA_LAUNCH("abc_write", launch_abc_write(gate, w.G, w.I, w.Id, p.B, p.T, p.H, p.m, st));
@@ -629,7 +634,7 @@ gsa_status_t fwd_core(const CallParams* params, int m_active, const void* q, con
     if (nseg > 1) {
         // first pass: every segment from empty memories, for its end memories alone; then the start
         // memories of all segments, and the final memories, by a scan over the segments
-        GSA_LAUNCH("segment_states", state_scans(p, segs, StateSet{k, w.I, w.Id, w.Kloc}, StateSet{v, w.I, w.Id, w.Vloc}, w, 0,
+        GSA_LAUNCH("segment_states", state_scans(p, segs, StateSet{k, I, w.Id, w.Kloc}, StateSet{v, I, w.Id, w.Vloc}, w, 0,
                                                   w.seg_decay, input_gate, st, dev_status));
         // (when the backward is to reuse them, the final memories land in the saved block first)
         float* KTc = save_gate ? w.KT : KT;
@@ -644,12 +649,12 @@ gsa_status_t fwd_core(const CallParams* params, int m_active, const void* q, con
         Kout = nullptr; Vout = nullptr;
     }
     // pass 1: o' = GLA(q, k, 1-a) with the decay on the slot (value) side
-    ValueSideArgs a1{q, k, w.I, w.G, Kin, Kout, w.okpart, p.B, p.T, p.H, p.d_k, w.Id};
-    a1.nseg = nseg; a1.tseg = tseg; a1.E = w.E;
+    ValueSideArgs a1{q, k, I, w.G, Kin, Kout, w.okpart, p.B, p.T, p.H, p.d_k, w.Id};
+    a1.nseg = nseg; a1.tseg = tseg; a1.E = w.E; a1.w_keeps = keeps;
     if (nseg == 1) a1.input_gate = input_gate;       // (several segments: the state runs have been there)
     // pass 2: o = GLA(softmax(o'), 1-a, v) with the decay on the slot (key) side
-    KeySideArgs a2{w.p, w.I, w.G, v, Vin, Vout, o, p.B, p.T, p.H, p.d_v, w.Pd, w.Id};
-    a2.nseg = nseg; a2.tseg = tseg; a2.E = w.E;
+    KeySideArgs a2{w.p, I, w.G, v, Vin, Vout, o, p.B, p.T, p.H, p.d_v, w.Pd, w.Id};
+    a2.nseg = nseg; a2.tseg = tseg; a2.E = w.E; a2.uk_keeps = keeps;
     if (use_fused(p)) {
         // One kernel for pass 1 -> softmax -> pass 2; the logits are written only if the caller wants
         // them.  The (batch, head) pairs flagged for strong decay take the general kernels and the
@@ -795,6 +800,8 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
     const int nseg = segs.n, tseg = segs.t;
     const bool left_out = !gate_is_saved && leaves_input_gate(p, true);
     const InputGate input_gate = input_gate_of(p, gate, left_out);
+    const float* I = reads_gate(p) ? gate : w.I;          // (of the scans in fp32: the general ones)
+    const int keeps = reads_gate(p);
     if (!gate_is_saved) {      // (a forward of the same call left the gate kernel's products otherwise)
         if (p.gate_kind == GSA_GATE_ABC) {
             GSA_CUDA(launch_clear_flags(w.strong, (size_t)p.B * p.H * nseg, st));
@@ -813,7 +820,7 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
         Kin = w.Kstart; Vin = w.Vstart;
         KTout = nullptr; VTout = nullptr;
     } else if (nseg > 1) {
-        GSA_LAUNCH("segment_states", state_scans(p, segs, StateSet{k, w.I, w.Id, w.Kloc}, StateSet{v, w.I, w.Id, w.Vloc}, w, 0,
+        GSA_LAUNCH("segment_states", state_scans(p, segs, StateSet{k, I, w.Id, w.Kloc}, StateSet{v, I, w.Id, w.Vloc}, w, 0,
                                                   w.seg_decay, input_gate, st, dev_status));
         GSA_LAUNCH("segment_combine", launch_segment_combine(w.seg_decay, {w.Kloc, K0, w.Kstart, KTout, p.d_k}, {w.Vloc, V0, w.Vstart, VTout, p.d_v}, p.B,
                                                              p.H, p.m, nseg, 0, st));
@@ -821,8 +828,8 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
         KTout = nullptr; VTout = nullptr;
     }
     if (ok == nullptr) {  // recompute pass 1 and its logits
-        ValueSideArgs a1{q, k, w.I, w.G, Kin, nullptr, w.okpart, p.B, p.T, p.H, p.d_k, w.Id};
-        a1.nseg = nseg; a1.tseg = tseg; a1.E = w.E;
+        ValueSideArgs a1{q, k, I, w.G, Kin, nullptr, w.okpart, p.B, p.T, p.H, p.d_k, w.Id};
+        a1.nseg = nseg; a1.tseg = tseg; a1.E = w.E; a1.w_keeps = keeps;
         if (nseg == 1) a1.input_gate = input_gate;
         GSA_LAUNCH("pass1_value_side", value_side(p, a1, 0, w.strong, st, dev_status));
         GSA_LAUNCH("slot_softmax", launch_slot_softmax_fwd(w.okpart, s.k, p.scale, p.slot_act, w.ok, w.p, p.B, p.T * p.H, p.m, pend.G,
@@ -830,12 +837,12 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
         ok = w.ok;
     }
     // gradient w.r.t. the pass-2 queries p: the pass-1 form on (dO, v, 1-a); carries V~
-    ValueSideArgs adp{dO, v, w.I, w.G, Vin, VTout, w.dppart, p.B, p.T, p.H, p.d_v, w.Id};
-    adp.nseg = nseg; adp.tseg = tseg; adp.E = w.E;
+    ValueSideArgs adp{dO, v, I, w.G, Vin, VTout, w.dppart, p.B, p.T, p.H, p.d_v, w.Id};
+    adp.nseg = nseg; adp.tseg = tseg; adp.E = w.E; adp.w_keeps = keeps;
     if (nseg == 1 && ok_saved != nullptr) adp.input_gate = input_gate;      // (otherwise the scans before it have been there)
     // dq: the pass-2 form on (dz, 1-a, k); carries K~
-    KeySideArgs adq{w.dz, w.I, w.G, k, Kin, KTout, dq, p.B, p.T, p.H, p.d_k, w.Zd, w.Id};
-    adq.nseg = nseg; adq.tseg = tseg; adq.E = w.E;
+    KeySideArgs adq{w.dz, I, w.G, k, Kin, KTout, dq, p.B, p.T, p.H, p.d_k, w.Zd, w.Id};
+    adq.nseg = nseg; adq.tseg = tseg; adq.E = w.E; adq.uk_keeps = keeps;
     const bool fused = use_fused(p);
     // With the forward's slot weights in the saved block (and the logits saved, so that nothing here
     // rewrites them), the dv and dI^v scans depend on nothing this call computes: they start at once,
@@ -878,8 +885,8 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
     } else {
         GSA_LAUNCH("bwd_dp_value_side", value_side(p, adp, 0, w.strong, sc, dev_status));
         if (early) {
-            KeySideArgs adv{w.I, w.p, w.G, dO, dVT, dV0, dv, p.B, p.T, p.H, p.d_v, w.Id, w.Pd};
-            adv.nseg = nseg; adv.tseg = tseg; adv.E = w.E;
+            KeySideArgs adv{I, w.p, w.G, dO, dVT, dV0, dv, p.B, p.T, p.H, p.d_v, w.Id, w.Pd};
+            adv.nseg = nseg; adv.tseg = tseg; adv.E = w.E; adv.uq_keeps = keeps;
             ValueSideArgs adIv{v, dO, w.p, w.G, dVT, nullptr, w.dIv, p.B, p.T, p.H, p.d_v, w.Pd};
             adIv.nseg = nseg; adIv.tseg = tseg; adIv.E = w.E;
             adv.single = adIv.single = p.tc_operands == GSA_TC_SINGLE;
@@ -912,12 +919,12 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
         dK0out = nullptr; dV0out = nullptr;
     }
     // time-reversed runs: dv and dI^v share the state dV~; dk and dI^k share dK~
-    KeySideArgs adv{w.I, w.p, w.G, dO, dVin, dV0out, dv, p.B, p.T, p.H, p.d_v, w.Id, w.Pd};
-    adv.nseg = nseg; adv.tseg = tseg; adv.E = w.E;
+    KeySideArgs adv{I, w.p, w.G, dO, dVin, dV0out, dv, p.B, p.T, p.H, p.d_v, w.Id, w.Pd};
+    adv.nseg = nseg; adv.tseg = tseg; adv.E = w.E; adv.uq_keeps = keeps;
     ValueSideArgs adIv{v, dO, w.p, w.G, dVin, nullptr, w.dIv, p.B, p.T, p.H, p.d_v, w.Pd};
     adIv.nseg = nseg; adIv.tseg = tseg; adIv.E = w.E;
-    KeySideArgs adk{w.I, w.dz, w.G, q, dKin, dK0out, dk, p.B, p.T, p.H, p.d_k, w.Id, w.Zd};
-    adk.nseg = nseg; adk.tseg = tseg; adk.E = w.E;
+    KeySideArgs adk{I, w.dz, w.G, q, dKin, dK0out, dk, p.B, p.T, p.H, p.d_k, w.Id, w.Zd};
+    adk.nseg = nseg; adk.tseg = tseg; adk.E = w.E; adk.uq_keeps = keeps;
     ValueSideArgs adIk{k, q, w.dz, w.G, dKin, nullptr, w.dIk, p.B, p.T, p.H, p.d_k, w.Zd};
     adIk.nseg = nseg; adIk.tseg = tseg; adIk.E = w.E;
     // the reversed scans that share a state run as one kernel each (dv with dI^v, dk with dI^k)
@@ -1103,7 +1110,7 @@ gsa_status_t gsa_shard_states(const gsa_params_t* params, const void* k, const v
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // one "segment" per batch element: the whole shard from empty memories, end memories only
     GSA_LAUNCH("gate_cumsum", gate_products(p, Segments{1, p.T}, gate, w, !leaves_input_gate(p, false), st));
-    GSA_LAUNCH("segment_states", state_scans(p, Segments{1, p.T}, StateSet{k, w.I, w.Id, KT}, StateSet{v, w.I, w.Id, VT}, w, 0, logdecay,
+    GSA_LAUNCH("segment_states", state_scans(p, Segments{1, p.T}, StateSet{k, reads_gate(p) ? gate : w.I, w.Id, KT}, StateSet{v, reads_gate(p) ? gate : w.I, w.Id, VT}, w, 0, logdecay,
                                               input_gate_of(p, gate, leaves_input_gate(p, false)), st,
                                               dev_status));
     return GSA_OK;

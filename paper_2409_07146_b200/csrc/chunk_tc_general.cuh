@@ -14,8 +14,8 @@
 // step on top, so the products are warp-level ones (mma.sync m16n8k16: 8.3 cycles each; 64 a state warp and step on the value
 // side, 88 on the key side).  What bounds it: one state warp's chain of splits and products (960 cycles a step by itself on the
 // value side, 1300 beside its scheduler's slot warp; the tensor pipe is 33 and 40% active).  32 K tokens, 16 heads of 128,
-// a = sigmoid(N(-2, 1)): pass 1 486 -> 206 us, pass 2 410 -> 236 (HBM's share of either: 105), state runs 205 -> 33, the forward
-// 1283 -> 659 us.  The scans before these took 128-token chunks on tcgen05 and walked the decay row by row, 28 k cycles a chunk.
+// a = sigmoid(N(-2, 1)): pass 1 486 -> 208 us, pass 2 410 -> 224 (HBM's share of either: 105), state runs 205 -> 29, the forward
+// 1283 -> 616 us.  The scans before these took 128-token chunks on tcgen05 and walked the decay row by row, 28 k cycles a chunk.
 //
 // Warps of two roles, meeting on mbarriers only:
 //   * four slot warps take the steps in turn: a step's rows by TMA, asked for one of a warp's steps ahead (by 16-byte asynchronous
@@ -24,6 +24,8 @@
 //     side: A by mma); at the end the output rows;
 //   * four state warps take every step: the state (value side: 16 slots x 128 channels a warp, key side: 32 channels x
 //     64 slots) stays in registers in fp32, in the fragment layout that serves as the next product's operand as it stands.
+//     (The slot warps' instructions count, as their schedulers' slots are the state warps', too: the decays within a step as products
+//     of its gates instead of an exponential each, and 1 - a taken from the gate tensor where that holds a: 648 -> 616 us.)
 //     (Eight of them, half the channels each: 209 and 252 us; two to a scheduler wait for the same pipes at the same time.  Splits
 //     and decays moved by hand behind other blocks' products: 209 and 250.)
 // Every wait is bounded: on expiry the CTA flags dev_status, runs out without waiting and returns.
@@ -65,7 +67,6 @@ __device__ __noinline__ void write_input_gate(const ValueSideArgs& a) {
                 float y[4] = {x[q].x, x[q].y, x[q].z, x[q].w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    if (a.input_gate.kind == GSA_GATE_A) { y[e] = 1.f - y[e]; continue; }
                     if (a.input_gate.kind == GSA_GATE_LOGITS) y[e] = log_gate_from_logit(y[e], a.input_gate.inv_tau);
                     y[e] = -expm1f(y[e]);
                 }
@@ -229,6 +230,11 @@ __device__ __forceinline__ f32x2 slots2(const unsigned char* tile, int row, int 
     const uint32_t at = (lane >> 4) * kStepPanel + ((lane & 15) >> 1) * 16 + (lane & 1) * 8;
     return *reinterpret_cast<const f32x2*>(tile + row * 128 + (at ^ ((row & 7) << 4)));
 }
+// ... of one that holds a where 1 - a is meant
+__device__ __forceinline__ f32x2 weights2(const unsigned char* tile, int row, int lane, bool keeps) {
+    const f32x2 x = slots2(tile, row, lane);
+    return keeps ? sub2(pack2(1.f, 1.f), x) : x;
+}
 // where 8 channels of a row of a d-sized tile are: 16-byte piece `piece` of 16
 __device__ __forceinline__ uint32_t x_at(uint32_t tile, int row, int piece) {
     return tile + (piece >> 3) * kStepPanel + row * 128 + (((piece & 7) ^ (row & 7)) << 4);
@@ -391,13 +397,22 @@ __device__ __noinline__ bool value_side_general(const StepMaps maps, const Value
             const float2 before = next;
             step_gates(g, gates, span.t_end - steps.token<REV>(n), lane);
 #pragma unroll
-            for (int j = 0; j < kSub; ++j) E[j] = slots2(weights, j, lane);
+            for (int j = 0; j < kSub; ++j) E[j] = weights2(weights, j, lane, a.w_keeps != 0);
             // decayed weights, total decay: what the state warps wait for
+            f32x2 gate[kSub];                                        // the gates, whose products the factors within a step are
 #pragma unroll
-            for (int j0 = 0; j0 < kSub; j0 += kBatch) {
+            for (int j = 0; j < kSub; ++j) gate[j] = decay2(j > 0 ? g[j - 1] : before, g[j]);
+            f32x2 run = REV ? gate[0] : pack2(1.f, 1.f);
+#pragma unroll
+            for (int i0 = 0; i0 < kSub; i0 += kBatch) {
+                const int j0 = REV ? i0 : kSub - kBatch - i0;
                 f32x2 f[kBatch];
 #pragma unroll
-                for (int j = 0; j < kBatch; ++j) f[j] = REV ? decay2(before, g[j0 + j]) : decay2(g[j0 + j], g[kSub - 1]);
+                for (int i = 0; i < kBatch; ++i) {
+                    const int j = REV ? i : kBatch - 1 - i, next = REV ? j0 + j + 1 : j0 + j;
+                    f[j] = run;
+                    if (next < kSub) run = mul2(run, gate[next]);
+                }
 #pragma unroll
                 for (int j = 0; j < kBatch; ++j) f[j] = mul2(E[j0 + j], f[j]);
                 store_pairs(mine, j0, lane, f);
@@ -420,8 +435,7 @@ __device__ __noinline__ bool value_side_general(const StepMaps maps, const Value
             for (int ii = 0; ii < kSub; ++ii) {
                 const int i = REV ? kSub - 1 - ii : ii;
                 if (ii > 0) {
-                    const int at = REV ? i + 1 : i;
-                    const f32x2 x = decay2(g[at - 1], g[at]);
+                    const f32x2 x = gate[REV ? i + 1 : i];
 #pragma unroll
                     for (int jj = 0; jj < ii; ++jj) E[REV ? kSub - 1 - jj : jj] = mul2(E[REV ? kSub - 1 - jj : jj], x);
                 }
@@ -440,8 +454,13 @@ __device__ __noinline__ bool value_side_general(const StepMaps maps, const Value
             }
             // + the row factor times the inter-step product
             f32x2 f[kSub];
+            run = REV ? pack2(1.f, 1.f) : gate[0];
 #pragma unroll
-            for (int j = 0; j < kSub; ++j) f[j] = REV ? decay2(g[j], g[kSub - 1]) : decay2(before, g[j]);
+            for (int i = 0; i < kSub; ++i) {
+                const int j = REV ? kSub - 1 - i : i;
+                f[j] = run;
+                if (i + 1 < kSub) run = mul2(run, gate[REV ? j : j + 1]);
+            }
             general_wait(ctl, &ctl->done[w], use & 1);
             const int t = steps.token<REV>(n);
             float* row = obase + (((size_t)span.b * a.T + t) * a.H + span.h) * kM;
@@ -588,19 +607,18 @@ __device__ __forceinline__ void step_product(float (&c)[2][4], uint32_t x, uint3
 // at the block's middle, to which both decay by factors <= 1; four levels L = 8, 4, 2, 1, of which a token plays one part in
 // each -- one pair of rows Z serves both sides -- and the diagonal.
 template <bool REV>
-__device__ __forceinline__ void step_weights(float (&c)[2][4], const unsigned char* uq, const unsigned char* uk, const unsigned char* gates,
-                                             const float2 (&g)[kSub], float2 before, int rows, unsigned char* mine, int lane) {
+__device__ __forceinline__ void step_weights(float (&c)[2][4], const f32x2 (&kd)[kSub], const unsigned char* uq, const unsigned char* uk, const unsigned char* gates,
+                                             const float2 (&g)[kSub], float2 before, int rows, bool uq_keeps, bool uk_keeps, unsigned char* mine, int lane) {
     unsigned char* Z = mine + kKeyZ;
     const float2 whole = make_float2(g[kSub - 1].x - before.x, g[kSub - 1].y - before.y);
     if (__all_sync(0xffffffffu, fminf(whole.x, whole.y) >= kFactorisedDecayMin)) {
-        // forward: (uq_i e_i) (uk_j / e_j);  reversed: (uq_i s_i) (uk_j / s_j)
+        // forward: (uq_i e_i) (uk_j s_j / e_last);  reversed: (uq_i s_i) (uk_j e_j / e_last)
+        const f32x2 inverse = decay2(g[kSub - 1], before);
 #pragma unroll
         for (int j0 = 0; j0 < kSub; j0 += kBatch) {
             f32x2 f[kBatch];
 #pragma unroll
-            for (int j = 0; j < kBatch; ++j) f[j] = REV ? decay2(g[kSub - 1], g[j0 + j]) : decay2(g[j0 + j], before);
-#pragma unroll
-            for (int j = 0; j < kBatch; ++j) f[j] = mul2(slots2(uk, j0 + j, lane), f[j]);
+            for (int j = 0; j < kBatch; ++j) f[j] = mul2(kd[j0 + j], inverse);
             store_pairs(Z, j0, lane, f);
         }
         __syncwarp();
@@ -620,7 +638,7 @@ __device__ __forceinline__ void step_weights(float (&c)[2][4], const unsigned ch
                 const int at = j0 + j, mid = (at & ~(2 * L - 1)) + L;         // the first token of the block's second half
                 const bool later = (at & L) != 0;
                 const float2 g0 = gate(mid - 1), g1 = gate(at);
-                f[j] = mul2(slots2(later != REV ? uq : uk, at, lane), later ? decay2(g0, g1) : decay2(g1, g0));
+                f[j] = mul2(weights2(later != REV ? uq : uk, at, lane, later != REV ? uq_keeps : uk_keeps), later ? decay2(g0, g1) : decay2(g1, g0));
             }
             store_pairs(Z, j0, lane, f);
         }
@@ -638,7 +656,7 @@ __device__ __forceinline__ void step_weights(float (&c)[2][4], const unsigned ch
     }
 #pragma unroll 1
     for (int j = 0; j < kSub; ++j) {
-        const float2 x = unpack2(mul2(slots2(uq, j, lane), slots2(uk, j, lane)));
+        const float2 x = unpack2(mul2(weights2(uq, j, lane, uq_keeps), weights2(uk, j, lane, uk_keeps)));
         float sum = x.x + x.y;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
@@ -681,23 +699,36 @@ __device__ __noinline__ bool key_side_general(const StepMaps maps, const KeySide
             // (the stage of this warp's next step: all are done with the step that it held, the one before this)
             load_step<REV, 1, 2>(ctl, ring, maps, steps, span, d0, n + kSlotWarps);
             next = gate_before<REV>(a.G, steps, span, a.T, a.H, n + kSlotWarps, lane);
+            f32x2 gate[kSub], kd[kSub];                              // the gates; the decayed uk
+#pragma unroll
+            for (int j = 0; j < kSub; ++j) gate[j] = decay2(j > 0 ? g[j - 1] : before, g[j]);
 #pragma unroll
             for (int side = 0; side < 2; ++side) {         // uq, then uk
+                // the products of the gates from the step's start through a token, and from behind it to the end
+                const bool from_start = (side != 0) == REV;
+                f32x2 run = from_start ? gate[0] : pack2(1.f, 1.f);
 #pragma unroll
-                for (int j0 = 0; j0 < kSub; j0 += kBatch) {
+                for (int i0 = 0; i0 < kSub; i0 += kBatch) {
+                    const int j0 = from_start ? i0 : kSub - kBatch - i0;
                     f32x2 f[kBatch];
 #pragma unroll
-                    for (int j = 0; j < kBatch; ++j)
-                        f[j] = (side != 0) == REV ? decay2(before, g[j0 + j]) : decay2(g[j0 + j], g[kSub - 1]);
+                    for (int i = 0; i < kBatch; ++i) {
+                        const int j = from_start ? i : kBatch - 1 - i, next = from_start ? j0 + j + 1 : j0 + j;
+                        f[j] = run;
+                        if (next < kSub) run = mul2(run, gate[next]);
+                    }
 #pragma unroll
-                    for (int j = 0; j < kBatch; ++j) f[j] = mul2(slots2(side != 0 ? keys : queries, j0 + j, lane), f[j]);
+                    for (int j = 0; j < kBatch; ++j) {
+                        f[j] = mul2(weights2(side != 0 ? keys : queries, j0 + j, lane, (side != 0 ? a.uk_keeps : a.uq_keeps) != 0), f[j]);
+                        if (side != 0) kd[j0 + j] = f[j];
+                    }
                     store_pairs(mine + (side != 0 ? kKeyUk : 0), j0, lane, f);
                 }
             }
             *reinterpret_cast<f32x2*>(mine + kKeyTotal + 8 * lane) = decay2(before, g[kSub - 1]);
             __syncwarp();
             float c[2][4];
-            step_weights<REV>(c, queries, keys, gates, g, before, rows, mine, lane);
+            step_weights<REV>(c, kd, queries, keys, gates, g, before, rows, a.uq_keeps != 0, a.uk_keeps != 0, mine, lane);
             unsigned char* A = mine + kKeyA;
 #pragma unroll
             for (int nn = 0; nn < 2; ++nn)

@@ -111,9 +111,9 @@ cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t sme
 //
 // reverse = 1 sums over i >= j instead (same decay product): the gradients w.r.t. keys,
 // values and the input gate are such time-reversed runs.
-// Where w is the input gate 1 - a and only the flagged pairs read it in fp32 (the general scans): the gate kernel leaves it
-// out but of the chunks that flag their pair, and the scans form the other rows of a flagged pair from the gate before they go
-// on (write_input_gate).
+// Where w is the input gate 1 - a and only the flagged pairs read it in fp32 (the general scans): a gate tensor that holds a
+// takes its place (w_keeps).  Otherwise the gate kernel leaves it out but of the chunks that flag their pair, and the scans form
+// the other rows of a flagged pair from the gate before they go on (write_input_gate).
 struct InputGate { const float* gate = nullptr; int kind = 0; float inv_tau = 0.f; };
 struct ValueSideArgs {
     const void* xq; const void* xk;   // io
@@ -133,6 +133,7 @@ struct ValueSideArgs {
     int nseg = 1, tseg = 0;
     const float* E = nullptr;         // kernels for 128 slots: exp(G), see launch_gate_cumsum_wide
     InputGate input_gate;             // forward-direction runs on the tensor cores; gate null: w is there
+    int w_keeps = 0;                  // general scans: w holds a, the weights are 1 - a
     float* seg_logdecay = nullptr;    // state runs, forward, K side: receives the segments' log-decay (launch_segment_logdecay)
 };
 struct KeySideArgs {
@@ -148,6 +149,7 @@ struct KeySideArgs {
     int single;                       // as in ValueSideArgs
     int nseg = 1, tseg = 0;           // likewise
     const float* E = nullptr;         // likewise
+    int uq_keeps = 0, uk_keeps = 0;   // general scans: uq, uk hold a and stand for 1 - a
 };
 
 // What scan `bhs` of a launch over B * nseg * H scans works on: batch element, head and the tokens [t0, t_end).
@@ -221,7 +223,7 @@ struct PendingDecay {
 // chunk whose total log-decay is below kFactorisedDecayMin (nseg > 1: [B*nseg*H], per segment).
 // decayed (nullable, bf16 [B,T,H,2M]): rows [high part | rounding residual] of I exp(-G), the
 // input-gate operand of the pipelined tensor-core kernels.  leave_out: I only of the chunks that decay
-// below kFactorisedDecayMin (see InputGate).  fast_log: take log a with the
+// below kFactorisedDecayMin (1, see InputGate), or not at all (2).  fast_log: take log a with the
 // hardware base-2 logarithm (absolute error 2^-21.4 for a in [0.5, 1], 3 ulp below), for bf16 io.
 // gate_kind: gsa_gate_t (a, log a, or logits with inv_tau = 1/tau)
 cudaError_t launch_clear_flags(int* flags, size_t n, cudaStream_t st);

@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
     const bool strong = strong_flag != nullptr && grp == (int)blockDim.y - 1 &&
                         fmin(before0 + acc0, before1 + acc1) < (double)kFactorisedDecayMin;
     // (1 - a left out: of the chunks that do not decide on the general scans by themselves, see InputGate)
-    const bool put_I = leave_out == 0 || __syncthreads_or(strong);
+    const bool put_I = leave_out == 0 || (leave_out == 1 && __syncthreads_or(strong));
     if (strong) {
         const int seg = nseg == 1 ? 0 : t_chunk / tseg;
         strong_flag[WIDE ? (b * nseg + seg) * (H / 2) + h / 2 : (b * nseg + seg) * H + h] = 1;
