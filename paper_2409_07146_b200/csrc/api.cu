@@ -891,7 +891,7 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
             adIv.nseg = nseg; adIv.tseg = tseg; adIv.E = w.E;
             adv.single = adIv.single = p.tc_operands == GSA_TC_SINGLE;
             if (g_pair_scans.load(std::memory_order_relaxed) != 0 && rev_pair_supported(adIv, adv, p.m)) {
-                GSA_CUDA(launch_rev_pair_tc(adIv, adv, p.m, w.strong, lanes->stream[0], dev_status));
+                GSA_CUDA(launch_rev_pair_tc(adIv, adv, p.m, w.strong, p.cu_seqlens != nullptr, lanes->stream[0], dev_status));
             } else {
                 GSA_CUDA(key_side(p, adv, 1, w.strong, lanes->stream[0], dev_status));
                 GSA_CUDA(value_side(p, adIv, 1, w.strong, lanes->stream[1], dev_status));
@@ -937,16 +937,16 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
         GSA_CUDA(cudaEventRecord(lanes->fork, st));
         for (int i = early ? 1 : 0; i < 2; ++i) GSA_CUDA(cudaStreamWaitEvent(lanes->stream[i], lanes->fork, 0));
         if (!fused) GSA_CUDA(key_side(p, adq, 0, w.strong, st, dev_status));
-        if (!early) GSA_CUDA(launch_rev_pair_tc(pIv, pv, p.m, w.strong, lanes->stream[0], dev_status));
-        GSA_CUDA(launch_rev_pair_tc(pIk, pk, p.m, w.strong, lanes->stream[1], dev_status));
+        if (!early) GSA_CUDA(launch_rev_pair_tc(pIv, pv, p.m, w.strong, p.cu_seqlens != nullptr, lanes->stream[0], dev_status));
+        GSA_CUDA(launch_rev_pair_tc(pIk, pk, p.m, w.strong, p.cu_seqlens != nullptr, lanes->stream[1], dev_status));
         for (int i = 0; i < 2; ++i) {
             GSA_CUDA(cudaEventRecord(lanes->join[i], lanes->stream[i]));
             GSA_CUDA(cudaStreamWaitEvent(st, lanes->join[i], 0));
         }
     } else if (paired) {
         if (!fused) GSA_LAUNCH("bwd_dq_key_side", key_side(p, adq, 0, w.strong, st, dev_status));
-        GSA_LAUNCH("bwd_dv_dIv_pair_rev", launch_rev_pair_tc(pIv, pv, p.m, w.strong, st, dev_status));
-        GSA_LAUNCH("bwd_dk_dIk_pair_rev", launch_rev_pair_tc(pIk, pk, p.m, w.strong, st, dev_status));
+        GSA_LAUNCH("bwd_dv_dIv_pair_rev", launch_rev_pair_tc(pIv, pv, p.m, w.strong, p.cu_seqlens != nullptr, st, dev_status));
+        GSA_LAUNCH("bwd_dk_dIk_pair_rev", launch_rev_pair_tc(pIk, pk, p.m, w.strong, p.cu_seqlens != nullptr, st, dev_status));
     } else if (side_by_side) {
         // the five scans side by side (see ScanLanes)
         GSA_CUDA(cudaEventRecord(lanes->fork, st));

@@ -13,7 +13,7 @@ value_side_general_kernel(const __grid_constant__ GeneralValueMaps maps, const _
 }
 __global__ void __launch_bounds__(kScanThreads, 1)
 key_side_general_kernel(const __grid_constant__ GeneralKeyMaps maps, const __grid_constant__ KeySideArgs a, const int* __restrict__ strong_flag, int32_t* dev_status) {
-    if (strong_flag[blockIdx.x] != 0) key_side_general<false>(maps.steps(), a, dev_status);
+    if (strong_flag[blockIdx.x] != 0) key_side_general<false>(maps.steps(), a, dev_status, blockIdx.y);
 }
 
 }  // namespace

@@ -669,7 +669,7 @@ __device__ __forceinline__ void step_weights(float (&c)[2][4], const f32x2 (&kd)
 }
 
 template <bool REV>
-__device__ __noinline__ bool key_side_general(const StepMaps maps, const KeySideArgs& args, int32_t* dev_status) {
+__device__ __noinline__ bool key_side_general(const StepMaps maps, const KeySideArgs& args, int32_t* dev_status, int slice) {
     const KeySideArgs a = args;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* ring = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -678,7 +678,7 @@ __device__ __noinline__ bool key_side_general(const StepMaps maps, const KeySide
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const ScanSpan span = scan_span(blockIdx.x, a.H, a.T, a.nseg, a.tseg);
-    const int d0 = blockIdx.y * kDST;
+    const int d0 = slice * kDST;
     const Steps steps = all_steps(span);
     general_ctl_init(ctl, tid);
 

@@ -384,7 +384,7 @@ key_side_lean_kernel(const __grid_constant__ CUtensorMap mapV, const __grid_cons
                      const int* strong_flag, int32_t* dev_status) {
     follow_previous_grid();
     if (strong_flag[blockIdx.x] != 0) {
-        key_side_general<REV>(general.steps(), a, dev_status);
+        key_side_general<REV>(general.steps(), a, dev_status, blockIdx.y);
         return;
     }
     extern __shared__ unsigned char smem_raw[];

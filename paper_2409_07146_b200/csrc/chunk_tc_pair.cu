@@ -70,11 +70,16 @@ rev_pair_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
                 const __grid_constant__ CUtensorMap mapOv, const __grid_constant__ CUtensorMap mapOk,
                 const __grid_constant__ GeneralPairMaps general, const __grid_constant__ ValueSideArgs av, const __grid_constant__ KeySideArgs ak, const int* strong_flag, int32_t* dev_status) {
     follow_previous_grid();
-    if (strong_flag[blockIdx.x] != 0) {             // the two general scans, one after the other
-        if (value_side_general<true>(StepMaps{{&general.y, &general.x}, {&general.w, nullptr}, &general.G}, av, dev_status, blockIdx.y))
-            key_side_general<true>(StepMaps{{&general.x, nullptr}, {&general.q, &general.w}, &general.G}, ak, dev_status);
+    // the two general scans, one after the other, or where the grid has both halves (slices + the slice) a CTA each
+    const int slices = av.D <= kDST ? 1 : av.D / kDST, slice = blockIdx.y < slices ? blockIdx.y : blockIdx.y - slices;
+    if (strong_flag[blockIdx.x] != 0) {
+        const bool first = (int)blockIdx.y < slices;
+        const bool fine = !first || value_side_general<true>(StepMaps{{&general.y, &general.x}, {&general.w, nullptr}, &general.G}, av, dev_status, slice);
+        if (fine && (!first || (int)gridDim.y == slices))
+            key_side_general<true>(StepMaps{{&general.x, nullptr}, {&general.q, &general.w}, &general.G}, ak, dev_status, slice);
         return;
     }
+    if ((int)blockIdx.y >= slices) return;
     const float* G = ak.G;
     const float* S0 = ak.S0;
     float* Send = ak.Send;
@@ -94,7 +99,7 @@ rev_pair_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
     const int tid = threadIdx.x, warp = tid >> 5, wq = warp & 3, half = (tid >> 7) & 1, row = tid & 127;
     const int sb = kHS * half;          // this thread's first slot
     const ScanSpan span = scan_span(blockIdx.x, H, T, nseg, tseg);
-    const int bh = blockIdx.x, slice = blockIdx.y, b = span.b, h = span.h;
+    const int bh = blockIdx.x, b = span.b, h = span.h;
     const int d0 = slice * kDST;
 
     if (tid == 0) {
@@ -460,7 +465,7 @@ bool rev_pair_supported(const ValueSideArgs& av, const KeySideArgs& ak, int M) {
            av.S0 == ak.S0 && av.Send == nullptr && !av.state_only && av.single == ak.single;
 }
 
-cudaError_t launch_rev_pair_tc(const ValueSideArgs& av, const KeySideArgs& ak, int M, const int* strong_flag,
+cudaError_t launch_rev_pair_tc(const ValueSideArgs& av, const KeySideArgs& ak, int M, const int* strong_flag, bool packed,
                                cudaStream_t st, int32_t* dev_status) {
     if (!rev_pair_supported(av, ak, M) || strong_flag == nullptr) return cudaErrorNotSupported;
     CUtensorMap mx, my, mw, mq, mov, mok;
@@ -477,7 +482,10 @@ cudaError_t launch_rev_pair_tc(const ValueSideArgs& av, const KeySideArgs& ak, i
     if (e == cudaSuccess) e = step_map(&general.q, ak.uq, ak.B, ak.T, ak.H, kM, 4);
     if (e == cudaSuccess) e = step_map(&general.G, ak.G, ak.B, ak.T, ak.H, kM, 4);
     if (e != cudaSuccess) return e;
-    const dim3 grid(av.B * av.nseg * av.H, tc_value_side_slices(av.D));
+    // Packed sequences flag a segment here and there (two offsets in a chunk): its CTAs are then what the launch waits for, and a
+    // second half of the grid, whose other CTAs leave at once, takes their key sides.  8 K tokens of 13 sequences, 4 heads of 512:
+    // 596 -> 568 us, 334 as before where none is flagged.
+    const dim3 grid(av.B * av.nseg * av.H, tc_value_side_slices(av.D) * (packed ? 2 : 1));
     constexpr size_t smem = kSmemPair > kSmemGeneral ? kSmemPair : kSmemGeneral;
     auto launch = [&](auto kernel, cudaError_t ready) {
         if (ready != cudaSuccess) return ready;

@@ -317,7 +317,7 @@ cudaError_t launch_state_scan_tc(const ValueSideArgs& k, const ValueSideArgs& v,
 // The two reversed scans that share a state (dv with dI^v, dk with dI^k) as one kernel
 // (chunk_tc_pair.cu): av / ak are the arguments the single reversed scans would get.
 bool rev_pair_supported(const ValueSideArgs& av, const KeySideArgs& ak, int M);
-cudaError_t launch_rev_pair_tc(const ValueSideArgs& av, const KeySideArgs& ak, int M, const int* strong_flag,
+cudaError_t launch_rev_pair_tc(const ValueSideArgs& av, const KeySideArgs& ak, int M, const int* strong_flag, bool packed,
                                cudaStream_t st, int32_t* dev_status);
 // the side stream of the calling host thread on the current device, with its fork / join events
 struct SideLane {
