@@ -204,13 +204,14 @@ decode_step_kernel(const IO* q, const IO* k, const IO* v,
     }
 }
 
-// Few (sequence, head) pairs: a pair is dealt out over a cluster of M / (8 RPW) CTAs, RPW rows of each memory to a warp, so
-// that one sequence uses more than H SMs.  A step of one CTA per pair is bound by the latency of its chain -- K rows in
+// Few (sequence, head) pairs: a pair is dealt out over a cluster of M / (8 RPW) CTAs, so that one sequence uses more than H SMs:
+// RPW rows of the key memory to a warp, and of the value memory a CTA's share of the channels, all slots of them.  A step of one
+// CTA per pair is bound by the latency of its chain -- K rows in
 // batches, logits, softmax, V rows in batches, sums -- and by what one SM can pull: 512 KB at d = 512, 9.6 us a launch
-// where 4 pairs keep 4 SMs busy.  Here every row of both memories is requested at once, before anything is used; the CTAs
-// exchange the M logits and the partial output rows through distributed shared memory (two cluster barriers).  The steps
-// of a stack of layers follow one another: each is placed while the one before it drains (24 layers of 4 pairs
-// of d = 512: 150 -> 118 us as calls, 111 -> 107 in a graph).
+// where 4 pairs keep 4 SMs busy.  Here all of both memories is requested at once, before anything is used; the CTAs
+// exchange the M logits through distributed shared memory and nothing else (two cluster barriers; with rows of the value memory
+// to a warp, too, the output's partial sums took a third: 24 layers of 4 pairs of d = 512, 109 us, so 88).  The steps
+// of a stack of layers follow one another: each is placed while the one before it drains (150 -> 118 us as calls then).
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 // the word at the same place of CTA `rank`'s shared memory <- x
@@ -221,40 +222,52 @@ __device__ __forceinline__ void store_to_rank(float* local, unsigned rank, float
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(x) : "memory");
 }
 
-template <typename IO, int DK, int DV, int RPW>
+template <int n> struct alignas(n * sizeof(float)) Floats { float x[n]; };
+
+template <typename IO, int DK, int DV, int M, int RPW>
 __global__ void __launch_bounds__(kDecodeWarps * 32)
 decode_split_kernel(const IO* q, const IO* k, const IO* v,
-                    const void* gate_raw, int M, int gate_bf16, int gate_row_of_head, int feature_map,
+                    const void* gate_raw, int gate_bf16, int gate_row_of_head, int feature_map,
                     int gate_kind, float inv_tau, float scale, int act, float* Ks, float* Vs,
                     IO* __restrict__ o) {
     follow_previous_grid();
-    const int C = M / (kDecodeWarps * RPW);                     // CTAs of the cluster, M <= 128, C <= 8
+    constexpr int C = M / (kDecodeWarps * RPW);                 // CTAs of the cluster
+    constexpr int kOwn = DV / C, W = kOwn < 32 ? 1 : kOwn / 32; // channels of the value memory a CTA, a lane
+    constexpr int kRows = M / kDecodeWarps;                     // rows of it a warp
+    static_assert(C <= 8 && (W == 1 || W == 2 || W == 4), "");
     const size_t pair = blockIdx.x / C;
     const int rank = blockIdx.x % C, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int row0 = (rank * kDecodeWarps + warp) * RPW;        // this warp's memory rows
-    __shared__ float s_z[128];
-    __shared__ float s_o[kDecodeWarps][DV];
-    __shared__ float s_part[8][DV];         // partial sums of this CTA's DV / C output channels, from every rank
+    const int row0 = (rank * kDecodeWarps + warp) * RPW;        // this warp's rows of the key memory
+    const int vrow0 = warp * kRows, c0 = rank * kOwn + W * lane;
+    const bool live = kOwn >= 32 || lane < kOwn;                // (narrow values: lanes without a channel)
+    __shared__ float s_z[M];
+    __shared__ Floats<W> s_o[kDecodeWarps][32];
     cluster_arrive();                       // (every CTA runs before another one writes to it)
 
     float* Kp = Ks + (pair * M + row0) * DK;
-    float* Vp = Vs + (pair * M + row0) * DV;
+    float* Vp = Vs + (pair * M + vrow0) * DV + c0;
     RowVec<DK> kr[RPW], qv, kv;
-    RowVec<DV> vr[RPW], vv;
+    Floats<W> vr[kRows];
 #pragma unroll
     for (int r = 0; r < RPW; ++r) kr[r].load(Kp + (size_t)r * DK, lane);
 #pragma unroll
-    for (int r = 0; r < RPW; ++r) vr[r].load(Vp + (size_t)r * DV, lane);
+    for (int r = 0; r < kRows; ++r)
+        if (live) vr[r] = *reinterpret_cast<const Floats<W>*>(Vp + (size_t)r * DV);
     qv.load_io(q + pair * DK, lane);
     kv.load_io(k + pair * DK, lane);
-    vv.load_io(v + pair * DV, lane);
-    float a[RPW], ia[RPW];
+    float vv[W];
 #pragma unroll
-    for (int r = 0; r < RPW; ++r) {
-        const size_t gi = (gate_row_of_head ? pair % gate_row_of_head : pair) * M + row0 + r;
-        decode_gate(gate_raw, gi, gate_bf16, gate_kind, inv_tau, a[r], ia[r]);
+    for (int w = 0; w < W; ++w) vv[w] = live ? io_to_float<IO>(v[pair * DV + c0 + w]) : 0.f;
+    const size_t gates = (gate_row_of_head ? pair % gate_row_of_head : pair) * M;
+    float a[RPW], ia[RPW], va, via;
+#pragma unroll
+    for (int r = 0; r < RPW; ++r) decode_gate(gate_raw, gates + row0 + r, gate_bf16, gate_kind, inv_tau, a[r], ia[r]);
+    decode_gate(gate_raw, gates + vrow0 + lane % kRows, gate_bf16, gate_kind, inv_tau, va, via);      // (lane r: the warp's row r)
+    if (feature_map == GSA_FEAT_SWISH) {
+        qv.swish(); kv.swish();
+#pragma unroll
+        for (int w = 0; w < W; ++w) vv[w] = vv[w] / (1.f + __expf(-vv[w]));
     }
-    if (feature_map == GSA_FEAT_SWISH) { qv.swish(); kv.swish(); vv.swish(); }
     float z[RPW];
 #pragma unroll
     for (int r = 0; r < RPW; ++r) {
@@ -278,66 +291,56 @@ decode_split_kernel(const IO* q, const IO* k, const IO* v,
     cluster_arrive();
     // (the memories leave while the logits travel)
 #pragma unroll
-    for (int r = 0; r < RPW; ++r) {
-        kr[r].store(Kp + (size_t)r * DK, lane);
+    for (int r = 0; r < RPW; ++r) kr[r].store(Kp + (size_t)r * DK, lane);
 #pragma unroll
-        for (int i = 0; i < RowVec<DV>::kN; ++i)
+    for (int r = 0; r < kRows; ++r) {
+        const float ar = __shfl_sync(0xffffffffu, va, r), ir = __shfl_sync(0xffffffffu, via, r);
 #pragma unroll
-            for (int w = 0; w < RowVec<DV>::kW; ++w) vr[r].v[i][w] = fmaf(a[r], vr[r].v[i][w], ia[r] * vv.v[i][w]);
-        vr[r].store(Vp + (size_t)r * DV, lane);
+        for (int w = 0; w < W; ++w) vr[r].x[w] = fmaf(ar, vr[r].x[w], ir * vv[w]);
+        if (live) *reinterpret_cast<Floats<W>*>(Vp + (size_t)r * DV) = vr[r];
     }
     cluster_wait();
-    // slot weights of this warp's rows, each warp by itself
-    float p[RPW];
+    // slot weights of this warp's rows of the value memory, each warp by itself (lane r: row r)
+    float p = s_z[vrow0 + lane % kRows];
     if (act != GSA_ACT_SOFTMAX) {
-#pragma unroll
-        for (int r = 0; r < RPW; ++r) p[r] = slot_act_value(z[r], act);
+        p = slot_act_value(p, act);
     } else {
         float zmax = -INFINITY, den = 0.f;
+#pragma unroll
         for (int s = lane; s < M; s += 32) zmax = fmaxf(zmax, s_z[s]);
 #pragma unroll
         for (int off = 16; off; off >>= 1) zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, off));
+#pragma unroll
         for (int s = lane; s < M; s += 32) den += __expf(s_z[s] - zmax);
 #pragma unroll
         for (int off = 16; off; off >>= 1) den += __shfl_xor_sync(0xffffffffu, den, off);
-        const float inv = 1.f / den;
-#pragma unroll
-        for (int r = 0; r < RPW; ++r) p[r] = __expf(z[r] - zmax) * inv;
+        p = __expf(p - zmax) * (1.f / den);
     }
-    RowVec<DV> acc;
+    Floats<W> acc;
 #pragma unroll
-    for (int i = 0; i < RowVec<DV>::kN; ++i)
+    for (int w = 0; w < W; ++w) acc.x[w] = 0.f;
 #pragma unroll
-        for (int w = 0; w < RowVec<DV>::kW; ++w) {
-            acc.v[i][w] = 0.f;
+    for (int r = 0; r < kRows; ++r) {
+        const float pr = __shfl_sync(0xffffffffu, p, r);
 #pragma unroll
-            for (int r = 0; r < RPW; ++r) acc.v[i][w] = fmaf(p[r], vr[r].v[i][w], acc.v[i][w]);
-        }
-    acc.store(&s_o[warp][0], lane);
+        for (int w = 0; w < W; ++w) acc.x[w] = fmaf(pr, vr[r].x[w], acc.x[w]);
+    }
+    s_o[warp][lane] = acc;
     __syncthreads();
-    // the CTA's partial sum of channel c goes to the CTA that owns the channel
-    const int own = DV / C;
-    for (int c = threadIdx.x; c < DV; c += kDecodeWarps * 32) {
+    for (int c = threadIdx.x; c < kOwn; c += kDecodeWarps * 32) {
         float sum = 0.f;
 #pragma unroll
-        for (int w = 0; w < kDecodeWarps; ++w) sum += s_o[w][c];
-        store_to_rank(&s_part[rank][c % own], c / own, sum);
-    }
-    cluster_arrive();
-    cluster_wait();
-    for (int c = threadIdx.x; c < own; c += kDecodeWarps * 32) {
-        float sum = 0.f;
-        for (int r = 0; r < C; ++r) sum += s_part[r][c];
-        o[pair * DV + rank * own + c] = float_to_io<IO>(sum);
+        for (int w = 0; w < kDecodeWarps; ++w) sum += s_o[w][c / W].x[c % W];
+        o[pair * DV + rank * kOwn + c] = float_to_io<IO>(sum);
     }
 }
 
-template <typename IO, int DK, int DV, int RPW>
+template <typename IO, int DK, int DV, int M, int RPW>
 static cudaError_t launch_decode_split(const gsa_params_t& p, const IO* q, const IO* k, const IO* v, const float* gate,
                                        float* Ks, float* Vs, IO* o, cudaStream_t st) {
-    const unsigned C = (unsigned)(p.m / (kDecodeWarps * RPW));
-    return launch_after(decode_split_kernel<IO, DK, DV, RPW>, ClusterGrid{dim3((unsigned)p.B * (unsigned)p.H * C), dim3(C, 1, 1)},
-                        dim3(kDecodeWarps * 32), 0, st, q, k, v, static_cast<const void*>(gate), (int)p.m,
+    constexpr unsigned C = M / (kDecodeWarps * RPW);
+    return launch_after(decode_split_kernel<IO, DK, DV, M, RPW>, ClusterGrid{dim3((unsigned)p.B * (unsigned)p.H * C), dim3(C, 1, 1)},
+                        dim3(kDecodeWarps * 32), 0, st, q, k, v, static_cast<const void*>(gate),
                               (int)(p.gate_dtype == GSA_BF16), (int)(p.gate_broadcast ? p.H : 0), (int)p.feature_map,
                               (int)p.gate_kind, p.tau > 0.f ? 1.f / p.tau : 0.f, p.scale, (int)p.slot_act, Ks, Vs, o);
 }
@@ -375,17 +378,22 @@ template <typename IO, int DK, int DV>
 static cudaError_t launch_decode_m(const gsa_params_t& p, const IO* q, const IO* k, const IO* v,
                                    const float* gate, float* Ks, float* Vs, IO* o, cudaStream_t st) {
     const unsigned pairs = (unsigned)p.B * (unsigned)p.H;
-    // The line between the kernels, us a step of one layer (64 slots) with one CTA a pair / a row a warp / two: 4 pairs of
-    // d = 512: 10.3 / 4.8 / 5.6, 16: 15.3 / 6.6 / 7.0, 64: 19.5 / 14.3 / 14.5, 80: 20.1 / 19.2 / 19.9, 128: 22.8 / 26.8 / 27.1;
-    // d = 256: 8 pairs 5.9 / 4.0 / 4.6, 64: 10.8 / 11.5 / 7.8; d = 128: 32 pairs 4.4 / 4.3 / 4.2, 128: 7.5 / 11.9 / 7.9 (a pair
-    // is little enough for one SM).  128 slots (two rows a warp; one CTA / two rows): 4 pairs of 512 15.6 / 5.6, 16: 16.1 /
-    // 10.5, 32: 20.1 / 19.2.  32 slots, half a pair each, one CTA / a row / two: 4 pairs of 512 5.9 / 4.7, 32: 6.4 / 5.1, 64:
-    // 7.0 / - / 6.7, 128: 11.7 / - / 14.6; 64 pairs of 256 4.4 / - / 4.9.  So: heads of 256 and more, a row a warp while no
-    // SM has two CTAs, two rows a warp while none has more than two, these not for 32 slots.
-    if constexpr (DK + DV >= 512) {
-        const long long ctas = (long long)pairs * (p.m / kDecodeWarps);
-        if (p.m <= 64 && ctas <= kSMs) return launch_decode_split<IO, DK, DV, 1>(p, q, k, v, gate, Ks, Vs, o, st);
-        if (p.m >= 64 && ctas / 2 <= 2 * kSMs) return launch_decode_split<IO, DK, DV, 2>(p, q, k, v, gate, Ks, Vs, o, st);
+    // The line between the kernels, us a step of one layer / of a layer of eight: one CTA a pair, against a row a warp or (from 19
+    // pairs on) two.  64 slots, d = 64: 12 pairs 4.2 / 3.8, 3.1 / 2.9; 48: 4.2 / 3.8, 3.3 / 3.3; 96: 4.5 / 3.9, 4.7 / 4.7.  128: 4 pairs
+    // 4.4 / 4.3, 3.1 / 2.9; 32: 4.5 / 4.4, 3.1 / 3.4; 64: 4.6 / 4.4, 4.6 / 4.0; 96: 5.1 / 4.5, 5.0 / 4.9.  256: 8 pairs 6.3 / 5.8, 3.1 /
+    // 3.1; 64: 6.6 / 6.4, 5.6 / 5.3; 96: 6.6 / 10.6, 5.4 / 7.0; 128: 6.3 / 12.1, 9.2 / 11.5.  512: 4 pairs 10.2 / 10.2, 3.5 / 3.4; 64: 11.9 /
+    // 19.0, 6.4 / 9.0; 96: 12.0 / 20.4, 10.9 / 14.6; 128: 10.9 / 22.1, 11.4 / 16.2.  32 slots, a row a warp: d = 64: 12 pairs 3.1 / 3.0, 3.0 /
+    // 2.8, 96: 3.0 / 3.2, 3.3 / 3.4; 128: 64 pairs 4.1 / 3.5, 3.1 / 3.1, 96: 4.2 / 3.5, 4.1 / 4.2; 512: 64 pairs 6.3 / 6.4, 4.3 / 4.6, 80:
+    // 6.4 / 8.3, 7.6 / 8.7.  128 slots, two rows a warp or four: d = 128: 4 pairs 7.2 / 7.2, 3.2 / 3.2, 64: 7.9 / 7.8, 6.2 / 6.1, 128: 7.6 /
+    // 12.3, 9.2 / 11.9; 512: 16 pairs 15.5 / 15.4, 5.8 / 5.7, 64: 15.9 / 21.7, 12.3 / 17.3, 96: 17.2 / 24.9, 17.7 / 24.7.
+    const long long eighths = 8LL * pairs, quarters = 4LL * pairs;           // CTAs of the clusters
+    constexpr int kTwice = 2 * kSMs, kSome = DK + DV >= 512 ? 400 : (DK + DV >= 256 ? kTwice : 3 * kSMs / 2);
+    if (p.m == 32 && quarters <= (DK + DV >= 256 ? kTwice : kSMs)) return launch_decode_split<IO, DK, DV, 32, 1>(p, q, k, v, gate, Ks, Vs, o, st);
+    if (p.m == 64 && eighths <= kSMs) return launch_decode_split<IO, DK, DV, 64, 1>(p, q, k, v, gate, Ks, Vs, o, st);
+    if (p.m == 64 && quarters <= kSome) return launch_decode_split<IO, DK, DV, 64, 2>(p, q, k, v, gate, Ks, Vs, o, st);
+    if constexpr (DK + DV >= 256) {
+        if (p.m == 128 && eighths <= kSMs) return launch_decode_split<IO, DK, DV, 128, 2>(p, q, k, v, gate, Ks, Vs, o, st);
+        if (p.m == 128 && quarters <= kTwice) return launch_decode_split<IO, DK, DV, 128, 4>(p, q, k, v, gate, Ks, Vs, o, st);
     }
     const int is_log = p.gate_kind;
     const float inv_tau = p.tau > 0.f ? 1.f / p.tau : 0.f;
