@@ -295,11 +295,13 @@ InputGate input_gate_of(const gsa_params_t& p, const float* gate, bool left_out)
     return left_out && !reads_gate(p) ? InputGate{gate, p.gate_kind, inv_tau(p)} : InputGate{};
 }
 
-// the gate kernel: G, 1 - a, the decayed rows and the strong-decay flags, cleared first (which the CUDA-core kernels do without)
+// the gate kernel: G, 1 - a, the decayed rows and the strong-decay flags, cleared first where several of its CTAs share one (the
+// CUDA-core kernels do without)
 // (input_gate = false: 1 - a is left out, see leaves_input_gate)
 cudaError_t gate_products(const gsa_params_t& p, Segments segs, const float* gate, const Workspace& w, bool input_gate,
                           cudaStream_t st) {
-    if (use_tc(p)) {
+    const int chunk = chunk_of(p), nchunks = (p.T + chunk - 1) / chunk;
+    if (use_tc(p) && (use_wide(p) || !owns_strong_flag(segs.n, nchunks))) {
         const cudaError_t e = launch_clear_flags(w.strong, (size_t)p.B * p.H * segs.n, st);
         if (e != cudaSuccess) return e;
     }

@@ -219,14 +219,17 @@ struct PendingDecay {
 };
 
 // launchers (definitions in the .cu files); all return cudaGetLastError() of the launch
-// strong_flag (nullable, [B*H] ints, zeroed by the caller): set to 1 for every (b,h) that has a
+cudaError_t launch_clear_flags(int* flags, size_t n, cudaStream_t st);
+// Is a strong-decay flag written by one CTA of the gate kernel alone (64-slot tiles)?  It then needs no clearing, which is a launch
+// of a short call's five: pairs or segments of a single chunk (a forward over 114 tokens, 8 heads of 256: 29.8 -> 27.0 us).
+__host__ __device__ inline bool owns_strong_flag(int nseg, int nchunks) { return nseg == nchunks; }
+// strong_flag (nullable, [B*H] ints, zeroed by launch_clear_flags, but see owns_strong_flag): set to 1 for every (b,h) that has a
 // chunk whose total log-decay is below kFactorisedDecayMin (nseg > 1: [B*nseg*H], per segment).
 // decayed (nullable, bf16 [B,T,H,2M]): rows [high part | rounding residual] of I exp(-G), the
 // input-gate operand of the pipelined tensor-core kernels.  leave_out: I only of the chunks that decay
 // below kFactorisedDecayMin (1, see InputGate), or not at all (2).  fast_log: take log a with the
 // hardware base-2 logarithm (absolute error 2^-21.4 for a in [0.5, 1], 3 ulp below), for bf16 io.
 // gate_kind: gsa_gate_t (a, log a, or logits with inv_tau = 1/tau)
-cudaError_t launch_clear_flags(int* flags, size_t n, cudaStream_t st);
 cudaError_t launch_gate_cumsum(const float* gate, int gate_kind, float inv_tau, float* G, float* I,
                                int B, int T, int H, int M, int chunk, int* strong_flag, int nseg, int tseg,
                                void* decayed, int fast_log, cudaStream_t st, const int* cu_seqlens = nullptr,

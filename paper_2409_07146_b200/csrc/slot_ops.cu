@@ -171,10 +171,13 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
     const bool strong = strong_flag != nullptr && grp == (int)blockDim.y - 1 &&
                         fmin(before0 + acc0, before1 + acc1) < (double)kFactorisedDecayMin;
     // (1 - a left out: of the chunks that do not decide on the general scans by themselves, see InputGate)
-    const bool put_I = leave_out == 0 || (leave_out == 1 && __syncthreads_or(strong));
-    if (strong) {
+    const bool owns_flag = !WIDE && strong_flag != nullptr && owns_strong_flag(nseg, (int)gridDim.y);
+    bool any_strong = strong;
+    if (owns_flag || leave_out == 1) any_strong = __syncthreads_or(strong);
+    const bool put_I = leave_out == 0 || (leave_out == 1 && any_strong);
+    if (strong || (owns_flag && threadIdx.x == 0 && grp == 0)) {
         const int seg = nseg == 1 ? 0 : t_chunk / tseg;
-        strong_flag[WIDE ? (b * nseg + seg) * (H / 2) + h / 2 : (b * nseg + seg) * H + h] = 1;
+        strong_flag[WIDE ? (b * nseg + seg) * (H / 2) + h / 2 : (b * nseg + seg) * H + h] = any_strong;
     }
     // second pass over the same rows: the sums of the groups before as a float pair (value, rest)
     const float b0h = (float)before0, b0l = (float)(before0 - (double)b0h);
