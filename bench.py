@@ -44,7 +44,7 @@ NCU_TRAFFIC = {
     "bwd_dv_key_side_rev": 130483200, "bwd_dk_key_side_rev": 132975616,
     "bwd_dv_dIv_pair_rev": 258483968, "bwd_dk_dIk_pair_rev": 257145344,
     "gate_cumsum": 17926144, "slot_softmax": 92744448, "slot_softmax_bwd": 118787072,
-    "gate_grad": 231503872,     # local + scan + carry
+    "gate_grad": 195975424,
 }
 
 
@@ -92,7 +92,7 @@ def kernel_algorithmic_bytes(label: str, w: W.Workload) -> int:
         # a pair of reversed scans as one kernel: both d-sized tiles and both decayed rows once
         "bwd_dv_dIv_pair_rev": 3 * w.d_v * e + 8 * m + 4 * m * nsv,  # dO, v, I exp(-G), p exp(G) -> dv, slices of dI^v
         "bwd_dk_dIk_pair_rev": 3 * w.d_k * e + 8 * m + 4 * m * nsk,  # q, k, I exp(-G), dz exp(G) -> dk, slices of dI^k
-        "gate_grad": 4 * m * (7 + nsk + nsv),   # u, gate, G, partials -> dgate; carry pass reads gate, r/w dgate
+        "gate_grad": 4 * m * (4 + nsk + nsv),                        # u, gate, G, slices -> dgate
         # fused chunk kernels: the slot rows between the passes stay on chip
         "fused_fwd": e * (2 * w.d_k + 2 * w.d_v) + 12 * m,           # q, k, v, I exp(-G), G -> o, o'
         "fused_bwd": e * (2 * w.d_k + 2 * w.d_v) + 24 * m,           # dO, v, k, I exp(-G), G, o' -> dq, u, p exp(G), dz exp(G)
@@ -457,12 +457,12 @@ def run_ours(args):
         per = {}
         for lab, ms in recs:
             per.setdefault(lab, []).append(ms)
-        # kernels behind one label: gate_grad is three; a chunk pass is one, with 128 slots two (the flagged pairs
+        # kernels behind one label: gate_cumsum is two (the strong-decay flags cleared, too); a chunk pass is one, with 128 slots two (the flagged pairs
         # have a launch of their own there)
         two = sum(len(v) for lab, v in per.items() if lab.endswith("_side") or lab.endswith("_side_rev")) if w.m == 128 else 0
         # a fused label is the fused kernel plus the three kernels that serve the flagged pairs
         fusedl = sum(len(v) for lab, v in per.items() if lab.startswith("fused"))
-        launches = (len(recs) + 2 * len(per.get("gate_grad", [])) + two + 3 * fusedl) // reps
+        launches = (len(recs) + len(per.get("gate_cumsum", [])) + two + 3 * fusedl) // reps
         kernels = []
         tot = sum(sum(v) for v in per.values())
         for lab, v in per.items():

@@ -16,7 +16,7 @@
 // state product.
 //
 // Only for (batch, head) pairs without a strong-decay chunk; the CTAs of flagged ones run the two general
-// scans, one after the other.  Geometry, operand pairs (bf16 value + rounding residual) and bounded waits are those
+// scans, one after the other -- in packed sequences by a CTA each, of a doubled grid.  Geometry, operand pairs (bf16 value + rounding residual) and bounded waits are those
 // of the pipelined single kernels.
 #include "chunk_tc_general.cuh"
 
