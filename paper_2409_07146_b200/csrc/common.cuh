@@ -209,6 +209,7 @@ struct PendingDecay {
     // 128 slots on the tensor-core kernels: G holds exp(G) itself, and a kernel may see the tensors as H = 2 x heads of
     // 64 slots (half_heads), both of which have the flag of their head
     int wide = 0, half_heads = 0;
+    // the answer for token t is that for all rows of its 128-token chunk, and not beyond: the next chunk may be another segment's
     __host__ __device__ bool pending_at(int b, int t, int h) const {
         if (G == nullptr) return false;
         const int seg = nseg == 1 ? 0 : t / tseg;

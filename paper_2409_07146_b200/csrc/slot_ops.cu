@@ -1100,9 +1100,12 @@ __global__ void __launch_bounds__(NT + 32) gate_grad_walk_kernel(
             GateGradRows<KIND, WIDE> r;
             // (in the order that GateGradRows names them: u, 1 - a, the gate, G, the slices)
             const int place[4] = {0, ntiles - 1, 1, 2};
+            // (asked for this thread's eight rows, which lie in one chunk: a tile of 256 may span two segments, a flagged one and
+            // another)
+            const bool pending = pend.pending_at(b, min(row0, T - 1), h);
             r.take([&](int tile, int i) {
                 return *reinterpret_cast<const float*>(smem + (tile < 4 ? place[tile] : first_slice + tile - 4) * (kTile * 4) + ((i * 4) << log_slots));
-            }, nslices, pend.pending_at(b, t0, h));
+            }, nslices, pending);
             __syncwarp();
             if ((threadIdx.x & 31) == 0)
                 asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar_empty[s])) : "memory");
