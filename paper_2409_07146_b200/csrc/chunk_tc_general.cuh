@@ -673,26 +673,39 @@ __device__ __forceinline__ void step_product(float (&c)[2][4], uint32_t x, uint3
 }
 
 // A_ij = sum_s uq_i[s] uk_j[s] prod a_r[s] of a step, on the kept triangle, as accumulator fragments.  While no slot's decay
-// over the step is below e^-60: the decayed rows' product, its uk divided by the step's total decay (kFactorisedDecayMin is the
-// bound of the pipelined kernels' chunks, too).  Otherwise by halves: i and j in the two halves of a block of 2 L tokens meet
+// over the step is below e^-60 (kFactorisedDecayMin is the bound of the pipelined kernels' chunks, too): a product of decayed rows,
+//   forward  (uq_i e_i / e_last) (uk_j s_j),     reversed  (uq_i s_i) (uk_j e_j / e_last),
+// one side as it is and the other divided by the step's total decay (in the frame of step_frame, where its factors cancel): the side that may hold a gradient of any size (dz), beside
+// the input gate.  Its rows with e, up to 2^-87, come 2^kLift larger (`lifted`) and the quotient 2^-kLift smaller, so that both stay
+// within fp32 for gradients of 1e-23 to 1e23.  (With the input gate's rows divided, and the gradient's as small as e makes them,
+// gradients of 1e-17 came out as what subnormal numbers leave of them.)
+// Otherwise by halves: i and j in the two halves of a block of 2 L tokens meet
 // at the block's middle, to which both decay by factors <= 1; four levels L = 8, 4, 2, 1, of which a token plays one part in
 // each -- one pair of rows Z serves both sides -- and the diagonal.
+constexpr int kLift = 43;              // half of -kFactorisedDecayMin log2 e
+__device__ __forceinline__ f32x2 both(float x) { return pack2(x, x); }
+constexpr float kLifted = (float)(1ull << kLift), kLowered = 1.f / kLifted;
 template <bool REV>
-__device__ __forceinline__ void step_weights(float (&c)[2][4], const f32x2 (&kd)[kSub], const unsigned char* uq, const unsigned char* uk, const unsigned char* gates,
+__device__ __forceinline__ void step_weights(float (&c)[2][4], const f32x2 (&lifted)[kSub], const unsigned char* uq, const unsigned char* uk, const unsigned char* gates,
                                              const float2 (&g)[kSub], float2 before, f32x2 inverse, int rows, bool uq_keeps, bool uk_keeps, unsigned char* mine, int lane) {
     unsigned char* Z = mine + kKeyZ;
     const float2 whole = make_float2(g[kSub - 1].x - before.x, g[kSub - 1].y - before.y);
     if (__all_sync(0xffffffffu, fminf(whole.x, whole.y) >= kFactorisedDecayMin)) {
-        // forward: (uq_i e_i) (uk_j s_j / e_last);  reversed: (uq_i s_i) (uk_j e_j / e_last)
+        const f32x2 quotient = mul2(inverse, both(kLowered * kLowered));
 #pragma unroll
         for (int j0 = 0; j0 < kSub; j0 += kBatch) {
             f32x2 f[kBatch];
 #pragma unroll
-            for (int j = 0; j < kBatch; ++j) f[j] = mul2(kd[j0 + j], inverse);
+            for (int j = 0; j < kBatch; ++j) f[j] = mul2(lifted[j0 + j], quotient);
             store_parts<2>(Z, j0, lane, f);
         }
         __syncwarp();
-        step_product(c, smem_u32(mine), smem_u32(Z), lane);
+        if (REV) step_product(c, smem_u32(mine), smem_u32(Z), lane);
+        else step_product(c, smem_u32(Z), smem_u32(mine + kKeyUk), lane);
+#pragma unroll
+        for (int nn = 0; nn < 2; ++nn)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) c[nn][e] *= kLifted;
         return;
     }
     // (rolled loops: few registers, little code beside the usual case)
@@ -770,7 +783,7 @@ __device__ __noinline__ bool key_side_general(const StepMaps maps, const KeySide
             // (the stage of this warp's next step: all are done with the step that it held, the one before this)
             load_step<REV, 1, 2>(ctl, ring, maps, steps, span, d0, n + kSlotWarps);
             next = step_bounds<REV>(a.G, steps, span, a.T, a.H, n + kSlotWarps, lane);
-            f32x2 gate[kSub], kd[kSub];                              // the gates; the decayed uk
+            f32x2 gate[kSub], lifted[kSub];                          // the gates, whose products the factors are; see step_weights
 #pragma unroll
             for (int j = 0; j < kSub; ++j) gate[j] = decay2(j > 0 ? g[j - 1] : before, g[j]);
 #pragma unroll
@@ -778,7 +791,7 @@ __device__ __noinline__ bool key_side_general(const StepMaps maps, const KeySide
                 // the products of the gates from the step's start through a token, and from behind it to the end
                 const bool from_start = (side != 0) == REV;
                 f32x2 run = side != 0 ? frame.weight : frame.out;
-                if (from_start) run = mul2(run, gate[0]);
+                if (from_start) run = mul2(run, mul2(gate[0], both(kLifted)));
 #pragma unroll
                 for (int i0 = 0; i0 < kSub; i0 += kBatch) {
                     const int j0 = from_start ? i0 : kSub - kBatch - i0;
@@ -792,7 +805,9 @@ __device__ __noinline__ bool key_side_general(const StepMaps maps, const KeySide
 #pragma unroll
                     for (int j = 0; j < kBatch; ++j) {
                         f[j] = mul2(weights2(side != 0 ? keys : queries, j0 + j, lane, (side != 0 ? a.uk_keeps : a.uq_keeps) != 0), f[j]);
-                        if (side != 0) kd[j0 + j] = f[j];
+                        if (!from_start) continue;
+                        lifted[j0 + j] = f[j];
+                        f[j] = mul2(f[j], both(kLowered));
                     }
                     store_parts<2>(mine + (side != 0 ? kKeyUk : 0), j0, lane, f);
                 }
@@ -800,7 +815,7 @@ __device__ __noinline__ bool key_side_general(const StepMaps maps, const KeySide
             *reinterpret_cast<f32x2*>(mine + kKeyTotal + 8 * lane) = frame.total;
             __syncwarp();
             float c[2][4];
-            step_weights<REV>(c, kd, queries, keys, gates, g, before, frame.inverse, rows, a.uq_keeps != 0, a.uk_keeps != 0, mine, lane);
+            step_weights<REV>(c, lifted, queries, keys, gates, g, before, frame.inverse, rows, a.uq_keeps != 0, a.uk_keeps != 0, mine, lane);
             unsigned char* A = mine + kKeyA;
 #pragma unroll
             for (int nn = 0; nn < 2; ++nn)

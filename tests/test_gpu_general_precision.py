@@ -1,6 +1,6 @@
 """How exact the scans of flagged (batch, head) pairs are beyond the tolerance of the other tests, root mean square against the fp64
 oracle: the fp32 outputs (logits, gate gradient, final memories), slots that keep nearly all over thousands of tokens beside one
-that forgets."""
+that forgets, and gradients near the ends of what fp32 holds."""
 import numpy as np
 import pytest
 
@@ -48,3 +48,15 @@ def test_slots_that_keep_over_many_tokens():
     ref = oracle.fwd(*(t[:, :, :few] for t in (x["q"], x["k"], x["v"], gate)), gate_is_log=True, K0=x["K0"][:, :few], V0=x["V0"][:, :few])
     errs = {n: rms_err(got[n][:, :few, 1:], ref[n][:, :, 1:]) for n in ("KT", "VT")}
     assert max(errs.values()) <= 1.6e-6, errs
+
+
+# e^-20 to e^-50 a step of 16 tokens in some slot, no more
+@pytest.mark.parametrize("size", [1e-20, 1e-17, 1.0, 1e17])
+def test_gradients_of_any_size(size):
+    B, T, H, d, m = 1, 400, 2, 128, 64
+    x = rand_inputs(17, B, T, H, d, d, m, "bf16")
+    x["dO"] = (x["dO"] * np.float32(2.0 ** np.round(np.log2(size)))).astype(np.float32)
+    x["gate"] = np.exp(-np.minimum(np.random.default_rng(5).gamma(3.0, 1.1, (B, T, H, m)), 3.4)).astype(np.float32)
+    got, ref = run_bwd(x, B, T, H, d, d, m, "bf16", impl="tc", log=True)
+    for n in ("dq", "dk", "dv"):                           # (the rounding to bfloat16 is 1.66e-3)
+        assert rms_err(got[n], ref[n]) <= 1.7e-3, n
