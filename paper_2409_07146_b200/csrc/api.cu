@@ -151,7 +151,7 @@ struct Carver {
 
 struct Workspace {
     float *G, *I, *E, *okpart, *ok, *p, *dz, *u, *dppart, *dIk, *dIv, *chunk_tot, *KT, *VT;
-    int* strong;     // [B*nseg*H] flags: this (b,h) has a chunk that decays too hard for the factorised form
+    int* strong;     // [B*nseg*H] flags: this (b,h) has a chunk that decays too hard for the factorised form; and as many: a large weight
     float *seg_decay, *Kloc, *Vloc, *Kstart, *Vstart;   // segment-parallel scheduling only
     float *dKend, *dVend;                               // ... backward: states entering each segment from the right
     // tensor-core path: bf16 rows [high | residual] of I exp(-G), p exp(G), dz exp(G), each [B,T,H,2m]
@@ -172,7 +172,7 @@ Workspace carve(const CallParams& p, int which, void* ws) {
     const Slices s = slices(p);
     Carver c{static_cast<char*>(ws), 0};
     const int nseg = segments_of(p).n;
-    w.strong = reinterpret_cast<int*>(c.take((size_t)p.B * p.H * nseg));
+    w.strong = reinterpret_cast<int*>(c.take(strong_flags(p.B, p.H, nseg)));
     if (nseg > 1) {
         const size_t pairs = (size_t)p.B * nseg * p.H;
         w.seg_decay = c.take(pairs * p.m);
@@ -226,7 +226,7 @@ GateSums carve_gate(const CallParams& p, void* base) {
     const size_t mt = (size_t)p.B * p.T * p.H * p.m;
     const int nseg = segments_of(p).n;
     Carver c{static_cast<char*>(base), 0};
-    g.strong = reinterpret_cast<int*>(c.take((size_t)p.B * p.H * nseg));
+    g.strong = reinterpret_cast<int*>(c.take(strong_flags(p.B, p.H, nseg)));
     g.G = c.take(mt);
     g.I = c.take(mt);
     g.E = use_wide(p) ? c.take(mt) : nullptr;
@@ -302,7 +302,7 @@ cudaError_t gate_products(const gsa_params_t& p, Segments segs, const float* gat
                           cudaStream_t st) {
     const int chunk = chunk_of(p), nchunks = (p.T + chunk - 1) / chunk;
     if (use_tc(p) && (use_wide(p) || !owns_strong_flag(segs.n, nchunks))) {
-        const cudaError_t e = launch_clear_flags(w.strong, (size_t)p.B * p.H * segs.n, st);
+        const cudaError_t e = launch_clear_flags(w.strong, strong_flags(p.B, p.H, segs.n), st);
         if (e != cudaSuccess) return e;
     }
     if (use_wide(p))
@@ -624,7 +624,7 @@ gsa_status_t fwd_core(const CallParams* params, int m_active, const void* q, con
     const float* I = reads_gate(p) ? gate : w.I;          // (of the scans in fp32: the general ones)
     const int keeps = reads_gate(p);
     if (p.gate_kind == GSA_GATE_ABC) {    // no decay, write weights from the cumulative softmax of the scores
-        GSA_CUDA(launch_clear_flags(w.strong, (size_t)p.B * p.H * nseg, st));
+        GSA_CUDA(launch_clear_flags(w.strong, strong_flags(p.B, p.H, nseg), st));
         GSA_LAUNCH("abc_write", launch_abc_write(gate, w.G, w.I, w.Id, p.B, p.T, p.H, p.m, st));
     } else
         GSA_LAUNCH("gate_cumsum", gate_products(p, segs, gate, w, !left_out, st));
@@ -806,7 +806,7 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
     const int keeps = reads_gate(p);
     if (!gate_is_saved) {      // (a forward of the same call left the gate kernel's products otherwise)
         if (p.gate_kind == GSA_GATE_ABC) {
-            GSA_CUDA(launch_clear_flags(w.strong, (size_t)p.B * p.H * nseg, st));
+            GSA_CUDA(launch_clear_flags(w.strong, strong_flags(p.B, p.H, nseg), st));
             GSA_LAUNCH("abc_write", launch_abc_write(gate, w.G, w.I, w.Id, p.B, p.T, p.H, p.m, st));
         } else
             GSA_LAUNCH("gate_cumsum", gate_products(p, segs, gate, w, !left_out, st));

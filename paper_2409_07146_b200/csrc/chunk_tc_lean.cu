@@ -688,8 +688,9 @@ state_scan_kernel(const __grid_constant__ CUtensorMap mapX0, const __grid_consta
         }
         if (!REV) write_input_gate(a);
         const StepMaps maps{{&general.x[second], nullptr}, {&general.w[second], nullptr}, &general.G};
-        if (value_side_general<REV, true>(maps, a, dev_status, slice) && BOTH)
-            value_side_general<REV, true>(StepMaps{{&general.x[1], nullptr}, {&general.w[1], nullptr}, &general.G}, sets.set[1], dev_status, 0);
+        const Steps steps = remembered_steps<REV, BOTH>(a, sets.set[1], slice, !REV && strong_flag[gridDim.x + blockIdx.x] != 0);
+        if (value_side_general<REV, true>(maps, a, dev_status, slice, steps) && BOTH)
+            value_side_general<REV, true>(StepMaps{{&general.x[1], nullptr}, {&general.w[1], nullptr}, &general.G}, sets.set[1], dev_status, 0, steps);
         return;
     }
     const float* G = a.G;

@@ -226,8 +226,10 @@ cudaError_t launch_clear_flags(int* flags, size_t n, cudaStream_t st);
 // (Up to eight chunks, their CTAs a cluster whose first one collects: the cluster's launch and barriers cost more than the clearing,
 // in a graph 24.6 -> 25.8 us at 130 tokens, 56 -> 60 at B = 2, T = 1024, 16 heads of 128.)
 __host__ __device__ inline bool owns_strong_flag(int nseg, int nchunks) { return nseg == nchunks; }
-// strong_flag (nullable, [B*H] ints, zeroed by launch_clear_flags, but see owns_strong_flag): set to 1 for every (b,h) that has a
-// chunk whose total log-decay is below kFactorisedDecayMin (nseg > 1: [B*nseg*H], per segment).
+// strong_flag (nullable, [2*B*H] ints, zeroed by launch_clear_flags, but see owns_strong_flag): set to 1 for every (b,h) that has a
+// chunk whose total log-decay is below kFactorisedDecayMin (nseg > 1: [2*B*nseg*H], per segment); behind these flags as many for a
+// weight 1 - a that is 2 or more or no finite number (64-slot tiles only).
+constexpr size_t strong_flags(int B, int H, int nseg) { return 2 * (size_t)B * H * nseg; }
 // decayed (nullable, bf16 [B,T,H,2M]): rows [high part | rounding residual] of I exp(-G), the
 // input-gate operand of the pipelined tensor-core kernels.  leave_out: I only of the chunks that decay
 // below kFactorisedDecayMin (1, see InputGate), or not at all (2).  fast_log: take log a with the

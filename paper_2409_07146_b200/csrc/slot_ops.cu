@@ -174,10 +174,22 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
     const bool owns_flag = !WIDE && strong_flag != nullptr && owns_strong_flag(nseg, (int)gridDim.y);
     bool any_strong = strong;
     if (owns_flag || leave_out == 1) any_strong = __syncthreads_or(strong);
+    // is there a weight that is 2 or more, or no finite number (the exponent's top bit)?  See remembered_steps.
+    uint32_t seen = 0;
+    if (!WIDE && strong_flag != nullptr) {
+#pragma unroll
+        for (int i = 0; i < kCumRows; ++i) seen |= __float_as_uint(inps[i].x) | __float_as_uint(inps[i].y);
+        seen &= 0x40000000u;
+        if (owns_flag) seen = __syncthreads_or(seen);
+    }
     const bool put_I = leave_out == 0 || (leave_out == 1 && any_strong);
     if (strong || (owns_flag && threadIdx.x == 0 && grp == 0)) {
         const int seg = nseg == 1 ? 0 : t_chunk / tseg;
         strong_flag[WIDE ? (b * nseg + seg) * (H / 2) + h / 2 : (b * nseg + seg) * H + h] = any_strong;
+    }
+    if (seen != 0 || (owns_flag && threadIdx.x == 0 && grp == 0)) {
+        const int seg = nseg == 1 ? 0 : t_chunk / tseg;
+        strong_flag[(int)gridDim.x * nseg + (b * nseg + seg) * H + h] = seen != 0;
     }
     // second pass over the same rows: the sums of the groups before as a float pair (value, rest)
     const float b0h = (float)before0, b0l = (float)(before0 - (double)b0h);
