@@ -219,15 +219,16 @@ GSA_API gsa_status_t gsa_bwd(const gsa_params_t* params, const void* q, const vo
  * tensor-core path also the forward's slot weights p (as the backward's reversed scans read them:
  * they depend on the saved logits only, and with them in hand the backward starts its dv scan at
  * once) and, where a long sequence is cut into segments, the segments' decay, the memories entering
- * every segment and the final memories, and with a feature map the activated q, k and v, in gate_save, a device block of gsa_workspace_bytes(params, GSA_WS_GATE) bytes, 256-byte
+ * every segment and the final memories, and with a feature map the activated q and k (and v where the sequence is cut), in
+ * gate_save, a device block of gsa_workspace_bytes(params, GSA_WS_GATE) bytes, 256-byte
  * aligned, owned by the caller; gsa_bwd_saved_gate reads them from there instead of running
- * the gate kernel (and the segments' forward-direction state runs) again.  Both calls must use the same params and the same q, k, v and gate
- * tensors; nothing checks that.  A missing, misaligned or short block is GSA_ERR_WORKSPACE.
+ * the gate kernel (and the segments' forward-direction state runs) again.  Both calls must use the same params and the same gate
+ * tensor, where ok_saved is given the q and k that it is of, and where the sequence is cut into segments the same k and v;
+ * nothing checks that.  A missing, misaligned or short block is GSA_ERR_WORKSPACE.
  * Its size, in slot-sized fp32 tensors [B,T,H,m]: 5 with bf16 io (84 MB at B = 8, T = 2048, H = 4,
  * m = 64; 32 slots count as 64), 7 with bf16 io and 128 slots (235 MB there), 2 on the fp32 CUDA-core
  * kernels; plus, where the scans are cut into segments, a set of memories [B,H,m,d_k + d_v] for every
- * segment and one for the end; plus, with a feature map, q, k and v again (gsa_fwd and gsa_bwd, without a block, form them in
- * their workspaces, twice).
+ * segment and one for the end; plus, with a feature map, q and k again (and v where the sequence is cut).
  */
 GSA_API gsa_status_t gsa_fwd_save_gate(const gsa_params_t* params, const void* q, const void* k,
                                        const void* v, const float* gate, const float* K0,

@@ -480,37 +480,48 @@ size_t gate_conv_bytes(const gsa_params_t& p, int which = GSA_WS_BWD) { return g
 // The layer's feature map: Swish(q), Swish(k), Swish(v) are formed once a call, in the part of the workspace
 // that follows everything else; the scans then read those copies.
 struct FeatureBuffers { void *q, *k, *v; size_t bytes; };
-FeatureBuffers carve_features(const gsa_params_t& p, void* base) {
+FeatureBuffers carve_features(const gsa_params_t& p, void* base, bool with_v = true) {
     FeatureBuffers f{nullptr, nullptr, nullptr, 0};
     if (p.feature_map != GSA_FEAT_SWISH) return f;
     const size_t e = p.io == GSA_BF16 ? 2 : 4, R = (size_t)p.B * p.T * p.H;
     const size_t nk = align_up(R * p.d_k * e, 256), nv = align_up(R * p.d_v * e, 256);
     char* b = static_cast<char*>(base);
     f.q = b; f.k = b + nk; f.v = b + 2 * nk;
-    f.bytes = 2 * nk + nv;
+    f.bytes = 2 * nk + (with_v ? nv : 0);
     return f;
 }
-// (a block that the forward keeps for the backward takes them in the workspace's place, behind what else it holds, and the
-// backward finds them there: B = 4, T = 1999, 5 heads of 512, 0.25 GB and 38 us less)
+// A block that the forward keeps for the backward takes q and k in the workspace's place, behind what else it holds, and a backward
+// that is given the logits, which are those of this q and k, finds them there; v too where the block holds the memories that enter
+// segments, which are those of this v.  What nothing in hand depends on is formed of the tensors that the backward is
+// handed, which may be others.  B = 4, T = 1999, 5 heads of 512: all formed again 41 us of the layer's training step, v alone 23 (588
+// in all).
+bool keeps_v(const CallParams& p) { return segments_of(internal_params(p)).n > 1; }
 gsa_status_t apply_feature_map(const CallParams& p, int which, const void** q, const void** k, const void** v, void* ws,
-                               size_t ws_bytes, bool kept, const void* block, size_t block_bytes, cudaStream_t st) {
+                               size_t ws_bytes, bool kept, const void* block, size_t block_bytes, bool with_logits, cudaStream_t st) {
     if (p.feature_map != GSA_FEAT_SWISH) return GSA_OK;
+    auto usable = [](const void* x) { return x != nullptr && (reinterpret_cast<uintptr_t>(x) & 255u) == 0; };
     const CallParams pi = internal_params(p);
-    const size_t before = kept ? carve_gate(pi, nullptr).bytes
-                               : carve(pi, which, nullptr).bytes + pad_bytes(p, which) + gate_conv_bytes(p, which);
-    void* base = kept ? const_cast<void*>(block) : ws;
-    if (base == nullptr || (reinterpret_cast<uintptr_t>(base) & 255u) != 0) return GSA_ERR_WORKSPACE;
-    const FeatureBuffers f = carve_features(p, static_cast<char*>(base) + before);
-    if ((kept ? block_bytes : ws_bytes) < before + f.bytes) return GSA_ERR_WORKSPACE;
-    if (kept && which == GSA_WS_BWD) {
-        *q = f.q; *k = f.k; *v = f.v;
-        return GSA_OK;
+    const bool v_kept = kept && keeps_v(p), formed = which == GSA_WS_FWD || !kept, qk_formed = formed || !with_logits, v_formed = formed || !v_kept;
+    FeatureBuffers f{nullptr, nullptr, nullptr, 0}, b = f;
+    if (kept) {
+        const size_t at = carve_gate(pi, nullptr).bytes;
+        b = carve_features(p, const_cast<char*>(static_cast<const char*>(block)) + at, v_kept);
+        if (!usable(block) || block_bytes < at + b.bytes) return GSA_ERR_WORKSPACE;
     }
+    // (the forward forms them where the backward will look)
+    const bool qk_in_block = kept && (which == GSA_WS_FWD || with_logits);
+    if (!qk_in_block || !v_kept) {
+        const size_t at = carve(pi, which, nullptr).bytes + pad_bytes(p, which) + gate_conv_bytes(p, which);
+        f = carve_features(p, static_cast<char*>(ws) + at);
+        if (!usable(ws) || ws_bytes < at + f.bytes) return GSA_ERR_WORKSPACE;
+    }
+    if (qk_in_block) { f.q = b.q; f.k = b.k; }
+    if (v_kept) f.v = b.v;
     const size_t R = (size_t)p.B * p.T * p.H;
     const void* const in[3] = {*q, *k, *v};
     void* const out[3] = {f.q, f.k, f.v};
-    const size_t n[3] = {R * p.d_k, R * p.d_k, R * p.d_v};
-    if (launch_swish_fwd(in, out, n, p.io, st) != cudaSuccess) return GSA_ERR_CUDA;
+    const size_t n[3] = {qk_formed ? R * p.d_k : 0, qk_formed ? R * p.d_k : 0, v_formed ? R * p.d_v : 0};
+    if ((qk_formed || v_formed) && launch_swish_fwd(in, out, n, p.io, st) != cudaSuccess) return GSA_ERR_CUDA;
     *q = f.q; *k = f.k; *v = f.v;
     return GSA_OK;
 }
@@ -574,7 +585,7 @@ const char* gsa_status_string(gsa_status_t status) {
 namespace {
 size_t workspace_bytes(const CallParams& p, int32_t which) {
     const CallParams pi = internal_params(p);
-    if (which == GSA_WS_GATE) return carve_gate(pi, nullptr).bytes + carve_features(p, nullptr).bytes;
+    if (which == GSA_WS_GATE) return carve_gate(pi, nullptr).bytes + carve_features(p, nullptr, keeps_v(p)).bytes;
     return carve(pi, which, nullptr).bytes + pad_bytes(p, which) + gate_conv_bytes(p, which) + carve_features(p, nullptr).bytes;
 }
 }  // namespace
@@ -706,7 +717,7 @@ gsa_status_t fwd_impl(const CallParams* params, const void* q, const void* k, co
         rc = gate_as_f32(*params, GSA_WS_FWD, gate, ws, ws_bytes, before, static_cast<cudaStream_t>(stream), &gate);
         if (rc != GSA_OK) return rc;
         rc = apply_feature_map(*params, GSA_WS_FWD, &q, &k, &v, ws, ws_bytes, save_gate, gate_save, gate_save_bytes,
-                               static_cast<cudaStream_t>(stream));
+                               true, static_cast<cudaStream_t>(stream));
         if (rc != GSA_OK) return rc;
     }
     if (!pads_slots(*params))
@@ -1004,7 +1015,7 @@ gsa_status_t bwd_impl(const CallParams* params, const void* q, const void* k, co
         rc = gate_as_f32(*params, GSA_WS_BWD, gate, ws, ws_bytes, before, static_cast<cudaStream_t>(stream), &gate);
         if (rc != GSA_OK) return rc;
         rc = apply_feature_map(*params, GSA_WS_BWD, &q, &k, &v, ws, ws_bytes, gate_is_saved, gate_saved, gate_saved_bytes,
-                               static_cast<cudaStream_t>(stream));
+                               ok_saved != nullptr, static_cast<cudaStream_t>(stream));
         if (rc != GSA_OK) return rc;
         if (params->gate_broadcast) {        // the per-token gate gradient lands in the workspace; its sum is returned
             const GateBoundary g = gate_boundary(*params, GSA_WS_BWD);
