@@ -151,7 +151,7 @@ struct Carver {
 
 struct Workspace {
     float *G, *I, *E, *okpart, *ok, *p, *dz, *u, *dppart, *dIk, *dIv, *chunk_tot, *KT, *VT;
-    int* strong;     // [B*nseg*H] flags: this (b,h) has a chunk that decays too hard for the factorised form; and as many: a large weight
+    int* strong;     // [B*nseg*H] flags: this (b,h) has a chunk that decays too hard for the factorised form
     float *seg_decay, *Kloc, *Vloc, *Kstart, *Vstart;   // segment-parallel scheduling only
     float *dKend, *dVend;                               // ... backward: states entering each segment from the right
     // tensor-core path: bf16 rows [high | residual] of I exp(-G), p exp(G), dz exp(G), each [B,T,H,2m]
@@ -172,7 +172,7 @@ Workspace carve(const CallParams& p, int which, void* ws) {
     const Slices s = slices(p);
     Carver c{static_cast<char*>(ws), 0};
     const int nseg = segments_of(p).n;
-    w.strong = reinterpret_cast<int*>(c.take(strong_flags(p.B, p.H, nseg)));
+    w.strong = reinterpret_cast<int*>(c.take((size_t)p.B * p.H * nseg));
     if (nseg > 1) {
         const size_t pairs = (size_t)p.B * nseg * p.H;
         w.seg_decay = c.take(pairs * p.m);
@@ -226,7 +226,7 @@ GateSums carve_gate(const CallParams& p, void* base) {
     const size_t mt = (size_t)p.B * p.T * p.H * p.m;
     const int nseg = segments_of(p).n;
     Carver c{static_cast<char*>(base), 0};
-    g.strong = reinterpret_cast<int*>(c.take(strong_flags(p.B, p.H, nseg)));
+    g.strong = reinterpret_cast<int*>(c.take((size_t)p.B * p.H * nseg));
     g.G = c.take(mt);
     g.I = c.take(mt);
     g.E = use_wide(p) ? c.take(mt) : nullptr;
@@ -295,6 +295,10 @@ InputGate input_gate_of(const gsa_params_t& p, const float* gate, bool left_out)
     return left_out && !reads_gate(p) ? InputGate{gate, p.gate_kind, inv_tau(p)} : InputGate{};
 }
 
+// [B*nseg*H] flags from the gate kernel for the state runs, which follow it: a weight that is not below 2 (see remembered_steps).  They
+// lie where pass 1 will write.
+int* large_weights(const Workspace& w) { return reinterpret_cast<int*>(w.okpart); }
+
 // the gate kernel: G, 1 - a, the decayed rows and the strong-decay flags, cleared first where several of its CTAs share one (the
 // CUDA-core kernels do without)
 // (input_gate = false: 1 - a is left out, see leaves_input_gate)
@@ -302,14 +306,15 @@ cudaError_t gate_products(const gsa_params_t& p, Segments segs, const float* gat
                           cudaStream_t st) {
     const int chunk = chunk_of(p), nchunks = (p.T + chunk - 1) / chunk;
     if (use_tc(p) && (use_wide(p) || !owns_strong_flag(segs.n, nchunks))) {
-        const cudaError_t e = launch_clear_flags(w.strong, strong_flags(p.B, p.H, segs.n), st);
+        const cudaError_t e = launch_clear_flags(w.strong, use_wide(p) ? nullptr : large_weights(w), (size_t)p.B * p.H * segs.n, st);
         if (e != cudaSuccess) return e;
     }
     if (use_wide(p))
         return launch_gate_cumsum_wide(gate, p.gate_kind, inv_tau(p), w.G, w.I, w.E, p.B, p.T, p.H, w.strong, segs.n, segs.t,
                                        w.Id, st, p.cu_seqlens, p.nseq);
     return launch_gate_cumsum(gate, p.gate_kind, inv_tau(p), w.G, w.I, p.B, p.T, p.H, p.m, chunk_of(p), use_tc(p) ? w.strong : nullptr, segs.n,
-                              segs.t, w.Id, p.io == GSA_BF16, st, p.cu_seqlens, p.nseq, reads_gate(p) ? 2 : (input_gate ? 0 : 1));
+                              segs.t, w.Id, p.io == GSA_BF16, st, p.cu_seqlens, p.nseq, reads_gate(p) ? 2 : (input_gate ? 0 : 1),
+                              use_tc(p) ? large_weights(w) : nullptr);
 }
 // the row factors that the tensor-core value_side scans leave to the slot kernels
 PendingDecay pending_decay(const gsa_params_t& p, Segments segs, const Workspace& w) {
@@ -336,7 +341,7 @@ cudaError_t state_scans(const gsa_params_t& p, Segments segs, StateSet ks, State
         return launch_state_scans_wide(a[0], a[1], reverse, w.strong, st, dev_status);
     }
     a[0].seg_logdecay = logdecay;
-    if (use_tc(p)) return launch_state_scan_tc(a[0], a[1], reverse, w.strong, st, dev_status);
+    if (use_tc(p)) return launch_state_scan_tc(a[0], a[1], reverse, w.strong, large_weights(w), st, dev_status);
     return launch_state_scan_simt(a[0], a[1], p.io, p.m, reverse, st);
 }
 
@@ -635,7 +640,7 @@ gsa_status_t fwd_core(const CallParams* params, int m_active, const void* q, con
     const float* I = reads_gate(p) ? gate : w.I;          // (of the scans in fp32: the general ones)
     const int keeps = reads_gate(p);
     if (p.gate_kind == GSA_GATE_ABC) {    // no decay, write weights from the cumulative softmax of the scores
-        GSA_CUDA(launch_clear_flags(w.strong, strong_flags(p.B, p.H, nseg), st));
+        GSA_CUDA(launch_clear_flags(w.strong, nullptr, (size_t)p.B * p.H * nseg, st));
         GSA_LAUNCH("abc_write", launch_abc_write(gate, w.G, w.I, w.Id, p.B, p.T, p.H, p.m, st));
     } else
         GSA_LAUNCH("gate_cumsum", gate_products(p, segs, gate, w, !left_out, st));
@@ -817,7 +822,7 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
     const int keeps = reads_gate(p);
     if (!gate_is_saved) {      // (a forward of the same call left the gate kernel's products otherwise)
         if (p.gate_kind == GSA_GATE_ABC) {
-            GSA_CUDA(launch_clear_flags(w.strong, strong_flags(p.B, p.H, nseg), st));
+            GSA_CUDA(launch_clear_flags(w.strong, nullptr, (size_t)p.B * p.H * nseg, st));
             GSA_LAUNCH("abc_write", launch_abc_write(gate, w.G, w.I, w.Id, p.B, p.T, p.H, p.m, st));
         } else
             GSA_LAUNCH("gate_cumsum", gate_products(p, segs, gate, w, !left_out, st));

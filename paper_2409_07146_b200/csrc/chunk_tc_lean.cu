@@ -662,6 +662,7 @@ struct ScanCtl {
 struct StateScanArgs {
     ValueSideArgs set[2];             // (xk, w and wd: the tile that enters the state and its weights; Send)
     int slices0;
+    const int* large_weight;          // forward: [scans], see launch_gate_cumsum
 };
 
 struct GeneralStateMaps { CUtensorMap x[2], w[2], G; };
@@ -688,7 +689,7 @@ state_scan_kernel(const __grid_constant__ CUtensorMap mapX0, const __grid_consta
         }
         if (!REV) write_input_gate(a);
         const StepMaps maps{{&general.x[second], nullptr}, {&general.w[second], nullptr}, &general.G};
-        const Steps steps = remembered_steps<REV, BOTH>(a, sets.set[1], slice, !REV && strong_flag[gridDim.x + blockIdx.x] != 0);
+        const Steps steps = remembered_steps<REV, BOTH>(a, sets.set[1], slice, !REV && sets.large_weight[blockIdx.x] != 0);
         if (value_side_general<REV, true>(maps, a, dev_status, slice, steps) && BOTH)
             value_side_general<REV, true>(StepMaps{{&general.x[1], nullptr}, {&general.w[1], nullptr}, &general.G}, sets.set[1], dev_status, 0, steps);
         return;
@@ -854,8 +855,8 @@ constexpr size_t kSmemLeanKey = 1024 + 14 * kPanelB + sizeof(LeanCtl);     // ke
 }  // namespace
 
 cudaError_t launch_state_scan_tc(const ValueSideArgs& k, const ValueSideArgs& v, int reverse, const int* strong_flag,
-                                 cudaStream_t st, int32_t* dev_status) {
-    StateScanArgs sets{{k, v}, tc_value_side_slices(k.D)};
+                                 const int* large_weight, cudaStream_t st, int32_t* dev_status) {
+    StateScanArgs sets{{k, v}, tc_value_side_slices(k.D), large_weight};
     CUtensorMap mx[2], mw[2];
     GeneralStateMaps general;
     cudaError_t e = step_map(&general.G, k.G, k.B, k.T, k.H, kM, 4);

@@ -220,16 +220,16 @@ struct PendingDecay {
 };
 
 // launchers (definitions in the .cu files); all return cudaGetLastError() of the launch
-cudaError_t launch_clear_flags(int* flags, size_t n, cudaStream_t st);
+// n of each (others nullable)
+cudaError_t launch_clear_flags(int* flags, int* others, size_t n, cudaStream_t st);
 // Is a strong-decay flag written by one CTA of the gate kernel alone (64-slot tiles)?  It then needs no clearing, which is a launch
 // of a short call's five: pairs or segments of a single chunk (a forward over 114 tokens, 8 heads of 256: 29.8 -> 27.0 us).
 // (Up to eight chunks, their CTAs a cluster whose first one collects: the cluster's launch and barriers cost more than the clearing,
 // in a graph 24.6 -> 25.8 us at 130 tokens, 56 -> 60 at B = 2, T = 1024, 16 heads of 128.)
 __host__ __device__ inline bool owns_strong_flag(int nseg, int nchunks) { return nseg == nchunks; }
-// strong_flag (nullable, [2*B*H] ints, zeroed by launch_clear_flags, but see owns_strong_flag): set to 1 for every (b,h) that has a
-// chunk whose total log-decay is below kFactorisedDecayMin (nseg > 1: [2*B*nseg*H], per segment); behind these flags as many for a
-// weight 1 - a that is 2 or more or no finite number (64-slot tiles only).
-constexpr size_t strong_flags(int B, int H, int nseg) { return 2 * (size_t)B * H * nseg; }
+// strong_flag (nullable, [B*H] ints, zeroed by launch_clear_flags, but see owns_strong_flag): set to 1 for every (b,h) that has a
+// chunk whose total log-decay is below kFactorisedDecayMin (nseg > 1: [B*nseg*H], per segment).  large_weight (with strong_flag
+// only, as many, alike): one with a weight 1 - a that is 2 or more or no finite number.
 // decayed (nullable, bf16 [B,T,H,2M]): rows [high part | rounding residual] of I exp(-G), the
 // input-gate operand of the pipelined tensor-core kernels.  leave_out: I only of the chunks that decay
 // below kFactorisedDecayMin (1, see InputGate), or not at all (2).  fast_log: take log a with the
@@ -238,7 +238,7 @@ constexpr size_t strong_flags(int B, int H, int nseg) { return 2 * (size_t)B * H
 cudaError_t launch_gate_cumsum(const float* gate, int gate_kind, float inv_tau, float* G, float* I,
                                int B, int T, int H, int M, int chunk, int* strong_flag, int nseg, int tseg,
                                void* decayed, int fast_log, cudaStream_t st, const int* cu_seqlens = nullptr,
-                               int nseq = 0, int leave_out = 0);
+                               int nseq = 0, int leave_out = 0, int* large_weight = nullptr);
 // The same for the tensor-core kernels with 128 slots, M = 2 x 64: `decayed` are bf16 [B,T,2H,192] rows [high | middle |
 // low part] of I exp(-G), E = exp(G), local to chunks of 128 tokens; both, and log a, to fp32 accuracy whatever the io
 // type.  G is local to 64 tokens, the chunks of the CUDA-core kernels that take the flagged pairs.
@@ -321,7 +321,7 @@ cudaError_t launch_key_side_general(const KeySideArgs& a, const int* strong_flag
 // end memories only, from empty ones, of the K and the V side in one launch: xk, w and wd of each set are the tile that
 // enters the state and its weights (key_side: xv, uk, uk_d)
 cudaError_t launch_state_scan_tc(const ValueSideArgs& k, const ValueSideArgs& v, int reverse, const int* strong_flag,
-                                 cudaStream_t st, int32_t* dev_status);
+                                 const int* large_weight, cudaStream_t st, int32_t* dev_status);
 // The two reversed scans that share a state (dv with dI^v, dk with dI^k) as one kernel
 // (chunk_tc_pair.cu): av / ak are the arguments the single reversed scans would get.
 bool rev_pair_supported(const ValueSideArgs& av, const KeySideArgs& ak, int M);

@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
                                                             int chunk, int* __restrict__ strong_flag, int nseg, int tseg,
                                                             __nv_bfloat16* __restrict__ decayed, int fast_log,
                                                             const int* cu_seqlens, int nseq,
-                                                            float* __restrict__ E, int leave_out) {
+                                                            float* __restrict__ E, int leave_out, int* __restrict__ large_weight) {
     follow_previous_grid();
     __shared__ double2 group_sum[16][M / 2];
     const int grp = threadIdx.y, s = 2 * threadIdx.x;          // blockDim.y = chunk / 8 <= 16
@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
     if (owns_flag || leave_out == 1) any_strong = __syncthreads_or(strong);
     // is there a weight that is 2 or more, or no finite number (the exponent's top bit)?  See remembered_steps.
     uint32_t seen = 0;
-    if (!WIDE && strong_flag != nullptr) {
+    if (!WIDE && large_weight != nullptr) {
 #pragma unroll
         for (int i = 0; i < kCumRows; ++i) seen |= __float_as_uint(inps[i].x) | __float_as_uint(inps[i].y);
         seen &= 0x40000000u;
@@ -187,9 +187,9 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
         const int seg = nseg == 1 ? 0 : t_chunk / tseg;
         strong_flag[WIDE ? (b * nseg + seg) * (H / 2) + h / 2 : (b * nseg + seg) * H + h] = any_strong;
     }
-    if (seen != 0 || (owns_flag && threadIdx.x == 0 && grp == 0)) {
+    if (seen != 0 || (owns_flag && large_weight != nullptr && threadIdx.x == 0 && grp == 0)) {
         const int seg = nseg == 1 ? 0 : t_chunk / tseg;
-        strong_flag[(int)gridDim.x * nseg + (b * nseg + seg) * H + h] = seen != 0;
+        large_weight[(b * nseg + seg) * H + h] = seen != 0;
     }
     // second pass over the same rows: the sums of the groups before as a float pair (value, rest)
     const float b0h = (float)before0, b0l = (float)(before0 - (double)b0h);
@@ -238,26 +238,29 @@ void launch_gate_kind(int gate_kind, dim3 grid, dim3 block, cudaStream_t st, con
 
 // a kernel rather than a memset, which the gate kernel could not follow closely (launch_after): a forward over 1431 tokens,
 // 4 heads of 512, 50.7 -> 48.0 us; one over 256 tokens in fp32, which needs no flags, 33.7 -> 30.2
-__global__ void clear_flags_kernel(int* __restrict__ flags, size_t n) {
+__global__ void clear_flags_kernel(int* __restrict__ flags, int* __restrict__ others, size_t n) {
     follow_previous_grid();
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) flags[i] = 0;
+    if (i < n) {
+        flags[i] = 0;
+        if (others != nullptr) others[i] = 0;
+    }
 }
-cudaError_t launch_clear_flags(int* flags, size_t n, cudaStream_t st) {
-    launch_after(clear_flags_kernel, dim3((unsigned)((n + 255) / 256)), 256, 0, st, flags, n);
+cudaError_t launch_clear_flags(int* flags, int* others, size_t n, cudaStream_t st) {
+    launch_after(clear_flags_kernel, dim3((unsigned)((n + 255) / 256)), 256, 0, st, flags, others, n);
     return cudaGetLastError();
 }
 
 cudaError_t launch_gate_cumsum(const float* gate, int gate_kind, float inv_tau, float* G, float* I, int B,
                                int T, int H, int M, int chunk, int* strong_flag, int nseg, int tseg, void* decayed, int fast_log,
-                               cudaStream_t st, const int* cu_seqlens, int nseq, int leave_out) {
+                               cudaStream_t st, const int* cu_seqlens, int nseq, int leave_out, int* large_weight) {
     if (chunk % kCumRows != 0 || chunk / kCumRows > 16 || (M / 2) * (chunk / kCumRows) > 1024) return cudaErrorInvalidValue;
     const int nchunks = (T + chunk - 1) / chunk;
     dim3 block(M / 2, chunk / kCumRows);
     dim3 grid(B * H, nchunks);
     auto launch = [&](auto m) {
         launch_gate_kind<decltype(m)::value, false>(gate_kind, grid, block, st, gate, inv_tau, G, I, T, H, chunk, strong_flag, nseg, tseg,
-                                                    static_cast<__nv_bfloat16*>(decayed), fast_log, cu_seqlens, nseq, (float*)nullptr, leave_out);
+                                                    static_cast<__nv_bfloat16*>(decayed), fast_log, cu_seqlens, nseq, (float*)nullptr, leave_out, large_weight);
     };
     if (M == 128) launch(std::integral_constant<int, 128>{});
     else if (M == 64) launch(std::integral_constant<int, 64>{});
@@ -270,7 +273,7 @@ cudaError_t launch_gate_cumsum_wide(const float* gate, int gate_kind, float inv_
                                     const int* cu_seqlens, int nseq) {
     constexpr int chunk = 128;
     launch_gate_kind<64, true>(gate_kind, dim3(2 * B * H, (T + chunk - 1) / chunk), dim3(32, chunk / kCumRows), st, gate, inv_tau, G, I, T,
-                               2 * H, chunk, strong_flag, nseg, tseg, static_cast<__nv_bfloat16*>(decayed), 0, cu_seqlens, nseq, E, 0);
+                               2 * H, chunk, strong_flag, nseg, tseg, static_cast<__nv_bfloat16*>(decayed), 0, cu_seqlens, nseq, E, 0, (int*)nullptr);
     return cudaGetLastError();
 }
 
