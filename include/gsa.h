@@ -226,8 +226,8 @@ GSA_API gsa_status_t gsa_bwd(const gsa_params_t* params, const void* q, const vo
  * tensor, where ok_saved is given the q and k that it is of, and where the sequence is cut into segments the same k and v;
  * nothing checks that.  A missing, misaligned or short block is GSA_ERR_WORKSPACE.
  * Its size, in slot-sized fp32 tensors [B,T,H,m]: 5 with bf16 io (84 MB at B = 8, T = 2048, H = 4,
- * m = 64; 32 slots count as 64), 7 with bf16 io and 128 slots (235 MB there), 2 on the fp32 CUDA-core
- * kernels; plus, where the scans are cut into segments, a set of memories [B,H,m,d_k + d_v] for every
+ * m = 64; 32 slots count as 64), 4 where the gate tensor holds a, 7 with bf16 io and 128 slots (235 MB there), 2 on the
+ * fp32 CUDA-core kernels; plus, where the scans are cut into segments, a set of memories [B,H,m,d_k + d_v] for every
  * segment and one for the end; plus, with a feature map, q and k again (and v where the sequence is cut).
  */
 GSA_API gsa_status_t gsa_fwd_save_gate(const gsa_params_t* params, const void* q, const void* k,

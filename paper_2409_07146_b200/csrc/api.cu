@@ -88,6 +88,10 @@ bool use_fused(const gsa_params_t& p) {
            fused_pair_supported(p.d_k, p.d_v, p.m);
 }
 
+// Do the general scans, which alone read 1 - a in fp32 on the tensor cores with 64 slots (see leaves_input_gate), take it from a gate tensor that
+// holds a?  Nothing writes 1 - a then.  (16 heads, 32 K tokens of strong gates: the gate kernel 94 -> 82 us)
+bool reads_gate(const gsa_params_t& p) { return use_tc(p) && !use_wide(p) && p.gate_kind == GSA_GATE_A; }
+
 float inv_tau(const gsa_params_t& p) { return p.tau > 0.f ? 1.f / p.tau : 0.f; }
 
 int chunk_of(const gsa_params_t& p) { return use_tc(p) ? tc_chunk() : kChunk; }
@@ -186,7 +190,7 @@ Workspace carve(const CallParams& p, int which, void* ws) {
         }
     }
     w.G = c.take(mt);
-    w.I = c.take(mt);
+    if (!reads_gate(p)) w.I = c.take(mt);
     w.okpart = c.take(mt * s.k);
     w.ok = c.take(mt);
     w.p = c.take(mt);
@@ -228,7 +232,7 @@ GateSums carve_gate(const CallParams& p, void* base) {
     Carver c{static_cast<char*>(base), 0};
     g.strong = reinterpret_cast<int*>(c.take((size_t)p.B * p.H * nseg));
     g.G = c.take(mt);
-    g.I = c.take(mt);
+    if (!reads_gate(p)) g.I = c.take(mt);
     g.E = use_wide(p) ? c.take(mt) : nullptr;
     g.Id = use_tc(p) ? c.take(decayed_floats(p)) : nullptr;
     // the slot weights p (fp32 for the pairs flagged for strong decay, the decayed operand pair for
@@ -288,9 +292,6 @@ cudaError_t key_side(const gsa_params_t& p, const KeySideArgs& a, int reverse, c
 bool leaves_input_gate(const gsa_params_t& p, bool gate_gradient_follows) {
     return use_tc(p) && !use_wide(p) && p.gate_kind != GSA_GATE_ABC && (p.gate_kind == GSA_GATE_A || !gate_gradient_follows);
 }
-// ... and where the gate tensor holds a it is what they read (16 heads, 32 K tokens of strong gates:
-// the gate kernel 94 -> 82 us)
-bool reads_gate(const gsa_params_t& p) { return use_tc(p) && !use_wide(p) && p.gate_kind == GSA_GATE_A; }
 InputGate input_gate_of(const gsa_params_t& p, const float* gate, bool left_out) {
     return left_out && !reads_gate(p) ? InputGate{gate, p.gate_kind, inv_tau(p)} : InputGate{};
 }
@@ -993,7 +994,7 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
         return GSA_OK;
     }
     // forget-gate gradient: reversed cumulative sum over the whole sequence
-    GSA_LAUNCH("gate_grad", launch_gate_grad(w.u, w.I, w.dIk, s.k, w.dIv, s.v, gate, p.gate_kind, inv_tau(p),
+    GSA_LAUNCH("gate_grad", launch_gate_grad(w.u, I, w.dIk, s.k, w.dIv, s.v, gate, p.gate_kind, inv_tau(p),
                               dKT, w.KT, dVT, w.VT, p.d_k, p.d_v, w.chunk_tot, dgate, p.B, p.T,
                               p.H, p.m, pend, st, dev_status, p.cu_seqlens, p.nseq));
     return GSA_OK;
