@@ -1220,15 +1220,17 @@ int gate_grad_blocks(int T) { return (T + kGG - 1) / kGG; }
 // take a 95th of it for a pair, and 0.12.  us at 2048 tokens, the three kernels / 16 / 32 / 64 slots: 20 pairs
 // (four slices a side) 44 / 44 / 66 / 120, logits 47 / 52 / 82 / 150, 28: 53 / 46 / 66 / 121, 40: 71 / 84 / 68 / 121, logits 75 / 97 /
 // 82 / 152, 72: 108 / 97 / 86 / 138; (one) 28: 36 / 31 / 46 / 80, 48: 53 / 56 / 47 / 80, 80: 75 / 76 / 80 / 76, 112: 100 / 117 / 82 / 78,
-// 160: 133 / 168 / 119 / 148, logits 151 / 199 / 156 / 195, 256: 219 / 256 / 160 / 152.
+// 160: 133 / 168 / 119 / 148, logits 151 / 199 / 156 / 195, 256: 219 / 256 / 160 / 152.  From 16 tokens to 8192 it holds, the walk being
+// ahead by its two launches less at short lengths, but for logits, whose walk takes more to a row: at 8192 tokens, one slice,
+// 48 pairs 184 / 234 / 207 / 394, 96: 357 / 408 / 395 / 399, four slices, 28 pairs 174 / 185 / 342 / 590.
 constexpr int kWalkWideSlices = 3, kWalkSmem = 200 << 10;
-int walk_slots(int pairs, int nslices) {
+int walk_slots(int pairs, int nslices, int gate_kind, int T) {
     if (nslices > kGGTmaMaxSlices) return 0;
-    const float wave[3] = {0.39f, 0.57f, 1.f};
+    const float wave[3] = {0.39f, 0.57f, 1.f}, more = gate_kind == GSA_GATE_LOGITS && T > 3072 ? 1.09f : 1.f;
     float best = 0.95f * ((float)pairs / 95.f + 0.12f);
     int log_slots = 0;
     for (int i = 0; i < 3; ++i) {
-        const float cost = wave[i] * (float)((((long long)pairs << (2 - i)) + kSMs - 1) / kSMs);
+        const float cost = more * wave[i] * (float)((((long long)pairs << (2 - i)) + kSMs - 1) / kSMs);
         if (cost < best) { best = cost; log_slots = 4 + i; }
     }
     return log_slots;
@@ -1246,7 +1248,7 @@ cudaError_t launch_gate_grad(const float* u, const float* I, const float* dIk_pa
         return launch_gate_grad(u, I, dIk_part, nsk, dIv_part, nsv, gate, gate_kind, inv_tau, dKT, KT, dVT, VT, d_k, d_v, blk_tot,
                                 dgate, B, T, 2 * H, 64, pend, st, dev_status, cu_seqlens, nseq);
     }
-    const int log_slots = M == 64 ? walk_slots(B * H, nsk + nsv) : 0;
+    const int log_slots = M == 64 ? walk_slots(B * H, nsk + nsv, gate_kind, T) : 0;
     if (log_slots != 0) {
         const int BH = B * H, nsl = nsk + nsv, cols = 1 << log_slots;
         return with_gate_kind(gate_kind, pend.wide, [&](auto kind, auto wide) {

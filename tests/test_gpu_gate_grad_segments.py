@@ -45,9 +45,10 @@ def dgate_of(d, kind, T, cu=None):
     return got, ref["dgate"]
 
 
-# 16 slots a CTA (28 .. 37 pairs, tiles of 256 rows), 32 (38 .. 74, tiles of 128), 64 slots of 128
+# 16 slots a CTA (28 .. 37 pairs, tiles of 256 rows), 32 (45 .. 74, tiles of 128; at 3200 tokens logits take the three kernels), 128 slots
 @pytest.mark.parametrize("B,H,T,dk,dv,m", [(1, 32, 1500, 128, 128, 64), (1, 32, 2304, 128, 128, 64), (2, 16, 1500, 128, 256, 64),
-                                           (1, 47, 1500, 64, 128, 64), (1, 16, 1500, 128, 128, 128)])
+                                           (1, 47, 1500, 64, 128, 64), (1, 48, 3200, 64, 64, 64),
+                                           (1, 16, 1500, 128, 128, 128)])
 @pytest.mark.parametrize("kind", ["a", "log", "logits"])
 def test_flagged_segments_beside_others(B, H, T, dk, dv, m, kind):
     d = rand_inputs(T + H + m, B, T, H, dk, dv, m, "bf16", init=True, final_grads=True)
