@@ -281,13 +281,14 @@ struct Steps {
 };
 __device__ __forceinline__ Steps all_steps(const ScanSpan& s) { return {s.t0, s.t_end, 0, (s.t_end - s.t0 + kSub - 1) / kSub}; }
 
-// End memories need only the chunks from which anything is left: those that every slot's decay carries below e^-180 on the way
-// to the span's end (reversed: its start) can change nothing in fp32, whatever follows, where their rows are below 2^65 and their
-// weights below 2 -- with gates that forget within a dozen tokens, all but one chunk of the span.  An infinity, a NaN or a row
-// beyond that stays in the memories however hard they forget, so the rows left out are looked through first, and where one of them is
-// found nothing is left out.  32 K tokens of such gates, 16 heads of 128, state runs 31 us without the look, 82 with, 220
+// End memories need only the chunks from which anything is left: with gates that forget within a dozen tokens, all but one chunk of
+// the span.  What every slot's decay carries below 2^-150 on the way to the span's end (reversed: its start) can change nothing
+// in fp32, whatever follows.  A memory whose weights are 1 - a is at most as large as the largest row, whose bound is 2^17: e^-130.
+// Reversed, with rows and weights below 2^17, it is below 2^65 for any T: e^-150.  An infinity, a NaN or a number beyond the
+// bound stays in the memories however hard they forget, or may, so the rows left out are looked through first, and where one of
+// them is found nothing is left out.  32 K tokens of such gates, 16 heads of 128, state runs 31 us without the look, 82 with, 220
 // walking all.
-constexpr float kForgotten = -180.f;
+template <bool REV> constexpr float kForgotten = REV ? -150.f : -130.f;
 // Every warp comes to the same result by itself.
 template <bool REV> __device__ __forceinline__ Steps last_steps(const ValueSideArgs& a, const ScanSpan& span, int lane) {
     Steps s = all_steps(span);
@@ -308,7 +309,7 @@ template <bool REV> __device__ __forceinline__ Steps last_steps(const ValueSideA
             if (kept != 0 || c0 + q >= chunks) continue;
             sum.x += g[q].x;
             sum.y += g[q].y;
-            if (__all_sync(0xffffffffu, fmaxf(sum.x, sum.y) < kForgotten)) kept = c0 + q + 1;
+            if (__all_sync(0xffffffffu, fmaxf(sum.x, sum.y) < kForgotten<REV>)) kept = c0 + q + 1;
         }
     }
     if (kept == 0 || kept == chunks) return s;
@@ -328,8 +329,8 @@ __device__ __forceinline__ uint4 load_once(const void* p) {
     asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
     return v;
 }
-// The steps of a state run.  All threads call it; BOTH: of two sets at once.  Whether the weights are below 2 the gate kernel has seen
-// of 1 - a (`large`); reversed they are looked through here.
+// The steps of a state run.  All threads call it; BOTH: of two sets at once.  Whether a weight 1 - a is not below 2 the gate kernel has
+// seen (`large`); reversed the weights are looked through here.
 template <bool REV, bool BOTH>
 __device__ __noinline__ Steps remembered_steps(const ValueSideArgs& a, const ValueSideArgs& b, int slice, bool large) {
     const ScanSpan span = scan_span(blockIdx.x, a.H, a.T, a.nseg, a.tseg);
@@ -339,7 +340,7 @@ __device__ __noinline__ Steps remembered_steps(const ValueSideArgs& a, const Val
     constexpr int kBatch = 8, kRows = kScanThreads / 16, kSets = BOTH ? 2 : 1;
     const int t_lo = REV ? span.t0 + kSub * kept.count : span.t0, t_hi = REV ? span.t_end : span.t0 + kSub * kept.first;
     const int piece = threadIdx.x & 15;
-    // (2^65 and more, and what is no finite number, has the exponent's two top bits, 2 and more its top one)
+    // (a magnitude of 2^17 or more, or no finite number, has bits from 0x4800 on and carries into the place of the sign)
     uint32_t rows_seen = 0, weights_seen = 0;
     for (int t0 = t_lo + (int)(threadIdx.x >> 4); t0 < t_hi; t0 += kBatch * kRows) {
         uint4 x[kSets][kBatch], w[kBatch];
@@ -356,16 +357,20 @@ __device__ __noinline__ Steps remembered_steps(const ValueSideArgs& a, const Val
         }
 #pragma unroll
         for (int q = 0; q < kBatch; ++q) {
-            weights_seen |= w[q].x | w[q].y | w[q].z | w[q].w;
+            if (REV) {
+                const uint32_t words[4] = {w[q].x, w[q].y, w[q].z, w[q].w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) weights_seen |= (words[e] & 0x7fffffffu) + 0x38000000u;
+            }
 #pragma unroll
             for (int i = 0; i < kSets; ++i) {
                 const uint32_t pairs[4] = {x[i][q].x, x[i][q].y, x[i][q].z, x[i][q].w};
 #pragma unroll
-                for (int e = 0; e < 4; ++e) rows_seen |= pairs[e] & (pairs[e] << 1);
+                for (int e = 0; e < 4; ++e) rows_seen |= (pairs[e] & 0x7fff7fffu) + 0x38003800u;
             }
         }
     }
-    return __syncthreads_or((rows_seen & 0x40004000u) | (weights_seen & 0x40000000u)) ? all : kept;
+    return __syncthreads_or((rows_seen & 0x80008000u) | (weights_seen & 0x80000000u)) ? all : kept;
 }
 
 // A slot warp's copies: the rows of step n into its stage.  A stage's tiles, in this order: NX d-sized ones (128 channels from

@@ -54,11 +54,24 @@ def test_what_never_fades_reaches_the_gradients_of_the_initial_memories():
     assert np.isfinite(got["dV0"][0, 0]).all()
 
 
-def test_large_rows_that_the_gates_forget():
+@pytest.mark.parametrize("large", [1e5, 1e6, 1e30])       # below the bound and beyond
+def test_large_rows_that_the_gates_forget(large):
     H, T, d_ = 3, 1300, 128
     d = forgetful(5, T, H, d_, d_)
-    d["v"][0, 20, 1] = 1e30                               # (the chunk is walked, and nothing is left of it)
+    d["v"][0, 20, 1] = large                              # (the chunk is walked, and nothing is left of it)
     got, gate = run_fwd(d, 1, T, H, d_, d_, 64, "bf16", impl="tc", log=True)
     ref = oracle.fwd(d["q"], d["k"], d["v"], gate, gate_is_log=True, K0=d["K0"], V0=d["V0"])
     assert rel_err(got["VT"], ref["VT"]) <= TOL["bf16"] and rel_err(got["KT"], ref["KT"]) <= TOL["bf16"]
     assert rel_err(got["o"][:, 600:], ref["o"][:, 600:], True) <= TOL["bf16"]
+
+
+@pytest.mark.parametrize("size", [4.0, 1e6])              # weights dz beyond 2, and beyond the bound
+def test_gradients_that_the_gates_forget(size):
+    H, T, d_ = 3, 1300, 128
+    d = forgetful(6, T, H, d_, d_)
+    d["dO"] = (d["dO"] * np.float32(2.0 ** np.round(np.log2(size)))).astype(np.float32)
+    d["dO"][:, 900:] *= 4
+    d["dKT"], d["dVT"] = d["dKT"] * np.float32(size), d["dVT"] * np.float32(size)
+    got, ref = run_bwd(d, 1, T, H, d_, d_, 64, "bf16", impl="tc", log=True)
+    for n in ("dK0", "dV0"):
+        assert rel_err(got[n], ref[n]) <= TOL["bf16"], n
