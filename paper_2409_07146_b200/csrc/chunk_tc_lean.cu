@@ -3,11 +3,11 @@
 // kFactorisedDecayMin), which is every pair of the paper's workloads except the strong-forgetting
 // stress case.
 //
-// Differences from the general scans (chunk_tc_general.cuh), which a CTA whose pair is flagged runs instead:
+// A CTA whose pair is flagged runs a general scan instead (chunk_tc_general.cuh).  What these have that those cannot:
 //   * the slot-sized operands arrive by TMA already multiplied by their decay factor and already
 //     in bfloat16 -- w exp(-G) or w exp(G) as a high/low pair, written once per (batch, head) by
 //     the element-wise kernels that produce w (gate kernel, slot softmax forward / backward)
-//     instead of being rebuilt by each of the D/128 slices of every scan;
+//     instead of being formed by each of the D/128 slices of every scan;
 //   * the per-chunk chain  product -> mask -> product -> read-out  is software-pipelined: the
 //     issuing lane queues the first product of chunk n+1 behind the last product of chunk n and
 //     requests every tile of chunk n+1 as soon as its buffer has been consumed, so the compute

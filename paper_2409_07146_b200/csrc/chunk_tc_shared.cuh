@@ -1,6 +1,5 @@
-// Pieces shared by the tensor-core chunk kernels (the general ones, which also carry the
-// strong-decay path, and the pipelined lean ones): tile geometry, accumulator columns, row
-// access to swizzled fp32 tiles, operand-row stores and the compute-thread barrier.
+// Pieces shared by the tensor-core chunk kernels (the pipelined ones and the general scans of strongly decaying pairs): tile
+// geometry, operand-row stores, masking in tensor memory and the compute-thread barriers.
 #pragma once
 #include <stdio.h>
 
@@ -19,15 +18,9 @@ constexpr int kM = 64;                 // slots
 constexpr int kPanelB = 128 * 128;     // bytes of a 128-row operand panel
 constexpr uint32_t kTmemCols = 512;
 constexpr int kComputeThreads = 256;   // 8 warps: two threads per chunk row
-// + two warps of one active lane each: MMA issue and tile copies (the general scans use the first for both)
+// + two warps of one active lane each: MMA issue and tile copies (the general scans use the first eight warps)
 constexpr int kScanThreads = kComputeThreads + 64;
 constexpr int kHS = kM / 2;            // slots per thread
-
-// accumulator columns
-constexpr int kColP = 0;       // P / A           [128 x 128]
-constexpr int kColO = 128;     // inter (+ intra for key_side) output
-constexpr int kColU = 256;     // state update    [128 x 64] (value_side: [128 x 128], high | low weight parts)
-constexpr int kColO2 = 384;    // value_side: intra-chunk output [128 x 128], high | low weight parts
 
 // Optional phase timing for development builds (-DGSA_TC_PROF): CTA 0 prints, for its fifth
 // chunk, the SM clock at each phase boundary.
@@ -142,12 +135,6 @@ __device__ __forceinline__ void mask_row_in_tmem(uint32_t tmem, int wq, int row,
     }
     tmem_st_wait();
 }
-
-// wait helper of the loops below: a wait that expires flags the CTA
-#define WAIT_OR_ABORT(bar, parity)                          \
-    do {                                                    \
-        if (!mbar_wait(bar, parity)) ctl->abort = 1;        \
-    } while (0)
 
 // What a kernel needs once per device before its first launch: its shared memory, and the check that no second CTA
 // fits beside it -- each CTA takes the whole tensor memory of its SM.
