@@ -81,8 +81,8 @@ __device__ __noinline__ void write_input_gate(const ValueSideArgs& a) {
 
 constexpr int kSub = 16;               // tokens of a step
 constexpr int kStages = 8;             // steps whose rows are on their way or in use
-constexpr int kStateWarps = 4, kSlotWarps = 4;       // one of each to a scheduler
-static_assert(kScanThreads >= 32 * (kStateWarps + kSlotWarps) && kStages == 2 * kSlotWarps, "");
+constexpr int kValueStateWarps = 8, kStateWarps = 4, kSlotWarps = 4;      // (two or) one, and one, to a scheduler
+static_assert(kValueScanThreads >= 32 * (kValueStateWarps + kSlotWarps) && kScanThreads >= 32 * (kStateWarps + kSlotWarps) && kStages == 2 * kSlotWarps, "");
 // tiles of a step, by TMA: two panels of [16 rows][128 bytes] with the 128-byte swizzle (128 channels in bf16, 64 slots in fp32)
 constexpr int kStepPanel = kSub * 128, kXTile = 2 * kStepPanel, kSlotTile = 2 * kStepPanel;
 // rows that the warps write, in bytes: eight rows 16 bytes apart modulo 128 meet in no bank
@@ -107,12 +107,12 @@ __device__ __forceinline__ void general_wait(GeneralCtl* ctl, uint64_t* bar, uin
     __syncwarp();
 }
 
-__device__ __forceinline__ void general_ctl_init(GeneralCtl* ctl, int tid) {
+__device__ __forceinline__ void general_ctl_init(GeneralCtl* ctl, int tid, int state_warps) {
     if (tid == 0) {
         for (int i = 0; i < kStages; ++i) mbar_init(&ctl->full[i], 1);
         for (int i = 0; i < kSlotWarps; ++i) {
             mbar_init(&ctl->ready[i], 1);
-            mbar_init(&ctl->done[i], kStateWarps);
+            mbar_init(&ctl->done[i], state_warps);
         }
         ctl->abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -458,7 +458,7 @@ __device__ __forceinline__ void step_gates(float2 (&g)[kSub], const unsigned cha
 // its own: with high/low pairs of the weights and of the state the gate gradient of gates sigmoid(N(0, 1)), 2048 tokens, is 2.0e-5 off
 // (rms), with three parts 3.5e-6; of sigmoid(N(-2, 1)) 2.1e-5 and 1.0e-5.  The 32 K tokens above take 620 us with pairs.)
 constexpr int kParts = 3;              // of the decayed weights, and of the state as the output's operand
-constexpr int kValueTotal = kParts * kDecTile, kValueO = kValueTotal + 4 * kM, kValueP = kValueO + kSub * kORow;
+constexpr int kValueTotal = kParts * kDecTile, kValueO = kValueTotal + 4 * kM, kValueP = kValueO + 2 * kSub * kORow;
 constexpr int kValueSlotB = kValueP + kSub * kPRow;
 constexpr int kValueStageB = 2 * kXTile + 2 * kSlotTile, kValueStateStageB = kXTile + 2 * kSlotTile;
 
@@ -493,6 +493,7 @@ __device__ __noinline__ bool value_side_general(const StepMaps maps, const Value
     extern __shared__ unsigned char smem_raw[];
     unsigned char* ring = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     constexpr int kStageB = STATES ? kValueStateStageB : kValueStageB;
+    constexpr int kWarps = STATES ? kStateWarps : kValueStateWarps;
     unsigned char* slots = ring + kStages * kStageB;                  // of the slot warps
     GeneralCtl* ctl = reinterpret_cast<GeneralCtl*>(slots + kSlotWarps * kValueSlotB);
 
@@ -500,11 +501,11 @@ __device__ __noinline__ bool value_side_general(const StepMaps maps, const Value
     const ScanSpan span = scan_span(blockIdx.x, a.H, a.T, a.nseg, a.tseg);
     const int d0 = slice * kDST;
     const Steps steps = STATES ? given : all_steps(span);
-    general_ctl_init(ctl, tid);
+    general_ctl_init(ctl, tid, kWarps);
 
-    if (warp >= kStateWarps && warp < kStateWarps + kSlotWarps) {
+    if (warp >= kWarps && warp < kWarps + kSlotWarps) {
         // =============================== slot warps: lane l has slots 2 l and 2 l + 1
-        const int w = warp - kStateWarps;
+        const int w = warp - kWarps;
         unsigned char* mine = slots + w * kValueSlotB;
         float* obase = STATES ? nullptr : a.out + (size_t)slice * a.B * a.T * a.H * kM + 2 * lane;
         load_step<REV, STATES ? 1 : 2, 1>(ctl, ring, maps, steps, span, d0, w);
@@ -589,24 +590,25 @@ __device__ __noinline__ bool value_side_general(const StepMaps maps, const Value
             float* row = obase + (((size_t)span.b * a.T + t) * a.H + span.h) * kM;
             const unsigned char* inter = mine + kValueO + 8 * lane;
 #pragma unroll
-            for (int j = 0; j < kSub; ++j) f[j] = fma2(f[j], *reinterpret_cast<const f32x2*>(inter + j * kORow), acc[j]);
+            for (int j = 0; j < kSub; ++j)
+                f[j] = fma2(f[j], add2(*reinterpret_cast<const f32x2*>(inter + j * kORow), *reinterpret_cast<const f32x2*>(inter + (kSub + j) * kORow)), acc[j]);
 #pragma unroll
             for (int j = 0; j < kSub; ++j)
                 if (t + j < span.t_end) *reinterpret_cast<f32x2*>(row + (size_t)j * a.H * kM) = f[j];
             __syncwarp();
         }
-    } else if (warp < kStateWarps) {
-        // =============================== state warps: S^T[16 slots][128 channels] as accumulator tiles [16 slots][8 channels]
-        constexpr int kTiles = kDST / 8;
-        const int s0 = 16 * warp, g = lane >> 2, t = lane & 3, q = lane >> 3, r = lane & 7;
-        const size_t state = ((size_t)blockIdx.x * kM + s0 + g) * a.D + d0 + 2 * t;
+    } else if (warp < kWarps) {
+        // =============================== state warps: S^T[16 slots][64 (STATES: 128) channels] as accumulator tiles [16 slots][8 channels]
+        constexpr int kTiles = kDST / 8 / (kWarps / 4);
+        const int s0 = 16 * (warp & 3), half = warp >> 2, c0 = d0 + 64 * half, g = lane >> 2, t = lane & 3, q = lane >> 3, r = lane & 7;
+        const size_t state = ((size_t)blockIdx.x * kM + s0 + g) * a.D + c0 + 2 * t;
         float S[kTiles][4];
 #pragma unroll
         for (int nt = 0; nt < kTiles; ++nt)
 #pragma unroll
             for (int e = 0; e < 4; e += 2) {
                 float2 x = make_float2(0.f, 0.f);
-                if (!STATES && d0 + 8 * nt < a.D && a.S0 != nullptr) x = *reinterpret_cast<const float2*>(a.S0 + state + (size_t)4 * e * a.D + 8 * nt);
+                if (!STATES && c0 + 8 * nt < a.D && a.S0 != nullptr) x = *reinterpret_cast<const float2*>(a.S0 + state + (size_t)4 * e * a.D + 8 * nt);
                 S[nt][e] = x.x;
                 S[nt][e + 1] = x.y;
             }
@@ -614,8 +616,8 @@ __device__ __noinline__ bool value_side_general(const StepMaps maps, const Value
         uint32_t at_q[kTiles / 2], at_k[kTiles / 2];
 #pragma unroll
         for (int kb = 0; kb < kTiles / 2; ++kb) {
-            at_q[kb] = x_at(0, (q >> 1) * 8 + r, 2 * kb + (q & 1));
-            at_k[kb] = x_at(0, (q & 1) * 8 + r, 2 * kb + (q >> 1));
+            at_q[kb] = x_at(0, (q >> 1) * 8 + r, 8 * half + 2 * kb + (q & 1));
+            at_k[kb] = x_at(0, (q & 1) * 8 + r, 8 * half + 2 * kb + (q >> 1));
         }
         bool ready = false;
         for (int n = 0; n < steps.count; ++n) {
@@ -672,7 +674,7 @@ __device__ __noinline__ bool value_side_general(const StepMaps maps, const Value
             }
             if (!STATES) {
                 // (columns of the product are tokens: rows of kORow bytes 8 banks apart)
-                float* o = reinterpret_cast<float*>(theirs + kValueO) + s0 + g;
+                float* o = reinterpret_cast<float*>(theirs + kValueO + half * kSub * kORow) + s0 + g;
 #pragma unroll
                 for (int nn = 0; nn < 2; ++nn)
 #pragma unroll
@@ -686,7 +688,7 @@ __device__ __noinline__ bool value_side_general(const StepMaps maps, const Value
             for (int nt = 0; nt < kTiles; ++nt)
 #pragma unroll
                 for (int e = 0; e < 4; e += 2)
-                    if (d0 + 8 * nt < a.D) *reinterpret_cast<float2*>(a.Send + state + (size_t)4 * e * a.D + 8 * nt) = make_float2(S[nt][e], S[nt][e + 1]);
+                    if (c0 + 8 * nt < a.D) *reinterpret_cast<float2*>(a.Send + state + (size_t)4 * e * a.D + 8 * nt) = make_float2(S[nt][e], S[nt][e + 1]);
         }
     }
     return general_finish(ctl, tid, dev_status);
@@ -818,7 +820,7 @@ __device__ __noinline__ bool key_side_general(const StepMaps maps, const KeySide
     const ScanSpan span = scan_span(blockIdx.x, a.H, a.T, a.nseg, a.tseg);
     const int d0 = slice * kDST;
     const Steps steps = all_steps(span);
-    general_ctl_init(ctl, tid);
+    general_ctl_init(ctl, tid, kStateWarps);
 
     if (warp >= kStateWarps && warp < kStateWarps + kSlotWarps) {
         // =============================== slot warps: lane l has slots 2 l and 2 l + 1

@@ -18,8 +18,11 @@ constexpr int kM = 64;                 // slots
 constexpr int kPanelB = 128 * 128;     // bytes of a 128-row operand panel
 constexpr uint32_t kTmemCols = 512;
 constexpr int kComputeThreads = 256;   // 8 warps: two threads per chunk row
-// + two warps of one active lane each: MMA issue and tile copies (the general scans use the first eight warps)
+// + two warps of one active lane each: MMA issue and tile copies
 constexpr int kScanThreads = kComputeThreads + 64;
+// ... of the kernels that also carry the general value_side scan, which has twelve warps (no register less a thread, both counts are
+// rounded up to 384; all kernels of a short call with twelve: a forward over 1431 tokens 48.4 -> 49.0 us)
+constexpr int kValueScanThreads = kComputeThreads + 128;
 constexpr int kHS = kM / 2;            // slots per thread
 
 // Optional phase timing for development builds (-DGSA_TC_PROF): CTA 0 prints, for its fifth
