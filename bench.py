@@ -92,7 +92,8 @@ def kernel_algorithmic_bytes(label: str, w: W.Workload) -> int:
         # a pair of reversed scans as one kernel: both d-sized tiles and both decayed rows once
         "bwd_dv_dIv_pair_rev": 3 * w.d_v * e + 8 * m + 4 * m * nsv,  # dO, v, I exp(-G), p exp(G) -> dv, slices of dI^v
         "bwd_dk_dIk_pair_rev": 3 * w.d_k * e + 8 * m + 4 * m * nsk,  # q, k, I exp(-G), dz exp(G) -> dk, slices of dI^k
-        "gate_grad": 4 * m * (4 + nsk + nsv),                        # u, gate, G, slices -> dgate
+        "gate_grad": 4 * m * (4 + nsk + nsv),                        # u, gate, G, slices -> dgate, in one kernel
+        "gate_grad_blocks": 4 * m * (7 + nsk + nsv),                 # ... in three, of which the last reads gate, r/w dgate
         # fused chunk kernels: the slot rows between the passes stay on chip
         "fused_fwd": e * (2 * w.d_k + 2 * w.d_v) + 12 * m,           # q, k, v, I exp(-G), G -> o, o'
         "fused_bwd": e * (2 * w.d_k + 2 * w.d_v) + 24 * m,           # dO, v, k, I exp(-G), G, o' -> dq, u, p exp(G), dz exp(G)
@@ -457,12 +458,14 @@ def run_ours(args):
         per = {}
         for lab, ms in recs:
             per.setdefault(lab, []).append(ms)
-        # kernels behind one label: gate_cumsum is two (the strong-decay flags cleared, too); a chunk pass is one, with 128 slots two (the flagged pairs
-        # have a launch of their own there)
+        # kernels behind one label: gate_cumsum is two where the strong-decay flags are cleared before it (not on the CUDA-core
+        # kernels, nor where a pair is one chunk of 128 tokens), gate_grad_blocks three; a chunk pass is one, with 128 slots
+        # two (the flagged pairs have a launch of their own there)
+        clears = len(per.get("gate_cumsum", [])) if w.io == "bf16" and (w.T > 128 or w.m == 128) else 0
         two = sum(len(v) for lab, v in per.items() if lab.endswith("_side") or lab.endswith("_side_rev")) if w.m == 128 else 0
         # a fused label is the fused kernel plus the three kernels that serve the flagged pairs
         fusedl = sum(len(v) for lab, v in per.items() if lab.startswith("fused"))
-        launches = (len(recs) + len(per.get("gate_cumsum", [])) + two + 3 * fusedl) // reps
+        launches = (len(recs) + clears + 2 * len(per.get("gate_grad_blocks", [])) + two + 3 * fusedl) // reps
         kernels = []
         tot = sum(sum(v) for v in per.values())
         for lab, v in per.items():

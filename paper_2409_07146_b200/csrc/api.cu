@@ -994,9 +994,13 @@ gsa_status_t bwd_core(const CallParams* params, int m_active, const void* q, con
         return GSA_OK;
     }
     // forget-gate gradient: reversed cumulative sum over the whole sequence
-    GSA_LAUNCH("gate_grad", launch_gate_grad(w.u, I, w.dIk, s.k, w.dIv, s.v, gate, p.gate_kind, inv_tau(p),
-                              dKT, w.KT, dVT, w.VT, p.d_k, p.d_v, w.chunk_tot, dgate, p.B, p.T,
-                              p.H, p.m, pend, st, dev_status, p.cu_seqlens, p.nseq));
+    auto gate_gradient = [&] {
+        return launch_gate_grad(w.u, I, w.dIk, s.k, w.dIv, s.v, gate, p.gate_kind, inv_tau(p), dKT, w.KT, dVT, w.VT, p.d_k, p.d_v,
+                                w.chunk_tot, dgate, p.B, p.T, p.H, p.m, pend, st, dev_status, p.cu_seqlens, p.nseq);
+    };
+    // (named by how many kernels it is)
+    if (gate_grad_kernels(p.B * p.H, p.m, use_wide(p), s.k + s.v, p.gate_kind, p.T) == 1) GSA_LAUNCH("gate_grad", gate_gradient());
+    else GSA_LAUNCH("gate_grad_blocks", gate_gradient());
     return GSA_OK;
 }
 

@@ -9,25 +9,27 @@
 // carried across it, and every decay factor that it forms is at most 1:
 //   value side   out_i = e_i (xq_i S) + sum_j P_ij w_j prod a_r,      S <- e_last S + xk^T (w_j s_j)
 //   key side     out_i = (uq_i e_i) S + sum_j A_ij xv_j,              S <- e_last S + (uk_j s_j)^T xv
-// with e_i the decay from the step's start through token i and s_j that from j to its end (time-reversed: e and s swap).
+// with e_i the decay from the step's start through token i and s_j that from j to its end (time-reversed: e and s swap).  (On the key
+// side one operand of A is lifted by up to e^60, see step_weights; slots that keep most of a chunk take the decay once a
+// chunk, with factors of up to e^0.5 on the rows until then, see step_frame.)
 // tcgen05, whose products have 128 (64) rows, would do four times the work of a 16-token step and a commit and a wait per
-// step on top, so the products are warp-level ones (mma.sync m16n8k16: 8.3 cycles each; 64 a state warp and step on the value
-// side, 88 on the key side).  What bounds it: one state warp's chain of splits and products (960 cycles a step by itself on the
-// value side, 1300 beside its scheduler's slot warp; the tensor pipe is 33 and 40% active).  32 K tokens, 16 heads of 128,
-// a = sigmoid(N(-2, 1)): pass 1 486 -> 208 us, pass 2 410 -> 224 (HBM's share of either: 105), state runs 205 -> 29, the forward
-// 1283 -> 616 us.  The scans before these took 128-token chunks on tcgen05 and walked the decay row by row, 28 k cycles a chunk.
+// step on top, so the products are warp-level ones (mma.sync m16n8k16: 8.3 cycles each; 48 a state warp and step on the value
+// side, 88 on the key side).  What bounds it: a state warp's chain of splits and products, 1830 and 1760 cycles a step of which it
+// waits for 110 and 100 (the slot warps are ahead; the tensor pipe is 42 and 40% active, 0.47 and 0.38 instructions a cycle
+// and scheduler).  32 K tokens, 16 heads of 128, a = sigmoid(N(-2, 1)): pass 1 486 -> 243 us, pass 2 410 -> 237 (HBM's share of either:
+// 105), state runs 205 -> 82, the forward 1285 -> 716.  The scans before these took 128-token chunks on tcgen05 and walked the
+// decay row by row, 28 k cycles a chunk.
 //
 // Warps of two roles, meeting on mbarriers only:
 //   * four slot warps take the steps in turn: a step's rows by TMA, asked for one of a warp's steps ahead (by 16-byte asynchronous
 //     copies of all lanes the warps were held up for 40 cycles a copy, 1400 a step); decay factors, a lane two slots; decayed
-//     operand rows as bf16 high/low pairs; the intra-step term (value side: P by mma, then running decay products in fp32; key
+//     operand rows as three bf16 parts (value side, whose outputs are fp32) or high/low pairs; the intra-step term (value side: P by mma, then running decay products in fp32; key
 //     side: A by mma); at the end the output rows;
-//   * four state warps take every step: the state (value side: 16 slots x 128 channels a warp, key side: 32 channels x
-//     64 slots) stays in registers in fp32, in the fragment layout that serves as the next product's operand as it stands.
-//     (The slot warps' instructions count, as their schedulers' slots are the state warps', too: the decays within a step as products
-//     of its gates instead of an exponential each, and 1 - a taken from the gate tensor where that holds a: 648 -> 616 us.)
-//     (Eight of them, half the channels each: 209 and 252 us; two to a scheduler wait for the same pipes at the same time.  Splits
-//     and decays moved by hand behind other blocks' products: 209 and 250.)
+//   * the state warps take every step: the state (value side, eight warps: 16 slots x 64 channels each; key side, four: 32
+//     channels x 64 slots; state runs, four: 16 slots x 128 channels) stays in registers in fp32, in the fragment layout that
+//     serves as the next product's operand as it stands.  Splitting it in three is what eight are for: four take 2300 cycles a step
+//     on the value side, 290 us; with high/low pairs (208 us) and on the key side (252) eight were no faster than four.  (There,
+//     too, splits and decays moved by hand behind other blocks' products: 209 and 250.)
 // Every wait is bounded: on expiry the CTA flags dev_status, runs out without waiting and returns.
 #pragma once
 #include "chunk_tc_shared.cuh"
@@ -39,7 +41,7 @@ using namespace tcchunk;
 
 // The rows of 1 - a of a flagged pair's moderate chunks, as the gate kernel forms them, where it has left them out
 // (InputGate).  Every CTA that is about to read them writes them all -- the same values -- and reads its own.  A warp a chunk.
-// (All chunks, strong ones too: 32 K tokens of strong gates, 16 heads, 1279 -> 1517 us.)
+// (All chunks, strong ones too: 32 K tokens of strong logits, 16 heads, 806 -> 948 us, of log gates 782 -> 883.)
 // Not inlined: within the pipelined kernels it costs the scan beside it registers (value_side of B = 8, T = 2048, 4 heads of 512,
 // 55 -> 64 us).
 __device__ __noinline__ void write_input_gate(const ValueSideArgs& a) {

@@ -291,6 +291,7 @@ cudaError_t launch_gate_grad(const float* u, const float* I, const float* dIk_pa
                              PendingDecay pend, cudaStream_t st, int32_t* dev_status, const int* cu_seqlens = nullptr,
                              int nseq = 0);
 int gate_grad_blocks(int T);       // entries per (b,h,slot) of launch_gate_grad's scratch
+int gate_grad_kernels(int pairs, int M, bool wide, int nslices, int gate_kind, int T);      // how many kernels it is
 // strong_flag != NULL: after the tensor-core kernels, for the flagged (batch, head) pairs alone; value_side then adds its
 // slices to their 128-wide ones, which those have zeroed
 cudaError_t launch_value_side_simt(const ValueSideArgs& a, int io, int M, int reverse,

@@ -53,8 +53,8 @@ __device__ __forceinline__ bool sequence_starts_at(const int* cu, int nseq, int 
 // What the first token of a packed sequence does to the running log gate.  The memories must lose all they carried
 // there: a log gate of -100, and that is what the CUDA-core kernels get.  On the tensor-core kernels it drops the chunk's
 // total below what the factorised decay can represent, and the whole (batch, head, segment) goes to the strong-decay
-// kernels: a training step on 8K tokens of 13 sequences, 4 heads of 512, takes 1490 us where every chunk with an offset
-// goes there.  A drop of kReset leaves e^-40 = 4e-18 of the old memories -- less than an fp32 rounding of the new ones
+// kernels: a training step on 8K tokens of 13 sequences, 4 heads of 512, takes 970 us where every chunk with an offset
+// goes there, 620 where the segments with two in a chunk do, 330 where none does.  A drop of kReset leaves e^-40 = 4e-18 of the old memories -- less than an fp32 rounding of the new ones
 // while the old are not 1e10 times larger, a slot's first write of 1e-4 of the new values and old values 1e6 times as
 // large -- and the chunk stays on the pipelined kernels where the decay of every slot leaves room for it: for one start in
 // a chunk down to a chunk's own decay of e^-20.  Everywhere else the chunk takes -100 and the strong-decay kernels.
@@ -1236,6 +1236,11 @@ int walk_slots(int pairs, int nslices, int gate_kind, int T) {
     return log_slots;
 }
 
+int gate_grad_kernels(int pairs, int M, bool wide, int nslices, int gate_kind, int T) {
+    if (!wide && M != 64) return 3;
+    return walk_slots(wide ? 2 * pairs : pairs, nslices, gate_kind, T) != 0 ? 1 : 3;
+}
+
 cudaError_t launch_gate_grad(const float* u, const float* I, const float* dIk_part, int nsk,
                              const float* dIv_part, int nsv, const float* gate,
                              int gate_kind, float inv_tau, const float* dKT, const float* KT,
@@ -1248,8 +1253,8 @@ cudaError_t launch_gate_grad(const float* u, const float* I, const float* dIk_pa
         return launch_gate_grad(u, I, dIk_part, nsk, dIv_part, nsv, gate, gate_kind, inv_tau, dKT, KT, dVT, VT, d_k, d_v, blk_tot,
                                 dgate, B, T, 2 * H, 64, pend, st, dev_status, cu_seqlens, nseq);
     }
-    const int log_slots = M == 64 ? walk_slots(B * H, nsk + nsv, gate_kind, T) : 0;
-    if (log_slots != 0) {
+    if (gate_grad_kernels(B * H, M, false, nsk + nsv, gate_kind, T) == 1) {
+        const int log_slots = walk_slots(B * H, nsk + nsv, gate_kind, T);
         const int BH = B * H, nsl = nsk + nsv, cols = 1 << log_slots;
         return with_gate_kind(gate_kind, pend.wide, [&](auto kind, auto wide) {
             auto launch = [&](auto threads) {

@@ -1,6 +1,5 @@
-"""Chunks of strong decay on the tensor-core kernels: the walk away from the diagonal takes 32 distances at a time.  One slot
-that forgets hard sends the pair there, the others' memory decides how far the walk goes: a few steps, past the first band,
-through all four; ragged chunks; both directions."""
+"""Chunks of strong decay on the tensor-core kernels.  One slot that forgets hard sends the pair to the scans that walk 16 tokens at
+a time; the others remember a step or two, a few of them, or all of the chunk; ragged chunks and steps; both directions."""
 import numpy as np
 import pytest
 
