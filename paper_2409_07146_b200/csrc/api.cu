@@ -271,6 +271,7 @@ cudaError_t value_side(const gsa_params_t& p, const ValueSideArgs& a, int revers
     if (use_tc(p)) {
         ValueSideArgs b = a;
         b.single = p.tc_operands == GSA_TC_SINGLE;
+        b.packed = p.cu_seqlens != nullptr;
         return launch_value_side_tc(b, p.m, reverse, strong, st, dev_status);
     }
     return launch_value_side_simt(a, p.io, p.m, reverse, st);

@@ -5,7 +5,7 @@
 namespace gsa {
 namespace {
 
-__global__ void __launch_bounds__(kValueScanThreads, 1)
+__global__ void __launch_bounds__(kScanThreads, 1)
 value_side_general_kernel(const __grid_constant__ GeneralValueMaps maps, const __grid_constant__ ValueSideArgs a, const int* __restrict__ strong_flag, int32_t* dev_status) {
     if (strong_flag[blockIdx.x] == 0) return;
     write_input_gate(a);
@@ -73,7 +73,7 @@ cudaError_t launch_value_side_general(const ValueSideArgs& a, const int* strong_
     if (e == cudaSuccess) e = prepare<value_side_general_kernel>(kSmemGeneral);
     if (e != cudaSuccess) return e;
     const dim3 grid(a.B * a.nseg * a.H, tc_value_side_slices(a.D));
-    value_side_general_kernel<<<grid, kValueScanThreads, kSmemGeneral, st>>>(maps, a, strong_flag, dev_status);
+    value_side_general_kernel<<<grid, kScanThreads, kSmemGeneral, st>>>(maps, a, strong_flag, dev_status);
     return cudaGetLastError();
 }
 

@@ -13,11 +13,11 @@
 // side one operand of A is lifted by up to e^60, see step_weights; slots that keep most of a chunk take the decay once a
 // chunk, with factors of up to e^0.5 on the rows until then, see step_frame.)
 // tcgen05, whose products have 128 (64) rows, would do four times the work of a 16-token step and a commit and a wait per
-// step on top, so the products are warp-level ones (mma.sync m16n8k16: 8.3 cycles each; 48 a state warp and step on the value
-// side, 88 on the key side).  What bounds it: a state warp's chain of splits and products, 1830 and 1760 cycles a step of which it
-// waits for 110 and 100 (the slot warps are ahead; the tensor pipe is 42 and 40% active, 0.47 and 0.38 instructions a cycle
-// and scheduler).  32 K tokens, 16 heads of 128, a = sigmoid(N(-2, 1)): pass 1 486 -> 243 us, pass 2 410 -> 237 (HBM's share of either:
-// 105), state runs 205 -> 82, the forward 1285 -> 716.  The scans before these took 128-token chunks on tcgen05 and walked the
+// step on top, so the products are warp-level ones (mma.sync m16n8k16: 8.3 cycles each; 96 a state warp and step on the value
+// side, 88 on the key side).  What bounds it: a state warp's chain of splits and products, 2300 and 1760 cycles a step of which it
+// waits for 180 and 100 (the slot warps are ahead; the tensor pipe is 35 and 40% active, 0.40 and 0.38 instructions a cycle
+// and scheduler).  32 K tokens, 16 heads of 128, a = sigmoid(N(-2, 1)): pass 1 486 -> 290 us, pass 2 410 -> 237 (HBM's share of either:
+// 105), state runs 205 -> 82, the forward 1285 -> 763.  The scans before these took 128-token chunks on tcgen05 and walked the
 // decay row by row, 28 k cycles a chunk.
 //
 // Warps of two roles, meeting on mbarriers only:
@@ -25,11 +25,13 @@
 //     copies of all lanes the warps were held up for 40 cycles a copy, 1400 a step); decay factors, a lane two slots; decayed
 //     operand rows as three bf16 parts (value side, whose outputs are fp32) or high/low pairs; the intra-step term (value side: P by mma, then running decay products in fp32; key
 //     side: A by mma); at the end the output rows;
-//   * the state warps take every step: the state (value side, eight warps: 16 slots x 64 channels each; key side, four: 32
-//     channels x 64 slots; state runs, four: 16 slots x 128 channels) stays in registers in fp32, in the fragment layout that
-//     serves as the next product's operand as it stands.  Splitting it in three is what eight are for: four take 2300 cycles a step
-//     on the value side, 290 us; with high/low pairs (208 us) and on the key side (252) eight were no faster than four.  (There,
-//     too, splits and decays moved by hand behind other blocks' products: 209 and 250.)
+//   * four state warps take every step: the state (value side: 16 slots x 128 channels a warp, key side: 32 channels x
+//     64 slots) stays in registers in fp32, in the fragment layout that serves as the next product's operand as it stands.  On the
+//     value side in packed sequences eight, half of the channels each: 1830 cycles a step, a training step on 8 K tokens of 13
+//     sequences, 4 heads of 512, 663 -> 624 us.  All calls with twelve warps: the forward above 716 us, but calls without a flagged
+//     pair are slower (see kPackedThreads).  Six, the last quarter of the channels by two warps that are idle otherwise: 780, their schedulers
+//     hold the others up.  (With high/low pairs, 208 us, and on the key side, 252, eight were no faster than four; splits
+//     and decays moved by hand behind other blocks' products: 209 and 250.)
 // Every wait is bounded: on expiry the CTA flags dev_status, runs out without waiting and returns.
 #pragma once
 #include "chunk_tc_shared.cuh"
@@ -83,8 +85,8 @@ __device__ __noinline__ void write_input_gate(const ValueSideArgs& a) {
 
 constexpr int kSub = 16;               // tokens of a step
 constexpr int kStages = 8;             // steps whose rows are on their way or in use
-constexpr int kValueStateWarps = 8, kStateWarps = 4, kSlotWarps = 4;      // (two or) one, and one, to a scheduler
-static_assert(kValueScanThreads >= 32 * (kValueStateWarps + kSlotWarps) && kScanThreads >= 32 * (kStateWarps + kSlotWarps) && kStages == 2 * kSlotWarps, "");
+constexpr int kStateWarps = 4, kSlotWarps = 4;       // one of each to a scheduler (value side, kPackedThreads: two and one)
+static_assert(kScanThreads >= 32 * (kStateWarps + kSlotWarps) && kPackedThreads == 32 * (2 * kStateWarps + kSlotWarps) && kStages == 2 * kSlotWarps, "");
 // tiles of a step, by TMA: two panels of [16 rows][128 bytes] with the 128-byte swizzle (128 channels in bf16, 64 slots in fp32)
 constexpr int kStepPanel = kSub * 128, kXTile = 2 * kStepPanel, kSlotTile = 2 * kStepPanel;
 // rows that the warps write, in bytes: eight rows 16 bytes apart modulo 128 meet in no bank
@@ -166,6 +168,7 @@ __device__ __forceinline__ f32x2 pack2(float x, float y) {
     asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
     return r;
 }
+__device__ __forceinline__ f32x2 both(float x) { return pack2(x, x); }
 __device__ __forceinline__ float2 unpack2(f32x2 v) {
     float2 r;
     asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
@@ -456,9 +459,9 @@ __device__ __forceinline__ void step_gates(float2 (&g)[kSub], const unsigned cha
 // value_side: out_i[s] = sum_{j<=i} <xq_i, xk_j> w_j[s] decay_ij[s]  + decayed (xq_i S)[s]
 // ======================================================================================
 // A slot warp's shared memory: the decayed weights w_j s_j [16][64] in three parts, the step's total decay, the inter-step
-// product [16][64] from the state warps, P.  (The outputs are fp32, and what a step takes from the one before it is not small beside
+// product [16][64] from the state warps (two sums), P.  (The outputs are fp32, and what a step takes from the one before it is not small beside
 // its own: with high/low pairs of the weights and of the state the gate gradient of gates sigmoid(N(0, 1)), 2048 tokens, is 2.0e-5 off
-// (rms), with three parts 3.5e-6; of sigmoid(N(-2, 1)) 2.1e-5 and 1.0e-5.  The 32 K tokens above take 620 us with pairs.)
+// (rms), with three parts 3.5e-6; of sigmoid(N(-2, 1)) 2.1e-5 and 1.0e-5.  Pass 1 of the 32 K tokens above takes 208 us with pairs.)
 constexpr int kParts = 3;              // of the decayed weights, and of the state as the output's operand
 constexpr int kValueTotal = kParts * kDecTile, kValueO = kValueTotal + 4 * kM, kValueP = kValueO + 2 * kSub * kORow;
 constexpr int kValueSlotB = kValueP + kSub * kPRow;
@@ -487,6 +490,104 @@ __device__ __forceinline__ void step_scores(uint32_t xq, uint32_t xk, unsigned c
         }
 }
 
+// A state warp: 16 slots, of the channels of NKB blocks of 16 (all, or half number `half`), as accumulator tiles S^T [16 slots][8
+// channels].
+template <bool STATES, int NKB>
+__device__ __forceinline__ void value_state_warp(GeneralCtl* ctl, unsigned char* ring, unsigned char* slots, const ValueSideArgs& a, const Steps& steps, int d0,
+                                                 int group, int half, int lane) {
+    constexpr int kTiles = 2 * NKB, kStageB = STATES ? kValueStateStageB : kValueStageB;
+    const int s0 = 16 * group, c0 = d0 + 16 * NKB * half, g = lane >> 2, t = lane & 3, q = lane >> 3, r = lane & 7;
+    const size_t state = ((size_t)blockIdx.x * kM + s0 + g) * a.D + c0 + 2 * t;
+    float S[kTiles][4];
+#pragma unroll
+    for (int nt = 0; nt < kTiles; ++nt)
+#pragma unroll
+        for (int e = 0; e < 4; e += 2) {
+            float2 x = make_float2(0.f, 0.f);
+            if (!STATES && c0 + 8 * nt < a.D && a.S0 != nullptr) x = *reinterpret_cast<const float2*>(a.S0 + state + (size_t)4 * e * a.D + 8 * nt);
+            S[nt][e] = x.x;
+            S[nt][e + 1] = x.y;
+        }
+    // the fragments' places in the tiles: channels 16 kb, 16 kb + 8
+    uint32_t at_q[NKB], at_k[NKB];
+#pragma unroll
+    for (int kb = 0; kb < NKB; ++kb) {
+        at_q[kb] = x_at(0, (q >> 1) * 8 + r, 2 * (NKB * half + kb) + (q & 1));
+        at_k[kb] = x_at(0, (q & 1) * 8 + r, 2 * (NKB * half + kb) + (q >> 1));
+    }
+    bool ready = false;
+    for (int n = 0; n < steps.count; ++n) {
+        const int st = n % kStages, w = n % kSlotWarps;
+        unsigned char* tile = ring + st * kStageB;
+        unsigned char* theirs = slots + w * kValueSlotB;
+        // (the slot warp has seen the rows land before it says that its own are ready)
+        if (!ready) general_wait(ctl, &ctl->ready[w], (n / kSlotWarps) & 1);
+        // W^T (rows: slots, k: tokens); xq (k: channels, columns: tokens); xk (k: tokens, columns: channels)
+        uint32_t wp[kParts][4], x[2][4], y[2][4];
+        const uint32_t wa = smem_u32(theirs) + ((q >> 1) * 8 + r) * kDecRow + 2 * (s0 + (q & 1) * 8);
+        const uint32_t qa = smem_u32(tile), ka = smem_u32(tile + (STATES ? 0 : kXTile));
+        if (!STATES) ldsm4(x[0], qa + at_q[0]);
+        ldsm4_trans(y[0], ka + at_k[0]);
+#pragma unroll
+        for (int i = kParts - 1; i >= 0; --i) ldsm4_trans(wp[i], wa + i * kDecTile);
+        const float* total = reinterpret_cast<const float*>(theirs + kValueTotal) + s0 + g;
+        const f32x2 dec[2] = {both(total[0]), both(total[8])};
+        float O[2][2][4] = {};     // [tokens 8 n ..][upper part of the state, the others]
+#pragma unroll
+        for (int kb = 0; kb < NKB; ++kb) {
+            const uint32_t (&xb)[4] = x[kb & 1], (&yb)[4] = y[kb & 1];
+            uint32_t sp[kParts][4];
+            if (!STATES) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float (&f)[4] = S[2 * kb + (e >> 1)];
+                    uint32_t part[kParts];
+                    split_triple(f[2 * (e & 1)], f[2 * (e & 1) + 1], part);
+#pragma unroll
+                    for (int i = 0; i < kParts; ++i) sp[i][e] = part[i];
+                }
+            }
+            if (kb + 1 < NKB) {
+                if (!STATES) ldsm4(x[(kb + 1) & 1], qa + at_q[kb + 1]);
+                ldsm4_trans(y[(kb + 1) & 1], ka + at_k[kb + 1]);
+            }
+            float U[2][4] = {};
+#pragma unroll
+            for (int i = kParts - 1; i >= 0; --i) {
+                mma16816(U[0], wp[i], yb[0], yb[1]);
+                mma16816(U[1], wp[i], yb[2], yb[3]);
+                if (!STATES) {
+                    mma16816(O[0][i > 0], sp[i], xb[0], xb[1]);
+                    mma16816(O[1][i > 0], sp[i], xb[2], xb[3]);
+                }
+            }
+            // (is the next step's there? asked while the products run)
+            if (kb == 2) ready = n + 1 < steps.count && __all_sync(0xffffffffu, mbar_try(&ctl->ready[(n + 1) % kSlotWarps], ((n + 1) / kSlotWarps) & 1));
+#pragma unroll
+            for (int nn = 0; nn < 2; ++nn)
+#pragma unroll
+                for (int e = 0; e < 4; e += 2) decay_add(S[2 * kb + nn][e], S[2 * kb + nn][e + 1], dec[e >> 1], U[nn][e], U[nn][e + 1]);
+        }
+        if (!STATES) {
+            // (columns of the product are tokens: rows of kORow bytes 8 banks apart)
+            float* o = reinterpret_cast<float*>(theirs + kValueO + half * kSub * kORow) + s0 + g;
+#pragma unroll
+            for (int nn = 0; nn < 2; ++nn)
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    o[(8 * nn + 2 * t + (e & 1)) * (kORow / 4) + 8 * (e >> 1)] = O[nn][0][e] + O[nn][1][e];
+        }
+        warp_arrive(&ctl->done[w], lane);
+    }
+    if (!ctl->abort && a.Send != nullptr) {           // (channels past D are zeros throughout and not written)
+#pragma unroll
+        for (int nt = 0; nt < kTiles; ++nt)
+#pragma unroll
+            for (int e = 0; e < 4; e += 2)
+                if (c0 + 8 * nt < a.D) *reinterpret_cast<float2*>(a.Send + state + (size_t)4 * e * a.D + 8 * nt) = make_float2(S[nt][e], S[nt][e + 1]);
+    }
+}
+
 // STATES: end memories only (from empty ones), of the steps given.
 template <bool REV, bool STATES = false>
 __device__ __noinline__ bool value_side_general(const StepMaps maps, const ValueSideArgs& args, int32_t* dev_status, int slice, Steps given = {}) {
@@ -495,7 +596,6 @@ __device__ __noinline__ bool value_side_general(const StepMaps maps, const Value
     extern __shared__ unsigned char smem_raw[];
     unsigned char* ring = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     constexpr int kStageB = STATES ? kValueStateStageB : kValueStageB;
-    constexpr int kWarps = STATES ? kStateWarps : kValueStateWarps;
     unsigned char* slots = ring + kStages * kStageB;                  // of the slot warps
     GeneralCtl* ctl = reinterpret_cast<GeneralCtl*>(slots + kSlotWarps * kValueSlotB);
 
@@ -503,11 +603,13 @@ __device__ __noinline__ bool value_side_general(const StepMaps maps, const Value
     const ScanSpan span = scan_span(blockIdx.x, a.H, a.T, a.nseg, a.tseg);
     const int d0 = slice * kDST;
     const Steps steps = STATES ? given : all_steps(span);
-    general_ctl_init(ctl, tid, kWarps);
+    // twice the state warps, half of the channels each
+    const bool halves = !STATES && blockDim.x == kPackedThreads;
+    general_ctl_init(ctl, tid, halves ? 2 * kStateWarps : kStateWarps);
 
-    if (warp >= kWarps && warp < kWarps + kSlotWarps) {
+    if (warp >= kStateWarps && warp < kStateWarps + kSlotWarps) {
         // =============================== slot warps: lane l has slots 2 l and 2 l + 1
-        const int w = warp - kWarps;
+        const int w = warp - kStateWarps;
         unsigned char* mine = slots + w * kValueSlotB;
         float* obase = STATES ? nullptr : a.out + (size_t)slice * a.B * a.T * a.H * kM + 2 * lane;
         load_step<REV, STATES ? 1 : 2, 1>(ctl, ring, maps, steps, span, d0, w);
@@ -592,106 +694,20 @@ __device__ __noinline__ bool value_side_general(const StepMaps maps, const Value
             float* row = obase + (((size_t)span.b * a.T + t) * a.H + span.h) * kM;
             const unsigned char* inter = mine + kValueO + 8 * lane;
 #pragma unroll
-            for (int j = 0; j < kSub; ++j)
-                f[j] = fma2(f[j], add2(*reinterpret_cast<const f32x2*>(inter + j * kORow), *reinterpret_cast<const f32x2*>(inter + (kSub + j) * kORow)), acc[j]);
+            for (int j = 0; j < kSub; ++j) {
+                f32x2 sum = *reinterpret_cast<const f32x2*>(inter + j * kORow);
+                if (halves) sum = add2(sum, *reinterpret_cast<const f32x2*>(inter + (kSub + j) * kORow));
+                f[j] = fma2(f[j], sum, acc[j]);
+            }
 #pragma unroll
             for (int j = 0; j < kSub; ++j)
                 if (t + j < span.t_end) *reinterpret_cast<f32x2*>(row + (size_t)j * a.H * kM) = f[j];
             __syncwarp();
         }
-    } else if (warp < kWarps) {
-        // =============================== state warps: S^T[16 slots][64 (STATES: 128) channels] as accumulator tiles [16 slots][8 channels]
-        constexpr int kTiles = kDST / 8 / (kWarps / 4);
-        const int s0 = 16 * (warp & 3), half = warp >> 2, c0 = d0 + 64 * half, g = lane >> 2, t = lane & 3, q = lane >> 3, r = lane & 7;
-        const size_t state = ((size_t)blockIdx.x * kM + s0 + g) * a.D + c0 + 2 * t;
-        float S[kTiles][4];
-#pragma unroll
-        for (int nt = 0; nt < kTiles; ++nt)
-#pragma unroll
-            for (int e = 0; e < 4; e += 2) {
-                float2 x = make_float2(0.f, 0.f);
-                if (!STATES && c0 + 8 * nt < a.D && a.S0 != nullptr) x = *reinterpret_cast<const float2*>(a.S0 + state + (size_t)4 * e * a.D + 8 * nt);
-                S[nt][e] = x.x;
-                S[nt][e + 1] = x.y;
-            }
-        // the fragments' places in the tiles: channels 16 kb, 16 kb + 8
-        uint32_t at_q[kTiles / 2], at_k[kTiles / 2];
-#pragma unroll
-        for (int kb = 0; kb < kTiles / 2; ++kb) {
-            at_q[kb] = x_at(0, (q >> 1) * 8 + r, 8 * half + 2 * kb + (q & 1));
-            at_k[kb] = x_at(0, (q & 1) * 8 + r, 8 * half + 2 * kb + (q >> 1));
-        }
-        bool ready = false;
-        for (int n = 0; n < steps.count; ++n) {
-            const int st = n % kStages, w = n % kSlotWarps;
-            unsigned char* tile = ring + st * kStageB;
-            unsigned char* theirs = slots + w * kValueSlotB;
-            // (the slot warp has seen the rows land before it says that its own are ready)
-            if (!ready) general_wait(ctl, &ctl->ready[w], (n / kSlotWarps) & 1);
-            // W^T (rows: slots, k: tokens); xq (k: channels, columns: tokens); xk (k: tokens, columns: channels)
-            uint32_t wp[kParts][4], x[2][4], y[2][4];
-            const uint32_t wa = smem_u32(theirs) + ((q >> 1) * 8 + r) * kDecRow + 2 * (s0 + (q & 1) * 8);
-            const uint32_t qa = smem_u32(tile), ka = smem_u32(tile + (STATES ? 0 : kXTile));
-            if (!STATES) ldsm4(x[0], qa + at_q[0]);
-            ldsm4_trans(y[0], ka + at_k[0]);
-#pragma unroll
-            for (int i = kParts - 1; i >= 0; --i) ldsm4_trans(wp[i], wa + i * kDecTile);
-            const float* total = reinterpret_cast<const float*>(theirs + kValueTotal) + s0 + g;
-            const f32x2 dec[2] = {pack2(total[0], total[0]), pack2(total[8], total[8])};
-            float O[2][2][4] = {};     // [tokens 8 n ..][upper part of the state, the others]
-#pragma unroll
-            for (int kb = 0; kb < kTiles / 2; ++kb) {
-                const uint32_t (&xb)[4] = x[kb & 1], (&yb)[4] = y[kb & 1];
-                uint32_t sp[kParts][4];
-                if (!STATES) {
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float (&f)[4] = S[2 * kb + (e >> 1)];
-                        uint32_t part[kParts];
-                        split_triple(f[2 * (e & 1)], f[2 * (e & 1) + 1], part);
-#pragma unroll
-                        for (int i = 0; i < kParts; ++i) sp[i][e] = part[i];
-                    }
-                }
-                if (kb + 1 < kTiles / 2) {
-                    if (!STATES) ldsm4(x[(kb + 1) & 1], qa + at_q[kb + 1]);
-                    ldsm4_trans(y[(kb + 1) & 1], ka + at_k[kb + 1]);
-                }
-                float U[2][4] = {};
-#pragma unroll
-                for (int i = kParts - 1; i >= 0; --i) {
-                    mma16816(U[0], wp[i], yb[0], yb[1]);
-                    mma16816(U[1], wp[i], yb[2], yb[3]);
-                    if (!STATES) {
-                        mma16816(O[0][i > 0], sp[i], xb[0], xb[1]);
-                        mma16816(O[1][i > 0], sp[i], xb[2], xb[3]);
-                    }
-                }
-                // (is the next step's there? asked while the products run)
-                if (kb == 2) ready = n + 1 < steps.count && __all_sync(0xffffffffu, mbar_try(&ctl->ready[(n + 1) % kSlotWarps], ((n + 1) / kSlotWarps) & 1));
-#pragma unroll
-                for (int nn = 0; nn < 2; ++nn)
-#pragma unroll
-                    for (int e = 0; e < 4; e += 2) decay_add(S[2 * kb + nn][e], S[2 * kb + nn][e + 1], dec[e >> 1], U[nn][e], U[nn][e + 1]);
-            }
-            if (!STATES) {
-                // (columns of the product are tokens: rows of kORow bytes 8 banks apart)
-                float* o = reinterpret_cast<float*>(theirs + kValueO + half * kSub * kORow) + s0 + g;
-#pragma unroll
-                for (int nn = 0; nn < 2; ++nn)
-#pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                        o[(8 * nn + 2 * t + (e & 1)) * (kORow / 4) + 8 * (e >> 1)] = O[nn][0][e] + O[nn][1][e];
-            }
-            warp_arrive(&ctl->done[w], lane);
-        }
-        if (!ctl->abort && a.Send != nullptr) {           // (channels past D are zeros throughout and not written)
-#pragma unroll
-            for (int nt = 0; nt < kTiles; ++nt)
-#pragma unroll
-                for (int e = 0; e < 4; e += 2)
-                    if (c0 + 8 * nt < a.D) *reinterpret_cast<float2*>(a.Send + state + (size_t)4 * e * a.D + 8 * nt) = make_float2(S[nt][e], S[nt][e + 1]);
-        }
+    } else if (!halves) {
+        if (warp < kStateWarps) value_state_warp<STATES, kDST / 16>(ctl, ring, slots, a, steps, d0, warp, 0, lane);
+    } else if (!STATES) {
+        value_state_warp<STATES, kDST / 32>(ctl, ring, slots, a, steps, d0, warp & 3, warp >= kStateWarps ? 1 : 0, lane);
     }
     return general_finish(ctl, tid, dev_status);
 }
@@ -742,7 +758,6 @@ __device__ __forceinline__ void step_product(float (&c)[2][4], uint32_t x, uint3
 // at the block's middle, to which both decay by factors <= 1; four levels L = 8, 4, 2, 1, of which a token plays one part in
 // each -- one pair of rows Z serves both sides -- and the diagonal.
 constexpr int kLift = 43;              // half of -kFactorisedDecayMin log2 e
-__device__ __forceinline__ f32x2 both(float x) { return pack2(x, x); }
 constexpr float kLifted = (float)(1ull << kLift), kLowered = 1.f / kLifted;
 template <bool REV>
 __device__ __forceinline__ void step_weights(float (&c)[2][4], const f32x2 (&lifted)[kSub], const unsigned char* uq, const unsigned char* uk, const unsigned char* gates,

@@ -116,7 +116,7 @@ constexpr int kLkA = 0, kLkO = 128 /* two buffers of 128 */, kLkU = 384;        
 //   sums the slices of `out` multiplies it in (see PendingDecay), so this kernel needs no G tile.
 // ======================================================================================
 template <bool REV, bool PAIRS>
-__global__ void __launch_bounds__(kValueScanThreads, 1)
+__global__ void __launch_bounds__(kPackedThreads, 1)
 value_side_lean_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
                        const __grid_constant__ CUtensorMap mapWd, const __grid_constant__ CUtensorMap mapO,
                        const __grid_constant__ GeneralValueMaps general, const __grid_constant__ ValueSideArgs a, const int* strong_flag, int32_t* dev_status) {
@@ -905,7 +905,7 @@ cudaError_t launch_value_side_tc(const ValueSideArgs& a, int M, int reverse, con
     constexpr size_t smem = kSmemLeanValue > kSmemGeneral ? kSmemLeanValue : kSmemGeneral;
     auto launch = [&](auto kernel, cudaError_t ready) {
         if (ready != cudaSuccess) return ready;
-        launch_after(kernel, grid, kValueScanThreads, smem, st, mq, mk, mw, mo, general, a, strong_flag, dev_status);
+        launch_after(kernel, grid, a.packed ? kPackedThreads : kScanThreads, smem, st, mq, mk, mw, mo, general, a, strong_flag, dev_status);
         return cudaGetLastError();
     };
 #define GSA_VALUE(REV, PAIRS) launch(value_side_lean_kernel<REV, PAIRS>, prepare<value_side_lean_kernel<REV, PAIRS>>(smem))

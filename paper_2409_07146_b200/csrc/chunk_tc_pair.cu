@@ -64,7 +64,7 @@ constexpr int kPcP = 0, kPcA = 128, kPcO2 = 256, kPcU = 384, kPcOI = 448;
 struct GeneralPairMaps { CUtensorMap x, y, w, q, G; };
 
 template <bool PAIRS>
-__global__ void __launch_bounds__(kValueScanThreads, 1)
+__global__ void __launch_bounds__(kPackedThreads, 1)
 rev_pair_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapY,
                 const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapQ,
                 const __grid_constant__ CUtensorMap mapOv, const __grid_constant__ CUtensorMap mapOk,
@@ -489,7 +489,7 @@ cudaError_t launch_rev_pair_tc(const ValueSideArgs& av, const KeySideArgs& ak, i
     constexpr size_t smem = kSmemPair > kSmemGeneral ? kSmemPair : kSmemGeneral;
     auto launch = [&](auto kernel, cudaError_t ready) {
         if (ready != cudaSuccess) return ready;
-        launch_after(kernel, grid, kValueScanThreads, smem, st, mx, my, mw, mq, mov, mok, general, av, ak, strong_flag, dev_status);
+        launch_after(kernel, grid, packed ? kPackedThreads : kScanThreads, smem, st, mx, my, mw, mq, mov, mok, general, av, ak, strong_flag, dev_status);
         return cudaGetLastError();
     };
     return av.single ? launch(rev_pair_kernel<false>, prepare<rev_pair_kernel<false>>(smem))

@@ -20,9 +20,10 @@ constexpr uint32_t kTmemCols = 512;
 constexpr int kComputeThreads = 256;   // 8 warps: two threads per chunk row
 // + two warps of one active lane each: MMA issue and tile copies
 constexpr int kScanThreads = kComputeThreads + 64;
-// ... of the kernels that also carry the general value_side scan, which has twelve warps (no register less a thread, both counts are
-// rounded up to 384; all kernels of a short call with twelve: a forward over 1431 tokens 48.4 -> 49.0 us)
-constexpr int kValueScanThreads = kComputeThreads + 128;
+// ... and of the kernels that carry the general value_side scan in packed sequences, which regularly flag a segment: four warps more
+// share its state (see value_side_general).  Not in other calls: twelve warps leave no registers to the CTAs of the next kernel, which
+// are placed while these drain (a forward over 700 tokens 45.9 -> 46.4 us, a training step B = 2, T = 1024, 16 heads of 128, 152 -> 155).
+constexpr int kPackedThreads = kScanThreads + 64;
 constexpr int kHS = kM / 2;            // slots per thread
 
 // Optional phase timing for development builds (-DGSA_TC_PROF): CTA 0 prints, for its fifth

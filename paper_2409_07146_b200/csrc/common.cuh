@@ -134,6 +134,7 @@ struct ValueSideArgs {
     const float* E = nullptr;         // kernels for 128 slots: exp(G), see launch_gate_cumsum_wide
     InputGate input_gate;             // forward-direction runs on the tensor cores; gate null: w is there
     int w_keeps = 0;                  // general scans: w holds a, the weights are 1 - a
+    int packed = 0;                   // tensor-core kernels: of packed sequences (how many warps the general scans get)
     float* seg_logdecay = nullptr;    // state runs, forward, K side: receives the segments' log-decay (launch_segment_logdecay)
 };
 struct KeySideArgs {

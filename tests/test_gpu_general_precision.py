@@ -3,9 +3,11 @@ oracle: the fp32 outputs (logits, gate gradient, final memories), slots that kee
 that forgets, and gradients near the ends of what fp32 holds."""
 import numpy as np
 import pytest
+import torch
 
+import paper_2409_07146_b200 as gsa
 from test_gpu_parity import run_bwd, run_fwd
-from util import rand_inputs
+from util import rand_inputs, to_dev, to_np
 
 import oracle
 
@@ -60,3 +62,26 @@ def test_gradients_of_any_size(size):
     got, ref = run_bwd(x, B, T, H, d, d, m, "bf16", impl="tc", log=True)
     for n in ("dq", "dk", "dv"):                           # (the rounding to bfloat16 is 1.66e-3)
         assert rms_err(got[n], ref[n]) <= 1.7e-3, n
+
+
+# calls of packed sequences, whose scans have twice the state warps: half a slice, one slice and two; a segment with two offsets in a chunk
+@pytest.mark.parametrize("dk,dv", [(64, 128), (128, 64), (256, 256)])
+def test_packed_calls(dk, dv):
+    B, T, H, m = 1, 1400, 2, 64
+    cu = [0, 300, 310, 1025, T]
+    x = rand_inputs(21 + dk, B, T, H, dk, dv, m, "bf16")
+    x["gate"] = np.log(sigmoid(np.random.default_rng(dk).standard_normal((B, T, H, m)))).astype(np.float32)
+    p = gsa.Params(B, T, H, dk, dv, m, io="bf16", gate_is_log=True, cu_seqlens=torch.tensor(cu, dtype=torch.int32, device="cuda"))
+    q, k, v, dO = (to_dev(x[n], "bf16") for n in ("q", "k", "v", "dO"))
+    gate = to_dev(x["gate"])
+    logits, KT, VT = torch.empty(B, T, H, m, device="cuda"), torch.empty(B, H, m, dk, device="cuda"), torch.empty(B, H, m, dv, device="cuda")
+    o = gsa.gsa_fwd(p, q, k, v, gate, ok_save=logits, KT=KT, VT=VT)
+    dq, dk_, dv_, dgate = gsa.gsa_bwd(p, q, k, v, gate, dO, ok_saved=logits)
+    args = (x["q"], x["k"], x["v"], x["gate"])
+    ref = dict(oracle.fwd_packed(*args, cu, gate_is_log=True), **oracle.bwd_packed(*args, x["dO"], cu, gate_is_log=True))
+    # (two offsets in a chunk of eleven: its G goes beyond -200, and an fp32 rounding of that is 200 * 2^-25 = 6e-6 to 1.2e-5 of a decay;
+    # a root of eleven less of the whole, beside the 1.2e-6 of the other chunks; the gate gradient of the scans
+    # in fp32 was 6.0e-6)
+    for n, t, bound in (("ok", logits, 3e-6), ("KT", KT, 4e-6), ("VT", VT, 4e-6), ("dgate", dgate, 8e-6),     # (memories: pairs in the state runs' products)
+                        ("o", o, 1.7e-3), ("dq", dq, 1.7e-3), ("dk", dk_, 1.7e-3), ("dv", dv_, 1.7e-3)):
+        assert rms_err(to_np(t), ref[n]) <= bound, (n, rms_err(to_np(t), ref[n]))
