@@ -120,6 +120,18 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
         }
         g[i] = make_float2(fmaxf(x.x, kLogGateMin), fmaxf(x.y, kLogGateMin));
     }
+    const bool owns_flag = !WIDE && strong_flag != nullptr && owns_strong_flag(nseg, (int)gridDim.y);
+    // is there a weight that is 2 or more, or no finite number (the exponent's top bit)?  See remembered_steps.  (Here, where nothing
+    // of it is kept: behind the sums two registers spill, 32 K tokens of 16 heads 84.6 -> 86.4 us.)
+    if (!WIDE && large_weight != nullptr) {
+        uint32_t seen = 0;
+#pragma unroll
+        for (int i = 0; i < kCumRows; ++i) seen |= __float_as_uint(inps[i].x) | __float_as_uint(inps[i].y);
+        bool large = (seen & 0x40000000u) != 0;
+        if (owns_flag) large = __syncthreads_or(large);
+        if (large || (owns_flag && threadIdx.x == 0 && grp == 0))
+            large_weight[(b * nseg + (nseg == 1 ? 0 : t_chunk / tseg)) * H + h] = large;
+    }
     // the first token of a packed sequence drops what the memories carried; its own write, 1 - a, is untouched
     if (cu_seqlens != nullptr && (starts[0] | starts[1] | starts[2] | starts[3]) != 0) {
         const uint32_t mine = (starts[(grp * kCumRows) >> 5] >> ((grp * kCumRows) & 31)) & ((1u << kCumRows) - 1);
@@ -171,25 +183,12 @@ __global__ void __launch_bounds__(M * 8 > 1024 ? 1024 : M * 8, M > 64 ? 1 : 2) g
     const bool strong = strong_flag != nullptr && grp == (int)blockDim.y - 1 &&
                         fmin(before0 + acc0, before1 + acc1) < (double)kFactorisedDecayMin;
     // (1 - a left out: of the chunks that do not decide on the general scans by themselves, see InputGate)
-    const bool owns_flag = !WIDE && strong_flag != nullptr && owns_strong_flag(nseg, (int)gridDim.y);
     bool any_strong = strong;
     if (owns_flag || leave_out == 1) any_strong = __syncthreads_or(strong);
-    // is there a weight that is 2 or more, or no finite number (the exponent's top bit)?  See remembered_steps.
-    uint32_t seen = 0;
-    if (!WIDE && large_weight != nullptr) {
-#pragma unroll
-        for (int i = 0; i < kCumRows; ++i) seen |= __float_as_uint(inps[i].x) | __float_as_uint(inps[i].y);
-        seen &= 0x40000000u;
-        if (owns_flag) seen = __syncthreads_or(seen);
-    }
     const bool put_I = leave_out == 0 || (leave_out == 1 && any_strong);
     if (strong || (owns_flag && threadIdx.x == 0 && grp == 0)) {
         const int seg = nseg == 1 ? 0 : t_chunk / tseg;
         strong_flag[WIDE ? (b * nseg + seg) * (H / 2) + h / 2 : (b * nseg + seg) * H + h] = any_strong;
-    }
-    if (seen != 0 || (owns_flag && large_weight != nullptr && threadIdx.x == 0 && grp == 0)) {
-        const int seg = nseg == 1 ? 0 : t_chunk / tseg;
-        large_weight[(b * nseg + seg) * H + h] = seen != 0;
     }
     // second pass over the same rows: the sums of the groups before as a float pair (value, rest)
     const float b0h = (float)before0, b0l = (float)(before0 - (double)b0h);
